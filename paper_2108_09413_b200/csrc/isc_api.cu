@@ -785,7 +785,7 @@ int isc_decide_certify_integer(const int32_t *counts0, const int32_t *counts, in
         if (counts0[c] < 0 || counts[c] < 0 || counts[c] > N) return ISC_ERR_ARG;
     int32_t q = 0;
     int64_t q2 = 0;
-    *out_class = decide_certify_integer(counts0, counts, n_classes, N, sigma, alpha, two_sided != 0, &q, &q2);
+    *out_class = decide_certify_integer(counts0, counts, n_classes, N, sigma, alpha, two_sided != 0, &q, &q2, nullptr);
     *out_q = q;
     if (out_q_squared) *out_q_squared = q2;
     return ISC_OK;
