@@ -9,10 +9,8 @@
 #include <string.h>
 
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <new>
-#include <thread>
 #include <vector>
 
 #include "isc.h"
@@ -62,17 +60,19 @@ struct isc_model {
     int ws_batch = 0;
 
     // per-call device scratch
-    uint8_t *d_x = nullptr;       size_t d_x_bytes = 0;
-    int32_t *d_counts = nullptr;  size_t d_counts_n = 0;
+    // One buffer: error word (16 bytes), vote counts, images.  A call's upload (zeros and images) and its download (error
+    // word and counts) are one copy each, through the pinned buffer, whose front both share.
+    uint8_t *d_io = nullptr;      size_t d_io_bytes = 0;
+    uint8_t *h_io = nullptr;      size_t h_io_bytes = 0;
     int8_t *d_logits = nullptr;   size_t d_logits_bytes = 0;
     uint32_t *d_cum = nullptr;    size_t d_cum_n = 0;
+    std::vector<uint32_t> h_cum;                // the cumulative table, without the guide
     double cum_sigma = -1.0;
     int cum_T = 0, cum_kind = -1, cum_steps = 0;
 
     isc::LinePlan *line = nullptr;
 
-    // isc_certify_batch: pinned copy of the vote counts, one event per image
-    int32_t *h_counts = nullptr;  size_t h_counts_bytes = 0;
+    // isc_certify_batch: one event per piece of the batch
     std::vector<cudaEvent_t> events;
 
     int64_t opt_batch = 0, opt_engine = 0, opt_noise = 0, opt_tensor_copy = 1;
@@ -349,9 +349,10 @@ int ensure_noise_table(isc_model *m, double sigma, cudaStream_t st)
     if (m->opt_noise) noise_table_rounded(sigma, cum); else noise_table(sigma, cum);
     // the guide table follows the cumulative one in the same allocation
     const size_t n_cum = cum.size();
+    m->h_cum = cum;
+    uint32_t i = 0;
     for (int j = 0; j <= isc::kNoiseGuide; ++j) {
         const uint64_t u = (uint64_t)j << (32 - isc::kNoiseGuideBits);
-        uint32_t i = 0;
         while (i + 1 < n_cum && u >= cum[i]) ++i;        // min{ i : u < cum[i] }, the last entry matching always
         cum.push_back(i);
     }
@@ -382,6 +383,13 @@ int check_stream_args(uint64_t image_id, int32_t phase, int64_t first, int64_t n
     return ISC_OK;
 }
 
+int check_certify_args(uint64_t last_image_id, int64_t N0, int64_t N, double sigma, double alpha)
+{
+    if (N0 < 1 || N < 1 || !(alpha > 0.0 && alpha < 1.0)) return ISC_ERR_ARG;
+    if (N0 > (1ll << 31) - 1 || N > (1ll << 31) - 1) return ISC_ERR_ARG;
+    return check_stream_args(last_image_id, 0, 0, std::max(N0, N), sigma);
+}
+
 NoiseStream make_stream(const isc_model *m, uint64_t seed, uint64_t image_id, int32_t phase, int64_t first)
 {
     NoiseStream ns;
@@ -408,7 +416,7 @@ int choose_engine(isc_model *m)
 }
 
 // Layer-by-layer forward of `batch` samples; leaves the logits in the last tensor's buffer.
-int generic_forward(isc_model *m, const uint8_t *d_x, const NoiseStream &ns, int batch, cudaStream_t st,
+int generic_forward(isc_model *m, const uint8_t *d_x, const NoiseStream &ns, int batch, cudaStream_t st, int32_t *d_err,
                     int stop_after_layer = -1, bool tensor_cores = false)
 {
     const int n = (int)m->glayers.size();
@@ -420,9 +428,9 @@ int generic_forward(isc_model *m, const uint8_t *d_x, const NoiseStream &ns, int
         const int8_t *res = L.res_tensor >= 0 ? (const int8_t *)m->bufs[(size_t)m->tensor_buf[(size_t)L.res_tensor]].p : nullptr;
         cudaError_t e;
         if (i == 0 && tensor_cores && m->wpacks[0])
-            e = launch_stem_conv(G, m->wpacks[0], m->tc_cst[0], m->tc_fast[0] != 0, d_x, m->in_c, ns, batch, out, m->d_tc_err, st);
+            e = launch_stem_conv(G, m->wpacks[0], m->tc_cst[0], m->tc_fast[0] != 0, d_x, m->in_c, ns, batch, out, d_err, st);
         else if (i == 0) e = launch_first_conv(G, d_x, m->in_c, ns, batch, out, st);
-        else if (tensor_cores && m->wpacks[(size_t)i]) e = launch_igemm_conv(G, m->wpacks[(size_t)i], m->tc_cst[(size_t)i], m->tc_fast[(size_t)i] != 0, m->tc_resk[(size_t)i], batch, in, res, out, m->d_tc_err, st, false, m->opt_tensor_copy != 0);
+        else if (tensor_cores && m->wpacks[(size_t)i]) e = launch_igemm_conv(G, m->wpacks[(size_t)i], m->tc_cst[(size_t)i], m->tc_fast[(size_t)i] != 0, m->tc_resk[(size_t)i], batch, in, res, out, d_err, st, false, m->opt_tensor_copy != 0);
         else if (L.op == ISC_CONV2D || L.op == ISC_FC) e = launch_conv(G, batch, in, res, out, st);
         else if (L.op == ISC_GAVGPOOL) e = launch_gavgpool(G, batch, in, out, st);
         else e = launch_maxpool(G, batch, in, out, st);
@@ -443,20 +451,10 @@ size_t generic_bytes_per_sample(const isc_model *m)
     return s;
 }
 
-// The Monte-Carlo loop for one image and one phase; adds votes into d_counts (device).
-int run_counts(isc_model *m, const uint8_t *d_x, uint64_t seed, uint64_t image_id, int32_t phase,
-               int64_t first, int64_t n, cudaStream_t st, int32_t *d_counts, int8_t *d_logits)
+// The Monte-Carlo loop for one image and one phase on the layer-by-layer engines; adds votes into d_counts (device).
+int layerwise_counts(isc_model *m, const uint8_t *d_x, uint64_t seed, uint64_t image_id, int32_t phase, int64_t first, int64_t n,
+                     cudaStream_t st, int32_t *d_counts, int8_t *d_logits, int32_t *d_err)
 {
-    const int engine = choose_engine(m);
-    if (engine < 0) return engine;
-    m->last_engine = engine;
-    if (engine == 3) {
-        NoiseStream ns = make_stream(m, seed, image_id, phase, first);
-        int64_t launches = 0;
-        int rc = isc::line_run(m->line, d_x, ns, n, (int)m->opt_batch, d_counts, d_logits, st, &launches);
-        m->launches += launches;
-        return rc;
-    }
     int64_t cap = m->opt_batch > 0 ? m->opt_batch : 4096;
     const size_t per = std::max<size_t>(generic_bytes_per_sample(m), 1);
     cap = std::min<int64_t>(cap, std::max<int64_t>(1, (int64_t)((3ull << 30) / per)));
@@ -468,7 +466,7 @@ int run_counts(isc_model *m, const uint8_t *d_x, uint64_t seed, uint64_t image_i
     for (int64_t done = 0; done < n; done += cap) {
         const int b = (int)std::min<int64_t>(cap, n - done);
         NoiseStream ns = make_stream(m, seed, image_id, phase, first + done);
-        rc = generic_forward(m, d_x, ns, b, st, -1, engine == 2);
+        rc = generic_forward(m, d_x, ns, b, st, d_err, -1, m->last_engine == 2);
         if (rc) return rc;
         const int8_t *lg = (const int8_t *)m->bufs[(size_t)m->tensor_buf[(size_t)last]].p;
         cudaError_t e = launch_votes(lg, m->shapes[(size_t)last].cp, m->n_classes, b, d_counts,
@@ -479,41 +477,110 @@ int run_counts(isc_model *m, const uint8_t *d_x, uint64_t seed, uint64_t image_i
     return ISC_OK;
 }
 
-int stage_image(isc_model *m, const uint8_t *x, size_t bytes, bool on_device, cudaStream_t st,
-                const uint8_t **d_x)
+constexpr size_t kCountsOff = 16;                        // of the counts in the call buffer: the error word comes first
+constexpr size_t kStagedBytes = 4u << 20;                // larger uploads and downloads do not go through the pinned buffer
+
+int ensure_pinned(isc_model *m, size_t need)
 {
-    if (on_device) { *d_x = x; return ISC_OK; }
-    void *p = m->d_x; size_t have = m->d_x_bytes;
-    int rc = ensure_bytes(&p, &have, bytes);
-    m->d_x = (uint8_t *)p; m->d_x_bytes = have;
-    if (rc) return rc;
-    CK(cudaMemcpyAsync(m->d_x, x, bytes, cudaMemcpyHostToDevice, st));
-    *d_x = m->d_x;
+    if (m->h_io_bytes >= need) return ISC_OK;
+    if (m->h_io) cudaFreeHost(m->h_io);
+    m->h_io = nullptr; m->h_io_bytes = 0;
+    need = (need + 4095) & ~(size_t)4095;
+    CK(cudaHostAlloc((void **)&m->h_io, need, cudaHostAllocDefault));
+    m->h_io_bytes = need;
     return ISC_OK;
 }
 
-// After the stream has been synchronised: has a bounded wait of a tensor-core kernel expired?
-int check_engines(isc_model *m)
+// The start of a call: error word and `n_counts` counts cleared, the images on the device.
+int begin_call(isc_model *m, const uint8_t *x, size_t x_bytes, bool x_on_device, size_t n_counts, cudaStream_t st, const uint8_t **d_x)
 {
+    const size_t head = kCountsOff + n_counts * sizeof(int32_t), x_off = (head + 15) & ~(size_t)15;
+    void *p = m->d_io;
+    int rc = ensure_bytes(&p, &m->d_io_bytes, x_off + (x_on_device ? 0 : x_bytes));
+    m->d_io = (uint8_t *)p;
+    if (rc) return rc;
+    const bool staged = !x_on_device && x_off + x_bytes <= kStagedBytes;
+    if ((rc = ensure_pinned(m, staged ? x_off + x_bytes : head))) return rc;
+    if (staged) {
+        memset(m->h_io, 0, x_off);
+        memcpy(m->h_io + x_off, x, x_bytes);
+        CK(cudaMemcpyAsync(m->d_io, m->h_io, x_off + x_bytes, cudaMemcpyHostToDevice, st));
+    } else {
+        CK(cudaMemsetAsync(m->d_io, 0, head, st));
+        if (!x_on_device) CK(cudaMemcpyAsync(m->d_io + x_off, x, x_bytes, cudaMemcpyHostToDevice, st));
+    }
+    *d_x = x_on_device ? x : m->d_io + x_off;
+    return ISC_OK;
+}
+int32_t *call_err(isc_model *m) { return (int32_t *)m->d_io; }
+int32_t *call_counts(isc_model *m) { return (int32_t *)(m->d_io + kCountsOff); }
+const int32_t *host_counts(const isc_model *m) { return (const int32_t *)(m->h_io + kCountsOff); }
+
+// The error word, then counts [first, first + n), back into the pinned buffer.
+int fetch_counts(isc_model *m, size_t first, size_t n, cudaStream_t st)
+{
+    const size_t off = first ? kCountsOff + first * sizeof(int32_t) : 0, end = kCountsOff + (first + n) * sizeof(int32_t);
+    CK(cudaMemcpyAsync(m->h_io + off, m->d_io + off, end - off, cudaMemcpyDeviceToHost, st));
+    return ISC_OK;
+}
+
+// After the stream has been synchronised and the error word fetched: has a bounded wait of a tensor-core kernel expired?
+int call_status(const isc_model *m)
+{
+    const int32_t e = *(const int32_t *)m->h_io;
+    if (m->last_engine == 3) return isc::line_status(e);
+    return e ? ISC_ERR_TIMEOUT : ISC_OK;
+}
+
+// Votes of `n_images` images, n_sel samples of phase 0 and n_est of phase 1 each; `decide(i, counts0, counts)` is called
+// for image after image while the kernels of later ones are in flight.
+template <typename Decide>
+int count_images(isc_model *m, const uint8_t *x, bool x_on_device, int n_images, uint64_t seed, uint64_t image_id0, int64_t n_sel,
+                 int64_t n_est, double sigma, cudaStream_t st, Decide decide)
+{
+    const int engine = choose_engine(m);
+    if (engine < 0) return engine;
+    m->last_engine = engine;
+    const size_t C = (size_t)m->n_classes, d = (size_t)m->in_c * m->in_h * m->in_w;
     int rc;
-    if (m->line && (rc = isc::line_check(m->line))) return rc;
-    if (m->d_tc_err && m->last_engine == 2) {
-        int32_t e = 0;
-        CK(cudaMemcpy(&e, m->d_tc_err, sizeof(e), cudaMemcpyDeviceToHost));
-        if (e != 0) {
-            cudaMemset(m->d_tc_err, 0, sizeof(e));
-            return ISC_ERR_TIMEOUT;
+    if ((rc = ensure_noise_table(m, sigma, st))) return rc;
+    const uint8_t *d_x;
+    if ((rc = begin_call(m, x, d * (size_t)n_images, x_on_device, 2 * C * (size_t)n_images, st, &d_x))) return rc;
+    // Pieces of the batch: as many images as make some sixty rounds of the resident engine's groups, so that a launch's
+    // last, partly empty round costs little, and the host's bounds still run under the next piece's kernels.
+    int piece = 1;
+    if (engine == 3)
+        piece = (int)std::max<int64_t>(1, std::min<int64_t>(n_images, 64 * isc::line_wave_samples(m->line) / (n_sel + n_est)));
+    const int n_pieces = (n_images + piece - 1) / piece;
+    while ((int)m->events.size() < n_pieces - 1) {
+        cudaEvent_t ev;
+        CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+        m->events.push_back(ev);
+    }
+    for (int k = 0; k < n_pieces && rc == ISC_OK; ++k) {
+        const int i0 = k * piece, n = std::min(piece, n_images - i0);
+        int32_t *c = call_counts(m) + (size_t)i0 * 2 * C;
+        if (engine == 3) {
+            const isc::LineWork w{d_x + (size_t)i0 * d, n, image_id0 + (uint64_t)i0, n_sel, n_est, 0, c, nullptr};
+            rc = isc::line_run(m->line, w, make_stream(m, seed, 0, 1, 0), (int)m->opt_batch, call_err(m), st, &m->launches);
+        } else {
+            const uint8_t *xi = d_x + (size_t)i0 * d;
+            rc = layerwise_counts(m, xi, seed, image_id0 + (uint64_t)i0, 0, 0, n_sel, st, c, nullptr, call_err(m));
+            if (rc == ISC_OK) rc = layerwise_counts(m, xi, seed, image_id0 + (uint64_t)i0, 1, 0, n_est, st, c + C, nullptr, call_err(m));
+        }
+        if (rc == ISC_OK) rc = fetch_counts(m, (size_t)i0 * 2 * C, (size_t)n * 2 * C, st);
+        if (rc == ISC_OK && k + 1 < n_pieces && cudaEventRecord(m->events[(size_t)k], st) != cudaSuccess) { cudaGetLastError(); rc = ISC_ERR_CUDA; }
+    }
+    if (rc == ISC_OK && n_pieces > 1 && cudaMemcpyAsync(m->h_io, m->d_io, kCountsOff, cudaMemcpyDeviceToHost, st) != cudaSuccess) { cudaGetLastError(); rc = ISC_ERR_CUDA; }
+    if (rc) { cudaStreamSynchronize(st); return rc; }
+    for (int k = 0; k < n_pieces; ++k) {
+        CK(k + 1 < n_pieces ? cudaEventSynchronize(m->events[(size_t)k]) : cudaStreamSynchronize(st));
+        for (int i = k * piece; i < std::min(n_images, (k + 1) * piece); ++i) {
+            const int32_t *c0 = host_counts(m) + (size_t)i * 2 * C;
+            decide(i, c0, c0 + C);
         }
     }
-    return ISC_OK;
-}
-
-int ensure_counts(isc_model *m, size_t n)
-{
-    void *p = m->d_counts; size_t have = m->d_counts_n * sizeof(int32_t);
-    int rc = ensure_bytes(&p, &have, n * sizeof(int32_t));
-    m->d_counts = (int32_t *)p; m->d_counts_n = have / sizeof(int32_t);
-    return rc;
+    return call_status(m);
 }
 
 }  // namespace
@@ -604,11 +671,10 @@ void isc_free_qmodel(isc_model *m)
     if (!m) return;
     for (void *p : m->param_allocs) cudaFree(p);
     for (DevBuf &b : m->bufs) if (b.p) cudaFree(b.p);
-    if (m->d_x) cudaFree(m->d_x);
-    if (m->d_counts) cudaFree(m->d_counts);
+    if (m->d_io) cudaFree(m->d_io);
     if (m->d_logits) cudaFree(m->d_logits);
     if (m->d_cum) cudaFree(m->d_cum);
-    if (m->h_counts) cudaFreeHost(m->h_counts);
+    if (m->h_io) cudaFreeHost(m->h_io);
     for (cudaEvent_t ev : m->events) cudaEventDestroy(ev);
     isc::line_free(m->line);
     delete m;
@@ -623,34 +689,48 @@ int isc_sample_counts(isc_model *m, const uint8_t *x_u8, uint64_t seed, uint64_t
     if (rc) return rc;
     if (n_samples > (1ll << 31) - 1) return ISC_ERR_ARG;
     cudaStream_t st = (cudaStream_t)cuda_stream;
+    const int engine = choose_engine(m);
+    if (engine < 0) return engine;
+    m->last_engine = engine;
     const size_t C = (size_t)m->n_classes;
+    const size_t logit_bytes = out_logits ? (size_t)n_samples * C : 0;
+    const size_t logits_off = kCountsOff + C * sizeof(int32_t);          // in the pinned buffer
+    const bool staged = logits_off + logit_bytes <= kStagedBytes;
     if ((rc = ensure_noise_table(m, sigma, st))) return rc;
-    if ((rc = ensure_counts(m, C))) return rc;
-    const uint8_t *d_x;
-    if ((rc = stage_image(m, x_u8, (size_t)m->in_c * m->in_h * m->in_w, false, st, &d_x))) return rc;
+    if ((rc = ensure_pinned(m, logits_off + (staged ? logit_bytes : 0)))) return rc;
     if (out_logits) {
         void *p = m->d_logits; size_t have = m->d_logits_bytes;
-        rc = ensure_bytes(&p, &have, (size_t)std::max<int64_t>(n_samples, 1) * C);
+        rc = ensure_bytes(&p, &have, std::max<size_t>(logit_bytes, C));
         m->d_logits = (int8_t *)p; m->d_logits_bytes = have;
         if (rc) return rc;
     }
-    CK(cudaMemsetAsync(m->d_counts, 0, C * sizeof(int32_t), st));
-    if ((rc = run_counts(m, d_x, seed, image_id, phase, first_sample, n_samples, st, m->d_counts,
-                         out_logits ? m->d_logits : nullptr))) {
+    const uint8_t *d_x;
+    if ((rc = begin_call(m, x_u8, (size_t)m->in_c * m->in_h * m->in_w, false, C, st, &d_x))) return rc;
+    int8_t *d_logits = out_logits ? m->d_logits : nullptr;
+    if (engine == 3) {
+        const isc::LineWork w{d_x, 1, image_id, 0, n_samples, 0, call_counts(m), d_logits};
+        rc = isc::line_run(m->line, w, make_stream(m, seed, 0, phase, first_sample), (int)m->opt_batch, call_err(m), st, &m->launches);
+    } else {
+        rc = layerwise_counts(m, d_x, seed, image_id, phase, first_sample, n_samples, st, call_counts(m), d_logits, call_err(m));
+    }
+    if (rc) {
         cudaStreamSynchronize(st);
         return rc;
     }
-    std::vector<int32_t> h(C);
+    if ((rc = fetch_counts(m, 0, C, st))) return rc;
     std::vector<int8_t> hl;
-    CK(cudaMemcpyAsync(h.data(), m->d_counts, C * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-    if (out_logits && n_samples > 0) {
-        hl.resize((size_t)n_samples * C);
-        CK(cudaMemcpyAsync(hl.data(), m->d_logits, hl.size(), cudaMemcpyDeviceToHost, st));
+    const int8_t *h_logits = (const int8_t *)m->h_io + logits_off;
+    if (logit_bytes) {
+        if (!staged) {
+            hl.resize(logit_bytes);
+            h_logits = hl.data();
+        }
+        CK(cudaMemcpyAsync(const_cast<int8_t *>(h_logits), m->d_logits, logit_bytes, cudaMemcpyDeviceToHost, st));
     }
     CK(cudaStreamSynchronize(st));
-    if ((rc = check_engines(m))) return rc;
-    memcpy(out_counts, h.data(), C * sizeof(int32_t));
-    if (out_logits && n_samples > 0) memcpy(out_logits, hl.data(), hl.size());
+    if ((rc = call_status(m))) return rc;
+    memcpy(out_counts, host_counts(m), C * sizeof(int32_t));
+    if (logit_bytes) memcpy(out_logits, h_logits, logit_bytes);
     return ISC_OK;
 }
 
@@ -672,80 +752,19 @@ int isc_certify_batch(isc_model *m, const uint8_t *x_u8, int x_on_device, int n_
                       int32_t *out_class, double *out_radius, int32_t *out_counts0, int32_t *out_counts)
 {
     if (!m || !x_u8 || !out_class || !out_radius || n_images < 0) return ISC_ERR_ARG;
-    if (N0 < 1 || N < 1 || !(alpha > 0.0 && alpha < 1.0)) return ISC_ERR_ARG;
-    if (N0 > (1ll << 31) - 1 || N > (1ll << 31) - 1) return ISC_ERR_ARG;
-    int rc = check_stream_args(image_id0 + (uint64_t)std::max(n_images - 1, 0), 0, 0, std::max(N0, N), sigma);
+    int rc = check_certify_args(image_id0 + (uint64_t)std::max(n_images - 1, 0), N0, N, sigma, alpha);
     if (rc) return rc;
     if (n_images == 0) return ISC_OK;
-    cudaStream_t st = (cudaStream_t)cuda_stream;
     const size_t C = (size_t)m->n_classes;
-    const size_t d = (size_t)m->in_c * m->in_h * m->in_w;
-    if ((rc = ensure_noise_table(m, sigma, st))) return rc;
-    if ((rc = ensure_counts(m, 2 * C * (size_t)n_images))) return rc;
-    const uint8_t *d_x;
-    if ((rc = stage_image(m, x_u8, d * (size_t)n_images, x_on_device != 0, st, &d_x))) return rc;
-    CK(cudaMemsetAsync(m->d_counts, 0, 2 * C * (size_t)n_images * sizeof(int32_t), st));
-    // Pinned staging for the counts and one event per image: the host bound of image i (Algorithm 1 steps 5-7, up to
-    // a hundred milliseconds of bisection at N = 100,000) runs on a worker thread while the kernels of the images
-    // after it are in flight.
-    const size_t need = 2 * C * (size_t)n_images * sizeof(int32_t);
-    if (m->h_counts_bytes < need) {
-        if (m->h_counts) cudaFreeHost(m->h_counts);
-        m->h_counts = nullptr; m->h_counts_bytes = 0;
-        CK(cudaHostAlloc((void **)&m->h_counts, need, cudaHostAllocDefault));
-        m->h_counts_bytes = need;
-    }
-    while ((int)m->events.size() < n_images) {
-        cudaEvent_t ev;
-        CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
-        m->events.push_back(ev);
-    }
-    int dev = 0;
-    CK(cudaGetDevice(&dev));
     std::vector<int32_t> cls((size_t)n_images, -1);
     std::vector<double> rad((size_t)n_images, 0.0);
-    std::atomic<int> enqueued(0);
-    std::atomic<bool> failed(false);
-    int32_t *h = m->h_counts;
-    const int n_cls = m->n_classes;
-    // a few workers, image i on worker i mod n_workers: one bound can take longer than one image's kernels
-    const int n_workers = std::max(1, std::min(std::min(n_images, 4), (int)std::thread::hardware_concurrency()));
-    auto work = [&, dev, h, n_cls](int first) {
-        if (cudaSetDevice(dev) != cudaSuccess) { failed = true; return; }
-        for (int i = first; i < n_images; i += n_workers) {
-            while (enqueued.load(std::memory_order_acquire) <= i) {
-                if (failed.load()) return;
-                std::this_thread::yield();
-            }
-            if (cudaEventSynchronize(m->events[(size_t)i]) != cudaSuccess) { failed = true; return; }
-            const int32_t *c0 = h + (size_t)i * 2 * C, *c1 = c0 + C;
-            double radius = 0.0;
-            cls[(size_t)i] = decide_certify(c0, c1, n_cls, N, sigma, alpha, &radius, nullptr);
-            rad[(size_t)i] = radius;
-        }
-    };
-    std::vector<std::thread> workers;
-    for (int t = 0; t < n_workers; ++t) workers.emplace_back(work, t);
-    for (int i = 0; i < n_images && rc == ISC_OK; ++i) {
-        int32_t *c0 = m->d_counts + (size_t)i * 2 * C;
-        rc = run_counts(m, d_x + (size_t)i * d, seed, image_id0 + (uint64_t)i, 0, 0, N0, st, c0, nullptr);
-        if (rc == ISC_OK)
-            rc = run_counts(m, d_x + (size_t)i * d, seed, image_id0 + (uint64_t)i, 1, 0, N, st, c0 + C, nullptr);
-        if (rc == ISC_OK && (cudaMemcpyAsync(h + (size_t)i * 2 * C, c0, 2 * C * sizeof(int32_t), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-                             cudaEventRecord(m->events[(size_t)i], st) != cudaSuccess)) {
-            cudaGetLastError();
-            rc = ISC_ERR_CUDA;
-        }
-        if (rc == ISC_OK) enqueued.store(i + 1, std::memory_order_release);
-    }
-    if (rc) failed = true;
-    for (std::thread &t : workers) t.join();
-    if (rc) { cudaStreamSynchronize(st); return rc; }
-    CK(cudaStreamSynchronize(st));
-    if (failed.load()) return ISC_ERR_CUDA;
-    if ((rc = check_engines(m))) return rc;
+    rc = count_images(m, x_u8, x_on_device != 0, n_images, seed, image_id0, N0, N, sigma, (cudaStream_t)cuda_stream,
+                      [&](int i, const int32_t *c0, const int32_t *c1) {
+                          cls[(size_t)i] = decide_certify(c0, c1, m->n_classes, N, sigma, alpha, &rad[(size_t)i], nullptr);
+                      });
+    if (rc) return rc;
     for (int i = 0; i < n_images; ++i) {
-        const int32_t *c0 = h + (size_t)i * 2 * C, *c1 = c0 + C;
+        const int32_t *c0 = host_counts(m) + (size_t)i * 2 * C, *c1 = c0 + C;
         out_class[i] = cls[(size_t)i];
         out_radius[i] = rad[(size_t)i];
         if (out_counts0) memcpy(out_counts0 + (size_t)i * C, c0, C * sizeof(int32_t));
@@ -796,18 +815,23 @@ int isc_certify_integer(isc_model *m, const uint8_t *x_u8, uint64_t seed, uint64
                         int32_t *out_q, int64_t *out_q_squared, int32_t *out_counts0, int32_t *out_counts)
 {
     if (!m || !x_u8 || !out_class || !out_q) return ISC_ERR_ARG;
-    const size_t C = (size_t)m->n_classes;
-    std::vector<int32_t> c0(C), c1(C);
-    int32_t cls = -1;
-    double radius = 0.0;
-    int rc = isc_certify_batch(m, x_u8, 0, 1, seed, image_id, N0, N, sigma, alpha, cuda_stream, &cls, &radius,
-                               c0.data(), c1.data());
+    int rc = check_certify_args(image_id, N0, N, sigma, alpha);
     if (rc) return rc;
-    rc = isc_decide_certify_integer(c0.data(), c1.data(), m->n_classes, N, sigma, alpha, two_sided, &cls, out_q, out_q_squared);
+    const size_t C = (size_t)m->n_classes;
+    int32_t cls = -1, q = 0;
+    int64_t q2 = 0;
+    rc = count_images(m, x_u8, false, 1, seed, image_id, N0, N, sigma, (cudaStream_t)cuda_stream,
+                      [&](int, const int32_t *c0, const int32_t *c1) {
+                          // the handle's table is Eq. 2's unless it draws from the rounded law
+                          cls = decide_certify_integer(c0, c1, m->n_classes, N, sigma, alpha, two_sided != 0, &q, &q2,
+                                                       m->cum_kind == 0 ? &m->h_cum : nullptr);
+                      });
     if (rc) return rc;
     *out_class = cls;
-    if (out_counts0) memcpy(out_counts0, c0.data(), C * sizeof(int32_t));
-    if (out_counts) memcpy(out_counts, c1.data(), C * sizeof(int32_t));
+    *out_q = q;
+    if (out_q_squared) *out_q_squared = q2;
+    if (out_counts0) memcpy(out_counts0, host_counts(m), C * sizeof(int32_t));
+    if (out_counts) memcpy(out_counts, host_counts(m) + C, C * sizeof(int32_t));
     return ISC_OK;
 }
 
@@ -892,13 +916,12 @@ int isc_debug_tensor(isc_model *m, const uint8_t *x_u8, uint64_t seed, uint64_t 
     cudaStream_t st = (cudaStream_t)cuda_stream;
     if ((rc = ensure_noise_table(m, sigma, st))) return rc;
     const uint8_t *d_x;
-    if ((rc = stage_image(m, x_u8, (size_t)m->in_c * m->in_h * m->in_w, false, st, &d_x))) return rc;
+    if ((rc = begin_call(m, x_u8, (size_t)m->in_c * m->in_h * m->in_w, false, (size_t)m->n_classes, st, &d_x))) return rc;
     NoiseStream ns = make_stream(m, seed, image_id, phase, j);
     if (m->opt_engine == 3) {       // read the tensor back from the resident engine
         if (!m->line) return ISC_ERR_UNSUPPORTED;
-        if ((rc = ensure_counts(m, (size_t)m->n_classes))) return rc;
         std::vector<int32_t> tmp(n);
-        rc = isc::line_debug_tensor(m->line, d_x, ns, tensor, tmp.data(), m->d_counts, st, &m->launches);
+        rc = isc::line_debug_tensor(m->line, d_x, ns, tensor, tmp.data(), call_counts(m), st, &m->launches);
         if (rc) return rc;
         memcpy(out, tmp.data(), n * sizeof(int32_t));
         return ISC_OK;
@@ -914,7 +937,7 @@ int isc_debug_tensor(isc_model *m, const uint8_t *x_u8, uint64_t seed, uint64_t 
         return e == cudaSuccess ? ISC_OK : ISC_ERR_CUDA;
     }
     if ((rc = ensure_workspace(m, 1))) return rc;
-    if ((rc = generic_forward(m, d_x, ns, 1, st, tensor - 1, m->opt_engine == 2 || (m->opt_engine == 0 && m->has_tc)))) return rc;
+    if ((rc = generic_forward(m, d_x, ns, 1, st, call_err(m), tensor - 1, m->opt_engine == 2 || (m->opt_engine == 0 && m->has_tc)))) return rc;
     std::vector<int8_t> h((size_t)s.h * s.w * s.cp);
     CK(cudaMemcpyAsync(h.data(), m->bufs[(size_t)m->tensor_buf[(size_t)tensor]].p, h.size(),
                        cudaMemcpyDeviceToHost, st));

@@ -72,6 +72,7 @@ constexpr int kCtrlBytes = 10240;
 constexpr int kMaxConv = 128;
 constexpr int kSmemLimit = 227 * 1024;
 constexpr int kTmemCols = 512;
+constexpr int kSideStreams = 8;             // concurrent launches when a launch does not fill the GPU
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // 2 s per wait
 
 enum { PH_FILL = 0, PH_INPUT = 1, PH_CONV = 2, PH_TAIL = 3 };
@@ -133,9 +134,13 @@ struct LineParams {
     const ConvSrc *conv_src;
     const uint8_t *bar_counts;
     int32_t n_bars, n_phases, n_conv, n_groups;
-    int32_t n_samples, in_c, in_H, in_W;
-    const uint8_t *x;                 // clean image, CHW
-    NoiseStream ns;
+    int32_t in_c, in_H, in_W;
+    // What the groups of four samples are: per image, groups_sel groups of the selection phase (n_sel samples from
+    // number 0 on), then groups_est of the estimation phase (n_est samples from ns.first_sample on).
+    int32_t groups_sel, groups_est, n_sel, n_est, phase_sel;
+    unsigned long long image_id0;     // of image 0
+    const uint8_t *x;                 // clean images, CHW, one after the other
+    NoiseStream ns;                   // ctr3_fixed: the estimation phase's number; ctr2 is not used
     uint32_t input_base, input_pitch16;   // line 0, lane 0 of the first layer's operand region
     // tail
     uint32_t tail_base, tail_plane, tail_pitch16, tail_logI;
@@ -144,8 +149,8 @@ struct LineParams {
     const int8_t *fc_w;               // [n_classes][64]
     const FcConst *fc_c;
     int32_t n_classes;
-    int32_t *counts;
-    int8_t *logits;                   // [n_samples][n_classes] or null
+    int32_t *counts;                  // [image][phases in use][n_classes]
+    int8_t *logits;                   // [n_est][n_classes] or null (one image, no selection phase)
     int32_t *err;
     unsigned long long *phase_cycles; // [4]: SM cycles per CTA spent in FILL, INPUT, everything else, TAIL, summed over CTAs and launches
     // debug
@@ -160,7 +165,6 @@ struct Ctrl {
     uint32_t tmem_base;
     volatile int abort_flag;
     uint32_t stored[kMaxBars];              // per unit: stores of its 16-channel chunks by a warp, counted over the whole run
-    int32_t hist[128];
     int32_t pooled[kG][64];                 // the tail's pooled features, one row per sample of the group
     long long cyc[4], cyc_mark;             // thread 0's phase clocks
     PhaseEntry ptab[kMaxPhases];
@@ -733,6 +737,23 @@ __device__ void fill_phase(const EpiCtx &c, uint32_t off, uint32_t bytes, uint32
     for (uint32_t o = (uint32_t)c.tid * 16u; o < bytes; o += kThreads * 16u) st_shared_v4(c.sbase + off + o, v);
 }
 
+// Which samples a group holds: image, phase, and the range of sample numbers.
+struct GroupJob {
+    int image, local, n;              // local: index of the group's first sample within the image's phase; n: samples of that phase
+    bool sel;
+};
+__device__ __forceinline__ GroupJob group_job(const LineParams &p, int grp)
+{
+    GroupJob g;
+    const int per_image = p.groups_sel + p.groups_est;
+    g.image = grp / per_image;
+    const int r = grp - g.image * per_image;
+    g.sel = r < p.groups_sel;
+    g.local = kG * (g.sel ? r : r - p.groups_sel);
+    g.n = g.sel ? p.n_sel : p.n_est;
+    return g;
+}
+
 // INPUT: one thread = four horizontally adjacent pixels of one sample, all input channels (Def. 3.3, Def. 3.4).
 __device__ void input_phase(const LineParams &p, const EpiCtx &c, int grp)
 {
@@ -742,15 +763,19 @@ __device__ void input_phase(const LineParams &p, const EpiCtx &c, int grp)
     const uint32_t *__restrict__ cum = p.ns.cum;
     const uint32_t *__restrict__ guide = p.ns.guide;
     const int T = p.ns.T;
-    const uint32_t key0 = p.ns.key0, key1 = p.ns.key1, ctr2 = p.ns.ctr2;
-    const uint8_t *__restrict__ x = p.x;
+    const GroupJob g = group_job(p, grp);
+    const unsigned long long image_id = p.image_id0 + (unsigned long long)g.image;
+    const uint32_t key0 = p.ns.key0, key1 = p.ns.key1, ctr2 = (uint32_t)image_id;
+    const uint32_t ctr3_fixed = (g.sel ? (uint32_t)p.phase_sel : p.ns.ctr3_fixed) | ((uint32_t)(image_id >> 32) & 0xFFFFu) << 16;
+    const long long j0 = (g.sel ? 0ll : p.ns.first_sample) + g.local;
+    const uint8_t *__restrict__ x = p.x + (size_t)g.image * (size_t)(in_c * H * W);
     for (int qi = c.tid; qi < quads; qi += kThreads) {
         // consecutive threads take consecutive samples: their stores fall into one 64-byte run
         const int s = qi & (kG - 1);
         const int rem = qi >> 2;
         const int y = rem / wq, x4 = rem - y * wq;
-        const long long j = p.ns.first_sample + (long long)grp * kG + s;
-        const uint32_t ctr3 = p.ns.ctr3_fixed | (uint32_t)(((j >> 32) & 0xFF) << 8);
+        const long long j = j0 + s;
+        const uint32_t ctr3 = ctr3_fixed | (uint32_t)(((j >> 32) & 0xFF) << 8);
         uint32_t px[4] = {0, 0, 0, 0};
         for (int ch = 0; ch < in_c; ++ch) {
             const uint32_t e = (uint32_t)((ch * H + y) * W + 4 * x4);
@@ -801,8 +826,9 @@ __device__ void tail_sample(const LineParams &p, const EpiCtx &c, int s, int grp
 {
     const int tail_C = p.tail_C;
     const int n_classes = p.n_classes;
-    const long long sample = (long long)grp * kG + s;          // index within this launch
-    const bool counted = sample < p.n_samples;
+    const GroupJob g = group_job(p, grp);
+    const int sample = g.local + s;                            // index within the image's phase
+    const bool counted = sample < g.n;
     int best_v = -1000, best_o = 0x7fffffff;
     for (int o0 = 0; o0 < n_classes; o0 += 32) {
         const int o = o0 + c.lane;
@@ -817,7 +843,7 @@ __device__ void tail_sample(const LineParams &p, const EpiCtx &c, int s, int grp
         v = v > 127 ? 127 : v;
         if (live) {
             if ((int)v > best_v) { best_v = (int)v; best_o = o; }
-            if (counted && p.logits) p.logits[sample * n_classes + o] = (int8_t)v;
+            if (counted && p.logits) p.logits[(long long)sample * n_classes + o] = (int8_t)v;
         }
     }
     // lowest index among the maxima
@@ -826,7 +852,10 @@ __device__ void tail_sample(const LineParams &p, const EpiCtx &c, int s, int grp
         const int ov = __shfl_xor_sync(0xffffffffu, best_v, d), oo = __shfl_xor_sync(0xffffffffu, best_o, d);
         if (ov > best_v || (ov == best_v && oo < best_o)) { best_v = ov; best_o = oo; }
     }
-    if (counted && c.lane == 0) atomicAdd(&c.ctrl->hist[best_o], 1);
+    if (counted && c.lane == 0) {
+        const int row = p.groups_sel ? 2 * g.image + (g.sel ? 0 : 1) : g.image;
+        atomicAdd(p.counts + (size_t)row * n_classes + best_o, 1);
+    }
 }
 
 __global__ void __launch_bounds__(kThreads, 1) k_line(const __grid_constant__ LineParams p)
@@ -841,7 +870,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_line(const __grid_constant__ Li
         mbar_init(smem_u32(&ctrl->drain), kIssuers);
         ctrl->abort_flag = 0;
     }
-    for (int i = threadIdx.x; i < 128; i += blockDim.x) ctrl->hist[i] = 0;
     for (int i = threadIdx.x; i < p.n_phases; i += blockDim.x) ctrl->ptab[i] = p.ptab[i];
     for (int i = threadIdx.x; i < p.n_conv; i += blockDim.x) ctrl->csrc[i] = p.conv_src[i];
     for (int i = threadIdx.x; i < kMaxBars; i += blockDim.x) ctrl->stored[i] = 0;
@@ -939,9 +967,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_line(const __grid_constant__ Li
         atomicAdd(p.phase_cycles + PH_TAIL, (unsigned long long)ctrl->cyc[PH_TAIL]);
         atomicAdd(p.phase_cycles + PH_CONV, (unsigned long long)(total - ctrl->cyc[PH_FILL] - ctrl->cyc[PH_INPUT] - ctrl->cyc[PH_TAIL]));
     }
-    if (!ctrl->abort_flag)
-        for (int i = threadIdx.x; i < p.n_classes; i += blockDim.x)
-            if (ctrl->hist[i]) atomicAdd(p.counts + i, ctrl->hist[i]);
     if (p.dump)
         for (uint32_t o = threadIdx.x * 16u; o < p.dump_bytes; o += blockDim.x * 16u)
             *reinterpret_cast<uint4 *>(p.dump + o) = ld_shared_v4(sbase + p.dump_off + o);
@@ -1070,6 +1095,9 @@ struct LinePlan {
     uint8_t *d_dump = nullptr;
     int sm_count = 0;
     bool attr_set = false;
+    // launches smaller than the GPU (see line_run)
+    cudaStream_t side[kSideStreams] = {};
+    cudaEvent_t fork_event = nullptr, join_event[kSideStreams] = {};
 };
 
 namespace {
@@ -1794,18 +1822,59 @@ int line_build(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_w
     return ISC_OK;
 }
 
+static void line_free_streams(LinePlan *p)
+{
+    for (int i = 0; i < kSideStreams; ++i) {
+        if (p->side[i]) cudaStreamDestroy(p->side[i]);
+        if (p->join_event[i]) cudaEventDestroy(p->join_event[i]);
+        p->side[i] = nullptr;
+        p->join_event[i] = nullptr;
+    }
+    if (p->fork_event) cudaEventDestroy(p->fork_event);
+    p->fork_event = nullptr;
+}
+
 void line_free(LinePlan *p)
 {
     if (!p) return;
+    line_free_streams(p);
     cudaFree(p->d_ptab); cudaFree(p->d_conv_src); cudaFree(p->d_bar_counts); cudaFree(p->d_blob); cudaFree(p->d_fc_w);
     cudaFree(p->d_fc_c); cudaFree(p->d_err); cudaFree(p->d_phase_cycles); cudaFree(p->d_dump);
     delete p;
 }
 
+static void line_free_streams(LinePlan *p);
+
+// The side streams start after what `st` holds so far ...
+static int line_fork(LinePlan *p, cudaStream_t st)
+{
+    if (!p->fork_event) {
+        bool ok = cudaEventCreateWithFlags(&p->fork_event, cudaEventDisableTiming) == cudaSuccess;
+        for (int i = 0; i < kSideStreams && ok; ++i)
+            ok = cudaStreamCreateWithFlags(&p->side[i], cudaStreamNonBlocking) == cudaSuccess &&
+                 cudaEventCreateWithFlags(&p->join_event[i], cudaEventDisableTiming) == cudaSuccess;
+        if (!ok) { cudaGetLastError(); line_free_streams(p); return ISC_ERR_CUDA; }
+    }
+    bool ok = cudaEventRecord(p->fork_event, st) == cudaSuccess;
+    for (int i = 0; i < kSideStreams && ok; ++i) ok = cudaStreamWaitEvent(p->side[i], p->fork_event, 0) == cudaSuccess;
+    if (!ok) { cudaGetLastError(); return ISC_ERR_CUDA; }
+    return ISC_OK;
+}
+
+// ... and `st` goes on after them.
+static int line_join(LinePlan *p, cudaStream_t st)
+{
+    bool ok = true;
+    for (int i = 0; i < kSideStreams; ++i)
+        ok = cudaEventRecord(p->join_event[i], p->side[i]) == cudaSuccess && cudaStreamWaitEvent(st, p->join_event[i], 0) == cudaSuccess && ok;
+    if (!ok) { cudaGetLastError(); return ISC_ERR_CUDA; }
+    return ISC_OK;
+}
+
 static int line_launch(LinePlan *p, LineParams &q, cudaStream_t st)
 {
     if (!p->attr_set) {
-        if (cudaFuncSetAttribute(k_line, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p->smem_bytes) != cudaSuccess) {
+        if (cudaFuncSetAttribute(k_line, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) != cudaSuccess) {
             cudaGetLastError();
             return ISC_ERR_CUDA;
         }
@@ -1818,37 +1887,83 @@ static int line_launch(LinePlan *p, LineParams &q, cudaStream_t st)
     return e == cudaSuccess ? ISC_OK : ISC_ERR_CUDA;
 }
 
-int line_run(LinePlan *p, const uint8_t *d_x, const NoiseStream &ns, int64_t n, int batch_hint, int32_t *d_counts,
-             int8_t *d_logits, cudaStream_t st, int64_t *launches)
+int64_t line_wave_samples(const LinePlan *p) { return (int64_t)kG * p->sm_count; }
+
+// Every call's work as launches of at most `batch_hint` samples (0: as few launches as possible).  A launch is a list
+// of groups over images and phases: CERTIFY's N0 = 100 samples take 25 of 148 SMs for a whole round when they are launched
+// alone.  Launches of less than eight rounds are dealt to side streams, so that the next ones' groups fill the SMs that
+// one launch leaves idle (64 groups at 256 samples: 0.49 M samples/s one after the other, 1.19 M so; 1,024 samples on
+// ResNet-20 4.3 M, with the fused phases 5.0 M); from eight rounds on what overlap could give is below the launches'
+// own 1-2 %.
+int line_run(LinePlan *p, const LineWork &w, const NoiseStream &ns, int batch_hint, int32_t *err, cudaStream_t st, int64_t *launches)
 {
-    const int64_t per_launch = batch_hint > 0 ? batch_hint : (1ll << 30);
-    for (int64_t done = 0; done < n; done += per_launch) {
-        const int64_t m = std::min(per_launch, n - done);
-        LineParams q = p->base;
-        q.x = d_x;
-        q.ns = ns;
-        q.ns.first_sample = ns.first_sample + done;
-        q.n_samples = (int32_t)m;
-        q.n_groups = (int32_t)((m + kG - 1) / kG);
-        q.counts = d_counts;
-        q.logits = d_logits ? d_logits + (size_t)done * p->n_classes : nullptr;
-        int rc = line_launch(p, q, st);
+    LineParams q = p->base;
+    q.ns = ns;
+    q.err = err;
+    q.phase_sel = w.phase_sel;
+    auto groups = [](int64_t n) { return (int32_t)((n + kG - 1) / kG); };
+    if (batch_hint <= 0) {
+        q.x = w.x;
+        q.image_id0 = w.image_id0;
+        q.counts = w.counts;
+        q.logits = w.logits;
+        q.n_sel = (int32_t)w.n_sel; q.n_est = (int32_t)w.n_est;
+        q.groups_sel = groups(w.n_sel); q.groups_est = groups(w.n_est);
+        const int64_t n = (int64_t)w.n_images * ((int64_t)q.groups_sel + q.groups_est);
+        if (n == 0) return ISC_OK;
+        if (n >= (1ll << 31)) return ISC_ERR_ARG;            // callers cut their images into launches far below this
+        q.n_groups = (int32_t)n;
         *launches += 1;
+        return line_launch(p, q, st);
+    }
+    const int64_t total = ((w.n_sel + batch_hint - 1) / batch_hint + (w.n_est + batch_hint - 1) / batch_hint) * w.n_images;
+    const bool side = total > 1 && batch_hint < 8 * kG * p->sm_count;
+    if (side) {
+        int rc = line_fork(p, st);
         if (rc) return rc;
     }
-    return ISC_OK;
+    int rc = ISC_OK;
+    int64_t at = 0;
+    for (int i = 0; i < w.n_images && rc == ISC_OK; ++i)
+        for (int ph = w.n_sel ? 0 : 1; ph < 2 && rc == ISC_OK; ++ph) {
+            const int64_t n = ph == 0 ? w.n_sel : w.n_est;
+            for (int64_t done = 0; done < n && rc == ISC_OK; done += batch_hint, ++at) {
+                const int64_t m = std::min<int64_t>(batch_hint, n - done);
+                q.x = w.x + (size_t)i * (size_t)(p->in_c * p->in_h * p->in_w);
+                q.image_id0 = w.image_id0 + (uint64_t)i;
+                q.counts = w.counts + (size_t)(w.n_sel ? 2 * i + ph : i) * p->n_classes;
+                q.logits = w.logits ? w.logits + (size_t)done * p->n_classes : nullptr;
+                q.n_sel = 0; q.groups_sel = 0;
+                q.n_est = (int32_t)m; q.groups_est = groups(m);
+                q.ns.ctr3_fixed = ph == 0 ? (uint32_t)w.phase_sel : ns.ctr3_fixed;
+                q.ns.first_sample = (ph == 0 ? 0 : ns.first_sample) + done;
+                q.n_groups = q.groups_est;
+                rc = line_launch(p, q, side ? p->side[at % kSideStreams] : st);
+                *launches += 1;
+            }
+        }
+    if (side) {
+        const int rj = line_join(p, st);
+        if (rc == ISC_OK) rc = rj;
+    }
+    return rc;
 }
 
-int line_check(LinePlan *p)
+// The error word of a launch, read back by the caller after the stream has been synchronised.
+int line_status(int32_t e)
+{
+    if (e == 0) return ISC_OK;
+    if (getenv("ISC_PLAN_DEBUG")) fprintf(stderr, "line engine: wait %d on barrier %d parity %d expired in CTA %d\n", e & 0xFF, (e >> 8) & 0xFFF, (e >> 20) & 1, (int)((unsigned)e >> 21));
+    return ISC_ERR_TIMEOUT;
+}
+
+// The same for the launches that use the plan's own error word, which is cleared.
+static int line_check(LinePlan *p)
 {
     int32_t e = 0;
     if (cudaMemcpy(&e, p->d_err, sizeof(e), cudaMemcpyDeviceToHost) != cudaSuccess) { cudaGetLastError(); return ISC_ERR_CUDA; }
-    if (e != 0) {
-        if (getenv("ISC_PLAN_DEBUG")) fprintf(stderr, "line engine: wait %d on barrier %d parity %d expired in CTA %d\n", e & 0xFF, (e >> 8) & 0xFFF, (e >> 20) & 1, (int)((unsigned)e >> 21));
-        cudaMemset(p->d_err, 0, sizeof(e));
-        return ISC_ERR_TIMEOUT;
-    }
-    return ISC_OK;
+    if (e != 0) cudaMemset(p->d_err, 0, sizeof(e));
+    return line_status(e);
 }
 
 int line_wait_probe(LinePlan *p, long long limit_ns, int32_t out[4], cudaStream_t st)
@@ -1879,7 +1994,10 @@ int line_debug_tensor(LinePlan *p, const uint8_t *d_x, const NoiseStream &ns, in
     if (tensor < 0 || tensor >= (int)p->tensors.size() || p->tensors[(size_t)tensor].buffer < 0) return ISC_ERR_UNSUPPORTED;
     const LGeo &t = p->tensors[(size_t)tensor];
     LineParams q = p->base;
-    q.x = d_x; q.ns = ns; q.n_samples = 1; q.n_groups = 1; q.counts = d_counts_scratch; q.logits = nullptr;
+    q.x = d_x; q.ns = ns; q.counts = d_counts_scratch; q.logits = nullptr;
+    q.image_id0 = (unsigned long long)ns.ctr2 | (unsigned long long)(ns.ctr3_fixed >> 16) << 32;
+    q.ns.ctr3_fixed &= 0xFFu;
+    q.n_sel = 0; q.groups_sel = 0; q.n_est = 1; q.groups_est = 1; q.n_groups = 1;
     q.stop_phase = t.producer_phase;
     q.dump_off = p->tensor_off[(size_t)tensor]; q.dump_bytes = t.bytes; q.dump = p->d_dump;
     int rc = line_launch(p, q, st);

@@ -21,20 +21,31 @@ void line_free(LinePlan *p);
 int line_plan_probe(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_w, int n_classes, int *rule,
                     uint32_t *smem_bytes);
 
-// Runs samples first..first+n-1 (ns.first_sample = first) and adds their votes to d_counts.
-int line_run(LinePlan *p, const uint8_t *d_x, const NoiseStream &ns, int64_t n, int batch_hint,
-             int32_t *d_counts, int8_t *d_logits, cudaStream_t st, int64_t *launches);
+// One call's samples: `n_images` images, each with n_sel samples 0 .. of phase `phase_sel` and n_est samples
+// ns.first_sample .. of the phase ns.ctr3_fixed.  Votes are added to counts[image][selection, estimation][class], or
+// counts[image][class] when n_sel is 0.  logits: one image, no selection phase.
+struct LineWork {
+    const uint8_t *x;
+    int n_images;
+    uint64_t image_id0;
+    int64_t n_sel, n_est;
+    int32_t phase_sel;
+    int32_t *counts;
+    int8_t *logits;
+};
+// `err` (device): receives a non-zero word if a bounded wait expired; line_status gives its meaning.
+int line_run(LinePlan *p, const LineWork &w, const NoiseStream &ns, int batch_hint, int32_t *err, cudaStream_t st, int64_t *launches);
+int line_status(int32_t err_word);
+// Groups that keep every SM busy once: a launch of many times this loses little in its last round.
+int64_t line_wave_samples(const LinePlan *p);
 
 // Debug read-back: runs one group up to the phase producing model tensor `tensor` and returns that
 // tensor of sample ns.first_sample as [C][H][W] int32 (host).
 int line_debug_tensor(LinePlan *p, const uint8_t *d_x, const NoiseStream &ns, int tensor, int32_t *out_chw,
                       int32_t *d_counts_scratch, cudaStream_t st, int64_t *launches);
 
-// After the stream has been synchronised: ISC_OK, or ISC_ERR_TIMEOUT if a bounded wait expired.
-int line_check(LinePlan *p);
-
 // Failure-path check without a failure: runs the engine's wait code (one thread) on a barrier and a counter that nothing
-// completes, with `limit_ns` as the wait limit.  Returns what line_check returns afterwards (ISC_ERR_TIMEOUT when the
+// completes, with `limit_ns` as the wait limit.  Returns the status of the error word afterwards (ISC_ERR_TIMEOUT when the
 // path works) and out[] = {first wait's result, second wait's result, abort flag, nanoseconds spent}.
 int line_wait_probe(LinePlan *p, long long limit_ns, int32_t out[4], cudaStream_t st);
 
