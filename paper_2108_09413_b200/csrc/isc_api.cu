@@ -262,7 +262,7 @@ int build_generic_engine(isc_model *m)
                 std::vector<int8_t> wp(stem_pack_bytes(G));
                 stem_pack_weights(G, H.w.data(), wp.data());
                 rc = upload(m, wp, &m->wpacks[0]); if (rc) return rc;
-                std::vector<int32_t> c4((size_t)G.coutp * 4);
+                std::vector<int32_t> c4((size_t)igemm_padded_cout(G) * 4);
                 m->tc_fast[0] = igemm_constants(G, bias.data(), mult.data(), shift.data(), c4.data(), false, nullptr) ? 1 : 0;
                 rc = upload(m, c4, &m->tc_cst[0]); if (rc) return rc;
             }
@@ -270,7 +270,7 @@ int build_generic_engine(isc_model *m)
                 std::vector<int8_t> wp(igemm_pack_bytes(G));
                 igemm_pack_weights(G, H.w.data(), wp.data());
                 rc = upload(m, wp, &m->wpacks[(size_t)i]); if (rc) return rc;
-                std::vector<int32_t> c4((size_t)G.coutp * 4);
+                std::vector<int32_t> c4((size_t)igemm_padded_cout(G) * 4);
                 m->tc_fast[(size_t)i] = igemm_constants(G, bias.data(), mult.data(), shift.data(), c4.data(), H.d.res_tensor >= 0, &m->tc_resk[(size_t)i]) ? 1 : 0;
                 rc = upload(m, c4, &m->tc_cst[(size_t)i]); if (rc) return rc;
                 m->has_tc = true;
@@ -430,7 +430,7 @@ int generic_forward(isc_model *m, const uint8_t *d_x, const NoiseStream &ns, int
         if (i == 0 && tensor_cores && m->wpacks[0])
             e = launch_stem_conv(G, m->wpacks[0], m->tc_cst[0], m->tc_fast[0] != 0, d_x, m->in_c, ns, batch, out, d_err, st);
         else if (i == 0) e = launch_first_conv(G, d_x, m->in_c, ns, batch, out, st);
-        else if (tensor_cores && m->wpacks[(size_t)i]) e = launch_igemm_conv(G, m->wpacks[(size_t)i], m->tc_cst[(size_t)i], m->tc_fast[(size_t)i] != 0, m->tc_resk[(size_t)i], batch, in, res, out, d_err, st, false, m->opt_tensor_copy != 0);
+        else if (tensor_cores && m->wpacks[(size_t)i] && igemm_fits(G, batch)) e = launch_igemm_conv(G, m->wpacks[(size_t)i], m->tc_cst[(size_t)i], m->tc_fast[(size_t)i] != 0, m->tc_resk[(size_t)i], batch, in, res, out, d_err, st, false, m->opt_tensor_copy != 0);
         else if (L.op == ISC_CONV2D || L.op == ISC_FC) e = launch_conv(G, batch, in, res, out, st);
         else if (L.op == ISC_GAVGPOOL) e = launch_gavgpool(G, batch, in, out, st);
         else e = launch_maxpool(G, batch, in, out, st);
@@ -459,6 +459,8 @@ int layerwise_counts(isc_model *m, const uint8_t *d_x, uint64_t seed, uint64_t i
     const size_t per = std::max<size_t>(generic_bytes_per_sample(m), 1);
     cap = std::min<int64_t>(cap, std::max<int64_t>(1, (int64_t)((3ull << 30) / per)));
     cap = std::min<int64_t>(cap, 32768);
+    if (m->last_engine == 2)                                // the tensor-core kernels' offsets are 32-bit
+        for (size_t b : m->buf_bytes) cap = std::min<int64_t>(cap, std::max<int64_t>(1, (int64_t)(((1ull << 31) - 1) / std::max<size_t>(b, 1))));
     const int batch_alloc = (int)std::min<int64_t>(cap, std::max<int64_t>(n, 1));
     int rc = ensure_workspace(m, batch_alloc);
     if (rc) return rc;

@@ -5,10 +5,10 @@
 //
 //   D[pixel, cout] = sum over (tap, cin) of A[pixel, (tap, cin)] * W[cout, (tap, cin)]
 //
-// A tile is 128 output pixels x N output channels (N = 64, 128 or 256) whose int32 accumulators live in tensor
+// A tile is 128 output pixels x N output channels (N a multiple of 16, at most 256) whose int32 accumulators live in tensor
 // memory.  The kernel is persistent (one CTA per SM, tiles dealt round-robin) and its warps have fixed roles that
 // meet only at mbarriers:
-//   * four warps gather operand rows: per reduction block (64 input channels of one filter tap) a lane issues four
+//   * four warps gather operand rows: per reduction block (four columns of 16 input channels of a filter tap) a lane issues four
 //     asynchronous 16-byte copies (through L1) into the K-major core-matrix layout (four lanes read one pixel's 64 bytes) whose
 //     completion arrives on the stage's barrier; a pixel outside the image is copied from a run of the input
 //     zero-point kept behind the repacked weights;
@@ -59,12 +59,14 @@ struct IgemmParams {
     alignas(64) CUtensorMap tmap_a;          // the input as (16 bytes, pixel, 16-byte column of the channels): see tma_a
     GLayer L;
     int tma_a;                               // 1 x 1 stride 1: the operand rows arrive by one tensor copy per block, the gather warps idle
-    int batch, n_tile, tmem_cols, stages;
+    int batch, n_tile, tiles_n, acc_stride, tmem_cols, stages;     // acc_stride: tensor-memory columns from one accumulator to the other
+    int units, n_blocks;                     // 16-byte columns of the reduction (filter tap, 16 input channels); blocks of four of them
     uint32_t scratch_off;                    // the epilogue warps' row scratch within the dynamic shared memory
     uint32_t m_total, tiles_m;               // batch * hout * wout (< 2^31); tiles of 128 of them
     const int8_t *in, *res;
     int8_t *out;
-    const int8_t *wpack;                     // [cout tile][tap][cin block][4 K columns][n_tile rows][16 bytes]
+    const int8_t *wpack;                     // [cout tile][block][4 K columns][n_tile rows][16 bytes]
+    const int8_t *zp_run;                    // 64 bytes of the input zero-point: the operand row of a pixel outside the image
     const int4 *cst;                         // per output channel: folded bias, multiplier, rounding addend, shift - 1
     int fast_requant, fast_residual, lo;     // every shift >= 2; residual rescale by 2^-31 or 2^-32; lower clamp
     uint32_t res_m2, res_k8;                 // residual multiplier and addend in the 2^-32 form; offset of the two-instruction form
@@ -212,6 +214,10 @@ struct EpiCtx {
     const volatile int *abort_flag;
 };
 
+// Bytes from one row of an epilogue warp's scratch to the next: an odd number of 16-byte columns, so that neither the
+// row-wise nor the coalesced access has bank conflicts.
+__host__ __device__ __forceinline__ uint32_t epi_row_stride(int n_tile) { return (((uint32_t)n_tile >> 4) | 1u) << 4; }
+
 // The epilogue of k_igemm.  Warp w owns lanes 32 (w mod 4) .. +31 of an accumulator (= 32 tile rows) and all N
 // columns; team w / 4 takes every other tile of the CTA (accumulator `team`).  A thread requantises its own row in
 // place in a per-warp scratch area in shared memory (row stride N + 16 bytes: conflict-free for the row-wise and
@@ -220,14 +226,15 @@ struct EpiCtx {
 // space that has just been read, so memory traffic runs under the arithmetic of the following columns.
 // kMode 0: 64-bit requantisation (any shift), 1: 32-bit form, 2 / 3: 32-bit form with the residual add (3: its
 // two-instruction form).
-template <int kMode>
+// kWhole: every tile has n_tile valid columns and n_tile is a multiple of 64.
+template <int kMode, bool kWhole>
 __device__ __forceinline__ bool epilogue_role(const IgemmParams &p, const EpiCtx &c)
 {
     const GLayer &L = p.L;
     const int warp = c.warp, lane = c.lane, n_tile = p.n_tile, tiles_n = c.tiles_n;
     const int q = warp & 3, team = warp / kEpiWarps;
     const uint32_t lane_base = (uint32_t)(q * 32) << 16;
-    const uint32_t row_stride = (uint32_t)n_tile + 16u;
+    const uint32_t row_stride = epi_row_stride(n_tile);
     const uint32_t scr0 = c.sbase + p.scratch_off + (uint32_t)warp * 32u * row_stride;
     const uint32_t scr_row = scr0 + (uint32_t)lane * row_stride;
     // coalesced access to 64 columns of the 32 rows: four lanes per row, eight rows per instruction
@@ -242,7 +249,9 @@ __device__ __forceinline__ bool epilogue_role(const IgemmParams &p, const EpiCtx
         rows = m0 < p.m_total ? min(32u, p.m_total - m0) : 0u;
         return base + (size_t)(m0 + (uint32_t)crow) * L.coutp + (int)(t - m_idx * tiles_n) * n_tile + cchunk * 16;
     };
-    auto residual_fetch = [&](const int8_t *src, uint32_t rows, int c0) {
+    auto tile_cols = [&](uint32_t t) { return kWhole ? n_tile : min(n_tile, L.coutp - (int)(t % (uint32_t)tiles_n) * n_tile); };       // a multiple of 16
+    auto residual_fetch = [&](const int8_t *src, uint32_t rows, int c0, int n_cols) {
+        if (!kWhole && c0 + cchunk * 16 >= n_cols) return;
 #pragma unroll
         for (int k = 0; k < 4; ++k)
             if ((uint32_t)(8 * k + crow) < rows) cp_async16(scr_co + (uint32_t)(8 * k) * row_stride + (uint32_t)c0, src + (size_t)k * co_step + c0);
@@ -253,7 +262,7 @@ __device__ __forceinline__ bool epilogue_role(const IgemmParams &p, const EpiCtx
     if (kMode >= 2 && t < c.n_tiles) {
         uint32_t rows;
         const int8_t *src = tile_ptr(p.res, t, rows);
-        for (int c0 = 0; c0 < n_tile; c0 += 64) residual_fetch(src, rows, c0);
+        for (int c0 = 0; c0 < n_tile; c0 += 64) residual_fetch(src, rows, c0, tile_cols(t));
     }
     for (int au = 0; t < c.n_tiles; t += t_step, ++au) {
         const uint32_t m_idx = t / (uint32_t)tiles_n;
@@ -270,13 +279,15 @@ __device__ __forceinline__ bool epilogue_role(const IgemmParams &p, const EpiCtx
             return false;
         }
         tc_fence_after();
-        const uint32_t acc_base = c.tmem + lane_base + (uint32_t)(team * n_tile);
+        const int n_cols = tile_cols(t), n_cols_next = res_next ? tile_cols(t + t_step) : 0;
+        const uint32_t acc_base = c.tmem + lane_base + (uint32_t)(team * p.acc_stride);
         const uint32_t cst0 = c.cst_s + (uint32_t)n0 * 16u;
         // 32 columns per step, the accumulators of the next step requested before this step's arithmetic
         auto step = [&](int (&acc)[2][16], int c0) {
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int cc = c0 + 16 * h;
+                if (!kWhole && h == 1 && cc >= n_cols) break;
                 uint4 v;
                 if (kMode == 3) {
                     v = requant16_fast<2>(acc[h], cst0 + (uint32_t)cc * 16u, ld_shared_v4(scr_row + (uint32_t)cc), p.res_m2, 0ll, p.res_k8, p.lo);
@@ -295,33 +306,39 @@ __device__ __forceinline__ bool epilogue_role(const IgemmParams &p, const EpiCtx
         int acc_a[2][16], acc_b[2][16];
         tmem_ld32_issue(acc_base, acc_a);
 #pragma unroll 1
-        for (int c0 = 0; c0 < n_tile; c0 += 64) {                   // N is a multiple of 64
+        for (int c0 = 0; c0 < n_cols; c0 += 64) {
+            const bool second = kWhole || c0 + 32 < n_cols, more = c0 + 64 < n_cols;
             tmem_ld32_wait(acc_a);
-            tmem_ld32_issue(acc_base + (uint32_t)c0 + 32u, acc_b);
+            if (second) tmem_ld32_issue(acc_base + (uint32_t)c0 + 32u, acc_b);
             step(acc_a, c0);
-            tmem_ld32_wait(acc_b);
-            if (c0 + 64 < n_tile) {
+            if (second) tmem_ld32_wait(acc_b);
+            if (more) {
                 tmem_ld32_issue(acc_base + (uint32_t)c0 + 64u, acc_a);
             } else {
                 tc_fence_before();
                 mbar_arrive(c.acc_free + 8u * (uint32_t)team);      // the accumulator is in registers: the next tile may overwrite it
             }
-            step(acc_b, c0 + 32);
+            if (second) step(acc_b, c0 + 32);
             __syncwarp();
+            const bool mine = kWhole || c0 + cchunk * 16 < n_cols;            // a row holds the tile's columns and no more
             uint4 v[4];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) v[k] = ld_shared_v4(scr_co + (uint32_t)(8 * k) * row_stride + (uint32_t)c0);
+            for (int k = 0; k < 4; ++k) v[k] = ld_shared_v4(mine ? scr_co + (uint32_t)(8 * k) * row_stride + (uint32_t)c0 : scr0);
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-                if ((uint32_t)(8 * k + crow) < rows) *reinterpret_cast<uint4 *>(dst + (size_t)k * co_step + c0) = v[k];
+                if (mine && (uint32_t)(8 * k + crow) < rows) *reinterpret_cast<uint4 *>(dst + (size_t)k * co_step + c0) = v[k];
             __syncwarp();
-            if (res_next) residual_fetch(res_next, rows_next, c0);
+            if (res_next) residual_fetch(res_next, rows_next, c0, n_cols_next);
         }
+        for (int c0 = (n_cols + 63) & ~63; !kWhole && c0 < n_cols_next; c0 += 64) residual_fetch(res_next, rows_next, c0, n_cols_next);
     }
     cp_async_wait_all();
     return true;
 }
 
+// kWhole: input channels and output tiles are multiples of 64 (what the wide bottleneck networks consist of); the other
+// form takes any layer.  Two kernels, because the general form's masks cost registers and a tenth of the speed.
+template <bool kWhole>
 __global__ void __launch_bounds__(kGemmThreads, 1) k_igemm(const __grid_constant__ IgemmParams p)
 {
     extern __shared__ __align__(128) uint8_t smem[];            // operand stages | requantisation constants | epilogue scratch
@@ -340,7 +357,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_igemm(const __grid_constant
         abort_s = 0;
     }
     if (warp == 0) tmem_alloc(smem_u32(&tmem_base_s), (uint32_t)p.tmem_cols);
-    for (int i = tid; i < L.coutp; i += kGemmThreads) cst_s[i] = __ldg(p.cst + i);
+    for (int i = tid; i < p.tiles_n * n_tile; i += kGemmThreads) cst_s[i] = __ldg(p.cst + i);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_proxy_async();
     tc_fence_before();
@@ -349,9 +366,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_igemm(const __grid_constant
     const uint32_t tmem = tmem_base_s;
 
     // tiles in m-major order (the CTAs of one wave share operand rows in L2), dealt round-robin to the CTAs
-    const int tiles_n = L.coutp / n_tile;
+    const int tiles_n = p.tiles_n;
     const uint32_t n_tiles = p.tiles_m * (uint32_t)tiles_n, grid_n = gridDim.x;
-    const int cblocks = L.cinp / kBlockK, nkb = L.kh * L.kw * cblocks;
+    const int cblocks = L.cinp / kBlockK, nkb = p.n_blocks;
     bool ok = true;
 
     if (warp < kAllEpiWarps) {
@@ -361,17 +378,17 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_igemm(const __grid_constant
         c.acc_full = smem_u32(&bar_acc_full[0]); c.acc_free = smem_u32(&bar_acc_free[0]);
         c.abort_flag = &abort_s;
         const bool fast = p.fast_requant && (!p.res || p.fast_residual);
-        if (fast && p.res && p.res_short) ok = epilogue_role<3>(p, c);
-        else if (fast && p.res) ok = epilogue_role<2>(p, c);
-        else if (fast) ok = epilogue_role<1>(p, c);
-        else ok = epilogue_role<0>(p, c);
+        if (fast && p.res && p.res_short) ok = epilogue_role<3, kWhole>(p, c);
+        else if (fast && p.res) ok = epilogue_role<2, kWhole>(p, c);
+        else if (fast) ok = epilogue_role<1, kWhole>(p, c);
+        else ok = epilogue_role<0, kWhole>(p, c);
     } else if (warp < kAllEpiWarps + kGatherWarps) {
         // ---- operand rows: per reduction block a warp copies 32 tile rows x 64 bytes with four asynchronous 16-byte
         // copies per lane (lane = 16-byte column x row within a group of eight, so that an instruction reads whole
         // 64-byte rows) whose completion arrives on the stage's barrier.  A row outside the image is copied from a
         // 64-byte run of the input zero-point that follows the repacked weights, so every row takes the same path.
         const int gw = warp - kAllEpiWarps, chunk = lane & 3, rsub = lane >> 2;
-        const int8_t *zp_src = p.wpack + (size_t)L.coutp * (size_t)(L.kh * L.kw) * (size_t)L.cinp + chunk * 16;
+        const int8_t *zp_src = p.zp_run + chunk * 16;
         const int8_t *in_c = p.in + chunk * 16;
         // K-major core matrices: 16-byte column j of row r at j * (128 rows * 16) + r * 16
         const uint32_t dst0 = sbase + (uint32_t)chunk * 2048u + (uint32_t)(32 * gw + rsub) * 16u;
@@ -390,6 +407,32 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_igemm(const __grid_constant
                 iy0[i] = valid ? oy * L.stride - L.pad : -0x100000;             // an invalid row is outside for every tap
                 ix0[i] = ox * L.stride - L.pad;
                 off[i] = (((int)b * L.hin + oy * L.stride - L.pad) * L.win + ix0[i]) * L.cinp;    // the tensor is < 2^31 bytes
+            }
+            if (!kWhole) {
+                // channels no multiple of 64: this lane's column of a block is a tap and 16 channels of its own; columns
+                // beyond the last one meet zero weights
+                const int c16s = L.cinp >> 4;
+                int u = chunk, c16 = chunk % c16s, r = (chunk / c16s) / L.kw, sx = (chunk / c16s) % L.kw;
+                for (int kb = 0; kb < nkb; ++kb, ring.advance(stages)) {
+                    if (ring.use >= 1) {
+                        ok = wait_bar<kHintLoad>(smem_u32(&bar_free[ring.s]), (uint32_t)(ring.use - 1) & 1u, &abort_s);
+                        if (!ok) break;
+                    }
+                    const uint32_t dst = dst0 + (uint32_t)ring.s * stage_bytes;
+                    const int add = (r * L.win + sx) * L.cinp + c16 * 16;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const bool inside = (unsigned)(iy0[i] + r) < (unsigned)L.hin && (unsigned)(ix0[i] + sx) < (unsigned)L.win && u < p.units;
+                        cp_async16_cached(dst + (uint32_t)i * 128u, inside ? p.in + (off[i] + add) : zp_src);
+                    }
+                    cp_async_arrive(smem_u32(&bar_full[ring.s]));
+                    u += 4; c16 += 4;
+                    while (c16 >= c16s) {
+                        c16 -= c16s;
+                        if (++sx == L.kw) { sx = 0; ++r; }
+                    }
+                }
+                continue;
             }
             for (int tap = 0, r = 0, sx = 0; tap < L.kh * L.kw && ok; ++tap, sx = (sx + 1 == L.kw) ? 0 : sx + 1, r += (sx == 0)) {
                 const int tap_off = (r * L.win + sx) * L.cinp;
@@ -430,9 +473,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_igemm(const __grid_constant
                     const uint32_t stage = sbase + (uint32_t)ring.s * stage_bytes;
 #pragma unroll
                     for (int k2 = 0; k2 < 2; ++k2) {
+                        if (!kWhole && k2 == 1 && 4 * kb + 2 >= p.units) break;            // the last block's second half is padding
                         const uint64_t ad = make_desc(stage + (uint32_t)k2 * 4096u, 2048u, 128u);
                         const uint64_t bd = make_desc(stage + a_bytes + (uint32_t)k2 * 2u * (uint32_t)n_tile * 16u, (uint32_t)n_tile * 16u, 128u);
-                        mma_i8(tmem + (uint32_t)(buf * n_tile), ad, bd, idesc, (kb > 0 || k2 > 0) ? 1u : 0u);
+                        mma_i8(tmem + (uint32_t)(buf * p.acc_stride), ad, bd, idesc, (kb > 0 || k2 > 0) ? 1u : 0u);
                     }
                     commit_to(smem_u32(&bar_free[ring.s]));
                 }
@@ -671,36 +715,54 @@ __global__ void __launch_bounds__(kStemThreads, 2) k_stem(const __grid_constant_
 
 // ------------------------------------------------------------------ host side
 
+// Output channels in as few tiles of at most 256 as possible, all of the same width (a multiple of 16; the last one may
+// be partly padding).  Every convolution and FC layer fits; pools do not.
 int igemm_tile_n(const GLayer &G)
 {
-    if ((G.op != ISC_CONV2D && G.op != ISC_FC) || G.cinp % kBlockK != 0 || G.cin != G.cinp) return 0;
-    if (G.coutp % 256 == 0) return 256;
-    if (G.coutp % 128 == 0) return 128;
-    if (G.coutp % 64 == 0) return 64;
-    return 0;
+    if (G.op != ISC_CONV2D && G.op != ISC_FC) return 0;
+    const int tiles = (G.coutp + 255) / 256;
+    return ((G.coutp + tiles - 1) / tiles + 15) & ~15;
 }
+
+namespace {
+
+int igemm_tiles(const GLayer &G) { return (G.coutp + 255) / 256; }
+int igemm_units(const GLayer &G) { return G.kh * G.kw * (G.cinp / 16); }
+int igemm_blocks(const GLayer &G) { return (igemm_units(G) + 3) / 4; }
+
+}  // namespace
+
+// constants of that many channels: the last tile's padding included
+int igemm_padded_cout(const GLayer &G) { return igemm_tiles(G) * igemm_tile_n(G); }
 
 // the repacked weights, then 64 bytes of the input zero-point (the operand row of a pixel outside the image)
 size_t igemm_pack_bytes(const GLayer &G)
 {
-    return (size_t)G.coutp * (size_t)(G.kh * G.kw) * (size_t)G.cinp + kBlockK;
+    return (size_t)igemm_padded_cout(G) * (size_t)igemm_blocks(G) * kBlockK + kBlockK;
 }
 
-// w: [cout][cin][kh][kw] as the model gives it -> [cout tile][tap][cin block][4 columns of 16 channels][n_tile rows][16]
+// w: [cout][cin][kh][kw] as the model gives it -> [cout tile][block][4 columns][n_tile rows][16]; column u of the
+// reduction is 16 input channels of one filter tap, tap-major
 void igemm_pack_weights(const GLayer &G, const int8_t *w, int8_t *out)
 {
-    const int n_tile = igemm_tile_n(G), taps = G.kh * G.kw, cblocks = G.cinp / kBlockK;
+    const int n_tile = igemm_tile_n(G), taps = G.kh * G.kw, c16s = G.cinp / 16, units = igemm_units(G), columns = 4 * igemm_blocks(G);
     size_t at = 0;
-    for (int t = 0; t < G.coutp / n_tile; ++t)
-        for (int tap = 0; tap < taps; ++tap)
-            for (int cb = 0; cb < cblocks; ++cb)
-                for (int j = 0; j < 4; ++j)
-                    for (int n = 0; n < n_tile; ++n)
-                        for (int e = 0; e < 16; ++e, ++at) {
-                            const int oc = t * n_tile + n, ci = cb * kBlockK + j * 16 + e;
-                            out[at] = (oc < G.cout && ci < G.cin) ? w[((size_t)oc * G.cin + ci) * taps + tap] : (int8_t)0;
-                        }
+    for (int t = 0; t < igemm_tiles(G); ++t)
+        for (int u = 0; u < columns; ++u) {
+            const int tap = u / c16s, c0 = (u - tap * c16s) * 16;
+            for (int n = 0; n < n_tile; ++n)
+                for (int e = 0; e < 16; ++e, ++at) {
+                    const int oc = t * n_tile + n, ci = c0 + e;
+                    out[at] = (u < units && oc < G.cout && ci < G.cin) ? w[((size_t)oc * G.cin + ci) * taps + tap] : (int8_t)0;
+                }
+        }
     for (int e = 0; e < kBlockK; ++e) out[at + e] = (int8_t)G.zp_in;
+}
+
+// 32-bit row and byte offsets inside the kernel
+bool igemm_fits(const GLayer &G, int64_t batch)
+{
+    return batch * G.hout * G.wout * igemm_tiles(G) < (1ll << 31) - 512 && batch * G.hin * G.win * G.cinp < (1ll << 31);
 }
 
 // The residual term F(u) = floor((u * m2 + R2) / 2^32), u = r + 128 in 0..255 (see requant16_fast), as
@@ -734,19 +796,21 @@ bool residual_short_form(int res_mult, int res_shift, int zp_res, uint32_t *k8, 
 bool igemm_constants(const GLayer &G, const int32_t *bias_folded, const int32_t *mult, const int32_t *shift, int32_t *out4,
                      bool has_residual, uint32_t *res_k8)
 {
+    // channels beyond the layer's own (padding of the tensor and of the last tile) come out as zero
     bool fast = true;
-    for (int o = 0; o < G.coutp; ++o) fast = fast && shift[o] - 1 >= 1;
+    for (int o = 0; o < G.cout; ++o) fast = fast && shift[o] - 1 >= 1;
     uint32_t k8 = 0;
     int32_t c_res = 0;
     bool short_form = fast && has_residual && residual_short_form(G.res_mult, G.res_shift, G.zp_res, &k8, &c_res);
-    for (int o = 0; o < G.coutp && short_form; ++o) {
+    for (int o = 0; o < G.cout && short_form; ++o) {
         const int s = shift[o] - 1;
         const long long add = (1ll << (s - 1)) + ((long long)G.zp_out - c_res) * (1ll << s);
         short_form = add > -(1ll << 31) && add < (1ll << 31);
     }
     if (!short_form) c_res = 0;
     if (res_k8) *res_k8 = short_form ? k8 : 0xFFFFFFFFu;
-    for (int o = 0; o < G.coutp; ++o) {
+    memset(out4, 0, sizeof(int32_t) * 4 * (size_t)igemm_padded_cout(G));
+    for (int o = 0; o < G.cout; ++o) {
         const int s = shift[o] - 1;
         out4[4 * o + 0] = bias_folded[o];
         out4[4 * o + 1] = mult[o];
@@ -807,16 +871,21 @@ cudaError_t launch_igemm_conv(const GLayer &G, const int8_t *wpack, const int32_
     p.batch = batch;
     p.n_tile = igemm_tile_n(G);
     if (p.n_tile == 0) return cudaErrorInvalidValue;
-    p.tmem_cols = 2 * p.n_tile;                                  // two accumulators: 128, 256 or 512 columns
-    const long long m_total = (long long)batch * G.hout * G.wout;
-    if (m_total >= (1ll << 31) / (G.coutp / p.n_tile) || (long long)batch * G.hin * G.win * G.cinp >= (1ll << 31)) return cudaErrorInvalidValue;
-    p.m_total = (uint32_t)m_total;
+    p.tiles_n = igemm_tiles(G);
+    p.units = igemm_units(G);
+    p.n_blocks = igemm_blocks(G);
+    p.acc_stride = (p.n_tile + 31) & ~31;                        // the epilogue loads 32 columns at a time
+    p.tmem_cols = 64;
+    while (p.tmem_cols < 2 * p.acc_stride) p.tmem_cols <<= 1;
+    if (!igemm_fits(G, batch)) return cudaErrorInvalidValue;
+    p.zp_run = wpack + igemm_pack_bytes(G) - kBlockK;
+    p.m_total = (uint32_t)((long long)batch * G.hout * G.wout);
     p.tiles_m = (p.m_total + kTileM - 1) / kTileM;
     p.in = in; p.res = res; p.out = out; p.wpack = wpack; p.err = err;
     if (p.tiles_m == 0) return cudaSuccess;
     // as many operand stages as fit beside the constants, at most kMaxStages
-    const size_t stage_bytes = (size_t)kTileM * kBlockK + (size_t)p.n_tile * kBlockK, cst_bytes = (size_t)G.coutp * 16;
-    const size_t scratch_bytes = (size_t)kAllEpiWarps * 32 * ((size_t)p.n_tile / (kEpiWarps / 4) + 16);
+    const size_t stage_bytes = (size_t)kTileM * kBlockK + (size_t)p.n_tile * kBlockK, cst_bytes = (size_t)p.tiles_n * p.n_tile * 16;
+    const size_t scratch_bytes = (size_t)kAllEpiWarps * 32 * epi_row_stride(p.n_tile);
     const size_t smem_limit = 226 * 1024;
     if (cst_bytes + scratch_bytes + 2 * stage_bytes > smem_limit) return cudaErrorInvalidValue;
     p.stages = (int)std::min<size_t>(kMaxStages, (smem_limit - cst_bytes - scratch_bytes) / stage_bytes);
@@ -827,13 +896,16 @@ cudaError_t launch_igemm_conv(const GLayer &G, const int8_t *wpack, const int32_
         int dev = 0;
         cudaError_t e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_limit);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_limit);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_limit);
         if (e != cudaSuccess) { n_sms = 0; return e; }
     }
     // persistent: one CTA per SM (shared memory and the 512 tensor-memory columns allow no second one at N = 256)
-    const uint32_t n_tiles = p.tiles_m * (uint32_t)(G.coutp / p.n_tile);
+    const uint32_t n_tiles = p.tiles_m * (uint32_t)p.tiles_n;
     const unsigned grid = std::min<uint32_t>(n_tiles, (uint32_t)n_sms);
-    k_igemm<<<grid, kGemmThreads, smem, st>>>(p);
+    const bool whole = G.cinp % kBlockK == 0 && p.n_tile % 64 == 0 && G.coutp == p.tiles_n * p.n_tile;
+    if (whole) k_igemm<true><<<grid, kGemmThreads, smem, st>>>(p);
+    else k_igemm<false><<<grid, kGemmThreads, smem, st>>>(p);
     return cudaGetLastError();
 }
 

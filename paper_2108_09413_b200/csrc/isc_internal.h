@@ -66,15 +66,16 @@ cudaError_t launch_votes(const int8_t *logits_nhwc, int cp, int n_classes, int b
                          int8_t *logits_out, cudaStream_t st);
 
 // ---- layer-by-layer tensor-core convolutions (isc_igemm.cu) ----
-// Output-channel tile of the implicit-GEMM kernel for this layer (64, 128 or 256), or 0 when the layer does not fit
-// it (input channels not a multiple of 64, output channels not a multiple of 64, pools).
+// Output-channel tile of the implicit-GEMM kernel for this layer (a multiple of 16 up to 256), or 0 for pools.
 int igemm_tile_n(const GLayer &G);
+int igemm_padded_cout(const GLayer &G);          // output channels with the last tile's padding: entries of the constants
+bool igemm_fits(const GLayer &G, int64_t batch);  // the batch's tensors are within the kernel's 32-bit offsets
 size_t igemm_pack_bytes(const GLayer &G);
 void igemm_pack_weights(const GLayer &G, const int8_t *w_oihw, int8_t *out);
 // The residual term F(u) = floor((u * m2 + R2) / 2^32), u = r + 128 in 0..255, of the 32-bit epilogues as
 // hi32((256 k + u) * m2) - c: the smallest k < 4096 for which the two agree on all 256 inputs (*k8 = 256 k), or false.
 bool residual_short_form(int res_mult, int res_shift, int zp_res, uint32_t *k8, int32_t *c);
-// Per-channel requantisation constants of the kernel's 32-bit epilogue (4 x int32 per padded output channel); returns
+// Per-channel requantisation constants of the kernel's 32-bit epilogue (4 x int32 for igemm_padded_cout channels); returns
 // whether the layer qualifies for it (every shift >= 2).
 bool igemm_constants(const GLayer &G, const int32_t *bias_folded, const int32_t *mult, const int32_t *shift, int32_t *out4,
                      bool has_residual, uint32_t *res_k8);
