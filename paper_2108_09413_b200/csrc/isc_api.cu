@@ -47,6 +47,7 @@ struct isc_model {
     std::vector<GLayer> glayers;
     std::vector<void *> param_allocs;
     std::vector<const int8_t *> wpacks;         // per layer: repacked weights of the tensor-core convolution, or null
+    std::vector<const int8_t *> hpacks;         // per layer: the same for the kernel with resident input tiles, where that takes the layer
     std::vector<const int32_t *> tc_cst;        // per layer: its epilogue constants
     std::vector<char> tc_fast;
     std::vector<uint32_t> tc_resk;           // per layer: offset of the residual term's two-instruction form, or 0xFFFFFFFF
@@ -211,6 +212,7 @@ int build_generic_engine(isc_model *m)
     m->glayers.resize((size_t)n);
     m->wpacks.assign((size_t)n, nullptr);
     m->tc_cst.assign((size_t)n, nullptr);
+    m->hpacks.assign((size_t)n, nullptr);
     m->tc_fast.assign((size_t)n, 0);
     m->tc_resk.assign((size_t)n, 0xFFFFFFFFu);
     for (int i = 0; i < n; ++i) {
@@ -263,17 +265,23 @@ int build_generic_engine(isc_model *m)
                 stem_pack_weights(G, H.w.data(), wp.data());
                 rc = upload(m, wp, &m->wpacks[0]); if (rc) return rc;
                 std::vector<int32_t> c4((size_t)igemm_padded_cout(G) * 4);
-                m->tc_fast[0] = igemm_constants(G, bias.data(), mult.data(), shift.data(), c4.data(), false, nullptr) ? 1 : 0;
+                m->tc_fast[0] = igemm_constants(G, bias.data(), mult.data(), shift.data(), c4.data(), igemm_padded_cout(G), false, nullptr) ? 1 : 0;
                 rc = upload(m, c4, &m->tc_cst[0]); if (rc) return rc;
             }
             if (i > 0 && igemm_tile_n(G)) {                 // the same layer for the tensor-core kernel
                 std::vector<int8_t> wp(igemm_pack_bytes(G));
                 igemm_pack_weights(G, H.w.data(), wp.data());
                 rc = upload(m, wp, &m->wpacks[(size_t)i]); if (rc) return rc;
-                std::vector<int32_t> c4((size_t)igemm_padded_cout(G) * 4);
-                m->tc_fast[(size_t)i] = igemm_constants(G, bias.data(), mult.data(), shift.data(), c4.data(), H.d.res_tensor >= 0, &m->tc_resk[(size_t)i]) ? 1 : 0;
+                const int n_cst = std::max(igemm_padded_cout(G), halo_padded_cout(G));
+                std::vector<int32_t> c4((size_t)n_cst * 4);
+                m->tc_fast[(size_t)i] = igemm_constants(G, bias.data(), mult.data(), shift.data(), c4.data(), n_cst, H.d.res_tensor >= 0, &m->tc_resk[(size_t)i]) ? 1 : 0;
                 rc = upload(m, c4, &m->tc_cst[(size_t)i]); if (rc) return rc;
                 m->has_tc = true;
+                if (halo_fits(G)) {
+                    std::vector<int8_t> hp(halo_pack_bytes(G));
+                    halo_pack(G, H.w.data(), hp.data());
+                    rc = upload(m, hp, &m->hpacks[(size_t)i]); if (rc) return rc;
+                }
             }
         }
         m->glayers[(size_t)i] = G;
@@ -430,6 +438,8 @@ int generic_forward(isc_model *m, const uint8_t *d_x, const NoiseStream &ns, int
         if (i == 0 && tensor_cores && m->wpacks[0])
             e = launch_stem_conv(G, m->wpacks[0], m->tc_cst[0], m->tc_fast[0] != 0, d_x, m->in_c, ns, batch, out, d_err, st);
         else if (i == 0) e = launch_first_conv(G, d_x, m->in_c, ns, batch, out, st);
+        else if (tensor_cores && m->hpacks[(size_t)i] && igemm_fits(G, batch))
+            e = launch_halo_conv(G, m->hpacks[(size_t)i], m->tc_cst[(size_t)i], m->tc_fast[(size_t)i] != 0, m->tc_resk[(size_t)i], batch, in, res, out, d_err, st);
         else if (tensor_cores && m->wpacks[(size_t)i] && igemm_fits(G, batch)) e = launch_igemm_conv(G, m->wpacks[(size_t)i], m->tc_cst[(size_t)i], m->tc_fast[(size_t)i] != 0, m->tc_resk[(size_t)i], batch, in, res, out, d_err, st, false, m->opt_tensor_copy != 0);
         else if (L.op == ISC_CONV2D || L.op == ISC_FC) e = launch_conv(G, batch, in, res, out, st);
         else if (L.op == ISC_GAVGPOOL) e = launch_gavgpool(G, batch, in, out, st);

@@ -33,6 +33,7 @@
 #include <cstdlib>
 #include <cstring>
 
+#include "isc_conv.cuh"
 #include "isc_epilogue.cuh"
 #include "isc_internal.h"
 #include "isc_tc.cuh"
@@ -40,12 +41,12 @@
 namespace isc {
 
 using namespace tc;
+using namespace conv;
 
 namespace {
 
 constexpr int kTileM = 128;
 constexpr int kBlockK = 64;                  // bytes of K per stage: two MMA K-steps
-constexpr unsigned kHintLoad = 20000, kHintEpi = 20000, kHintMma = 20000;      // suspend-time hint of a barrier wait (ns), by role
 constexpr int kMaxStages = 16;
 constexpr int kStemThreads = 256;           // k_stem: two threads per tile row; two CTAs per SM (registers allow no third, nor two of 512 threads)
 constexpr size_t kStemSmemLimit = 108 * 1024;          // dynamic shared memory of k_stem: two CTAs per SM
@@ -53,7 +54,6 @@ constexpr int kEpiWarps = 4, kEpiTeams = 2, kGatherWarps = 4;          // a team
 constexpr int kAllEpiWarps = kEpiWarps * kEpiTeams;
 static_assert(kEpiWarps == 4, "an epilogue warp owns all N columns of its 32 rows");
 constexpr int kGemmThreads = 32 * (kAllEpiWarps + kGatherWarps + 2);      // k_igemm: + the MMA warp + the weights warp
-constexpr unsigned long long kWaitLimitNs = 2000000000ull;
 
 struct IgemmParams {
     alignas(64) CUtensorMap tmap_a;          // the input as (16 bytes, pixel, 16-byte column of the channels): see tma_a
@@ -76,136 +76,6 @@ struct IgemmParams {
     int32_t *err;
 };
 
-__device__ __forceinline__ void mma_i8(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate)
-{
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
-                 ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
-}
-__device__ __forceinline__ void commit_to(uint32_t bar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-
-__device__ __forceinline__ long long mul_wide(int a, int b)
-{
-    long long d;
-    asm("mul.wide.s32 %0, %1, %2;" : "=l"(d) : "r"(a), "r"(b));
-    return d;
-}
-__device__ __forceinline__ long long mad_wide_u(uint32_t a, uint32_t b, long long c)
-{
-    long long d;
-    asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
-    return d;
-}
-
-// 16 accumulators -> 16 int8 outputs with 32-bit arithmetic.  With s = shift - 1 >= 1,
-//   rs((acc + bias) * mult, 31 + shift) + zp_out = (hi32((acc + bias) * mult) + c) >> s,  c = 2^(s-1) + zp_out * 2^s,
-// exactly (the rounding half 2^(31+s) is a multiple of 2^32, so the product's low word cannot change the floor), and
-//   rs((r - zp_res) * res_mult, n) = hi32(u * m2 + R2),  u = r + 128, m2 = res_mult * 2^(32-n), n = 31 or 32,
-// with R2 = (2^(n-1) - (128 + zp_res) * res_mult) * 2^(32-n) (kRes = 1).  kRes = 2 is the same term without the
-// 64-bit addend: hi32((256 k + u) * m2) - c_r for an offset k that the host has checked on all 256 values of u
-// (residual_short_form); 256 k is merged into u by the byte permute that extracts u, and c_r is folded into c.
-// `cst` points at this block's constants in shared memory.
-template <int kRes>
-__device__ __forceinline__ uint4 requant16_fast(const int *acc, uint32_t cst, uint4 rv, uint32_t m2, long long r2, uint32_t k8, int lo)
-{
-    const uint32_t rw[4] = {rv.x ^ 0x80808080u, rv.y ^ 0x80808080u, rv.z ^ 0x80808080u, rv.w ^ 0x80808080u};
-    uint32_t packed[4];
-#pragma unroll
-    for (int g = 0; g < 4; ++g) {
-        int y[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            int4 c;
-            asm("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(c.x), "=r"(c.y), "=r"(c.z), "=r"(c.w) : "r"(cst + (4 * g + k) * 16));
-            int v = (hi32(mul_wide(acc[4 * g + k] + c.x, c.y)) + c.z) >> c.w;
-            if (kRes == 1) v += hi32(mad_wide_u(__byte_perm(rw[g], 0u, 0x4440u | (uint32_t)k), m2, r2));
-            if (kRes == 2) v += hi32(mad_wide_u(__byte_perm(rw[g], k8, 0x7650u | (uint32_t)k), m2, 0ll));
-            y[k] = max(v, lo);
-        }
-        packed[g] = pack4_sat(y[0], y[1], y[2], y[3]);
-    }
-    return make_uint4(packed[0], packed[1], packed[2], packed[3]);
-}
-
-// 32 accumulator columns of this thread's lane, asynchronously; the registers are valid after tmem_ld32_wait(),
-// which names them so that no use can move above it
-__device__ __forceinline__ void tmem_ld32_issue(uint32_t taddr, int (&v)[2][16])
-{
-    tmem_ld16_issue(taddr, v[0]);
-    tmem_ld16_issue(taddr + 16u, v[1]);
-}
-__device__ __forceinline__ void tmem_ld32_wait(int (&v)[2][16])
-{
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(v[0][0]), "+r"(v[0][1]), "+r"(v[0][2]), "+r"(v[0][3]), "+r"(v[0][4]), "+r"(v[0][5]), "+r"(v[0][6]), "+r"(v[0][7]),
-                   "+r"(v[0][8]), "+r"(v[0][9]), "+r"(v[0][10]), "+r"(v[0][11]), "+r"(v[0][12]), "+r"(v[0][13]), "+r"(v[0][14]), "+r"(v[0][15]),
-                   "+r"(v[1][0]), "+r"(v[1][1]), "+r"(v[1][2]), "+r"(v[1][3]), "+r"(v[1][4]), "+r"(v[1][5]), "+r"(v[1][6]), "+r"(v[1][7]),
-                   "+r"(v[1][8]), "+r"(v[1][9]), "+r"(v[1][10]), "+r"(v[1][11]), "+r"(v[1][12]), "+r"(v[1][13]), "+r"(v[1][14]), "+r"(v[1][15])
-                 :: "memory");
-}
-
-// Bounded wait for a phase of an mbarrier; false after the limit (the caller raises the error word).
-__device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity)
-{
-    if (mbar_test(bar, parity)) return true;
-    const unsigned long long t0 = globaltimer();
-    for (int spin = 0;; ++spin) {
-        if (mbar_try(bar, parity)) return true;
-        if ((spin & 7) == 7 && globaltimer() - t0 > kWaitLimitNs) return false;
-    }
-}
-// The same for the roles of k_igemm, which also give up when another role has raised the CTA's abort flag.  With
-// `kHintNs` the wait is parked in hardware for up to that long per attempt instead of polling (the abort flag and
-// the time limit are looked at every eighth attempt).
-template <unsigned kHintNs>
-__device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, const volatile int *abort_flag)
-{
-    if (mbar_test(bar, parity)) return true;
-    const unsigned long long t0 = globaltimer();
-    for (int spin = 0;; ++spin) {
-        if (kHintNs) {
-            // parked in hardware until the phase completes or the hint runs out
-            uint32_t done;
-            asm volatile("{\n\t.reg .pred p;\n\t"
-                         "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-                         "selp.u32 %0, 1, 0, p;\n\t}"
-                         : "=r"(done) : "r"(bar), "r"(parity), "r"(kHintNs) : "memory");
-            if (done) return true;
-        } else if (mbar_try(bar, parity)) {
-            return true;
-        }
-        if ((spin & 7) == 7 && (*abort_flag || globaltimer() - t0 > kWaitLimitNs)) return false;
-    }
-}
-
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-// the same through L1: the taps of a 3 x 3 filter read a pixel's row nine times, and every CTA reads the zero-point run
-__device__ __forceinline__ void cp_async16_cached(uint32_t dst, const void *src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-// one arrival on `bar` (counted in its initial count) once every cp.async this thread has issued so far is complete
-__device__ __forceinline__ void cp_async_arrive(uint32_t bar)
-{
-    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-// all of this thread's copy groups but the newest are complete
-__device__ __forceinline__ void cp_async_wait_one() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
-
-// A stage ring position: index and how many times the ring has wrapped.
-struct Ring {
-    int s = 0, use = 0;
-    __device__ __forceinline__ void advance(int stages) { if (++s == stages) { s = 0; ++use; } }
-};
-
 // What an epilogue warp needs from the kernel's prologue.
 struct EpiCtx {
     uint32_t sbase, tmem, n_tiles, grid_n;
@@ -213,10 +83,6 @@ struct EpiCtx {
     uint32_t cst_s, acc_full, acc_free;       // shared-memory addresses: constants, the two accumulators' barriers
     const volatile int *abort_flag;
 };
-
-// Bytes from one row of an epilogue warp's scratch to the next: an odd number of 16-byte columns, so that neither the
-// row-wise nor the coalesced access has bank conflicts.
-__host__ __device__ __forceinline__ uint32_t epi_row_stride(int n_tile) { return (((uint32_t)n_tile >> 4) | 1u) << 4; }
 
 // The epilogue of k_igemm.  Warp w owns lanes 32 (w mod 4) .. +31 of an accumulator (= 32 tile rows) and all N
 // columns; team w / 4 takes every other tile of the CTA (accumulator `team`).  A thread requantises its own row in
@@ -793,7 +659,7 @@ bool residual_short_form(int res_mult, int res_shift, int zp_res, uint32_t *k8, 
 // condition of the 32-bit form).  `bias_folded`, `mult`, `shift` are the layer's host arrays padded to coutp.  For a
 // layer with a residual operand whose term has the two-instruction form, that form's constant is folded into the
 // rounding addends and *res_k8 is its offset; otherwise *res_k8 = 0xFFFFFFFF.
-bool igemm_constants(const GLayer &G, const int32_t *bias_folded, const int32_t *mult, const int32_t *shift, int32_t *out4,
+bool igemm_constants(const GLayer &G, const int32_t *bias_folded, const int32_t *mult, const int32_t *shift, int32_t *out4, int n_out,
                      bool has_residual, uint32_t *res_k8)
 {
     // channels beyond the layer's own (padding of the tensor and of the last tile) come out as zero
@@ -809,7 +675,7 @@ bool igemm_constants(const GLayer &G, const int32_t *bias_folded, const int32_t 
     }
     if (!short_form) c_res = 0;
     if (res_k8) *res_k8 = short_form ? k8 : 0xFFFFFFFFu;
-    memset(out4, 0, sizeof(int32_t) * 4 * (size_t)igemm_padded_cout(G));
+    memset(out4, 0, sizeof(int32_t) * 4 * (size_t)n_out);
     for (int o = 0; o < G.cout; ++o) {
         const int s = shift[o] - 1;
         out4[4 * o + 0] = bias_folded[o];
