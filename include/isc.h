@@ -170,10 +170,11 @@ int isc_sample_counts(isc_model *m, const uint8_t *x_u8, uint64_t seed, uint64_t
  * service whose device memory is handed out up front by its own pool, a real-time loop
  * that cannot afford the implicit device synchronisation of an allocation, a process
  * running under a memory budget enforced by refusing allocations.  For them this entry
- * point computes the same vote counts as isc_sample_counts with the layer-by-layer
- * kernels, but takes every byte of its device work space (activation buffers, noise
- * table, staged image, counts) from one fixed 32 MiB array that is part of the library
- * image.  It calls no cudaMalloc / cudaFree and no allocating library routine; the model
+ * point computes the same vote counts as isc_sample_counts, but takes every byte of its
+ * device work space (activation buffers, noise table, staged image, counts) from one fixed
+ * 32 MiB array that is part of the library image.  The kernels are those isc_sample_counts
+ * takes: the resident engine where the model fits it (it needs no activation buffers), else
+ * the layer-by-layer ones, with tensor cores unless the "engine" option is 1.  It calls no cudaMalloc / cudaFree and no allocating library routine; the model
  * handle must have been loaded beforehand (loading does allocate).  Each GPU on which the
  * library is loaded holds that array until the process exits.
  *
@@ -329,7 +330,8 @@ int isc_debug_residual_form(int32_t res_mult, int32_t res_shift, int32_t zp_res,
  *              output channels are multiples of 64, 3 = the line-tiled
  *              shared-memory-resident tensor-core kernel (2 and 3 give
  *              ISC_ERR_UNSUPPORTED at the next call if the model does not fit).
- * isc_get_info reads back: "engine" (the engine the last call used), "gpu_launches"
+ * isc_get_info reads back: "engine" (the engine the last call used; 1 after every
+ * isc_sample_counts_static, whichever kernels it took), "gpu_launches"
  * (kernel launches issued by this handle so far), "macs_per_sample",
  * "has_line_engine" (1 if the model fits engine 3), "has_tensor_core_layers" (1 if
  * engine 2 has a layer to run) and, for engine 3, "cycles_fill",

@@ -215,15 +215,15 @@ int32_t table_quantile(const std::vector<uint32_t> &cum, uint32_t p_fx)
 }  // namespace
 
 int32_t decide_certify_integer(const int32_t *counts0, const int32_t *counts, int n_classes, int64_t N, double sigma,
-                               double alpha, bool two_sided, int32_t *q, int64_t *q_squared, const std::vector<uint32_t> *table)
+                               double alpha, bool two_sided, int32_t *q, int64_t *q_squared, const uint32_t *table, size_t n_table)
 {
     *q = 0; *q_squared = 0;
     const int c_a = first_max(counts0, n_classes);           // Algorithm 1 steps 2, 4, 5, 6
     const double p_a = lower_conf_bound(counts[c_a], N, alpha);
     if (!(p_a > 0.5)) return -1;
-    std::vector<uint32_t> own;
-    if (!table) noise_table(sigma, own);
-    const std::vector<uint32_t> &cum = table ? *table : own;
+    std::vector<uint32_t> cum;
+    if (table) cum.assign(table, table + n_table);
+    else noise_table(sigma, cum);
     const int32_t q_a = table_quantile(cum, to_fixed32(p_a));
     if (!two_sided) {                                         // Theorem 3.2 steps 2-3: radius and squared radius in pixel levels
         *q = q_a;

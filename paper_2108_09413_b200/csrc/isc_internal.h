@@ -111,9 +111,9 @@ double binom_pvalue_half(int64_t n_a, int64_t m);
 int32_t decide_certify(const int32_t *counts0, const int32_t *counts, int n_classes, int64_t N,
                        double sigma, double alpha, double *radius, double *p_lower);
 int32_t decide_predict(const int32_t *counts, int n_classes, double alpha);
-// `table`: Eq. 2's cumulative table for sigma if the caller has it, else null
+// `table`: Eq. 2's cumulative table for sigma (n_table entries) if the caller has it, else null
 int32_t decide_certify_integer(const int32_t *counts0, const int32_t *counts, int n_classes, int64_t N, double sigma,
-                               double alpha, bool two_sided, int32_t *q, int64_t *q_squared, const std::vector<uint32_t> *table);
+                               double alpha, bool two_sided, int32_t *q, int64_t *q_squared, const uint32_t *table, size_t n_table);
 int noise_halfwidth(double sigma);
 void noise_table(double sigma, std::vector<uint32_t> &cum);
 void noise_table_rounded(double sigma, std::vector<uint32_t> &cum);
