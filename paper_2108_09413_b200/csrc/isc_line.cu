@@ -165,7 +165,8 @@ struct Ctrl {
     uint32_t tmem_base;
     volatile int abort_flag;
     uint32_t stored[kMaxBars];              // per unit: stores of its 16-channel chunks by a warp, counted over the whole run
-    int32_t pooled[kG][64];                 // the tail's pooled features, one row per sample of the group
+    int32_t pool_sum[kG][64];               // the tail's sums over the pixels, zero between groups
+    alignas(16) int8_t pooled[kG][64];      // its pooled features, one row per sample of the group
     long long cyc[4], cyc_mark;             // thread 0's phase clocks
     PhaseEntry ptab[kMaxPhases];
     ConvSrc csrc[kMaxConv];
@@ -754,89 +755,123 @@ __device__ __forceinline__ GroupJob group_job(const LineParams &p, int grp)
     return g;
 }
 
-// INPUT: one thread = four horizontally adjacent pixels of one sample, all input channels (Def. 3.3, Def. 3.4).
-__device__ void input_phase(const LineParams &p, const EpiCtx &c, int grp)
+// INPUT: one item = four horizontally adjacent pixels of one sample and input channel, one Philox block (Def. 3.3,
+// Def. 3.4).  Items of all channels share one index space (3072 items of a 32 x 32 x 3 image for 640 threads; with the
+// channels of a pixel in one thread it was 1024, two rounds of which the second is mostly idle), and the four table
+// searches run interleaved in a fixed number of steps instead of one after the other.  Out of line, like the tail's last
+// step: the convolutions' loops pay for every register and instruction that these phases share with them.
+__device__ __noinline__ void input_phase(const LineParams &p, const EpiCtx &c, int grp)
 {
     const int H = p.in_H, W = p.in_W, in_c = p.in_c;
-    const int wq = W >> 2;
-    const int quads = kG * H * wq;
+    const int log_wq = 31 - __clz(W >> 2);                  // W is a power of two
+    const int quads = kG * H * (W >> 2);
     const uint32_t *__restrict__ cum = p.ns.cum;
     const uint32_t *__restrict__ guide = p.ns.guide;
-    const int T = p.ns.T;
+    const int T = p.ns.T, steps = p.ns.guide_steps;
     const GroupJob g = group_job(p, grp);
     const unsigned long long image_id = p.image_id0 + (unsigned long long)g.image;
     const uint32_t key0 = p.ns.key0, key1 = p.ns.key1, ctr2 = (uint32_t)image_id;
     const uint32_t ctr3_fixed = (g.sel ? (uint32_t)p.phase_sel : p.ns.ctr3_fixed) | ((uint32_t)(image_id >> 32) & 0xFFFFu) << 16;
     const long long j0 = (g.sel ? 0ll : p.ns.first_sample) + g.local;
     const uint8_t *__restrict__ x = p.x + (size_t)g.image * (size_t)(in_c * H * W);
-    for (int qi = c.tid; qi < quads; qi += kThreads) {
+    int ch = 0;
+    for (int i = c.tid, qi = c.tid; i < quads * in_c; i += kThreads, qi += kThreads) {
+        while (qi >= quads) { qi -= quads; ++ch; }
         // consecutive threads take consecutive samples: their stores fall into one 64-byte run
         const int s = qi & (kG - 1);
         const int rem = qi >> 2;
-        const int y = rem / wq, x4 = rem - y * wq;
+        const int y = rem >> log_wq, x4 = rem & ((1 << log_wq) - 1);
         const long long j = j0 + s;
         const uint32_t ctr3 = ctr3_fixed | (uint32_t)(((j >> 32) & 0xFF) << 8);
-        uint32_t px[4] = {0, 0, 0, 0};
-        for (int ch = 0; ch < in_c; ++ch) {
-            const uint32_t e = (uint32_t)((ch * H + y) * W + 4 * x4);
-            const uint4 r = philox4x32_10(make_uint4(e >> 2, (uint32_t)(j & 0xFFFFFFFFll), ctr2, ctr3), key0, key1);
+        const uint32_t e = (uint32_t)((ch * H + y) * W + 4 * x4);
+        const uint4 r = philox4x32_10(make_uint4(e >> 2, (uint32_t)(j & 0xFFFFFFFFll), ctr2, ctr3), key0, key1);
+        const uint32_t clean = __ldg(reinterpret_cast<const uint32_t *>(x + e));
+        int z[4];
+        if (guide) {
+            noise_levels4(r, cum, guide, T, steps, z);
+        } else {
             const uint32_t u[4] = {r.x, r.y, r.z, r.w};
-            const uint32_t clean = __ldg(reinterpret_cast<const uint32_t *>(x + e));
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                int v = (int)((clean >> (8 * k)) & 0xFF) + (guide ? noise_level_guided(u[k], cum, guide, T) : noise_level(u[k], cum, T));
-                v = min(255, max(0, v));
-                px[k] |= (uint32_t)v << (8 * ch);
-            }
+            for (int k = 0; k < 4; ++k) z[k] = noise_level(u[k], cum, T);
         }
-        // the input has one row band: line = row, position = column * 4 + sample
-        const uint32_t pos = (uint32_t)y * p.input_pitch16 + (uint32_t)(4 * x4) * kG + (uint32_t)s;
+        // the input has one row band: line = row, position = column * 4 + sample; the bytes beyond the input channels
+        // meet zero weights
+        const uint32_t at = c.sbase + p.input_base + ((uint32_t)y * p.input_pitch16 + (uint32_t)(4 * x4) * kG + (uint32_t)s) * 16u + (uint32_t)ch;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) st_shared_v4(c.sbase + p.input_base + (pos + (uint32_t)k * kG) * 16u, make_uint4(px[k], 0, 0, 0));
+        for (int k = 0; k < 4; ++k) {
+            const int v = min(255, max(0, (int)((clean >> (8 * k)) & 0xFFu) + z[k]));
+            asm volatile("st.shared.u8 [%0], %1;" ::"r"(at + (uint32_t)k * (kG * 16u)), "r"(v) : "memory");
+        }
     }
 }
 
-// TAIL, first half: global average pool.  One thread sums one (sample, channel) pair over the pixels and
-// requantises it; consecutive threads take the four samples of consecutive channels (one shared-memory wavefront).
+// TAIL: global average pool, FC, argmax and vote (Algorithm 1 steps 1-4), in three steps between barriers.
+// First step: a thread adds up four channels (one word) of one sample over a share of the pixels; consecutive threads take
+// the words of the four samples of a position (64 contiguous bytes), the shares meet in shared-memory additions.  (One
+// thread per channel and sample left most of the CTA idle over 64 to 1024 pixels: with the noise phase before it, a
+// network that ends at a 32 x 32 map spent 43 us a group more, the tiny CNN 15 us a call.)
+__device__ void tail_sum(const LineParams &p, const EpiCtx &c)
+{
+    const int units = p.tail_C, parts = kThreads / units, part = c.tid / units, u = c.tid - part * units;       // a unit is (word, sample)
+    if (part >= parts) return;
+    const int word = u >> 2, s = u & (kG - 1);
+    const int log_w = 31 - __clz(p.tail_W), log_n = 31 - __clz(p.tail_n_lines);                                  // powers of two
+    const uint32_t base = c.sbase + p.tail_base + (uint32_t)(word >> 2) * p.tail_plane + (uint32_t)(word & 3) * 4u + (uint32_t)s * 16u;
+    int sum[4] = {0, 0, 0, 0}, n = 0;
+    for (int i = part; i < p.tail_H * p.tail_W; i += parts, ++n) {
+        const int y = i >> log_w, x = i & (p.tail_W - 1);
+        const int line = y & (p.tail_n_lines - 1), band = y >> log_n;
+        const uint32_t pos = (uint32_t)line * p.tail_pitch16 + ((uint32_t)x << p.tail_logI) + (uint32_t)(band * 4);
+        const int v = (int)lds32(base + pos * 16u);
+        sum[0] = __dp4a(v, 1, sum[0]);
+        sum[1] = __dp4a(v, 1 << 8, sum[1]);
+        sum[2] = __dp4a(v, 1 << 16, sum[2]);
+        sum[3] = __dp4a(v, 1 << 24, sum[3]);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) atomicAdd(&c.ctrl->pool_sum[s][4 * word + k], sum[k] - n * p.pool_zp_in);
+}
+
+// Second step: the sums' requantisation.
 __device__ void tail_pool(const LineParams &p, const EpiCtx &c)
 {
-    const int tail_W = p.tail_W, n_lines = p.tail_n_lines, hw = p.tail_H * p.tail_W;
     for (int q = c.tid; q < kG * p.tail_C; q += kThreads) {
         const int s = q & (kG - 1), ch = q >> 2;
-        const uint32_t base = c.sbase + p.tail_base + (uint32_t)(ch >> 4) * p.tail_plane + (uint32_t)(ch & 15);
-        int sum = 0;
-        for (int i = 0; i < hw; ++i) {
-            const int y = i / tail_W, x = i - y * tail_W;
-            const int line = y % n_lines, band = y / n_lines;
-            const uint32_t pos = (uint32_t)line * p.tail_pitch16 + ((uint32_t)x << p.tail_logI) + (uint32_t)(band * 4 + s);
-            int v;
-            asm volatile("ld.shared.s8 %0, [%1];" : "=r"(v) : "r"(base + pos * 16u));
-            sum += v - p.pool_zp_in;
-        }
+        const int sum = c.ctrl->pool_sum[s][ch];
+        c.ctrl->pool_sum[s][ch] = 0;
         long long v = ((long long)sum * p.pool_mult + (1ll << (p.pool_n - 1))) >> p.pool_n;
         v += p.pool_zp_out;
         v = v < p.pool_lo ? p.pool_lo : v;
         v = v > 127 ? 127 : v;
-        c.ctrl->pooled[s][ch] = (int32_t)v;
+        c.ctrl->pooled[s][ch] = (int8_t)v;
     }
 }
 
-// TAIL, second half: FC, argmax and vote; one warp carries one sample (Algorithm 1 steps 1-4).
-__device__ void tail_sample(const LineParams &p, const EpiCtx &c, int s, int grp)
+// Third step: FC, argmax and vote; one warp carries one sample, a lane one class (features beyond the last meet zero weights).
+__device__ __noinline__ void tail_sample(const LineParams &p, const EpiCtx &c, int s, int grp)
 {
-    const int tail_C = p.tail_C;
     const int n_classes = p.n_classes;
     const GroupJob g = group_job(p, grp);
     const int sample = g.local + s;                            // index within the image's phase
     const bool counted = sample < g.n;
     int best_v = -1000, best_o = 0x7fffffff;
+    uint4 f[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) f[k] = ld_shared_v4(smem_u32(&c.ctrl->pooled[s][16 * k]));
     for (int o0 = 0; o0 < n_classes; o0 += 32) {
         const int o = o0 + c.lane;
         const bool live = o < n_classes;
         const FcConst k = p.fc_c[live ? o : 0];
-        const int8_t *wrow = p.fc_w + (size_t)(live ? o : 0) * 64;
+        const uint4 *wrow = reinterpret_cast<const uint4 *>(p.fc_w + (size_t)(live ? o : 0) * 64);
         int acc = k.bias;
-        for (int cc = 0; cc < tail_C; ++cc) acc += c.ctrl->pooled[s][cc] * (int)__ldg(wrow + cc);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint4 w = __ldg(wrow + q);
+            acc = __dp4a((int)f[q].x, (int)w.x, acc);
+            acc = __dp4a((int)f[q].y, (int)w.y, acc);
+            acc = __dp4a((int)f[q].z, (int)w.z, acc);
+            acc = __dp4a((int)f[q].w, (int)w.w, acc);
+        }
         long long v = ((long long)acc * k.mult + (1ll << (k.n - 1))) >> k.n;
         v += k.zp_out;
         v = v < k.lo ? k.lo : v;
@@ -873,6 +908,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_line(const __grid_constant__ Li
     for (int i = threadIdx.x; i < p.n_phases; i += blockDim.x) ctrl->ptab[i] = p.ptab[i];
     for (int i = threadIdx.x; i < p.n_conv; i += blockDim.x) ctrl->csrc[i] = p.conv_src[i];
     for (int i = threadIdx.x; i < kMaxBars; i += blockDim.x) ctrl->stored[i] = 0;
+    for (int i = threadIdx.x; i < kG * 64; i += blockDim.x) (&ctrl->pool_sum[0][0])[i] = 0;
     if (warp == 0) tmem_alloc(smem_u32(&ctrl->tmem_base), kTmemCols);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_proxy_async();
@@ -946,9 +982,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_line(const __grid_constant__ Li
             if (live) {
                 if (e.x == PH_FILL) fill_phase(c, e.y, e.z, e.w);
                 else if (e.x == PH_INPUT) input_phase(p, c, grp);
-                else tail_pool(p, c);
+                else tail_sum(p, c);
             }
             if (e.x == PH_TAIL) {
+                __syncthreads();
+                if (live) tail_pool(p, c);
                 __syncthreads();
                 if (live && warp < kG) tail_sample(p, c, warp, grp);
             }
