@@ -70,6 +70,8 @@ constexpr int kMaxBars = 128;
 constexpr int kMaxLines = 32;               // output lines of one convolution
 constexpr int kCtrlBytes = 10240;
 constexpr int kMaxConv = 128;
+constexpr int kOpChains = 4;                // MMA chains of an operation at most
+constexpr int kOpChainTries[] = {kOpChains, 1};   // a record of merged chains may name more units than it has room for
 constexpr int kSmemLimit = 227 * 1024;
 constexpr int kTmemCols = 512;
 constexpr int kSideStreams = 8;             // concurrent launches when a launch does not fill the GPU
@@ -78,9 +80,9 @@ constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // 2 s per wait
 enum { PH_FILL = 0, PH_INPUT = 1, PH_CONV = 2, PH_TAIL = 3 };
 enum { ERR_NONE = 0, ERR_WAIT_DONE = 1, ERR_WAIT_WEIGHTS = 2, ERR_WAIT_READY = 3, ERR_WAIT_FULL = 4, ERR_WAIT_DRAIN = 5 };
 enum { CF_STACKED = 1, CF_RES = 2, CF_LO = 4, CF_SCATTER = 8, CF_GENERAL = 16, CF_RSHORT = 32 };     // CF_GENERAL: the pass that decides everything at run time; CF_RSHORT: residual term without the 64-bit addend
-// OPF_WAIT_ALL: every unit of the previous convolution; OPF_NULL: no MMAs, arrivals only; OPF_WAITS / OPF_WAITS4: the
-// record names counters to test (two / four slots in use); bits 4-6: how many of them are distinct; bits 8-9: arrivals
-enum { OPF_WAIT_ALL = 1, OPF_WAITS = 2, OPF_NULL = 4, OPF_WAITS4 = 8 };
+// OPF_WAIT_ALL: every unit of the previous convolution; OPF_WAITS / OPF_WAITS4: the record names counters to test (two /
+// four slots in use); bits 4-6: how many of them are distinct; bits 8-9: arrivals; bits 10-12: MMA chains
+enum { OPF_WAIT_ALL = 1, OPF_WAITS = 2, OPF_WAITS4 = 8 };
 
 // ---- what the kernel reads -------------------------------------------------------------------
 
@@ -97,15 +99,16 @@ struct alignas(16) ConvSrc {
     uint32_t dep_first, dep_units, dep_mult, dep_local_uses;     // dep_local | dep_uses << 16
 };
 
-// One MMA chain in the form the issuing thread consumes: accumulator columns, what to add to the operand
-// descriptors' start addresses, and the barriers (as byte offsets, 0xFFFF = none) of its dependencies and completions.
+// MMA chains over up to kOpChains consecutive input lines in the form an issuing thread consumes: accumulator columns, what
+// to add to the operand descriptors' start addresses, and the barriers (as byte offsets, 0xFFFF = none) of its dependencies
+// and completions.
 struct alignas(16) LOp {
     uint32_t d_col;         // first accumulator column within the bank
     uint32_t idesc;         // instruction descriptor (N = blocks * cout)
     uint32_t a_add, b_add;  // 16-byte units: (input line + 1) * pitch, first weight block * block size
     uint16_t wait[4];       // 8 * unit of the previous convolution that must be stored
     uint16_t commit[3];     // 8 * unit of this convolution whose accumulators are complete after the chain
-    uint16_t flags;         // OPF_* | distinct waits << 4 | arrivals << 8
+    uint16_t flags;         // OPF_* | distinct waits << 4 | arrivals << 8 | chains << 10
 };
 static_assert(sizeof(LOp) == 32, "one operation is two 16-byte loads");
 
@@ -295,7 +298,7 @@ struct Waiter {
 struct PrevConv { uint32_t done_addr, expected, n_lines; };    // counters of its units, their value when stored; n_lines = 0: nothing to wait for
 
 struct IssueCtx {
-    uint32_t desc, ops, n_ops, s16, b_lo0, kstep16, d0, stacked, full_addr, cg, issuer;
+    uint32_t desc, ops, n_ops, s16, b_lo0, kstep16, d0, stacked, full_addr, cg, issuer, pitch16, cols;
 };
 
 // The first, cheap read of a "stored" counter by an issuing thread.  A plain load by default: an acquiring one costs
@@ -373,22 +376,36 @@ __device__ __forceinline__ bool issue_ops(Waiter w, const IssueCtx &ic, const Pr
             if (m < 0 && !wait_units_slow(w, prev, r1)) return false;
         }
         tc_fence_after();
-        const uint32_t d = ic.d0 + r0.x;
-        if (fl & OPF_NULL) {
+        if (KS == 2) {
+            // chains over consecutive lines
+            const uint32_t n_chains = (fl >> 10) & 7u;        // 0: a record that only carries this thread's arrivals
+            uint32_t d = ic.d0 + r0.x, a_add = r0.z;
+            auto chain = [&]() {
+#pragma unroll
+                for (int k = 0; k < NK; ++k)
+                    mma_i8(d, ((uint64_t)ahi << 32) | (uint64_t)(alo[k] + a_add), ((uint64_t)bhi << 32) | (uint64_t)(blo[k] + r0.w), r0.y, k > 0 ? 1u : acc_first);
+                d += ic.cols;
+                a_add += ic.pitch16;
+            };
+            if (n_chains == kOpChains) {
+#pragma unroll
+                for (int c = 0; c < kOpChains; ++c) chain();
+            } else {
+                for (uint32_t c = 0; c < n_chains; ++c) chain();
+            }
+        } else if (!(fl & (7u << 10))) {
             // a record that only carries this thread's arrivals on units it did not add to
         } else if (KS > 0) {
+            const uint32_t d = ic.d0 + r0.x;
 #pragma unroll
-            for (int k = 0; k < NK; ++k) {
-                const uint64_t ad = ((uint64_t)ahi << 32) | (uint64_t)(alo[k] + r0.z);
-                const uint64_t bd = ((uint64_t)bhi << 32) | (uint64_t)(blo[k] + r0.w);
-                mma_i8(d, ad, bd, r0.y, k > 0 ? 1u : acc_first);
-            }
+            for (int k = 0; k < NK; ++k)
+                mma_i8(d, ((uint64_t)ahi << 32) | (uint64_t)(alo[k] + r0.z), ((uint64_t)bhi << 32) | (uint64_t)(blo[k] + r0.w), r0.y, k > 0 ? 1u : acc_first);
         } else {
+            const uint32_t d = ic.d0 + r0.x;
             for (uint32_t k = 0; k < n_ksteps; ++k) {
                 const uint32_t a_lo = lds32(ic.desc + offsetof(LConvDesc, a_lo) + 4 * k) + ic.s16;
-                const uint64_t ad = ((uint64_t)ahi << 32) | (uint64_t)(a_lo + r0.z);
-                const uint64_t bd = ((uint64_t)bhi << 32) | (uint64_t)(ic.b_lo0 + ic.s16 + k * ic.kstep16 + r0.w);
-                mma_i8(d, ad, bd, r0.y, k > 0 ? 1u : acc_first);
+                mma_i8(d, ((uint64_t)ahi << 32) | (uint64_t)(a_lo + r0.z), ((uint64_t)bhi << 32) | (uint64_t)(ic.b_lo0 + ic.s16 + k * ic.kstep16 + r0.w), r0.y,
+                       k > 0 ? 1u : acc_first);
             }
         }
         const uint32_t nc = (fl >> 8) & 3u;
@@ -452,6 +469,8 @@ __device__ __noinline__ bool issuer_conv(const LineParams &p, Ctrl *ctrl, uint32
     ic.full_addr = smem_u32(&ctrl->bars[h3.z + (use & 1u) * h4.z]);      // the class has two sets of barriers, used in turn
     ic.cg = cg;
     ic.issuer = (uint32_t)issuer;
+    ic.pitch16 = h1.y;
+    ic.cols = lds32(desc + offsetof(LConvDesc, cols));
     bool ok;
     switch (h0.z) {
     case 1: ok = issue_ops<1>(w, ic, prev, 1); break;
@@ -1161,7 +1180,8 @@ struct ConvPlan {
     std::vector<Unit> units;
 };
 
-bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_w, int n_classes, LinePlan *plan,
+// op_chains: MMA chains that one operation may hold at most
+bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_w, int n_classes, int op_chains, LinePlan *plan,
                 std::vector<uint8_t> *blob_out, std::vector<uint32_t> *blob_offsets, std::vector<PhaseEntry> *ptab_out,
                 std::vector<ConvSrc> *csrc_out, std::vector<uint8_t> *bar_counts_out)
 {
@@ -1323,11 +1343,12 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
             if (in.nb == 1) return -1;
             return p < 0 ? in.n_lines - 1 : 0;
         };
-        struct ProtoOp { int a_line, b_block, n_blocks, d_line; std::vector<int> need; std::vector<int> outs; int ready; };
+        struct ProtoOp { int a_line, b_block, n_blocks, d_line, n_chains; std::vector<int> need; std::vector<int> outs; int ready; };
         std::vector<ProtoOp> proto;
         if (cp.stacked) {
             for (int p = -1; p <= in.n_lines; ++p) {
                 ProtoOp o;
+                o.n_chains = 1;
                 o.a_line = p;
                 const int y_lo = std::max(p - 1, 0), y_hi = std::min(p + 1, in.n_lines - 1);
                 o.b_block = y_lo - (p - 1); o.n_blocks = y_hi - y_lo + 1; o.d_line = y_lo;
@@ -1339,6 +1360,7 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
         } else {
             for (int j = 0; j < cp.m; ++j) {
                 ProtoOp o;
+                o.n_chains = 1;
                 const int cline = cp.scatter ? 2 * j : j;
                 o.a_line = cline; o.b_block = 0; o.n_blocks = 1; o.d_line = j;
                 o.outs.push_back(j);
@@ -1354,6 +1376,26 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
             for (int l : o.need) o.ready = std::max(o.ready, prev_time(l));
         }
         std::stable_sort(proto.begin(), proto.end(), [](const ProtoOp &a, const ProtoOp &b) { return a.ready < b.ready; });
+        // In the long convolutions of two K-steps (stage 1 of a CIFAR ResNet: 34 chains of two MMAs) chains over consecutive
+        // lines with the same blocks make one operation: an issuing thread spends more on a record than on its MMAs
+        // (10,270 -> 9,390 cycles a convolution; ResNet-110 485.7 -> 459.8 us a round of 592 samples).  With three and more
+        // K-steps a chain is worth a record of its own.
+        if (cp.stacked && cp.kunits.size() == 2 && cp.m >= 16) {
+            std::vector<ProtoOp> merged;
+            for (const ProtoOp &o : proto) {
+                ProtoOp *l = merged.empty() ? nullptr : &merged.back();
+                if (l && l->n_chains < op_chains && l->a_line + l->n_chains == o.a_line && l->d_line + l->n_chains == o.d_line &&
+                    l->n_blocks == o.n_blocks && l->b_block == o.b_block) {
+                    l->n_chains += 1;
+                    l->ready = std::max(l->ready, o.ready);
+                    for (int n : o.need) if (std::find(l->need.begin(), l->need.end(), n) == l->need.end()) l->need.push_back(n);
+                    for (int y : o.outs) if (std::find(l->outs.begin(), l->outs.end(), y) == l->outs.end()) l->outs.push_back(y);
+                } else {
+                    merged.push_back(o);
+                }
+            }
+            proto.swap(merged);
+        }
         // completion of each output line = the last operation that contributes to it
         std::vector<int> last_op((size_t)cp.m, -1);
         for (size_t i = 0; i < proto.size(); ++i)
@@ -1389,7 +1431,7 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
         cp.use_local = class_uses[(size_t)cp.cls]++;
         const bool wait_all = pv && pv->cls != cp.cls;
         // Record i belongs to issuing thread i mod kIssuers; every thread needs a record to carry its arrivals.
-        auto null_op = []() { ProtoOp o; o.a_line = 0; o.b_block = 0; o.n_blocks = 0; o.d_line = 0; o.ready = 0; return o; };
+        auto null_op = []() { ProtoOp o; o.a_line = 0; o.b_block = 0; o.n_blocks = 0; o.d_line = 0; o.n_chains = 0; o.ready = 0; return o; };
         while (proto.size() < (size_t)kIssuers) proto.push_back(null_op());
         // Each thread arrives on every unit's barrier once: after its last record that adds to the unit, or with any
         // of its records if it has none (at most three arrivals fit a record; empty records are added as needed).
@@ -1411,9 +1453,10 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
             for (int u = 0; u < cp.n_units && fits; ++u)
                 for (int wi = 0; wi < kIssuers && fits; ++wi) {
                     if (has[(size_t)u][(size_t)wi]) continue;
+                    // in a long convolution the record just before the unit completes, else any
                     int carrier = -1;
-                    for (size_t i = (size_t)wi; i < proto.size() && carrier < 0; i += kIssuers)
-                        if (commits[i].size() < 3) carrier = (int)i;
+                    for (size_t i = (size_t)wi; i < proto.size(); i += kIssuers)
+                        if (commits[i].size() < 3 && (carrier < 0 || (cp.m >= 16 && (int)i <= unit_last_op[(size_t)u]))) carrier = (int)i;
                     if (carrier < 0) fits = false;
                     else commits[(size_t)carrier].push_back(u);
                 }
@@ -1438,7 +1481,7 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
             const size_t wi = i % kIssuers;
             LOp op;
             memset(&op, 0xFF, sizeof(op));
-            op.flags = o.n_blocks == 0 ? OPF_NULL : 0;
+            op.flags = (uint16_t)(o.n_chains << 10);
             op.d_col = (uint32_t)(o.d_line * cp.cols);
             const uint32_t a_fmt_bit = cp.in_tensor == 0 ? 0u : 1u;
             op.idesc = (2u << 4) | (a_fmt_bit << 7) | (1u << 10) | ((uint32_t)((std::max(o.n_blocks, 1) * L.cout) >> 3) << 17) | ((128u >> 4) << 24);
@@ -1657,7 +1700,7 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
         for (size_t k = 0; k < cp.kunits.size(); ++k)
             for (const LOp &op : cp.ops) {
                 const long long lo_b = (long long)in.line0 - (long long)in.pitch * 16 + (long long)op.a_add * 16 + cp.a_delta[k];
-                const long long hi_b = lo_b + cp.a_lbo[k] + 128 * 16;
+                const long long hi_b = lo_b + cp.a_lbo[k] + 128 * 16 + (long long)std::max(((op.flags >> 10) & 7) - 1, 0) * in.pitch * 16;
                 if (lo_b < 0 || hi_b > (long long)in.bytes) PLAN_FAIL(18);
             }
         memcpy(blob.data(), &D, sizeof(D));
@@ -1759,13 +1802,16 @@ int line_plan_probe(const LayerIn *layers, int n_layers, int in_c, int in_h, int
     *smem_bytes = 0;
     bool ok = structure_ok(layers, n_layers, n_classes);
     if (ok) {
-        LinePlan plan;
-        std::vector<uint8_t> blob, bar_counts;
-        std::vector<uint32_t> blob_off;
-        std::vector<PhaseEntry> ptab;
-        std::vector<ConvSrc> csrc;
-        ok = build_plan(layers, n_layers, in_c, in_h, in_w, n_classes, &plan, &blob, &blob_off, &ptab, &csrc, &bar_counts);
-        if (ok) *smem_bytes = plan.smem_bytes;
+        for (int chains : kOpChainTries) {
+            LinePlan plan;
+            std::vector<uint8_t> blob, bar_counts;
+            std::vector<uint32_t> blob_off;
+            std::vector<PhaseEntry> ptab;
+            std::vector<ConvSrc> csrc;
+            ok = build_plan(layers, n_layers, in_c, in_h, in_w, n_classes, chains, &plan, &blob, &blob_off, &ptab, &csrc, &bar_counts);
+            if (ok) *smem_bytes = plan.smem_bytes;
+            if (ok) break;
+        }
     }
     *rule = ok ? 0 : g_plan_rule;
     return ok ? 1 : 0;
@@ -1777,15 +1823,19 @@ int line_build(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_w
     if (!structure_ok(layers, n_layers, n_classes)) return ISC_OK;
     const isc_layer &LP = layers[n_layers - 2].d, &LF = layers[n_layers - 1].d;
 
-    LinePlan *plan = new LinePlan();
+    LinePlan *plan = nullptr;
     std::vector<uint8_t> blob, bar_counts;
     std::vector<uint32_t> blob_off;
     std::vector<PhaseEntry> ptab;
     std::vector<ConvSrc> csrc;
-    if (!build_plan(layers, n_layers, in_c, in_h, in_w, n_classes, plan, &blob, &blob_off, &ptab, &csrc, &bar_counts)) {
+    for (int chains : kOpChainTries) {
+        plan = new LinePlan();
+        blob.clear(); bar_counts.clear(); blob_off.clear(); ptab.clear(); csrc.clear();
+        if (build_plan(layers, n_layers, in_c, in_h, in_w, n_classes, chains, plan, &blob, &blob_off, &ptab, &csrc, &bar_counts)) break;
         delete plan;
-        return ISC_OK;
+        plan = nullptr;
     }
+    if (!plan) return ISC_OK;
     plan->in_c = in_c; plan->in_h = in_h; plan->in_w = in_w; plan->n_classes = n_classes;
 
     int dev = 0;
