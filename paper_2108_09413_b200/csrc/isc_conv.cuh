@@ -90,6 +90,39 @@ __device__ __forceinline__ uint4 requant16_fast(const int *acc, uint32_t cst, ui
     return make_uint4(packed[0], packed[1], packed[2], packed[3]);
 }
 
+// One output (see requant16_fast); kClamp: the lower clamp is above -128, which the packing saturates at.
+template <int kRes, bool kClamp>
+__device__ __forceinline__ int requant1(int acc, const int4 &c, uint32_t rword, int k, uint32_t m2, long long r2, uint32_t k8, int lo)
+{
+    int v = (hi32(mul_wide(acc + c.x, c.y)) + c.z) >> c.w;
+    if (kRes == 1) v += hi32(mad_wide_u(__byte_perm(rword, 0u, 0x4440u | (uint32_t)k), m2, r2));
+    if (kRes == 2) v += hi32(mad_wide_u(__byte_perm(rword, k8, 0x7650u | (uint32_t)k), m2, 0ll));
+    return kClamp ? max(v, lo) : v;
+}
+
+// 16 channels of two rows: a channel's constants are read once for both, because their reads bound the form above (a
+// 16-byte broadcast per output: six outputs a clock and SM).  r0, r1: the residual bytes, offset by 128.
+template <int kRes, bool kClamp>
+__device__ __forceinline__ void requant16x2(const int (&a)[2][16], uint32_t cst, const uint32_t (&r0)[4], const uint32_t (&r1)[4], uint32_t m2, long long r2, uint32_t k8, int lo, uint4 (&o)[2])
+{
+    uint32_t w0[4], w1[4];
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+        int y0[4], y1[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            int4 cs;
+            asm("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(cs.x), "=r"(cs.y), "=r"(cs.z), "=r"(cs.w) : "r"(cst + (uint32_t)(4 * g + k) * 16u));
+            y0[k] = requant1<kRes, kClamp>(a[0][4 * g + k], cs, r0[g], k, m2, r2, k8, lo);
+            y1[k] = requant1<kRes, kClamp>(a[1][4 * g + k], cs, r1[g], k, m2, r2, k8, lo);
+        }
+        w0[g] = pack4_sat(y0[0], y0[1], y0[2], y0[3]);
+        w1[g] = pack4_sat(y1[0], y1[1], y1[2], y1[3]);
+    }
+    o[0] = make_uint4(w0[0], w0[1], w0[2], w0[3]);
+    o[1] = make_uint4(w1[0], w1[1], w1[2], w1[3]);
+}
+
 // 32 accumulator columns of this thread's lane, asynchronously; the registers are valid after tmem_ld32_wait(),
 // which names them so that no use can move above it
 __device__ __forceinline__ void tmem_ld32_issue(uint32_t taddr, int (&v)[2][16])

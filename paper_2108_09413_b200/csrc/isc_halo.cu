@@ -77,16 +77,6 @@ struct HaloParams {
     int32_t *err;
 };
 
-// Constants of one channel for one output of each of the two rows.
-template <int kRes, bool kClamp>
-__device__ __forceinline__ int requant1(int acc, const int4 &c, uint32_t rword, int k, uint32_t m2, long long r2, uint32_t k8, int lo)
-{
-    int v = (hi32(mul_wide(acc + c.x, c.y)) + c.z) >> c.w;
-    if (kRes == 1) v += hi32(mad_wide_u(__byte_perm(rword, 0u, 0x4440u | (uint32_t)k), m2, r2));
-    if (kRes == 2) v += hi32(mad_wide_u(__byte_perm(rword, k8, 0x7650u | (uint32_t)k), m2, 0ll));
-    return kClamp ? max(v, lo) : v;
-}
-
 struct RoleCtx {
     uint32_t sbase, tmem, acc_full, acc_free;
     int warp, lane;
@@ -195,22 +185,7 @@ __device__ __forceinline__ bool halo_epilogue(const HaloParams &p, const RoleCtx
                 }
             } else {
                 constexpr int kRes = kMode == 3 ? 2 : kMode == 2 ? 1 : 0;
-                uint32_t w0[4], w1[4];
-#pragma unroll
-                for (int g = 0; g < 4; ++g) {
-                    int y0[4], y1[4];
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        int4 cs;
-                        asm("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(cs.x), "=r"(cs.y), "=r"(cs.z), "=r"(cs.w) : "r"(cst0 + (uint32_t)(cc + 4 * g + k) * 16u));
-                        y0[k] = requant1<kRes, kClamp>(a[0][4 * g + k], cs, r0[g], k, p.res_m2, p.res_r2, p.res_k8, p.lo);
-                        y1[k] = requant1<kRes, kClamp>(a[1][4 * g + k], cs, r1[g], k, p.res_m2, p.res_r2, p.res_k8, p.lo);
-                    }
-                    w0[g] = pack4_sat(y0[0], y0[1], y0[2], y0[3]);
-                    w1[g] = pack4_sat(y1[0], y1[1], y1[2], y1[3]);
-                }
-                o[0] = make_uint4(w0[0], w0[1], w0[2], w0[3]);
-                o[1] = make_uint4(w1[0], w1[1], w1[2], w1[3]);
+                requant16x2<kRes, kClamp>(a, cst0 + (uint32_t)cc * 16u, r0, r1, p.res_m2, p.res_r2, p.res_k8, p.lo, o);
             }
             st_shared_v4(scr, o[0]);
             st_shared_v4(scr + mt_step, o[1]);

@@ -22,6 +22,10 @@
 //     accumulator each: a thread owns one tile row, 32 columns per step with the next step's accumulators already
 //     requested; the rows pass through a per-warp scratch area so that, every 64 columns, the results leave and the
 //     next tile's residual rows arrive as contiguous runs, under the arithmetic of the following columns.
+// 1 x 1 layers that expand the channels, which the epilogue bounds, take tiles of 256 pixels x 128 channels (kPair): a
+// thread then owns two rows and reads a channel's constants once for both.  64 -> 256 channels at 56 x 56, 512 samples:
+// 222 -> 184 us, with a residual operand 286 -> 265 us; 256 -> 128: 159 -> 135 us.  (Sixteen epilogue warps instead of
+// eight: 203 and 294 us against 196 and 280.)
 // Every wait is bounded; on expiry a role raises the CTA's abort flag and the error word, the others leave their
 // loops, and the CTA frees its tensor memory and returns.
 #include <cuda.h>
@@ -48,6 +52,7 @@ namespace {
 constexpr int kTileM = 128;
 constexpr int kBlockK = 64;                  // bytes of K per stage: two MMA K-steps
 constexpr int kMaxStages = 16;
+constexpr int kPairN = 128;                  // channels of a paired tile: two operands of 128 rows, two tiles in tensor memory
 constexpr int kStemThreads = 256;           // k_stem: two threads per tile row; two CTAs per SM (registers allow no third, nor two of 512 threads)
 constexpr size_t kStemSmemLimit = 108 * 1024;          // dynamic shared memory of k_stem: two CTAs per SM
 constexpr int kEpiWarps = 4, kEpiTeams = 2, kGatherWarps = 4;          // a team of epilogue warps takes every other tile
@@ -202,9 +207,112 @@ __device__ __forceinline__ bool epilogue_role(const IgemmParams &p, const EpiCtx
     return true;
 }
 
+// The epilogue of a paired tile: 256 pixels (two M operands) x kPairN channels.  A thread owns one row of each operand, so
+// that a channel's constants are read once for two outputs.  Scratch and memory traffic as above, 64 columns of the 64
+// rows at a time.  kMode 1 to 3 as above; kClamp: the lower clamp is above -128.
+template <int kMode, bool kClamp>
+__device__ __forceinline__ bool epilogue_pair(const IgemmParams &p, const EpiCtx &c)
+{
+    constexpr int kRes = kMode == 3 ? 2 : kMode == 2 ? 1 : 0;
+    const GLayer &L = p.L;
+    const int lane = c.lane, tiles_n = c.tiles_n, q = c.warp & 3, team = c.warp / kEpiWarps;
+    constexpr uint32_t row_stride = kPairN + 16, mt_step = 32u * row_stride;
+    const uint32_t scr0 = c.sbase + p.scratch_off + (uint32_t)c.warp * (2u * mt_step);
+    const uint32_t scr_row = scr0 + (uint32_t)lane * row_stride;
+    const int crow = lane >> 2, cchunk = lane & 3;
+    const uint32_t scr_co = scr0 + (uint32_t)crow * row_stride + (uint32_t)cchunk * 16u;
+    const size_t co_step = (size_t)8 * L.coutp, co_mt = (size_t)kTileM * L.coutp;
+    // this lane's coalesced position in tile t; `rem` pixels of the tensor are left at the warp's first row
+    auto tile_ptr = [&](const int8_t *base, uint32_t t, uint32_t &rem) {
+        const uint32_t m_idx = t / (uint32_t)tiles_n, m0 = m_idx * (2u * kTileM) + (uint32_t)q * 32u;
+        rem = m0 < p.m_total ? p.m_total - m0 : 0u;
+        return base + (size_t)(m0 + (uint32_t)crow) * L.coutp + (int)(t - m_idx * tiles_n) * kPairN + cchunk * 16;
+    };
+    auto residual_fetch = [&](const int8_t *src, uint32_t rem, int c0) {
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if ((uint32_t)(mt * kTileM + 8 * k + crow) < rem)
+                    cp_async16(scr_co + (uint32_t)mt * mt_step + (uint32_t)(8 * k) * row_stride + (uint32_t)c0, src + (size_t)mt * co_mt + (size_t)k * co_step + c0);
+    };
+    const uint32_t t_step = (uint32_t)kEpiTeams * c.grid_n;
+    uint32_t t = blockIdx.x + (uint32_t)team * c.grid_n;
+    if (kRes && t < c.n_tiles) {
+        uint32_t rem;
+        const int8_t *src = tile_ptr(p.res, t, rem);
+        for (int c0 = 0; c0 < kPairN; c0 += 64) residual_fetch(src, rem, c0);
+    }
+    const uint32_t acc0 = c.tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(team * p.acc_stride);
+    for (int au = 0; t < c.n_tiles; t += t_step, ++au) {
+        const int n0 = (int)(t % (uint32_t)tiles_n) * kPairN;
+        uint32_t rem, rem_next = 0;
+        int8_t *dst = const_cast<int8_t *>(tile_ptr(p.out, t, rem));
+        const int8_t *res_next = (kRes && t + t_step < c.n_tiles) ? tile_ptr(p.res, t + t_step, rem_next) : nullptr;
+        if (kRes) cp_async_wait_all();                              // the tile's residual rows, requested during the previous tile
+        __syncwarp();
+        if (!wait_bar<kHintEpi>(c.acc_full + 8u * (uint32_t)team, (uint32_t)au & 1u, c.abort_flag)) {
+            cp_async_wait_all();
+            return false;
+        }
+        tc_fence_after();
+        const uint32_t cst0 = c.cst_s + (uint32_t)n0 * 16u;
+        auto load = [&](int (&a)[2][16], int cc) {
+            tmem_ld16_issue(acc0 + (uint32_t)cc, a[0]);
+            tmem_ld16_issue(acc0 + (uint32_t)(kPairN + cc), a[1]);
+        };
+        auto step = [&](int (&a)[2][16], int cc) {
+            const uint32_t scr = scr_row + (uint32_t)cc;
+            uint32_t r0[4] = {0, 0, 0, 0}, r1[4] = {0, 0, 0, 0};
+            if (kRes) {
+                const uint4 u = ld_shared_v4(scr), v = ld_shared_v4(scr + mt_step);
+                r0[0] = u.x ^ 0x80808080u; r0[1] = u.y ^ 0x80808080u; r0[2] = u.z ^ 0x80808080u; r0[3] = u.w ^ 0x80808080u;
+                r1[0] = v.x ^ 0x80808080u; r1[1] = v.y ^ 0x80808080u; r1[2] = v.z ^ 0x80808080u; r1[3] = v.w ^ 0x80808080u;
+            }
+            uint4 o[2];
+            requant16x2<kRes, kClamp>(a, cst0 + (uint32_t)cc * 16u, r0, r1, p.res_m2, p.res_r2, p.res_k8, p.lo, o);
+            st_shared_v4(scr, o[0]);
+            st_shared_v4(scr + mt_step, o[1]);
+        };
+        int acc_a[2][16], acc_b[2][16];
+        load(acc_a, 0);
+#pragma unroll 1
+        for (int cc = 0; cc < kPairN; cc += 32) {
+            tmem_ld32_wait(acc_a);
+            load(acc_b, cc + 16);
+            step(acc_a, cc);
+            tmem_ld32_wait(acc_b);
+            if (cc + 32 < kPairN) {
+                load(acc_a, cc + 32);
+            } else {
+                tc_fence_before();
+                mbar_arrive(c.acc_free + 8u * (uint32_t)team);      // the accumulators are in registers: the next tile may overwrite them
+            }
+            step(acc_b, cc + 16);
+            if (!(cc & 32)) continue;
+            const int c0 = cc - 32;
+            __syncwarp();
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt) {
+                uint4 v[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) v[k] = ld_shared_v4(scr_co + (uint32_t)mt * mt_step + (uint32_t)(8 * k) * row_stride + (uint32_t)c0);
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if ((uint32_t)(mt * kTileM + 8 * k + crow) < rem) *reinterpret_cast<uint4 *>(dst + (size_t)mt * co_mt + (size_t)k * co_step + c0) = v[k];
+            }
+            __syncwarp();
+            if (res_next) residual_fetch(res_next, rem_next, c0);
+        }
+    }
+    cp_async_wait_all();
+    return true;
+}
+
 // kWhole: input channels and output tiles are multiples of 64 (what the wide bottleneck networks consist of); the other
 // form takes any layer.  Two kernels, because the general form's masks cost registers and a tenth of the speed.
-template <bool kWhole>
+// kPair: tiles of 256 pixels x 128 channels, operand rows by tensor copy (see igemm_paired).
+template <bool kWhole, bool kPair>
 __global__ void __launch_bounds__(kGemmThreads, 1) k_igemm(const __grid_constant__ IgemmParams p)
 {
     extern __shared__ __align__(128) uint8_t smem[];            // operand stages | requantisation constants | epilogue scratch
@@ -215,7 +323,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_igemm(const __grid_constant
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t sbase = smem_u32(smem);
     const int n_tile = p.n_tile, stages = p.stages;
-    const uint32_t a_bytes = kTileM * kBlockK, b_bytes = (uint32_t)n_tile * kBlockK, stage_bytes = a_bytes + b_bytes;
+    constexpr uint32_t a_half = kTileM * kBlockK, a_bytes = kPair ? 2 * a_half : a_half;
+    const uint32_t b_bytes = (uint32_t)n_tile * kBlockK, stage_bytes = a_bytes + b_bytes;
     int4 *cst_s = reinterpret_cast<int4 *>(smem + (size_t)stages * stage_bytes);
     if (tid == 0) {
         for (int s = 0; s < stages; ++s) { mbar_init(smem_u32(&bar_full[s]), p.tma_a ? 1 : kGatherWarps * 32 + 1); mbar_init(smem_u32(&bar_free[s]), 1); }
@@ -244,6 +353,12 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_igemm(const __grid_constant
         c.acc_full = smem_u32(&bar_acc_full[0]); c.acc_free = smem_u32(&bar_acc_free[0]);
         c.abort_flag = &abort_s;
         const bool fast = p.fast_requant && (!p.res || p.fast_residual);
+        if constexpr (kPair) {
+            const bool clamp = p.lo > -128;
+            if (p.res && p.res_short) ok = clamp ? epilogue_pair<3, true>(p, c) : epilogue_pair<3, false>(p, c);
+            else if (p.res) ok = clamp ? epilogue_pair<2, true>(p, c) : epilogue_pair<2, false>(p, c);
+            else ok = clamp ? epilogue_pair<1, true>(p, c) : epilogue_pair<1, false>(p, c);
+        } else
         if (fast && p.res && p.res_short) ok = epilogue_role<3, kWhole>(p, c);
         else if (fast && p.res) ok = epilogue_role<2, kWhole>(p, c);
         else if (fast) ok = epilogue_role<1, kWhole>(p, c);
@@ -260,7 +375,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_igemm(const __grid_constant
         const uint32_t dst0 = sbase + (uint32_t)chunk * 2048u + (uint32_t)(32 * gw + rsub) * 16u;
         Ring ring;
         const uint32_t px_per_sample = (uint32_t)(L.hout * L.wout);
-        for (uint32_t t = blockIdx.x; t < n_tiles && ok && !p.tma_a; t += grid_n) {
+        for (uint32_t t = blockIdx.x; t < n_tiles && ok && !kPair && !p.tma_a; t += grid_n) {
             const uint32_t m0 = (t / (uint32_t)tiles_n) * kTileM + (uint32_t)(32 * gw + rsub);
             int iy0[4], ix0[4], off[4];                         // this lane's four rows: 8 apart
 #pragma unroll
@@ -343,6 +458,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_igemm(const __grid_constant
                         const uint64_t ad = make_desc(stage + (uint32_t)k2 * 4096u, 2048u, 128u);
                         const uint64_t bd = make_desc(stage + a_bytes + (uint32_t)k2 * 2u * (uint32_t)n_tile * 16u, (uint32_t)n_tile * 16u, 128u);
                         mma_i8(tmem + (uint32_t)(buf * p.acc_stride), ad, bd, idesc, (kb > 0 || k2 > 0) ? 1u : 0u);
+                        if (kPair) mma_i8(tmem + (uint32_t)(buf * p.acc_stride + kPairN), ad + (uint64_t)(a_half >> 4), bd, idesc, (kb > 0 || k2 > 0) ? 1u : 0u);
                     }
                     commit_to(smem_u32(&bar_free[ring.s]));
                 }
@@ -365,9 +481,12 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_igemm(const __grid_constant
                     if (p.tma_a) {
                         // box {16 bytes, 128 pixels, 4 columns} of the 3-D view lands as [column][pixel][16 bytes], which is
                         // the K-major core-matrix layout; pixels beyond the last one are filled with zeros and never stored
-                        asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
-                                     ::"r"(sbase + (uint32_t)ring.s * stage_bytes), "l"(reinterpret_cast<uint64_t>(&p.tmap_a)), "r"(0),
-                                       "r"((int)((t / (uint32_t)tiles_n) * kTileM)), "r"(kb * 4), "r"(smem_u32(&bar_full[ring.s])) : "memory");
+#pragma unroll
+                        for (int mt = 0; mt < (kPair ? 2 : 1); ++mt)
+                            asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+                                         ::"r"(sbase + (uint32_t)ring.s * stage_bytes + (uint32_t)mt * a_half), "l"(reinterpret_cast<uint64_t>(&p.tmap_a)), "r"(0),
+                                           "r"((int)((t / (uint32_t)tiles_n) * (kPair ? 2 * kTileM : kTileM)) + mt * kTileM), "r"(kb * 4),
+                                           "r"(smem_u32(&bar_full[ring.s])) : "memory");
                     }
                     bulk_g2s(sbase + (uint32_t)ring.s * stage_bytes + a_bytes, wtile + (size_t)kb * b_bytes, b_bytes, smem_u32(&bar_full[ring.s]));
                 }
@@ -581,18 +700,41 @@ __global__ void __launch_bounds__(kStemThreads, 2) k_stem(const __grid_constant_
 
 // ------------------------------------------------------------------ host side
 
+namespace {
+
+// Paired tiles are 128 channels wide, and an MMA of that width reads its operands at the shared memory's full bandwidth.
+// That pays where there are no more than 128 channels (the tile is as wide anyway) and in short reductions, where the
+// epilogue's constants weigh more (512 -> 256 channels at 28 x 28 became 84 -> 121 us, 512 -> 2048 at 7 x 7 57 -> 76 us).
+bool igemm_pairable(const GLayer &G)
+{
+    return G.kh == 1 && G.kw == 1 && G.stride == 1 && G.pad == 0 && G.cinp % kBlockK == 0 && G.coutp % kPairN == 0 &&
+           (G.coutp == kPairN || G.cinp <= 128);
+}
+
+// Whether a launch of `tiles_m` x `tiles_n` single tiles, which the CTAs take in rounds, pairs them: unless the coarser
+// rounds would cost more than the cheaper epilogue saves (a fifth).
+bool igemm_paired(uint32_t tiles_m, uint32_t tiles_n, uint32_t n_sms)
+{
+    const uint32_t single = (tiles_m * tiles_n + n_sms - 1) / n_sms, pairs = ((tiles_m + 1) / 2 * tiles_n + n_sms - 1) / n_sms;
+    return 8 * pairs <= 5 * single;
+}
+
+}  // namespace
+
 // Output channels in as few tiles of at most 256 as possible, all of the same width (a multiple of 16; the last one may
 // be partly padding).  Every convolution and FC layer fits; pools do not.
+// A 1 x 1 stride-1 layer for which paired tiles pay has tiles of 128, whether a launch pairs them or not.
 int igemm_tile_n(const GLayer &G)
 {
     if (G.op != ISC_CONV2D && G.op != ISC_FC) return 0;
+    if (igemm_pairable(G)) return kPairN;
     const int tiles = (G.coutp + 255) / 256;
     return ((G.coutp + tiles - 1) / tiles + 15) & ~15;
 }
 
 namespace {
 
-int igemm_tiles(const GLayer &G) { return (G.coutp + 255) / 256; }
+int igemm_tiles(const GLayer &G) { return igemm_pairable(G) ? G.coutp / kPairN : (G.coutp + 255) / 256; }
 int igemm_units(const GLayer &G) { return G.kh * G.kw * (G.cinp / 16); }
 int igemm_blocks(const GLayer &G) { return (igemm_units(G) + 3) / 4; }
 
@@ -628,7 +770,7 @@ void igemm_pack_weights(const GLayer &G, const int8_t *w, int8_t *out)
 // 32-bit row and byte offsets inside the kernel
 bool igemm_fits(const GLayer &G, int64_t batch)
 {
-    return batch * G.hout * G.wout * igemm_tiles(G) < (1ll << 31) - 512 && batch * G.hin * G.win * G.cinp < (1ll << 31);
+    return batch * G.hout * G.wout * ((G.coutp + 255) / 256) < (1ll << 31) - 512 && batch * G.hin * G.win * G.cinp < (1ll << 31);
 }
 
 // The residual term F(u) = floor((u * m2 + R2) / 2^32), u = r + 128 in 0..255 (see requant16_fast), as
@@ -740,38 +882,42 @@ cudaError_t launch_igemm_conv(const GLayer &G, const int8_t *wpack, const int32_
     p.tiles_n = igemm_tiles(G);
     p.units = igemm_units(G);
     p.n_blocks = igemm_blocks(G);
-    p.acc_stride = (p.n_tile + 31) & ~31;                        // the epilogue loads 32 columns at a time
-    p.tmem_cols = 64;
-    while (p.tmem_cols < 2 * p.acc_stride) p.tmem_cols <<= 1;
     if (!igemm_fits(G, batch)) return cudaErrorInvalidValue;
     p.zp_run = wpack + igemm_pack_bytes(G) - kBlockK;
     p.m_total = (uint32_t)((long long)batch * G.hout * G.wout);
     p.tiles_m = (p.m_total + kTileM - 1) / kTileM;
     p.in = in; p.res = res; p.out = out; p.wpack = wpack; p.err = err;
     if (p.tiles_m == 0) return cudaSuccess;
-    // as many operand stages as fit beside the constants, at most kMaxStages
-    const size_t stage_bytes = (size_t)kTileM * kBlockK + (size_t)p.n_tile * kBlockK, cst_bytes = (size_t)p.tiles_n * p.n_tile * 16;
-    const size_t scratch_bytes = (size_t)kAllEpiWarps * 32 * epi_row_stride(p.n_tile);
     const size_t smem_limit = 226 * 1024;
-    if (cst_bytes + scratch_bytes + 2 * stage_bytes > smem_limit) return cudaErrorInvalidValue;
-    p.stages = (int)std::min<size_t>(kMaxStages, (smem_limit - cst_bytes - scratch_bytes) / stage_bytes);
-    p.scratch_off = (uint32_t)((size_t)p.stages * stage_bytes + cst_bytes);
-    const size_t smem = (size_t)p.stages * stage_bytes + cst_bytes + scratch_bytes;
     static int n_sms = 0;
     if (n_sms == 0) {
         int dev = 0;
         cudaError_t e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_limit);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_limit);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_limit);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_limit);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_limit);
         if (e != cudaSuccess) { n_sms = 0; return e; }
     }
+    const bool paired = igemm_pairable(G) && p.tma_a && p.fast_requant && (!res || p.fast_residual) && igemm_paired(p.tiles_m, (uint32_t)p.tiles_n, (uint32_t)n_sms);
+    if (paired) p.tiles_m = (p.tiles_m + 1) / 2;
+    p.acc_stride = paired ? 2 * kPairN : (p.n_tile + 31) & ~31;          // the epilogue loads 32 columns at a time
+    p.tmem_cols = 64;
+    while (p.tmem_cols < 2 * p.acc_stride) p.tmem_cols <<= 1;
+    // as many operand stages as fit beside the constants, at most kMaxStages
+    const size_t stage_bytes = (size_t)kTileM * kBlockK * (paired ? 2 : 1) + (size_t)p.n_tile * kBlockK, cst_bytes = (size_t)p.tiles_n * p.n_tile * 16;
+    const size_t scratch_bytes = (size_t)kAllEpiWarps * 32 * (paired ? 2 : 1) * epi_row_stride(p.n_tile);
+    if (cst_bytes + scratch_bytes + 2 * stage_bytes > smem_limit) return cudaErrorInvalidValue;
+    p.stages = (int)std::min<size_t>(kMaxStages, (smem_limit - cst_bytes - scratch_bytes) / stage_bytes);
+    p.scratch_off = (uint32_t)((size_t)p.stages * stage_bytes + cst_bytes);
+    const size_t smem = (size_t)p.stages * stage_bytes + cst_bytes + scratch_bytes;
     // persistent: one CTA per SM (shared memory and the 512 tensor-memory columns allow no second one at N = 256)
     const uint32_t n_tiles = p.tiles_m * (uint32_t)p.tiles_n;
     const unsigned grid = std::min<uint32_t>(n_tiles, (uint32_t)n_sms);
     const bool whole = G.cinp % kBlockK == 0 && p.n_tile % 64 == 0 && G.coutp == p.tiles_n * p.n_tile;
-    if (whole) k_igemm<true><<<grid, kGemmThreads, smem, st>>>(p);
-    else k_igemm<false><<<grid, kGemmThreads, smem, st>>>(p);
+    if (paired) k_igemm<true, true><<<grid, kGemmThreads, smem, st>>>(p);
+    else if (whole) k_igemm<true, false><<<grid, kGemmThreads, smem, st>>>(p);
+    else k_igemm<false, false><<<grid, kGemmThreads, smem, st>>>(p);
     return cudaGetLastError();
 }
 
