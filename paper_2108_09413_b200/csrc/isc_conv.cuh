@@ -174,6 +174,26 @@ __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, const vo
     }
 }
 
+// A wait of a whole warp: every lane polls, all go on together.
+__device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, const volatile int *abort_flag)
+{
+    return __all_sync(0xffffffffu, wait_bar<kHintMma>(bar, parity, abort_flag)) != 0;
+}
+
+// MMA and commit by one lane of a converged warp: predicated, no branch
+__device__ __forceinline__ void mma_i8_if(uint32_t lane0, uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate)
+{
+    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+                 "@q tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
+                 ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(lane0) : "memory");
+}
+__device__ __forceinline__ void commit_if(uint32_t lane0, uint32_t bar)
+{
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+                 "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+                 ::"r"(bar), "r"(lane0) : "memory");
+}
+
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src)
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");

@@ -53,8 +53,8 @@ constexpr int kTileM = 128;
 constexpr int kBlockK = 64;                  // bytes of K per stage: two MMA K-steps
 constexpr int kMaxStages = 16;
 constexpr int kPairN = 128;                  // channels of a paired tile: two operands of 128 rows, two tiles in tensor memory
-constexpr int kStemThreads = 256;           // k_stem: two threads per tile row; two CTAs per SM (registers allow no third, nor two of 512 threads)
-constexpr size_t kStemSmemLimit = 108 * 1024;          // dynamic shared memory of k_stem: two CTAs per SM
+constexpr int kStemEpi = 8, kStemThreads = 32 * (kStemEpi + 1);        // k_stem: two threads per tile row and the MMA warp; two CTAs per SM
+constexpr size_t kStemSmemPair = 108 * 1024, kStemSmemLimit = 220 * 1024;       // dynamic shared memory of k_stem: for two CTAs per SM; at most
 constexpr int kEpiWarps = 4, kEpiTeams = 2, kGatherWarps = 4;          // a team of epilogue warps takes every other tile
 constexpr int kAllEpiWarps = kEpiWarps * kEpiTeams;
 static_assert(kEpiWarps == 4, "an epilogue warp owns all N columns of its 32 rows");
@@ -516,14 +516,23 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_igemm(const __grid_constant
 // One CTA = one sample x one band of output rows.  The band's input rows are drawn (Philox -> inverse-CDF table ->
 // add -> saturate to 0..255, Def. 3.3 / Eq. 2) into a shared-memory patch as 4 bytes per pixel, padded with the input
 // zero-point, and never written to memory.  The GEMM takes one filter row per K-step: eight horizontally adjacent
-// pixels x 4 bytes = 32 bytes of K (pixels beyond the filter width meet zero weights), so a tile of 128 output pixels
-// is `kh` MMAs.  Each thread copies its pixel's `kh` windows from the patch into the K-major operand stage; tiles
-// alternate between two stages and two halves of the accumulator columns, so the requantisation of one tile runs
-// while the MMAs of the next are in flight.
+// pixels x 4 bytes = 32 bytes of K (pixels beyond the filter width meet zero weights), so 128 output pixels are `kh`
+// MMAs.  The patch is spread once into positions of 16 bytes, position i of a row being the four pixels from i * stride
+// on, with the rows ordered by (row mod stride, row / stride): output pixel (y, x) then reads filter row r at position
+// r's first + y * pitch + x, and a filter row is an address offset of the operand descriptor (the second 16 bytes of K
+// lie 4 / stride positions on, or in a second plane when that is no whole number).  Copying each output pixel's kh
+// windows into an operand stage moved five times as many bytes and put a CTA barrier before every tile.  A tile is
+// 256 positions (two M operands), so that a thread requantises two rows and reads a channel's constants once for both;
+// the positions behind a row's last pixel are computed and not stored.  A ninth warp issues the MMAs.  7 x 7 stride 2 on
+// 224 x 224, 512 samples: 975 -> 823 us; 3 x 3 on 32 x 32, 4096 samples: 352 -> 311 us.  What is left is the noise: its
+// Philox rounds and table searches take the integer pipes for most of the kernel's time.
 struct StemParams {
     GLayer L;
-    int in_c, band_rows, n_bands, tiles_per_band, tmem_cols;
-    uint32_t patch_bytes, w_bytes;
+    int in_c, band_rows, n_bands, tmem_cols;
+    int pitch, rows_class, planes;           // positions of a row; rows of one (row mod stride) class; planes of positions
+    uint32_t plane_pos, k_step;              // positions of a plane; bytes from the first to the second 16 bytes of K
+    uint32_t w_bytes, pos_off, patch_off;
+    int slots;                               // pairs of accumulators in tensor memory
     uint32_t tab_off;                        // the noise tables' copy in shared memory (after the patch), 0: searched in global memory
     const uint8_t *x;                        // clean image, CHW
     NoiseStream ns;
@@ -534,23 +543,68 @@ struct StemParams {
     int32_t *err;
 };
 
+// Rows 32 (warp mod 4) .. + 31 of both operands of every tile, half of the channels.
+template <bool kFast, bool kClamp>
+__device__ __forceinline__ bool stem_epilogue(const StemParams &p, uint32_t tmem, uint32_t cst, uint32_t bar_full, uint32_t bar_free, int n_tiles, int band_rows,
+                                              size_t first_px, const volatile int *abort_flag)
+{
+    const GLayer &L = p.L;
+    const int N = L.coutp, row = (int)threadIdx.x & (kTileM - 1), half = (N / 16 + 1) / 2 * 16;
+    const int c_begin = threadIdx.x >= kTileM ? half : 0, c_end = threadIdx.x >= kTileM ? N : half;
+    const uint32_t lanes = tmem + ((uint32_t)(row & ~31) << 16);
+    for (int t = 0; t < n_tiles; ++t) {
+        const int slot = p.slots == 2 ? t & 1 : 0, use = p.slots == 2 ? t >> 1 : t;
+        int8_t *dst[2];
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt) {
+            const int f = t * 2 * kTileM + mt * kTileM + row, y = f / p.pitch, x = f - y * p.pitch;
+            dst[mt] = y < band_rows && x < L.wout ? p.out + (first_px + (size_t)(y * L.wout + x)) * L.coutp : nullptr;
+        }
+        if (!wait_bar<kHintEpi>(bar_full + 8u * (uint32_t)slot, (uint32_t)use & 1u, abort_flag)) return false;
+        tc_fence_after();
+        const uint32_t acc = lanes + (uint32_t)(slot * 2 * N);
+#pragma unroll 1
+        for (int c0 = c_begin; c0 < c_end; c0 += 16) {
+            int a[2][16];
+            tmem_ld16_issue(acc + (uint32_t)c0, a[0]);
+            tmem_ld16_issue(acc + (uint32_t)(N + c0), a[1]);
+            tmem_ld32_wait(a);
+            uint4 o[2];
+            if (kFast) {
+                const uint32_t none[4] = {0, 0, 0, 0};
+                requant16x2<0, kClamp>(a, cst + (uint32_t)c0 * 16u, none, none, 0u, 0ll, 0u, p.lo, o);
+            } else {
+#pragma unroll
+                for (int mt = 0; mt < 2; ++mt) {
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) a[mt][k] += __ldg(L.bias + c0 + k);
+                    o[mt] = epilogue16(a[mt], L, c0, nullptr);
+                }
+            }
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt)
+                if (dst[mt]) *reinterpret_cast<uint4 *>(dst[mt] + c0) = o[mt];
+        }
+        tc_fence_before();
+        mbar_arrive(bar_free + 8u * (uint32_t)slot);
+    }
+    return true;
+}
+
 __global__ void __launch_bounds__(kStemThreads, 2) k_stem(const __grid_constant__ StemParams p)
 {
-    extern __shared__ __align__(128) uint8_t smem[];
-    __shared__ unsigned long long bar_w, bar_full[2];
+    extern __shared__ __align__(128) uint8_t smem[];        // weights | positions | patch | noise tables
+    __shared__ unsigned long long bar_w, bar_full[2], bar_free[2];
     __shared__ uint32_t tmem_base_s;
     __shared__ volatile int abort_s;
     __shared__ __align__(16) int4 cst_s[256];
     const GLayer &L = p.L;
-    const int tid = threadIdx.x, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = (int)warp_uniform((uint32_t)tid >> 5);
     const uint32_t sbase = smem_u32(smem);
     const int N = L.coutp, kh = L.kh;
-    const uint32_t a_bytes = (uint32_t)kh * kTileM * 32u;
-    const uint32_t w_off = 0, a_off = p.w_bytes, patch_off = a_off + 2u * a_bytes;        // weights | two operand stages | patch
     if (tid == 0) {
         mbar_init(smem_u32(&bar_w), 1);
-        mbar_init(smem_u32(&bar_full[0]), 1);
-        mbar_init(smem_u32(&bar_full[1]), 1);
+        for (int i = 0; i < 2; ++i) { mbar_init(smem_u32(&bar_full[i]), 1); mbar_init(smem_u32(&bar_free[i]), 2 * kTileM); }
         abort_s = 0;
     }
     if (warp == 0) tmem_alloc(smem_u32(&tmem_base_s), (uint32_t)p.tmem_cols);
@@ -563,7 +617,7 @@ __global__ void __launch_bounds__(kStemThreads, 2) k_stem(const __grid_constant_
     const uint32_t tmem = tmem_base_s;
     if (tid == 0) {
         mbar_expect_tx(smem_u32(&bar_w), p.w_bytes);
-        bulk_g2s(sbase + w_off, p.wpack, p.w_bytes, smem_u32(&bar_w));
+        bulk_g2s(sbase, p.wpack, p.w_bytes, smem_u32(&bar_w));
     }
 
     // ---- the band's noisy input rows
@@ -573,7 +627,7 @@ __global__ void __launch_bounds__(kStemThreads, 2) k_stem(const __grid_constant_
     const int wpad = L.win + 2 * L.pad + 8;                     // 8 more pixels: the windows of the last columns stay inside
     const int iy0 = oy0 * L.stride - L.pad;
     const int rows_in = (oy1 - oy0 - 1) * L.stride + kh;
-    uint32_t *patch = reinterpret_cast<uint32_t *>(smem + patch_off);
+    uint32_t *patch = reinterpret_cast<uint32_t *>(smem + p.patch_off);
     const uint32_t zp_fill = (uint32_t)(L.zp_in & 0xFF) * (0x01010101u >> (8 * (4 - p.in_c)));
     for (int i = tid; i < rows_in * wpad; i += kStemThreads) patch[i] = zp_fill;
     if (p.tab_off && p.ns.guide) {
@@ -627,68 +681,50 @@ __global__ void __launch_bounds__(kStemThreads, 2) k_stem(const __grid_constant_
     }
     __syncthreads();
 
-    // ---- tiles of 128 output pixels of the band.  Thread = tile row `px` x one of kStemThreads / 128 groups: the
-    // groups share the filter rows' windows and the 16-channel chunks round-robin.
-    const int band_px = (oy1 - oy0) * L.wout;
-    const int n_tiles = (band_px + kTileM - 1) / kTileM;
-    const uint32_t idesc = (2u << 4) | (0u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(kTileM >> 4) << 24);
-    const int px_row = tid & (kTileM - 1), grp = tid >> 7;
+    // ---- the patch as positions (see above)
+    const uint32_t pos = sbase + p.pos_off;
+    for (int i = tid; i < p.planes * rows_in * p.pitch; i += kStemThreads) {
+        int y = i / p.pitch;
+        const int x = i - y * p.pitch, plane = y >= rows_in ? 1 : 0;
+        y -= plane * rows_in;
+        const uint32_t *src = patch + y * wpad + x * L.stride + 4 * plane;
+        const int at = (y % L.stride * p.rows_class + y / L.stride) * p.pitch + x;
+        st_shared_v4(pos + ((uint32_t)plane * p.plane_pos + (uint32_t)at) * 16u, make_uint4(src[0], src[1], src[2], src[3]));
+    }
+    fence_proxy_async();
+    __syncthreads();
+
+    const int band_rows = oy1 - oy0, n_tiles = (band_rows * p.pitch + 2 * kTileM - 1) / (2 * kTileM);
     bool ok = true;
-    if (tid == 0) ok = wait_bar(smem_u32(&bar_w), 0);
-    for (int t = 0; t <= n_tiles; ++t) {
-        if (t < n_tiles) {
-            // operand stage of tile t: free once the MMAs of tile t - 2 are complete (waited for by its epilogue below)
-            const uint32_t stage = sbase + a_off + (uint32_t)(t & 1) * a_bytes;
-            const int px = t * kTileM + px_row;
-            const int pp = px < band_px ? px : 0;
-            const int oyl = pp / L.wout, ox = pp - oyl * L.wout;
-            for (int r = grp; r < kh; r += kStemThreads / kTileM) {
-                const uint32_t *src = patch + (oyl * L.stride + r) * wpad + ox * L.stride;
-                st_shared_v4(stage + (uint32_t)r * 4096u + 0u * 2048u + px_row * 16, make_uint4(src[0], src[1], src[2], src[3]));
-                st_shared_v4(stage + (uint32_t)r * 4096u + 1u * 2048u + px_row * 16, make_uint4(src[4], src[5], src[6], src[7]));
+    if (warp < kStemEpi) {
+        const size_t first_px = ((size_t)b * L.hout + oy0) * L.wout;
+        const uint32_t cst = smem_u32(cst_s), full = smem_u32(&bar_full[0]), free_ = smem_u32(&bar_free[0]);
+        if (!p.fast_requant) ok = stem_epilogue<false, true>(p, tmem, cst, full, free_, n_tiles, band_rows, first_px, &abort_s);
+        else if (p.lo > -128) ok = stem_epilogue<true, true>(p, tmem, cst, full, free_, n_tiles, band_rows, first_px, &abort_s);
+        else ok = stem_epilogue<true, false>(p, tmem, cst, full, free_, n_tiles, band_rows, first_px, &abort_s);
+    } else {
+        const uint32_t lane0 = elect_one() ? 1u : 0u;
+        const uint32_t idesc = (2u << 4) | (0u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(kTileM >> 4) << 24);
+        ok = wait_warp(smem_u32(&bar_w), 0u, &abort_s);
+        tc_fence_after();
+        for (int t = 0; t < n_tiles && ok; ++t) {
+            const int slot = p.slots == 2 ? t & 1 : 0, use = p.slots == 2 ? t >> 1 : t;
+            if (use >= 1) {
+                ok = wait_warp(smem_u32(&bar_free[slot]), (uint32_t)(use - 1) & 1u, &abort_s);
+                if (!ok) break;
+                tc_fence_after();
             }
-            fence_proxy_async();
-        }
-        __syncthreads();
-        if (t < n_tiles && tid == 0) {
-            tc_fence_after();
-            if (ok && !abort_s) {
-                const uint32_t stage = sbase + a_off + (uint32_t)(t & 1) * a_bytes;
+            for (int mt = 0; mt < 2; ++mt)
                 for (int r = 0; r < kh; ++r) {
-                    const uint64_t ad = make_desc(stage + (uint32_t)r * 4096u, 2048u, 128u);
-                    const uint64_t bd = make_desc(sbase + w_off + (uint32_t)r * 2u * (uint32_t)N * 16u, (uint32_t)N * 16u, 128u);
-                    mma_i8(tmem + (uint32_t)(t & 1) * (uint32_t)N, ad, bd, idesc, r > 0 ? 1u : 0u);
+                    const int at = (r % L.stride * p.rows_class + r / L.stride) * p.pitch + t * 2 * kTileM + mt * kTileM;
+                    const uint64_t ad = make_desc(pos + (uint32_t)at * 16u, p.k_step, 128u);
+                    const uint64_t bd = make_desc(sbase + (uint32_t)r * 2u * (uint32_t)N * 16u, (uint32_t)N * 16u, 128u);
+                    mma_i8_if(lane0, tmem + (uint32_t)((slot * 2 + mt) * N), ad, bd, idesc, r > 0 ? 1u : 0u);
                 }
-            }
-            commit_to(smem_u32(&bar_full[t & 1]));
-        }
-        if (t >= 1) {
-            // epilogue of tile t - 1 while the MMAs of tile t run
-            const int tt = t - 1;
-            if (ok && !abort_s) ok = wait_bar(smem_u32(&bar_full[tt & 1]), (uint32_t)(tt >> 1) & 1u);
-            if (!ok) abort_s = 1;
-            tc_fence_after();
-            const int px = tt * kTileM + px_row;
-            const bool valid = px < band_px;
-            const size_t m = ((size_t)b * L.hout + oy0) * L.wout + (size_t)(valid ? px : 0);
-            for (int c0 = 16 * grp; c0 < N; c0 += 16 * (kStemThreads / kTileM)) {
-                int acc[16];
-                tmem_ld16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(tt & 1) * (uint32_t)N + (uint32_t)c0, acc);
-                if (valid && !abort_s) {
-                    uint4 v;
-                    if (p.fast_requant) {
-                        v = requant16_fast<0>(acc, smem_u32(cst_s + c0), make_uint4(0, 0, 0, 0), 0u, 0ll, 0u, p.lo);
-                    } else {
-#pragma unroll
-                        for (int o = 0; o < 16; ++o) acc[o] += __ldg(L.bias + c0 + o);
-                        v = epilogue16(acc, L, c0, nullptr);
-                    }
-                    *reinterpret_cast<uint4 *>(p.out + m * L.coutp + c0) = v;
-                }
-            }
-            tc_fence_before();
+            commit_if(lane0, smem_u32(&bar_full[slot]));
         }
     }
+    if (!ok) abort_s = 1;
     if (!ok) atomicCAS(p.err, 0, 1 + (int)blockIdx.x);
     tc_fence_before();
     __syncthreads();
@@ -923,28 +959,48 @@ cudaError_t launch_igemm_conv(const GLayer &G, const int8_t *wpack, const int32_
 
 // ---- the stem
 
+size_t stem_pack_bytes(const GLayer &G) { return (size_t)G.kh * G.coutp * 32; }
+
 namespace {
 
-int stem_band_rows(const GLayer &G)
+struct StemConfig {
+    int band_rows, pitch, rows_class, planes;
+    uint32_t plane_pos, k_step, w_bytes, pos_bytes, patch_bytes;
+    size_t smem() const { return (size_t)w_bytes + pos_bytes + patch_bytes; }
+};
+
+// Bands of eight output rows, or of fewer if two CTAs per SM and their noise tables do not fit otherwise.
+bool stem_config(const GLayer &G, int in_c, StemConfig *c)
 {
-    const int wpad = G.win + 2 * G.pad + 8;
-    int rows = 8;
-    while (rows > 1 && (size_t)((rows - 1) * G.stride + G.kh) * wpad * 4 > 24 * 1024) rows >>= 1;
-    return rows;
+    if (G.op != ISC_CONV2D || in_c > 4 || G.kw > 8 || G.kh > 8 || G.coutp % 16 != 0 || G.coutp > 256) return false;
+    const bool second = G.kw > 4, whole = 4 % G.stride == 0;
+    c->planes = second && !whole ? 2 : 1;
+    c->pitch = G.wout + (second && whole ? 4 / G.stride : 0);
+    c->w_bytes = (uint32_t)stem_pack_bytes(G);
+    for (int rows = 8; rows >= 1; rows >>= 1) {
+        const int rows_in = (rows - 1) * G.stride + G.kh;
+        const size_t patch = ((size_t)rows_in * (G.win + 2 * G.pad + 8) * 4 + 15) & ~(size_t)15;
+        c->band_rows = rows;
+        c->rows_class = (rows_in + G.stride - 1) / G.stride;
+        const size_t plane_pos = (size_t)G.stride * c->rows_class * c->pitch + 2 * kTileM + 8;        // the last tile reads beyond the last row
+        const size_t total = c->w_bytes + plane_pos * c->planes * 16 + patch;
+        if (total > (rows > 1 ? 94 : 214) * (size_t)1024) continue;
+        c->plane_pos = (uint32_t)plane_pos;
+        c->pos_bytes = (uint32_t)(plane_pos * c->planes * 16);
+        c->patch_bytes = (uint32_t)patch;
+        c->k_step = !second ? 16u : whole ? 16u * (uint32_t)(4 / G.stride) : c->plane_pos * 16u;
+        return c->k_step < (1u << 18);
+    }
+    return false;
 }
 
 }  // namespace
 
 bool stem_fits(const GLayer &G, int in_c)
 {
-    if (G.op != ISC_CONV2D || in_c > 4 || G.kw > 8 || G.kh > 8 || G.coutp % 16 != 0 || G.coutp > 256) return false;
-    const int rows = stem_band_rows(G);
-    const size_t patch = (size_t)((rows - 1) * G.stride + G.kh) * (G.win + 2 * G.pad + 8) * 4;
-    const size_t total = (size_t)G.kh * G.coutp * 32 + 2 * (size_t)G.kh * kTileM * 32 + patch;
-    return total <= 100 * 1024;
+    StemConfig c;
+    return stem_config(G, in_c, &c);
 }
-
-size_t stem_pack_bytes(const GLayer &G) { return (size_t)G.kh * G.coutp * 32; }
 
 // w: [cout][cin][kh][kw] -> [filter row][2 columns of 16 bytes][coutp rows][16]: byte pix * 4 + ch of a row's 32
 void stem_pack_weights(const GLayer &G, const int8_t *w, int8_t *out)
@@ -965,24 +1021,27 @@ cudaError_t launch_stem_conv(const GLayer &G, const int8_t *wpack, const int32_t
     StemParams p;
     p.L = G;
     p.in_c = in_c;
-    p.band_rows = stem_band_rows(G);
+    StemConfig c;
+    if (!stem_config(G, in_c, &c)) return cudaErrorInvalidValue;
+    p.band_rows = c.band_rows;
     p.n_bands = (G.hout + p.band_rows - 1) / p.band_rows;
-    p.tiles_per_band = (p.band_rows * G.wout + kTileM - 1) / kTileM;
+    p.pitch = c.pitch; p.rows_class = c.rows_class; p.planes = c.planes;
+    p.plane_pos = c.plane_pos; p.k_step = c.k_step;
+    p.w_bytes = c.w_bytes; p.pos_off = c.w_bytes; p.patch_off = c.w_bytes + c.pos_bytes;
+    p.slots = G.coutp <= 64 ? 2 : 1;                             // two CTAs share the 512 columns of an SM
     int cols = 32;
-    while (cols < 2 * G.coutp) cols <<= 1;
+    while (cols < p.slots * 2 * G.coutp) cols <<= 1;
     p.tmem_cols = cols;
-    p.w_bytes = (uint32_t)stem_pack_bytes(G);
-    p.patch_bytes = (uint32_t)(((p.band_rows - 1) * G.stride + G.kh) * (G.win + 2 * G.pad + 8) * 4);
     p.x = x_chw; p.ns = ns; p.wpack = wpack;
     p.cst = reinterpret_cast<const int4 *>(cst);
     p.fast_requant = fast ? 1 : 0;
     p.lo = G.relu ? (G.zp_out > -128 ? G.zp_out : -128) : -128;
     p.out = out; p.err = err;
-    size_t smem = (size_t)p.w_bytes + 2 * (size_t)G.kh * kTileM * 32 + p.patch_bytes;
+    size_t smem = c.smem();
     // the noise tables go to shared memory when two CTAs per SM still fit and the guide table follows the cumulative one
     const size_t tab_bytes = ((size_t)(2 * ns.T + 1 + kNoiseGuide + 1) * 4 + 15) & ~(size_t)15;
     p.tab_off = 0;
-    if (ns.guide == ns.cum + (2 * ns.T + 1) && smem + tab_bytes <= kStemSmemLimit) {
+    if (ns.guide == ns.cum + (2 * ns.T + 1) && smem + tab_bytes <= (smem <= kStemSmemPair ? kStemSmemPair : kStemSmemLimit)) {
         p.tab_off = (uint32_t)smem;
         smem += tab_bytes;
     }
