@@ -8,6 +8,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
+#include "isc_conv.cuh"
 #include "isc_epilogue.cuh"
 #include "isc_internal.h"
 
@@ -230,31 +233,51 @@ __global__ void k_gavgpool(GLayer L, int batch, const int8_t *__restrict__ in, i
     out[idx] = (int8_t)q;
 }
 
-__global__ void k_maxpool(GLayer L, int batch, const int8_t *__restrict__ in, int8_t *__restrict__ out)
+// Thread = one output pixel x 16 channels.  A tap outside the image repeats one inside the window, which changes no
+// maximum, so that all taps of a 3 x 3 window (K = 3) are loaded without branches and together; the maximum of signed
+// bytes is that of the 16-bit halves whose high byte they are (two packed maxima and a shift per four channels instead
+// of an emulated four-byte one).  With 64-bit index arithmetic and a branch per tap the 3 x 3 stride-2 pool of a 112 x 112
+// x 64 map took 146 us for 512 samples, now 84 us (6.1 TB/s of the measured 6.5).  K = 0: any window.
+template <int K>
+__global__ void k_maxpool(GLayer L, conv::FastDiv by_c16, conv::FastDiv by_w, uint32_t n, const int8_t *__restrict__ in, int8_t *__restrict__ out)
 {
-    const int c16s = L.cinp >> 4;
-    const int64_t total = (int64_t)batch * L.hout * L.wout * c16s;
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= total) return;
-    const int g = (int)(idx % c16s);
-    const int64_t px = idx / c16s;
-    const int ox = (int)(px % L.wout);
-    const int oy = (int)((px / L.wout) % L.hout);
-    const int b = (int)(px / ((int64_t)L.wout * L.hout));
-    uint4 m = make_uint4(0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u);
-    for (int r = 0; r < L.kh; ++r) {
-        const int iy = oy * L.stride + r - L.pad;
-        if (iy < 0 || iy >= L.hin) continue;
-        for (int s = 0; s < L.kw; ++s) {
-            const int ix = ox * L.stride + s - L.pad;
-            if (ix < 0 || ix >= L.win) continue;
-            const uint4 a = __ldg(reinterpret_cast<const uint4 *>(
-                in + (((size_t)b * L.hin + iy) * L.win + ix) * L.cinp) + g);
-            m.x = __vmaxs4(m.x, a.x); m.y = __vmaxs4(m.y, a.y);
-            m.z = __vmaxs4(m.z, a.z); m.w = __vmaxs4(m.w, a.w);
+    const uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= n) return;
+    uint32_t g, ox;
+    const uint32_t px = by_c16.divmod(idx, g), oy = by_w.divmod(px, ox);
+    const int kh = K ? K : L.kh, kw = K ? K : L.kw, y0 = (int)oy * L.stride - L.pad, x0 = (int)ox * L.stride - L.pad;
+    const int8_t *src = in + (size_t)blockIdx.y * L.hin * L.win * L.cinp + g * 16;
+    uint32_t odd[4], even[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) odd[k] = even[k] = 0x80008000u;
+    if (y0 + kh > 0 && y0 < L.hin && x0 + kw > 0 && x0 < L.win) {
+        auto tap = [&](int r, int c) {
+            const int iy = min(max(y0 + r, 0), L.hin - 1), ix = min(max(x0 + c, 0), L.win - 1);
+            return __ldg(reinterpret_cast<const uint4 *>(src + (size_t)(iy * L.win + ix) * L.cinp));
+        };
+        auto take = [&](const uint4 &a) {
+            const uint32_t w[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                odd[k] = __vmaxs2(odd[k], w[k]);
+                even[k] = __vmaxs2(even[k], w[k] << 8);
+            }
+        };
+        if (K) {
+            uint4 a[K ? K * K : 1];
+#pragma unroll
+            for (int i = 0; i < K * K; ++i) a[i] = tap(i / (K ? K : 1), i % (K ? K : 1));
+#pragma unroll
+            for (int i = 0; i < K * K; ++i) take(a[i]);
+        } else {
+            for (int r = 0; r < kh; ++r)
+                for (int c = 0; c < kw; ++c) take(tap(r, c));
         }
     }
-    *reinterpret_cast<uint4 *>(out + (size_t)px * L.cinp + g * 16) = m;
+    uint32_t m[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) m[k] = __byte_perm(even[k], odd[k], 0x7351u);
+    *reinterpret_cast<uint4 *>(out + ((size_t)blockIdx.y * L.hout * L.wout + px) * L.cinp + g * 16) = make_uint4(m[0], m[1], m[2], m[3]);
 }
 
 // ------------------------------------------------------------------ votes
@@ -328,8 +351,15 @@ cudaError_t launch_gavgpool(const GLayer &L, int batch, const int8_t *in, int8_t
 
 cudaError_t launch_maxpool(const GLayer &L, int batch, const int8_t *in, int8_t *out, cudaStream_t st)
 {
-    const int64_t n = (int64_t)batch * L.hout * L.wout * (L.cinp >> 4);
-    k_maxpool<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(L, batch, in, out);
+    const uint32_t n = (uint32_t)(L.hout * L.wout * (L.cinp >> 4));
+    const conv::FastDiv by_c16 = conv::FastDiv::make((uint32_t)(L.cinp >> 4)), by_w = conv::FastDiv::make((uint32_t)L.wout);
+    for (int b = 0; b < batch; b += 65535) {                     // a launch's second grid dimension holds no more
+        const dim3 grid((n + 127) / 128, (unsigned)std::min(batch - b, 65535));
+        const int8_t *src = in + (size_t)b * L.hin * L.win * L.cinp;
+        int8_t *dst = out + (size_t)b * L.hout * L.wout * L.cinp;
+        if (L.kh == 3 && L.kw == 3) k_maxpool<3><<<grid, 128, 0, st>>>(L, by_c16, by_w, n, src, dst);
+        else k_maxpool<0><<<grid, 128, 0, st>>>(L, by_c16, by_w, n, src, dst);
+    }
     return cudaGetLastError();
 }
 
