@@ -326,8 +326,7 @@ int isc_debug_residual_form(int32_t res_mult, int32_t res_shift, int32_t zp_res,
  *   "batch"  : noisy samples per launch (0 = choose automatically).
  *   "engine" : 0 = automatic (3 if the model fits it, else 2 if any layer fits it, else 1),
  *              1 = layer-by-layer kernels without tensor cores, 2 = layer-by-layer with
- *              the tcgen05 implicit-GEMM kernel for every convolution whose input and
- *              output channels are multiples of 64, 3 = the line-tiled
+ *              the tcgen05 kernels for every convolution and FC layer, 3 = the line-tiled
  *              shared-memory-resident tensor-core kernel (2 and 3 give
  *              ISC_ERR_UNSUPPORTED at the next call if the model does not fit).
  * isc_get_info reads back: "engine" (the engine the last call used; 1 after every

@@ -61,17 +61,6 @@ __device__ __forceinline__ void fence_proxy_async()
 {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
-__device__ __forceinline__ void st_release(uint32_t addr, uint32_t v)
-{
-    asm volatile("st.release.cta.shared::cta.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
-}
-__device__ __forceinline__ uint4 ld_acquire_v4(uint32_t addr)
-{
-    uint4 v;
-    asm volatile("ld.acquire.cta.shared::cta.v4.u32 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
-    return v;
-}
 __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint4 v)
 {
     asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
@@ -87,10 +76,6 @@ __device__ __forceinline__ uint32_t lds32(uint32_t addr)
     uint32_t v;
     asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
     return v;
-}
-__device__ __forceinline__ void named_bar(int id, int n)
-{
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -114,27 +99,6 @@ __device__ __forceinline__ bool elect_one()
 // A value every lane of the warp holds, in a form the compiler knows to be the same in all lanes.
 __device__ __forceinline__ uint32_t warp_uniform(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
 
-// The tensor-core instructions below are issued by one elected lane of a converged warp; their operands are
-// computed by the whole warp from warp-uniform values.
-__device__ __forceinline__ void mma_i8_first(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc)
-{
-    if (!elect_one()) return;
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, 0, 0;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
-                 ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc) : "memory");
-}
-__device__ __forceinline__ void mma_i8_acc(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc)
-{
-    if (!elect_one()) return;
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.b32 p, 0, 0;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
-                 ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc) : "memory");
-}
-__device__ __forceinline__ void mma_commit(uint32_t bar)
-{
-    if (!elect_one()) return;
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
 // asynchronous 16-column load of this thread's tensor-memory lane; the registers are valid after tmem_ld_wait()
 __device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, int (&v)[16])
 {
@@ -169,25 +133,6 @@ __device__ __forceinline__ uint32_t pack4_sat(int v0, int v1, int v2, int v3)
     asm("cvt.pack.sat.s8.s32.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(v1), "r"(v0), "r"(hi));
     return d;
 }
-// a * b + c as one 32x32+64 multiply-add
-// Per-channel requantisation constants as stored in the blob: the 64-bit addend, then multiplier and shift.
-// Loading the addend as one 64-bit register keeps it in an aligned register pair without any packing code.
-struct ChanConst { long long B; int mult, s; };
-__device__ __forceinline__ ChanConst ld_chan_const(uint32_t addr)
-{
-    long long b, ms;
-    asm volatile("ld.shared.v2.b64 {%0,%1}, [%2];" : "=l"(b), "=l"(ms) : "r"(addr));
-    ChanConst c;
-    c.B = b;
-    asm("mov.b64 {%0, %1}, %2;" : "=r"(c.mult), "=r"(c.s) : "l"(ms));
-    return c;
-}
-__device__ __forceinline__ long long mad_wide(int a, int b, long long c)
-{
-    long long d;
-    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
-    return d;
-}
 __device__ __forceinline__ int hi32(long long v)
 {
     int lo, hi;
@@ -200,15 +145,6 @@ __device__ __forceinline__ int lo32(long long v)
     asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "l"(v));
     return lo;
 }
-// byte K of w, sign-extended (one byte-permute with sign replication)
-template <int K>
-__device__ __forceinline__ int sbyte(uint32_t w)
-{
-    int d;
-    asm("prmt.b32 %0, %1, 0, %2;" : "=r"(d) : "r"(w), "n"(((8 | K) << 12) | ((8 | K) << 8) | ((8 | K) << 4) | K));
-    return d;
-}
-
 __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1)
 {
 #pragma unroll
