@@ -182,9 +182,10 @@ __device__ __forceinline__ int noise_level_guided(uint32_t u, const uint32_t *__
     return (int)lo - T;
 }
 
-// The same search for the four uniforms of one Philox block with a fixed number of bisection steps (`steps` covers the
-// widest guide interval; a step on an interval that has already closed changes nothing, since u < cum[result]), so
-// that the four dependent load chains run interleaved.
+// The same search for the four uniforms of one Philox block, step by step together, so that the four dependent load chains
+// run interleaved (a step on an interval that has already closed changes nothing, since u < cum[result]).  `steps`
+// covers the widest guide interval, which lies in the far tail and is ten steps wide; a warp's 128 uniforms seldom
+// need more than four, so the loop ends when all are found.
 __device__ __forceinline__ void noise_levels4(uint4 u4, const uint32_t *__restrict__ cum, const uint32_t *__restrict__ guide, int T,
                                               int steps, int (&z)[4])
 {
@@ -196,7 +197,7 @@ __device__ __forceinline__ void noise_levels4(uint4 u4, const uint32_t *__restri
         lo[k] = __ldg(guide + j);
         hi[k] = __ldg(guide + j + 1);
     }
-    for (int s = 0; s < steps; ++s) {
+    for (int s = 0; s < steps && ((lo[0] ^ hi[0]) | (lo[1] ^ hi[1]) | (lo[2] ^ hi[2]) | (lo[3] ^ hi[3])); ++s) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const uint32_t mid = (lo[k] + hi[k]) >> 1;
@@ -222,7 +223,7 @@ __device__ __forceinline__ void noise_levels4_shared(uint4 u4, uint32_t cum_s, u
         lo[k] = lds32(guide_s + 4u * j);
         hi[k] = lds32(guide_s + 4u * j + 4u);
     }
-    for (int s = 0; s < steps; ++s) {
+    for (int s = 0; s < steps && ((lo[0] ^ hi[0]) | (lo[1] ^ hi[1]) | (lo[2] ^ hi[2]) | (lo[3] ^ hi[3])); ++s) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const uint32_t mid = (lo[k] + hi[k]) >> 1;
