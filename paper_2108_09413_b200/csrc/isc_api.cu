@@ -271,10 +271,12 @@ int build_generic_engine(isc_model *m)
                 m->tc_fast[0] = igemm_constants(G, bias.data(), mult.data(), shift.data(), c4.data(), igemm_padded_cout(G), false, nullptr) ? 1 : 0;
                 rc = upload(m, c4, &m->tc_cst[0]); if (rc) return rc;
             }
-            if (i > 0 && igemm_tile_n(G)) {                 // the same layer for the tensor-core kernel
-                std::vector<int8_t> wp(igemm_pack_bytes(G));
-                igemm_pack_weights(G, H.w.data(), wp.data());
-                rc = upload(m, wp, &m->wpacks[(size_t)i]); if (rc) return rc;
+            if (i > 0 && (igemm_takes(G) || halo_fits(G))) {      // the same layer for the tensor-core kernels
+                if (igemm_takes(G)) {
+                    std::vector<int8_t> wp(igemm_pack_bytes(G));
+                    igemm_pack_weights(G, H.w.data(), wp.data());
+                    rc = upload(m, wp, &m->wpacks[(size_t)i]); if (rc) return rc;
+                }
                 const int n_cst = std::max(igemm_padded_cout(G), halo_padded_cout(G));
                 std::vector<int32_t> c4((size_t)n_cst * 4);
                 m->tc_fast[(size_t)i] = igemm_constants(G, bias.data(), mult.data(), shift.data(), c4.data(), n_cst, H.d.res_tensor >= 0, &m->tc_resk[(size_t)i]) ? 1 : 0;
@@ -457,9 +459,9 @@ int generic_forward(isc_model *m, int8_t *const *bufs, const uint8_t *d_x, const
         if (i == 0 && tensor_cores && m->wpacks[0])
             e = launch_stem_conv(G, m->wpacks[0], m->tc_cst[0], m->tc_fast[0] != 0, d_x, m->in_c, ns, batch, out, d_err, st);
         else if (i == 0) e = launch_first_conv(G, d_x, m->in_c, ns, batch, out, st);
-        else if (tensor_cores && m->hpacks[(size_t)i] && igemm_fits(G, batch))
+        else if (tensor_cores && m->hpacks[(size_t)i] && halo_offsets_fit(G, batch))
             e = launch_halo_conv(G, m->hpacks[(size_t)i], m->tc_cst[(size_t)i], m->tc_fast[(size_t)i] != 0, m->tc_resk[(size_t)i], batch, in, res, out, d_err, st);
-        else if (tensor_cores && m->wpacks[(size_t)i] && igemm_fits(G, batch)) e = launch_igemm_conv(G, m->wpacks[(size_t)i], m->tc_cst[(size_t)i], m->tc_fast[(size_t)i] != 0, m->tc_resk[(size_t)i], batch, in, res, out, d_err, st, false, m->opt_tensor_copy != 0);
+        else if (tensor_cores && m->wpacks[(size_t)i] && conv_offsets_fit(G, batch)) e = launch_igemm_conv(G, m->wpacks[(size_t)i], m->tc_cst[(size_t)i], m->tc_fast[(size_t)i] != 0, m->tc_resk[(size_t)i], batch, in, res, out, d_err, st, false, m->opt_tensor_copy != 0);
         else if (L.op == ISC_CONV2D || L.op == ISC_FC) e = launch_conv(G, batch, in, res, out, st);
         else if (L.op == ISC_GAVGPOOL) e = launch_gavgpool(G, batch, in, out, st);
         else e = launch_maxpool(G, batch, in, out, st);

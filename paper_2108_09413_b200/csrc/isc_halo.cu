@@ -498,6 +498,14 @@ bool halo_fits(const GLayer &G)
     return halo_config(G, &c);
 }
 
+// Besides the tensors' offsets: positions, those of one more image and a halo included, are divided as numbers below 2^31.
+bool halo_offsets_fit(const GLayer &G, int64_t batch)
+{
+    HaloConfig c;
+    return halo_config(G, &c) && conv_offsets_fit(G, batch) &&
+           (batch + 1) * (int64_t)c.hp * c.wp + c.positions_tile + 2 * kTile < (1ll << 31);
+}
+
 size_t halo_pack_bytes(const GLayer &G)
 {
     HaloConfig c;
@@ -540,9 +548,8 @@ cudaError_t launch_halo_conv(const GLayer &G, const int8_t *wpack, const int32_t
                              const int8_t *in, const int8_t *res, int8_t *out, int32_t *err, cudaStream_t st)
 {
     HaloConfig c;
-    if (!halo_config(G, &c)) return cudaErrorInvalidValue;
+    if (!halo_config(G, &c) || !halo_offsets_fit(G, batch)) return cudaErrorInvalidValue;
     const long long positions = (long long)batch * c.hp * c.wp;
-    if (positions >= (1ll << 31) - 2 * kTile || !igemm_fits(G, batch)) return cudaErrorInvalidValue;
     if (batch <= 0) return cudaSuccess;
     static int n_sms = 0;
     if (n_sms == 0) {

@@ -758,11 +758,10 @@ bool igemm_paired(uint32_t tiles_m, uint32_t tiles_n, uint32_t n_sms)
 }  // namespace
 
 // Output channels in as few tiles of at most 256 as possible, all of the same width (a multiple of 16; the last one may
-// be partly padding).  Every convolution and FC layer fits; pools do not.
+// be partly padding).
 // A 1 x 1 stride-1 layer for which paired tiles pay has tiles of 128, whether a launch pairs them or not.
 int igemm_tile_n(const GLayer &G)
 {
-    if (G.op != ISC_CONV2D && G.op != ISC_FC) return 0;
     if (igemm_pairable(G)) return kPairN;
     const int tiles = (G.coutp + 255) / 256;
     return ((G.coutp + tiles - 1) / tiles + 15) & ~15;
@@ -774,7 +773,25 @@ int igemm_tiles(const GLayer &G) { return igemm_pairable(G) ? G.coutp / kPairN :
 int igemm_units(const GLayer &G) { return G.kh * G.kw * (G.cinp / 16); }
 int igemm_blocks(const GLayer &G) { return (igemm_units(G) + 3) / 4; }
 
+// Dynamic shared memory of a launch: the constants of every output channel, the epilogue warps' scratch, and operand
+// stages, of which two are needed at least.
+constexpr size_t kSmemLimit = 226 * 1024;
+struct IgemmSmem {
+    size_t cst, scratch, stage;
+    bool fits() const { return cst + scratch + 2 * stage <= kSmemLimit; }
+};
+IgemmSmem igemm_smem(const GLayer &G, bool paired)
+{
+    const size_t n_tile = (size_t)igemm_tile_n(G), rows = paired ? 2 : 1;
+    return IgemmSmem{(size_t)igemm_tiles(G) * n_tile * 16, (size_t)kAllEpiWarps * 32 * rows * epi_row_stride((int)n_tile),
+                     (size_t)kTileM * kBlockK * rows + n_tile * kBlockK};
+}
+
 }  // namespace
+
+// Convolutions and FC layers whose constants leave room for the operands: up to 6,912 output channels in tiles of 256,
+// 10,112 in tiles of 128.  Wider ones stay on the plain kernel.
+bool igemm_takes(const GLayer &G) { return (G.op == ISC_CONV2D || G.op == ISC_FC) && igemm_smem(G, false).fits(); }
 
 // constants of that many channels: the last tile's padding included
 int igemm_padded_cout(const GLayer &G) { return igemm_tiles(G) * igemm_tile_n(G); }
@@ -803,8 +820,8 @@ void igemm_pack_weights(const GLayer &G, const int8_t *w, int8_t *out)
     for (int e = 0; e < kBlockK; ++e) out[at + e] = (int8_t)G.zp_in;
 }
 
-// 32-bit row and byte offsets inside the kernel
-bool igemm_fits(const GLayer &G, int64_t batch)
+// 32-bit row and byte offsets inside the tensor-core kernels
+bool conv_offsets_fit(const GLayer &G, int64_t batch)
 {
     return batch * G.hout * G.wout * ((G.coutp + 255) / 256) < (1ll << 31) - 512 && batch * G.hin * G.win * G.cinp < (1ll << 31);
 }
@@ -913,40 +930,37 @@ cudaError_t launch_igemm_conv(const GLayer &G, const int8_t *wpack, const int32_
         p.res_r2 = ((1ll << (res_n - 1)) - (128ll + G.zp_res) * (long long)G.res_mult) * (1ll << (32 - res_n));
     }
     p.batch = batch;
+    if (!igemm_takes(G) || !conv_offsets_fit(G, batch)) return cudaErrorInvalidValue;
     p.n_tile = igemm_tile_n(G);
-    if (p.n_tile == 0) return cudaErrorInvalidValue;
     p.tiles_n = igemm_tiles(G);
     p.units = igemm_units(G);
     p.n_blocks = igemm_blocks(G);
-    if (!igemm_fits(G, batch)) return cudaErrorInvalidValue;
     p.zp_run = wpack + igemm_pack_bytes(G) - kBlockK;
     p.m_total = (uint32_t)((long long)batch * G.hout * G.wout);
     p.tiles_m = (p.m_total + kTileM - 1) / kTileM;
     p.in = in; p.res = res; p.out = out; p.wpack = wpack; p.err = err;
     if (p.tiles_m == 0) return cudaSuccess;
-    const size_t smem_limit = 226 * 1024;
     static int n_sms = 0;
     if (n_sms == 0) {
         int dev = 0;
         cudaError_t e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_limit);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_limit);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_limit);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
         if (e != cudaSuccess) { n_sms = 0; return e; }
     }
-    const bool paired = igemm_pairable(G) && p.tma_a && p.fast_requant && (!res || p.fast_residual) && igemm_paired(p.tiles_m, (uint32_t)p.tiles_n, (uint32_t)n_sms);
+    const bool paired = igemm_pairable(G) && igemm_smem(G, true).fits() && p.tma_a && p.fast_requant && (!res || p.fast_residual) &&
+                        igemm_paired(p.tiles_m, (uint32_t)p.tiles_n, (uint32_t)n_sms);
     if (paired) p.tiles_m = (p.tiles_m + 1) / 2;
     p.acc_stride = paired ? 2 * kPairN : (p.n_tile + 31) & ~31;          // the epilogue loads 32 columns at a time
     p.tmem_cols = 64;
     while (p.tmem_cols < 2 * p.acc_stride) p.tmem_cols <<= 1;
     // as many operand stages as fit beside the constants, at most kMaxStages
-    const size_t stage_bytes = (size_t)kTileM * kBlockK * (paired ? 2 : 1) + (size_t)p.n_tile * kBlockK, cst_bytes = (size_t)p.tiles_n * p.n_tile * 16;
-    const size_t scratch_bytes = (size_t)kAllEpiWarps * 32 * (paired ? 2 : 1) * epi_row_stride(p.n_tile);
-    if (cst_bytes + scratch_bytes + 2 * stage_bytes > smem_limit) return cudaErrorInvalidValue;
-    p.stages = (int)std::min<size_t>(kMaxStages, (smem_limit - cst_bytes - scratch_bytes) / stage_bytes);
-    p.scratch_off = (uint32_t)((size_t)p.stages * stage_bytes + cst_bytes);
-    const size_t smem = (size_t)p.stages * stage_bytes + cst_bytes + scratch_bytes;
+    const IgemmSmem s = igemm_smem(G, paired);
+    p.stages = (int)std::min<size_t>(kMaxStages, (kSmemLimit - s.cst - s.scratch) / s.stage);
+    p.scratch_off = (uint32_t)((size_t)p.stages * s.stage + s.cst);
+    const size_t smem = (size_t)p.stages * s.stage + s.cst + s.scratch;
     // persistent: one CTA per SM (shared memory and the 512 tensor-memory columns allow no second one at N = 256)
     const uint32_t n_tiles = p.tiles_m * (uint32_t)p.tiles_n;
     const unsigned grid = std::min<uint32_t>(n_tiles, (uint32_t)n_sms);

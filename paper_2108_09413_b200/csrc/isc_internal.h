@@ -66,10 +66,10 @@ cudaError_t launch_votes(const int8_t *logits_nhwc, int cp, int n_classes, int b
                          int8_t *logits_out, cudaStream_t st);
 
 // ---- layer-by-layer tensor-core convolutions (isc_igemm.cu) ----
-// Output-channel tile of the implicit-GEMM kernel for this layer (a multiple of 16 up to 256), or 0 for pools.
-int igemm_tile_n(const GLayer &G);
+bool igemm_takes(const GLayer &G);               // whether the implicit-GEMM kernel has a form for this layer
+int igemm_tile_n(const GLayer &G);               // its output-channel tile (a multiple of 16 up to 256)
 int igemm_padded_cout(const GLayer &G);          // output channels with the last tile's padding: entries of the constants
-bool igemm_fits(const GLayer &G, int64_t batch);  // the batch's tensors are within the kernel's 32-bit offsets
+bool conv_offsets_fit(const GLayer &G, int64_t batch);  // the batch's tensors are within the tensor-core kernels' 32-bit offsets
 size_t igemm_pack_bytes(const GLayer &G);
 void igemm_pack_weights(const GLayer &G, const int8_t *w_oihw, int8_t *out);
 // The residual term F(u) = floor((u * m2 + R2) / 2^32), u = r + 128 in 0..255, of the 32-bit epilogues as
@@ -91,6 +91,7 @@ cudaError_t launch_igemm_conv(const GLayer &G, const int8_t *wpack, const int32_
 // ---- stride-1 "same" convolutions with the input tile in shared memory (isc_halo.cu) ----
 // Odd square filters from 3 x 3 on whose tile fits.  Constants as igemm_constants makes them, for halo_padded_cout channels.
 bool halo_fits(const GLayer &G);
+bool halo_offsets_fit(const GLayer &G, int64_t batch);
 int halo_padded_cout(const GLayer &G);
 size_t halo_pack_bytes(const GLayer &G);
 void halo_pack(const GLayer &G, const int8_t *w_oihw, int8_t *out);

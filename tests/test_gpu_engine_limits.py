@@ -1,0 +1,22 @@
+"""Calls at the limits of what an engine takes: whichever kernels they end up on, the results are the CPU oracle's."""
+import numpy as np
+import pytest
+
+import oracle
+import workloads as wl
+import paper_2108_09413_b200 as isc
+from test_host_dispatch import _hidden_layer_net
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("cin,cout", [(24, 6912), (24, 6913), (64, 10112), (64, 10240)])
+def test_layers_around_the_shared_memory_limit_of_the_tensor_core_kernel(cin, cout):
+    model = _hidden_layer_net(wl, cin, cout)
+    gm, om = isc.Model(model), oracle.Model(model)
+    x = wl.images(1, shape=model["in_shape"], seed=3)[0]
+    ec, el = oracle.sample_counts(om, x, 5, 1, 1, 0, 19, 0.25, want_logits=True)
+    gc, gl = gm.sample_counts(x, 5, 1, 1, 0, 19, 0.25, want_logits=True)
+    np.testing.assert_array_equal(gl, el)
+    np.testing.assert_array_equal(gc, ec)
+    np.testing.assert_array_equal(gm.sample_counts_static(x, 5, 1, 1, 0, 19, 0.25), ec)

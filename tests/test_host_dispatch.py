@@ -1,0 +1,79 @@
+"""The library's host code without a GPU: which kernels a call takes, and what it asks of the CUDA runtime for them.
+
+Every test runs in a process of its own in which a stand-in for the CUDA runtime (host/fake_cudart.c) is preloaded:
+device memory is host memory, kernels do nothing, launches are recorded and are refused for the reason for which the
+real runtime refuses them (more dynamic shared memory than the kernel was granted on the current device)."""
+import ctypes as C
+import os
+import subprocess
+import sys
+import threading
+
+import numpy as np
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+
+
+@pytest.fixture(scope="session")
+def fake_runtime(tmp_path_factory):
+    so = str(tmp_path_factory.mktemp("fake") / "libfakecudart.so")
+    subprocess.run(["gcc", "-O1", "-Wall", "-shared", "-fPIC", "-pthread", "-I", "/usr/local/cuda/include", "-o", so,
+                    os.path.join(HERE, "host", "fake_cudart.c")], check=True)
+    return so
+
+
+# ------------------------------------------------------------------ in the process with the stand-in
+
+def _fake():
+    f = C.CDLL(os.environ["LD_PRELOAD"])
+    f.fake_launch_name.restype = C.c_char_p
+    f.fake_allocated.restype = C.c_size_t
+    f.fake_watch.argtypes = [C.c_void_p]
+    return f
+
+
+def _kernels(f):
+    names = ("k_line", "k_stem", "k_halo", "k_igemm", "k_first_conv", "k_conv", "k_gavgpool", "k_maxpool", "k_votes")
+    return [next(n for n in names if n in f.fake_launch_name(i).decode()) for i in range(f.fake_launches())]
+
+
+def _hidden_layer_net(wl, cin, cout):
+    """stem -> 1 x 1 convolution from `cin` to `cout` channels -> pool -> FC"""
+    rng = wl.SplitMix64(5)
+    L = [wl._conv(rng, 0, 3, cin, 3, 1, 1, True, 3, -128), wl._conv(rng, 1, cin, cout, 1, 1, 0, True, -128, -128),
+         wl._gavgpool(2, cout, 16, -128), wl._conv(rng, 3, cout, 5, 1, 1, 0, False, -128, 0, op=wl.OP_FC)]
+    return dict(in_shape=(3, 4, 4), n_classes=5, layers=L)
+
+
+def layer_too_wide_for_shared_memory():
+    """The implicit-GEMM kernel keeps a layer's constants in shared memory: a layer whose constants leave no room for two
+    operand stages runs on the plain kernel, through every entry point."""
+    import paper_2108_09413_b200 as isc
+    import workloads as wl
+    f = _fake()
+    for cin, cout, kernel in ((24, 6912, "k_igemm"), (24, 6913, "k_conv"), (24, 8200, "k_conv"), (64, 10112, "k_igemm"), (64, 10240, "k_conv")):
+        model = _hidden_layer_net(wl, cin, cout)
+        gm = isc.Model(model)
+        x = wl.images(1, shape=model["in_shape"])[0]
+        for call in (gm.sample_counts, gm.sample_counts_static):
+            f.fake_reset()
+            call(x, 1, 0, 1, 0, 9, 0.25)
+            assert _kernels(f) == ["k_stem", kernel, "k_gavgpool", "k_igemm", "k_votes"], (cin, cout, _kernels(f))
+
+
+# ------------------------------------------------------------------ the tests
+
+SCENARIOS = [layer_too_wide_for_shared_memory]
+
+
+@pytest.mark.parametrize("scenario", [s.__name__ for s in SCENARIOS])
+def test_host_code(scenario, fake_runtime):
+    r = subprocess.run([sys.executable, os.path.abspath(__file__), scenario], cwd=ROOT, timeout=300, capture_output=True, text=True,
+                       env=dict(os.environ, LD_PRELOAD=fake_runtime, PYTHONPATH=ROOT))
+    assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-4000:]
+
+
+if __name__ == "__main__":
+    globals()[sys.argv[1]]()
