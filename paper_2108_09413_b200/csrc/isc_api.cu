@@ -52,6 +52,7 @@ struct isc_model {
     std::vector<char> tc_fast;
     std::vector<uint32_t> tc_resk;           // per layer: offset of the residual term's two-instruction form, or 0xFFFFFFFF
     bool has_tc = false;
+    isc::TcDevice tc;
     int32_t *d_tc_err = nullptr;
 
     // activation buffers: tensor t lives in pool buffer tensor_buf[t] (bytes per sample buf_bytes[b])
@@ -444,11 +445,21 @@ std::vector<int8_t *> own_buffers(const isc_model *m)
     return b;
 }
 
+int ready_tensor_cores(isc_model *m)
+{
+    if (!m->tc.n_sms) CK(tc_prepare(&m->tc));
+    return ISC_OK;
+}
+
 // Layer-by-layer forward of `batch` samples in the activation buffers `bufs`; leaves the logits in the last tensor's.
 int generic_forward(isc_model *m, int8_t *const *bufs, const uint8_t *d_x, const NoiseStream &ns, int batch, cudaStream_t st, int32_t *d_err,
                     int stop_after_layer = -1, bool tensor_cores = false)
 {
     const int n = (int)m->glayers.size();
+    if (tensor_cores) {
+        int rc = ready_tensor_cores(m);
+        if (rc) return rc;
+    }
     for (int i = 0; i < n; ++i) {
         const GLayer &G = m->glayers[(size_t)i];
         const isc_layer &L = m->layers[(size_t)i].d;
@@ -460,8 +471,8 @@ int generic_forward(isc_model *m, int8_t *const *bufs, const uint8_t *d_x, const
             e = launch_stem_conv(G, m->wpacks[0], m->tc_cst[0], m->tc_fast[0] != 0, d_x, m->in_c, ns, batch, out, d_err, st);
         else if (i == 0) e = launch_first_conv(G, d_x, m->in_c, ns, batch, out, st);
         else if (tensor_cores && m->hpacks[(size_t)i] && halo_offsets_fit(G, batch))
-            e = launch_halo_conv(G, m->hpacks[(size_t)i], m->tc_cst[(size_t)i], m->tc_fast[(size_t)i] != 0, m->tc_resk[(size_t)i], batch, in, res, out, d_err, st);
-        else if (tensor_cores && m->wpacks[(size_t)i] && conv_offsets_fit(G, batch)) e = launch_igemm_conv(G, m->wpacks[(size_t)i], m->tc_cst[(size_t)i], m->tc_fast[(size_t)i] != 0, m->tc_resk[(size_t)i], batch, in, res, out, d_err, st, false, m->opt_tensor_copy != 0);
+            e = launch_halo_conv(m->tc, G, m->hpacks[(size_t)i], m->tc_cst[(size_t)i], m->tc_fast[(size_t)i] != 0, m->tc_resk[(size_t)i], batch, in, res, out, d_err, st);
+        else if (tensor_cores && m->wpacks[(size_t)i] && conv_offsets_fit(G, batch)) e = launch_igemm_conv(m->tc, G, m->wpacks[(size_t)i], m->tc_cst[(size_t)i], m->tc_fast[(size_t)i] != 0, m->tc_resk[(size_t)i], batch, in, res, out, d_err, st, false, m->opt_tensor_copy != 0);
         else if (L.op == ISC_CONV2D || L.op == ISC_FC) e = launch_conv(G, batch, in, res, out, st);
         else if (L.op == ISC_GAVGPOOL) e = launch_gavgpool(G, batch, in, out, st);
         else e = launch_maxpool(G, batch, in, out, st);
@@ -1018,6 +1029,7 @@ int isc_debug_wait_timeout(isc_model *m, int64_t limit_ns, void *cuda_stream, in
         while (li < m->glayers.size() && !m->wpacks[li]) ++li;
         if (li >= m->glayers.size()) return ISC_ERR_UNSUPPORTED;
         int rc = ensure_workspace(m, 1);
+        if (rc == ISC_OK) rc = ready_tensor_cores(m);
         if (rc) return rc;
         const GLayer &G = m->glayers[li];
         const isc_layer &L = m->layers[li].d;
@@ -1025,7 +1037,7 @@ int isc_debug_wait_timeout(isc_model *m, int64_t limit_ns, void *cuda_stream, in
         const int8_t *in = (const int8_t *)m->bufs[(size_t)m->tensor_buf[(size_t)L.in_tensor]].p;
         const int8_t *res = L.res_tensor >= 0 ? (const int8_t *)m->bufs[(size_t)m->tensor_buf[(size_t)L.res_tensor]].p : nullptr;
         const auto t0 = std::chrono::steady_clock::now();
-        if (launch_igemm_conv(G, m->wpacks[li], m->tc_cst[li], m->tc_fast[li] != 0, m->tc_resk[li], 1, in, res, out, m->d_tc_err, st, true) != cudaSuccess)
+        if (launch_igemm_conv(m->tc, G, m->wpacks[li], m->tc_cst[li], m->tc_fast[li] != 0, m->tc_resk[li], 1, in, res, out, m->d_tc_err, st, true) != cudaSuccess)
             return ISC_ERR_CUDA;
         CK(cudaStreamSynchronize(st));
         const long long ns = std::chrono::duration_cast<std::chrono::nanoseconds>(std::chrono::steady_clock::now() - t0).count();

@@ -544,21 +544,15 @@ void halo_pack(const GLayer &G, const int8_t *w, int8_t *out)
     for (int e = 0; e < 64; ++e) out[at + e] = (int8_t)G.zp_in;
 }
 
-cudaError_t launch_halo_conv(const GLayer &G, const int8_t *wpack, const int32_t *cst, bool fast, uint32_t res_k8, int batch,
+cudaError_t halo_prepare() { return cudaFuncSetAttribute(k_halo, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax); }
+
+cudaError_t launch_halo_conv(const TcDevice &dev, const GLayer &G, const int8_t *wpack, const int32_t *cst, bool fast, uint32_t res_k8, int batch,
                              const int8_t *in, const int8_t *res, int8_t *out, int32_t *err, cudaStream_t st)
 {
     HaloConfig c;
     if (!halo_config(G, &c) || !halo_offsets_fit(G, batch)) return cudaErrorInvalidValue;
     const long long positions = (long long)batch * c.hp * c.wp;
     if (batch <= 0) return cudaSuccess;
-    static int n_sms = 0;
-    if (n_sms == 0) {
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_halo, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
-        if (e != cudaSuccess) { n_sms = 0; return e; }
-    }
     HaloParams p;
     memset(&p, 0, sizeof(p));
     p.L = G;
@@ -597,7 +591,7 @@ cudaError_t launch_halo_conv(const GLayer &G, const int8_t *wpack, const int32_t
         p.res_r2 = ((1ll << (res_n - 1)) - (128ll + G.zp_res) * (long long)G.res_mult) * (1ll << (32 - res_n));
     }
     p.err = err;
-    k_halo<<<std::min<uint32_t>(p.n_items, (uint32_t)n_sms), kThreads, c.smem, st>>>(p);
+    k_halo<<<std::min<uint32_t>(p.n_items, (uint32_t)dev.n_sms), kThreads, c.smem, st>>>(p);
     return cudaGetLastError();
 }
 

@@ -881,7 +881,30 @@ bool igemm_constants(const GLayer &G, const int32_t *bias_folded, const int32_t 
     return fast;
 }
 
-cudaError_t launch_igemm_conv(const GLayer &G, const int8_t *wpack, const int32_t *cst, bool fast, uint32_t res_k8, int batch, const int8_t *in,
+typedef CUresult (*EncodeFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
+                             const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+cudaError_t tc_prepare(TcDevice *dev)
+{
+    TcDevice d;
+    int ordinal = 0;
+    cudaError_t e = cudaGetDevice(&ordinal);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&d.n_sms, cudaDevAttrMultiProcessorCount, ordinal);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_stem, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStemSmemLimit);
+    if (e == cudaSuccess) e = halo_prepare();
+    if (e != cudaSuccess) { cudaGetLastError(); return e; }
+    void *fn = nullptr;
+    cudaDriverEntryPointQueryResult qr;
+    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qr) == cudaSuccess && qr == cudaDriverEntryPointSuccess) d.encode = fn;
+    else cudaGetLastError();
+    *dev = d;
+    return cudaSuccess;
+}
+
+cudaError_t launch_igemm_conv(const TcDevice &dev, const GLayer &G, const int8_t *wpack, const int32_t *cst, bool fast, uint32_t res_k8, int batch, const int8_t *in,
                               const int8_t *res, int8_t *out, int32_t *err, cudaStream_t st, bool debug_stall, bool tensor_copy)
 {
     IgemmParams p;
@@ -893,25 +916,12 @@ cudaError_t launch_igemm_conv(const GLayer &G, const int8_t *wpack, const int32_
     p.fast_residual = (res_n == 31 || res_n == 32) ? 1 : 0;
     p.debug_stall = debug_stall ? 1 : 0;
     // A 1 x 1 stride-1 layer reads its input as the matrix [pixel][channel]: the tile's operand rows are a box of the
-    // view (16 bytes, pixel, 16-byte column) and come by tensor copy.  The encoder is the driver's, looked up at run
-    // time; without it (or if it refuses the view) the gather warps do the work.
+    // view (16 bytes, pixel, 16-byte column) and come by tensor copy.  Without the driver's encoder (or if it refuses the
+    // view) the gather warps do the work.
     p.tma_a = 0;
     memset(&p.tmap_a, 0, sizeof(p.tmap_a));
     if (tensor_copy && G.kh == 1 && G.kw == 1 && G.stride == 1 && G.pad == 0) {
-        typedef CUresult (*EncodeFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
-                                     const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-        static EncodeFn encode = nullptr;
-        static bool looked_up = false;
-        if (!looked_up) {
-            void *fn = nullptr;
-            cudaDriverEntryPointQueryResult qr;
-            if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qr) == cudaSuccess && qr == cudaDriverEntryPointSuccess)
-                encode = (EncodeFn)fn;
-            else
-                cudaGetLastError();
-            looked_up = true;
-        }
-        if (encode) {
+        if (const EncodeFn encode = (EncodeFn)dev.encode) {
             const cuuint64_t dims[3] = {16, (cuuint64_t)batch * G.hin * G.win, (cuuint64_t)(G.cinp / 16)};
             const cuuint64_t strides[2] = {(cuuint64_t)G.cinp, 16};
             const cuuint32_t box[3] = {16, (cuuint32_t)kTileM, (cuuint32_t)(kBlockK / 16)}, estr[3] = {1, 1, 1};
@@ -940,18 +950,8 @@ cudaError_t launch_igemm_conv(const GLayer &G, const int8_t *wpack, const int32_
     p.tiles_m = (p.m_total + kTileM - 1) / kTileM;
     p.in = in; p.res = res; p.out = out; p.wpack = wpack; p.err = err;
     if (p.tiles_m == 0) return cudaSuccess;
-    static int n_sms = 0;
-    if (n_sms == 0) {
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
-        if (e != cudaSuccess) { n_sms = 0; return e; }
-    }
     const bool paired = igemm_pairable(G) && igemm_smem(G, true).fits() && p.tma_a && p.fast_requant && (!res || p.fast_residual) &&
-                        igemm_paired(p.tiles_m, (uint32_t)p.tiles_n, (uint32_t)n_sms);
+                        igemm_paired(p.tiles_m, (uint32_t)p.tiles_n, (uint32_t)dev.n_sms);
     if (paired) p.tiles_m = (p.tiles_m + 1) / 2;
     p.acc_stride = paired ? 2 * kPairN : (p.n_tile + 31) & ~31;          // the epilogue loads 32 columns at a time
     p.tmem_cols = 64;
@@ -963,7 +963,7 @@ cudaError_t launch_igemm_conv(const GLayer &G, const int8_t *wpack, const int32_
     const size_t smem = (size_t)p.stages * s.stage + s.cst + s.scratch;
     // persistent: one CTA per SM (shared memory and the 512 tensor-memory columns allow no second one at N = 256)
     const uint32_t n_tiles = p.tiles_m * (uint32_t)p.tiles_n;
-    const unsigned grid = std::min<uint32_t>(n_tiles, (uint32_t)n_sms);
+    const unsigned grid = std::min<uint32_t>(n_tiles, (uint32_t)dev.n_sms);
     const bool whole = G.cinp % kBlockK == 0 && p.n_tile % 64 == 0 && G.coutp == p.tiles_n * p.n_tile;
     if (paired) k_igemm<true, true><<<grid, kGemmThreads, smem, st>>>(p);
     else if (whole) k_igemm<true, false><<<grid, kGemmThreads, smem, st>>>(p);
@@ -1058,12 +1058,6 @@ cudaError_t launch_stem_conv(const GLayer &G, const int8_t *wpack, const int32_t
     if (ns.guide == ns.cum + (2 * ns.T + 1) && smem + tab_bytes <= (smem <= kStemSmemPair ? kStemSmemPair : kStemSmemLimit)) {
         p.tab_off = (uint32_t)smem;
         smem += tab_bytes;
-    }
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k_stem, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStemSmemLimit);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
     }
     if (batch <= 0) return cudaSuccess;
     dim3 grid((unsigned)p.n_bands, (unsigned)batch);

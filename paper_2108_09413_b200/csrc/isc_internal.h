@@ -66,6 +66,13 @@ cudaError_t launch_votes(const int8_t *logits_nhwc, int cp, int n_classes, int b
                          int8_t *logits_out, cudaStream_t st);
 
 // ---- layer-by-layer tensor-core convolutions (isc_igemm.cu) ----
+// What their launches need of the device.  A handle keeps its own (calls on one handle do not overlap, so nothing here is
+// shared between threads), filled by tc_prepare, which also raises the kernels' shared-memory limits.
+struct TcDevice {
+    int n_sms = 0;
+    void *encode = nullptr;   // the driver's cuTensorMapEncodeTiled, or null
+};
+cudaError_t tc_prepare(TcDevice *dev);
 bool igemm_takes(const GLayer &G);               // whether the implicit-GEMM kernel has a form for this layer
 int igemm_tile_n(const GLayer &G);               // its output-channel tile (a multiple of 16 up to 256)
 int igemm_padded_cout(const GLayer &G);          // output channels with the last tile's padding: entries of the constants
@@ -84,7 +91,7 @@ bool igemm_constants(const GLayer &G, const int32_t *bias_folded, const int32_t 
 // (after their 2 s limit) and the CTAs leave through the abort path -- nothing faults or hangs.  `tensor_copy`: a
 // 1 x 1 stride-1 layer may take its operand rows by tensor copy (false: the gather warps bring them, as for every
 // other layer).
-cudaError_t launch_igemm_conv(const GLayer &G, const int8_t *wpack, const int32_t *cst, bool fast, uint32_t res_k8, int batch, const int8_t *in,
+cudaError_t launch_igemm_conv(const TcDevice &dev, const GLayer &G, const int8_t *wpack, const int32_t *cst, bool fast, uint32_t res_k8, int batch, const int8_t *in,
                               const int8_t *res, int8_t *out, int32_t *err, cudaStream_t st, bool debug_stall = false,
                               bool tensor_copy = true);
 
@@ -95,7 +102,8 @@ bool halo_offsets_fit(const GLayer &G, int64_t batch);
 int halo_padded_cout(const GLayer &G);
 size_t halo_pack_bytes(const GLayer &G);
 void halo_pack(const GLayer &G, const int8_t *w_oihw, int8_t *out);
-cudaError_t launch_halo_conv(const GLayer &G, const int8_t *wpack, const int32_t *cst, bool fast, uint32_t res_k8, int batch,
+cudaError_t halo_prepare();                      // part of tc_prepare
+cudaError_t launch_halo_conv(const TcDevice &dev, const GLayer &G, const int8_t *wpack, const int32_t *cst, bool fast, uint32_t res_k8, int batch,
                              const int8_t *in, const int8_t *res, int8_t *out, int32_t *err, cudaStream_t st);
 
 // The first convolution (<= 4 input channels, filter at most 8 x 8) on the tensor cores, noise drawn into its staging.

@@ -8,6 +8,7 @@ import os
 import subprocess
 import sys
 import threading
+import time
 
 import numpy as np
 import pytest
@@ -63,9 +64,45 @@ def layer_too_wide_for_shared_memory():
             assert _kernels(f) == ["k_stem", kernel, "k_gavgpool", "k_igemm", "k_votes"], (cin, cout, _kernels(f))
 
 
+def _filter_net(wl):
+    """a network whose kernels need more shared memory than a launch has by default: stem, resident filter, 1 x 1, FC"""
+    rng = wl.SplitMix64(6)
+    L = [wl._conv(rng, 0, 3, 96, 7, 1, 3, True, 3, -128), wl._conv(rng, 1, 96, 96, 3, 1, 1, True, -128, -128),
+         wl._conv(rng, 2, 96, 256, 1, 1, 0, True, -128, -128), wl._gavgpool(3, 256, 24 * 36, -128),
+         wl._conv(rng, 4, 256, 5, 1, 1, 0, False, -128, 0, op=wl.OP_FC)]
+    return dict(in_shape=(3, 24, 36), n_classes=5, layers=L)
+
+
+def first_calls_in_two_threads():
+    """Two handles used for the first time at once: neither may launch before the kernels' shared-memory limits are raised,
+    however long that takes the other."""
+    import paper_2108_09413_b200 as isc
+    import workloads as wl
+    f = _fake()
+    model = _filter_net(wl)
+    x = wl.images(1, shape=model["in_shape"])[0]
+    handles = [isc.Model(model) for _ in range(2)]
+    f.fake_set_attribute_delay(200_000)
+    failed = []
+
+    def first_call(gm, wait_s):
+        time.sleep(wait_s)
+        try:
+            gm.sample_counts(x, 1, 0, 1, 0, 9, 0.25)
+        except isc.IscError as e:
+            failed.append(e)
+    threads = [threading.Thread(target=first_call, args=a) for a in zip(handles, (0.0, 0.1))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed, failed
+    assert sorted(set(_kernels(f))) == ["k_gavgpool", "k_halo", "k_igemm", "k_stem", "k_votes"]
+
+
 # ------------------------------------------------------------------ the tests
 
-SCENARIOS = [layer_too_wide_for_shared_memory]
+SCENARIOS = [layer_too_wide_for_shared_memory, first_calls_in_two_threads]
 
 
 @pytest.mark.parametrize("scenario", [s.__name__ for s in SCENARIOS])
