@@ -447,7 +447,9 @@ std::vector<int8_t *> own_buffers(const isc_model *m)
 
 int ready_tensor_cores(isc_model *m)
 {
-    if (!m->tc.n_sms) CK(tc_prepare(&m->tc));
+    int device = -1;
+    CK(cudaGetDevice(&device));
+    if (device != m->tc.ordinal) CK(tc_prepare(&m->tc, device));
     return ISC_OK;
 }
 

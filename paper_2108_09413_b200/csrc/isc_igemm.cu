@@ -884,12 +884,11 @@ bool igemm_constants(const GLayer &G, const int32_t *bias_folded, const int32_t 
 typedef CUresult (*EncodeFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
                              const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-cudaError_t tc_prepare(TcDevice *dev)
+cudaError_t tc_prepare(TcDevice *dev, int ordinal)
 {
     TcDevice d;
-    int ordinal = 0;
-    cudaError_t e = cudaGetDevice(&ordinal);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&d.n_sms, cudaDevAttrMultiProcessorCount, ordinal);
+    d.ordinal = ordinal;
+    cudaError_t e = cudaDeviceGetAttribute(&d.n_sms, cudaDevAttrMultiProcessorCount, ordinal);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);

@@ -66,13 +66,14 @@ cudaError_t launch_votes(const int8_t *logits_nhwc, int cp, int n_classes, int b
                          int8_t *logits_out, cudaStream_t st);
 
 // ---- layer-by-layer tensor-core convolutions (isc_igemm.cu) ----
-// What their launches need of the device.  A handle keeps its own (calls on one handle do not overlap, so nothing here is
-// shared between threads), filled by tc_prepare, which also raises the kernels' shared-memory limits.
+// What their launches need of the current device.  A handle keeps its own (calls on one handle do not overlap, so nothing
+// here is shared between threads), filled by tc_prepare, which also raises the kernels' shared-memory limits there: those
+// are a property of each device.
 struct TcDevice {
-    int n_sms = 0;
+    int ordinal = -1, n_sms = 0;
     void *encode = nullptr;   // the driver's cuTensorMapEncodeTiled, or null
 };
-cudaError_t tc_prepare(TcDevice *dev);
+cudaError_t tc_prepare(TcDevice *dev, int ordinal);
 bool igemm_takes(const GLayer &G);               // whether the implicit-GEMM kernel has a form for this layer
 int igemm_tile_n(const GLayer &G);               // its output-channel tile (a multiple of 16 up to 256)
 int igemm_padded_cout(const GLayer &G);          // output channels with the last tile's padding: entries of the constants

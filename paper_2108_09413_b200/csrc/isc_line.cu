@@ -1151,7 +1151,7 @@ struct LinePlan {
     unsigned long long *d_phase_cycles = nullptr;
     uint8_t *d_dump = nullptr;
     int sm_count = 0;
-    bool attr_set = false;
+    int attr_device = -1;                // the device on which k_line's shared-memory limit has been raised
     // launches smaller than the GPU (see line_run)
     cudaStream_t side[kSideStreams] = {};
     cudaEvent_t fork_event = nullptr, join_event[kSideStreams] = {};
@@ -1961,13 +1961,13 @@ static int line_join(LinePlan *p, cudaStream_t st)
 
 static int line_launch(LinePlan *p, LineParams &q, cudaStream_t st)
 {
-    if (!p->attr_set) {
-        if (cudaFuncSetAttribute(k_line, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) != cudaSuccess) {
-            cudaGetLastError();
-            return ISC_ERR_CUDA;
-        }
-        p->attr_set = true;
+    int device = -1;
+    bool ok = cudaGetDevice(&device) == cudaSuccess;
+    if (ok && device != p->attr_device) {
+        ok = cudaFuncSetAttribute(k_line, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) == cudaSuccess;
+        if (ok) p->attr_device = device;
     }
+    if (!ok) { cudaGetLastError(); return ISC_ERR_CUDA; }
     const int grid = std::max(1, std::min(q.n_groups, p->sm_count));
     k_line<<<grid, kThreads, p->smem_bytes, st>>>(q);
     const cudaError_t e = cudaGetLastError();

@@ -100,9 +100,30 @@ def first_calls_in_two_threads():
     assert sorted(set(_kernels(f))) == ["k_gavgpool", "k_halo", "k_igemm", "k_stem", "k_votes"]
 
 
+def every_device():
+    """Shared-memory limits are a property of each device: handles on two devices work in one process, and so does a handle
+    that is used with another device current than before (its memory being visible there)."""
+    import paper_2108_09413_b200 as isc
+    import workloads as wl
+    f = _fake()
+    for model, kernels in ((_filter_net(wl), ["k_gavgpool", "k_halo", "k_igemm", "k_stem", "k_votes"]), (wl.resnet20(), ["k_line"])):
+        x = wl.images(1, shape=model["in_shape"])[0]
+        handles = []
+        for device in (0, 1):
+            f.fake_set_device(device)
+            handles.append(isc.Model(model))
+        for device, gm in ((0, handles[0]), (1, handles[1]), (2, handles[0]), (0, handles[0]), (3, handles[1])):
+            f.fake_set_device(device)
+            for call in (gm.sample_counts, gm.sample_counts_static):
+                f.fake_reset()
+                call(x, 1, 0, 1, 0, 9, 0.25)
+                assert sorted(set(_kernels(f))) == kernels
+                assert all(f.fake_launch_ok(i) and f.fake_launch_device(i) == device for i in range(f.fake_launches()))
+
+
 # ------------------------------------------------------------------ the tests
 
-SCENARIOS = [layer_too_wide_for_shared_memory, first_calls_in_two_threads]
+SCENARIOS = [layer_too_wide_for_shared_memory, first_calls_in_two_threads, every_device]
 
 
 @pytest.mark.parametrize("scenario", [s.__name__ for s in SCENARIOS])
