@@ -132,7 +132,8 @@ int isc_certify(isc_model *m, const uint8_t *x_u8, uint64_t seed, uint64_t image
  * isc_certify_batch -- Algorithm 1 for n_images images; image i uses image_id0 + i and
  * gives exactly what isc_certify gives for it.
  *   x_u8        : [n_images][C][H][W] bytes; a HOST pointer, or a DEVICE pointer when
- *                 x_on_device != 0 (the images are then read in place).
+ *                 x_on_device != 0 (the images are then read in place, or copied on the device
+ *                 first when the pointer is not a multiple of 4).
  *   out_class[n_images], out_radius[n_images] : host.
  *   out_counts0 / out_counts : host, [n_images][n_classes] int32, or NULL.
  */

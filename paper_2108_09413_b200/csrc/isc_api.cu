@@ -550,12 +550,14 @@ int ensure_pinned(isc_model *m, size_t need)
     return ISC_OK;
 }
 
-// The start of a call: error word and `n_counts` counts cleared, the images on the device.
+// The start of a call: error word and `n_counts` counts cleared, the images on the device.  The kernels read images as
+// 32-bit words where an image row is whole words; device images that are not aligned for that are copied like host images.
 int begin_call(isc_model *m, const uint8_t *x, size_t x_bytes, bool x_on_device, size_t n_counts, cudaStream_t st, const uint8_t **d_x)
 {
     const size_t head = kCountsOff + n_counts * sizeof(int32_t), x_off = (head + 15) & ~(size_t)15;
+    const bool in_place = x_on_device && (uintptr_t)x % 4 == 0;
     void *p = m->d_io;
-    int rc = ensure_bytes(&p, &m->d_io_bytes, x_off + (x_on_device ? 0 : x_bytes));
+    int rc = ensure_bytes(&p, &m->d_io_bytes, x_off + (in_place ? 0 : x_bytes));
     m->d_io = (uint8_t *)p;
     if (rc) return rc;
     const bool staged = !x_on_device && x_off + x_bytes <= kStagedBytes;
@@ -566,9 +568,9 @@ int begin_call(isc_model *m, const uint8_t *x, size_t x_bytes, bool x_on_device,
         CK(cudaMemcpyAsync(m->d_io, m->h_io, x_off + x_bytes, cudaMemcpyHostToDevice, st));
     } else {
         CK(cudaMemsetAsync(m->d_io, 0, head, st));
-        if (!x_on_device) CK(cudaMemcpyAsync(m->d_io + x_off, x, x_bytes, cudaMemcpyHostToDevice, st));
+        if (!in_place) CK(cudaMemcpyAsync(m->d_io + x_off, x, x_bytes, x_on_device ? cudaMemcpyDefault : cudaMemcpyHostToDevice, st));
     }
-    *d_x = x_on_device ? x : m->d_io + x_off;
+    *d_x = in_place ? x : m->d_io + x_off;
     return ISC_OK;
 }
 int32_t *call_err(isc_model *m) { return (int32_t *)m->d_io; }

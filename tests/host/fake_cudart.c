@@ -78,9 +78,9 @@ cudaError_t cudaLaunchKernel(const void *func, dim3 grid, dim3 block, void **arg
     const int ok = f && (smem <= 48 * 1024 || smem <= (size_t)f->smem[device]);
     if (f && n_launches < MAX_LAUNCHES) {
         int seen = 0;
-        /* the first argument of the kernels in question is a structure of more than 160 bytes */
+        /* the first argument of the kernels in question is a structure of more than 256 bytes */
         if (watched && (strstr(f->name, "k_stem") || strstr(f->name, "k_line")))
-            for (int i = 0; i < 160 / 8; ++i) seen |= ((const void **)args[0])[i] == watched;
+            for (int i = 0; i < 256 / 8; ++i) seen |= ((const void **)args[0])[i] == watched;
         launches[n_launches++] = (Launch){f->name, device, st ? st->priority : 0, ok, seen};
     }
     pthread_mutex_unlock(&lock);

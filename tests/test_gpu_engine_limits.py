@@ -20,3 +20,19 @@ def test_layers_around_the_shared_memory_limit_of_the_tensor_core_kernel(cin, co
     np.testing.assert_array_equal(gl, el)
     np.testing.assert_array_equal(gc, ec)
     np.testing.assert_array_equal(gm.sample_counts_static(x, 5, 1, 1, 0, 19, 0.25), ec)
+
+
+@pytest.mark.parametrize("net", ["resident", "layerwise"])
+def test_device_images_of_any_alignment(net):
+    import torch
+    model = wl.spread_model("resnet20") if net == "resident" else wl.resnet50(hw=32, blocks=(1, 1, 1, 1))
+    gm = isc.Model(model)
+    xs = wl.images(3, shape=model["in_shape"], seed=8)
+    expected = gm.certify_batch(xs, 3, 7, 0, 20, 150, 0.25, 0.001)
+    for offset in (0, 1, 2, 3, 5):
+        buf = torch.zeros(xs.size + 16, dtype=torch.uint8, device="cuda")
+        buf[offset:offset + xs.size] = torch.from_numpy(xs.ravel()).cuda()
+        torch.cuda.synchronize()
+        got = gm.certify_batch(None, 3, 7, 0, 20, 150, 0.25, 0.001, device_ptr=buf.data_ptr() + offset)
+        for g, e in zip(got, expected):
+            np.testing.assert_array_equal(g, e)

@@ -121,9 +121,27 @@ def every_device():
                 assert all(f.fake_launch_ok(i) and f.fake_launch_device(i) == device for i in range(f.fake_launches()))
 
 
+def device_images_of_any_alignment():
+    """The kernels read an image's rows as 32-bit words: device images are read in place where their address allows that,
+    and from an aligned copy where it does not."""
+    import paper_2108_09413_b200 as isc
+    import workloads as wl
+    f = _fake()
+    for model in (wl.resnet20(), _filter_net(wl)):
+        gm = isc.Model(model)
+        size = int(np.prod(model["in_shape"]))
+        room = np.zeros(2 * size + 64, np.uint8)
+        base = (room.ctypes.data + 15) // 16 * 16
+        for offset in (0, 1, 2, 3, 4, 7):
+            f.fake_reset()
+            f.fake_watch(base + offset)
+            gm.certify_batch(None, 2, 1, 0, 5, 9, 0.25, 0.001, device_ptr=base + offset)
+            assert any(f.fake_launch_watched(i) for i in range(f.fake_launches())) == (offset % 4 == 0), offset
+
+
 # ------------------------------------------------------------------ the tests
 
-SCENARIOS = [layer_too_wide_for_shared_memory, first_calls_in_two_threads, every_device]
+SCENARIOS = [layer_too_wide_for_shared_memory, first_calls_in_two_threads, every_device, device_images_of_any_alignment]
 
 
 @pytest.mark.parametrize("scenario", [s.__name__ for s in SCENARIOS])
