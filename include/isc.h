@@ -173,17 +173,19 @@ int isc_sample_counts(isc_model *m, const uint8_t *x_u8, uint64_t seed, uint64_t
  * running under a memory budget enforced by refusing allocations.  For them this entry
  * point computes the same vote counts as isc_sample_counts, but takes every byte of its
  * device work space (activation buffers, noise table, staged image, counts) from one fixed
- * 32 MiB array that is part of the library image.  The kernels are those isc_sample_counts
- * takes: the resident engine where the model fits it (it needs no activation buffers), else
- * the layer-by-layer ones, with tensor cores unless the "engine" option is 1.  It calls no cudaMalloc / cudaFree and no allocating library routine; the model
- * handle must have been loaded beforehand (loading does allocate).  Each GPU on which the
- * library is loaded holds that array until the process exits.
+ * 32 MiB array that is part of the library image.  The engine is the one isc_sample_counts
+ * would take, by the "engine" option or by itself: the resident one needs no activation
+ * buffers, the layer-by-layer ones have theirs in the array.  It calls no cudaMalloc / cudaFree
+ * and no allocating library routine; the model handle must have been loaded beforehand (loading
+ * does allocate).  Each GPU on which the library is loaded holds that array until the process
+ * exits.
  *
  *   arguments  : as isc_sample_counts (x_u8 and out_counts are host pointers); no logits.
  *   limits     : returns ISC_ERR_UNSUPPORTED, doing nothing, when one sample's activation
  *                buffers do not fit in the array, when the image exceeds 1 MiB, when the
- *                noise table exceeds 16384 entries (sigma above about 4.5) or when
- *                n_classes exceeds 4096.  Any n_samples is accepted: samples are processed
+ *                noise table exceeds 16384 entries (sigma above about 4.5), when
+ *                n_classes exceeds 4096, or when the model does not fit the engine that the
+ *                "engine" option names.  Any n_samples is accepted: samples are processed
  *                in batches as large as the array allows.
  *   first call : the first call made on a device looks up the array's device address (the
  *                device must be current); make that call before starting a stream capture.

@@ -1114,6 +1114,8 @@ extern "C" int isc_sample_counts_static(isc_model *m, const uint8_t *x_u8, uint6
     if ((size_t)(2 * T + 1) * sizeof(uint32_t) > kStaticTableBytes) return ISC_ERR_UNSUPPORTED;
     if (d > kStaticImageBytes) return ISC_ERR_UNSUPPORTED;
     if (per_sample > ISC_STATIC_SCRATCH_BYTES - fixed - 4096) return ISC_ERR_UNSUPPORTED;
+    const int engine = choose_engine(m);
+    if (engine < 0) return engine;
 
     unsigned char *base = nullptr;
     if ((rc = static_scratch_base(&base))) return rc;
@@ -1139,14 +1141,13 @@ extern "C" int isc_sample_counts_static(isc_model *m, const uint8_t *x_u8, uint6
     // (ResNet-20, 2,000 samples: 4.1 ms with the plain kernels, 0.56 ms on the resident engine.)
     // The resident engine needs no work space but this; the layer-by-layer kernels take their activation buffers from the
     // rest of the array, as many samples at a time as fit.
-    const bool plain = m->opt_engine == 1;
-    if (m->line && !plain) {
+    if (engine == 3) {
         // (its parameters carry the image's number on their own)
         ns.ctr3_fixed = (uint32_t)phase;
         const isc::LineWork w{d_x, 1, image_id, 0, n_samples, 0, d_counts, nullptr};
         rc = isc::line_run(m->line, w, ns, 0, d_err, st, &m->launches);
     } else {
-        const bool tensor_cores = m->has_tc && !plain;
+        const bool tensor_cores = engine == 2;
         const int64_t cap = std::min<int64_t>(tensor_cores ? tensor_core_cap(m) : 32768, (int64_t)((ISC_STATIC_SCRATCH_BYTES - fixed - 4096) / per_sample));
         std::vector<int8_t *> buf(m->buf_bytes.size());
         size_t off = fixed + 4096;

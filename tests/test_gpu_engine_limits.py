@@ -36,3 +36,12 @@ def test_device_images_of_any_alignment(net):
         got = gm.certify_batch(None, 3, 7, 0, 20, 150, 0.25, 0.001, device_ptr=buf.data_ptr() + offset)
         for g, e in zip(got, expected):
             np.testing.assert_array_equal(g, e)
+
+
+def test_static_entry_point_on_the_engine_it_is_told():
+    gm = isc.Model(wl.spread_model("resnet20"))
+    x = wl.spread_image()
+    expected = gm.sample_counts(x, 9, 5, 1, 3, 1203, 0.25)
+    for engine in (1, 2, 3):
+        gm.set_option("engine", engine)
+        np.testing.assert_array_equal(gm.sample_counts_static(x, 9, 5, 1, 3, 1203, 0.25), expected)

@@ -139,9 +139,34 @@ def device_images_of_any_alignment():
             assert any(f.fake_launch_watched(i) for i in range(f.fake_launches())) == (offset % 4 == 0), offset
 
 
+def static_entry_point_takes_the_engine_it_is_told():
+    """The allocation-free entry point takes the engine that isc_sample_counts takes under the same option, and refuses what
+    that refuses, launching nothing."""
+    import paper_2108_09413_b200 as isc
+    import workloads as wl
+    f = _fake()
+    for model in (wl.resnet20(), _filter_net(wl)):
+        gm = isc.Model(model)
+        x = wl.images(1, shape=model["in_shape"])[0]
+        for engine in (0, 1, 2, 3):
+            gm.set_option("engine", engine)
+            taken = []
+            for call in (gm.sample_counts, gm.sample_counts_static):
+                f.fake_reset()
+                try:
+                    call(x, 1, 0, 1, 0, 9, 0.25)
+                except isc.IscError as e:
+                    assert e.code == -3 and f.fake_launches() == 0
+                taken.append(_kernels(f))
+            assert taken[0] == taken[1], (engine, taken)
+            assert ("k_line" in taken[1]) == (gm.get_info("has_line_engine") == 1 and engine in (0, 3))
+            assert bool(taken[1]) == (engine != 3 or gm.get_info("has_line_engine") == 1)
+
+
 # ------------------------------------------------------------------ the tests
 
-SCENARIOS = [layer_too_wide_for_shared_memory, first_calls_in_two_threads, every_device, device_images_of_any_alignment]
+SCENARIOS = [layer_too_wide_for_shared_memory, first_calls_in_two_threads, every_device, device_images_of_any_alignment,
+             static_entry_point_takes_the_engine_it_is_told]
 
 
 @pytest.mark.parametrize("scenario", [s.__name__ for s in SCENARIOS])
