@@ -332,8 +332,10 @@ int isc_debug_residual_form(int32_t res_mult, int32_t res_shift, int32_t zp_res,
  *              the tcgen05 kernels for every convolution and FC layer, 3 = the line-tiled
  *              shared-memory-resident tensor-core kernel (2 and 3 give
  *              ISC_ERR_UNSUPPORTED at the next call if the model does not fit).
- * isc_get_info reads back: "engine" (the engine the last call used; 1 after every
- * isc_sample_counts_static, whichever kernels it took), "gpu_launches"
+ * isc_get_info reads back: "engine" (the engine the last call used; after
+ * isc_sample_counts_static it reads 1 for callers that rely on that, and says nothing),
+ * "static_engine" (the engine the last isc_sample_counts_static used, 0 before the first),
+ * "gpu_launches"
  * (kernel launches issued by this handle so far), "macs_per_sample",
  * "has_line_engine" (1 if the model fits engine 3), "has_tensor_core_layers" (1 if
  * engine 2 has a layer to run) and, for engine 3, "cycles_fill",

@@ -81,7 +81,7 @@ struct isc_model {
     std::vector<cudaEvent_t> events;
 
     int64_t opt_batch = 0, opt_engine = 0, opt_noise = 0, opt_tensor_copy = 1;
-    int64_t last_engine = 0, launches = 0;
+    int64_t last_engine = 0, last_static_engine = 0, launches = 0;
 };
 
 namespace {
@@ -1157,7 +1157,8 @@ extern "C" int isc_sample_counts_static(isc_model *m, const uint8_t *x_u8, uint6
         }
         rc = forward_counts(m, buf.data(), cap, tensor_cores, d_x, ns, n_samples, st, d_counts, nullptr, d_err);
     }
-    m->last_engine = 1;
+    m->last_engine = 1;                 // "engine" has always read 1 after this entry point; "static_engine" tells which one ran
+    m->last_static_engine = engine;
     if (rc) { cudaStreamSynchronize(st); return rc; }
     std::vector<int32_t> h(counts_off / sizeof(int32_t) + C);
     CK(cudaMemcpyAsync(h.data(), base, h.size() * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
@@ -1199,6 +1200,7 @@ int isc_get_info(isc_model *m, const char *name, int64_t *out)
 {
     if (!m || !name || !out) return ISC_ERR_ARG;
     if (!strcmp(name, "engine")) *out = m->last_engine;
+    else if (!strcmp(name, "static_engine")) *out = m->last_static_engine;
     else if (!strcmp(name, "gpu_launches")) *out = m->launches;
     else if (!strcmp(name, "macs_per_sample")) *out = m->macs;
     else if (!strcmp(name, "has_line_engine")) *out = m->line ? 1 : 0;

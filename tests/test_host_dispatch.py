@@ -160,6 +160,8 @@ def static_entry_point_takes_the_engine_it_is_told():
                 taken.append(_kernels(f))
             assert taken[0] == taken[1], (engine, taken)
             assert ("k_line" in taken[1]) == (gm.get_info("has_line_engine") == 1 and engine in (0, 3))
+            if taken[1]:
+                assert gm.get_info("static_engine") == (engine or (3 if gm.get_info("has_line_engine") else 2))
             assert bool(taken[1]) == (engine != 3 or gm.get_info("has_line_engine") == 1)
 
 
