@@ -46,8 +46,8 @@ struct isc_model {
     // device parameters of the layer-by-layer engine
     std::vector<GLayer> glayers;
     std::vector<void *> param_allocs;
-    std::vector<const int8_t *> wpacks;         // per layer: repacked weights of the tensor-core convolution, or null
-    std::vector<const int8_t *> hpacks;         // per layer: the same for the kernel with resident input tiles, where that takes the layer
+    std::vector<const int8_t *> wpacks;         // per layer: weights repacked for k_igemm (layer 0: k_stem), or null
+    std::vector<const int8_t *> hpacks;         // per layer: weights repacked for k_halo, which takes the layer then, or null
     std::vector<const int32_t *> tc_cst;        // per layer: its epilogue constants
     std::vector<char> tc_fast;
     std::vector<uint32_t> tc_resk;           // per layer: offset of the residual term's two-instruction form, or 0xFFFFFFFF
@@ -272,22 +272,16 @@ int build_generic_engine(isc_model *m)
                 m->tc_fast[0] = igemm_constants(G, bias.data(), mult.data(), shift.data(), c4.data(), igemm_padded_cout(G), false, nullptr) ? 1 : 0;
                 rc = upload(m, c4, &m->tc_cst[0]); if (rc) return rc;
             }
-            if (i > 0 && (igemm_takes(G) || halo_fits(G))) {      // the same layer for the tensor-core kernels
-                if (igemm_takes(G)) {
-                    std::vector<int8_t> wp(igemm_pack_bytes(G));
-                    igemm_pack_weights(G, H.w.data(), wp.data());
-                    rc = upload(m, wp, &m->wpacks[(size_t)i]); if (rc) return rc;
-                }
-                const int n_cst = std::max(igemm_padded_cout(G), halo_padded_cout(G));
+            const bool halo = i > 0 && halo_fits(G);
+            if (halo || (i > 0 && igemm_takes(G))) {        // the same layer for the tensor-core kernel that takes it
+                std::vector<int8_t> wp(halo ? halo_pack_bytes(G) : igemm_pack_bytes(G));
+                if (halo) halo_pack(G, H.w.data(), wp.data()); else igemm_pack_weights(G, H.w.data(), wp.data());
+                rc = upload(m, wp, halo ? &m->hpacks[(size_t)i] : &m->wpacks[(size_t)i]); if (rc) return rc;
+                const int n_cst = halo ? halo_padded_cout(G) : igemm_padded_cout(G);
                 std::vector<int32_t> c4((size_t)n_cst * 4);
                 m->tc_fast[(size_t)i] = igemm_constants(G, bias.data(), mult.data(), shift.data(), c4.data(), n_cst, H.d.res_tensor >= 0, &m->tc_resk[(size_t)i]) ? 1 : 0;
                 rc = upload(m, c4, &m->tc_cst[(size_t)i]); if (rc) return rc;
                 m->has_tc = true;
-                if (halo_fits(G)) {
-                    std::vector<int8_t> hp(halo_pack_bytes(G));
-                    halo_pack(G, H.w.data(), hp.data());
-                    rc = upload(m, hp, &m->hpacks[(size_t)i]); if (rc) return rc;
-                }
             }
         }
         m->glayers[(size_t)i] = G;

@@ -1931,8 +1931,6 @@ void line_free(LinePlan *p)
     delete p;
 }
 
-static void line_free_streams(LinePlan *p);
-
 // The side streams start after what `st` holds so far ...
 static int line_fork(LinePlan *p, cudaStream_t st)
 {

@@ -165,10 +165,23 @@ def static_entry_point_takes_the_engine_it_is_told():
             assert bool(taken[1]) == (engine != 3 or gm.get_info("has_line_engine") == 1)
 
 
+def weights_are_on_the_device_once_per_kernel():
+    """A filter layer's weights are uploaded for the plain kernel and for the one tensor-core kernel that takes the layer."""
+    import paper_2108_09413_b200 as isc
+    import workloads as wl
+    f = _fake()
+    rng = wl.SplitMix64(6)
+    L = [wl._conv(rng, 0, 3, 256, 3, 1, 1, True, 3, -128), wl._conv(rng, 1, 256, 256, 3, 1, 1, True, -128, -128),
+         wl._gavgpool(2, 256, 24 * 24, -128), wl._conv(rng, 3, 256, 5, 1, 1, 0, False, -128, 0, op=wl.OP_FC)]
+    gm = isc.Model(dict(in_shape=(3, 24, 24), n_classes=5, layers=L))
+    assert 2.0 <= f.fake_allocated() / L[1]["w"].size < 2.3
+    gm.close()
+
+
 # ------------------------------------------------------------------ the tests
 
 SCENARIOS = [layer_too_wide_for_shared_memory, first_calls_in_two_threads, every_device, device_images_of_any_alignment,
-             static_entry_point_takes_the_engine_it_is_told]
+             static_entry_point_takes_the_engine_it_is_told, weights_are_on_the_device_once_per_kernel]
 
 
 @pytest.mark.parametrize("scenario", [s.__name__ for s in SCENARIOS])
