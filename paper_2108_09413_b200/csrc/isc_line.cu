@@ -1154,6 +1154,7 @@ struct LinePlan {
     int attr_device = -1;                // the device on which k_line's shared-memory limit has been raised
     // launches smaller than the GPU (see line_run)
     cudaStream_t side[kSideStreams] = {};
+    int side_priority = 0, side_device = 0;
     cudaEvent_t fork_event = nullptr, join_event[kSideStreams] = {};
 };
 
@@ -1931,13 +1932,19 @@ void line_free(LinePlan *p)
     delete p;
 }
 
-// The side streams start after what `st` holds so far ...
+// The side streams start after what `st` holds so far.  They have its priority and live on the current device: a call on
+// a stream of another priority than the last one's makes them anew (what they held then has been joined and waited for).
 static int line_fork(LinePlan *p, cudaStream_t st)
 {
+    int priority = 0, device = 0;
+    if (cudaStreamGetPriority(st, &priority) != cudaSuccess || cudaGetDevice(&device) != cudaSuccess) { cudaGetLastError(); return ISC_ERR_CUDA; }
+    if (p->fork_event && (p->side_priority != priority || p->side_device != device)) line_free_streams(p);
     if (!p->fork_event) {
+        p->side_priority = priority;
+        p->side_device = device;
         bool ok = cudaEventCreateWithFlags(&p->fork_event, cudaEventDisableTiming) == cudaSuccess;
         for (int i = 0; i < kSideStreams && ok; ++i)
-            ok = cudaStreamCreateWithFlags(&p->side[i], cudaStreamNonBlocking) == cudaSuccess &&
+            ok = cudaStreamCreateWithPriority(&p->side[i], cudaStreamNonBlocking, priority) == cudaSuccess &&
                  cudaEventCreateWithFlags(&p->join_event[i], cudaEventDisableTiming) == cudaSuccess;
         if (!ok) { cudaGetLastError(); line_free_streams(p); return ISC_ERR_CUDA; }
     }

@@ -12,8 +12,8 @@
 #define MAX_LAUNCHES 65536
 
 typedef struct { const void *host; const char *name; int smem[MAX_DEVICES]; } Func;
-typedef struct { const char *name; int device, priority, ok, watched; } Launch;
-struct CUstream_st { int priority; };
+typedef struct { const char *name; int device, stream_device, priority, ok, watched; } Launch;
+struct CUstream_st { int priority, device; };
 
 static Func funcs[MAX_FUNCS];
 static int n_funcs, n_launches, set_attribute_delay_us;
@@ -33,6 +33,7 @@ int fake_launches(void) { return n_launches; }
 const char *fake_launch_name(int i) { return launches[i].name; }
 int fake_launch_device(int i) { return launches[i].device; }
 int fake_launch_priority(int i) { return launches[i].priority; }
+int fake_launch_stream_device(int i) { return launches[i].stream_device; }
 int fake_launch_ok(int i) { return launches[i].ok; }
 /* 1: the word `watch` stands in the launch's first argument */
 void fake_watch(const void *word) { watched = word; }
@@ -81,7 +82,7 @@ cudaError_t cudaLaunchKernel(const void *func, dim3 grid, dim3 block, void **arg
         /* the first argument of the kernels in question is a structure of more than 256 bytes */
         if (watched && (strstr(f->name, "k_stem") || strstr(f->name, "k_line")))
             for (int i = 0; i < 256 / 8; ++i) seen |= ((const void **)args[0])[i] == watched;
-        launches[n_launches++] = (Launch){f->name, device, st ? st->priority : 0, ok, seen};
+        launches[n_launches++] = (Launch){f->name, device, st ? st->device : device, st ? st->priority : 0, ok, seen};
     }
     pthread_mutex_unlock(&lock);
     if (!ok) last = cudaErrorInvalidValue;
@@ -148,6 +149,7 @@ cudaError_t cudaStreamCreateWithPriority(cudaStream_t *st, unsigned flags, int p
     (void)flags;
     *st = malloc(sizeof(**st));
     (*st)->priority = priority;
+    (*st)->device = device;
     return cudaSuccess;
 }
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t *st, unsigned flags) { return cudaStreamCreateWithPriority(st, flags, 0); }

@@ -178,10 +178,31 @@ def weights_are_on_the_device_once_per_kernel():
     gm.close()
 
 
+def side_streams_keep_the_callers_priority():
+    """Short launches are dealt to side streams of the engine's own: with the priority of the stream that the call is on."""
+    import paper_2108_09413_b200 as isc
+    import workloads as wl
+    f = _fake()
+    gm = isc.Model(wl.tiny_cnn())
+    gm.set_option("batch", 64)
+    x = wl.images(1)[0]
+    for device, priority in ((0, 0), (0, -5), (0, -5), (0, -1), (1, -1), (0, None)):
+        f.fake_set_device(device)
+        stream = C.c_void_p()
+        if priority is not None:
+            f.cudaStreamCreateWithPriority(C.byref(stream), 1, priority)
+        f.fake_reset()
+        gm.sample_counts(x, 1, 0, 1, 0, 500, 0.25, stream=stream.value)
+        assert f.fake_launches() == 8
+        for i in range(8):
+            assert (f.fake_launch_priority(i), f.fake_launch_stream_device(i)) == (priority or 0, device)
+
+
 # ------------------------------------------------------------------ the tests
 
 SCENARIOS = [layer_too_wide_for_shared_memory, first_calls_in_two_threads, every_device, device_images_of_any_alignment,
-             static_entry_point_takes_the_engine_it_is_told, weights_are_on_the_device_once_per_kernel]
+             static_entry_point_takes_the_engine_it_is_told, weights_are_on_the_device_once_per_kernel,
+             side_streams_keep_the_callers_priority]
 
 
 @pytest.mark.parametrize("scenario", [s.__name__ for s in SCENARIOS])
