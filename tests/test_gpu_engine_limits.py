@@ -25,7 +25,7 @@ def test_layers_around_the_shared_memory_limit_of_the_tensor_core_kernel(cin, co
 @pytest.mark.parametrize("net", ["resident", "layerwise"])
 def test_device_images_of_any_alignment(net):
     import torch
-    model = wl.spread_model("resnet20") if net == "resident" else wl.resnet50(hw=32, blocks=(1, 1, 1, 1))
+    model = wl.spread_model("resnet20") if net == "resident" else wl.resnet50(hw=64, blocks=(1, 1, 1, 1))
     gm = isc.Model(model)
     xs = wl.images(3, shape=model["in_shape"], seed=8)
     expected = gm.certify_batch(xs, 3, 7, 0, 20, 150, 0.25, 0.001)
