@@ -308,6 +308,16 @@ int isc_debug_tensor(isc_model *m, const uint8_t *x_u8, uint64_t seed, uint64_t 
 int isc_debug_wait_timeout(isc_model *m, int64_t limit_ns, void *cuda_stream, int32_t *out4);
 
 /*
+ * isc_debug_stalled_launch -- the same probe for the kernel that runs layer `layer` (0 = the first)
+ * on the layer-by-layer tensor-core engine: the first convolution's, the filter kernel with resident
+ * input tiles, or the implicit-GEMM kernel.
+ *   returns : ISC_ERR_TIMEOUT when the path works as designed, ISC_OK if no wait expired,
+ *             ISC_ERR_UNSUPPORTED if no tensor-core kernel takes the layer.
+ *   out2    : host, 2 int32: the kernel's error word, host nanoseconds of the launch, saturated.
+ */
+int isc_debug_stalled_launch(isc_model *m, int layer, void *cuda_stream, int32_t *out2);
+
+/*
  * isc_debug_residual_form -- host only.  The tensor-core engines compute the residual operand's
  * rescale rs((r - zp_res) * res_mult, 31 - res_shift) (the skip path's term of the residual add)
  * as floor((u * m2 + R2) / 2^32), u = r + 128, and, where an offset k < 4096 exists for which

@@ -53,7 +53,7 @@ struct isc_model {
     std::vector<uint32_t> tc_resk;           // per layer: offset of the residual term's two-instruction form, or 0xFFFFFFFF
     bool has_tc = false;
     isc::TcDevice tc;
-    int32_t *d_tc_err = nullptr;
+    int32_t *d_tc_err = nullptr;                // error word of the stalled launches (see stalled_launch)
 
     // activation buffers: tensor t lives in pool buffer tensor_buf[t] (bytes per sample buf_bytes[b])
     std::vector<int> tensor_buf;
@@ -286,13 +286,6 @@ int build_generic_engine(isc_model *m)
         }
         m->glayers[(size_t)i] = G;
     }
-    if (m->has_tc) {
-        std::vector<int32_t> zero(1, 0);
-        const int32_t *p = nullptr;
-        int rc = upload(m, zero, &p); if (rc) return rc;
-        m->d_tc_err = const_cast<int32_t *>(p);
-    }
-
     // buffer plan: greedy reuse by last use
     std::vector<int> last_use((size_t)n + 1, -1);
     for (int i = 0; i < n; ++i) {
@@ -636,6 +629,46 @@ int count_images(isc_model *m, const uint8_t *x, bool x_on_device, int n_images,
         }
     }
     return call_status(m);
+}
+
+// One launch of the tensor-core kernel that takes layer `li`, on one sample's work space, with the weights held back: the
+// kernel's own waits run out and its CTAs leave through the abort path; the error word must be up afterwards.
+int stalled_launch(isc_model *m, size_t li, cudaStream_t st, int32_t *err, int32_t *ns)
+{
+    if (!m->wpacks[li] && !m->hpacks[li]) return ISC_ERR_UNSUPPORTED;
+    const GLayer &G = m->glayers[li];
+    const isc_layer &L = m->layers[li].d;
+    const uint8_t *d_x = nullptr;
+    int rc = ensure_workspace(m, 1);
+    if (rc == ISC_OK) rc = ready_tensor_cores(m);
+    if (rc == ISC_OK && li == 0) {                           // the stem draws its noise first: on an empty image
+        const std::vector<uint8_t> x((size_t)m->in_c * m->in_h * m->in_w, 0);
+        rc = ensure_noise_table(m, 0.25, st);
+        if (rc == ISC_OK) rc = begin_call(m, x.data(), x.size(), false, (size_t)m->n_classes, st, &d_x);
+        if (rc == ISC_OK) CK(cudaStreamSynchronize(st));
+    }
+    if (rc) return rc;
+    if (!m->d_tc_err) {
+        const int32_t *p = nullptr;
+        if ((rc = upload(m, std::vector<int32_t>(1, 0), &p))) return rc;
+        m->d_tc_err = const_cast<int32_t *>(p);
+    }
+    int8_t *out = (int8_t *)m->bufs[(size_t)m->tensor_buf[li + 1]].p;
+    const int8_t *in = li ? (const int8_t *)m->bufs[(size_t)m->tensor_buf[(size_t)L.in_tensor]].p : nullptr;
+    const int8_t *res = L.res_tensor >= 0 ? (const int8_t *)m->bufs[(size_t)m->tensor_buf[(size_t)L.res_tensor]].p : nullptr;
+    const bool fast = m->tc_fast[li] != 0;
+    const auto t0 = std::chrono::steady_clock::now();
+    cudaError_t e;
+    if (li == 0) e = launch_stem_conv(G, m->wpacks[0], m->tc_cst[0], fast, d_x, m->in_c, make_stream(m, 1, 0, 1, 0), 1, out, m->d_tc_err, st, true);
+    else if (m->hpacks[li]) e = launch_halo_conv(m->tc, G, m->hpacks[li], m->tc_cst[li], fast, m->tc_resk[li], 1, in, res, out, m->d_tc_err, st, true);
+    else e = launch_igemm_conv(m->tc, G, m->wpacks[li], m->tc_cst[li], fast, m->tc_resk[li], 1, in, res, out, m->d_tc_err, st, true);
+    if (e != cudaSuccess) return ISC_ERR_CUDA;
+    CK(cudaStreamSynchronize(st));
+    const long long t = std::chrono::duration_cast<std::chrono::nanoseconds>(std::chrono::steady_clock::now() - t0).count();
+    CK(cudaMemcpy(err, m->d_tc_err, sizeof(*err), cudaMemcpyDeviceToHost));
+    CK(cudaMemset(m->d_tc_err, 0, sizeof(*err)));
+    *ns = (int32_t)std::min<long long>(t, 0x7FFFFFFF);
+    return *err != 0 ? ISC_ERR_TIMEOUT : ISC_OK;
 }
 
 }  // namespace
@@ -1019,37 +1052,31 @@ int isc_debug_wait_timeout(isc_model *m, int64_t limit_ns, void *cuda_stream, in
 {
     if (!m || !out4) return ISC_ERR_ARG;
     if (!m->line && m->has_tc) {
-        // The layer-by-layer tensor-core engine: one launch of its first implicit-GEMM layer on one sample's work
-        // space with the weights held back, so that the kernel's own waits run out and its CTAs leave through the
-        // abort path; the error word must be up afterwards.
-        cudaStream_t st = (cudaStream_t)cuda_stream;
+        // the layer-by-layer tensor-core engine: its first implicit-GEMM layer
         size_t li = 1;
         while (li < m->glayers.size() && !m->wpacks[li]) ++li;
         if (li >= m->glayers.size()) return ISC_ERR_UNSUPPORTED;
-        int rc = ensure_workspace(m, 1);
-        if (rc == ISC_OK) rc = ready_tensor_cores(m);
-        if (rc) return rc;
-        const GLayer &G = m->glayers[li];
-        const isc_layer &L = m->layers[li].d;
-        int8_t *out = (int8_t *)m->bufs[(size_t)m->tensor_buf[li + 1]].p;
-        const int8_t *in = (const int8_t *)m->bufs[(size_t)m->tensor_buf[(size_t)L.in_tensor]].p;
-        const int8_t *res = L.res_tensor >= 0 ? (const int8_t *)m->bufs[(size_t)m->tensor_buf[(size_t)L.res_tensor]].p : nullptr;
-        const auto t0 = std::chrono::steady_clock::now();
-        if (launch_igemm_conv(m->tc, G, m->wpacks[li], m->tc_cst[li], m->tc_fast[li] != 0, m->tc_resk[li], 1, in, res, out, m->d_tc_err, st, true) != cudaSuccess)
-            return ISC_ERR_CUDA;
-        CK(cudaStreamSynchronize(st));
-        const long long ns = std::chrono::duration_cast<std::chrono::nanoseconds>(std::chrono::steady_clock::now() - t0).count();
-        int32_t e = 0;
-        CK(cudaMemcpy(&e, m->d_tc_err, sizeof(e), cudaMemcpyDeviceToHost));
-        CK(cudaMemset(m->d_tc_err, 0, sizeof(e)));
-        out4[0] = 0; out4[1] = 0; out4[2] = e; out4[3] = (int32_t)std::min<long long>(ns, 0x7FFFFFFF);
-        return e != 0 ? ISC_ERR_TIMEOUT : ISC_OK;
+        int32_t e = 0, ns = 0;
+        const int rc = stalled_launch(m, li, (cudaStream_t)cuda_stream, &e, &ns);
+        if (rc != ISC_OK && rc != ISC_ERR_TIMEOUT) return rc;
+        out4[0] = 0; out4[1] = 0; out4[2] = e; out4[3] = ns;
+        return rc;
     }
     if (!m->line) return ISC_ERR_UNSUPPORTED;
     int32_t tmp[4] = {0, 0, 0, 0};
     const int rc = isc::line_wait_probe(m->line, limit_ns, tmp, (cudaStream_t)cuda_stream);
     if (rc == ISC_ERR_ARG || rc == ISC_ERR_CUDA) return rc;
     memcpy(out4, tmp, sizeof(tmp));
+    return rc;
+}
+
+int isc_debug_stalled_launch(isc_model *m, int layer, void *cuda_stream, int32_t *out2)
+{
+    if (!m || !out2 || layer < 0 || layer >= (int)m->layers.size()) return ISC_ERR_ARG;
+    int32_t e = 0, ns = 0;
+    const int rc = stalled_launch(m, (size_t)layer, (cudaStream_t)cuda_stream, &e, &ns);
+    if (rc != ISC_OK && rc != ISC_ERR_TIMEOUT) return rc;
+    out2[0] = e; out2[1] = ns;
     return rc;
 }
 

@@ -74,6 +74,7 @@ struct HaloParams {
     int fast, lo, res_short;
     uint32_t res_m2, res_k8;
     long long res_r2;
+    int debug_stall;                         // test hook: the weights are never sent, so that the kernel's waits run out
     int32_t *err;
 };
 
@@ -391,7 +392,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_halo(const __grid_constant__ Ha
         ok = L.kh == 3 ? issue_role<3>(p, sbase, tmem, mt, a_bars, b_bars, acc_bars, &abort_s) : issue_role<0>(p, sbase, tmem, mt, a_bars, b_bars, acc_bars, &abort_s);
     } else {
         // ---- one thread streams the repacked weights
-        if (lane == 0) {
+        if (lane == 0 && !p.debug_stall) {
             if (p.resident) {
                 const uint32_t blocks = (uint32_t)(p.tiles_n * p.n_blocks);
                 mbar_expect_tx(b_bars.x, blocks * block_bytes);
@@ -427,6 +428,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_halo(const __grid_constant__ Ha
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    __syncwarp();                                         // lanes that gave up a wait on their own meet again
     if (warp == 0) tmem_dealloc(tmem, (uint32_t)p.tmem_cols);
 }
 
@@ -547,7 +549,7 @@ void halo_pack(const GLayer &G, const int8_t *w, int8_t *out)
 cudaError_t halo_prepare() { return cudaFuncSetAttribute(k_halo, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax); }
 
 cudaError_t launch_halo_conv(const TcDevice &dev, const GLayer &G, const int8_t *wpack, const int32_t *cst, bool fast, uint32_t res_k8, int batch,
-                             const int8_t *in, const int8_t *res, int8_t *out, int32_t *err, cudaStream_t st)
+                             const int8_t *in, const int8_t *res, int8_t *out, int32_t *err, cudaStream_t st, bool debug_stall)
 {
     HaloConfig c;
     if (!halo_config(G, &c) || !halo_offsets_fit(G, batch)) return cudaErrorInvalidValue;
@@ -590,6 +592,7 @@ cudaError_t launch_halo_conv(const TcDevice &dev, const GLayer &G, const int8_t 
         p.res_m2 = (uint32_t)((unsigned long long)(uint32_t)G.res_mult << (32 - res_n));
         p.res_r2 = ((1ll << (res_n - 1)) - (128ll + G.zp_res) * (long long)G.res_mult) * (1ll << (32 - res_n));
     }
+    p.debug_stall = debug_stall ? 1 : 0;
     p.err = err;
     k_halo<<<std::min<uint32_t>(p.n_items, (uint32_t)dev.n_sms), kThreads, c.smem, st>>>(p);
     return cudaGetLastError();

@@ -506,6 +506,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_igemm(const __grid_constant
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    __syncwarp();                                         // lanes that gave up a wait on their own meet again
     if (warp == 0) tmem_dealloc(tmem, (uint32_t)p.tmem_cols);
 }
 
@@ -539,6 +540,7 @@ struct StemParams {
     const int8_t *wpack;                     // [filter row][2 K columns][coutp rows][16 bytes]
     const int4 *cst;
     int fast_requant, lo;
+    int debug_stall;                         // test hook: the weights are never sent, so that the kernel's waits run out
     int8_t *out;
     int32_t *err;
 };
@@ -615,7 +617,7 @@ __global__ void __launch_bounds__(kStemThreads, 2) k_stem(const __grid_constant_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_base_s;
-    if (tid == 0) {
+    if (tid == 0 && !p.debug_stall) {
         mbar_expect_tx(smem_u32(&bar_w), p.w_bytes);
         bulk_g2s(sbase, p.wpack, p.w_bytes, smem_u32(&bar_w));
     }
@@ -729,6 +731,7 @@ __global__ void __launch_bounds__(kStemThreads, 2) k_stem(const __grid_constant_
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    __syncwarp();                                         // lanes that gave up a wait on their own meet again
     if (warp == 0) tmem_dealloc(tmem, (uint32_t)p.tmem_cols);
 }
 
@@ -1029,7 +1032,7 @@ void stem_pack_weights(const GLayer &G, const int8_t *w, int8_t *out)
 }
 
 cudaError_t launch_stem_conv(const GLayer &G, const int8_t *wpack, const int32_t *cst, bool fast, const uint8_t *x_chw, int in_c,
-                             const NoiseStream &ns, int batch, int8_t *out, int32_t *err, cudaStream_t st)
+                             const NoiseStream &ns, int batch, int8_t *out, int32_t *err, cudaStream_t st, bool debug_stall)
 {
     StemParams p;
     p.L = G;
@@ -1050,6 +1053,7 @@ cudaError_t launch_stem_conv(const GLayer &G, const int8_t *wpack, const int32_t
     p.fast_requant = fast ? 1 : 0;
     p.lo = G.relu ? (G.zp_out > -128 ? G.zp_out : -128) : -128;
     p.out = out; p.err = err;
+    p.debug_stall = debug_stall ? 1 : 0;
     size_t smem = c.smem();
     // the noise tables go to shared memory when two CTAs per SM still fit and the guide table follows the cumulative one
     const size_t tab_bytes = ((size_t)(2 * ns.T + 1 + kNoiseGuide + 1) * 4 + 15) & ~(size_t)15;

@@ -105,14 +105,14 @@ size_t halo_pack_bytes(const GLayer &G);
 void halo_pack(const GLayer &G, const int8_t *w_oihw, int8_t *out);
 cudaError_t halo_prepare();                      // part of tc_prepare
 cudaError_t launch_halo_conv(const TcDevice &dev, const GLayer &G, const int8_t *wpack, const int32_t *cst, bool fast, uint32_t res_k8, int batch,
-                             const int8_t *in, const int8_t *res, int8_t *out, int32_t *err, cudaStream_t st);
+                             const int8_t *in, const int8_t *res, int8_t *out, int32_t *err, cudaStream_t st, bool debug_stall = false);
 
 // The first convolution (<= 4 input channels, filter at most 8 x 8) on the tensor cores, noise drawn into its staging.
 bool stem_fits(const GLayer &G, int in_c);
 size_t stem_pack_bytes(const GLayer &G);
 void stem_pack_weights(const GLayer &G, const int8_t *w_oihw, int8_t *out);
 cudaError_t launch_stem_conv(const GLayer &G, const int8_t *wpack, const int32_t *cst, bool fast, const uint8_t *x_chw, int in_c,
-                             const NoiseStream &ns, int batch, int8_t *out, int32_t *err, cudaStream_t st);
+                             const NoiseStream &ns, int batch, int8_t *out, int32_t *err, cudaStream_t st, bool debug_stall = false);
 
 // ---- host decision rules (isc_decide.cpp) ----
 double lower_conf_bound(int64_t k, int64_t n, double alpha);

@@ -5,7 +5,7 @@ import pytest
 import oracle
 import workloads as wl
 import paper_2108_09413_b200 as isc
-from test_host_dispatch import _hidden_layer_net
+from test_host_dispatch import _every_kernel_net, _hidden_layer_net
 
 pytestmark = pytest.mark.gpu
 
@@ -45,3 +45,23 @@ def test_static_entry_point_on_the_engine_it_is_told():
     for engine in (1, 2, 3):
         gm.set_option("engine", engine)
         np.testing.assert_array_equal(gm.sample_counts_static(x, 9, 5, 1, 3, 1203, 0.25), expected)
+
+
+def test_stalled_layers_leave_through_their_abort_path():
+    """One launch of every kernel of the layer-by-layer tensor-core engine whose weights are held back: the first
+    convolution, the filter kernel with its weights resident and with a ring of them, the implicit GEMM.  Its waits run
+    out after their own two seconds, the error word is up (ISC_ERR_TIMEOUT = -6), and the handle then computes the right
+    logits.  Nothing here faults, traps or hangs the GPU."""
+    model = _every_kernel_net(wl)
+    gm, om = isc.Model(model), oracle.Model(model)
+    gm.set_option("engine", 2)
+    x = wl.images(1, shape=model["in_shape"])[0]
+    for layer in (0, 2, 3, 4):
+        rc, (err_word, ns) = gm.debug_stalled_launch(layer)
+        assert rc == -6 and err_word >= 1, layer
+        assert 1_900_000_000 <= ns
+        got = gm.sample_counts(x, 11, 3, 1, 0, 3, 0.5, want_logits=True)
+        exp = oracle.sample_counts(om, x, 11, 3, 1, 0, 3, 0.5, want_logits=True)
+        np.testing.assert_array_equal(got[1], exp[1])
+        np.testing.assert_array_equal(got[0], exp[0])
+    assert gm.debug_stalled_launch(1)[0] == -3 and gm.debug_stalled_launch(len(model["layers"]))[0] == -1

@@ -198,11 +198,38 @@ def side_streams_keep_the_callers_priority():
             assert (f.fake_launch_priority(i), f.fake_launch_stream_device(i)) == (priority or 0, device)
 
 
+def _every_kernel_net(wl):
+    """stem, max-pool, 3 x 3 with resident weights, 3 x 3 with a ring of them, 1 x 1, pool, FC"""
+    rng = wl.SplitMix64(6)
+    L = [wl._conv(rng, 0, 3, 64, 5, 1, 2, True, 3, -128), wl._maxpool(1, 64, 3, 2, 1, -128), wl._conv(rng, 2, 64, 64, 3, 1, 1, True, -128, -128),
+         wl._conv(rng, 3, 64, 256, 3, 1, 1, True, -128, -128), wl._conv(rng, 4, 256, 64, 1, 1, 0, True, -128, -128),
+         wl._gavgpool(5, 64, 100, -128), wl._conv(rng, 6, 64, 7, 1, 1, 0, False, -128, 0, op=wl.OP_FC)]
+    return dict(in_shape=(3, 20, 20), n_classes=7, layers=L)
+
+
+def stalled_launches_reach_every_kernel():
+    """The probe of the bounded waits launches the kernel that runs the layer, and refuses layers without one."""
+    import paper_2108_09413_b200 as isc
+    import workloads as wl
+    f = _fake()
+    gm = isc.Model(_every_kernel_net(wl))
+    gm.set_option("engine", 2)
+    x = wl.images(1, shape=(3, 20, 20))[0]
+    gm.sample_counts(x, 1, 0, 1, 0, 9, 0.25)
+    taken = _kernels(f)
+    assert taken == ["k_stem", "k_maxpool", "k_halo", "k_halo", "k_igemm", "k_gavgpool", "k_igemm", "k_votes"]
+    for layer, kernel in enumerate(taken[:-1]):
+        f.fake_reset()
+        tensor_cores = kernel in ("k_stem", "k_halo", "k_igemm")
+        assert gm.debug_stalled_launch(layer)[0] == (0 if tensor_cores else -3)      # 0: the stand-in's kernels raise no error word
+        assert _kernels(f) == ([kernel] if tensor_cores else [])
+
+
 # ------------------------------------------------------------------ the tests
 
 SCENARIOS = [layer_too_wide_for_shared_memory, first_calls_in_two_threads, every_device, device_images_of_any_alignment,
              static_entry_point_takes_the_engine_it_is_told, weights_are_on_the_device_once_per_kernel,
-             side_streams_keep_the_callers_priority]
+             side_streams_keep_the_callers_priority, stalled_launches_reach_every_kernel]
 
 
 @pytest.mark.parametrize("scenario", [s.__name__ for s in SCENARIOS])
