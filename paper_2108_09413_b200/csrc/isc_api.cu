@@ -1159,7 +1159,7 @@ extern "C" int isc_sample_counts_static(isc_model *m, const uint8_t *x_u8, uint6
     ns.T = T;
     ns.guide = n_tab > n_cum ? ns.cum + n_cum : nullptr;
     ns.guide_steps = n_tab > n_cum ? m->tab_steps : 0;
-    // (ResNet-20, 2,000 samples: 4.1 ms with the plain kernels, 0.56 ms on the resident engine.)
+    // (ResNet-20, 2,000 samples: 4.1 ms with the plain kernels, 0.53 ms on the resident engine.)
     // The resident engine needs no work space but this; the layer-by-layer kernels take their activation buffers from the
     // rest of the array, as many samples at a time as fit.
     if (engine == 3) {

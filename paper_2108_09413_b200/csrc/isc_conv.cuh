@@ -140,19 +140,9 @@ __device__ __forceinline__ void tmem_ld32_wait(int (&v)[2][16])
                  :: "memory");
 }
 
-// Bounded wait for a phase of an mbarrier; false after the limit (the caller raises the error word).
-__device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity)
-{
-    if (mbar_test(bar, parity)) return true;
-    const unsigned long long t0 = globaltimer();
-    for (int spin = 0;; ++spin) {
-        if (mbar_try(bar, parity)) return true;
-        if ((spin & 7) == 7 && globaltimer() - t0 > kWaitLimitNs) return false;
-    }
-}
-// The same for the roles of k_igemm, which also give up when another role has raised the CTA's abort flag.  With
-// `kHintNs` the wait is parked in hardware for up to that long per attempt instead of polling (the abort flag and
-// the time limit are looked at every eighth attempt).
+// Bounded wait of a role for a phase of an mbarrier: false after the limit (the caller raises the error word) or when
+// another role has raised the CTA's abort flag.  With `kHintNs` the wait is parked in hardware for up to that long per
+// attempt instead of polling (the abort flag and the time limit are looked at every eighth attempt).
 template <unsigned kHintNs>
 __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, const volatile int *abort_flag)
 {

@@ -658,7 +658,8 @@ __device__ __noinline__ void store_strided(uint32_t desc, uint32_t sbase, uint32
 }
 
 // The general pass (strided convolutions, a lower clamp above -128, a lone line): one line at a time, every
-// property decided at run time.  The networks of the benchmark reach it in their two strided shortcuts only.
+// property decided at run time.  A CIFAR ResNet reaches it in the four convolutions of its two stage transitions (the
+// stride-2 3 x 3 and the 1 x 1 shortcut).
 __device__ __noinline__ void epi_conv_general(Waiter w, const EpiConv &E, const EpiCtx &c, uint32_t desc, uint32_t flags, int32_t lo,
                                               uint32_t passes, uint32_t n_passes)
 {
@@ -777,7 +778,7 @@ __device__ __forceinline__ GroupJob group_job(const LineParams &p, int grp)
 // INPUT: one item = four horizontally adjacent pixels of one sample and input channel, one Philox block (Def. 3.3,
 // Def. 3.4).  Items of all channels share one index space (3072 items of a 32 x 32 x 3 image for 640 threads; with the
 // channels of a pixel in one thread it was 1024, two rounds of which the second is mostly idle), and the four table
-// searches run interleaved in a fixed number of steps instead of one after the other.  Out of line, like the tail's last
+// searches run interleaved, until all four are found, instead of one after the other.  Out of line, like the tail's last
 // step: the convolutions' loops pay for every register and instruction that these phases share with them.
 __device__ __noinline__ void input_phase(const LineParams &p, const EpiCtx &c, int grp)
 {
