@@ -1987,8 +1987,8 @@ int64_t line_wave_samples(const LinePlan *p) { return (int64_t)kG * p->sm_count;
 // of groups over images and phases: CERTIFY's N0 = 100 samples take 25 of 148 SMs for a whole round when they are launched
 // alone.  Launches of less than eight rounds are dealt to side streams, so that the next ones' groups fill the SMs that
 // one launch leaves idle (64 groups at 256 samples: 0.49 M samples/s one after the other, 1.19 M so; 1,024 samples on
-// ResNet-20 4.3 M, with the fused phases 5.0 M); from eight rounds on what overlap could give is below the launches'
-// own 1-2 %.
+// ResNet-20 4.3 M, with the fused phases 5.0 M).  From eight rounds on launches run one after the other: 16,384 samples
+// each, 27.7 rounds, give 1.28 M samples/s on ResNet-110 where shorter ones that overlap give 1.32 M.
 int line_run(LinePlan *p, const LineWork &w, const NoiseStream &ns, int batch_hint, int32_t *err, cudaStream_t st, int64_t *launches)
 {
     LineParams q = p->base;
