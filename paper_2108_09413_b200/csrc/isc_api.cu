@@ -50,7 +50,7 @@ struct isc_model {
     std::vector<const int8_t *> hpacks;         // per layer: weights repacked for k_halo, which takes the layer then, or null
     std::vector<const int32_t *> tc_cst;        // per layer: its epilogue constants
     std::vector<char> tc_fast;
-    std::vector<uint32_t> tc_resk;           // per layer: offset of the residual term's two-instruction form, or 0xFFFFFFFF
+    std::vector<isc::ResidualForm> tc_resk;  // per layer: the residual term as a single-precision product, where that exists
     bool has_tc = false;
     isc::TcDevice tc;
     int32_t *d_tc_err = nullptr;                // error word of the stalled launches (see stalled_launch)
@@ -218,7 +218,7 @@ int build_generic_engine(isc_model *m)
     m->tc_cst.assign((size_t)n, nullptr);
     m->hpacks.assign((size_t)n, nullptr);
     m->tc_fast.assign((size_t)n, 0);
-    m->tc_resk.assign((size_t)n, 0xFFFFFFFFu);
+    m->tc_resk.assign((size_t)n, isc::ResidualForm());
     for (int i = 0; i < n; ++i) {
         const HostLayer &H = m->layers[(size_t)i];
         const isc_layer &L = H.d;

@@ -26,12 +26,6 @@ __device__ __forceinline__ void commit_to(uint32_t bar)
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-__device__ __forceinline__ long long mul_wide(int a, int b)
-{
-    long long d;
-    asm("mul.wide.s32 %0, %1, %2;" : "=l"(d) : "r"(a), "r"(b));
-    return d;
-}
 __device__ __forceinline__ long long mad_wide_u(uint32_t a, uint32_t b, long long c)
 {
     long long d;
@@ -64,9 +58,12 @@ struct FastDiv {
 //   rs((acc + bias) * mult, 31 + shift) + zp_out = (hi32((acc + bias) * mult) + c) >> s,  c = 2^(s-1) + zp_out * 2^s,
 // exactly (the rounding half 2^(31+s) is a multiple of 2^32, so the product's low word cannot change the floor), and
 //   rs((r - zp_res) * res_mult, n) = hi32(u * m2 + R2),  u = r + 128, m2 = res_mult * 2^(32-n), n = 31 or 32,
-// with R2 = (2^(n-1) - (128 + zp_res) * res_mult) * 2^(32-n) (kRes = 1).  kRes = 2 is the same term without the
-// 64-bit addend: hi32((256 k + u) * m2) - c_r for an offset k that the host has checked on all 256 values of u
-// (residual_short_form); 256 k is merged into u by the byte permute that extracts u, and c_r is folded into c.
+// with R2 = (2^(n-1) - (128 + zp_res) * res_mult) * 2^(32-n) (kRes = 1).  kRes = 2 is the same term as a single-precision
+// product: round((256 k + u) * m) - c_r for an offset k and a multiplier m that the host has checked on all 256 values of
+// u (residual_form; m2 then holds m's bits); 256 k is merged into u by the byte permute that extracts u, and c_r is folded
+// into c.  A wide or high multiply takes four issue cycles of a scheduler here, two more than the single-precision one with
+// everything around it: cycles per output and scheduler, sixteen warps looping over the sequence alone: add, mul.wide, add,
+// shift 6.8, add, mad.hi, shift 6.3; with the residual term by permute, mul.wide, add 12.2, by permute, multiply, add 10.
 // `cst` points at this block's constants in shared memory.
 template <int kRes>
 __device__ __forceinline__ uint4 requant16_fast(const int *acc, uint32_t cst, uint4 rv, uint32_t m2, long long r2, uint32_t k8, int lo)
@@ -80,9 +77,9 @@ __device__ __forceinline__ uint4 requant16_fast(const int *acc, uint32_t cst, ui
         for (int k = 0; k < 4; ++k) {
             int4 c;
             asm("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(c.x), "=r"(c.y), "=r"(c.z), "=r"(c.w) : "r"(cst + (4 * g + k) * 16));
-            int v = (hi32(mul_wide(acc[4 * g + k] + c.x, c.y)) + c.z) >> c.w;
+            int v = mad_hi(acc[4 * g + k] + c.x, c.y, c.z) >> c.w;
             if (kRes == 1) v += hi32(mad_wide_u(__byte_perm(rw[g], 0u, 0x4440u | (uint32_t)k), m2, r2));
-            if (kRes == 2) v += hi32(mad_wide_u(__byte_perm(rw[g], k8, 0x7650u | (uint32_t)k), m2, 0ll));
+            if (kRes == 2) v += mul_denormal(__byte_perm(rw[g], k8, 0x7650u | (uint32_t)k), m2);
             y[k] = max(v, lo);
         }
         packed[g] = pack4_sat(y[0], y[1], y[2], y[3]);
@@ -94,9 +91,9 @@ __device__ __forceinline__ uint4 requant16_fast(const int *acc, uint32_t cst, ui
 template <int kRes, bool kClamp>
 __device__ __forceinline__ int requant1(int acc, const int4 &c, uint32_t rword, int k, uint32_t m2, long long r2, uint32_t k8, int lo)
 {
-    int v = (hi32(mul_wide(acc + c.x, c.y)) + c.z) >> c.w;
+    int v = mad_hi(acc + c.x, c.y, c.z) >> c.w;
     if (kRes == 1) v += hi32(mad_wide_u(__byte_perm(rword, 0u, 0x4440u | (uint32_t)k), m2, r2));
-    if (kRes == 2) v += hi32(mad_wide_u(__byte_perm(rword, k8, 0x7650u | (uint32_t)k), m2, 0ll));
+    if (kRes == 2) v += mul_denormal(__byte_perm(rword, k8, 0x7650u | (uint32_t)k), m2);
     return kClamp ? max(v, lo) : v;
 }
 

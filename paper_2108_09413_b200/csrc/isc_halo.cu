@@ -86,7 +86,7 @@ struct RoleCtx {
 
 // The epilogue of one warp: rows 32 q .. + 31 of both M operands of its team's output tiles, at most 64 channels.
 // kMode 0: 64-bit requantisation (any shift), 1: 32-bit form, 2 / 3: 32-bit form with the residual add (3: its
-// two-instruction form).  kClamp: the lower clamp is above -128.
+// single-precision form).  kClamp: the lower clamp is above -128.
 template <int kMode, bool kClamp>
 __device__ __forceinline__ bool halo_epilogue(const HaloParams &p, const RoleCtx &c)
 {
@@ -548,7 +548,7 @@ void halo_pack(const GLayer &G, const int8_t *w, int8_t *out)
 
 cudaError_t halo_prepare() { return cudaFuncSetAttribute(k_halo, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax); }
 
-cudaError_t launch_halo_conv(const TcDevice &dev, const GLayer &G, const int8_t *wpack, const int32_t *cst, bool fast, uint32_t res_k8, int batch,
+cudaError_t launch_halo_conv(const TcDevice &dev, const GLayer &G, const int8_t *wpack, const int32_t *cst, bool fast, const ResidualForm &form, int batch,
                              const int8_t *in, const int8_t *res, int8_t *out, int32_t *err, cudaStream_t st, bool debug_stall)
 {
     HaloConfig c;
@@ -586,9 +586,11 @@ cudaError_t launch_halo_conv(const TcDevice &dev, const GLayer &G, const int8_t 
     p.lo = G.relu ? (G.zp_out > -128 ? G.zp_out : -128) : -128;
     const int res_n = 31 - G.res_shift;
     p.fast = fast && (!res || res_n == 31 || res_n == 32);
-    p.res_short = res && res_k8 != 0xFFFFFFFFu;
-    p.res_k8 = p.res_short ? res_k8 : 0u;
-    if (res && p.fast) {
+    p.res_short = res && form.exists();
+    p.res_k8 = p.res_short ? form.k8 : 0u;
+    if (p.res_short) {
+        p.res_m2 = form.m_bits;
+    } else if (res && p.fast) {
         p.res_m2 = (uint32_t)((unsigned long long)(uint32_t)G.res_mult << (32 - res_n));
         p.res_r2 = ((1ll << (res_n - 1)) - (128ll + G.zp_res) * (long long)G.res_mult) * (1ll << (32 - res_n));
     }

@@ -33,6 +33,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -74,8 +75,8 @@ struct IgemmParams {
     const int8_t *zp_run;                    // 64 bytes of the input zero-point: the operand row of a pixel outside the image
     const int4 *cst;                         // per output channel: folded bias, multiplier, rounding addend, shift - 1
     int fast_requant, fast_residual, lo;     // every shift >= 2; residual rescale by 2^-31 or 2^-32; lower clamp
-    uint32_t res_m2, res_k8;                 // residual multiplier and addend in the 2^-32 form; offset of the two-instruction form
-    int res_short;                           // the two-instruction form reproduces the residual term (see requant16_fast)
+    uint32_t res_m2, res_k8;                 // residual multiplier in the 2^-32 form, or as a single-precision number; that form's offset
+    int res_short;                           // the residual term is a single-precision product (see requant16_fast)
     int debug_stall;                         // test hook: the weights are never sent, so every wait of the kernel runs out
     long long res_r2;
     int32_t *err;
@@ -96,7 +97,7 @@ struct EpiCtx {
 // 64 contiguous bytes per row and requests the same columns of the residual rows of its next tile into the
 // space that has just been read, so memory traffic runs under the arithmetic of the following columns.
 // kMode 0: 64-bit requantisation (any shift), 1: 32-bit form, 2 / 3: 32-bit form with the residual add (3: its
-// two-instruction form).
+// single-precision form).
 // kWhole: every tile has n_tile valid columns and n_tile is a multiple of 64.
 template <int kMode, bool kWhole>
 __device__ __forceinline__ bool epilogue_role(const IgemmParams &p, const EpiCtx &c)
@@ -853,26 +854,58 @@ bool residual_short_form(int res_mult, int res_shift, int zp_res, uint32_t *k8, 
     return false;
 }
 
+ResidualForm residual_form(int res_mult, int res_shift, int zp_res, int32_t *c_out)
+{
+    ResidualForm f;
+    const int n = 31 - res_shift;
+    if ((n != 31 && n != 32) || res_mult < (1 << 30)) return f;
+    // res_mult / 2^n = mant * 2^-e with a mantissa of 24 bits, and the numbers next to it
+    const int64_t nearest = ((int64_t)res_mult + 64) >> 7;                     // 2^23 .. 2^24
+    const int e = n - 7;
+    for (int64_t mant : {nearest, nearest + 1, nearest - 1}) {
+        if (mant < (1 << 23) || mant > (1 << 24)) continue;
+        for (uint32_t k = 0; k < 4096; ++k) {
+            int64_t c = 0;
+            bool same = true;
+            for (int u = 0; u < 256 && same; ++u) {
+                const int64_t want = ((int64_t)(u - 128 - zp_res) * res_mult + (1ll << (n - 1))) >> n;      // arithmetic shift: floor
+                const int64_t x = (int64_t)(256u * k + (uint32_t)u) * mant, q = x >> e, r = x & ((1ll << e) - 1), half = 1ll << (e - 1);
+                const int64_t got = q + (r > half || (r == half && (q & 1)) ? 1 : 0);
+                if (u == 0) c = got - want;
+                same = got - want == c;
+            }
+            if (!same) continue;
+            const float m = (float)ldexp((double)mant, -e);
+            f.k8 = k << 8;
+            memcpy(&f.m_bits, &m, sizeof(m));
+            *c_out = (int32_t)c;
+            return f;
+        }
+    }
+    return f;
+}
+
 // Per output channel {folded bias, multiplier, rounding addend, shift - 1}; returns whether every shift is >= 2 (the
 // condition of the 32-bit form).  `bias_folded`, `mult`, `shift` are the layer's host arrays padded to coutp.  For a
-// layer with a residual operand whose term has the two-instruction form, that form's constant is folded into the
-// rounding addends and *res_k8 is its offset; otherwise *res_k8 = 0xFFFFFFFF.
+// layer with a residual operand whose term is a single-precision product, that product's constant is folded into the
+// rounding addends.
 bool igemm_constants(const GLayer &G, const int32_t *bias_folded, const int32_t *mult, const int32_t *shift, int32_t *out4, int n_out,
-                     bool has_residual, uint32_t *res_k8)
+                     bool has_residual, ResidualForm *form)
 {
     // channels beyond the layer's own (padding of the tensor and of the last tile) come out as zero
     bool fast = true;
     for (int o = 0; o < G.cout; ++o) fast = fast && shift[o] - 1 >= 1;
-    uint32_t k8 = 0;
     int32_t c_res = 0;
-    bool short_form = fast && has_residual && residual_short_form(G.res_mult, G.res_shift, G.zp_res, &k8, &c_res);
+    ResidualForm f;
+    if (fast && has_residual) f = residual_form(G.res_mult, G.res_shift, G.zp_res, &c_res);
+    bool short_form = f.exists();
     for (int o = 0; o < G.cout && short_form; ++o) {
         const int s = shift[o] - 1;
         const long long add = (1ll << (s - 1)) + ((long long)G.zp_out - c_res) * (1ll << s);
         short_form = add > -(1ll << 31) && add < (1ll << 31);
     }
     if (!short_form) c_res = 0;
-    if (res_k8) *res_k8 = short_form ? k8 : 0xFFFFFFFFu;
+    if (form) *form = short_form ? f : ResidualForm();
     memset(out4, 0, sizeof(int32_t) * 4 * (size_t)n_out);
     for (int o = 0; o < G.cout; ++o) {
         const int s = shift[o] - 1;
@@ -906,7 +939,7 @@ cudaError_t tc_prepare(TcDevice *dev, int ordinal)
     return cudaSuccess;
 }
 
-cudaError_t launch_igemm_conv(const TcDevice &dev, const GLayer &G, const int8_t *wpack, const int32_t *cst, bool fast, uint32_t res_k8, int batch, const int8_t *in,
+cudaError_t launch_igemm_conv(const TcDevice &dev, const GLayer &G, const int8_t *wpack, const int32_t *cst, bool fast, const ResidualForm &form, int batch, const int8_t *in,
                               const int8_t *res, int8_t *out, int32_t *err, cudaStream_t st, bool debug_stall, bool tensor_copy)
 {
     IgemmParams p;
@@ -935,9 +968,11 @@ cudaError_t launch_igemm_conv(const TcDevice &dev, const GLayer &G, const int8_t
         }
     }
     p.res_m2 = 0; p.res_r2 = 0;
-    p.res_short = (res && res_k8 != 0xFFFFFFFFu) ? 1 : 0;
-    p.res_k8 = p.res_short ? res_k8 : 0u;
-    if (res && p.fast_residual) {
+    p.res_short = res && form.exists() ? 1 : 0;
+    p.res_k8 = p.res_short ? form.k8 : 0u;
+    if (p.res_short) {
+        p.res_m2 = form.m_bits;
+    } else if (res && p.fast_residual) {
         p.res_m2 = (uint32_t)((unsigned long long)(uint32_t)G.res_mult << (32 - res_n));
         p.res_r2 = ((1ll << (res_n - 1)) - (128ll + G.zp_res) * (long long)G.res_mult) * (1ll << (32 - res_n));
     }

@@ -81,18 +81,26 @@ bool conv_offsets_fit(const GLayer &G, int64_t batch);  // the batch's tensors a
 size_t igemm_pack_bytes(const GLayer &G);
 void igemm_pack_weights(const GLayer &G, const int8_t *w_oihw, int8_t *out);
 // The residual term F(u) = floor((u * m2 + R2) / 2^32), u = r + 128 in 0..255, of the 32-bit epilogues as
-// hi32((256 k + u) * m2) - c: the smallest k < 4096 for which the two agree on all 256 inputs (*k8 = 256 k), or false.
+// floor((256 k + u) * m2 / 2^32) - c: the smallest k < 4096 for which the two agree on all 256 inputs (*k8 = 256 k), or false.
 bool residual_short_form(int res_mult, int res_shift, int zp_res, uint32_t *k8, int32_t *c);
+// The same term as a single-precision product, round((256 k + u) * m) - c, with round to nearest even and m one of the
+// three single-precision numbers nearest to the multiplier: what the kernels compute where it exists (for more than 99 %
+// of all multipliers), the 64-bit form otherwise.
+struct ResidualForm {
+    uint32_t k8 = 0xFFFFFFFFu, m_bits = 0;       // 256 k; m as stored
+    bool exists() const { return k8 != 0xFFFFFFFFu; }
+};
+ResidualForm residual_form(int res_mult, int res_shift, int zp_res, int32_t *c);
 // Per-channel requantisation constants of the kernel's 32-bit epilogue (4 x int32 for `n_out` channels); returns
 // whether the layer qualifies for it (every shift >= 2).
 bool igemm_constants(const GLayer &G, const int32_t *bias_folded, const int32_t *mult, const int32_t *shift, int32_t *out4, int n_out,
-                     bool has_residual, uint32_t *res_k8);
+                     bool has_residual, ResidualForm *form);
 // `cst` / `fast`: what igemm_constants produced (device copy).  `err` (device) receives a non-zero word if a bounded
 // wait inside the kernel expired.  `debug_stall`: the kernel's weights are never sent, so that its waits run out
 // (after their 2 s limit) and the CTAs leave through the abort path -- nothing faults or hangs.  `tensor_copy`: a
 // 1 x 1 stride-1 layer may take its operand rows by tensor copy (false: the gather warps bring them, as for every
 // other layer).
-cudaError_t launch_igemm_conv(const TcDevice &dev, const GLayer &G, const int8_t *wpack, const int32_t *cst, bool fast, uint32_t res_k8, int batch, const int8_t *in,
+cudaError_t launch_igemm_conv(const TcDevice &dev, const GLayer &G, const int8_t *wpack, const int32_t *cst, bool fast, const ResidualForm &form, int batch, const int8_t *in,
                               const int8_t *res, int8_t *out, int32_t *err, cudaStream_t st, bool debug_stall = false,
                               bool tensor_copy = true);
 
@@ -104,7 +112,7 @@ int halo_padded_cout(const GLayer &G);
 size_t halo_pack_bytes(const GLayer &G);
 void halo_pack(const GLayer &G, const int8_t *w_oihw, int8_t *out);
 cudaError_t halo_prepare();                      // part of tc_prepare
-cudaError_t launch_halo_conv(const TcDevice &dev, const GLayer &G, const int8_t *wpack, const int32_t *cst, bool fast, uint32_t res_k8, int batch,
+cudaError_t launch_halo_conv(const TcDevice &dev, const GLayer &G, const int8_t *wpack, const int32_t *cst, bool fast, const ResidualForm &form, int batch,
                              const int8_t *in, const int8_t *res, int8_t *out, int32_t *err, cudaStream_t st, bool debug_stall = false);
 
 // The first convolution (<= 4 input channels, filter at most 8 x 8) on the tensor cores, noise drawn into its staging.

@@ -79,7 +79,7 @@ constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // 2 s per wait
 
 enum { PH_FILL = 0, PH_INPUT = 1, PH_CONV = 2, PH_TAIL = 3 };
 enum { ERR_NONE = 0, ERR_WAIT_DONE = 1, ERR_WAIT_WEIGHTS = 2, ERR_WAIT_READY = 3, ERR_WAIT_FULL = 4, ERR_WAIT_DRAIN = 5 };
-enum { CF_STACKED = 1, CF_RES = 2, CF_LO = 4, CF_SCATTER = 8, CF_GENERAL = 16, CF_RSHORT = 32 };     // CF_GENERAL: the pass that decides everything at run time; CF_RSHORT: residual term without the 64-bit addend
+enum { CF_STACKED = 1, CF_RES = 2, CF_LO = 4, CF_SCATTER = 8, CF_GENERAL = 16, CF_RSHORT = 32 };     // CF_GENERAL: the pass that decides everything at run time; CF_RSHORT: residual term as a single-precision product
 // OPF_WAIT_ALL: every unit of the previous convolution; OPF_WAITS / OPF_WAITS4: the record names counters to test (two /
 // four slots in use); bits 4-6: how many of them are distinct; bits 8-9: arrivals; bits 10-12: MMA chains
 enum { OPF_WAIT_ALL = 1, OPF_WAITS = 2, OPF_WAITS4 = 8 };
@@ -206,8 +206,8 @@ __device__ __forceinline__ long long mad_wide_u(uint32_t a, uint32_t b, long lon
 //   rs((acc + bias) * mult, 31 + shift) + zp_out = (hi32((acc + bias) * mult) + c) >> s,   c = 2^(s-1) + zp_out * 2^s,
 // exactly: the rounding half 2^(31+s) is a multiple of 2^32, so the low word of the product cannot change the floor.
 // For s = 0 the half sits in the low word: the result is hi32 + (bit 31 of the low word) + c with c = zp_out.
-// The integer pipe issues multiplies, shifts and packs at half rate here, a 64-bit addend costs two more
-// instructions: this form is the cheapest exact one found (add, wide multiply, add, shift).
+// A scheduler issues a wide or high multiply in four cycles here, shifts, permutes and packs in two, additions in one: this
+// form is the cheapest exact one found (add, mad.hi, shift).
 struct ChanConst4 { int bias, mult, c, s; };
 // A plain load (the blob is complete in shared memory; the address derives from a value read after the wait for it)
 // that the compiler may schedule ahead of the tensor-memory wait.
@@ -524,18 +524,18 @@ static_assert(sizeof(LPass) == 32, "one pass is two 16-byte loads");
 // One output of the common pass (every channel has s >= 1).
 //   residual: y += floor((u * m2 + R2) / 2^32) with u = r + 128 the residual byte as an unsigned number,
 //   m2 = res_mult * 2^(32-n) and R2 the rounding half and the zero-points folded: rs((r - zp_res) * res_mult, n).
-//   kRes = 2: the same term as hi32((256 k + u) * m2) - c_r, for an offset k that the planner has checked on all 256
-//   values of u (residual_short_form): `res_r2` then holds 256 k, which the byte permute that extracts u merges
-//   into it, and c_r is folded into the channel's rounding addend.
+//   kRes = 2: the same term as a single-precision product round((256 k + u) * m) - c_r, for an offset k and a multiplier m
+//   that the planner has checked on all 256 values of u (residual_form): `res_r2` then holds 256 k, which the byte
+//   permute that extracts u merges into it, `res_m2` m's bits, and c_r is folded into the channel's rounding addend.
 template <int kRes, int K>
 __device__ __forceinline__ int requant1(int acc, const ChanConst4 &cs, uint32_t rword, uint32_t res_m2, long long res_r2)
 {
-    int y = (hi32(mul_wide(acc + cs.bias, cs.mult)) + cs.c) >> cs.s;
+    int y = mad_hi(acc + cs.bias, cs.mult, cs.c) >> cs.s;
     if (kRes == 1) y += hi32(mad_wide_u(ubyte<K>(rword), res_m2, res_r2));
     if (kRes == 2) {
         uint32_t u;
         asm("prmt.b32 %0, %1, %2, %3;" : "=r"(u) : "r"(rword), "r"((uint32_t)lo32(res_r2)), "n"(0x7650 | K));
-        y += hi32(mad_wide_u(u, res_m2, 0ll));
+        y += mul_denormal(u, res_m2);
     }
     return y;
 }
@@ -1674,10 +1674,11 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
             D.res_m2 = (uint32_t)m2;
             D.res_r2_lo = (uint32_t)((unsigned long long)r2 & 0xFFFFFFFFull);
             D.res_r2_hi = (uint32_t)((unsigned long long)r2 >> 32);
-            // the fast pass takes the term without the 64-bit addend when that form exists and its constant fits into
+            // the fast pass takes the term as a single-precision product when that exists and its constant fits into
             // every channel's rounding addend
-            uint32_t k8 = 0;
-            bool short_form = !cp.general && residual_short_form(L.res_mult, L.res_shift, L.zp_res, &k8, &res_c);
+            ResidualForm form;
+            if (!cp.general) form = residual_form(L.res_mult, L.res_shift, L.zp_res, &res_c);
+            bool short_form = form.exists();
             for (int oc = 0; oc < L.cout && short_form; ++oc) {
                 const int sft = ML.shift[oc] - 1;
                 const long long add = sft >= 1 ? (1ll << (sft - 1)) + ((long long)L.zp_out - res_c) * (1ll << sft) : (1ll << 40);
@@ -1685,7 +1686,8 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
             }
             if (short_form) {
                 D.flags |= CF_RSHORT;
-                D.res_r2_lo = k8;
+                D.res_m2 = form.m_bits;
+                D.res_r2_lo = form.k8;
                 D.res_r2_hi = 0;
             } else {
                 res_c = 0;

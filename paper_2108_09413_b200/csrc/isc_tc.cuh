@@ -145,6 +145,15 @@ __device__ __forceinline__ int lo32(long long v)
     asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "l"(v));
     return lo;
 }
+// hi32(a * b) + c in one instruction
+__device__ __forceinline__ int mad_hi(int a, int b, int c)
+{
+    int d;
+    asm("mad.hi.s32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+    return d;
+}
+// round-to-nearest(v * m) for an integer v < 2^23, as an integer: both are read as denormal numbers, whose unit is one
+__device__ __forceinline__ int mul_denormal(uint32_t v, uint32_t m_bits) { return __float_as_int(__fmul_rn(__uint_as_float(v), __uint_as_float(m_bits))); }
 __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1)
 {
 #pragma unroll
