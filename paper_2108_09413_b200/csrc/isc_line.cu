@@ -79,7 +79,7 @@ constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // 2 s per wait
 
 enum { PH_FILL = 0, PH_INPUT = 1, PH_CONV = 2, PH_TAIL = 3 };
 enum { ERR_NONE = 0, ERR_WAIT_DONE = 1, ERR_WAIT_WEIGHTS = 2, ERR_WAIT_READY = 3, ERR_WAIT_FULL = 4, ERR_WAIT_DRAIN = 5 };
-enum { CF_STACKED = 1, CF_RES = 2, CF_LO = 4, CF_SCATTER = 8, CF_GENERAL = 16, CF_RSHORT = 32 };     // CF_GENERAL: the pass that decides everything at run time; CF_RSHORT: residual term as a single-precision product
+enum { CF_RES = 2, CF_SCATTER = 8, CF_GENERAL = 16 };         // CF_GENERAL: the pass that decides everything at run time
 // OPF_WAIT_ALL: every unit of the previous convolution; OPF_WAITS / OPF_WAITS4: the record names counters to test (two /
 // four slots in use); bits 4-6: how many of them are distinct; bits 8-9: arrivals; bits 10-12: MMA chains
 enum { OPF_WAIT_ALL = 1, OPF_WAITS = 2, OPF_WAITS4 = 8 };
@@ -87,7 +87,7 @@ enum { OPF_WAIT_ALL = 1, OPF_WAITS = 2, OPF_WAITS4 = 8 };
 // ---- what the kernel reads -------------------------------------------------------------------
 
 // One entry per phase, copied to shared memory when the kernel starts.
-//   CONV: a = shared-memory offset of the blob      FILL: a = offset, b = bytes, c = halo byte
+//   CONV: a = shared-memory offset of the blob, b = convolutions that follow each other from here on      FILL: a = offset, b = bytes, c = halo byte
 struct alignas(16) PhaseEntry { uint32_t kind, a, b, c; };
 
 // Where the blob of convolution c comes from (global) and goes to (shared).
@@ -112,20 +112,20 @@ struct alignas(16) LOp {
 };
 static_assert(sizeof(LOp) == 32, "one operation is two 16-byte loads");
 
-// Head of every blob: everything the issuing thread and the epilogue need to know about the convolution.
+// Head of every blob: first what an epilogue warp reads, then what only some need.
 struct alignas(16) LConvDesc {
-    uint32_t n_ops, n_passes, n_ksteps, flags;
-    uint32_t a_base, pitch16, bblock16, n_banks;            // a_base: line -1, lane 0, plane 0 of the input
-    uint32_t idesc[3], cols;                                // instruction descriptors for 1, 2, 3 blocks; columns per line
-    uint32_t d_base[2], bar_full, bar_done;                 // accumulator bank bases; barrier indices of this class
-    uint32_t use_local, uses_per_group, n_lines, n_chunks;
-    uint32_t w_rel, c_rel, ops_rel, passes_rel;
-    // epilogue: where results go (line 0, lane 0, plane 0), geometry of the output and of the scattered input
-    uint32_t out_base, out_plane, out_pitch16, out_n_lines;
-    uint32_t out_log_lines, out_nb, out_logI, res_base;
-    uint32_t res_plane, in_logI, in_I, in_n_lines;
-    int32_t lo; uint32_t res_m2, res_r2_lo, res_r2_hi;
-    uint32_t b_lo0, kstep16, recs_per_item, pad1;       // low word of the first K-step's weight descriptor (shared-memory base 0); records per (unit, chunk)
+    uint32_t flags, n_items, recs_per_item, d_base;         // (unit, chunk) pairs; records of the pass table for each; first accumulator column
+    uint32_t bar_full, bar_done, use_local, uses_per_group;  // barrier indices of this class
+    uint32_t n_units, c_rel, passes_rel, out_base;          // units (their barriers); constants, pass table; output (line 0, lane 0, plane 0)
+    uint32_t res_base, res_m2, res_k8, dup_delta;           // residual operand and its term; bytes from a band's first row to its copy below the band above it, 0: one band
+    // geometry of the output and of the scattered input
+    uint32_t out_plane, out_pitch16, out_log_lines, out_logI;
+    uint32_t in_logI, in_n_lines, out_nb, vec_rel;           // vec_rel: start values for the accumulators' next use, 16 channels each
+    // the general pass
+    int32_t lo; uint32_t res_r2_lo, res_r2_hi, gen_res_m2;
+    // issuing threads
+    uint32_t n_ops, n_ksteps, ops_rel, n_chunks;
+    uint32_t b_lo0, kstep16, pitch16, cols;                  // b_lo0: low word of the first K-step's weight descriptor (shared-memory base 0)
     uint32_t a_lo[kMaxKsteps + 2];             // low words of the operand descriptors of line -1 (shared-memory base 0)
 };
 static_assert(sizeof(LConvDesc) % 16 == 0, "blob sections stay 16-byte aligned");
@@ -157,6 +157,7 @@ struct LineParams {
     int32_t *err;
     unsigned long long *phase_cycles; // [4]: SM cycles per CTA spent in FILL, INPUT, everything else, TAIL, summed over CTAs and launches
     // debug
+    const int32_t *acc_init;          // [kTmemCols]: the accumulators' values before the first group
     int32_t stop_phase;
     uint32_t dump_off, dump_bytes;
     uint8_t *dump;
@@ -177,22 +178,44 @@ struct Ctrl {
 static_assert(sizeof(Ctrl) <= kCtrlBytes - 16, "control block too large");
 
 // ------------------------------------------------------------------ device helpers
+//
+// Nothing on a convolution's path may use local memory: with 227 KB of shared memory per SM the first-level cache is too
+// small for 640 threads' stacks, and every spilled register or structure on the stack costs a trip to the second level
+// (a convolution's fixed cost per warp was 2,900 cycles so).  Hence the kernel makes no calls, and shared memory is addressed
+// through the array's constant address.
+extern __shared__ __align__(128) uint8_t smem[];
+__device__ __forceinline__ Ctrl *the_ctrl() { return reinterpret_cast<Ctrl *>(smem); }
+__device__ __forceinline__ uint32_t the_base() { return smem_u32(smem); }
+#define CTRL_ADDR(member) (the_base() + (uint32_t)offsetof(Ctrl, member))
 
-__device__ __forceinline__ void mma_i8(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate)
+// D += A * B: accumulators start from their channels' folded biases (see LPass)
+__device__ __forceinline__ void mma_i8(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc)
 {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.b32 p, 0, 0;\n\t"
                  "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
-                 ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
+                 ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc) : "memory");
 }
 __device__ __forceinline__ void commit_to(uint32_t bar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
-__device__ __forceinline__ void tmem_st16_zero(uint32_t taddr)
+// 16 columns of half a warp's tensor-memory lanes (16, from `taddr` on) in fragment form: a thread holds columns 2 c, 2 c + 1
+// (c = lane mod 4) of rows lane / 4 (v[0], v[1]) and lane / 4 + 8 (v[2], v[3]), then the same eight columns on (v[4..7]).
+__device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, int (&v)[8])
 {
-    const int z = 0;
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1};"
-                 ::"r"(taddr), "r"(z) : "memory");
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "r"(taddr) : "memory");
+}
+// every load issued so far is complete; names the registers so that no use can move above it
+__device__ __forceinline__ void tmem_ld_frag_wait(int (&v)[8])
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]) :: "memory");
+}
+// the same 16 columns of the 16 lanes take the value of their column; b: the values of this thread's four columns
+__device__ __forceinline__ void tmem_st_columns(uint32_t taddr, uint4 b)
+{
+    asm volatile("tcgen05.st.sync.aligned.16x256b.x2.b32 [%0], {%1,%2,%1,%2,%3,%4,%3,%4};" ::"r"(taddr), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w) : "memory");
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ long long mad_wide_u(uint32_t a, uint32_t b, long long c)
@@ -201,22 +224,23 @@ __device__ __forceinline__ long long mad_wide_u(uint32_t a, uint32_t b, long lon
     asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
     return d;
 }
-// Per-channel requantisation constants as stored in the blob (16 bytes): folded bias, multiplier, rounding addend
-// and shift.  With s = shift - 1 >= 1,
-//   rs((acc + bias) * mult, 31 + shift) + zp_out = (hi32((acc + bias) * mult) + c) >> s,   c = 2^(s-1) + zp_out * 2^s,
+// Per-channel requantisation constants of a thread's four channels 4 c .. 4 c + 3 of a chunk, as stored in the blob (48 bytes):
+// multipliers, rounding addends, shifts.  The accumulators start from the folded bias.  With s = shift - 1 >= 1,
+//   rs(acc * mult, 31 + shift) + zp_out = (hi32(acc * mult) + c) >> s,   c = 2^(s-1) + zp_out * 2^s,
 // exactly: the rounding half 2^(31+s) is a multiple of 2^32, so the low word of the product cannot change the floor.
 // For s = 0 the half sits in the low word: the result is hi32 + (bit 31 of the low word) + c with c = zp_out.
 // A scheduler issues a wide or high multiply in four cycles here, shifts, permutes and packs in two, additions in one: this
-// form is the cheapest exact one found (add, mad.hi, shift).
-struct ChanConst4 { int bias, mult, c, s; };
-// A plain load (the blob is complete in shared memory; the address derives from a value read after the wait for it)
-// that the compiler may schedule ahead of the tensor-memory wait.
-__device__ __forceinline__ ChanConst4 ld_chan_const_early(uint32_t addr)
+// form is the cheapest exact one found (mad.hi, shift; 5.1 cycles per output where add, wide multiply, add, shift take 6.8).
+struct ChanConsts { int mult[4], c[4], s[4]; };
+__device__ __forceinline__ ChanConsts ld_chan_consts(uint32_t addr)
 {
-    ChanConst4 c;
-    asm("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(c.bias), "=r"(c.mult), "=r"(c.c), "=r"(c.s) : "r"(addr));
-    return c;
+    ChanConsts k;
+    asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(k.mult[0]), "=r"(k.mult[1]), "=r"(k.mult[2]), "=r"(k.mult[3]) : "r"(addr));
+    asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(k.c[0]), "=r"(k.c[1]), "=r"(k.c[2]), "=r"(k.c[3]) : "r"(addr + 16u));
+    asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(k.s[0]), "=r"(k.s[1]), "=r"(k.s[2]), "=r"(k.s[3]) : "r"(addr + 32u));
+    return k;
 }
+constexpr uint32_t kChunkConstBytes = 4 * 48, kVecBytes = 64;
 __device__ __forceinline__ long long mul_wide(int a, int b)
 {
     long long d;
@@ -239,33 +263,23 @@ __device__ __forceinline__ uint32_t ld_acquire_u32(uint32_t addr)
     asm volatile("ld.acquire.cta.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
     return v;
 }
-// byte K of w, zero-extended
-template <int K>
-__device__ __forceinline__ uint32_t ubyte(uint32_t w)
-{
-    uint32_t d;
-    asm("prmt.b32 %0, %1, 0, %2;" : "=r"(d) : "r"(w), "n"(0x4440 | K));
-    return d;
-}
-
+// Bounded waits.  On expiry: the abort flag and the error word, wait kind | index of the barrier within the control block << 8 |
+// parity waited for << 20 | CTA << 21.
 struct Waiter {
-    Ctrl *ctrl;
     int32_t *err;
     unsigned long long limit_ns = kWaitLimitNs;
-    __device__ __forceinline__ bool aborted() const { return ctrl->abort_flag != 0; }
-    // the error word: wait kind | index of the barrier within the control block << 8 | parity waited for << 20 | CTA << 21
-    __device__ __noinline__ void fail(int code, uint32_t bar, uint32_t parity)
+    static __device__ __forceinline__ bool aborted() { return ld_volatile_u32(CTRL_ADDR(abort_flag)) != 0u; }
+    __device__ __forceinline__ void fail(int code, uint32_t bar, uint32_t parity) const
     {
-        ctrl->abort_flag = 1;
-        const uint32_t idx = (bar - smem_u32(ctrl)) >> 3;
+        the_ctrl()->abort_flag = 1;
+        const uint32_t idx = (bar - the_base()) >> 3;
         atomicCAS(err, 0, (int)((uint32_t)code | ((idx & 0xFFFu) << 8) | ((parity & 1u) << 20) | (blockIdx.x << 21)));
     }
     // Wait for a phase of an mbarrier.  Each attempt parks the thread in hardware for a bounded time,
-    // so a waiting warp does not compete for issue slots.
-    __device__ __forceinline__ bool barrier(uint32_t bar, uint32_t parity, int code)
+    // so a waiting warp does not compete for issue slots; the clock is read only when the first gives up.
+    __device__ __forceinline__ bool barrier(uint32_t bar, uint32_t parity, int code) const
     {
-        if (mbar_test(bar, parity)) return true;
-        if (mbar_try(bar, parity)) return true;         // parks the thread; the clock is read only when this gives up
+        if (mbar_try(bar, parity)) return true;
         const unsigned long long t0 = globaltimer();
         for (int spin = 0;; ++spin) {
             if (mbar_try(bar, parity)) return true;
@@ -276,12 +290,8 @@ struct Waiter {
         }
     }
     // Wait until a counter in shared memory has reached `expected` (counters only grow).
-    __device__ __forceinline__ bool counter(uint32_t addr, uint32_t expected, int code)
+    __device__ __forceinline__ bool counter(uint32_t addr, uint32_t expected, int code) const
     {
-        // The first test is a plain load: an acquiring one costs over a hundred cycles here.  What the counter guards
-        // was made visible to the tensor cores' reads by the storing warp (proxy fence, then a releasing add) and is
-        // read by MMAs that are issued only after the value has been seen.
-        if ((int32_t)(ld_volatile_u32(addr) - expected) >= 0) return true;
         const unsigned long long t0 = globaltimer();
         for (int spin = 0;; ++spin) {
             if ((int32_t)(ld_acquire_u32(addr) - expected) >= 0) return true;
@@ -297,39 +307,28 @@ struct Waiter {
 
 struct PrevConv { uint32_t done_addr, expected, n_lines; };    // counters of its units, their value when stored; n_lines = 0: nothing to wait for
 
-struct IssueCtx {
-    uint32_t desc, ops, n_ops, s16, b_lo0, kstep16, d0, stacked, full_addr, cg, issuer, pitch16, cols;
+// The barrier of the next blob: three, used in turn.
+struct WeightSlot {
+    uint32_t slot = 0, parity = 0;
+    __device__ __forceinline__ void advance() { if (++slot == 3u) { slot = 0; parity ^= 1u; } }
 };
 
-// The first, cheap read of a "stored" counter by an issuing thread.  A plain load by default: an acquiring one costs
-// over a hundred cycles per test on the issue path.  What the counter guards was published by the storing warp with a
-// proxy fence and a releasing add; the MMAs that read it are issued after the value was seen (control dependency)
-// and after tcgen05.fence::after_thread_sync.  Building with -DISC_ACQUIRE_POLL takes the acquiring form instead, so
-// that a divergence could be traced to this choice.
+struct IssueCtx {
+    uint32_t desc, ops, n_ops, s16, b_lo0, kstep16, d0, full_addr, issuer, pitch16, cols;
+};
+
+// How an issuing thread polls a "stored" counter.  A volatile load by default (a weak one could be moved out of the loop): an
+// acquiring one costs over a hundred cycles per test on the issue path.  What the counter guards was published by the
+// storing warp with a proxy fence and a releasing add; the MMAs that read it are issued after the value was seen (control
+// dependency) and after tcgen05.fence::after_thread_sync.  Building with -DISC_ACQUIRE_POLL takes the acquiring form
+// instead, so that a divergence could be traced to this choice.
 __device__ __forceinline__ uint32_t ld_counter(uint32_t addr)
 {
 #ifdef ISC_ACQUIRE_POLL
     return ld_acquire_u32(addr);
 #else
-    return lds32(addr);
+    return ld_volatile_u32(addr);
 #endif
-}
-
-// The dependency test of an operation when its first, cheap form did not pass (or the operation waits for the whole
-// previous convolution): bounded waits on every counter the record names.  Kept out of line: the issue loop is
-// latency-bound, every instruction on its path counts.
-__device__ __noinline__ bool wait_units_slow(Waiter w, const PrevConv &prev, uint4 r1)
-{
-    const uint32_t fl = r1.w >> 16;
-    if (fl & OPF_WAIT_ALL)
-        for (uint32_t l = 0; l < prev.n_lines; ++l)
-            if (!w.counter(prev.done_addr + 4 * l, prev.expected, ERR_WAIT_DONE)) return false;
-    const uint32_t nw = (fl >> 4) & 7u;
-    const uint32_t off[4] = {r1.x & 0xFFFFu, r1.x >> 16, r1.y & 0xFFFFu, r1.y >> 16};
-#pragma unroll
-    for (uint32_t k = 0; k < 4; ++k)
-        if (k < nw && !w.counter(prev.done_addr + off[k], prev.expected, ERR_WAIT_DONE)) return false;
-    return true;
 }
 
 // The operations of one convolution that belong to one issuing thread (every kIssuers-th record).  The low words of
@@ -357,7 +356,6 @@ __device__ __forceinline__ bool issue_ops(Waiter w, const IssueCtx &ic, const Pr
     }
     uint32_t at = ic.ops + 32u * ic.issuer;           // the table ends with kIssuers spare records: reads run one ahead
     uint4 n0 = ld_shared_v4(at), n1 = ld_shared_v4(at + 16);
-    const uint32_t acc_first = ic.stacked;
     for (uint32_t i = ic.issuer; i < ic.n_ops; i += kIssuers) {
         const uint4 r0 = n0, r1 = n1;         // d_col, idesc, a_add, b_add | wait 0-1, wait 2-3, commit 0-1, commit 2 and flags
         at += 32u * kIssuers;
@@ -365,15 +363,25 @@ __device__ __forceinline__ bool issue_ops(Waiter w, const IssueCtx &ic, const Pr
         const uint32_t fl = r1.w >> 16;
         // units of the previous convolution this operation depends on
         if (fl & (OPF_WAIT_ALL | OPF_WAITS)) {
-            int32_t m = -1;
-            if (!(fl & OPF_WAIT_ALL)) {
-                m = min((int32_t)(ld_counter(prev.done_addr + (r1.x & 0xFFFFu)) - prev.expected),
-                        (int32_t)(ld_counter(prev.done_addr + (r1.x >> 16)) - prev.expected));
-                if (fl & OPF_WAITS4)
-                    m = min(m, min((int32_t)(ld_counter(prev.done_addr + (r1.y & 0xFFFFu)) - prev.expected),
-                                   (int32_t)(ld_counter(prev.done_addr + (r1.y >> 16)) - prev.expected)));
+            if (fl & OPF_WAIT_ALL) {
+                for (uint32_t l = 0; l < prev.n_lines; ++l)
+                    if (!w.counter(prev.done_addr + 4 * l, prev.expected, ERR_WAIT_DONE)) return false;
             }
-            if (m < 0 && !wait_units_slow(w, prev, r1)) return false;
+            if (fl & OPF_WAITS) {
+                const unsigned long long t0 = globaltimer();
+                for (int spin = 0;; ++spin) {
+                    int32_t m = min((int32_t)(ld_counter(prev.done_addr + (r1.x & 0xFFFFu)) - prev.expected),
+                                    (int32_t)(ld_counter(prev.done_addr + (r1.x >> 16)) - prev.expected));
+                    if (fl & OPF_WAITS4)
+                        m = min(m, min((int32_t)(ld_counter(prev.done_addr + (r1.y & 0xFFFFu)) - prev.expected),
+                                       (int32_t)(ld_counter(prev.done_addr + (r1.y >> 16)) - prev.expected)));
+                    if (m >= 0) break;
+                    if ((spin & 63) == 63) {
+                        if (Waiter::aborted()) return false;
+                        if (globaltimer() - t0 > w.limit_ns) { w.fail(ERR_WAIT_DONE, prev.done_addr + (r1.x & 0xFFFFu), 0); return false; }
+                    }
+                }
+            }
         }
         tc_fence_after();
         if (KS == 2) {
@@ -383,7 +391,7 @@ __device__ __forceinline__ bool issue_ops(Waiter w, const IssueCtx &ic, const Pr
             auto chain = [&]() {
 #pragma unroll
                 for (int k = 0; k < NK; ++k)
-                    mma_i8(d, ((uint64_t)ahi << 32) | (uint64_t)(alo[k] + a_add), ((uint64_t)bhi << 32) | (uint64_t)(blo[k] + r0.w), r0.y, k > 0 ? 1u : acc_first);
+                    mma_i8(d, ((uint64_t)ahi << 32) | (uint64_t)(alo[k] + a_add), ((uint64_t)bhi << 32) | (uint64_t)(blo[k] + r0.w), r0.y);
                 d += ic.cols;
                 a_add += ic.pitch16;
             };
@@ -399,13 +407,12 @@ __device__ __forceinline__ bool issue_ops(Waiter w, const IssueCtx &ic, const Pr
             const uint32_t d = ic.d0 + r0.x;
 #pragma unroll
             for (int k = 0; k < NK; ++k)
-                mma_i8(d, ((uint64_t)ahi << 32) | (uint64_t)(alo[k] + r0.z), ((uint64_t)bhi << 32) | (uint64_t)(blo[k] + r0.w), r0.y, k > 0 ? 1u : acc_first);
+                mma_i8(d, ((uint64_t)ahi << 32) | (uint64_t)(alo[k] + r0.z), ((uint64_t)bhi << 32) | (uint64_t)(blo[k] + r0.w), r0.y);
         } else {
             const uint32_t d = ic.d0 + r0.x;
             for (uint32_t k = 0; k < n_ksteps; ++k) {
                 const uint32_t a_lo = lds32(ic.desc + offsetof(LConvDesc, a_lo) + 4 * k) + ic.s16;
-                mma_i8(d, ((uint64_t)ahi << 32) | (uint64_t)(a_lo + r0.z), ((uint64_t)bhi << 32) | (uint64_t)(ic.b_lo0 + ic.s16 + k * ic.kstep16 + r0.w), r0.y,
-                       k > 0 ? 1u : acc_first);
+                mma_i8(d, ((uint64_t)ahi << 32) | (uint64_t)(a_lo + r0.z), ((uint64_t)bhi << 32) | (uint64_t)(ic.b_lo0 + ic.s16 + k * ic.kstep16 + r0.w), r0.y);
             }
         }
         const uint32_t nc = (fl >> 8) & 3u;
@@ -431,89 +438,69 @@ __device__ __forceinline__ void issue_weights(const ConvSrc *src, uint32_t sbase
 
 // The copy of convolution `target`'s blob, by lane 0 of the loader warp, once the convolution it names is complete:
 // the blob takes the place of things that convolution (or an earlier one) was the last to use.
-__device__ __noinline__ bool loader_copy(const LineParams &p, Ctrl *ctrl, uint32_t sbase, int target, uint32_t cg_target, int it)
+__device__ __forceinline__ bool loader_copy(const LineParams &p, int target, uint32_t wslot, int it)
 {
-    Waiter w{ctrl, p.err};
-    const ConvSrc *src = ctrl->csrc + target;
+    const Waiter w{p.err};
+    const ConvSrc *src = the_ctrl()->csrc + target;
     if ((int)(src->bytes_phase >> 24) > p.stop_phase) return true;
     const uint32_t n = src->dep_units;
     if (n) {
         const uint32_t expected = src->dep_mult * ((uint32_t)it * (src->dep_local_uses >> 16) + (src->dep_local_uses & 0xFFFFu) + 1u);
-        const uint32_t first = smem_u32(&ctrl->stored[src->dep_first]);
+        const uint32_t first = CTRL_ADDR(stored) + 4u * src->dep_first;
         for (uint32_t l = 0; l < n; ++l)
             if (!w.counter(first + 4 * l, expected, ERR_WAIT_DONE)) return false;
     }
-    issue_weights(src, sbase, smem_u32(&ctrl->wbar[cg_target % 3]));
+    issue_weights(src, the_base(), CTRL_ADDR(wbar) + 8u * wslot);
     return true;
 }
 
 // One convolution's share of an issuing warp, by its lane 0.  Returns false after a wait has expired.
-__device__ __noinline__ bool issuer_conv(const LineParams &p, Ctrl *ctrl, uint32_t sbase, uint32_t tmem, uint32_t blob_off,
-                                         uint32_t cg, int issuer, int it, PrevConv &prev)
+__device__ __forceinline__ bool issuer_conv(const LineParams &p, uint32_t tmem, uint32_t blob_off, WeightSlot ws, uint32_t issuer, int it, PrevConv &prev)
 {
-    Waiter w{ctrl, p.err};
-    if (!w.barrier(smem_u32(&ctrl->wbar[cg % 3]), (cg / 3) & 1, ERR_WAIT_WEIGHTS)) return false;
-    const uint32_t desc = sbase + blob_off;
-    const uint4 h0 = ld_shared_v4(desc);                                    // n_ops, n_passes, n_ksteps, flags
-    const uint4 h1 = ld_shared_v4(desc + offsetof(LConvDesc, a_base));      // a_base, pitch16, bblock16, n_banks
-    const uint4 h3 = ld_shared_v4(desc + offsetof(LConvDesc, d_base));      // d_base[2], bar_full, bar_done
-    const uint4 h4 = ld_shared_v4(desc + offsetof(LConvDesc, use_local));   // use_local, uses_per_group, n_lines, n_chunks
-    const uint4 h5 = ld_shared_v4(desc + offsetof(LConvDesc, w_rel));       // w_rel, c_rel, ops_rel, passes_rel
-    const uint4 hb = ld_shared_v4(desc + offsetof(LConvDesc, b_lo0));       // b_lo0, kstep16
-    const uint32_t use = (uint32_t)it * h4.y + h4.x;
+    const Waiter w{p.err};
+    if (!w.barrier(CTRL_ADDR(wbar) + 8u * ws.slot, ws.parity, ERR_WAIT_WEIGHTS)) return false;
+    const uint32_t desc = the_base() + blob_off;
+    const uint4 h0 = ld_shared_v4(desc);                                    // flags, n_items, recs_per_item, d_base
+    const uint4 h1 = ld_shared_v4(desc + offsetof(LConvDesc, bar_full));    // bar_full, bar_done, use_local, uses_per_group
+    const uint4 h2 = ld_shared_v4(desc + offsetof(LConvDesc, n_ops));       // n_ops, n_ksteps, ops_rel, n_chunks
+    const uint4 h3 = ld_shared_v4(desc + offsetof(LConvDesc, b_lo0));       // b_lo0, kstep16, pitch16, cols
+    const uint32_t n_units = lds32(desc + offsetof(LConvDesc, n_units));
+    const uint32_t use = (uint32_t)it * h1.w + h1.z;
     IssueCtx ic;
-    ic.desc = desc; ic.ops = desc + h5.z; ic.n_ops = h0.x;
-    ic.s16 = sbase >> 4; ic.b_lo0 = hb.x; ic.kstep16 = hb.y;
-    ic.d0 = tmem + ((h1.w > 1 && (use & 1u)) ? h3.y : h3.x);
-    ic.stacked = (h0.w & CF_STACKED) ? 1u : 0u;
-    ic.full_addr = smem_u32(&ctrl->bars[h3.z + (use & 1u) * h4.z]);      // the class has two sets of barriers, used in turn
-    ic.cg = cg;
-    ic.issuer = (uint32_t)issuer;
-    ic.pitch16 = h1.y;
-    ic.cols = lds32(desc + offsetof(LConvDesc, cols));
+    ic.desc = desc; ic.ops = desc + h2.z; ic.n_ops = h2.x;
+    ic.s16 = the_base() >> 4; ic.b_lo0 = h3.x; ic.kstep16 = h3.y;
+    ic.d0 = tmem + h0.w;
+    ic.full_addr = CTRL_ADDR(bars) + 8u * (h1.x + (use & 1u) * n_units);      // the class has two sets of barriers, used in turn
+    ic.issuer = issuer;
+    ic.pitch16 = h3.z;
+    ic.cols = h3.w;
     bool ok;
-    switch (h0.z) {
+    switch (h2.y) {
     case 1: ok = issue_ops<1>(w, ic, prev, 1); break;
     case 2: ok = issue_ops<2>(w, ic, prev, 2); break;
     case 3: ok = issue_ops<3>(w, ic, prev, 3); break;
     case 5: ok = issue_ops<5>(w, ic, prev, 5); break;
+    case 6: ok = issue_ops<6>(w, ic, prev, 6); break;
     case 9: ok = issue_ops<9>(w, ic, prev, 9); break;
-    case 18: ok = issue_ops<18>(w, ic, prev, 18); break;
-    default: ok = issue_ops<0>(w, ic, prev, h0.z); break;
+    default: ok = issue_ops<0>(w, ic, prev, h2.y); break;
     }
     if (!ok) return false;
-    prev.done_addr = smem_u32(&ctrl->stored[h3.w]);
-    prev.expected = 4u * h4.w * (use + 1u);
-    prev.n_lines = h4.z;
+    prev.done_addr = CTRL_ADDR(stored) + 4u * h1.y;
+    prev.expected = 4u * h2.w * (use + 1u);
+    prev.n_lines = n_units;
     return true;
 }
 
 // ------------------------------------------------------------------ epilogue warps
 
-struct EpiCtx {
-    Ctrl *ctrl;
-    uint32_t sbase, tmem_lane;          // tensor-memory address of this warp's 32 lanes, column 0
-    int warp, set, quarter, lane, tid;
-    uint32_t lane_idx;                  // position within a line: quarter * 32 + lane
-};
-
-// What an epilogue warp keeps in registers for the whole of a convolution: addresses already specialised to the
-// thread (its position within a line, its 32 lanes of tensor memory), so that a pass only adds the offsets of its
-// table record.  The geometry that only strided convolutions need stays in the blob's header.
-struct EpiConv {
-    uint32_t tmem0;                       // tensor-memory address of this warp's lanes, first column of the bank
-    uint32_t full_addr, done_addr, parity;
-    uint32_t const_addr;
-    uint32_t out_thread, res_thread;      // line 0, this thread's position, plane 0 of the output / residual
-    uint32_t dup_delta;                   // bytes from a band's first row to its copy below the band above; 0: one band
-    uint32_t dup_up, dup_dn;              // this thread's band has a band above / below
-    uint32_t res_m2;
-    long long res_r2;
-};
-
-// One pass of the table: lines (a unit), chunk, and the offsets they imply.
+// A thread works on four positions of a line (rows quarter * 32 + lane / 4 + 8 i) and the four channels 4 c .. 4 c + 3 of a chunk
+// (c = lane mod 4), one word: constants stay in registers for a whole convolution, and eight positions x 16 bytes make one
+// conflict-free store.  (The columns of the weights are ordered so that a thread's accumulator columns are these channels.)
+// One record of the pass table: one or two lines of a unit and a chunk.
 struct alignas(16) LPass {
-    uint32_t meta;          // unit | lines << 8 | chunk << 12 | line 0 first / last row of its band << 16, 17 | line 1 << 18, 19
+    // unit | lines << 8 | chunk << 12 | line 0 first / last row of its band << 16, 17 | line 1 << 18, 19 | start values of line 0, 1 << 20, 26:
+    // the accumulators read take the folded biases of the channels that the next convolution on these columns puts there
+    uint32_t meta;
     uint32_t lines;         // line 0 | line 1 << 8
     uint32_t tcol[2];       // accumulator columns of the two lines' chunk within the bank
     uint32_t out[2];        // byte offset of the two lines' chunk (line within its plane + plane) in the output
@@ -521,241 +508,219 @@ struct alignas(16) LPass {
 };
 static_assert(sizeof(LPass) == 32, "one pass is two 16-byte loads");
 
-// One output of the common pass (every channel has s >= 1).
-//   residual: y += floor((u * m2 + R2) / 2^32) with u = r + 128 the residual byte as an unsigned number,
-//   m2 = res_mult * 2^(32-n) and R2 the rounding half and the zero-points folded: rs((r - zp_res) * res_mult, n).
-//   kRes = 2: the same term as a single-precision product round((256 k + u) * m) - c_r, for an offset k and a multiplier m
-//   that the planner has checked on all 256 values of u (residual_form): `res_r2` then holds 256 k, which the byte
-//   permute that extracts u merges into it, `res_m2` m's bits, and c_r is folded into the channel's rounding addend.
-template <int kRes, int K>
-__device__ __forceinline__ int requant1(int acc, const ChanConst4 &cs, uint32_t rword, uint32_t res_m2, long long res_r2)
+// Four outputs of one position.
+//   kResidual: y += round((256 k + u) * m) - c_r with u = r + 128 the residual byte as an unsigned number, for an offset k
+//   and a multiplier m that the planner has checked on all 256 values of u (residual_form): rs((r - zp_res) * res_mult, n).
+//   `k8` holds 256 k, which the byte permute that extracts u merges into it; c_r is folded into the rounding addends.
+template <bool kResidual>
+__device__ __forceinline__ uint32_t requant4(int a0, int a1, int a2, int a3, const ChanConsts &k, uint32_t rword, uint32_t m2, uint32_t k8)
 {
-    int y = mad_hi(acc + cs.bias, cs.mult, cs.c) >> cs.s;
-    if (kRes == 1) y += hi32(mad_wide_u(ubyte<K>(rword), res_m2, res_r2));
-    if (kRes == 2) {
-        uint32_t u;
-        asm("prmt.b32 %0, %1, %2, %3;" : "=r"(u) : "r"(rword), "r"((uint32_t)lo32(res_r2)), "n"(0x7650 | K));
-        y += mul_denormal(u, res_m2);
+    int y0 = mad_hi(a0, k.mult[0], k.c[0]) >> k.s[0], y1 = mad_hi(a1, k.mult[1], k.c[1]) >> k.s[1];
+    int y2 = mad_hi(a2, k.mult[2], k.c[2]) >> k.s[2], y3 = mad_hi(a3, k.mult[3], k.c[3]) >> k.s[3];
+    if (kResidual) {
+        y0 += mul_denormal(__byte_perm(rword, k8, 0x7650u), m2);
+        y1 += mul_denormal(__byte_perm(rword, k8, 0x7651u), m2);
+        y2 += mul_denormal(__byte_perm(rword, k8, 0x7652u), m2);
+        y3 += mul_denormal(__byte_perm(rword, k8, 0x7653u), m2);
     }
-    return y;
+    return pack4_sat(y0, y1, y2, y3);
 }
 
-__device__ __forceinline__ void st_shared_v4_if(uint32_t addr, uint4 v, uint32_t flag)
+__device__ __forceinline__ void st_shared_u32(uint32_t addr, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
+__device__ __forceinline__ void st_shared_u32_if(uint32_t addr, uint32_t v, uint32_t flag)
 {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %5, 0;\n\t@p st.shared.v4.u32 [%0], {%1,%2,%3,%4};\n\t}"
-                 ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(flag) : "memory");
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p st.shared.u32 [%0], %1;\n\t}" ::"r"(addr), "r"(v), "r"(flag) : "memory");
 }
 
-// The wait of a pass for its unit's accumulators.  The first attempt parks the thread in hardware for a bounded
-// time and nearly always succeeds; the timed loop is kept out of line so that the pass body stays small.
-__device__ __noinline__ bool wait_full_slow(Waiter w, uint32_t bar, uint32_t parity) { return w.barrier(bar, parity, ERR_WAIT_FULL); }
-
-__device__ __forceinline__ bool wait_full(Waiter w, uint32_t bar, uint32_t parity)
-{
-    bool ok = mbar_try(bar, parity);
-    if (!ok) ok = wait_full_slow(w, bar, parity);
-    return __all_sync(0xffffffffu, ok);
-}
-
-// After a pass: the stores become visible to the tensor cores' reads, the tensor-memory accesses are ordered
+// After an item: the stores become visible to the tensor cores' reads, the tensor-memory accesses are ordered
 // before the arrival, and the warp counts one stored chunk of the unit.
-__device__ __forceinline__ void pass_done(const EpiConv &E, const EpiCtx &c, uint32_t unit)
+__device__ __forceinline__ void pass_done(uint32_t counter, int lane)
 {
+    tmem_st_wait();
     tc_fence_before();
     fence_proxy_async();
     __syncwarp();
-    if (c.lane == 0) red_release_add(E.done_addr + 4u * unit, 1u);
+    if (lane == 0) red_release_add(counter, 1u);
 }
 
-// The common pass: two output lines, one 16-channel chunk, results stored where the next convolution reads them.
-// The accumulator columns are left at zero: stacked chains accumulate from their first K-step on.
-template <int kRes>
-__device__ __forceinline__ void epi_pass2(const EpiConv &E, const EpiCtx &c, uint4 q0, uint4 q1)
+// Stride 2: where position `pos` of even input line number `line` goes (even columns survive, and every row of an even line
+// is an even row), relative to the output's line 0, lane 0, plane 0, with its line and band.
+struct Scatter { uint32_t log_i, half_lines, log_lines, log_o, pitch; };
+__device__ __forceinline__ uint32_t scatter_to(const Scatter &g, uint32_t pos, uint32_t line, uint32_t &oline, uint32_t &oband)
 {
-    const uint32_t ch = (q0.x >> 12) & 0xFu;
-    tc_fence_after();
-    int acc0[16], acc1[16];
-    tmem_ld16_issue(E.tmem0 + q0.z, acc0);
-    tmem_ld16_issue(E.tmem0 + q0.w, acc1);
-    uint32_t r0[4] = {0, 0, 0, 0}, r1[4] = {0, 0, 0, 0};
-    if (kRes) {
-        const uint4 a = ld_shared_v4(E.res_thread + q1.z), b = ld_shared_v4(E.res_thread + q1.w);
-        r0[0] = a.x ^ 0x80808080u; r0[1] = a.y ^ 0x80808080u; r0[2] = a.z ^ 0x80808080u; r0[3] = a.w ^ 0x80808080u;
-        r1[0] = b.x ^ 0x80808080u; r1[1] = b.y ^ 0x80808080u; r1[2] = b.z ^ 0x80808080u; r1[3] = b.w ^ 0x80808080u;
-    }
-    tmem_ld_wait();
-    tmem_st16_zero(E.tmem0 + q0.z);
-    tmem_st16_zero(E.tmem0 + q0.w);
-    const uint32_t cbase = E.const_addr + ch * 256u;
-    const uint32_t m2 = E.res_m2;
-    const long long r2 = E.res_r2;
-    uint32_t o0[4], o1[4];
-#pragma unroll
-    for (int g = 0; g < 4; ++g) {
-        const ChanConst4 c0 = ld_chan_const_early(cbase + (4 * g + 0) * 16), c1 = ld_chan_const_early(cbase + (4 * g + 1) * 16);
-        const ChanConst4 c2 = ld_chan_const_early(cbase + (4 * g + 2) * 16), c3 = ld_chan_const_early(cbase + (4 * g + 3) * 16);
-        o0[g] = pack4_sat(requant1<kRes, 0>(acc0[4 * g + 0], c0, r0[g], m2, r2), requant1<kRes, 1>(acc0[4 * g + 1], c1, r0[g], m2, r2),
-                          requant1<kRes, 2>(acc0[4 * g + 2], c2, r0[g], m2, r2), requant1<kRes, 3>(acc0[4 * g + 3], c3, r0[g], m2, r2));
-        o1[g] = pack4_sat(requant1<kRes, 0>(acc1[4 * g + 0], c0, r1[g], m2, r2), requant1<kRes, 1>(acc1[4 * g + 1], c1, r1[g], m2, r2),
-                          requant1<kRes, 2>(acc1[4 * g + 2], c2, r1[g], m2, r2), requant1<kRes, 3>(acc1[4 * g + 3], c3, r1[g], m2, r2));
-    }
-    const uint4 v0 = make_uint4(o0[0], o0[1], o0[2], o0[3]), v1 = make_uint4(o1[0], o1[1], o1[2], o1[3]);
-    const uint32_t a0 = E.out_thread + q1.x, a1 = E.out_thread + q1.y;
-    st_shared_v4(a0, v0);
-    st_shared_v4(a1, v1);
-    if (E.dup_delta) {
-        // first row of a lower band: also the row below the band above it; last row of an upper band: the row above
-        // the next band
-        st_shared_v4_if(a0 + E.dup_delta, v0, (q0.x >> 16) & E.dup_up);
-        st_shared_v4_if(a0 - E.dup_delta, v0, (q0.x >> 17) & E.dup_dn);
-        st_shared_v4_if(a1 + E.dup_delta, v1, (q0.x >> 18) & E.dup_up);
-        st_shared_v4_if(a1 - E.dup_delta, v1, (q0.x >> 19) & E.dup_dn);
-    }
+    const uint32_t x = pos >> g.log_i, band = (pos & ((1u << g.log_i) - 1u)) >> 2, row = line + band * g.half_lines;
+    oline = row & ((1u << g.log_lines) - 1u);
+    oband = row >> g.log_lines;
+    return (oline * g.pitch + ((x >> 1) << g.log_o) + (oband << 2) + (pos & 3u)) * 16u;
 }
 
-// The items (unit, chunk) of a convolution that belong to this warp's set: one wait, one or two records of two lines
-// each, one arrival.
-template <int kRes>
-__device__ __forceinline__ void epi_conv_fast(Waiter w, const EpiConv &E_in, const EpiCtx &c_in, uint32_t passes, uint32_t n_items,
-                                            uint32_t item_bytes)
+// The items (unit, chunk) of a convolution that belong to this warp's set: one wait, one or two records of two lines each,
+// one arrival.  kScatter: stride 2, results go to the next geometry (2.1 instead of 4.0 us a convolution of the first
+// transition when that was a pass of run-time decisions, line by line).
+template <bool kResidual, bool kScatter>
+__device__ __forceinline__ bool epi_conv_fast(Waiter w, uint32_t tmem_lane, uint32_t warp, uint32_t lane, uint32_t desc, uint4 h0, uint4 h1, uint4 h2, uint4 h3, uint32_t use)
 {
-    const EpiConv E = E_in;
-    const EpiCtx c = c_in;
+    const uint32_t tmem0 = tmem_lane + h0.w, full = CTRL_ADDR(bars) + 8u * (h1.x + (use & 1u) * h2.x), done = CTRL_ADDR(stored) + 4u * h1.y;
+    const uint32_t parity = (use >> 1) & 1u, word = lane & 3u, row0 = (warp & 3u) * 32u + (lane >> 2);
+    const uint32_t out = the_base() + h2.w + (kScatter ? word * 4u : row0 * 16u + word * 4u), res = the_base() + h3.x + row0 * 16u + word * 4u;
+    const uint32_t vecs = desc + lds32(desc + offsetof(LConvDesc, vec_rel)) + word * 16u;
+    const uint32_t m2 = h3.y, k8 = h3.z, dup = h3.w;
+    // The bands of a thread's rows: they differ in bits 3 and 4 of the position, of which a band number has bits 2 and 3 at
+    // most.  Bit 0, 1: rows of even number have a band above, below; bit 2, 3: those of odd number.
+    const uint32_t nb = lds32(desc + offsetof(LConvDesc, out_nb));
+    uint32_t bands = 0;
+    if (!kScatter) {
+        const uint32_t a = (row0 >> 2) & (nb - 1u), b = ((row0 >> 2) + 2u) & (nb - 1u);
+        bands = (a >= 1u ? 1u : 0u) | (a + 1u < nb ? 2u : 0u) | (b >= 1u ? 4u : 0u) | (b + 1u < nb ? 8u : 0u);
+    }
+    Scatter g;
+    if (kScatter) {
+        const uint4 g0 = ld_shared_v4(desc + offsetof(LConvDesc, out_plane)), g1 = ld_shared_v4(desc + offsetof(LConvDesc, in_logI));
+        g.pitch = g0.y; g.log_lines = g0.z; g.log_o = g0.w; g.log_i = g1.x; g.half_lines = g1.y >> 1;
+    }
+    const uint32_t rec_bytes = 32u * h0.z, rec_stop = desc + h2.z + rec_bytes * h0.y;
 #pragma unroll 1
-    for (uint32_t i = (uint32_t)c.set; i < n_items; i += kSets) {
-        const uint32_t rec = passes + item_bytes * i;
-        const uint4 q0 = ld_shared_v4(rec), q1 = ld_shared_v4(rec + 16u);
-        if (!wait_full(w, E.full_addr + 8u * (q0.x & 0xFFu), E.parity)) return;     // aborted: every other wait falls through too
-        epi_pass2<kRes>(E, c, q0, q1);
-        if (item_bytes > 32u) {
-            const uint4 p0 = ld_shared_v4(rec + 32u), p1 = ld_shared_v4(rec + 48u);
-            epi_pass2<kRes>(E, c, p0, p1);
-        }
-        tmem_st_wait();
-        pass_done(E, c, q0.x & 0xFFu);
-    }
-}
-
-// Stride 2: stores one position's 16 channels of a plane where the output's layout wants them (`line` is the ordinal
-// of an even input line; even columns and even rows survive), with the copies that the line layout asks for.
-__device__ __noinline__ void store_strided(uint32_t desc, uint32_t sbase, uint32_t lane_idx, uint32_t ch, uint32_t line, uint4 o)
-{
-    const uint4 h6 = ld_shared_v4(desc + offsetof(LConvDesc, out_base));       // out_base, out_plane, out_pitch16, out_n_lines
-    const uint4 h7 = ld_shared_v4(desc + offsetof(LConvDesc, out_log_lines));  // out_log_lines, out_nb, out_logI, res_base
-    const uint4 h8 = ld_shared_v4(desc + offsetof(LConvDesc, res_plane));      // res_plane, in_logI, in_I, in_n_lines
-    const uint32_t x_i = lane_idx >> h8.y, band_i = (lane_idx & (h8.z - 1u)) >> 2, s = lane_idx & 3u;
-    const uint32_t r_i = 2u * line + band_i * h8.w;
-    if ((x_i & 1u) || (r_i & 1u)) return;
-    const uint32_t r_o = r_i >> 1, x_o = x_i >> 1;
-    const uint32_t oline = r_o & (h6.w - 1u);
-    const uint32_t olane = (x_o << h7.z) + ((r_o >> h7.x) << 2) + s;
-    const uint32_t addr = sbase + h6.x + ch * h6.y + (oline * h6.z + olane) * 16u;
-    st_shared_v4(addr, o);
-    const uint32_t band = (olane >> 2) & (h7.y - 1u);
-    // first row of a lower band: also the row below the band above it; last row of an upper band: the row above the next
-    if (oline == 0 && band >= 1) st_shared_v4(addr + (h6.w * h6.z - 4u) * 16u, o);
-    if (oline == h6.w - 1u && band + 1u < h7.y) st_shared_v4(addr - (h6.w * h6.z - 4u) * 16u, o);
-}
-
-// The general pass (strided convolutions, a lower clamp above -128, a lone line): one line at a time, every
-// property decided at run time.  A CIFAR ResNet reaches it in the four convolutions of its two stage transitions (the
-// stride-2 3 x 3 and the 1 x 1 shortcut).
-__device__ __noinline__ void epi_conv_general(Waiter w, const EpiConv &E, const EpiCtx &c, uint32_t desc, uint32_t flags, int32_t lo,
-                                              uint32_t passes, uint32_t n_passes)
-{
-    const bool res = flags & CF_RES, scatter = flags & CF_SCATTER;
-    for (uint32_t i = (uint32_t)c.set; i < n_passes; i += kSets) {
-        const uint4 q0 = ld_shared_v4(passes + 32u * i), q1 = ld_shared_v4(passes + 32u * i + 16u);
-        const uint32_t unit = q0.x & 0xFFu, ch = (q0.x >> 12) & 0xFu, n = (q0.x >> 8) & 0xFu;
-        if (!wait_full(w, E.full_addr + 8u * unit, E.parity)) return;
+    for (uint32_t rec = desc + h2.z + rec_bytes * (warp >> 2); rec < rec_stop; rec += rec_bytes * (kSets - 1)) {
+        const uint32_t rec_end = rec + rec_bytes;
+        const uint32_t meta = lds32(rec), unit = meta & 0xFFu, ch = (meta >> 12) & 0xFu;
+        const ChanConsts k = ld_chan_consts(desc + h2.y + word * 48u + ch * kChunkConstBytes);
+        const bool ok = w.barrier(full + 8u * unit, parity, ERR_WAIT_FULL);
+        if (!__all_sync(0xffffffffu, ok)) return false;                 // aborted: every other wait falls through too
         tc_fence_after();
-        for (uint32_t j = 0; j < n; ++j) {
-            const uint32_t tcol = j ? q0.w : q0.z, out = j ? q1.y : q1.x, rs = j ? q1.w : q1.z;
-            int acc[16];
-            tmem_ld16(E.tmem0 + tcol, acc);
-            tmem_st16_zero(E.tmem0 + tcol);
-            uint4 rv = make_uint4(0, 0, 0, 0);
-            if (res) rv = ld_shared_v4(E.res_thread + rs);
-            const uint32_t rw[4] = {rv.x ^ 0x80808080u, rv.y ^ 0x80808080u, rv.z ^ 0x80808080u, rv.w ^ 0x80808080u};
-            uint32_t o[4];
+#pragma unroll 1
+        for (; rec < rec_end; rec += 32u) {
+            const uint4 q0 = ld_shared_v4(rec), q1 = ld_shared_v4(rec + 16u);
+            // Four steps: two lines x two halves of 16 positions; the next step's accumulators are requested before this
+            // step's arithmetic.  (All 32 accumulators at once left no registers for the addresses.)
+            int acc[2][8];
+            tmem_ld_frag(tmem0 + q0.z, acc[0]);
+            uint4 start;
 #pragma unroll
-            for (int g = 0; g < 4; ++g) {
+            for (int st = 0; st < 4; ++st) {
+                const int l = st >> 1, h = st & 1;
+                int (&v)[8] = acc[st & 1];
+                const uint32_t tcol = tmem0 + (l ? q0.w : q0.z) + (h ? 16u << 16 : 0u), to = out + (l ? q1.y : q1.x);
+                const uint32_t from = res + (l ? q1.w : q1.z) + (uint32_t)h * 256u;
+                uint32_t r0 = 0, r1 = 0;
+                if (kResidual) { r0 = lds32(from) ^ 0x80808080u; r1 = lds32(from + 128u) ^ 0x80808080u; }
+                if (h == 0) start = ld_shared_v4(vecs + (l ? q0.x >> 26 : (q0.x >> 20) & 63u) * kVecBytes);
+                tmem_ld_frag_wait(v);
+                if (st < 3) tmem_ld_frag(tmem0 + (st == 0 ? q0.z + (16u << 16) : st == 1 ? q0.w : q0.w + (16u << 16)), acc[(st + 1) & 1]);
+                tmem_st_columns(tcol, start);
+                if (kScatter) {
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        const uint32_t pos = row0 + 16u * (uint32_t)h + 8u * (uint32_t)j;
+                        if ((pos >> g.log_i) & 1u) continue;
+                        const uint32_t o = requant4<false>(v[2 * j], v[2 * j + 1], v[2 * j + 4], v[2 * j + 5], k, 0u, 0u, 0u);
+                        uint32_t oline, oband;
+                        // q1 holds the chunk's plane here, not a line's offset
+                        const uint32_t at = to + scatter_to(g, pos, (q0.y >> (8 * l)) & 0xFFu, oline, oband);
+                        st_shared_u32(at, o);
+                        if (dup) {
+                            st_shared_u32_if(at + dup, o, oline == 0u && oband >= 1u);
+                            st_shared_u32_if(at - dup, o, oline + 1u == (1u << g.log_lines) && oband + 1u < nb);
+                        }
+                    }
+                } else {
+                    const uint32_t o0 = requant4<kResidual>(v[0], v[1], v[4], v[5], k, r0, m2, k8), at = to + (uint32_t)h * 256u;
+                    st_shared_u32(at, o0);
+                    const uint32_t o1 = requant4<kResidual>(v[2], v[3], v[6], v[7], k, r1, m2, k8);
+                    st_shared_u32(at + 128u, o1);
+                    const uint32_t edges = (q0.x >> (16 + 2 * l)) & 3u;
+                    if (dup && edges) {
+                        // first row of a lower band: also the row below the band above it; last row of an upper band: the
+                        // row above the next band
+                        const uint32_t e = bands & (edges | edges << 2);
+                        st_shared_u32_if(at + dup, o0, e & 1u);
+                        st_shared_u32_if(at - dup, o0, e & 2u);
+                        st_shared_u32_if(at + 128u + dup, o1, e & 4u);
+                        st_shared_u32_if(at + 128u - dup, o1, e & 8u);
+                    }
+                }
+            }
+        }
+        pass_done(done + 4u * unit, (int)lane);
+    }
+    return true;
+}
+
+// The general pass: a lower clamp above -128, a shift of one, a residual term without the single-precision form, a lone
+// line; one line at a time, every property decided at run time.
+__device__ __forceinline__ bool epi_conv_general(Waiter w, uint32_t tmem_lane, uint32_t warp, uint32_t lane, uint32_t desc, uint4 h0, uint4 h1, uint4 h2, uint4 h3, uint32_t use)
+{
+    const bool res = h0.x & CF_RES, scatter = h0.x & CF_SCATTER;
+    const uint32_t tmem0 = tmem_lane + h0.w, full = CTRL_ADDR(bars) + 8u * (h1.x + (use & 1u) * h2.x), done = CTRL_ADDR(stored) + 4u * h1.y;
+    const uint32_t parity = (use >> 1) & 1u, word = lane & 3u, row0 = (warp & 3u) * 32u + (lane >> 2), dup = h3.w;
+    const uint4 g0 = ld_shared_v4(desc + offsetof(LConvDesc, out_plane)), g1 = ld_shared_v4(desc + offsetof(LConvDesc, in_logI));
+    const uint4 gl = ld_shared_v4(desc + offsetof(LConvDesc, lo));
+    const int lo = (int)gl.x;
+    const long long r2 = (long long)(((unsigned long long)gl.z << 32) | gl.y);
+    const uint32_t nb = g1.z, vecs = desc + g1.w + word * 16u;
+    const Scatter g{g1.x, g1.y >> 1, g0.z, g0.w, g0.y};
+#pragma unroll 1
+    for (uint32_t i = warp >> 2; i < h0.y; i += kSets) {
+        const uint32_t rec = desc + h2.z + 32u * i;                   // one record per item
+        const uint4 q0 = ld_shared_v4(rec), q1 = ld_shared_v4(rec + 16u);
+        const uint32_t unit = q0.x & 0xFFu, n = (q0.x >> 8) & 0xFu;
+        const ChanConsts k = ld_chan_consts(desc + h2.y + word * 48u + ((q0.x >> 12) & 0xFu) * kChunkConstBytes);
+        const bool ok = w.barrier(full + 8u * unit, parity, ERR_WAIT_FULL);
+        if (!__all_sync(0xffffffffu, ok)) return false;
+        tc_fence_after();
+#pragma unroll 1
+        for (uint32_t l = 0; l < n; ++l) {
+            const uint32_t tcol = l ? q0.w : q0.z, to = the_base() + h2.w + word * 4u + (l ? q1.y : q1.x), line = (q0.y >> (8u * l)) & 0xFFu;
+            const uint32_t from = the_base() + h3.x + word * 4u + (l ? q1.w : q1.z), edges = q0.x >> (16u + 2u * l);
+            const uint4 start = ld_shared_v4(vecs + ((q0.x >> (20u + 6u * l)) & 63u) * kVecBytes);
+          for (uint32_t h = 0; h < 2; ++h) {
+            int a[8];
+            tmem_ld_frag(tmem0 + tcol + (h * 16u << 16), a);
+            tmem_ld_frag_wait(a);
+            tmem_st_columns(tmem0 + tcol + (h * 16u << 16), start);
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const uint32_t pos = row0 + 16u * h + 8u * (uint32_t)j;
+                const uint32_t rword = res ? lds32(from + pos * 16u) ^ 0x80808080u : 0u;
                 int y[4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const ChanConst4 cs = ld_chan_const_early(E.const_addr + ch * 256u + (4 * g + k) * 16);
-                    const long long prod = mul_wide(acc[4 * g + k] + cs.bias, cs.mult);
-                    int v = cs.s ? (hi32(prod) + cs.c) >> cs.s : hi32(prod) + (int)((uint32_t)lo32(prod) >> 31) + cs.c;
-                    if (res) v += hi32(mad_wide_u((rw[g] >> (8 * k)) & 0xFFu, E.res_m2, E.res_r2));
-                    y[k] = max(v, lo);
+                for (int q = 0; q < 4; ++q) {
+                    const long long prod = mul_wide(a[2 * j + (q & 1) + 4 * (q >> 1)], k.mult[q]);
+                    int v = k.s[q] ? (hi32(prod) + k.c[q]) >> k.s[q] : hi32(prod) + (int)((uint32_t)lo32(prod) >> 31) + k.c[q];
+                    if (res) v += hi32(mad_wide_u((rword >> (8 * q)) & 0xFFu, gl.w, r2));
+                    y[q] = max(v, lo);
                 }
-                o[g] = pack4_sat(y[0], y[1], y[2], y[3]);
-            }
-            const uint4 v = make_uint4(o[0], o[1], o[2], o[3]);
-            if (scatter) {
-                store_strided(desc, c.sbase, c.lane_idx, ch, (q0.y >> (8 * j)) & 0xFFu, v);
-            } else {
-                const uint32_t addr = E.out_thread + out;
-                st_shared_v4(addr, v);
-                if (E.dup_delta) {
-                    if (((q0.x >> (16 + 2 * j)) & 1u) & E.dup_up) st_shared_v4(addr + E.dup_delta, v);
-                    if (((q0.x >> (17 + 2 * j)) & 1u) & E.dup_dn) st_shared_v4(addr - E.dup_delta, v);
+                const uint32_t o = pack4_sat(y[0], y[1], y[2], y[3]);
+                uint32_t at = to + pos * 16u, up, dn;
+                if (scatter) {
+                    if ((pos >> g.log_i) & 1u) continue;
+                    uint32_t oline, oband;
+                    at = to + scatter_to(g, pos, line, oline, oband);
+                    up = oline == 0u && oband >= 1u;
+                    dn = oline + 1u == (1u << g.log_lines) && oband + 1u < nb;
+                } else {
+                    const uint32_t band = (pos >> 2) & (nb - 1u);
+                    up = (edges & 1u) && band >= 1u;
+                    dn = (edges & 2u) && band + 1u < nb;
+                }
+                st_shared_u32(at, o);
+                if (dup) {
+                    st_shared_u32_if(at + dup, o, up);
+                    st_shared_u32_if(at - dup, o, dn);
                 }
             }
+          }
         }
-        tmem_st_wait();
-        pass_done(E, c, unit);
+        pass_done(done + 4u * unit, (int)lane);
     }
-}
-
-__device__ __forceinline__ void epi_conv(const LineParams &p, const EpiCtx &c, uint32_t blob_off, uint32_t cg, int it)
-{
-    Waiter w{c.ctrl, p.err};
-    bool ok = w.barrier(smem_u32(&c.ctrl->wbar[cg % 3]), (cg / 3) & 1, ERR_WAIT_WEIGHTS);
-    ok = __all_sync(0xffffffffu, ok);
-    if (!ok) return;                    // the abort flag is up: every other wait falls through as well
-    const uint32_t desc = c.sbase + blob_off;
-    const uint4 h0 = ld_shared_v4(desc);
-    const uint4 h1 = ld_shared_v4(desc + offsetof(LConvDesc, a_base));
-    const uint4 h3 = ld_shared_v4(desc + offsetof(LConvDesc, d_base));
-    const uint4 h4 = ld_shared_v4(desc + offsetof(LConvDesc, use_local));
-    const uint4 h5 = ld_shared_v4(desc + offsetof(LConvDesc, w_rel));
-    const uint4 h6 = ld_shared_v4(desc + offsetof(LConvDesc, out_base));       // out_base, out_plane, out_pitch16, out_n_lines
-    const uint4 h7 = ld_shared_v4(desc + offsetof(LConvDesc, out_log_lines));  // out_log_lines, out_nb, out_logI, res_base
-    const uint4 h9 = ld_shared_v4(desc + offsetof(LConvDesc, lo));             // lo, res_m2, res_r2
-    const uint32_t use = (uint32_t)it * h4.y + h4.x;
-    EpiConv E;
-    E.tmem0 = c.tmem_lane + ((h1.w > 1 && (use & 1u)) ? h3.y : h3.x);
-    E.full_addr = smem_u32(&c.ctrl->bars[h3.z + (use & 1u) * h4.z]);
-    E.done_addr = smem_u32(&c.ctrl->stored[h3.w]);
-    E.parity = (use >> 1) & 1u;
-    E.const_addr = desc + h5.y;
-    E.out_thread = c.sbase + h6.x + c.lane_idx * 16u;
-    E.res_thread = c.sbase + h7.w + c.lane_idx * 16u;
-    const uint32_t band = (c.lane_idx >> 2) & (h7.y - 1u);
-    E.dup_delta = h7.y > 1u ? (h6.w * h6.z - 4u) * 16u : 0u;
-    E.dup_up = band >= 1u ? 1u : 0u;
-    E.dup_dn = band + 1u < h7.y ? 1u : 0u;
-    E.res_m2 = h9.y;
-    E.res_r2 = (long long)(((unsigned long long)h9.w << 32) | h9.z);
-    const uint32_t passes = desc + h5.w, n_passes = h0.y;
-    const uint32_t flags = h0.w;
-    if (flags & CF_GENERAL) {
-        epi_conv_general(w, E, c, desc, flags, (int32_t)h9.x, passes, n_passes);
-        return;
-    }
-    const uint32_t rpi = lds32(desc + offsetof(LConvDesc, recs_per_item));
-    if (flags & CF_RSHORT) epi_conv_fast<2>(w, E, c, passes, n_passes / rpi, 32u * rpi);
-    else if (flags & CF_RES) epi_conv_fast<1>(w, E, c, passes, n_passes / rpi, 32u * rpi);
-    else epi_conv_fast<0>(w, E, c, passes, n_passes / rpi, 32u * rpi);
+    return true;
 }
 
 // FILL: the region takes its halo value everywhere
-__device__ void fill_phase(const EpiCtx &c, uint32_t off, uint32_t bytes, uint32_t halo)
+__device__ __forceinline__ void fill_phase(uint32_t off, uint32_t bytes, uint32_t halo)
 {
     const uint32_t word = (halo & 0xFFu) * 0x01010101u;
     const uint4 v = make_uint4(word, word, word, word);
-    for (uint32_t o = (uint32_t)c.tid * 16u; o < bytes; o += kThreads * 16u) st_shared_v4(c.sbase + off + o, v);
+    for (uint32_t o = threadIdx.x * 16u; o < bytes; o += kThreads * 16u) st_shared_v4(the_base() + off + o, v);
 }
 
 // Which samples a group holds: image, phase, and the range of sample numbers.
@@ -778,9 +743,8 @@ __device__ __forceinline__ GroupJob group_job(const LineParams &p, int grp)
 // INPUT: one item = four horizontally adjacent pixels of one sample and input channel, one Philox block (Def. 3.3,
 // Def. 3.4).  Items of all channels share one index space (3072 items of a 32 x 32 x 3 image for 640 threads; with the
 // channels of a pixel in one thread it was 1024, two rounds of which the second is mostly idle), and the four table
-// searches run interleaved, until all four are found, instead of one after the other.  Out of line, like the tail's last
-// step: the convolutions' loops pay for every register and instruction that these phases share with them.
-__device__ __noinline__ void input_phase(const LineParams &p, const EpiCtx &c, int grp)
+// searches run interleaved, until all four are found, instead of one after the other.
+__device__ __forceinline__ void input_phase(const LineParams &p, int grp)
 {
     const int H = p.in_H, W = p.in_W, in_c = p.in_c;
     const int log_wq = 31 - __clz(W >> 2);                  // W is a power of two
@@ -795,7 +759,7 @@ __device__ __noinline__ void input_phase(const LineParams &p, const EpiCtx &c, i
     const long long j0 = (g.sel ? 0ll : p.ns.first_sample) + g.local;
     const uint8_t *__restrict__ x = p.x + (size_t)g.image * (size_t)(in_c * H * W);
     int ch = 0;
-    for (int i = c.tid, qi = c.tid; i < quads * in_c; i += kThreads, qi += kThreads) {
+    for (int i = (int)threadIdx.x, qi = i; i < quads * in_c; i += kThreads, qi += kThreads) {
         while (qi >= quads) { qi -= quads; ++ch; }
         // consecutive threads take consecutive samples: their stores fall into one 64-byte run
         const int s = qi & (kG - 1);
@@ -816,7 +780,7 @@ __device__ __noinline__ void input_phase(const LineParams &p, const EpiCtx &c, i
         }
         // the input has one row band: line = row, position = column * 4 + sample; the bytes beyond the input channels
         // meet zero weights
-        const uint32_t at = c.sbase + p.input_base + ((uint32_t)y * p.input_pitch16 + (uint32_t)(4 * x4) * kG + (uint32_t)s) * 16u + (uint32_t)ch;
+        const uint32_t at = the_base() + p.input_base + ((uint32_t)y * p.input_pitch16 + (uint32_t)(4 * x4) * kG + (uint32_t)s) * 16u + (uint32_t)ch;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const int v = min(255, max(0, (int)((clean >> (8 * k)) & 0xFFu) + z[k]));
@@ -830,13 +794,13 @@ __device__ __noinline__ void input_phase(const LineParams &p, const EpiCtx &c, i
 // the words of the four samples of a position (64 contiguous bytes), the shares meet in shared-memory additions.  (One
 // thread per channel and sample left most of the CTA idle over 64 to 1024 pixels: with the noise phase before it, a
 // network that ends at a 32 x 32 map spent 43 us a group more, the tiny CNN 15 us a call.)
-__device__ void tail_sum(const LineParams &p, const EpiCtx &c)
+__device__ __forceinline__ void tail_sum(const LineParams &p)
 {
-    const int units = p.tail_C, parts = kThreads / units, part = c.tid / units, u = c.tid - part * units;       // a unit is (word, sample)
+    const int units = p.tail_C, parts = kThreads / units, part = (int)threadIdx.x / units, u = (int)threadIdx.x - part * units;       // a unit is (word, sample)
     if (part >= parts) return;
     const int word = u >> 2, s = u & (kG - 1);
     const int log_w = 31 - __clz(p.tail_W), log_n = 31 - __clz(p.tail_n_lines);                                  // powers of two
-    const uint32_t base = c.sbase + p.tail_base + (uint32_t)(word >> 2) * p.tail_plane + (uint32_t)(word & 3) * 4u + (uint32_t)s * 16u;
+    const uint32_t base = the_base() + p.tail_base + (uint32_t)(word >> 2) * p.tail_plane + (uint32_t)(word & 3) * 4u + (uint32_t)s * 16u;
     int sum[4] = {0, 0, 0, 0}, n = 0;
     for (int i = part; i < p.tail_H * p.tail_W; i += parts, ++n) {
         const int y = i >> log_w, x = i & (p.tail_W - 1);
@@ -849,27 +813,28 @@ __device__ void tail_sum(const LineParams &p, const EpiCtx &c)
         sum[3] = __dp4a(v, 1 << 24, sum[3]);
     }
 #pragma unroll
-    for (int k = 0; k < 4; ++k) atomicAdd(&c.ctrl->pool_sum[s][4 * word + k], sum[k] - n * p.pool_zp_in);
+    for (int k = 0; k < 4; ++k) atomicAdd(&the_ctrl()->pool_sum[s][4 * word + k], sum[k] - n * p.pool_zp_in);
 }
 
 // Second step: the sums' requantisation.
-__device__ void tail_pool(const LineParams &p, const EpiCtx &c)
+__device__ __forceinline__ void tail_pool(const LineParams &p)
 {
-    for (int q = c.tid; q < kG * p.tail_C; q += kThreads) {
+    for (int q = (int)threadIdx.x; q < kG * p.tail_C; q += kThreads) {
         const int s = q & (kG - 1), ch = q >> 2;
-        const int sum = c.ctrl->pool_sum[s][ch];
-        c.ctrl->pool_sum[s][ch] = 0;
+        const int sum = the_ctrl()->pool_sum[s][ch];
+        the_ctrl()->pool_sum[s][ch] = 0;
         long long v = ((long long)sum * p.pool_mult + (1ll << (p.pool_n - 1))) >> p.pool_n;
         v += p.pool_zp_out;
         v = v < p.pool_lo ? p.pool_lo : v;
         v = v > 127 ? 127 : v;
-        c.ctrl->pooled[s][ch] = (int8_t)v;
+        the_ctrl()->pooled[s][ch] = (int8_t)v;
     }
 }
 
 // Third step: FC, argmax and vote; one warp carries one sample, a lane one class (features beyond the last meet zero weights).
-__device__ __noinline__ void tail_sample(const LineParams &p, const EpiCtx &c, int s, int grp)
+__device__ __forceinline__ void tail_sample(const LineParams &p, int s, int grp)
 {
+    const int lane = (int)threadIdx.x & 31;
     const int n_classes = p.n_classes;
     const GroupJob g = group_job(p, grp);
     const int sample = g.local + s;                            // index within the image's phase
@@ -877,9 +842,9 @@ __device__ __noinline__ void tail_sample(const LineParams &p, const EpiCtx &c, i
     int best_v = -1000, best_o = 0x7fffffff;
     uint4 f[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) f[k] = ld_shared_v4(smem_u32(&c.ctrl->pooled[s][16 * k]));
+    for (int k = 0; k < 4; ++k) f[k] = ld_shared_v4(CTRL_ADDR(pooled) + (uint32_t)(64 * s + 16 * k));
     for (int o0 = 0; o0 < n_classes; o0 += 32) {
-        const int o = o0 + c.lane;
+        const int o = o0 + lane;
         const bool live = o < n_classes;
         const FcConst k = p.fc_c[live ? o : 0];
         const uint4 *wrow = reinterpret_cast<const uint4 *>(p.fc_w + (size_t)(live ? o : 0) * 64);
@@ -907,117 +872,156 @@ __device__ __noinline__ void tail_sample(const LineParams &p, const EpiCtx &c, i
         const int ov = __shfl_xor_sync(0xffffffffu, best_v, d), oo = __shfl_xor_sync(0xffffffffu, best_o, d);
         if (ov > best_v || (ov == best_v && oo < best_o)) { best_v = ov; best_o = oo; }
     }
-    if (counted && c.lane == 0) {
+    if (counted && lane == 0) {
         const int row = p.groups_sel ? 2 * g.image + (g.sel ? 0 : 1) : g.image;
         atomicAdd(p.counts + (size_t)row * n_classes + best_o, 1);
     }
 }
 
+// A phase of the whole CTA: everything before it is complete in all warps, and it is before anything after it.  Nothing inside
+// can raise the abort flag, so that all warps skip it or none.  Thread 0 keeps the time (phases run between barriers, so one
+// thread's clock measures them).
+__device__ __forceinline__ void cta_phase(const LineParams &p, uint4 e, int grp)
+{
+    Ctrl *ctrl = the_ctrl();
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const bool live = !Waiter::aborted();
+    if (threadIdx.x == 0) ctrl->cyc_mark = clock64();
+    if (live) {
+        if (e.x == PH_FILL) fill_phase(e.y, e.z, e.w);
+        else if (e.x == PH_INPUT) input_phase(p, grp);
+        else tail_sum(p);
+    }
+    if (e.x == PH_TAIL) {
+        __syncthreads();
+        if (live) tail_pool(p);
+        __syncthreads();
+        if (live && threadIdx.x < 32 * kG) tail_sample(p, (int)(threadIdx.x >> 5), grp);
+    }
+    fence_proxy_async();
+    __syncthreads();
+    if (threadIdx.x == 0) ctrl->cyc[e.x & 3u] += clock64() - ctrl->cyc_mark;
+}
+
+// The roles' shares of the convolutions from phase `ph` on, up to the next phase of the whole CTA.  After the abort flag is
+// up a role skips its convolutions and goes on through the phases.
+struct RoleState {
+    WeightSlot ws;              // of the next convolution (loader: of the next copy)
+    bool ok = true;
+    PrevConv prev{0u, 0u, 0u};
+    int next_copy = 0;
+};
+
+__device__ __forceinline__ void epilogue_run(const LineParams &p, uint32_t tmem, uint32_t warp, uint32_t lane, int ph, int stop, int it, RoleState &r)
+{
+    const Waiter w{p.err};
+    const uint32_t tmem_lane = tmem + ((warp & 3u) * 32u << 16);
+    for (; ph < stop; ++ph) {
+        if (r.ok) r.ok = __all_sync(0xffffffffu, w.barrier(CTRL_ADDR(wbar) + 8u * r.ws.slot, r.ws.parity, ERR_WAIT_WEIGHTS));
+        r.ws.advance();
+        if (!r.ok) continue;
+        const uint32_t desc = the_base() + lds32(CTRL_ADDR(ptab) + 16u * (uint32_t)ph + 4u);
+        const uint4 h0 = ld_shared_v4(desc), h1 = ld_shared_v4(desc + 16u), h2 = ld_shared_v4(desc + 32u), h3 = ld_shared_v4(desc + 48u);
+        const uint32_t use = (uint32_t)it * h1.w + h1.z;
+        if (h0.x & CF_GENERAL) r.ok = epi_conv_general(w, tmem_lane, warp, lane, desc, h0, h1, h2, h3, use);
+        else if (h0.x & CF_SCATTER) r.ok = epi_conv_fast<false, true>(w, tmem_lane, warp, lane, desc, h0, h1, h2, h3, use);
+        else if (h0.x & CF_RES) r.ok = epi_conv_fast<true, false>(w, tmem_lane, warp, lane, desc, h0, h1, h2, h3, use);
+        else r.ok = epi_conv_fast<false, false>(w, tmem_lane, warp, lane, desc, h0, h1, h2, h3, use);
+    }
+}
+
+__device__ __forceinline__ void issuer_run(const LineParams &p, uint32_t tmem, uint32_t issuer, int ph, int stop, int it, RoleState &r)
+{
+    for (; ph < stop; ++ph, r.ws.advance())
+        if (r.ok && !Waiter::aborted()) r.ok = issuer_conv(p, tmem, lds32(CTRL_ADDR(ptab) + 16u * (uint32_t)ph + 4u), r.ws, issuer, it, r.prev);
+}
+
+__device__ __forceinline__ void loader_run(const LineParams &p, int ph, int stop, int it, RoleState &r)
+{
+    for (; ph < stop && r.next_copy < p.n_conv; ++ph, ++r.next_copy, r.ws.advance())
+        if (r.ok && !Waiter::aborted()) r.ok = loader_copy(p, r.next_copy, r.ws.slot, it);
+}
+
 __global__ void __launch_bounds__(kThreads, 1) k_line(const __grid_constant__ LineParams p)
 {
-    extern __shared__ __align__(128) uint8_t smem[];
-    Ctrl *ctrl = reinterpret_cast<Ctrl *>(smem);
-    const uint32_t sbase = smem_u32(smem);
-    const int warp = (int)warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
-    for (int i = threadIdx.x; i < p.n_bars; i += blockDim.x) mbar_init(smem_u32(&ctrl->bars[i]), p.bar_counts[i]);
+    Ctrl *ctrl = the_ctrl();
+    const uint32_t warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31u;
+    for (int i = threadIdx.x; i < p.n_bars; i += blockDim.x) mbar_init(CTRL_ADDR(bars) + 8u * (uint32_t)i, p.bar_counts[i]);
     if (threadIdx.x == 0) {
-        for (int s = 0; s < 3; ++s) mbar_init(smem_u32(&ctrl->wbar[s]), 1);
-        mbar_init(smem_u32(&ctrl->drain), kIssuers);
+        for (uint32_t s = 0; s < 3; ++s) mbar_init(CTRL_ADDR(wbar) + 8u * s, 1);
+        mbar_init(CTRL_ADDR(drain), kIssuers);
         ctrl->abort_flag = 0;
     }
     for (int i = threadIdx.x; i < p.n_phases; i += blockDim.x) ctrl->ptab[i] = p.ptab[i];
     for (int i = threadIdx.x; i < p.n_conv; i += blockDim.x) ctrl->csrc[i] = p.conv_src[i];
     for (int i = threadIdx.x; i < kMaxBars; i += blockDim.x) ctrl->stored[i] = 0;
     for (int i = threadIdx.x; i < kG * 64; i += blockDim.x) (&ctrl->pool_sum[0][0])[i] = 0;
-    if (warp == 0) tmem_alloc(smem_u32(&ctrl->tmem_base), kTmemCols);
+    if (warp == 0) tmem_alloc(CTRL_ADDR(tmem_base), kTmemCols);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_proxy_async();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = ctrl->tmem_base;
-
-    EpiCtx c;
-    c.ctrl = ctrl; c.sbase = sbase;
-    c.warp = warp; c.set = warp >> 2; c.quarter = warp & 3; c.lane = lane; c.tid = threadIdx.x;
-    c.lane_idx = (uint32_t)((warp & 3) * 32 + lane);
-    c.tmem_lane = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-    const bool issuer = warp >= kEpiWarps && warp < kEpiWarps + kIssuers, loader = warp == kLoaderWarp, epi = warp < kEpiWarps;
-    // accumulators of stacked convolutions start from zero
-    if (epi) {
-        for (uint32_t col = (uint32_t)c.set * 16u; col < (uint32_t)kTmemCols; col += kSets * 16u) tmem_st16_zero(c.tmem_lane + col);
+    // accumulators start from the folded biases of the first convolution that uses them
+    if (warp < kEpiWarps) {
+        const uint32_t lanes = tmem + ((warp & 3u) * 32u << 16);
+        for (uint32_t col = (warp >> 2) * 16u; col < (uint32_t)kTmemCols; col += kSets * 16u) {
+            const uint4 b = __ldg(reinterpret_cast<const uint4 *>(p.acc_init + col) + (lane & 3u));
+            tmem_st_columns(lanes + col, b);
+            tmem_st_columns(lanes + col + (16u << 16), b);
+        }
         tmem_st_wait();
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-
-    const uint32_t ptab = smem_u32(ctrl->ptab);
-    const int n_phases = p.n_phases, stop_phase = p.stop_phase;
-    bool role_ok = true;
-    int it = 0;
-    // thread 0 keeps the time the CTA spends in its CTA-wide phases (they run between barriers, so one thread's clock
-    // measures them); what is left of the kernel's duration is the convolutions
     if (threadIdx.x == 0) {
         ctrl->cyc[PH_FILL] = ctrl->cyc[PH_INPUT] = ctrl->cyc[PH_TAIL] = 0;
-        ctrl->cyc[PH_CONV] = clock64();         // until the end: the start time
+        ctrl->cyc[PH_CONV] = clock64();         // until the end: the start time; what phases leave of the duration is the convolutions
     }
+    const int end = min(p.n_phases, p.stop_phase + 1);
+    RoleState r;
+    int it = 0;
     for (int grp = blockIdx.x; grp < p.n_groups; grp += gridDim.x, ++it) {
-        PrevConv prev{0u, 0u, 0u};
-        int conv_index = 0;
-        bool first_phase = true;
-        for (int ph = 0; ph < n_phases && ph <= stop_phase; ++ph) {
-            const uint4 e = ld_shared_v4(ptab + 16 * ph);
-            if (e.x == PH_CONV) {
-                const uint32_t cg = (uint32_t)it * (uint32_t)p.n_conv + (uint32_t)conv_index;
-                if (issuer) {
-                    if (lane == 0 && role_ok && !ctrl->abort_flag)
-                        role_ok = issuer_conv(p, ctrl, sbase, tmem, e.y, cg, warp - kEpiWarps, it, prev);
-                    __syncwarp();
-                } else if (loader) {
-                    if (lane == 0 && role_ok && !ctrl->abort_flag && conv_index + 1 < p.n_conv)
-                        role_ok = loader_copy(p, ctrl, sbase, conv_index + 1, cg + 1u, it);
-                    __syncwarp();
-                } else if (!ctrl->abort_flag) {
-                    epi_conv(p, c, e.y, cg, it);
-                }
-                conv_index += 1;
-                first_phase = false;
+        // the first blob of the group: everything of the previous group is complete
+        if (warp == kLoaderWarp && p.n_conv > 0) {
+            if (lane == 0 && r.ok && !Waiter::aborted()) r.ok = loader_copy(p, 0, r.ws.slot, it);
+            r.ws.advance();
+            r.next_copy = 1;
+        }
+        for (int ph = 0; ph < end;) {
+            const uint4 e = ld_shared_v4(CTRL_ADDR(ptab) + 16u * (uint32_t)ph);
+            if (e.x != PH_CONV) {
+                cta_phase(p, e, grp);
+                r.prev.n_lines = 0;
+                ++ph;
                 continue;
             }
-            // CTA-wide phase: everything before it is complete in all warps
-            tc_fence_before();
-            __syncthreads();
-            tc_fence_after();
-            prev.n_lines = 0;
-            if (first_phase) {
-                // the first blob of the group: everything of the previous group is complete
-                if (loader && lane == 0 && p.n_conv > 0 && role_ok && !ctrl->abort_flag)
-                    role_ok = loader_copy(p, ctrl, sbase, 0, (uint32_t)it * (uint32_t)p.n_conv, it);
-                first_phase = false;
+            const int stop = min(end, ph + (int)e.z);
+            if (warp < kEpiWarps) {
+                epilogue_run(p, tmem, warp, lane, ph, stop, it, r);
+            } else if (lane == 0) {
+                if (warp < kLoaderWarp) issuer_run(p, tmem, warp - kEpiWarps, ph, stop, it, r);
+                else loader_run(p, ph, stop, it, r);
             }
-            // every warp of the CTA takes part in these phases; nothing inside them can raise the abort flag
-            const bool live = !ctrl->abort_flag;
-            if (threadIdx.x == 0) ctrl->cyc_mark = clock64();
-            if (live) {
-                if (e.x == PH_FILL) fill_phase(c, e.y, e.z, e.w);
-                else if (e.x == PH_INPUT) input_phase(p, c, grp);
-                else tail_sum(p, c);
-            }
-            if (e.x == PH_TAIL) {
-                __syncthreads();
-                if (live) tail_pool(p, c);
-                __syncthreads();
-                if (live && warp < kG) tail_sample(p, c, warp, grp);
-            }
-            fence_proxy_async();
-            __syncthreads();
-            if (threadIdx.x == 0) ctrl->cyc[e.x & 3u] += clock64() - ctrl->cyc_mark;
+            ph = stop;
         }
+        __syncwarp();
         tc_fence_before();
         __syncthreads();
         tc_fence_after();
     }
+    // no tensor-core work may be in flight when tensor memory is released
+    if (warp >= kEpiWarps && warp < kLoaderWarp && lane == 0) {
+        const Waiter w{p.err};
+        commit_to(CTRL_ADDR(drain));
+        w.barrier(CTRL_ADDR(drain), 0, ERR_WAIT_DRAIN);
+    }
+    __syncwarp();
     if (threadIdx.x == 0 && p.phase_cycles) {
         const long long total = clock64() - ctrl->cyc[PH_CONV];
         atomicAdd(p.phase_cycles + PH_FILL, (unsigned long long)ctrl->cyc[PH_FILL]);
@@ -1027,13 +1031,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_line(const __grid_constant__ Li
     }
     if (p.dump)
         for (uint32_t o = threadIdx.x * 16u; o < p.dump_bytes; o += blockDim.x * 16u)
-            *reinterpret_cast<uint4 *>(p.dump + o) = ld_shared_v4(sbase + p.dump_off + o);
-    // no tensor-core work may be in flight when tensor memory is released
-    if (issuer && lane == 0) {
-        Waiter w{ctrl, p.err};
-        commit_to(smem_u32(&ctrl->drain));
-        w.barrier(smem_u32(&ctrl->drain), 0, ERR_WAIT_DRAIN);
-    }
+            *reinterpret_cast<uint4 *>(p.dump + o) = ld_shared_v4(the_base() + p.dump_off + o);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -1045,8 +1043,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_line(const __grid_constant__ Li
 // through at once.  out[0..1] = what the two waits returned, out[2] = the abort flag, out[3] = nanoseconds spent.
 __global__ void k_wait_probe(int32_t *err, unsigned long long limit_ns, int32_t *out)
 {
-    extern __shared__ __align__(128) uint8_t smem[];
-    Ctrl *ctrl = reinterpret_cast<Ctrl *>(smem);
+    Ctrl *ctrl = the_ctrl();
     if (threadIdx.x == 0) {
         mbar_init(smem_u32(&ctrl->bars[0]), 1);
         ctrl->abort_flag = 0;
@@ -1055,7 +1052,7 @@ __global__ void k_wait_probe(int32_t *err, unsigned long long limit_ns, int32_t 
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     __syncthreads();
     if (threadIdx.x == 0) {
-        Waiter w{ctrl, err, limit_ns};
+        const Waiter w{err, limit_ns};
         const unsigned long long t0 = globaltimer();
         out[0] = w.barrier(smem_u32(&ctrl->bars[0]), 0, ERR_WAIT_FULL) ? 1 : 0;
         out[1] = w.counter(smem_u32(&ctrl->stored[0]), 1u, ERR_WAIT_DONE) ? 1 : 0;
@@ -1145,6 +1142,7 @@ struct LinePlan {
     PhaseEntry *d_ptab = nullptr;
     ConvSrc *d_conv_src = nullptr;
     uint8_t *d_bar_counts = nullptr;
+    int32_t *d_acc_init = nullptr;
     uint8_t *d_blob = nullptr;
     int8_t *d_fc_w = nullptr;
     FcConst *d_fc_c = nullptr;
@@ -1166,6 +1164,8 @@ struct ConvPlan {
     int layer = -1, phase = -1;
     int in_tensor = -1, out_tensor = -1;
     bool stacked = false, scatter = false, general = false;
+    ResidualForm res_form;              // of the residual term, and its constant
+    int32_t res_c = 0;
     int recs_per_item = 1;              // records of the pass table per (unit, chunk)
     int m = 0;                          // output lines (ordinals)
     int n_chunks = 0, cols = 0, n_banks = 1;
@@ -1185,7 +1185,7 @@ struct ConvPlan {
 // op_chains: MMA chains that one operation may hold at most
 bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_w, int n_classes, int op_chains, LinePlan *plan,
                 std::vector<uint8_t> *blob_out, std::vector<uint32_t> *blob_offsets, std::vector<PhaseEntry> *ptab_out,
-                std::vector<ConvSrc> *csrc_out, std::vector<uint8_t> *bar_counts_out)
+                std::vector<ConvSrc> *csrc_out, std::vector<uint8_t> *bar_counts_out, std::vector<int32_t> *acc_init_out)
 {
     const int n_conv_layers = n_layers - 2;
     // ---- tensors of the model (tensor t = output of layer t-1)
@@ -1292,7 +1292,7 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
         if (cp.scatter && (in.n_lines & 1)) PLAN_FAIL(6);
         cp.m = cp.scatter ? in.n_lines / 2 : in.n_lines;
         if (cp.m > kMaxLines || cp.m * cp.cols > kTmemCols) PLAN_FAIL(7);
-        cp.stacked = L.kh == 3 && L.stride == 1 && 3 * L.cout <= 128 && in.n_lines >= 2;
+        cp.stacked = L.kh == 3 && L.stride == 1 && in.n_lines >= 2;
         cp.n_banks = kTmemCols / (cp.m * cp.cols) >= 2 ? 2 : 1;
         if (L.res_tensor >= 0) {
             const LGeo &r = T[(size_t)L.res_tensor];
@@ -1332,7 +1332,7 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
         // ---- operations
         const ConvPlan *pv = (!convs.empty() && convs.back().phase == ph - 1) ? &convs.back() : nullptr;
         // same lines and chunks: the same barriers (class) and, with one bank, the same accumulator columns
-        const bool same_class = pv && pv->m == cp.m && pv->n_chunks == cp.n_chunks;
+        const bool same_class = pv && pv->m == cp.m && pv->n_chunks == cp.n_chunks && pv->scatter == cp.scatter;
         // the previous convolution produced this one's input, line for line
         const bool aligned = pv && in.producer_conv == (int)convs.size() - 1 && !pv->scatter;
         // Same class: the same barriers, and with one bank the same accumulator columns.  An operation then waits for
@@ -1410,8 +1410,20 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
         // counter) covers `upl` lines = one or two records.  Long convolutions take four-line units: every barrier
         // arrival costs an issuing thread a tcgen05.commit and every unit costs an epilogue warp a wait and an arrival.
         const int sup = cp.m >= 2 ? 2 : 1;
-        bool general = cp.scatter || (cp.m & 1) || (L.relu && L.zp_out > -128);
+        // the fast pass covers pairs of lines with the saturating pack as the only clamp, and a residual term that is a
+        // single-precision product whose constant fits into every channel's rounding addend
+        bool general = (cp.m & 1) || (L.relu && L.zp_out > -128);
         for (int oc = 0; oc < L.cout; ++oc) general = general || layers[cp.layer].shift[oc] == 1;
+        if (!general && L.res_tensor >= 0) {
+            cp.res_form = residual_form(L.res_mult, L.res_shift, L.zp_res, &cp.res_c);
+            general = !cp.res_form.exists();
+            for (int oc = 0; oc < L.cout && !general; ++oc) {
+                const int sft = layers[cp.layer].shift[oc] - 1;
+                const long long add = sft >= 1 ? (1ll << (sft - 1)) + ((long long)L.zp_out - cp.res_c) * (1ll << sft) : (1ll << 40);
+                general = add < -(1ll << 31) || add >= (1ll << 31);
+            }
+            if (general) cp.res_c = 0;
+        }
         cp.general = general;
         const int upl = (!general && cp.m >= 16 && cp.m % 4 == 0) ? 4 : sup;
         cp.recs_per_item = upl / sup;
@@ -1431,7 +1443,7 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
         }
         cp.cls = class_of[key];
         cp.use_local = class_uses[(size_t)cp.cls]++;
-        const bool wait_all = pv && pv->cls != cp.cls;
+        const bool wait_all = pv && (pv->cls != cp.cls || !same_class);
         // Record i belongs to issuing thread i mod kIssuers; every thread needs a record to carry its arrivals.
         auto null_op = []() { ProtoOp o; o.a_line = 0; o.b_block = 0; o.n_blocks = 0; o.d_line = 0; o.n_chains = 0; o.ready = 0; return o; };
         while (proto.size() < (size_t)kIssuers) proto.push_back(null_op());
@@ -1536,7 +1548,7 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
                     const int line = order[(size_t)first + q];
                     P.lines |= (uint32_t)line << (8 * q);
                     P.tcol[q] = (uint32_t)(line * cp.cols + ch * 16);
-                    P.out[q] = (uint32_t)(line * out.pitch) * 16u + (uint32_t)ch * out.plane_bytes;
+                    P.out[q] = (cp.scatter ? 0u : (uint32_t)(line * out.pitch) * 16u) + (uint32_t)ch * out.plane_bytes;
                     P.res[q] = L.res_tensor >= 0 ? (uint32_t)(line * out.pitch) * 16u + (uint32_t)ch * T[(size_t)L.res_tensor].plane_bytes : 0u;
                     if (!cp.scatter) {
                         if (line == 0) P.meta |= 1u << (16 + 2 * q);
@@ -1550,6 +1562,50 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
     }
     const int n_conv = (int)convs.size();
     if (n_conv > kMaxConv) PLAN_FAIL(22);
+    // ---- start values of the accumulators: whoever reads 16 columns leaves in them the folded biases of the channels that
+    // the next convolution on these columns (in the cyclic order of the groups) puts there
+    std::vector<std::vector<int32_t>> bias((size_t)n_conv);
+    for (int c = 0; c < n_conv; ++c) {
+        const isc_layer &L = layers[convs[(size_t)c].layer].d;
+        const LayerIn &ML = layers[convs[(size_t)c].layer];
+        const int per = L.cin * L.kh * L.kw;
+        for (int oc = 0; oc < L.cout; ++oc) {
+            long long wsum = 0;
+            for (int q = 0; q < per; ++q) wsum += ML.w[(size_t)oc * per + q];
+            const long long b = (long long)ML.bias[oc] - (long long)L.zp_in * wsum;
+            if (b < -(1ll << 31) || b >= (1ll << 31)) PLAN_FAIL(24);
+            bias[(size_t)c].push_back((int32_t)b);
+        }
+    }
+    auto bank_base = [&](int c) { const ConvPlan &cp = convs[(size_t)c]; return (cp.n_banks > 1 && (cp.use_local & 1)) ? cp.m * cp.cols : 0; };
+    // the convolution after `c` that uses column `col`, and its 16 channels there: *first; -1: none
+    auto next_user = [&](int c, int col, int *first) {
+        for (int d = 1; d <= n_conv; ++d) {
+            const int q = (c + d) % n_conv, at = col - bank_base(q);
+            if (at < 0 || at >= convs[(size_t)q].m * convs[(size_t)q].cols) continue;
+            *first = at % convs[(size_t)q].cols;
+            return q;
+        }
+        return -1;
+    };
+    std::vector<std::vector<std::pair<int, int>>> vecs((size_t)n_conv);         // per convolution: (next user, its first channel)
+    for (int c = 0; c < n_conv; ++c)
+        for (LPass &P : convs[(size_t)c].passes)
+            for (uint32_t q = 0; q < ((P.meta >> 8) & 0xFu); ++q) {
+                std::pair<int, int> key;
+                key.first = next_user(c, bank_base(c) + (int)P.tcol[q], &key.second);
+                std::vector<std::pair<int, int>> &v = vecs[(size_t)c];
+                const size_t at = (size_t)(std::find(v.begin(), v.end(), key) - v.begin());
+                if (at == v.size()) v.push_back(key);
+                if (at >= 64) PLAN_FAIL(26);
+                P.meta |= (uint32_t)at << (20 + 6 * q);
+            }
+    acc_init_out->assign((size_t)kTmemCols, 0);
+    for (int col = 0; col < kTmemCols; col += 16) {
+        int first = 0;
+        const int q = next_user(n_conv - 1, col, &first);
+        for (int b = 0; b < 16 && q >= 0; ++b) (*acc_init_out)[(size_t)col + b] = bias[(size_t)q][(size_t)first + b];
+    }
     // ---- barriers: per class, one per output line for "accumulators complete" and one for "line stored"
     std::vector<int> class_full(class_lines.size()), class_done(class_lines.size());
     bar_counts_out->clear();
@@ -1562,7 +1618,7 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
     if ((int)bar_counts_out->size() > kMaxBars) PLAN_FAIL(14);
     // ---- blob sizes and shared-memory placement in order of birth
     std::vector<uint32_t> w_bytes((size_t)n_conv), w_off((size_t)n_conv), w_rel((size_t)n_conv), c_rel((size_t)n_conv),
-        ops_rel((size_t)n_conv), passes_rel((size_t)n_conv);
+        ops_rel((size_t)n_conv), passes_rel((size_t)n_conv), vec_rel((size_t)n_conv);
     for (int c = 0; c < n_conv; ++c) {
         const ConvPlan &cp = convs[(size_t)c];
         const isc_layer &L = layers[cp.layer].d;
@@ -1572,7 +1628,8 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
         passes_rel[(size_t)c] = at; at += (uint32_t)cp.passes.size() * (uint32_t)sizeof(LPass);
         at = (at + 127u) & ~127u;
         w_rel[(size_t)c] = at; at += (uint32_t)cp.kunits.size() * rows * 32u;
-        c_rel[(size_t)c] = at; at += (uint32_t)L.cout * 16u;
+        c_rel[(size_t)c] = at; at += (uint32_t)(L.cout / 16) * kChunkConstBytes;
+        vec_rel[(size_t)c] = at; at += (uint32_t)vecs[(size_t)c].size() * kVecBytes;
         w_bytes[(size_t)c] = (at + 127u) & ~127u;
     }
     std::vector<AllocReq> reqs, placed;
@@ -1631,70 +1688,42 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
         const isc_layer &L = ML.d;
         const LGeo &in = T[(size_t)cp.in_tensor], &out = T[(size_t)cp.out_tensor];
         E.a = w_off[(size_t)c];
+        for (int q = ph; q < n_phases && skel[(size_t)q].kind == PH_CONV; ++q) E.b += 1;
         std::vector<uint8_t> blob(w_bytes[(size_t)c], 0);
         LConvDesc D;
         memset(&D, 0, sizeof(D));
-        int32_t res_c = 0;                    // constant of the residual term's short form, folded into the rounding addends
-        D.n_ops = (uint32_t)cp.ops.size(); D.n_passes = (uint32_t)cp.passes.size(); D.n_ksteps = (uint32_t)cp.kunits.size();
-        D.flags = (cp.stacked ? CF_STACKED : 0u) | (L.res_tensor >= 0 ? CF_RES : 0u) | (cp.scatter ? CF_SCATTER : 0u);
-        const int lo = L.relu ? std::max(-128, L.zp_out) : -128;
-        if (lo > -128) D.flags |= CF_LO;
-        D.lo = lo;
-        // the fast pass covers pairs of lines stored in place with the saturating pack as the only clamp
-        if (cp.general) D.flags |= CF_GENERAL;
-        D.recs_per_item = (uint32_t)cp.recs_per_item;
-        // operand base: line -1, lane 0, plane 0 of the input
-        D.a_base = plan->tensor_off[(size_t)cp.in_tensor] + in.line0 - (uint32_t)in.pitch * 16u;
-        D.pitch16 = (uint32_t)in.pitch;
-        D.bblock16 = (uint32_t)L.cout * 2u;
-        D.n_banks = (uint32_t)cp.n_banks;
-        const uint32_t a_fmt = cp.in_tensor == 0 ? 0u : 1u;
-        for (int nbk = 1; nbk <= 3; ++nbk)
-            D.idesc[nbk - 1] = (2u << 4) | (a_fmt << 7) | (1u << 10) | ((uint32_t)((nbk * L.cout) >> 3) << 17) | ((128u >> 4) << 24);
-        D.cols = (uint32_t)cp.cols;
-        D.d_base[0] = 0; D.d_base[1] = cp.n_banks > 1 ? (uint32_t)(cp.m * cp.cols) : 0u;
+        D.flags = (L.res_tensor >= 0 ? CF_RES : 0u) | (cp.scatter ? CF_SCATTER : 0u) | (cp.general ? CF_GENERAL : 0u);
+        D.n_items = (uint32_t)(cp.n_units * cp.n_chunks); D.recs_per_item = (uint32_t)cp.recs_per_item; D.d_base = (uint32_t)bank_base(c);
         D.bar_full = (uint32_t)class_full[(size_t)cp.cls]; D.bar_done = (uint32_t)class_done[(size_t)cp.cls];
         D.use_local = (uint32_t)cp.use_local; D.uses_per_group = (uint32_t)class_uses[(size_t)cp.cls];
-        D.n_lines = (uint32_t)cp.n_units; D.n_chunks = (uint32_t)cp.n_chunks;
-        D.w_rel = w_rel[(size_t)c]; D.c_rel = c_rel[(size_t)c]; D.ops_rel = ops_rel[(size_t)c]; D.passes_rel = passes_rel[(size_t)c];
+        D.n_units = (uint32_t)cp.n_units; D.c_rel = c_rel[(size_t)c]; D.passes_rel = passes_rel[(size_t)c];
         D.out_base = plan->tensor_off[(size_t)cp.out_tensor] + out.line0;
-        D.out_plane = out.plane_bytes; D.out_pitch16 = (uint32_t)out.pitch; D.out_n_lines = (uint32_t)out.n_lines;
-        D.out_log_lines = (uint32_t)ilog2(out.n_lines); D.out_nb = (uint32_t)out.nb; D.out_logI = (uint32_t)ilog2(out.I);
+        D.dup_delta = out.nb > 1 ? (uint32_t)(out.n_lines * out.pitch - 4) * 16u : 0u;
+        D.out_plane = out.plane_bytes; D.out_pitch16 = (uint32_t)out.pitch;
+        D.out_log_lines = (uint32_t)ilog2(out.n_lines); D.out_logI = (uint32_t)ilog2(out.I);
         if ((1 << D.out_log_lines) != out.n_lines) PLAN_FAIL(16);
-        D.in_logI = (uint32_t)ilog2(in.I); D.in_I = (uint32_t)in.I; D.in_n_lines = (uint32_t)in.n_lines;
+        D.in_logI = (uint32_t)ilog2(in.I); D.in_n_lines = (uint32_t)in.n_lines; D.out_nb = (uint32_t)out.nb; D.vec_rel = vec_rel[(size_t)c];
+        D.lo = L.relu ? std::max(-128, L.zp_out) : -128;
+        D.n_ops = (uint32_t)cp.ops.size(); D.n_ksteps = (uint32_t)cp.kunits.size(); D.ops_rel = ops_rel[(size_t)c]; D.n_chunks = (uint32_t)cp.n_chunks;
+        D.pitch16 = (uint32_t)in.pitch; D.cols = (uint32_t)cp.cols;
+        // operand base: line -1, lane 0, plane 0 of the input
+        const uint32_t a_base = plan->tensor_off[(size_t)cp.in_tensor] + in.line0 - (uint32_t)in.pitch * 16u;
         if (L.res_tensor >= 0) {
-            const LGeo &r = T[(size_t)L.res_tensor];
-            D.res_base = plan->tensor_off[(size_t)L.res_tensor] + r.line0;
-            D.res_plane = r.plane_bytes;
+            const LGeo &rt = T[(size_t)L.res_tensor];
+            D.res_base = plan->tensor_off[(size_t)L.res_tensor] + rt.line0;
             const int res_n = 31 - L.res_shift;
             const unsigned long long m2 = (unsigned long long)(uint32_t)L.res_mult << (32 - res_n);
             if (L.res_mult <= 0 || m2 >= (1ull << 32)) PLAN_FAIL(17);
             // rs((r - zp) * mult, n) = floor(((u - 128 - zp) * mult + 2^(n-1)) * 2^(32-n) / 2^32), u = r + 128
             const long long r2 = (((1ll << (res_n - 1)) - (128ll + L.zp_res) * (long long)L.res_mult)) * (1ll << (32 - res_n));
-            D.res_m2 = (uint32_t)m2;
+            D.gen_res_m2 = (uint32_t)m2;
             D.res_r2_lo = (uint32_t)((unsigned long long)r2 & 0xFFFFFFFFull);
             D.res_r2_hi = (uint32_t)((unsigned long long)r2 >> 32);
-            // the fast pass takes the term as a single-precision product when that exists and its constant fits into
-            // every channel's rounding addend
-            ResidualForm form;
-            if (!cp.general) form = residual_form(L.res_mult, L.res_shift, L.zp_res, &res_c);
-            bool short_form = form.exists();
-            for (int oc = 0; oc < L.cout && short_form; ++oc) {
-                const int sft = ML.shift[oc] - 1;
-                const long long add = sft >= 1 ? (1ll << (sft - 1)) + ((long long)L.zp_out - res_c) * (1ll << sft) : (1ll << 40);
-                short_form = add > -(1ll << 31) && add < (1ll << 31);
-            }
-            if (short_form) {
-                D.flags |= CF_RSHORT;
-                D.res_m2 = form.m_bits;
-                D.res_r2_lo = form.k8;
-                D.res_r2_hi = 0;
-            } else {
-                res_c = 0;
-            }
+            D.res_m2 = cp.res_form.m_bits;
+            D.res_k8 = cp.res_form.k8;
         }
         for (size_t k = 0; k < cp.kunits.size(); ++k) {
-            const long long a = (long long)D.a_base + cp.a_delta[k];
+            const long long a = (long long)a_base + cp.a_delta[k];
             if (a < 0 || (a & 15) || (cp.a_lbo[k] & 15u)) PLAN_FAIL(21);
             D.a_lo[k] = (uint32_t)(a >> 4) | ((cp.a_lbo[k] >> 4) << 16);
         }
@@ -1719,7 +1748,8 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
                 if (halves[hf] < 0) continue;
                 const ConvPlan::Unit &u = cp.units[(size_t)halves[hf]];
                 for (uint32_t n = 0; n < rows; ++n) {
-                    const int oc = (int)(n % (uint32_t)L.cout), blk = (int)(n / (uint32_t)L.cout);
+                    // columns of 16 in the order of the epilogue's fragments: column 8 h + 2 c + e is channel 4 c + 2 h + e
+                    const int col = (int)(n % (uint32_t)L.cout), oc = (col & ~15) | ((col & 6) << 1) | ((col & 8) >> 2) | (col & 1), blk = (int)(n / (uint32_t)L.cout);
                     const int r = cp.stacked ? 2 - blk : u.r;
                     const int tap = L.kh == 3 ? r * 3 + (u.s + 1) : 0;
                     for (int b = 0; b < 16; ++b) {
@@ -1731,21 +1761,18 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
                 }
             }
         }
-        bool any_shift_one = false;
         for (int oc = 0; oc < L.cout; ++oc) {
-            long long wsum = 0;
-            for (int q = 0; q < L.cin * taps; ++q) wsum += ML.w[(size_t)oc * L.cin * taps + q];
             const int sh = ML.shift[oc];
             if (sh < 1 || sh > 20) PLAN_FAIL(19);
-            const long long biasf = (long long)ML.bias[oc] - (long long)L.zp_in * wsum;
-            if (biasf < -(1ll << 31) || biasf >= (1ll << 31)) PLAN_FAIL(24);
             const int sft = sh - 1;
-            const int32_t addend = sft ? (int32_t)((1ll << (sft - 1)) + ((long long)L.zp_out - res_c) * (1ll << sft)) : L.zp_out;
-            int32_t cst[4] = {(int32_t)biasf, ML.mult[oc], addend, sft};
-            memcpy(&blob[c_rel[(size_t)c] + (size_t)oc * 16], cst, 16);
-            if (sft == 0) any_shift_one = true;
+            const int32_t cst[3] = {ML.mult[oc], sft ? (int32_t)((1ll << (sft - 1)) + ((long long)L.zp_out - cp.res_c) * (1ll << sft)) : L.zp_out, sft};
+            for (int q = 0; q < 3; ++q)
+                memcpy(&blob[c_rel[(size_t)c] + (size_t)(oc / 16) * kChunkConstBytes + (size_t)(oc % 16 / 4) * 48 + (size_t)q * 16 + (size_t)(oc % 4) * 4], &cst[q], 4);
+            if (sft == 0 && !cp.general) PLAN_FAIL(25);      // a shift of one puts the rounding half in the product's low word
         }
-        if (any_shift_one && !cp.general) PLAN_FAIL(25);      // a shift of one puts the rounding half in the product's low word
+        for (size_t v = 0; v < vecs[(size_t)c].size(); ++v)
+            if (vecs[(size_t)c][v].first >= 0)
+                memcpy(&blob[vec_rel[(size_t)c] + v * kVecBytes], &bias[(size_t)vecs[(size_t)c][v].first][(size_t)vecs[(size_t)c][v].second], kVecBytes);
         (*blob_offsets)[(size_t)c] = (uint32_t)blob_out->size();
         blob_out->insert(blob_out->end(), blob.begin(), blob.end());
         (*csrc_out)[(size_t)c].bytes_phase = w_bytes[(size_t)c] | ((uint32_t)ph << 24);
@@ -1812,7 +1839,8 @@ int line_plan_probe(const LayerIn *layers, int n_layers, int in_c, int in_h, int
             std::vector<uint32_t> blob_off;
             std::vector<PhaseEntry> ptab;
             std::vector<ConvSrc> csrc;
-            ok = build_plan(layers, n_layers, in_c, in_h, in_w, n_classes, chains, &plan, &blob, &blob_off, &ptab, &csrc, &bar_counts);
+            std::vector<int32_t> acc_init;
+            ok = build_plan(layers, n_layers, in_c, in_h, in_w, n_classes, chains, &plan, &blob, &blob_off, &ptab, &csrc, &bar_counts, &acc_init);
             if (ok) *smem_bytes = plan.smem_bytes;
             if (ok) break;
         }
@@ -1832,10 +1860,11 @@ int line_build(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_w
     std::vector<uint32_t> blob_off;
     std::vector<PhaseEntry> ptab;
     std::vector<ConvSrc> csrc;
+    std::vector<int32_t> acc_init;
     for (int chains : kOpChainTries) {
         plan = new LinePlan();
         blob.clear(); bar_counts.clear(); blob_off.clear(); ptab.clear(); csrc.clear();
-        if (build_plan(layers, n_layers, in_c, in_h, in_w, n_classes, chains, plan, &blob, &blob_off, &ptab, &csrc, &bar_counts)) break;
+        if (build_plan(layers, n_layers, in_c, in_h, in_w, n_classes, chains, plan, &blob, &blob_off, &ptab, &csrc, &bar_counts, &acc_init)) break;
         delete plan;
         plan = nullptr;
     }
@@ -1877,6 +1906,7 @@ int line_build(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_w
     up((void **)&plan->d_ptab, ptab.data(), ptab.size() * sizeof(PhaseEntry));
     up((void **)&plan->d_conv_src, csrc.data(), csrc.size() * sizeof(ConvSrc));
     up((void **)&plan->d_bar_counts, bar_counts.data(), bar_counts.size());
+    up((void **)&plan->d_acc_init, acc_init.data(), acc_init.size() * sizeof(int32_t));
     up((void **)&plan->d_fc_w, fcw.data(), fcw.size());
     up((void **)&plan->d_fc_c, fcc.data(), fcc.size() * sizeof(FcConst));
     int32_t zero = 0;
@@ -1891,6 +1921,7 @@ int line_build(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_w
     b.ptab = plan->d_ptab;
     b.conv_src = plan->d_conv_src;
     b.bar_counts = plan->d_bar_counts;
+    b.acc_init = plan->d_acc_init;
     b.n_bars = plan->n_bars;
     b.n_phases = plan->n_phases;
     b.n_conv = plan->n_conv;
@@ -1930,7 +1961,7 @@ void line_free(LinePlan *p)
 {
     if (!p) return;
     line_free_streams(p);
-    cudaFree(p->d_ptab); cudaFree(p->d_conv_src); cudaFree(p->d_bar_counts); cudaFree(p->d_blob); cudaFree(p->d_fc_w);
+    cudaFree(p->d_ptab); cudaFree(p->d_conv_src); cudaFree(p->d_bar_counts); cudaFree(p->d_acc_init); cudaFree(p->d_blob); cudaFree(p->d_fc_w);
     cudaFree(p->d_fc_c); cudaFree(p->d_err); cudaFree(p->d_phase_cycles); cudaFree(p->d_dump);
     delete p;
 }
