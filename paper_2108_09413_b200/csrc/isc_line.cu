@@ -70,8 +70,7 @@ constexpr int kMaxBars = 128;
 constexpr int kMaxLines = 32;               // output lines of one convolution
 constexpr int kCtrlBytes = 10240;
 constexpr int kMaxConv = 128;
-constexpr int kOpChains = 4;                // MMA chains of an operation at most
-constexpr int kOpChainTries[] = {kOpChains, 1};   // a record of merged chains may name more units than it has room for
+constexpr int kOpChainTries[] = {2, 1};     // MMA chains of an operation at most; a record of two may name more units than it has room for
 constexpr int kSmemLimit = 227 * 1024;
 constexpr int kTmemCols = 512;
 constexpr int kSideStreams = 8;             // concurrent launches when a launch does not fill the GPU
@@ -79,7 +78,7 @@ constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // 2 s per wait
 
 enum { PH_FILL = 0, PH_INPUT = 1, PH_CONV = 2, PH_TAIL = 3 };
 enum { ERR_NONE = 0, ERR_WAIT_DONE = 1, ERR_WAIT_WEIGHTS = 2, ERR_WAIT_READY = 3, ERR_WAIT_FULL = 4, ERR_WAIT_DRAIN = 5 };
-enum { CF_RES = 2, CF_SCATTER = 8, CF_GENERAL = 16 };         // CF_GENERAL: the pass that decides everything at run time
+enum { CF_PAIRED = 1, CF_RES = 2, CF_SCATTER = 8, CF_GENERAL = 16 };         // CF_PAIRED: chains over two lines; CF_GENERAL: the pass that decides everything at run time
 // OPF_WAIT_ALL: every unit of the previous convolution; OPF_WAITS / OPF_WAITS4: the record names counters to test (two /
 // four slots in use); bits 4-6: how many of them are distinct; bits 8-9: arrivals; bits 10-12: MMA chains
 enum { OPF_WAIT_ALL = 1, OPF_WAITS = 2, OPF_WAITS4 = 8 };
@@ -99,17 +98,20 @@ struct alignas(16) ConvSrc {
     uint32_t dep_first, dep_units, dep_mult, dep_local_uses;     // dep_local | dep_uses << 16
 };
 
-// MMA chains over up to kOpChains consecutive input lines in the form an issuing thread consumes: accumulator columns, what
-// to add to the operand descriptors' start addresses, and the barriers (as byte offsets, 0xFFFF = none) of its dependencies
-// and completions.
+// MMA chains over an input line, or over up to two consecutive pairs of lines (paired convolutions), in the form an issuing
+// thread consumes: accumulator columns, what to add to the operand descriptors' start addresses, and the barriers (as byte
+// offsets, 0xFFFF = none) of its dependencies and completions.
 struct alignas(16) LOp {
     uint32_t d_col;         // first accumulator column within the bank
-    uint32_t idesc;         // instruction descriptor (N = blocks * cout)
-    uint32_t a_add, b_add;  // 16-byte units: (input line + 1) * pitch, first weight block * block size
-    uint16_t wait[4];       // 8 * unit of the previous convolution that must be stored
+    uint32_t idesc;         // instruction descriptor (N = blocks * cout; paired: blocks = 0)
+    uint32_t a_add, b_add;  // 16-byte units: (input line + 1) * pitch, first weight block * block size; paired: kPairInner, or per K-step
+                            // k, at bit 7 k: output lines (3 bits), first weight block (2), first output line behind d_col's (2)
+    uint16_t wait[4];       // 4 * unit of the previous convolution that must be stored
     uint16_t commit[3];     // 8 * unit of this convolution whose accumulators are complete after the chain
     uint16_t flags;         // OPF_* | distinct waits << 4 | arrivals << 8 | chains << 10
 };
+// a pair of lines away from the tensor's edges: lines p - 1 .. p + 1, p - 1 .. p + 2, p .. p + 2
+constexpr uint32_t kPairInner = (3u | 0u << 3 | 0u << 5) | (4u | 0u << 3 | 0u << 5) << 7 | (3u | 0u << 3 | 1u << 5) << 14;
 static_assert(sizeof(LOp) == 32, "one operation is two 16-byte loads");
 
 // Head of every blob: first what an epilogue warp reads, then what only some need.
@@ -212,10 +214,17 @@ __device__ __forceinline__ void tmem_ld_frag_wait(int (&v)[8])
     asm volatile("tcgen05.wait::ld.sync.aligned;"
                  : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]) :: "memory");
 }
-// the same 16 columns of the 16 lanes take the value of their column; b: the values of this thread's four columns
-__device__ __forceinline__ void tmem_st_columns(uint32_t taddr, uint4 b)
+// 16 columns of all 32 lanes take the values at `vec` (shared memory), one per column.  (In fragment form, four values per
+// thread, the store's eight registers had to be copied together each time: 230 instead of 60 cycles of a pass of 1,050.)
+__device__ __forceinline__ void tmem_st_columns(uint32_t taddr, uint4 a, uint4 b, uint4 c, uint4 d)
 {
-    asm volatile("tcgen05.st.sync.aligned.16x256b.x2.b32 [%0], {%1,%2,%1,%2,%3,%4,%3,%4};" ::"r"(taddr), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w) : "memory");
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
+                 ::"r"(taddr), "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w),
+                   "r"(c.x), "r"(c.y), "r"(c.z), "r"(c.w), "r"(d.x), "r"(d.y), "r"(d.z), "r"(d.w) : "memory");
+}
+__device__ __forceinline__ void tmem_st_columns(uint32_t taddr, uint32_t vec)
+{
+    tmem_st_columns(taddr, ld_shared_v4(vec), ld_shared_v4(vec + 16u), ld_shared_v4(vec + 32u), ld_shared_v4(vec + 48u));
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ long long mad_wide_u(uint32_t a, uint32_t b, long long c)
@@ -336,8 +345,45 @@ __device__ __forceinline__ uint32_t ld_counter(uint32_t addr)
 // fields.  The counters an operation depends on are read together (unused slots repeat the first one) and compared
 // once; what the counters guard was made visible to the tensor cores' reads by the storing warp (proxy fence, then a
 // releasing add) and is read by MMAs that are issued only after the values have been seen.
+__device__ __forceinline__ bool op_wait(const Waiter &w, const PrevConv &prev, uint4 r1)
+{
+    const uint32_t fl = r1.w >> 16;
+    if (fl & OPF_WAIT_ALL) {
+        for (uint32_t l = 0; l < prev.n_lines; ++l)
+            if (!w.counter(prev.done_addr + 4 * l, prev.expected, ERR_WAIT_DONE)) return false;
+    }
+    if (fl & OPF_WAITS) {
+        const unsigned long long t0 = globaltimer();
+        for (int spin = 0;; ++spin) {
+            int32_t m = min((int32_t)(ld_counter(prev.done_addr + (r1.x & 0xFFFFu)) - prev.expected),
+                            (int32_t)(ld_counter(prev.done_addr + (r1.x >> 16)) - prev.expected));
+            if (fl & OPF_WAITS4)
+                m = min(m, min((int32_t)(ld_counter(prev.done_addr + (r1.y & 0xFFFFu)) - prev.expected),
+                               (int32_t)(ld_counter(prev.done_addr + (r1.y >> 16)) - prev.expected)));
+            if (m >= 0) break;
+            if ((spin & 63) == 63) {
+                if (Waiter::aborted()) return false;
+                if (globaltimer() - t0 > w.limit_ns) { w.fail(ERR_WAIT_DONE, prev.done_addr + (r1.x & 0xFFFFu), 0); return false; }
+            }
+        }
+    }
+    tc_fence_after();
+    return true;
+}
+__device__ __forceinline__ void op_commit(const IssueCtx &ic, uint4 r1)
+{
+    const uint32_t nc = (r1.w >> 24) & 3u;
+    if (nc) {
+        commit_to(ic.full_addr + (r1.z & 0xFFFFu));
+        if (nc > 1) {
+            commit_to(ic.full_addr + (r1.z >> 16));
+            if (nc > 2) commit_to(ic.full_addr + (r1.w & 0xFFFFu));
+        }
+    }
+}
+
 template <int KS>
-__device__ __forceinline__ bool issue_ops(Waiter w, const IssueCtx &ic, const PrevConv &prev, uint32_t n_ksteps)
+__device__ __forceinline__ bool issue_ops(const Waiter &w, const IssueCtx &ic, const PrevConv &prev, uint32_t n_ksteps)
 {
     constexpr int NK = KS > 0 ? KS : 1;
     uint32_t alo[NK], blo[NK];
@@ -360,69 +406,59 @@ __device__ __forceinline__ bool issue_ops(Waiter w, const IssueCtx &ic, const Pr
         const uint4 r0 = n0, r1 = n1;         // d_col, idesc, a_add, b_add | wait 0-1, wait 2-3, commit 0-1, commit 2 and flags
         at += 32u * kIssuers;
         n0 = ld_shared_v4(at); n1 = ld_shared_v4(at + 16);
-        const uint32_t fl = r1.w >> 16;
-        // units of the previous convolution this operation depends on
-        if (fl & (OPF_WAIT_ALL | OPF_WAITS)) {
-            if (fl & OPF_WAIT_ALL) {
-                for (uint32_t l = 0; l < prev.n_lines; ++l)
-                    if (!w.counter(prev.done_addr + 4 * l, prev.expected, ERR_WAIT_DONE)) return false;
-            }
-            if (fl & OPF_WAITS) {
-                const unsigned long long t0 = globaltimer();
-                for (int spin = 0;; ++spin) {
-                    int32_t m = min((int32_t)(ld_counter(prev.done_addr + (r1.x & 0xFFFFu)) - prev.expected),
-                                    (int32_t)(ld_counter(prev.done_addr + (r1.x >> 16)) - prev.expected));
-                    if (fl & OPF_WAITS4)
-                        m = min(m, min((int32_t)(ld_counter(prev.done_addr + (r1.y & 0xFFFFu)) - prev.expected),
-                                       (int32_t)(ld_counter(prev.done_addr + (r1.y >> 16)) - prev.expected)));
-                    if (m >= 0) break;
-                    if ((spin & 63) == 63) {
-                        if (Waiter::aborted()) return false;
-                        if (globaltimer() - t0 > w.limit_ns) { w.fail(ERR_WAIT_DONE, prev.done_addr + (r1.x & 0xFFFFu), 0); return false; }
-                    }
-                }
-            }
-        }
-        tc_fence_after();
-        if (KS == 2) {
-            // chains over consecutive lines
-            const uint32_t n_chains = (fl >> 10) & 7u;        // 0: a record that only carries this thread's arrivals
-            uint32_t d = ic.d0 + r0.x, a_add = r0.z;
-            auto chain = [&]() {
-#pragma unroll
-                for (int k = 0; k < NK; ++k)
-                    mma_i8(d, ((uint64_t)ahi << 32) | (uint64_t)(alo[k] + a_add), ((uint64_t)bhi << 32) | (uint64_t)(blo[k] + r0.w), r0.y);
-                d += ic.cols;
-                a_add += ic.pitch16;
-            };
-            if (n_chains == kOpChains) {
-#pragma unroll
-                for (int c = 0; c < kOpChains; ++c) chain();
-            } else {
-                for (uint32_t c = 0; c < n_chains; ++c) chain();
-            }
-        } else if (!(fl & (7u << 10))) {
+        if (!op_wait(w, prev, r1)) return false;
+        const uint32_t d = ic.d0 + r0.x;
+        if (!(r1.w & (7u << 26))) {
             // a record that only carries this thread's arrivals on units it did not add to
         } else if (KS > 0) {
-            const uint32_t d = ic.d0 + r0.x;
 #pragma unroll
             for (int k = 0; k < NK; ++k)
                 mma_i8(d, ((uint64_t)ahi << 32) | (uint64_t)(alo[k] + r0.z), ((uint64_t)bhi << 32) | (uint64_t)(blo[k] + r0.w), r0.y);
         } else {
-            const uint32_t d = ic.d0 + r0.x;
             for (uint32_t k = 0; k < n_ksteps; ++k) {
                 const uint32_t a_lo = lds32(ic.desc + offsetof(LConvDesc, a_lo) + 4 * k) + ic.s16;
                 mma_i8(d, ((uint64_t)ahi << 32) | (uint64_t)(a_lo + r0.z), ((uint64_t)bhi << 32) | (uint64_t)(ic.b_lo0 + ic.s16 + k * ic.kstep16 + r0.w), r0.y);
             }
         }
-        const uint32_t nc = (fl >> 8) & 3u;
-        if (nc) {
-            commit_to(ic.full_addr + (r1.z & 0xFFFFu));
-            if (nc > 1) {
-                commit_to(ic.full_addr + (r1.z >> 16));
-                if (nc > 2) commit_to(ic.full_addr + (r1.w & 0xFFFFu));
+        op_commit(ic, r1);
+    }
+    return true;
+}
+
+// The same for paired convolutions (see build_plan): three MMAs for two lines.
+__device__ __forceinline__ bool issue_pairs(const Waiter &w, const IssueCtx &ic, const PrevConv &prev)
+{
+    const uint32_t ahi = (uint32_t)(make_desc(0, 0, 128) >> 32), bhi = (uint32_t)(make_desc(0, 128, 256) >> 32);
+    const uint4 v = ld_shared_v4(ic.desc + offsetof(LConvDesc, a_lo));
+    const uint32_t alo[3] = {v.x + ic.s16, v.y + ic.s16, v.z + ic.s16}, c2 = 2u * ic.cols;
+    const uint32_t blo[3] = {ic.b_lo0 + ic.s16, ic.b_lo0 + ic.s16 + 3u * c2, ic.b_lo0 + ic.s16 + 7u * c2};
+    const uint32_t n1_bits = ic.cols >> 3 << 17;                        // N of one block in the instruction descriptor
+    uint32_t at = ic.ops + 32u * ic.issuer;
+    uint4 n0 = ld_shared_v4(at), n1 = ld_shared_v4(at + 16);
+    for (uint32_t i = ic.issuer; i < ic.n_ops; i += kIssuers) {
+        const uint4 r0 = n0, r1 = n1;
+        at += 32u * kIssuers;
+        n0 = ld_shared_v4(at); n1 = ld_shared_v4(at + 16);
+        if (!op_wait(w, prev, r1)) return false;
+        uint32_t d = ic.d0 + r0.x, a_add = r0.z;
+        const uint32_t n_pairs = (r1.w >> 26) & 7u;
+        if (r0.w == kPairInner) {
+            for (uint32_t q = 0; q < n_pairs; ++q) {
+                mma_i8(d, ((uint64_t)ahi << 32) | (uint64_t)(alo[0] + a_add), ((uint64_t)bhi << 32) | (uint64_t)blo[0], r0.y + 3u * n1_bits);
+                mma_i8(d, ((uint64_t)ahi << 32) | (uint64_t)(alo[1] + a_add), ((uint64_t)bhi << 32) | (uint64_t)blo[1], r0.y + 4u * n1_bits);
+                mma_i8(d + ic.cols, ((uint64_t)ahi << 32) | (uint64_t)(alo[2] + a_add), ((uint64_t)bhi << 32) | (uint64_t)blo[2], r0.y + 3u * n1_bits);
+                d += c2;
+                a_add += 2u * ic.pitch16;
+            }
+        } else if (n_pairs) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const uint32_t f = r0.w >> (7 * k);
+                mma_i8(d + ((f >> 5) & 3u) * ic.cols, ((uint64_t)ahi << 32) | (uint64_t)(alo[k] + a_add), ((uint64_t)bhi << 32) | (uint64_t)(blo[k] + ((f >> 3) & 3u) * c2),
+                       r0.y + (f & 7u) * n1_bits);
             }
         }
+        op_commit(ic, r1);
     }
     return true;
 }
@@ -475,9 +511,9 @@ __device__ __forceinline__ bool issuer_conv(const LineParams &p, uint32_t tmem, 
     ic.pitch16 = h3.z;
     ic.cols = h3.w;
     bool ok;
-    switch (h2.y) {
+    if (h0.x & CF_PAIRED) ok = issue_pairs(w, ic, prev);
+    else switch (h2.y) {
     case 1: ok = issue_ops<1>(w, ic, prev, 1); break;
-    case 2: ok = issue_ops<2>(w, ic, prev, 2); break;
     case 3: ok = issue_ops<3>(w, ic, prev, 3); break;
     case 5: ok = issue_ops<5>(w, ic, prev, 5); break;
     case 6: ok = issue_ops<6>(w, ic, prev, 6); break;
@@ -563,63 +599,69 @@ __device__ __forceinline__ bool epi_conv_fast(Waiter w, uint32_t tmem_lane, uint
     const uint32_t tmem0 = tmem_lane + h0.w, full = CTRL_ADDR(bars) + 8u * (h1.x + (use & 1u) * h2.x), done = CTRL_ADDR(stored) + 4u * h1.y;
     const uint32_t parity = (use >> 1) & 1u, word = lane & 3u, row0 = (warp & 3u) * 32u + (lane >> 2);
     const uint32_t out = the_base() + h2.w + (kScatter ? word * 4u : row0 * 16u + word * 4u), res = the_base() + h3.x + row0 * 16u + word * 4u;
-    const uint32_t vecs = desc + lds32(desc + offsetof(LConvDesc, vec_rel)) + word * 16u;
+    const uint32_t vecs = desc + lds32(desc + offsetof(LConvDesc, vec_rel));
     const uint32_t m2 = h3.y, k8 = h3.z, dup = h3.w;
     // The bands of a thread's rows: they differ in bits 3 and 4 of the position, of which a band number has bits 2 and 3 at
     // most.  Bit 0, 1: rows of even number have a band above, below; bit 2, 3: those of odd number.
     const uint32_t nb = lds32(desc + offsetof(LConvDesc, out_nb));
     uint32_t bands = 0;
+    // Stride 2 (see scatter_to): the rows of a thread are in one band, and steps of 8 positions go on by whole columns, so
+    // that the output line is worked out once per input line.
+    uint32_t sc_row = 0, sc_at = 0, sc_pitch = 0, sc_log = 0, sc_odd = 0;
+    if (kScatter) {
+        const uint4 g0 = ld_shared_v4(desc + offsetof(LConvDesc, out_plane)), g1 = ld_shared_v4(desc + offsetof(LConvDesc, in_logI));
+        const uint32_t log_i = g1.x, log_o = g0.w;
+        sc_pitch = g0.y;
+        sc_log = g0.z | log_i << 8 | log_o << 16;
+        sc_row = ((row0 & ((1u << log_i) - 1u)) >> 2) * (g1.y >> 1);
+        sc_at = (row0 >> (log_i + 1u) << log_o) + (row0 & 3u);
+        sc_odd = ((row0 >> log_i) & 1u) | (((row0 + 8u) >> log_i) & 1u) << 1;         // bit j: position row0 + 8 j (+ 16) is in an odd column
+    }
     if (!kScatter) {
         const uint32_t a = (row0 >> 2) & (nb - 1u), b = ((row0 >> 2) + 2u) & (nb - 1u);
         bands = (a >= 1u ? 1u : 0u) | (a + 1u < nb ? 2u : 0u) | (b >= 1u ? 4u : 0u) | (b + 1u < nb ? 8u : 0u);
     }
-    Scatter g;
-    if (kScatter) {
-        const uint4 g0 = ld_shared_v4(desc + offsetof(LConvDesc, out_plane)), g1 = ld_shared_v4(desc + offsetof(LConvDesc, in_logI));
-        g.pitch = g0.y; g.log_lines = g0.z; g.log_o = g0.w; g.log_i = g1.x; g.half_lines = g1.y >> 1;
-    }
-    const uint32_t rec_bytes = 32u * h0.z, rec_stop = desc + h2.z + rec_bytes * h0.y;
+    const uint32_t consts = desc + h2.y + word * 48u, rec_bytes = 32u * h0.z, rec_stop = desc + h2.z + rec_bytes * h0.y;
 #pragma unroll 1
     for (uint32_t rec = desc + h2.z + rec_bytes * (warp >> 2); rec < rec_stop; rec += rec_bytes * (kSets - 1)) {
         const uint32_t rec_end = rec + rec_bytes;
-        const uint32_t meta = lds32(rec), unit = meta & 0xFFu, ch = (meta >> 12) & 0xFu;
-        const ChanConsts k = ld_chan_consts(desc + h2.y + word * 48u + ch * kChunkConstBytes);
+        uint4 q0 = ld_shared_v4(rec), q1 = ld_shared_v4(rec + 16u);
+        const uint32_t unit = q0.x & 0xFFu;
+        const ChanConsts k = ld_chan_consts(consts + ((q0.x >> 12) & 0xFu) * kChunkConstBytes);
         const bool ok = w.barrier(full + 8u * unit, parity, ERR_WAIT_FULL);
         if (!__all_sync(0xffffffffu, ok)) return false;                 // aborted: every other wait falls through too
         tc_fence_after();
 #pragma unroll 1
-        for (; rec < rec_end; rec += 32u) {
-            const uint4 q0 = ld_shared_v4(rec), q1 = ld_shared_v4(rec + 16u);
+        for (;;) {
             // Four steps: two lines x two halves of 16 positions; the next step's accumulators are requested before this
             // step's arithmetic.  (All 32 accumulators at once left no registers for the addresses.)
             int acc[2][8];
             tmem_ld_frag(tmem0 + q0.z, acc[0]);
-            uint4 start;
 #pragma unroll
             for (int st = 0; st < 4; ++st) {
                 const int l = st >> 1, h = st & 1;
                 int (&v)[8] = acc[st & 1];
-                const uint32_t tcol = tmem0 + (l ? q0.w : q0.z) + (h ? 16u << 16 : 0u), to = out + (l ? q1.y : q1.x);
+                const uint32_t to = out + (l ? q1.y : q1.x);
                 const uint32_t from = res + (l ? q1.w : q1.z) + (uint32_t)h * 256u;
                 uint32_t r0 = 0, r1 = 0;
                 if (kResidual) { r0 = lds32(from) ^ 0x80808080u; r1 = lds32(from + 128u) ^ 0x80808080u; }
-                if (h == 0) start = ld_shared_v4(vecs + (l ? q0.x >> 26 : (q0.x >> 20) & 63u) * kVecBytes);
                 tmem_ld_frag_wait(v);
                 if (st < 3) tmem_ld_frag(tmem0 + (st == 0 ? q0.z + (16u << 16) : st == 1 ? q0.w : q0.w + (16u << 16)), acc[(st + 1) & 1]);
-                tmem_st_columns(tcol, start);
+                if (h == 1) tmem_st_columns(tmem0 + (l ? q0.w : q0.z), vecs + (l ? q0.x >> 26 : (q0.x >> 20) & 63u) * kVecBytes);
                 if (kScatter) {
+                    // q1 holds the chunk's plane here, not a line's offset
+                    const uint32_t lines = 1u << (sc_log & 0xFFu), row = ((q0.y >> (8 * l)) & 0xFFu) + sc_row, oline = row & (lines - 1u), oband = row >> (sc_log & 0xFFu);
+                    const uint32_t up = oline == 0u && oband >= 1u, dn = oline + 1u == lines && oband + 1u < nb;
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
-                        const uint32_t pos = row0 + 16u * (uint32_t)h + 8u * (uint32_t)j;
-                        if ((pos >> g.log_i) & 1u) continue;
+                        if ((sc_odd >> j) & 1u) continue;
                         const uint32_t o = requant4<false>(v[2 * j], v[2 * j + 1], v[2 * j + 4], v[2 * j + 5], k, 0u, 0u, 0u);
-                        uint32_t oline, oband;
-                        // q1 holds the chunk's plane here, not a line's offset
-                        const uint32_t at = to + scatter_to(g, pos, (q0.y >> (8 * l)) & 0xFFu, oline, oband);
+                        const uint32_t col = (uint32_t)(16 * h + 8 * j) >> (((sc_log >> 8) & 0xFFu) + 1u) << (sc_log >> 16);
+                        const uint32_t at = to + (oline * sc_pitch + sc_at + col + (oband << 2)) * 16u;
                         st_shared_u32(at, o);
                         if (dup) {
-                            st_shared_u32_if(at + dup, o, oline == 0u && oband >= 1u);
-                            st_shared_u32_if(at - dup, o, oline + 1u == (1u << g.log_lines) && oband + 1u < nb);
+                            st_shared_u32_if(at + dup, o, up);
+                            st_shared_u32_if(at - dup, o, dn);
                         }
                     }
                 } else {
@@ -639,6 +681,10 @@ __device__ __forceinline__ bool epi_conv_fast(Waiter w, uint32_t tmem_lane, uint
                     }
                 }
             }
+            rec += 32u;
+            if (rec == rec_end) break;
+            q0 = ld_shared_v4(rec);
+            q1 = ld_shared_v4(rec + 16u);
         }
         pass_done(done + 4u * unit, (int)lane);
     }
@@ -656,7 +702,7 @@ __device__ __forceinline__ bool epi_conv_general(Waiter w, uint32_t tmem_lane, u
     const uint4 gl = ld_shared_v4(desc + offsetof(LConvDesc, lo));
     const int lo = (int)gl.x;
     const long long r2 = (long long)(((unsigned long long)gl.z << 32) | gl.y);
-    const uint32_t nb = g1.z, vecs = desc + g1.w + word * 16u;
+    const uint32_t nb = g1.z, vecs = desc + g1.w;
     const Scatter g{g1.x, g1.y >> 1, g0.z, g0.w, g0.y};
 #pragma unroll 1
     for (uint32_t i = warp >> 2; i < h0.y; i += kSets) {
@@ -671,44 +717,44 @@ __device__ __forceinline__ bool epi_conv_general(Waiter w, uint32_t tmem_lane, u
         for (uint32_t l = 0; l < n; ++l) {
             const uint32_t tcol = l ? q0.w : q0.z, to = the_base() + h2.w + word * 4u + (l ? q1.y : q1.x), line = (q0.y >> (8u * l)) & 0xFFu;
             const uint32_t from = the_base() + h3.x + word * 4u + (l ? q1.w : q1.z), edges = q0.x >> (16u + 2u * l);
-            const uint4 start = ld_shared_v4(vecs + ((q0.x >> (20u + 6u * l)) & 63u) * kVecBytes);
-          for (uint32_t h = 0; h < 2; ++h) {
-            int a[8];
-            tmem_ld_frag(tmem0 + tcol + (h * 16u << 16), a);
-            tmem_ld_frag_wait(a);
-            tmem_st_columns(tmem0 + tcol + (h * 16u << 16), start);
+#pragma unroll 1
+            for (uint32_t h = 0; h < 2; ++h) {
+                int a[8];
+                tmem_ld_frag(tmem0 + tcol + (h * 16u << 16), a);
+                tmem_ld_frag_wait(a);
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                const uint32_t pos = row0 + 16u * h + 8u * (uint32_t)j;
-                const uint32_t rword = res ? lds32(from + pos * 16u) ^ 0x80808080u : 0u;
-                int y[4];
+                for (int j = 0; j < 2; ++j) {
+                    const uint32_t pos = row0 + 16u * h + 8u * (uint32_t)j;
+                    const uint32_t rword = res ? lds32(from + pos * 16u) ^ 0x80808080u : 0u;
+                    int y[4];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const long long prod = mul_wide(a[2 * j + (q & 1) + 4 * (q >> 1)], k.mult[q]);
-                    int v = k.s[q] ? (hi32(prod) + k.c[q]) >> k.s[q] : hi32(prod) + (int)((uint32_t)lo32(prod) >> 31) + k.c[q];
-                    if (res) v += hi32(mad_wide_u((rword >> (8 * q)) & 0xFFu, gl.w, r2));
-                    y[q] = max(v, lo);
-                }
-                const uint32_t o = pack4_sat(y[0], y[1], y[2], y[3]);
-                uint32_t at = to + pos * 16u, up, dn;
-                if (scatter) {
-                    if ((pos >> g.log_i) & 1u) continue;
-                    uint32_t oline, oband;
-                    at = to + scatter_to(g, pos, line, oline, oband);
-                    up = oline == 0u && oband >= 1u;
-                    dn = oline + 1u == (1u << g.log_lines) && oband + 1u < nb;
-                } else {
-                    const uint32_t band = (pos >> 2) & (nb - 1u);
-                    up = (edges & 1u) && band >= 1u;
-                    dn = (edges & 2u) && band + 1u < nb;
-                }
-                st_shared_u32(at, o);
-                if (dup) {
-                    st_shared_u32_if(at + dup, o, up);
-                    st_shared_u32_if(at - dup, o, dn);
+                    for (int q = 0; q < 4; ++q) {
+                        const long long prod = mul_wide(a[2 * j + (q & 1) + 4 * (q >> 1)], k.mult[q]);
+                        int v = k.s[q] ? (hi32(prod) + k.c[q]) >> k.s[q] : hi32(prod) + (int)((uint32_t)lo32(prod) >> 31) + k.c[q];
+                        if (res) v += hi32(mad_wide_u((rword >> (8 * q)) & 0xFFu, gl.w, r2));
+                        y[q] = max(v, lo);
+                    }
+                    const uint32_t o = pack4_sat(y[0], y[1], y[2], y[3]);
+                    uint32_t at = to + pos * 16u, up, dn;
+                    if (scatter) {
+                        if ((pos >> g.log_i) & 1u) continue;
+                        uint32_t oline, oband;
+                        at = to + scatter_to(g, pos, line, oline, oband);
+                        up = oline == 0u && oband >= 1u;
+                        dn = oline + 1u == (1u << g.log_lines) && oband + 1u < nb;
+                    } else {
+                        const uint32_t band = (pos >> 2) & (nb - 1u);
+                        up = (edges & 1u) && band >= 1u;
+                        dn = (edges & 2u) && band + 1u < nb;
+                    }
+                    st_shared_u32(at, o);
+                    if (dup) {
+                        st_shared_u32_if(at + dup, o, up);
+                        st_shared_u32_if(at - dup, o, dn);
+                    }
                 }
             }
-          }
+            tmem_st_columns(tmem0 + tcol, vecs + ((q0.x >> (20u + 6u * l)) & 63u) * kVecBytes);
         }
         pass_done(done + 4u * unit, (int)lane);
     }
@@ -970,9 +1016,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_line(const __grid_constant__ Li
     if (warp < kEpiWarps) {
         const uint32_t lanes = tmem + ((warp & 3u) * 32u << 16);
         for (uint32_t col = (warp >> 2) * 16u; col < (uint32_t)kTmemCols; col += kSets * 16u) {
-            const uint4 b = __ldg(reinterpret_cast<const uint4 *>(p.acc_init + col) + (lane & 3u));
-            tmem_st_columns(lanes + col, b);
-            tmem_st_columns(lanes + col + (16u << 16), b);
+            const uint4 *v = reinterpret_cast<const uint4 *>(p.acc_init + col);
+            tmem_st_columns(lanes + col, __ldg(v), __ldg(v + 1), __ldg(v + 2), __ldg(v + 3));
         }
         tmem_st_wait();
     }
@@ -1163,7 +1208,7 @@ namespace {
 struct ConvPlan {
     int layer = -1, phase = -1;
     int in_tensor = -1, out_tensor = -1;
-    bool stacked = false, scatter = false, general = false;
+    bool stacked = false, paired = false, scatter = false, general = false;
     ResidualForm res_form;              // of the residual term, and its constant
     int32_t res_c = 0;
     int recs_per_item = 1;              // records of the pass table per (unit, chunk)
@@ -1315,7 +1360,18 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
             const int dr = cp.stacked ? 0 : u.r - 1;
             return (long long)u.pl * in.plane_bytes + ((long long)dr * in.pitch + (long long)u.s * in.I) * 16;
         };
-        for (size_t a = 0; a < cp.units.size(); a += 2) {
+        // Three units (16 input channels): two lines share their odd ones.  The K-steps of lines p and p + 1 are (p: left, centre),
+        // (p: right, p + 1: left), (p + 1: centre, right); the middle one adds to four output lines, with zero weights where a line
+        // does not reach.  Three MMAs for two lines instead of four with half of every second one empty: stage 1 of a CIFAR
+        // ResNet takes 2,450 instead of 2,990 cycles of operand reads a convolution.
+        cp.paired = cp.stacked && cp.units.size() == 3 && in.n_lines % 2 == 0;
+        if (cp.paired) {
+            const long long u0 = unit_addr(cp.units[0]), u1 = unit_addr(cp.units[1]), u2 = unit_addr(cp.units[2]), pitch = (long long)in.pitch * 16;
+            cp.a_delta = {(int)u0, (int)u2, (int)(pitch + u1)};
+            cp.a_lbo = {(uint32_t)(u1 - u0), (uint32_t)(pitch + u0 - u2), (uint32_t)(u2 - u1)};
+            cp.kunits = {{0, 1}, {2, 0}, {1, 2}};
+        }
+        for (size_t a = 0; a < cp.units.size() && !cp.paired; a += 2) {
             if (a + 1 < cp.units.size()) {
                 const long long d = unit_addr(cp.units[a + 1]) - unit_addr(cp.units[a]);
                 if (d <= 0 || d >= (1 << 18)) PLAN_FAIL(10);
@@ -1347,7 +1403,23 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
         };
         struct ProtoOp { int a_line, b_block, n_blocks, d_line, n_chains; std::vector<int> need; std::vector<int> outs; int ready; };
         std::vector<ProtoOp> proto;
-        if (cp.stacked) {
+        if (cp.paired) {
+            for (int p = -1; p <= in.n_lines - 1; p += 2) {
+                ProtoOp o;
+                o.n_chains = 1;
+                o.a_line = p;
+                const int y_lo = std::max(p - 1, 0), y_hi = std::min(p + 2, in.n_lines - 1);
+                o.d_line = y_lo; o.n_blocks = 3;
+                const int y_hi0 = std::min(p + 1, in.n_lines - 1), y_lo2 = std::max(p, 0);
+                o.b_block = (y_hi0 - y_lo + 1) | (y_lo - (p - 1)) << 3 | ((y_hi - y_lo + 1) | (y_lo - (p - 1)) << 3) << 7 |
+                            ((y_hi - y_lo2 + 1) | (y_lo2 - p) << 3 | (y_lo2 - y_lo) << 5) << 14;
+                for (int y = y_lo; y <= y_hi; ++y) o.outs.push_back(y);
+                for (int l = p; l <= p + 1 && aligned; ++l)
+                    if (src_line(l) >= 0) o.need.push_back(src_line(l));
+                if (slots) for (int y = y_lo; y <= y_hi; ++y) o.need.push_back(y);
+                proto.push_back(o);
+            }
+        } else if (cp.stacked) {
             for (int p = -1; p <= in.n_lines; ++p) {
                 ProtoOp o;
                 o.n_chains = 1;
@@ -1378,16 +1450,14 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
             for (int l : o.need) o.ready = std::max(o.ready, prev_time(l));
         }
         std::stable_sort(proto.begin(), proto.end(), [](const ProtoOp &a, const ProtoOp &b) { return a.ready < b.ready; });
-        // In the long convolutions of two K-steps (stage 1 of a CIFAR ResNet: 34 chains of two MMAs) chains over consecutive
-        // lines with the same blocks make one operation: an issuing thread spends more on a record than on its MMAs
-        // (10,270 -> 9,390 cycles a convolution; ResNet-110 485.7 -> 459.8 us a round of 592 samples).  With three and more
-        // K-steps a chain is worth a record of its own.
-        if (cp.stacked && cp.kunits.size() == 2 && cp.m >= 16) {
+        // In long paired convolutions two consecutive pairs make one operation: an issuing thread spends as much on a record as on
+        // its MMAs.
+        if (cp.paired && cp.m >= 16) {
             std::vector<ProtoOp> merged;
             for (const ProtoOp &o : proto) {
                 ProtoOp *l = merged.empty() ? nullptr : &merged.back();
-                if (l && l->n_chains < op_chains && l->a_line + l->n_chains == o.a_line && l->d_line + l->n_chains == o.d_line &&
-                    l->n_blocks == o.n_blocks && l->b_block == o.b_block) {
+                if (l && l->n_chains < op_chains && l->a_line + 2 * l->n_chains == o.a_line && l->d_line + 2 * l->n_chains == o.d_line &&
+                    l->b_block == (int)kPairInner && o.b_block == (int)kPairInner) {
                     l->n_chains += 1;
                     l->ready = std::max(l->ready, o.ready);
                     for (int n : o.need) if (std::find(l->need.begin(), l->need.end(), n) == l->need.end()) l->need.push_back(n);
@@ -1498,9 +1568,10 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
             op.flags = (uint16_t)(o.n_chains << 10);
             op.d_col = (uint32_t)(o.d_line * cp.cols);
             const uint32_t a_fmt_bit = cp.in_tensor == 0 ? 0u : 1u;
-            op.idesc = (2u << 4) | (a_fmt_bit << 7) | (1u << 10) | ((uint32_t)((std::max(o.n_blocks, 1) * L.cout) >> 3) << 17) | ((128u >> 4) << 24);
+            op.idesc = (2u << 4) | (a_fmt_bit << 7) | (1u << 10) | ((128u >> 4) << 24);
+            if (!cp.paired) op.idesc |= (uint32_t)((std::max(o.n_blocks, 1) * L.cout) >> 3) << 17;
             op.a_add = (uint32_t)(o.a_line + 1) * (uint32_t)in.pitch;
-            op.b_add = (uint32_t)o.b_block * (uint32_t)L.cout * 2u;
+            op.b_add = cp.paired ? (uint32_t)o.b_block : (uint32_t)o.b_block * (uint32_t)L.cout * 2u;
             if (i < (size_t)kIssuers && wait_all) {
                 op.flags |= OPF_WAIT_ALL;
                 std::fill(waited[wi].begin(), waited[wi].end(), 1);
@@ -1600,11 +1671,13 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
                 if (at >= 64) PLAN_FAIL(26);
                 P.meta |= (uint32_t)at << (20 + 6 * q);
             }
+    // the columns of 16 are in the order of the epilogue's fragments: column 8 h + 2 c + e is channel 4 c + 2 h + e
+    auto channel_of = [](int col) { return (col & ~15) | ((col & 6) << 1) | ((col & 8) >> 2) | (col & 1); };
     acc_init_out->assign((size_t)kTmemCols, 0);
     for (int col = 0; col < kTmemCols; col += 16) {
         int first = 0;
         const int q = next_user(n_conv - 1, col, &first);
-        for (int b = 0; b < 16 && q >= 0; ++b) (*acc_init_out)[(size_t)col + b] = bias[(size_t)q][(size_t)first + b];
+        for (int b = 0; b < 16 && q >= 0; ++b) (*acc_init_out)[(size_t)col + b] = bias[(size_t)q][(size_t)channel_of(first + b)];
     }
     // ---- barriers: per class, one per output line for "accumulators complete" and one for "line stored"
     std::vector<int> class_full(class_lines.size()), class_done(class_lines.size());
@@ -1627,7 +1700,7 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
         ops_rel[(size_t)c] = at; at += ((uint32_t)cp.ops.size() + (uint32_t)kIssuers) * (uint32_t)sizeof(LOp);    // spare records: reads run one ahead
         passes_rel[(size_t)c] = at; at += (uint32_t)cp.passes.size() * (uint32_t)sizeof(LPass);
         at = (at + 127u) & ~127u;
-        w_rel[(size_t)c] = at; at += (uint32_t)cp.kunits.size() * rows * 32u;
+        w_rel[(size_t)c] = at; at += cp.paired ? 10u * (uint32_t)L.cout * 32u : (uint32_t)cp.kunits.size() * rows * 32u;
         c_rel[(size_t)c] = at; at += (uint32_t)(L.cout / 16) * kChunkConstBytes;
         vec_rel[(size_t)c] = at; at += (uint32_t)vecs[(size_t)c].size() * kVecBytes;
         w_bytes[(size_t)c] = (at + 127u) & ~127u;
@@ -1692,7 +1765,7 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
         std::vector<uint8_t> blob(w_bytes[(size_t)c], 0);
         LConvDesc D;
         memset(&D, 0, sizeof(D));
-        D.flags = (L.res_tensor >= 0 ? CF_RES : 0u) | (cp.scatter ? CF_SCATTER : 0u) | (cp.general ? CF_GENERAL : 0u);
+        D.flags = (L.res_tensor >= 0 ? CF_RES : 0u) | (cp.scatter ? CF_SCATTER : 0u) | (cp.general ? CF_GENERAL : 0u) | (cp.paired ? CF_PAIRED : 0u);
         D.n_items = (uint32_t)(cp.n_units * cp.n_chunks); D.recs_per_item = (uint32_t)cp.recs_per_item; D.d_base = (uint32_t)bank_base(c);
         D.bar_full = (uint32_t)class_full[(size_t)cp.cls]; D.bar_done = (uint32_t)class_done[(size_t)cp.cls];
         D.use_local = (uint32_t)cp.use_local; D.uses_per_group = (uint32_t)class_uses[(size_t)cp.cls];
@@ -1733,33 +1806,37 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
         for (size_t k = 0; k < cp.kunits.size(); ++k)
             for (const LOp &op : cp.ops) {
                 const long long lo_b = (long long)in.line0 - (long long)in.pitch * 16 + (long long)op.a_add * 16 + cp.a_delta[k];
-                const long long hi_b = lo_b + cp.a_lbo[k] + 128 * 16 + (long long)std::max(((op.flags >> 10) & 7) - 1, 0) * in.pitch * 16;
+                const long long hi_b = lo_b + cp.a_lbo[k] + 128 * 16 + (long long)std::max(((op.flags >> 10) & 7) - 1, 0) * 2 * in.pitch * 16;
                 if (lo_b < 0 || hi_b > (long long)in.bytes) PLAN_FAIL(18);
             }
         memcpy(blob.data(), &D, sizeof(D));
         memcpy(blob.data() + ops_rel[(size_t)c], cp.ops.data(), cp.ops.size() * sizeof(LOp));
         memcpy(blob.data() + passes_rel[(size_t)c], cp.passes.data(), cp.passes.size() * sizeof(LPass));
-        // weights: per K-step, rows = block * cout + oc (block b = vertical tap 2 - b when stacked)
+        // weights: per K-step, rows = block * cout + column; block b is vertical tap 2 - b when stacked, and 3 - b for the second
+        // line's unit of a pair's middle K-step
         const int taps = L.kh * L.kw;
-        const uint32_t rows = (uint32_t)(cp.stacked ? 3 : 1) * (uint32_t)L.cout;
+        size_t at_row = 0;
         for (size_t k = 0; k < cp.kunits.size(); ++k) {
+            const bool middle = cp.paired && k == 1;
+            const uint32_t rows = (uint32_t)(middle ? 4 : cp.stacked ? 3 : 1) * (uint32_t)L.cout;
             const int halves[2] = {cp.kunits[k].first, cp.kunits[k].second};
             for (int hf = 0; hf < 2; ++hf) {
                 if (halves[hf] < 0) continue;
                 const ConvPlan::Unit &u = cp.units[(size_t)halves[hf]];
                 for (uint32_t n = 0; n < rows; ++n) {
-                    // columns of 16 in the order of the epilogue's fragments: column 8 h + 2 c + e is channel 4 c + 2 h + e
-                    const int col = (int)(n % (uint32_t)L.cout), oc = (col & ~15) | ((col & 6) << 1) | ((col & 8) >> 2) | (col & 1), blk = (int)(n / (uint32_t)L.cout);
-                    const int r = cp.stacked ? 2 - blk : u.r;
+                    const int oc = channel_of((int)(n % (uint32_t)L.cout)), blk = (int)(n / (uint32_t)L.cout);
+                    const int r = !cp.stacked ? u.r : middle && hf == 1 ? 3 - blk : 2 - blk;
+                    if (r < 0 || r > 2) continue;
                     const int tap = L.kh == 3 ? r * 3 + (u.s + 1) : 0;
                     for (int b = 0; b < 16; ++b) {
                         const int ci = u.pl * 16 + b;
                         if (ci >= L.cin) continue;
                         const int8_t wv = ML.w[((size_t)oc * L.cin + ci) * taps + tap];
-                        blob[w_rel[(size_t)c] + k * rows * 32 + (size_t)(n / 8) * 256 + (size_t)hf * 128 + (size_t)(n % 8) * 16 + b] = (uint8_t)wv;
+                        blob[w_rel[(size_t)c] + (at_row + n / 8 * 8) * 32 + (size_t)hf * 128 + (size_t)(n % 8) * 16 + b] = (uint8_t)wv;
                     }
                 }
             }
+            at_row += rows;
         }
         for (int oc = 0; oc < L.cout; ++oc) {
             const int sh = ML.shift[oc];
@@ -1771,8 +1848,8 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
             if (sft == 0 && !cp.general) PLAN_FAIL(25);      // a shift of one puts the rounding half in the product's low word
         }
         for (size_t v = 0; v < vecs[(size_t)c].size(); ++v)
-            if (vecs[(size_t)c][v].first >= 0)
-                memcpy(&blob[vec_rel[(size_t)c] + v * kVecBytes], &bias[(size_t)vecs[(size_t)c][v].first][(size_t)vecs[(size_t)c][v].second], kVecBytes);
+            for (int b = 0; b < 16 && vecs[(size_t)c][v].first >= 0; ++b)
+                memcpy(&blob[vec_rel[(size_t)c] + v * kVecBytes + (size_t)b * 4], &bias[(size_t)vecs[(size_t)c][v].first][(size_t)channel_of(vecs[(size_t)c][v].second + b)], 4);
         (*blob_offsets)[(size_t)c] = (uint32_t)blob_out->size();
         blob_out->insert(blob_out->end(), blob.begin(), blob.end());
         (*csrc_out)[(size_t)c].bytes_phase = w_bytes[(size_t)c] | ((uint32_t)ph << 24);
