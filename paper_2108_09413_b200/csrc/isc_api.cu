@@ -441,14 +441,16 @@ int ready_tensor_cores(isc_model *m)
 }
 
 // Layer-by-layer forward of `batch` samples in the activation buffers `bufs`; leaves the logits in the last tensor's.
+// `chained`: the stream's last operation is a kernel of such a forward too (see launch_chained).
 int generic_forward(isc_model *m, int8_t *const *bufs, const uint8_t *d_x, const NoiseStream &ns, int batch, cudaStream_t st, int32_t *d_err,
-                    int stop_after_layer = -1, bool tensor_cores = false)
+                    int stop_after_layer = -1, bool tensor_cores = false, bool chained = false)
 {
     const int n = (int)m->glayers.size();
     if (tensor_cores) {
         int rc = ready_tensor_cores(m);
         if (rc) return rc;
     }
+    const bool follows = tensor_cores && m->tc.chained;
     for (int i = 0; i < n; ++i) {
         const GLayer &G = m->glayers[(size_t)i];
         const isc_layer &L = m->layers[(size_t)i].d;
@@ -457,14 +459,14 @@ int generic_forward(isc_model *m, int8_t *const *bufs, const uint8_t *d_x, const
         const int8_t *res = L.res_tensor >= 0 ? bufs[m->tensor_buf[(size_t)L.res_tensor]] : nullptr;
         cudaError_t e;
         if (i == 0 && tensor_cores && m->wpacks[0])
-            e = launch_stem_conv(G, m->wpacks[0], m->tc_cst[0], m->tc_fast[0] != 0, d_x, m->in_c, ns, batch, out, d_err, st);
+            e = launch_stem_conv(G, m->wpacks[0], m->tc_cst[0], m->tc_fast[0] != 0, d_x, m->in_c, ns, batch, out, d_err, st, false, chained && m->tc.chained);
         else if (i == 0) e = launch_first_conv(G, d_x, m->in_c, ns, batch, out, st);
         else if (tensor_cores && m->hpacks[(size_t)i] && halo_offsets_fit(G, batch))
             e = launch_halo_conv(m->tc, G, m->hpacks[(size_t)i], m->tc_cst[(size_t)i], m->tc_fast[(size_t)i] != 0, m->tc_resk[(size_t)i], batch, in, res, out, d_err, st);
         else if (tensor_cores && m->wpacks[(size_t)i] && conv_offsets_fit(G, batch)) e = launch_igemm_conv(m->tc, G, m->wpacks[(size_t)i], m->tc_cst[(size_t)i], m->tc_fast[(size_t)i] != 0, m->tc_resk[(size_t)i], batch, in, res, out, d_err, st, false, m->opt_tensor_copy != 0);
-        else if (L.op == ISC_CONV2D || L.op == ISC_FC) e = launch_conv(G, batch, in, res, out, st);
-        else if (L.op == ISC_GAVGPOOL) e = launch_gavgpool(G, batch, in, out, st);
-        else e = launch_maxpool(G, batch, in, out, st);
+        else if (L.op == ISC_CONV2D || L.op == ISC_FC) e = launch_conv(G, batch, in, res, out, st, follows);
+        else if (L.op == ISC_GAVGPOOL) e = launch_gavgpool(G, batch, in, out, st, follows);
+        else e = launch_maxpool(G, batch, in, out, st, follows);
         m->launches += 1;
         if (e != cudaSuccess) {
             if (getenv("ISC_DEBUG_CUDA")) fprintf(stderr, "isc: layer %d launch: %s\n", i, cudaGetErrorString(e));
@@ -490,11 +492,11 @@ int forward_counts(isc_model *m, int8_t *const *bufs, int64_t cap, bool tensor_c
     const int last = (int)m->glayers.size();
     for (int64_t done = 0; done < n; done += cap) {
         const int b = (int)std::min<int64_t>(cap, n - done);
-        int rc = generic_forward(m, bufs, d_x, ns, b, st, d_err, -1, tensor_cores);
+        int rc = generic_forward(m, bufs, d_x, ns, b, st, d_err, -1, tensor_cores, done > 0);
         if (rc) return rc;
         ns.first_sample += b;
         cudaError_t e = launch_votes(bufs[m->tensor_buf[(size_t)last]], m->shapes[(size_t)last].cp, m->n_classes, b, d_counts,
-                                     d_logits ? d_logits + (size_t)done * m->n_classes : nullptr, st);
+                                     d_logits ? d_logits + (size_t)done * m->n_classes : nullptr, st, tensor_cores && m->tc.chained);
         m->launches += 1;
         if (e != cudaSuccess) return ISC_ERR_CUDA;
     }

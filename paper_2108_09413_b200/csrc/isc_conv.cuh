@@ -54,6 +54,31 @@ struct FastDiv {
     }
 };
 
+// The layers of a network as a chain of launches: a kernel may start when every block of the one before has started and
+// leaves it room, sets itself up (barriers, tensor memory, constants; the stem also draws its noise), and waits for the end
+// of the one before (chain_wait: complete, and its results visible) before it touches an activation.  Every kernel of a
+// chain waits in every block, so the end of one is the end of all before it.  ResNet-50 at 100 samples, 57 launches: 1,753 ->
+// 1,598 us; 4096 samples of a 20-layer network of 32 to 128 channels twice over: 2,961 -> 2,794 us.
+__device__ __forceinline__ void chain_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <typename... Params, typename... Args>
+cudaError_t launch_chained(bool chained, void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, const Args &...args)
+{
+    if (!chained) {
+        kernel<<<grid, threads, smem, st>>>(args...);
+        return cudaGetLastError();
+    }
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cfg.attrs = &attr; cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
+}
+
 // 16 accumulators -> 16 int8 outputs with 32-bit arithmetic.  With s = shift - 1 >= 1,
 //   rs((acc + bias) * mult, 31 + shift) + zp_out = (hi32((acc + bias) * mult) + c) >> s,  c = 2^(s-1) + zp_out * 2^s,
 // exactly (the rounding half 2^(31+s) is a multiple of 2^32, so the product's low word cannot change the floor), and

@@ -78,6 +78,8 @@ k_first_conv(GLayer L, const uint8_t *__restrict__ x, int in_c, NoiseStream ns, 
              int8_t *__restrict__ out)
 {
     extern __shared__ uint32_t patch[];   // [rows_in][wpad] packed 4 channels
+    conv::chain_start();
+    conv::chain_wait();
     const int b = blockIdx.y;
     const int64_t j = ns.first_sample + b;
     const int oy0 = blockIdx.x * band_rows;
@@ -165,6 +167,8 @@ __global__ void __launch_bounds__(128)
 k_conv(GLayer L, int batch, const int8_t *__restrict__ in, const int8_t *__restrict__ res,
        int8_t *__restrict__ out)
 {
+    conv::chain_start();
+    conv::chain_wait();
     const int64_t npx = (int64_t)batch * L.hout * L.wout;
     const int64_t px = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (px >= npx) return;
@@ -213,6 +217,8 @@ k_conv(GLayer L, int batch, const int8_t *__restrict__ in, const int8_t *__restr
 
 __global__ void k_gavgpool(GLayer L, int batch, const int8_t *__restrict__ in, int8_t *__restrict__ out)
 {
+    conv::chain_start();
+    conv::chain_wait();
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= batch * L.cinp) return;
     const int b = idx / L.cinp, c = idx - b * L.cinp;
@@ -241,6 +247,8 @@ __global__ void k_gavgpool(GLayer L, int batch, const int8_t *__restrict__ in, i
 template <int K>
 __global__ void k_maxpool(GLayer L, conv::FastDiv by_c16, conv::FastDiv by_w, uint32_t n, const int8_t *__restrict__ in, int8_t *__restrict__ out)
 {
+    conv::chain_start();
+    conv::chain_wait();
     const uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= n) return;
     uint32_t g, ox;
@@ -288,7 +296,9 @@ __global__ void k_votes(const int8_t *__restrict__ logits, int cp, int n_classes
                         int32_t *__restrict__ counts, int8_t *__restrict__ logits_out)
 {
     extern __shared__ int32_t hist[];
+    conv::chain_start();
     for (int i = threadIdx.x; i < n_classes; i += blockDim.x) hist[i] = 0;
+    conv::chain_wait();
     __syncthreads();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b < batch) {
@@ -334,22 +344,20 @@ cudaError_t launch_noisy_input(const uint8_t *x_chw, int in_c, int in_h, int in_
 }
 
 cudaError_t launch_conv(const GLayer &L, int batch, const int8_t *in, const int8_t *res, int8_t *out,
-                        cudaStream_t st)
+                        cudaStream_t st, bool chained)
 {
     const int64_t npx = (int64_t)batch * L.hout * L.wout;
     dim3 grid((unsigned)((npx + 127) / 128), L.coutp >> 4);
-    k_conv<<<grid, 128, 0, st>>>(L, batch, in, res, out);
-    return cudaGetLastError();
+    return conv::launch_chained(chained, k_conv, grid, 128, 0, st, L, batch, in, res, out);
 }
 
-cudaError_t launch_gavgpool(const GLayer &L, int batch, const int8_t *in, int8_t *out, cudaStream_t st)
+cudaError_t launch_gavgpool(const GLayer &L, int batch, const int8_t *in, int8_t *out, cudaStream_t st, bool chained)
 {
     const int n = batch * L.cinp;
-    k_gavgpool<<<(n + 127) / 128, 128, 0, st>>>(L, batch, in, out);
-    return cudaGetLastError();
+    return conv::launch_chained(chained, k_gavgpool, dim3((unsigned)((n + 127) / 128)), 128, 0, st, L, batch, in, out);
 }
 
-cudaError_t launch_maxpool(const GLayer &L, int batch, const int8_t *in, int8_t *out, cudaStream_t st)
+cudaError_t launch_maxpool(const GLayer &L, int batch, const int8_t *in, int8_t *out, cudaStream_t st, bool chained)
 {
     const uint32_t n = (uint32_t)(L.hout * L.wout * (L.cinp >> 4));
     const conv::FastDiv by_c16 = conv::FastDiv::make((uint32_t)(L.cinp >> 4)), by_w = conv::FastDiv::make((uint32_t)L.wout);
@@ -357,18 +365,17 @@ cudaError_t launch_maxpool(const GLayer &L, int batch, const int8_t *in, int8_t 
         const dim3 grid((n + 127) / 128, (unsigned)std::min(batch - b, 65535));
         const int8_t *src = in + (size_t)b * L.hin * L.win * L.cinp;
         int8_t *dst = out + (size_t)b * L.hout * L.wout * L.cinp;
-        if (L.kh == 3 && L.kw == 3) k_maxpool<3><<<grid, 128, 0, st>>>(L, by_c16, by_w, n, src, dst);
-        else k_maxpool<0><<<grid, 128, 0, st>>>(L, by_c16, by_w, n, src, dst);
+        const cudaError_t e = conv::launch_chained(chained, L.kh == 3 && L.kw == 3 ? k_maxpool<3> : k_maxpool<0>, grid, 128, 0, st, L, by_c16, by_w, n, src, dst);
+        if (e != cudaSuccess) return e;
     }
-    return cudaGetLastError();
+    return cudaSuccess;
 }
 
 cudaError_t launch_votes(const int8_t *logits_nhwc, int cp, int n_classes, int batch, int32_t *counts,
-                         int8_t *logits_out, cudaStream_t st)
+                         int8_t *logits_out, cudaStream_t st, bool chained)
 {
-    k_votes<<<(batch + 127) / 128, 128, n_classes * sizeof(int32_t), st>>>(logits_nhwc, cp, n_classes, batch,
-                                                                          counts, logits_out);
-    return cudaGetLastError();
+    return conv::launch_chained(chained, k_votes, dim3((unsigned)((batch + 127) / 128)), 128, n_classes * sizeof(int32_t), st, logits_nhwc, cp, n_classes, batch,
+                                counts, logits_out);
 }
 
 }  // namespace isc

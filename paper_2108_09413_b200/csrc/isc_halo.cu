@@ -281,6 +281,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_halo(const __grid_constant__ Ha
     __shared__ unsigned long long bar_a_full[kMaxRing], bar_a_free[kMaxRing], bar_b_full[kMaxRing], bar_b_free[kMaxRing], bar_acc_full[4], bar_acc_free[4];
     __shared__ uint32_t tmem_base_s;
     __shared__ volatile int abort_s;
+    chain_start();
     const GLayer &L = p.L;
     const int tid = threadIdx.x, warp = (int)warp_uniform((uint32_t)tid >> 5), lane = tid & 31;
     const uint32_t sbase = smem_u32(smem);
@@ -301,6 +302,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_halo(const __grid_constant__ Ha
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_base_s;
+    chain_wait();
     const uint32_t block_bytes = (uint32_t)(p.n_tile * L.kh) * 32u;
     const uint2 a_bars = make_uint2(smem_u32(&bar_a_full[0]), smem_u32(&bar_a_free[0])), b_bars = make_uint2(smem_u32(&bar_b_full[0]), smem_u32(&bar_b_free[0])),
                 acc_bars = make_uint2(smem_u32(&bar_acc_full[0]), smem_u32(&bar_acc_free[0]));
@@ -596,8 +598,7 @@ cudaError_t launch_halo_conv(const TcDevice &dev, const GLayer &G, const int8_t 
     }
     p.debug_stall = debug_stall ? 1 : 0;
     p.err = err;
-    k_halo<<<std::min<uint32_t>(p.n_items, (uint32_t)dev.n_sms), kThreads, c.smem, st>>>(p);
-    return cudaGetLastError();
+    return launch_chained(dev.chained, k_halo, dim3(std::min<uint32_t>(p.n_items, (uint32_t)dev.n_sms)), kThreads, c.smem, st, p);
 }
 
 }  // namespace isc

@@ -320,6 +320,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_igemm(const __grid_constant
     __shared__ unsigned long long bar_full[kMaxStages], bar_free[kMaxStages], bar_acc_full[2], bar_acc_free[2];
     __shared__ uint32_t tmem_base_s;
     __shared__ volatile int abort_s;
+    chain_start();
     const GLayer &L = p.L;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t sbase = smem_u32(smem);
@@ -340,6 +341,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_igemm(const __grid_constant
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_base_s;
+    chain_wait();
 
     // tiles in m-major order (the CTAs of one wave share operand rows in L2), dealt round-robin to the CTAs
     const int tiles_n = p.tiles_n;
@@ -601,6 +603,7 @@ __global__ void __launch_bounds__(kStemThreads, 2) k_stem(const __grid_constant_
     __shared__ uint32_t tmem_base_s;
     __shared__ volatile int abort_s;
     __shared__ __align__(16) int4 cst_s[256];
+    chain_start();
     const GLayer &L = p.L;
     const int tid = threadIdx.x, warp = (int)warp_uniform((uint32_t)tid >> 5);
     const uint32_t sbase = smem_u32(smem);
@@ -697,6 +700,7 @@ __global__ void __launch_bounds__(kStemThreads, 2) k_stem(const __grid_constant_
     fence_proxy_async();
     __syncthreads();
 
+    chain_wait();                                         // the noise needed nothing of the launch before; the output buffer does
     const int band_rows = oy1 - oy0, n_tiles = (band_rows * p.pitch + 2 * kTileM - 1) / (2 * kTileM);
     bool ok = true;
     if (warp < kStemEpi) {
@@ -924,6 +928,8 @@ cudaError_t tc_prepare(TcDevice *dev, int ordinal)
 {
     TcDevice d;
     d.ordinal = ordinal;
+    int major = 0;
+    d.chained = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, ordinal) == cudaSuccess && major >= 9;
     cudaError_t e = cudaDeviceGetAttribute(&d.n_sms, cudaDevAttrMultiProcessorCount, ordinal);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
@@ -1002,10 +1008,7 @@ cudaError_t launch_igemm_conv(const TcDevice &dev, const GLayer &G, const int8_t
     const uint32_t n_tiles = p.tiles_m * (uint32_t)p.tiles_n;
     const unsigned grid = std::min<uint32_t>(n_tiles, (uint32_t)dev.n_sms);
     const bool whole = G.cinp % kBlockK == 0 && p.n_tile % 64 == 0 && G.coutp == p.tiles_n * p.n_tile;
-    if (paired) k_igemm<true, true><<<grid, kGemmThreads, smem, st>>>(p);
-    else if (whole) k_igemm<true, false><<<grid, kGemmThreads, smem, st>>>(p);
-    else k_igemm<false, false><<<grid, kGemmThreads, smem, st>>>(p);
-    return cudaGetLastError();
+    return launch_chained(dev.chained, paired ? k_igemm<true, true> : whole ? k_igemm<true, false> : k_igemm<false, false>, dim3(grid), kGemmThreads, smem, st, p);
 }
 
 // ---- the stem
@@ -1067,7 +1070,7 @@ void stem_pack_weights(const GLayer &G, const int8_t *w, int8_t *out)
 }
 
 cudaError_t launch_stem_conv(const GLayer &G, const int8_t *wpack, const int32_t *cst, bool fast, const uint8_t *x_chw, int in_c,
-                             const NoiseStream &ns, int batch, int8_t *out, int32_t *err, cudaStream_t st, bool debug_stall)
+                             const NoiseStream &ns, int batch, int8_t *out, int32_t *err, cudaStream_t st, bool debug_stall, bool chained)
 {
     StemParams p;
     p.L = G;
@@ -1099,8 +1102,7 @@ cudaError_t launch_stem_conv(const GLayer &G, const int8_t *wpack, const int32_t
     }
     if (batch <= 0) return cudaSuccess;
     dim3 grid((unsigned)p.n_bands, (unsigned)batch);
-    k_stem<<<grid, kStemThreads, smem, st>>>(p);
-    return cudaGetLastError();
+    return launch_chained(chained, k_stem, grid, kStemThreads, smem, st, p);
 }
 
 }  // namespace isc

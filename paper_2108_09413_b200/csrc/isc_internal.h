@@ -59,11 +59,11 @@ cudaError_t launch_first_conv(const GLayer &L, const uint8_t *x_chw, int in_c, c
 cudaError_t launch_noisy_input(const uint8_t *x_chw, int in_c, int in_h, int in_w, const NoiseStream &ns,
                                int batch, int32_t *out_chw, cudaStream_t st);
 cudaError_t launch_conv(const GLayer &L, int batch, const int8_t *in, const int8_t *res, int8_t *out,
-                        cudaStream_t st);
-cudaError_t launch_gavgpool(const GLayer &L, int batch, const int8_t *in, int8_t *out, cudaStream_t st);
-cudaError_t launch_maxpool(const GLayer &L, int batch, const int8_t *in, int8_t *out, cudaStream_t st);
+                        cudaStream_t st, bool chained = false);
+cudaError_t launch_gavgpool(const GLayer &L, int batch, const int8_t *in, int8_t *out, cudaStream_t st, bool chained = false);
+cudaError_t launch_maxpool(const GLayer &L, int batch, const int8_t *in, int8_t *out, cudaStream_t st, bool chained = false);
 cudaError_t launch_votes(const int8_t *logits_nhwc, int cp, int n_classes, int batch, int32_t *counts,
-                         int8_t *logits_out, cudaStream_t st);
+                         int8_t *logits_out, cudaStream_t st, bool chained = false);
 
 // ---- layer-by-layer tensor-core convolutions (isc_igemm.cu) ----
 // What their launches need of the current device.  A handle keeps its own (calls on one handle do not overlap, so nothing
@@ -71,6 +71,7 @@ cudaError_t launch_votes(const int8_t *logits_nhwc, int cp, int n_classes, int b
 // are a property of each device.
 struct TcDevice {
     int ordinal = -1, n_sms = 0;
+    bool chained = false;     // layers may be launched ahead of the end of the one before (see launch_chained)
     void *encode = nullptr;   // the driver's cuTensorMapEncodeTiled, or null
 };
 cudaError_t tc_prepare(TcDevice *dev, int ordinal);
@@ -120,7 +121,7 @@ bool stem_fits(const GLayer &G, int in_c);
 size_t stem_pack_bytes(const GLayer &G);
 void stem_pack_weights(const GLayer &G, const int8_t *w_oihw, int8_t *out);
 cudaError_t launch_stem_conv(const GLayer &G, const int8_t *wpack, const int32_t *cst, bool fast, const uint8_t *x_chw, int in_c,
-                             const NoiseStream &ns, int batch, int8_t *out, int32_t *err, cudaStream_t st, bool debug_stall = false);
+                             const NoiseStream &ns, int batch, int8_t *out, int32_t *err, cudaStream_t st, bool debug_stall = false, bool chained = false);
 
 // ---- host decision rules (isc_decide.cpp) ----
 double lower_conf_bound(int64_t k, int64_t n, double alpha);
