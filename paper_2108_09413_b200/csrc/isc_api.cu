@@ -441,8 +441,8 @@ int ready_tensor_cores(isc_model *m)
 }
 
 // Layer-by-layer forward of `batch` samples in the activation buffers `bufs`; leaves the logits in the last tensor's.
-// `chained`: the stream's last operation is a kernel of such a forward too (see launch_chained).
-int generic_forward(isc_model *m, int8_t *const *bufs, const uint8_t *d_x, const NoiseStream &ns, int batch, cudaStream_t st, int32_t *d_err,
+// run: what the samples are (`ns`: only the seed and the tables).  `chained`: the stream's last operation is a kernel of such a forward too (see launch_chained).
+int generic_forward(isc_model *m, int8_t *const *bufs, const uint8_t *d_x, const NoiseStream &ns, const SampleRun &run, int batch, cudaStream_t st, int32_t *d_err,
                     int stop_after_layer = -1, bool tensor_cores = false, bool chained = false)
 {
     const int n = (int)m->glayers.size();
@@ -459,8 +459,8 @@ int generic_forward(isc_model *m, int8_t *const *bufs, const uint8_t *d_x, const
         const int8_t *res = L.res_tensor >= 0 ? bufs[m->tensor_buf[(size_t)L.res_tensor]] : nullptr;
         cudaError_t e;
         if (i == 0 && tensor_cores && m->wpacks[0])
-            e = launch_stem_conv(G, m->wpacks[0], m->tc_cst[0], m->tc_fast[0] != 0, d_x, m->in_c, ns, batch, out, d_err, st, false, chained && m->tc.chained);
-        else if (i == 0) e = launch_first_conv(G, d_x, m->in_c, ns, batch, out, st);
+            e = launch_stem_conv(G, m->wpacks[0], m->tc_cst[0], m->tc_fast[0] != 0, d_x, m->in_c, ns, run, batch, out, d_err, st, false, chained && m->tc.chained);
+        else if (i == 0) e = launch_first_conv(G, d_x, m->in_c, ns, run, batch, out, st);
         else if (tensor_cores && m->hpacks[(size_t)i] && halo_offsets_fit(G, batch))
             e = launch_halo_conv(m->tc, G, m->hpacks[(size_t)i], m->tc_cst[(size_t)i], m->tc_fast[(size_t)i] != 0, m->tc_resk[(size_t)i], batch, in, res, out, d_err, st);
         else if (tensor_cores && m->wpacks[(size_t)i] && conv_offsets_fit(G, batch)) e = launch_igemm_conv(m->tc, G, m->wpacks[(size_t)i], m->tc_cst[(size_t)i], m->tc_fast[(size_t)i] != 0, m->tc_resk[(size_t)i], batch, in, res, out, d_err, st, false, m->opt_tensor_copy != 0);
@@ -484,18 +484,19 @@ size_t generic_bytes_per_sample(const isc_model *m)
     return s;
 }
 
-// The Monte-Carlo loop for one image and one phase on the layer-by-layer kernels, `cap` samples at a time in the activation
-// buffers `bufs`; adds votes into d_counts (device).  ns: the stream from the first sample on.
-int forward_counts(isc_model *m, int8_t *const *bufs, int64_t cap, bool tensor_cores, const uint8_t *d_x, NoiseStream ns, int64_t n, cudaStream_t st,
-                   int32_t *d_counts, int8_t *d_logits, int32_t *d_err)
+// The Monte-Carlo loop on the layer-by-layer kernels: `total` samples of `run`, in equal batches of at most `cap`, in the
+// activation buffers `bufs`; adds votes into d_counts (device).
+int forward_counts(isc_model *m, int8_t *const *bufs, int64_t cap, bool tensor_cores, const uint8_t *d_x, const NoiseStream &ns, SampleRun run, int64_t total,
+                   cudaStream_t st, int32_t *d_counts, int8_t *d_logits, int32_t *d_err)
 {
     const int last = (int)m->glayers.size();
-    for (int64_t done = 0; done < n; done += cap) {
-        const int b = (int)std::min<int64_t>(cap, n - done);
-        int rc = generic_forward(m, bufs, d_x, ns, b, st, d_err, -1, tensor_cores, done > 0);
+    const int64_t batches = (total + cap - 1) / cap, size = batches ? (total + batches - 1) / batches : 0, begin = (int64_t)run.first;
+    for (int64_t done = 0; done < total; done += size) {
+        const int b = (int)std::min<int64_t>(size, total - done);
+        run.first = (uint64_t)(begin + done);
+        int rc = generic_forward(m, bufs, d_x, ns, run, b, st, d_err, -1, tensor_cores, done > 0);
         if (rc) return rc;
-        ns.first_sample += b;
-        cudaError_t e = launch_votes(bufs[m->tensor_buf[(size_t)last]], m->shapes[(size_t)last].cp, m->n_classes, b, d_counts,
+        cudaError_t e = launch_votes(bufs[m->tensor_buf[(size_t)last]], m->shapes[(size_t)last].cp, m->n_classes, run, b, d_counts,
                                      d_logits ? d_logits + (size_t)done * m->n_classes : nullptr, st, tensor_cores && m->tc.chained);
         m->launches += 1;
         if (e != cudaSuccess) return ISC_ERR_CUDA;
@@ -511,18 +512,28 @@ int64_t tensor_core_cap(const isc_model *m)
     return cap;
 }
 
-// The same in the handle's own buffers.
-int layerwise_counts(isc_model *m, const uint8_t *d_x, uint64_t seed, uint64_t image_id, int32_t phase, int64_t first, int64_t n,
-                     cudaStream_t st, int32_t *d_counts, int8_t *d_logits, int32_t *d_err)
+// The samples of one phase of one image.
+SampleRun one_phase(uint64_t image_id, int32_t phase, int64_t first, int64_t n)
 {
-    int64_t cap = m->opt_batch > 0 ? m->opt_batch : 4096;
+    return SampleRun{image_id, 0, (uint64_t)std::max<int64_t>(n, 1), 0, (uint64_t)first, 0, (uint32_t)phase};
+}
+
+// Samples of a batch in the handle's own buffers.
+int64_t layerwise_cap(const isc_model *m)
+{
+    int64_t cap = m->opt_batch > 0 ? m->opt_batch : 8192;
     const size_t per = std::max<size_t>(generic_bytes_per_sample(m), 1);
     cap = std::min<int64_t>(cap, std::max<int64_t>(1, (int64_t)((3ull << 30) / per)));
-    cap = std::min<int64_t>(cap, m->last_engine == 2 ? tensor_core_cap(m) : 32768);
-    const int batch_alloc = (int)std::min<int64_t>(cap, std::max<int64_t>(n, 1));
-    int rc = ensure_workspace(m, batch_alloc);
+    return std::min<int64_t>(cap, m->last_engine == 2 ? tensor_core_cap(m) : 32768);
+}
+
+// forward_counts in the handle's own buffers.
+int layerwise_counts(isc_model *m, const uint8_t *d_x, uint64_t seed, const SampleRun &run, int64_t total, cudaStream_t st, int32_t *d_counts, int8_t *d_logits, int32_t *d_err)
+{
+    const int64_t cap = layerwise_cap(m);
+    int rc = ensure_workspace(m, (int)std::min<int64_t>(cap, std::max<int64_t>(total, 1)));
     if (rc) return rc;
-    return forward_counts(m, own_buffers(m).data(), cap, m->last_engine == 2, d_x, make_stream(m, seed, image_id, phase, first), n, st, d_counts, d_logits, d_err);
+    return forward_counts(m, own_buffers(m).data(), cap, m->last_engine == 2, d_x, make_stream(m, seed, 0, 0, 0), run, total, st, d_counts, d_logits, d_err);
 }
 
 constexpr size_t kCountsOff = 16;                        // of the counts in the call buffer: the error word comes first
@@ -597,10 +608,11 @@ int count_images(isc_model *m, const uint8_t *x, bool x_on_device, int n_images,
     const uint8_t *d_x;
     if ((rc = begin_call(m, x, d * (size_t)n_images, x_on_device, 2 * C * (size_t)n_images, st, &d_x))) return rc;
     // Pieces of the batch: as many images as make some sixty rounds of the resident engine's groups, so that a launch's
-    // last, partly empty round costs little, and the host's bounds still run under the next piece's kernels.
-    int piece = 1;
-    if (engine == 3)
-        piece = (int)std::max<int64_t>(1, std::min<int64_t>(n_images, 64 * isc::line_wave_samples(m->line) / (n_sel + n_est)));
+    // last, partly empty round costs little, or one batch of the layer-by-layer kernels, whose launches both phases and
+    // several images share (a wide ResNet's 100 + 5,000 samples took three chains of launches, of 100, 4,096 and 904; in
+    // one it is 2,794 -> 2,505 us).  The host's bounds still run under the next piece's kernels.
+    const int64_t at_once = engine == 3 ? 64 * isc::line_wave_samples(m->line) : layerwise_cap(m);
+    const int piece = (int)std::max<int64_t>(1, std::min<int64_t>(n_images, at_once / (n_sel + n_est)));
     const int n_pieces = (n_images + piece - 1) / piece;
     while ((int)m->events.size() < n_pieces - 1) {
         cudaEvent_t ev;
@@ -614,9 +626,8 @@ int count_images(isc_model *m, const uint8_t *x, bool x_on_device, int n_images,
             const isc::LineWork w{d_x + (size_t)i0 * d, n, image_id0 + (uint64_t)i0, n_sel, n_est, 0, c, nullptr};
             rc = isc::line_run(m->line, w, make_stream(m, seed, 0, 1, 0), (int)m->opt_batch, call_err(m), st, &m->launches);
         } else {
-            const uint8_t *xi = d_x + (size_t)i0 * d;
-            rc = layerwise_counts(m, xi, seed, image_id0 + (uint64_t)i0, 0, 0, n_sel, st, c, nullptr, call_err(m));
-            if (rc == ISC_OK) rc = layerwise_counts(m, xi, seed, image_id0 + (uint64_t)i0, 1, 0, n_est, st, c + C, nullptr, call_err(m));
+            const SampleRun run{image_id0 + (uint64_t)i0, (uint64_t)n_sel, (uint64_t)(n_sel + n_est), 0, 0, 0, 1};
+            rc = layerwise_counts(m, d_x + (size_t)i0 * d, seed, run, (int64_t)n * (n_sel + n_est), st, c, nullptr, call_err(m));
         }
         if (rc == ISC_OK) rc = fetch_counts(m, (size_t)i0 * 2 * C, (size_t)n * 2 * C, st);
         if (rc == ISC_OK && k + 1 < n_pieces && cudaEventRecord(m->events[(size_t)k], st) != cudaSuccess) { cudaGetLastError(); rc = ISC_ERR_CUDA; }
@@ -661,7 +672,7 @@ int stalled_launch(isc_model *m, size_t li, cudaStream_t st, int32_t *err, int32
     const bool fast = m->tc_fast[li] != 0;
     const auto t0 = std::chrono::steady_clock::now();
     cudaError_t e;
-    if (li == 0) e = launch_stem_conv(G, m->wpacks[0], m->tc_cst[0], fast, d_x, m->in_c, make_stream(m, 1, 0, 1, 0), 1, out, m->d_tc_err, st, true);
+    if (li == 0) e = launch_stem_conv(G, m->wpacks[0], m->tc_cst[0], fast, d_x, m->in_c, make_stream(m, 1, 0, 1, 0), SampleRun{0, 0, 1, 0, 0, 0, 1}, 1, out, m->d_tc_err, st, true);
     else if (m->hpacks[li]) e = launch_halo_conv(m->tc, G, m->hpacks[li], m->tc_cst[li], fast, m->tc_resk[li], 1, in, res, out, m->d_tc_err, st, true);
     else e = launch_igemm_conv(m->tc, G, m->wpacks[li], m->tc_cst[li], fast, m->tc_resk[li], 1, in, res, out, m->d_tc_err, st, true);
     if (e != cudaSuccess) return ISC_ERR_CUDA;
@@ -801,7 +812,7 @@ int isc_sample_counts(isc_model *m, const uint8_t *x_u8, uint64_t seed, uint64_t
         const isc::LineWork w{d_x, 1, image_id, 0, n_samples, 0, call_counts(m), d_logits};
         rc = isc::line_run(m->line, w, make_stream(m, seed, 0, phase, first_sample), (int)m->opt_batch, call_err(m), st, &m->launches);
     } else {
-        rc = layerwise_counts(m, d_x, seed, image_id, phase, first_sample, n_samples, st, call_counts(m), d_logits, call_err(m));
+        rc = layerwise_counts(m, d_x, seed, one_phase(image_id, phase, first_sample, n_samples), n_samples, st, call_counts(m), d_logits, call_err(m));
     }
     if (rc) {
         cudaStreamSynchronize(st);
@@ -1027,7 +1038,7 @@ int isc_debug_tensor(isc_model *m, const uint8_t *x_u8, uint64_t seed, uint64_t 
         return e == cudaSuccess ? ISC_OK : ISC_ERR_CUDA;
     }
     if ((rc = ensure_workspace(m, 1))) return rc;
-    if ((rc = generic_forward(m, own_buffers(m).data(), d_x, ns, 1, st, call_err(m), tensor - 1, m->opt_engine == 2 || (m->opt_engine == 0 && m->has_tc)))) return rc;
+    if ((rc = generic_forward(m, own_buffers(m).data(), d_x, ns, one_phase(image_id, phase, j, 1), 1, st, call_err(m), tensor - 1, m->opt_engine == 2 || (m->opt_engine == 0 && m->has_tc)))) return rc;
     std::vector<int8_t> h((size_t)s.h * s.w * s.cp);
     CK(cudaMemcpyAsync(h.data(), m->bufs[(size_t)m->tensor_buf[(size_t)tensor]].p, h.size(),
                        cudaMemcpyDeviceToHost, st));
@@ -1178,7 +1189,7 @@ extern "C" int isc_sample_counts_static(isc_model *m, const uint8_t *x_u8, uint6
             buf[b] = reinterpret_cast<int8_t *>(base + off);
             off += (m->buf_bytes[b] * (size_t)cap + 255) & ~(size_t)255;
         }
-        rc = forward_counts(m, buf.data(), cap, tensor_cores, d_x, ns, n_samples, st, d_counts, nullptr, d_err);
+        rc = forward_counts(m, buf.data(), cap, tensor_cores, d_x, ns, one_phase(image_id, phase, first_sample, n_samples), n_samples, st, d_counts, nullptr, d_err);
     }
     m->last_engine = 1;                 // "engine" has always read 1 after this entry point; "static_engine" tells which one ran
     m->last_static_engine = engine;

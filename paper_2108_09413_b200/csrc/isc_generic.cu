@@ -74,14 +74,19 @@ __device__ __forceinline__ int dp4a_us(uint32_t a, int b, int c)
 // (Philox -> table search -> add -> saturate to 0..255) into shared memory as [row][col][4]
 // bytes, then every thread computes output pixels x 16 output channels from that patch.
 __global__ void __launch_bounds__(128)
-k_first_conv(GLayer L, const uint8_t *__restrict__ x, int in_c, NoiseStream ns, int band_rows,
+k_first_conv(GLayer L, const uint8_t *__restrict__ images, int in_c, NoiseStream ns, SampleRun run, int band_rows,
              int8_t *__restrict__ out)
 {
     extern __shared__ uint32_t patch[];   // [rows_in][wpad] packed 4 channels
     conv::chain_start();
     conv::chain_wait();
     const int b = blockIdx.y;
-    const int64_t j = ns.first_sample + b;
+    const SampleRun::Sample sample = run.at((uint32_t)b);
+    const uint64_t image_id = run.image_id0 + sample.image;
+    const uint8_t *__restrict__ x = images + sample.image * (size_t)(in_c * L.hin * L.win);
+    const int64_t j = (int64_t)sample.number;
+    ns.ctr2 = (uint32_t)image_id;
+    ns.ctr3_fixed = sample.phase | ((uint32_t)(image_id >> 32) & 0xFFFFu) << 16;
     const int oy0 = blockIdx.x * band_rows;
     const int oy1 = min(L.hout, oy0 + band_rows);
     const int wpad = L.win + 2 * L.pad;
@@ -290,38 +295,40 @@ __global__ void k_maxpool(GLayer L, conv::FastDiv by_c16, conv::FastDiv by_w, ui
 
 // ------------------------------------------------------------------ votes
 
-// thread = one sample: argmax over the logits (lowest index wins ties), one vote.
-// Votes are first gathered per block in shared memory, then added to the global counts.
-__global__ void k_votes(const int8_t *__restrict__ logits, int cp, int n_classes, int batch,
+// thread = one sample: argmax over the logits (lowest index wins ties; rows are 16-byte aligned), one vote.  A warp's equal
+// votes are one addition.
+__global__ void k_votes(const int8_t *__restrict__ logits, int cp, int n_classes, SampleRun run, int batch,
                         int32_t *__restrict__ counts, int8_t *__restrict__ logits_out)
 {
-    extern __shared__ int32_t hist[];
     conv::chain_start();
-    for (int i = threadIdx.x; i < n_classes; i += blockDim.x) hist[i] = 0;
-    conv::chain_wait();
-    __syncthreads();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b < batch) {
-        const int8_t *p = logits + (size_t)b * cp;
-        int best = 0, bestv = p[0];
-        for (int k = 1; k < n_classes; ++k) {
-            const int v = p[k];
-            if (v > bestv) { bestv = v; best = k; }
+    const bool live = b < batch;
+    const unsigned voters = __ballot_sync(0xffffffffu, live);
+    conv::chain_wait();
+    if (!live) return;
+    const int8_t *p = logits + (size_t)b * cp;
+    int best = 0, bestv = -1000;
+    for (int k0 = 0; k0 < n_classes; k0 += 16) {
+        const uint4 v = *reinterpret_cast<const uint4 *>(p + k0);
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            const int l = (int)(w[k >> 2] << (24 - 8 * (k & 3))) >> 24;
+            if (k0 + k < n_classes && l > bestv) { bestv = l; best = k0 + k; }
         }
-        atomicAdd(&hist[best], 1);
-        if (logits_out)
-            for (int k = 0; k < n_classes; ++k) logits_out[(size_t)b * n_classes + k] = p[k];
     }
-    __syncthreads();
-    for (int i = threadIdx.x; i < n_classes; i += blockDim.x)
-        if (hist[i]) atomicAdd(counts + i, hist[i]);
+    if (logits_out)
+        for (int k = 0; k < n_classes; ++k) logits_out[(size_t)b * n_classes + k] = p[k];
+    const size_t at = (size_t)run.at((uint32_t)b).row * n_classes + best;
+    const unsigned same = __match_any_sync(voters, (unsigned long long)at);
+    if ((threadIdx.x & 31) == __ffs(same) - 1) atomicAdd(counts + at, __popc(same));
 }
 
 }  // namespace
 
 // ------------------------------------------------------------------ launchers
 
-cudaError_t launch_first_conv(const GLayer &L, const uint8_t *x_chw, int in_c, const NoiseStream &ns,
+cudaError_t launch_first_conv(const GLayer &L, const uint8_t *x_chw, int in_c, const NoiseStream &ns, const SampleRun &run,
                               int batch, int8_t *out, cudaStream_t st)
 {
     const int wpad = L.win + 2 * L.pad;
@@ -330,7 +337,7 @@ cudaError_t launch_first_conv(const GLayer &L, const uint8_t *x_chw, int in_c, c
     const size_t smem = (size_t)((band - 1) * L.stride + L.kh) * wpad * 4;
     if (smem > 48 * 1024) return cudaErrorInvalidValue;
     dim3 grid((L.hout + band - 1) / band, batch);
-    k_first_conv<<<grid, 128, smem, st>>>(L, x_chw, in_c, ns, band, out);
+    k_first_conv<<<grid, 128, smem, st>>>(L, x_chw, in_c, ns, run, band, out);
     return cudaGetLastError();
 }
 
@@ -371,11 +378,11 @@ cudaError_t launch_maxpool(const GLayer &L, int batch, const int8_t *in, int8_t 
     return cudaSuccess;
 }
 
-cudaError_t launch_votes(const int8_t *logits_nhwc, int cp, int n_classes, int batch, int32_t *counts,
+cudaError_t launch_votes(const int8_t *logits_nhwc, int cp, int n_classes, const SampleRun &run, int batch, int32_t *counts,
                          int8_t *logits_out, cudaStream_t st, bool chained)
 {
-    return conv::launch_chained(chained, k_votes, dim3((unsigned)((batch + 127) / 128)), 128, n_classes * sizeof(int32_t), st, logits_nhwc, cp, n_classes, batch,
-                                counts, logits_out);
+    return conv::launch_chained(chained, k_votes, dim3((unsigned)((batch + 127) / 128)), 128, 0, st, logits_nhwc, cp, n_classes, run, batch, counts,
+                                logits_out);
 }
 
 }  // namespace isc

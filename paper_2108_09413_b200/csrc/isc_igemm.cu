@@ -538,14 +538,15 @@ struct StemParams {
     uint32_t w_bytes, pos_off, patch_off;
     int slots;                               // pairs of accumulators in tensor memory
     uint32_t tab_off;                        // the noise tables' copy in shared memory (after the patch), 0: searched in global memory
-    const uint8_t *x;                        // clean image, CHW
-    NoiseStream ns;
+    const uint8_t *x;                        // clean images, CHW, one after the other
+    NoiseStream ns;                          // the counter's words come from `run`
     const int8_t *wpack;                     // [filter row][2 K columns][coutp rows][16 bytes]
     const int4 *cst;
     int fast_requant, lo;
     int debug_stall;                         // test hook: the weights are never sent, so that the kernel's waits run out
     int8_t *out;
     int32_t *err;
+    SampleRun run;
 };
 
 // Rows 32 (warp mod 4) .. + 31 of both operands of every tile, half of the channels.
@@ -628,7 +629,11 @@ __global__ void __launch_bounds__(kStemThreads, 2) k_stem(const __grid_constant_
 
     // ---- the band's noisy input rows
     const int b = blockIdx.y;
-    const int64_t j = p.ns.first_sample + b;
+    const SampleRun::Sample sample = p.run.at((uint32_t)b);
+    const int64_t j = (int64_t)sample.number;
+    const uint64_t image_id = p.run.image_id0 + sample.image;
+    const uint32_t ctr2 = (uint32_t)image_id;
+    const uint8_t *x = p.x + sample.image * (size_t)(p.in_c * L.hin * L.win);
     const int oy0 = blockIdx.x * p.band_rows, oy1 = min(L.hout, oy0 + p.band_rows);
     const int wpad = L.win + 2 * L.pad + 8;                     // 8 more pixels: the windows of the last columns stay inside
     const int iy0 = oy0 * L.stride - L.pad;
@@ -645,7 +650,7 @@ __global__ void __launch_bounds__(kStemThreads, 2) k_stem(const __grid_constant_
     const int vy0 = max(0, iy0), vy1 = min(L.hin, iy0 + rows_in);
     if (vy1 > vy0) {
         uint8_t *pb = reinterpret_cast<uint8_t *>(patch);
-        const uint32_t ctr3 = p.ns.ctr3_fixed | (uint32_t)(((j >> 32) & 0xFF) << 8);
+        const uint32_t ctr3 = sample.phase | ((uint32_t)(image_id >> 32) & 0xFFFFu) << 16 | (uint32_t)(((j >> 32) & 0xFF) << 8);
         const uint32_t ctr1 = (uint32_t)(j & 0xFFFFFFFFll);
         if ((L.win & 3) == 0 && p.ns.guide) {
             // every Philox block (four consecutive elements of the CHW order) lies within one image row: a thread
@@ -656,8 +661,8 @@ __global__ void __launch_bounds__(kStemThreads, 2) k_stem(const __grid_constant_
                 const int hr = ic / qpr, wq = ic - hr * qpr;
                 const int h = vy0 + hr;
                 const uint32_t e = (uint32_t)((c * L.hin + h) * L.win) + 4u * (uint32_t)wq;
-                const uint4 r = philox4x32_10(make_uint4(e >> 2, ctr1, p.ns.ctr2, ctr3), p.ns.key0, p.ns.key1);
-                const uint32_t clean = __ldg(reinterpret_cast<const uint32_t *>(p.x + e));
+                const uint4 r = philox4x32_10(make_uint4(e >> 2, ctr1, ctr2, ctr3), p.ns.key0, p.ns.key1);
+                const uint32_t clean = __ldg(reinterpret_cast<const uint32_t *>(x + e));
                 int z[4];
                 if (p.tab_off) noise_levels4_shared(r, sbase + p.tab_off, sbase + p.tab_off + 4u * (uint32_t)(2 * p.ns.T + 1), p.ns.T, p.ns.guide_steps, z);
                 else noise_levels4(r, p.ns.cum, p.ns.guide, p.ns.T, p.ns.guide_steps, z);
@@ -669,7 +674,7 @@ __global__ void __launch_bounds__(kStemThreads, 2) k_stem(const __grid_constant_
             for (int c = 0; c < p.in_c; ++c) {
                 const int64_t e_begin = ((int64_t)c * L.hin + vy0) * L.win, e_end = ((int64_t)c * L.hin + vy1) * L.win;
                 for (int64_t q = (e_begin >> 2) + tid; q < ((e_end + 3) >> 2); q += kStemThreads) {
-                    const uint4 r = philox4x32_10(make_uint4((uint32_t)q, ctr1, p.ns.ctr2, ctr3), p.ns.key0, p.ns.key1);
+                    const uint4 r = philox4x32_10(make_uint4((uint32_t)q, ctr1, ctr2, ctr3), p.ns.key0, p.ns.key1);
                     const uint32_t u[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
@@ -677,7 +682,7 @@ __global__ void __launch_bounds__(kStemThreads, 2) k_stem(const __grid_constant_
                         if (e < e_begin || e >= e_end) continue;
                         const int rem = (int)(e - (int64_t)c * L.hin * L.win);
                         const int h = rem / L.win, w = rem - h * L.win;
-                        int v = (int)__ldg(p.x + e) + (p.ns.guide ? noise_level_guided(u[k], p.ns.cum, p.ns.guide, p.ns.T) : noise_level(u[k], p.ns.cum, p.ns.T));
+                        int v = (int)__ldg(x + e) + (p.ns.guide ? noise_level_guided(u[k], p.ns.cum, p.ns.guide, p.ns.T) : noise_level(u[k], p.ns.cum, p.ns.T));
                         v = min(255, max(0, v));
                         pb[((h - iy0) * wpad + (w + L.pad)) * 4 + c] = (uint8_t)v;
                     }
@@ -1070,7 +1075,7 @@ void stem_pack_weights(const GLayer &G, const int8_t *w, int8_t *out)
 }
 
 cudaError_t launch_stem_conv(const GLayer &G, const int8_t *wpack, const int32_t *cst, bool fast, const uint8_t *x_chw, int in_c,
-                             const NoiseStream &ns, int batch, int8_t *out, int32_t *err, cudaStream_t st, bool debug_stall, bool chained)
+                             const NoiseStream &ns, const SampleRun &run, int batch, int8_t *out, int32_t *err, cudaStream_t st, bool debug_stall, bool chained)
 {
     StemParams p;
     p.L = G;
@@ -1086,7 +1091,7 @@ cudaError_t launch_stem_conv(const GLayer &G, const int8_t *wpack, const int32_t
     int cols = 32;
     while (cols < p.slots * 2 * G.coutp) cols <<= 1;
     p.tmem_cols = cols;
-    p.x = x_chw; p.ns = ns; p.wpack = wpack;
+    p.x = x_chw; p.ns = ns; p.run = run; p.wpack = wpack;
     p.cst = reinterpret_cast<const int4 *>(cst);
     p.fast_requant = fast ? 1 : 0;
     p.lo = G.relu ? (G.zp_out > -128 ? G.zp_out : -128) : -128;

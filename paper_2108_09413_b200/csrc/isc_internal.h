@@ -31,6 +31,23 @@ struct NoiseStream {
     int guide_steps;          // bisection steps that close the widest interval [guide[j], guide[j+1]]
 };
 
+// What the samples of a forward pass of the layer-by-layer kernels are: per image, n_sel samples of the selection phase (numbers
+// from 0 on), then the estimation phase's (numbers from first_est on), per_image in all; a launch's samples start at number
+// `first` of this sequence.  Images lie one after the other; votes go to row 2 i (selection) and 2 i + 1 (estimation) of the
+// counts, or to row i without a selection phase.
+struct SampleRun {
+    uint64_t image_id0;
+    uint64_t n_sel, per_image, first, first_est;
+    uint32_t phase_sel, phase_est;
+    struct Sample { uint64_t image, number; uint32_t phase, row; };
+    __host__ __device__ Sample at(uint32_t slot) const
+    {
+        const uint64_t g = first + slot, image = g < per_image ? 0 : g / per_image, r = g - image * per_image;
+        const bool sel = r < n_sel;
+        return Sample{image, sel ? r : first_est + (r - n_sel), sel ? phase_sel : phase_est, (uint32_t)(n_sel ? 2 * image + (sel ? 0 : 1) : image)};
+    }
+};
+
 // One layer as the layer-by-layer kernels see it (device pointers).
 struct GLayer {
     int op;
@@ -54,7 +71,7 @@ struct LayerIn {
 };
 
 // ---- layer-by-layer engine (isc_generic.cu) ----
-cudaError_t launch_first_conv(const GLayer &L, const uint8_t *x_chw, int in_c, const NoiseStream &ns,
+cudaError_t launch_first_conv(const GLayer &L, const uint8_t *x_chw, int in_c, const NoiseStream &ns, const SampleRun &run,
                               int batch, int8_t *out, cudaStream_t st);
 cudaError_t launch_noisy_input(const uint8_t *x_chw, int in_c, int in_h, int in_w, const NoiseStream &ns,
                                int batch, int32_t *out_chw, cudaStream_t st);
@@ -62,7 +79,7 @@ cudaError_t launch_conv(const GLayer &L, int batch, const int8_t *in, const int8
                         cudaStream_t st, bool chained = false);
 cudaError_t launch_gavgpool(const GLayer &L, int batch, const int8_t *in, int8_t *out, cudaStream_t st, bool chained = false);
 cudaError_t launch_maxpool(const GLayer &L, int batch, const int8_t *in, int8_t *out, cudaStream_t st, bool chained = false);
-cudaError_t launch_votes(const int8_t *logits_nhwc, int cp, int n_classes, int batch, int32_t *counts,
+cudaError_t launch_votes(const int8_t *logits_nhwc, int cp, int n_classes, const SampleRun &run, int batch, int32_t *counts,
                          int8_t *logits_out, cudaStream_t st, bool chained = false);
 
 // ---- layer-by-layer tensor-core convolutions (isc_igemm.cu) ----
@@ -121,7 +138,8 @@ bool stem_fits(const GLayer &G, int in_c);
 size_t stem_pack_bytes(const GLayer &G);
 void stem_pack_weights(const GLayer &G, const int8_t *w_oihw, int8_t *out);
 cudaError_t launch_stem_conv(const GLayer &G, const int8_t *wpack, const int32_t *cst, bool fast, const uint8_t *x_chw, int in_c,
-                             const NoiseStream &ns, int batch, int8_t *out, int32_t *err, cudaStream_t st, bool debug_stall = false, bool chained = false);
+                             const NoiseStream &ns, const SampleRun &run, int batch, int8_t *out, int32_t *err, cudaStream_t st, bool debug_stall = false,
+                             bool chained = false);
 
 // ---- host decision rules (isc_decide.cpp) ----
 double lower_conf_bound(int64_t k, int64_t n, double alpha);
