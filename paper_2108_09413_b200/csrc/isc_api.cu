@@ -280,6 +280,7 @@ int build_generic_engine(isc_model *m)
                 const int n_cst = halo ? halo_padded_cout(G) : igemm_padded_cout(G);
                 std::vector<int32_t> c4((size_t)n_cst * 4);
                 m->tc_fast[(size_t)i] = igemm_constants(G, bias.data(), mult.data(), shift.data(), c4.data(), n_cst, H.d.res_tensor >= 0, &m->tc_resk[(size_t)i]) ? 1 : 0;
+                if (!halo) igemm_order_constants(G, c4.data(), n_cst);
                 rc = upload(m, c4, &m->tc_cst[(size_t)i]); if (rc) return rc;
                 m->has_tc = true;
             }
@@ -464,7 +465,7 @@ int generic_forward(isc_model *m, int8_t *const *bufs, const uint8_t *d_x, const
         else if (tensor_cores && m->hpacks[(size_t)i] && halo_offsets_fit(G, batch))
             e = launch_halo_conv(m->tc, G, m->hpacks[(size_t)i], m->tc_cst[(size_t)i], m->tc_fast[(size_t)i] != 0, m->tc_resk[(size_t)i], batch, in, res, out, d_err, st);
         else if (tensor_cores && m->wpacks[(size_t)i] && conv_offsets_fit(G, batch)) e = launch_igemm_conv(m->tc, G, m->wpacks[(size_t)i], m->tc_cst[(size_t)i], m->tc_fast[(size_t)i] != 0, m->tc_resk[(size_t)i], batch, in, res, out, d_err, st, false, m->opt_tensor_copy != 0);
-        else if (L.op == ISC_CONV2D || L.op == ISC_FC) e = launch_conv(G, batch, in, res, out, st, follows);
+        else if (L.op == ISC_CONV2D || L.op == ISC_FC) e = launch_conv(G, batch, in, res, out, st);
         else if (L.op == ISC_GAVGPOOL) e = launch_gavgpool(G, batch, in, out, st, follows);
         else e = launch_maxpool(G, batch, in, out, st, follows);
         m->launches += 1;

@@ -78,8 +78,6 @@ k_first_conv(GLayer L, const uint8_t *__restrict__ images, int in_c, NoiseStream
              int8_t *__restrict__ out)
 {
     extern __shared__ uint32_t patch[];   // [rows_in][wpad] packed 4 channels
-    conv::chain_start();
-    conv::chain_wait();
     const int b = blockIdx.y;
     const SampleRun::Sample sample = run.at((uint32_t)b);
     const uint64_t image_id = run.image_id0 + sample.image;
@@ -172,8 +170,6 @@ __global__ void __launch_bounds__(128)
 k_conv(GLayer L, int batch, const int8_t *__restrict__ in, const int8_t *__restrict__ res,
        int8_t *__restrict__ out)
 {
-    conv::chain_start();
-    conv::chain_wait();
     const int64_t npx = (int64_t)batch * L.hout * L.wout;
     const int64_t px = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (px >= npx) return;
@@ -220,7 +216,7 @@ k_conv(GLayer L, int batch, const int8_t *__restrict__ in, const int8_t *__restr
 
 // ------------------------------------------------------------------ pools
 
-__global__ void k_gavgpool(GLayer L, int batch, const int8_t *__restrict__ in, int8_t *__restrict__ out)
+__global__ void k_gavgpool(GLayer L, int batch, const int8_t *in, int8_t *out)
 {
     conv::chain_start();
     conv::chain_wait();
@@ -266,7 +262,9 @@ __global__ void k_maxpool(GLayer L, conv::FastDiv by_c16, conv::FastDiv by_w, ui
     if (y0 + kh > 0 && y0 < L.hin && x0 + kw > 0 && x0 < L.win) {
         auto tap = [&](int r, int c) {
             const int iy = min(max(y0 + r, 0), L.hin - 1), ix = min(max(x0 + c, 0), L.win - 1);
-            return __ldg(reinterpret_cast<const uint4 *>(src + (size_t)(iy * L.win + ix) * L.cinp));
+            uint4 v;                                             // not through the read-only path: the layer before may still have been running when this one started
+            asm volatile("ld.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(src + (size_t)(iy * L.win + ix) * L.cinp));
+            return v;
         };
         auto take = [&](const uint4 &a) {
             const uint32_t w[4] = {a.x, a.y, a.z, a.w};
@@ -297,7 +295,7 @@ __global__ void k_maxpool(GLayer L, conv::FastDiv by_c16, conv::FastDiv by_w, ui
 
 // thread = one sample: argmax over the logits (lowest index wins ties; rows are 16-byte aligned), one vote.  A warp's equal
 // votes are one addition.
-__global__ void k_votes(const int8_t *__restrict__ logits, int cp, int n_classes, SampleRun run, int batch,
+__global__ void k_votes(const int8_t *logits, int cp, int n_classes, SampleRun run, int batch,
                         int32_t *__restrict__ counts, int8_t *__restrict__ logits_out)
 {
     conv::chain_start();
@@ -351,11 +349,12 @@ cudaError_t launch_noisy_input(const uint8_t *x_chw, int in_c, int in_h, int in_
 }
 
 cudaError_t launch_conv(const GLayer &L, int batch, const int8_t *in, const int8_t *res, int8_t *out,
-                        cudaStream_t st, bool chained)
+                        cudaStream_t st)
 {
     const int64_t npx = (int64_t)batch * L.hout * L.wout;
     dim3 grid((unsigned)((npx + 127) / 128), L.coutp >> 4);
-    return conv::launch_chained(chained, k_conv, grid, 128, 0, st, L, batch, in, res, out);
+    k_conv<<<grid, 128, 0, st>>>(L, batch, in, res, out);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_gavgpool(const GLayer &L, int batch, const int8_t *in, int8_t *out, cudaStream_t st, bool chained)

@@ -18,14 +18,10 @@
 //   * one thread issues two tcgen05.mma (kind::i8, K = 32) per stage and commits the stage back to the loaders;
 //     accumulators alternate between two column ranges, so a tile's reduction runs under the previous one's
 //     epilogue;
-//   * two teams of four warps requantise (fixed-point multiplier, shift, zero-points, residual add, clamp), one
-//     accumulator each: a thread owns one tile row, 32 columns per step with the next step's accumulators already
-//     requested; the rows pass through a per-warp scratch area so that, every 64 columns, the results leave and the
-//     next tile's residual rows arrive as contiguous runs, under the arithmetic of the following columns.
+//   * sixteen warps requantise (fixed-point multiplier, shift, zero-points, residual add, clamp), shared among the
+//     accumulators in flight (epilogue_whole); in the general form eight warps, one tile row per thread (epilogue_rows).
 // 1 x 1 layers that expand the channels, which the epilogue bounds, take tiles of 256 pixels x 128 channels (kPair): a
-// thread then owns two rows and reads a channel's constants once for both.  64 -> 256 channels at 56 x 56, 512 samples:
-// 222 -> 184 us, with a residual operand 286 -> 265 us; 256 -> 128: 159 -> 135 us.  (Sixteen epilogue warps instead of
-// eight: 203 and 294 us against 196 and 280.)
+// thread then reads a channel's constants once for two operands.
 // Every wait is bounded; on expiry a role raises the CTA's abort flag and the error word, the others leave their
 // loops, and the CTA frees its tensor memory and returns.
 #include <cuda.h>
@@ -37,6 +33,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <vector>
 
 #include "isc_conv.cuh"
 #include "isc_epilogue.cuh"
@@ -56,18 +53,23 @@ constexpr int kMaxStages = 16;
 constexpr int kPairN = 128;                  // channels of a paired tile: two operands of 128 rows, two tiles in tensor memory
 constexpr int kStemEpi = 8, kStemThreads = 32 * (kStemEpi + 1);        // k_stem: two threads per tile row and the MMA warp; two CTAs per SM
 constexpr size_t kStemSmemPair = 108 * 1024, kStemSmemLimit = 220 * 1024;       // dynamic shared memory of k_stem: for two CTAs per SM; at most
-constexpr int kEpiWarps = 4, kEpiTeams = 2, kGatherWarps = 4;          // a team of epilogue warps takes every other tile
-constexpr int kAllEpiWarps = kEpiWarps * kEpiTeams;
-static_assert(kEpiWarps == 4, "an epilogue warp owns all N columns of its 32 rows");
-constexpr int kGemmThreads = 32 * (kAllEpiWarps + kGatherWarps + 2);      // k_igemm: + the MMA warp + the weights warp
+constexpr int kRowTeams = 2, kRowWarps = 4 * kRowTeams;                // epilogue_rows: a team of four warps takes every other tile
+// Warps of k_igemm by role: epilogue, gather, and one each for MMAs and weights.  Whole tiles whose operands come by tensor copy
+// need no gather warps and have sixteen epilogue warps; beside four gather warps sixteen would leave a thread 80 registers,
+// and two gather warps were too few (3 x 3 stride 2, 128 channels at 56 x 56: 156 -> 202 us).
+__host__ __device__ constexpr int igemm_epi_warps(bool whole, bool copy) { return whole && copy ? 16 : kRowWarps; }
+__host__ __device__ constexpr int igemm_gather_warps(bool whole, bool copy) { return whole && copy ? 0 : 4; }
+__host__ __device__ constexpr int igemm_threads(bool whole, bool copy) { return 32 * (igemm_epi_warps(whole, copy) + igemm_gather_warps(whole, copy) + 2); }
 
 struct IgemmParams {
     alignas(64) CUtensorMap tmap_a;          // the input as (16 bytes, pixel, 16-byte column of the channels): see tma_a
+    alignas(64) CUtensorMap tmap_res;        // the residual operand as (channel, pixel), boxes of a tile: prefetched into L2
     GLayer L;
+    int prefetch_res;
     int tma_a;                               // 1 x 1 stride 1: the operand rows arrive by one tensor copy per block, the gather warps idle
-    int batch, n_tile, tiles_n, acc_stride, tmem_cols, stages;     // acc_stride: tensor-memory columns from one accumulator to the other
+    int batch, n_tile, tiles_n, n_acc, acc_stride, tmem_cols, stages;     // accumulators in tensor memory; columns from one to the next
     int units, n_blocks;                     // 16-byte columns of the reduction (filter tap, 16 input channels); blocks of four of them
-    uint32_t scratch_off;                    // the epilogue warps' row scratch within the dynamic shared memory
+    uint32_t scratch_off;                    // epilogue_rows: the warps' row scratch within the dynamic shared memory
     uint32_t m_total, tiles_m;               // batch * hout * wout (< 2^31); tiles of 128 of them
     const int8_t *in, *res;
     int8_t *out;
@@ -86,11 +88,11 @@ struct IgemmParams {
 struct EpiCtx {
     uint32_t sbase, tmem, n_tiles, grid_n;
     int tiles_n, warp, lane;
-    uint32_t cst_s, acc_full, acc_free;       // shared-memory addresses: constants, the two accumulators' barriers
+    uint32_t cst_s, acc_full, acc_free;       // shared-memory addresses: constants, the accumulators' barriers
     const volatile int *abort_flag;
 };
 
-// The epilogue of k_igemm.  Warp w owns lanes 32 (w mod 4) .. +31 of an accumulator (= 32 tile rows) and all N
+// The epilogue of the general form.  Warp w owns lanes 32 (w mod 4) .. +31 of an accumulator (= 32 tile rows) and all N
 // columns; team w / 4 takes every other tile of the CTA (accumulator `team`).  A thread requantises its own row in
 // place in a per-warp scratch area in shared memory (row stride N + 16 bytes: conflict-free for the row-wise and
 // for the coalesced access).  After every 64 columns the warp writes those columns of its 32 rows out as runs of
@@ -98,13 +100,12 @@ struct EpiCtx {
 // space that has just been read, so memory traffic runs under the arithmetic of the following columns.
 // kMode 0: 64-bit requantisation (any shift), 1: 32-bit form, 2 / 3: 32-bit form with the residual add (3: its
 // single-precision form).
-// kWhole: every tile has n_tile valid columns and n_tile is a multiple of 64.
-template <int kMode, bool kWhole>
-__device__ __forceinline__ bool epilogue_role(const IgemmParams &p, const EpiCtx &c)
+template <int kMode>
+__device__ __forceinline__ bool epilogue_rows(const IgemmParams &p, const EpiCtx &c)
 {
     const GLayer &L = p.L;
     const int warp = c.warp, lane = c.lane, n_tile = p.n_tile, tiles_n = c.tiles_n;
-    const int q = warp & 3, team = warp / kEpiWarps;
+    const int q = warp & 3, team = warp >> 2;
     const uint32_t lane_base = (uint32_t)(q * 32) << 16;
     const uint32_t row_stride = epi_row_stride(n_tile);
     const uint32_t scr0 = c.sbase + p.scratch_off + (uint32_t)warp * 32u * row_stride;
@@ -121,15 +122,15 @@ __device__ __forceinline__ bool epilogue_role(const IgemmParams &p, const EpiCtx
         rows = m0 < p.m_total ? min(32u, p.m_total - m0) : 0u;
         return base + (size_t)(m0 + (uint32_t)crow) * L.coutp + (int)(t - m_idx * tiles_n) * n_tile + cchunk * 16;
     };
-    auto tile_cols = [&](uint32_t t) { return kWhole ? n_tile : min(n_tile, L.coutp - (int)(t % (uint32_t)tiles_n) * n_tile); };       // a multiple of 16
+    auto tile_cols = [&](uint32_t t) { return min(n_tile, L.coutp - (int)(t % (uint32_t)tiles_n) * n_tile); };       // a multiple of 16
     auto residual_fetch = [&](const int8_t *src, uint32_t rows, int c0, int n_cols) {
-        if (!kWhole && c0 + cchunk * 16 >= n_cols) return;
+        if (c0 + cchunk * 16 >= n_cols) return;
 #pragma unroll
         for (int k = 0; k < 4; ++k)
             if ((uint32_t)(8 * k + crow) < rows) cp_async16(scr_co + (uint32_t)(8 * k) * row_stride + (uint32_t)c0, src + (size_t)k * co_step + c0);
     };
-    // the team's tiles: every kEpiTeams-th of the CTA's
-    const uint32_t t_step = (uint32_t)kEpiTeams * c.grid_n;
+    // the team's tiles: every kRowTeams-th of the CTA's
+    const uint32_t t_step = (uint32_t)kRowTeams * c.grid_n;
     uint32_t t = blockIdx.x + (uint32_t)team * c.grid_n;
     if (kMode >= 2 && t < c.n_tiles) {
         uint32_t rows;
@@ -159,7 +160,7 @@ __device__ __forceinline__ bool epilogue_role(const IgemmParams &p, const EpiCtx
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int cc = c0 + 16 * h;
-                if (!kWhole && h == 1 && cc >= n_cols) break;
+                if (h == 1 && cc >= n_cols) break;
                 uint4 v;
                 if (kMode == 3) {
                     v = requant16_fast<2>(acc[h], cst0 + (uint32_t)cc * 16u, ld_shared_v4(scr_row + (uint32_t)cc), p.res_m2, 0ll, p.res_k8, p.lo);
@@ -179,7 +180,7 @@ __device__ __forceinline__ bool epilogue_role(const IgemmParams &p, const EpiCtx
         tmem_ld32_issue(acc_base, acc_a);
 #pragma unroll 1
         for (int c0 = 0; c0 < n_cols; c0 += 64) {
-            const bool second = kWhole || c0 + 32 < n_cols, more = c0 + 64 < n_cols;
+            const bool second = c0 + 32 < n_cols, more = c0 + 64 < n_cols;
             tmem_ld32_wait(acc_a);
             if (second) tmem_ld32_issue(acc_base + (uint32_t)c0 + 32u, acc_b);
             step(acc_a, c0);
@@ -192,7 +193,7 @@ __device__ __forceinline__ bool epilogue_role(const IgemmParams &p, const EpiCtx
             }
             if (second) step(acc_b, c0 + 32);
             __syncwarp();
-            const bool mine = kWhole || c0 + cchunk * 16 < n_cols;            // a row holds the tile's columns and no more
+            const bool mine = c0 + cchunk * 16 < n_cols;            // a row holds the tile's columns and no more
             uint4 v[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) v[k] = ld_shared_v4(mine ? scr_co + (uint32_t)(8 * k) * row_stride + (uint32_t)c0 : scr0);
@@ -202,122 +203,128 @@ __device__ __forceinline__ bool epilogue_role(const IgemmParams &p, const EpiCtx
             __syncwarp();
             if (res_next) residual_fetch(res_next, rows_next, c0, n_cols_next);
         }
-        for (int c0 = (n_cols + 63) & ~63; !kWhole && c0 < n_cols_next; c0 += 64) residual_fetch(res_next, rows_next, c0, n_cols_next);
+        for (int c0 = (n_cols + 63) & ~63; c0 < n_cols_next; c0 += 64) residual_fetch(res_next, rows_next, c0, n_cols_next);
     }
     cp_async_wait_all();
     return true;
 }
 
-// The epilogue of a paired tile: 256 pixels (two M operands) x kPairN channels.  A thread owns one row of each operand, so
-// that a channel's constants are read once for two outputs.  Scratch and memory traffic as above, 64 columns of the 64
-// rows at a time.  kMode 1 to 3 as above; kClamp: the lower clamp is above -128.
-template <int kMode, bool kClamp>
-__device__ __forceinline__ bool epilogue_pair(const IgemmParams &p, const EpiCtx &c)
+__device__ __forceinline__ void st_global_v4(void *p, const uint32_t (&v)[4])
 {
-    constexpr int kRes = kMode == 3 ? 2 : kMode == 2 ? 1 : 0;
+    asm volatile("st.global.L1::no_allocate.v4.u32 [%0], {%1,%2,%3,%4};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
+}
+__device__ __forceinline__ void ld_global_v4(const void *p, uint32_t (&v)[4])
+{
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "l"(p) : "memory");
+}
+
+// The epilogue of whole tiles (every column valid, a multiple of 64 of them).  Accumulators are read as fragments: of 16
+// columns a thread holds four in each of four rows per operand (lane / 4 + 8 i), and the columns of the weights are ordered
+// so that its columns of four such chunks are 16 consecutive channels (igemm_channel).  A thread's four constants of a chunk
+// serve eight outputs each in a paired tile, residual rows are read and results written straight from registers (four lanes
+// make 64 contiguous bytes of a pixel), nothing passes through shared memory, and sixteen warps have registers enough.  (One row
+// per thread took a 16-byte constant per one or two outputs, a scratch row in shared memory both ways, and eight warps, two
+// per scheduler, which left its latency exposed: 64 -> 256 channels with a residual operand at 56 x 56, 512 samples: 280 us in all, now 253.)
+// n_acc accumulators are in flight.  Of the four warps of a quarter two take every other tile, and in it every other unit; with
+// four accumulators (64 columns) each takes every fourth tile.
+// kMode 0: 64-bit requantisation (any shift), 1: 32-bit form, 2 / 3: 32-bit form with the residual add (3: its
+// single-precision form).  kClamp: the lower clamp is above -128.
+template <int kMode, bool kPair, bool kClamp, int kWarps>
+__device__ __forceinline__ bool epilogue_whole(const IgemmParams &p, const EpiCtx &c)
+{
+    constexpr uint32_t kMT = kPair ? 2 : 1;
     const GLayer &L = p.L;
-    const int lane = c.lane, tiles_n = c.tiles_n, q = c.warp & 3, team = c.warp / kEpiWarps;
-    constexpr uint32_t row_stride = kPairN + 16, mt_step = 32u * row_stride;
-    const uint32_t scr0 = c.sbase + p.scratch_off + (uint32_t)c.warp * (2u * mt_step);
-    const uint32_t scr_row = scr0 + (uint32_t)lane * row_stride;
-    const int crow = lane >> 2, cchunk = lane & 3;
-    const uint32_t scr_co = scr0 + (uint32_t)crow * row_stride + (uint32_t)cchunk * 16u;
-    const size_t co_step = (size_t)8 * L.coutp, co_mt = (size_t)kTileM * L.coutp;
-    // this lane's coalesced position in tile t; `rem` pixels of the tensor are left at the warp's first row
-    auto tile_ptr = [&](const int8_t *base, uint32_t t, uint32_t &rem) {
-        const uint32_t m_idx = t / (uint32_t)tiles_n, m0 = m_idx * (2u * kTileM) + (uint32_t)q * 32u;
-        rem = m0 < p.m_total ? p.m_total - m0 : 0u;
-        return base + (size_t)(m0 + (uint32_t)crow) * L.coutp + (int)(t - m_idx * tiles_n) * kPairN + cchunk * 16;
-    };
-    auto residual_fetch = [&](const int8_t *src, uint32_t rem, int c0) {
-#pragma unroll
-        for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if ((uint32_t)(mt * kTileM + 8 * k + crow) < rem)
-                    cp_async16(scr_co + (uint32_t)mt * mt_step + (uint32_t)(8 * k) * row_stride + (uint32_t)c0, src + (size_t)mt * co_mt + (size_t)k * co_step + c0);
-    };
-    const uint32_t t_step = (uint32_t)kEpiTeams * c.grid_n;
-    uint32_t t = blockIdx.x + (uint32_t)team * c.grid_n;
-    if (kRes && t < c.n_tiles) {
-        uint32_t rem;
-        const int8_t *src = tile_ptr(p.res, t, rem);
-        for (int c0 = 0; c0 < kPairN; c0 += 64) residual_fetch(src, rem, c0);
-    }
-    const uint32_t acc0 = c.tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(team * p.acc_stride);
-    for (int au = 0; t < c.n_tiles; t += t_step, ++au) {
-        const int n0 = (int)(t % (uint32_t)tiles_n) * kPairN;
-        uint32_t rem, rem_next = 0;
-        int8_t *dst = const_cast<int8_t *>(tile_ptr(p.out, t, rem));
-        const int8_t *res_next = (kRes && t + t_step < c.n_tiles) ? tile_ptr(p.res, t + t_step, rem_next) : nullptr;
-        if (kRes) cp_async_wait_all();                              // the tile's residual rows, requested during the previous tile
-        __syncwarp();
-        if (!wait_bar<kHintEpi>(c.acc_full + 8u * (uint32_t)team, (uint32_t)au & 1u, c.abort_flag)) {
-            cp_async_wait_all();
-            return false;
-        }
-        tc_fence_after();
-        const uint32_t cst0 = c.cst_s + (uint32_t)n0 * 16u;
-        auto load = [&](int (&a)[2][16], int cc) {
-            tmem_ld16_issue(acc0 + (uint32_t)cc, a[0]);
-            tmem_ld16_issue(acc0 + (uint32_t)(kPairN + cc), a[1]);
-        };
-        auto step = [&](int (&a)[2][16], int cc) {
-            const uint32_t scr = scr_row + (uint32_t)cc;
-            uint32_t r0[4] = {0, 0, 0, 0}, r1[4] = {0, 0, 0, 0};
-            if (kRes) {
-                const uint4 u = ld_shared_v4(scr), v = ld_shared_v4(scr + mt_step);
-                r0[0] = u.x ^ 0x80808080u; r0[1] = u.y ^ 0x80808080u; r0[2] = u.z ^ 0x80808080u; r0[3] = u.w ^ 0x80808080u;
-                r1[0] = v.x ^ 0x80808080u; r1[1] = v.y ^ 0x80808080u; r1[2] = v.z ^ 0x80808080u; r1[3] = v.w ^ 0x80808080u;
-            }
-            uint4 o[2];
-            requant16x2<kRes, kClamp>(a, cst0 + (uint32_t)cc * 16u, r0, r1, p.res_m2, p.res_r2, p.res_k8, p.lo, o);
-            st_shared_v4(scr, o[0]);
-            st_shared_v4(scr + mt_step, o[1]);
-        };
-        int acc_a[2][16], acc_b[2][16];
-        load(acc_a, 0);
+    const uint32_t word = (uint32_t)c.lane & 3u, q = (uint32_t)c.warp & 3u, w4 = (uint32_t)c.warp >> 2;
+    const uint32_t n_acc = (uint32_t)p.n_acc, team = w4 & (n_acc - 1u), split = (uint32_t)(kWarps / 4) / n_acc, part = w4 / n_acc;
+    const uint32_t n_units = kMT * ((uint32_t)p.n_tile >> 6), coutp = (uint32_t)L.coutp;       // a unit: 128 rows x 64 columns
+    const uint32_t acc0 = c.tmem + (q * 32u << 16) + team * (uint32_t)p.acc_stride, bar_full = c.acc_full + 8u * team, bar_free = c.acc_free + 8u * team;
+    const bool has_res = kMode >= 2 || (kMode == 0 && p.res);
+    uint32_t use = 0;
+    for (uint32_t t = blockIdx.x + team * c.grid_n; t < c.n_tiles; t += n_acc * c.grid_n, ++use) {
+        const uint32_t m_idx = t / (uint32_t)c.tiles_n, n0 = (t - m_idx * (uint32_t)c.tiles_n) * (uint32_t)p.n_tile + word * 16u;
+        bool ready = false;
 #pragma unroll 1
-        for (int cc = 0; cc < kPairN; cc += 32) {
-            tmem_ld32_wait(acc_a);
-            load(acc_b, cc + 16);
-            step(acc_a, cc);
-            tmem_ld32_wait(acc_b);
-            if (cc + 32 < kPairN) {
-                load(acc_a, cc + 32);
-            } else {
-                tc_fence_before();
-                mbar_arrive(c.acc_free + 8u * (uint32_t)team);      // the accumulators are in registers: the next tile may overwrite them
+        for (uint32_t unit = part; unit < n_units; unit += split) {
+            const uint32_t mt = kPair ? unit & 1u : 0u, col = (kPair ? unit >> 1 : unit) * 64u;
+            const uint32_t row = (m_idx * kMT + mt) * (uint32_t)kTileM + q * 32u + ((uint32_t)c.lane >> 2);
+            const uint32_t rem = row < p.m_total ? p.m_total - row : 0u;                 // valid rows are this thread's first ones
+            const size_t at = (size_t)row * coutp + n0 + col;
+            uint32_t io[4][4];                                                          // residual bytes, then results
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) io[i][k] = 0;
+                if (has_res && (uint32_t)(8 * i) < rem) ld_global_v4(p.res + at + (size_t)(8 * i) * coutp, io[i]);
             }
-            step(acc_b, cc + 16);
-            if (!(cc & 32)) continue;
-            const int c0 = cc - 32;
-            __syncwarp();
+            if (!ready) {
+                ready = __all_sync(0xffffffffu, wait_bar<kHintEpi>(bar_full, use & 1u, c.abort_flag));
+                if (!ready) return false;
+                tc_fence_after();
+            }
+            const uint32_t acc = acc0 + mt * kPairN + col, cst = c.cst_s + (n0 + col) * 16u - word * 240u;       // n0 has the thread's 16 channels
+            int a[2][8];
+            tmem_ld_frag(acc, a[0]);
 #pragma unroll
-            for (int mt = 0; mt < 2; ++mt) {
-                uint4 v[4];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) v[k] = ld_shared_v4(scr_co + (uint32_t)mt * mt_step + (uint32_t)(8 * k) * row_stride + (uint32_t)c0);
+            for (int ch = 0; ch < 4; ++ch) {
+                int4 k4[4];
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
-                    if ((uint32_t)(mt * kTileM + 8 * k + crow) < rem) *reinterpret_cast<uint4 *>(dst + (size_t)mt * co_mt + (size_t)k * co_step + c0) = v[k];
+                    asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(k4[k].x), "=r"(k4[k].y), "=r"(k4[k].z), "=r"(k4[k].w) : "r"(cst + (uint32_t)(ch * 256 + k * 64)));
+#pragma unroll
+                for (int hf = 0; hf < 2; ++hf) {
+                    tmem_ld_frag_wait(a[hf]);
+                    // the next accumulators, before this step's arithmetic
+                    if (hf == 0) tmem_ld_frag(acc + (uint32_t)(ch * 16) + (16u << 16), a[1]);
+                    else if (ch < 3) tmem_ld_frag(acc + (uint32_t)(ch * 16 + 16), a[0]);
+                    else if (unit + split >= n_units) {
+                        tc_fence_before();
+                        mbar_arrive(bar_free);                  // the accumulators are in registers: the next tile may overwrite them
+                    }
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        uint32_t &w = io[2 * hf + j][ch];
+                        const uint32_t rw = w ^ 0x80808080u;
+                        int y[4];
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const int v = a[hf][2 * j + (k & 1) + 4 * (k >> 1)];
+                            if (kMode == 0) {
+                                const int o = (int)(n0 + col) + 4 * ch + k;
+                                const long long rt = has_res ? residual_term(byte_of(w, k), L.zp_res, L.res_mult, L.res_shift) : 0ll;
+                                y[k] = o < L.cout ? requant_clamp(v + __ldg(L.bias + o), __ldg(L.mult + o), __ldg(L.shift + o), rt, L.zp_out, p.lo) : 0;
+                            } else {
+                                y[k] = requant1<kMode == 3 ? 2 : kMode == 2 ? 1 : 0, kClamp>(v, k4[k], rw, k, p.res_m2, p.res_r2, p.res_k8, p.lo);
+                            }
+                        }
+                        w = pack4_sat(y[0], y[1], y[2], y[3]);
+                    }
+                }
             }
-            __syncwarp();
-            if (res_next) residual_fetch(res_next, rem_next, c0);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if ((uint32_t)(8 * i) < rem) st_global_v4(p.out + at + (size_t)(8 * i) * coutp, io[i]);
+        }
+        if (!ready) {                                                                   // fewer units than parts: let the tile go
+            if (!__all_sync(0xffffffffu, wait_bar<kHintEpi>(bar_full, use & 1u, c.abort_flag))) return false;
+            tc_fence_before();
+            mbar_arrive(bar_free);
         }
     }
-    cp_async_wait_all();
     return true;
 }
 
 // kWhole: input channels and output tiles are multiples of 64 (what the wide bottleneck networks consist of); the other
 // form takes any layer.  Two kernels, because the general form's masks cost registers and a tenth of the speed.
-// kPair: tiles of 256 pixels x 128 channels, operand rows by tensor copy (see igemm_paired).
-template <bool kWhole, bool kPair>
-__global__ void __launch_bounds__(kGemmThreads, 1) k_igemm(const __grid_constant__ IgemmParams p)
+// kPair: tiles of 256 pixels x 128 channels (see igemm_paired).  kCopy: operand rows by tensor copy (the general form
+// looks at tma_a instead).
+template <bool kWhole, bool kPair, bool kCopy>
+__global__ void __launch_bounds__(igemm_threads(kWhole, kCopy), 1) k_igemm(const __grid_constant__ IgemmParams p)
 {
-    extern __shared__ __align__(128) uint8_t smem[];            // operand stages | requantisation constants | epilogue scratch
-    __shared__ unsigned long long bar_full[kMaxStages], bar_free[kMaxStages], bar_acc_full[2], bar_acc_free[2];
+    extern __shared__ __align__(128) uint8_t smem[];            // operand stages | requantisation constants | scratch of the general form's epilogue
+    constexpr int kEpi = igemm_epi_warps(kWhole, kCopy), kGatherWarps = igemm_gather_warps(kWhole, kCopy), kGemmThreads = igemm_threads(kWhole, kCopy);
+    constexpr int kGatherRows = kGatherWarps ? kTileM / kGatherWarps : 8;          // tile rows of a gather warp
+    const bool copied = kWhole ? kCopy : p.tma_a != 0;
+    __shared__ unsigned long long bar_full[kMaxStages], bar_free[kMaxStages], bar_acc_full[4], bar_acc_free[4];
     __shared__ uint32_t tmem_base_s;
     __shared__ volatile int abort_s;
     chain_start();
@@ -329,8 +336,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_igemm(const __grid_constant
     const uint32_t b_bytes = (uint32_t)n_tile * kBlockK, stage_bytes = a_bytes + b_bytes;
     int4 *cst_s = reinterpret_cast<int4 *>(smem + (size_t)stages * stage_bytes);
     if (tid == 0) {
-        for (int s = 0; s < stages; ++s) { mbar_init(smem_u32(&bar_full[s]), p.tma_a ? 1 : kGatherWarps * 32 + 1); mbar_init(smem_u32(&bar_free[s]), 1); }
-        for (int i = 0; i < 2; ++i) { mbar_init(smem_u32(&bar_acc_full[i]), 1); mbar_init(smem_u32(&bar_acc_free[i]), kEpiWarps * 32); }
+        for (int s = 0; s < stages; ++s) { mbar_init(smem_u32(&bar_full[s]), copied ? 1 : kGatherWarps * 32 + 1); mbar_init(smem_u32(&bar_free[s]), 1); }
+        for (int i = 0; i < p.n_acc; ++i) { mbar_init(smem_u32(&bar_acc_full[i]), 1); mbar_init(smem_u32(&bar_acc_free[i]), kEpi * 32 / p.n_acc); }
         abort_s = 0;
     }
     if (warp == 0) tmem_alloc(smem_u32(&tmem_base_s), (uint32_t)p.tmem_cols);
@@ -349,40 +356,42 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_igemm(const __grid_constant
     const int cblocks = L.cinp / kBlockK, nkb = p.n_blocks;
     bool ok = true;
 
-    if (warp < kAllEpiWarps) {
+    if (warp < kEpi) {
         EpiCtx c;
         c.sbase = sbase; c.tmem = tmem; c.n_tiles = n_tiles; c.grid_n = grid_n; c.tiles_n = tiles_n; c.warp = warp; c.lane = lane;
         c.cst_s = smem_u32(cst_s);
         c.acc_full = smem_u32(&bar_acc_full[0]); c.acc_free = smem_u32(&bar_acc_free[0]);
         c.abort_flag = &abort_s;
-        const bool fast = p.fast_requant && (!p.res || p.fast_residual);
-        if constexpr (kPair) {
-            const bool clamp = p.lo > -128;
-            if (p.res && p.res_short) ok = clamp ? epilogue_pair<3, true>(p, c) : epilogue_pair<3, false>(p, c);
-            else if (p.res) ok = clamp ? epilogue_pair<2, true>(p, c) : epilogue_pair<2, false>(p, c);
-            else ok = clamp ? epilogue_pair<1, true>(p, c) : epilogue_pair<1, false>(p, c);
-        } else
-        if (fast && p.res && p.res_short) ok = epilogue_role<3, kWhole>(p, c);
-        else if (fast && p.res) ok = epilogue_role<2, kWhole>(p, c);
-        else if (fast) ok = epilogue_role<1, kWhole>(p, c);
-        else ok = epilogue_role<0, kWhole>(p, c);
-    } else if (warp < kAllEpiWarps + kGatherWarps) {
-        // ---- operand rows: per reduction block a warp copies 32 tile rows x 64 bytes with four asynchronous 16-byte
-        // copies per lane (lane = 16-byte column x row within a group of eight, so that an instruction reads whole
+        const bool fast = p.fast_requant && (!p.res || p.fast_residual), clamp = p.lo > -128;
+        if constexpr (kWhole) {
+            if (!kPair && !fast) ok = epilogue_whole<0, kPair, true, kEpi>(p, c);              // paired tiles take the 32-bit form only
+            else if (p.res && p.res_short) ok = clamp ? epilogue_whole<3, kPair, true, kEpi>(p, c) : epilogue_whole<3, kPair, false, kEpi>(p, c);
+            else if (p.res) ok = epilogue_whole<2, kPair, true, kEpi>(p, c);
+            else ok = clamp ? epilogue_whole<1, kPair, true, kEpi>(p, c) : epilogue_whole<1, kPair, false, kEpi>(p, c);
+        } else {
+            if (fast && p.res && p.res_short) ok = epilogue_rows<3>(p, c);
+            else if (fast && p.res) ok = epilogue_rows<2>(p, c);
+            else if (fast) ok = epilogue_rows<1>(p, c);
+            else ok = epilogue_rows<0>(p, c);
+        }
+    } else if (warp < kEpi + kGatherWarps) {
+        // ---- operand rows: per reduction block a warp copies its tile rows x 64 bytes with asynchronous 16-byte
+        // copies (lane = 16-byte column x row within a group of eight, so that an instruction reads whole
         // 64-byte rows) whose completion arrives on the stage's barrier.  A row outside the image is copied from a
         // 64-byte run of the input zero-point that follows the repacked weights, so every row takes the same path.
-        const int gw = warp - kAllEpiWarps, chunk = lane & 3, rsub = lane >> 2;
+        const int gw = warp - kEpi, chunk = lane & 3, rsub = lane >> 2;
         const int8_t *zp_src = p.zp_run + chunk * 16;
         const int8_t *in_c = p.in + chunk * 16;
         // K-major core matrices: 16-byte column j of row r at j * (128 rows * 16) + r * 16
-        const uint32_t dst0 = sbase + (uint32_t)chunk * 2048u + (uint32_t)(32 * gw + rsub) * 16u;
+        const uint32_t dst0 = sbase + (uint32_t)chunk * 2048u + (uint32_t)(kGatherRows * gw + rsub) * 16u;
         Ring ring;
         const uint32_t px_per_sample = (uint32_t)(L.hout * L.wout);
-        for (uint32_t t = blockIdx.x; t < n_tiles && ok && !kPair && !p.tma_a; t += grid_n) {
-            const uint32_t m0 = (t / (uint32_t)tiles_n) * kTileM + (uint32_t)(32 * gw + rsub);
-            int iy0[4], ix0[4], off[4];                         // this lane's four rows: 8 apart
+        for (uint32_t t = blockIdx.x; t < n_tiles && ok && !copied; t += grid_n) {
+            const uint32_t m0 = (t / (uint32_t)tiles_n) * kTileM + (uint32_t)(kGatherRows * gw + rsub);
+            constexpr int kRows = kGatherRows / 8;
+            int iy0[kRows], ix0[kRows], off[kRows];             // this lane's rows: 8 apart
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
+            for (int i = 0; i < kRows; ++i) {
                 const uint32_t m = m0 + 8u * (uint32_t)i;
                 const bool valid = m < p.m_total;
                 const uint32_t mm = valid ? m : 0u;
@@ -405,7 +414,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_igemm(const __grid_constant
                     const uint32_t dst = dst0 + (uint32_t)ring.s * stage_bytes;
                     const int add = (r * L.win + sx) * L.cinp + c16 * 16;
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
+                    for (int i = 0; i < kRows; ++i) {
                         const bool inside = (unsigned)(iy0[i] + r) < (unsigned)L.hin && (unsigned)(ix0[i] + sx) < (unsigned)L.win && u < p.units;
                         cp_async16_cached(dst + (uint32_t)i * 128u, inside ? p.in + (off[i] + add) : zp_src);
                     }
@@ -420,9 +429,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_igemm(const __grid_constant
             }
             for (int tap = 0, r = 0, sx = 0; tap < L.kh * L.kw && ok; ++tap, sx = (sx + 1 == L.kw) ? 0 : sx + 1, r += (sx == 0)) {
                 const int tap_off = (r * L.win + sx) * L.cinp;
-                bool inside[4];
+                bool inside[kRows];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) inside[i] = (unsigned)(iy0[i] + r) < (unsigned)L.hin && (unsigned)(ix0[i] + sx) < (unsigned)L.win;
+                for (int i = 0; i < kRows; ++i) inside[i] = (unsigned)(iy0[i] + r) < (unsigned)L.hin && (unsigned)(ix0[i] + sx) < (unsigned)L.win;
                 for (int cb = 0; cb < cblocks; ++cb, ring.advance(stages)) {
                     if (ring.use >= 1) {
                         ok = wait_bar<kHintLoad>(smem_u32(&bar_free[ring.s]), (uint32_t)(ring.use - 1) & 1u, &abort_s);
@@ -430,7 +439,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_igemm(const __grid_constant
                     }
                     const uint32_t dst = dst0 + (uint32_t)ring.s * stage_bytes;
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
+                    for (int i = 0; i < kRows; ++i) {
                         cp_async16_cached(dst + (uint32_t)i * 128u, inside[i] ? in_c + (off[i] + tap_off + cb * kBlockK) : zp_src);
                     }
                     cp_async_arrive(smem_u32(&bar_full[ring.s]));
@@ -438,14 +447,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_igemm(const __grid_constant
             }
         }
         cp_async_wait_all();
-    } else if (warp == kAllEpiWarps + kGatherWarps) {
+    } else if (warp == kEpi + kGatherWarps) {
         // ---- one thread issues the MMAs: two K-steps per stage, accumulators alternate between two column ranges
         if (lane == 0) {
             const uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n_tile >> 3) << 17) | ((uint32_t)(kTileM >> 4) << 24);
             Ring ring;
             int j = 0;
             for (uint32_t t = blockIdx.x; t < n_tiles && ok; t += grid_n, ++j) {
-                const int buf = j & 1, au = j >> 1;
+                const int buf = j & (p.n_acc - 1), au = p.n_acc == 4 ? j >> 2 : j >> 1;
                 if (au >= 1) {
                     ok = wait_bar<kHintMma>(smem_u32(&bar_acc_free[buf]), (uint32_t)(au - 1) & 1u, &abort_s);
                     if (!ok) break;
@@ -474,14 +483,18 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_igemm(const __grid_constant
         if (lane == 0 && !p.debug_stall) {
             Ring ring;
             for (uint32_t t = blockIdx.x; t < n_tiles && ok; t += grid_n) {
+                // the tile's residual bytes, about a tile ahead of their use (258 -> 253 us)
+                if (kWhole && p.prefetch_res)
+                    asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];"
+                                 ::"l"(reinterpret_cast<uint64_t>(&p.tmap_res)), "r"((int)(t % (uint32_t)tiles_n) * n_tile), "r"((int)(t / (uint32_t)tiles_n) * (kPair ? 2 * kTileM : kTileM)) : "memory");
                 const int8_t *wtile = p.wpack + (size_t)(t % tiles_n) * (size_t)nkb * b_bytes;
                 for (int kb = 0; kb < nkb; ++kb, ring.advance(stages)) {
                     if (ring.use >= 1) {
                         ok = wait_bar<kHintLoad>(smem_u32(&bar_free[ring.s]), (uint32_t)(ring.use - 1) & 1u, &abort_s);
                         if (!ok) break;
                     }
-                    mbar_expect_tx(smem_u32(&bar_full[ring.s]), p.tma_a ? a_bytes + b_bytes : b_bytes);
-                    if (p.tma_a) {
+                    mbar_expect_tx(smem_u32(&bar_full[ring.s]), copied ? a_bytes + b_bytes : b_bytes);
+                    if (copied) {
                         // box {16 bytes, 128 pixels, 4 columns} of the 3-D view lands as [column][pixel][16 bytes], which is
                         // the K-major core-matrix layout; pixels beyond the last one are filled with zeros and never stored
 #pragma unroll
@@ -782,6 +795,17 @@ int igemm_tile_n(const GLayer &G)
 
 namespace {
 
+// Whole tiles: input channels and the output channels' tiles are multiples of 64.
+bool igemm_whole(const GLayer &G) { return G.cinp % kBlockK == 0 && igemm_tile_n(G) % 64 == 0 && G.coutp % igemm_tile_n(G) == 0; }
+
+// The output channel of a column of the accumulators: in whole tiles, column 16 t + 8 h + 2 c + e of 64 is channel
+// 16 c + 4 t + 2 h + e (see epilogue_whole).
+int igemm_channel(const GLayer &G, int col)
+{
+    if (!igemm_whole(G)) return col;
+    return (col & ~63) | ((col & 6) << 3) | ((col & 48) >> 2) | ((col & 8) >> 2) | (col & 1);
+}
+
 int igemm_tiles(const GLayer &G) { return igemm_pairable(G) ? G.coutp / kPairN : (G.coutp + 255) / 256; }
 int igemm_units(const GLayer &G) { return G.kh * G.kw * (G.cinp / 16); }
 int igemm_blocks(const GLayer &G) { return (igemm_units(G) + 3) / 4; }
@@ -796,7 +820,7 @@ struct IgemmSmem {
 IgemmSmem igemm_smem(const GLayer &G, bool paired)
 {
     const size_t n_tile = (size_t)igemm_tile_n(G), rows = paired ? 2 : 1;
-    return IgemmSmem{(size_t)igemm_tiles(G) * n_tile * 16, (size_t)kAllEpiWarps * 32 * rows * epi_row_stride((int)n_tile),
+    return IgemmSmem{(size_t)igemm_tiles(G) * n_tile * 16, (size_t)kRowWarps * 32 * rows * epi_row_stride((int)n_tile),
                      (size_t)kTileM * kBlockK * rows + n_tile * kBlockK};
 }
 
@@ -826,11 +850,23 @@ void igemm_pack_weights(const GLayer &G, const int8_t *w, int8_t *out)
             const int tap = u / c16s, c0 = (u - tap * c16s) * 16;
             for (int n = 0; n < n_tile; ++n)
                 for (int e = 0; e < 16; ++e, ++at) {
-                    const int oc = t * n_tile + n, ci = c0 + e;
+                    const int oc = t * n_tile + igemm_channel(G, n), ci = c0 + e;
                     out[at] = (u < units && oc < G.cout && ci < G.cin) ? w[((size_t)oc * G.cin + ci) * taps + tap] : (int8_t)0;
                 }
         }
     for (int e = 0; e < kBlockK; ++e) out[at + e] = (int8_t)G.zp_in;
+}
+
+// The constants of igemm_constants in the order in which the kernel reads them: the four of channels 16 c + 4 t + k, c = 0 to 3, of
+// 64 lie side by side.
+void igemm_order_constants(const GLayer &G, int32_t *out4, int n_out)
+{
+    if (!igemm_whole(G)) return;
+    const std::vector<int32_t> in(out4, out4 + 4 * (size_t)n_out);
+    for (int o = 0; o < n_out; ++o) {
+        const int at = (o & ~63) | (o & 15) << 2 | ((o >> 4) & 3);
+        memcpy(out4 + 4 * (size_t)at, &in[4 * (size_t)o], 16);
+    }
 }
 
 // 32-bit row and byte offsets inside the tensor-core kernels
@@ -936,9 +972,10 @@ cudaError_t tc_prepare(TcDevice *dev, int ordinal)
     int major = 0;
     d.chained = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, ordinal) == cudaSuccess && major >= 9;
     cudaError_t e = cudaDeviceGetAttribute(&d.n_sms, cudaDevAttrMultiProcessorCount, ordinal);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<true, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<true, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_igemm<false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_stem, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStemSmemLimit);
     if (e == cudaSuccess) e = halo_prepare();
     if (e != cudaSuccess) { cudaGetLastError(); return e; }
@@ -1001,19 +1038,31 @@ cudaError_t launch_igemm_conv(const TcDevice &dev, const GLayer &G, const int8_t
     const bool paired = igemm_pairable(G) && igemm_smem(G, true).fits() && p.tma_a && p.fast_requant && (!res || p.fast_residual) &&
                         igemm_paired(p.tiles_m, (uint32_t)p.tiles_n, (uint32_t)dev.n_sms);
     if (paired) p.tiles_m = (p.tiles_m + 1) / 2;
-    p.acc_stride = paired ? 2 * kPairN : (p.n_tile + 31) & ~31;          // the epilogue loads 32 columns at a time
+    const bool whole = igemm_whole(G);
+    p.acc_stride = paired ? 2 * kPairN : (p.n_tile + 31) & ~31;          // epilogue_rows loads 32 columns at a time
+    // the same view's encoder for the residual operand (its rows are a multiple of 16 bytes, its boxes at most 256 x 256)
+    p.prefetch_res = 0;
+    memset(&p.tmap_res, 0, sizeof(p.tmap_res));
+    if (const EncodeFn encode = whole && res && p.tma_a ? (EncodeFn)dev.encode : nullptr) {
+        const cuuint64_t dims[2] = {(cuuint64_t)G.coutp, (cuuint64_t)p.m_total}, strides[1] = {(cuuint64_t)G.coutp};
+        const cuuint32_t box[2] = {(cuuint32_t)p.n_tile, (cuuint32_t)(paired ? 2 * kTileM : kTileM)}, estr[2] = {1, 1};
+        p.prefetch_res = encode(&p.tmap_res, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<int8_t *>(res), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                                CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    }
+    p.n_acc = whole && p.tma_a && p.acc_stride <= 64 ? 4 : 2;
     p.tmem_cols = 64;
-    while (p.tmem_cols < 2 * p.acc_stride) p.tmem_cols <<= 1;
+    while (p.tmem_cols < p.n_acc * p.acc_stride) p.tmem_cols <<= 1;
     // as many operand stages as fit beside the constants, at most kMaxStages
-    const IgemmSmem s = igemm_smem(G, paired);
+    IgemmSmem s = igemm_smem(G, paired);
+    if (whole) s.scratch = 0;
     p.stages = (int)std::min<size_t>(kMaxStages, (kSmemLimit - s.cst - s.scratch) / s.stage);
     p.scratch_off = (uint32_t)((size_t)p.stages * s.stage + s.cst);
     const size_t smem = (size_t)p.stages * s.stage + s.cst + s.scratch;
     // persistent: one CTA per SM (shared memory and the 512 tensor-memory columns allow no second one at N = 256)
     const uint32_t n_tiles = p.tiles_m * (uint32_t)p.tiles_n;
     const unsigned grid = std::min<uint32_t>(n_tiles, (uint32_t)dev.n_sms);
-    const bool whole = G.cinp % kBlockK == 0 && p.n_tile % 64 == 0 && G.coutp == p.tiles_n * p.n_tile;
-    return launch_chained(dev.chained, paired ? k_igemm<true, true> : whole ? k_igemm<true, false> : k_igemm<false, false>, dim3(grid), kGemmThreads, smem, st, p);
+    return launch_chained(dev.chained, paired ? k_igemm<true, true, true> : !whole ? k_igemm<false, false, false> : p.tma_a ? k_igemm<true, false, true> : k_igemm<true, false, false>,
+                          dim3(grid), igemm_threads(whole, p.tma_a != 0), smem, st, p);
 }
 
 // ---- the stem

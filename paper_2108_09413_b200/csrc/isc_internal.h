@@ -76,7 +76,7 @@ cudaError_t launch_first_conv(const GLayer &L, const uint8_t *x_chw, int in_c, c
 cudaError_t launch_noisy_input(const uint8_t *x_chw, int in_c, int in_h, int in_w, const NoiseStream &ns,
                                int batch, int32_t *out_chw, cudaStream_t st);
 cudaError_t launch_conv(const GLayer &L, int batch, const int8_t *in, const int8_t *res, int8_t *out,
-                        cudaStream_t st, bool chained = false);
+                        cudaStream_t st);
 cudaError_t launch_gavgpool(const GLayer &L, int batch, const int8_t *in, int8_t *out, cudaStream_t st, bool chained = false);
 cudaError_t launch_maxpool(const GLayer &L, int batch, const int8_t *in, int8_t *out, cudaStream_t st, bool chained = false);
 cudaError_t launch_votes(const int8_t *logits_nhwc, int cp, int n_classes, const SampleRun &run, int batch, int32_t *counts,
@@ -113,6 +113,7 @@ ResidualForm residual_form(int res_mult, int res_shift, int zp_res, int32_t *c);
 // whether the layer qualifies for it (every shift >= 2).
 bool igemm_constants(const GLayer &G, const int32_t *bias_folded, const int32_t *mult, const int32_t *shift, int32_t *out4, int n_out,
                      bool has_residual, ResidualForm *form);
+void igemm_order_constants(const GLayer &G, int32_t *out4, int n_out);      // ... in the order in which k_igemm reads them
 // `cst` / `fast`: what igemm_constants produced (device copy).  `err` (device) receives a non-zero word if a bounded
 // wait inside the kernel expired.  `debug_stall`: the kernel's weights are never sent, so that its waits run out
 // (after their 2 s limit) and the CTAs leave through the abort path -- nothing faults or hangs.  `tensor_copy`: a

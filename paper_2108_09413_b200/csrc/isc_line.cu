@@ -201,19 +201,6 @@ __device__ __forceinline__ void commit_to(uint32_t bar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
-// 16 columns of half a warp's tensor-memory lanes (16, from `taddr` on) in fragment form: a thread holds columns 2 c, 2 c + 1
-// (c = lane mod 4) of rows lane / 4 (v[0], v[1]) and lane / 4 + 8 (v[2], v[3]), then the same eight columns on (v[4..7]).
-__device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, int (&v)[8])
-{
-    asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "r"(taddr) : "memory");
-}
-// every load issued so far is complete; names the registers so that no use can move above it
-__device__ __forceinline__ void tmem_ld_frag_wait(int (&v)[8])
-{
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]) :: "memory");
-}
 // 16 columns of all 32 lanes take the values at `vec` (shared memory), one per column.  (In fragment form, four values per
 // thread, the store's eight registers had to be copied together each time: 230 instead of 60 cycles of a pass of 1,050.)
 __device__ __forceinline__ void tmem_st_columns(uint32_t taddr, uint4 a, uint4 b, uint4 c, uint4 d)
