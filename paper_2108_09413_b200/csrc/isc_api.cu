@@ -460,7 +460,7 @@ int generic_forward(isc_model *m, int8_t *const *bufs, const uint8_t *d_x, const
         const int8_t *res = L.res_tensor >= 0 ? bufs[m->tensor_buf[(size_t)L.res_tensor]] : nullptr;
         cudaError_t e;
         if (i == 0 && tensor_cores && m->wpacks[0])
-            e = launch_stem_conv(G, m->wpacks[0], m->tc_cst[0], m->tc_fast[0] != 0, d_x, m->in_c, ns, run, batch, out, d_err, st, false, chained && m->tc.chained);
+            e = launch_stem_conv(m->tc, G, m->wpacks[0], m->tc_cst[0], m->tc_fast[0] != 0, d_x, m->in_c, ns, run, batch, out, d_err, st, false, chained);
         else if (i == 0) e = launch_first_conv(G, d_x, m->in_c, ns, run, batch, out, st);
         else if (tensor_cores && m->hpacks[(size_t)i] && halo_offsets_fit(G, batch))
             e = launch_halo_conv(m->tc, G, m->hpacks[(size_t)i], m->tc_cst[(size_t)i], m->tc_fast[(size_t)i] != 0, m->tc_resk[(size_t)i], batch, in, res, out, d_err, st);
@@ -673,7 +673,7 @@ int stalled_launch(isc_model *m, size_t li, cudaStream_t st, int32_t *err, int32
     const bool fast = m->tc_fast[li] != 0;
     const auto t0 = std::chrono::steady_clock::now();
     cudaError_t e;
-    if (li == 0) e = launch_stem_conv(G, m->wpacks[0], m->tc_cst[0], fast, d_x, m->in_c, make_stream(m, 1, 0, 1, 0), SampleRun{0, 0, 1, 0, 0, 0, 1}, 1, out, m->d_tc_err, st, true);
+    if (li == 0) e = launch_stem_conv(m->tc, G, m->wpacks[0], m->tc_cst[0], fast, d_x, m->in_c, make_stream(m, 1, 0, 1, 0), SampleRun{0, 0, 1, 0, 0, 0, 1}, 1, out, m->d_tc_err, st, true);
     else if (m->hpacks[li]) e = launch_halo_conv(m->tc, G, m->hpacks[li], m->tc_cst[li], fast, m->tc_resk[li], 1, in, res, out, m->d_tc_err, st, true);
     else e = launch_igemm_conv(m->tc, G, m->wpacks[li], m->tc_cst[li], fast, m->tc_resk[li], 1, in, res, out, m->d_tc_err, st, true);
     if (e != cudaSuccess) return ISC_ERR_CUDA;

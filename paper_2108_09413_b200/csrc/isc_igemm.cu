@@ -530,7 +530,8 @@ __global__ void __launch_bounds__(igemm_threads(kWhole, kCopy), 1) k_igemm(const
 // ------------------------------------------------------------------ first convolution on the tensor cores
 //
 // The stem of a network whose input is the noisy image (Def. 3.4): a k x k convolution over <= 4 input channels.
-// One CTA = one sample x one band of output rows.  The band's input rows are drawn (Philox -> inverse-CDF table ->
+// A piece of work is one sample x one band of output rows; a CTA takes every grid-th (with a CTA for each, the set-up, the
+// weights and the noise tables' copy were a sixth of a small image's time: 3 x 3 on 32 x 32, 5,100 samples: 388 -> 330 us).  The band's input rows are drawn (Philox -> inverse-CDF table ->
 // add -> saturate to 0..255, Def. 3.3 / Eq. 2) into a shared-memory patch as 4 bytes per pixel, padded with the input
 // zero-point, and never written to memory.  The GEMM takes one filter row per K-step: eight horizontally adjacent
 // pixels x 4 bytes = 32 bytes of K (pixels beyond the filter width meet zero weights), so 128 output pixels are `kh`
@@ -546,6 +547,7 @@ __global__ void __launch_bounds__(igemm_threads(kWhole, kCopy), 1) k_igemm(const
 struct StemParams {
     GLayer L;
     int in_c, band_rows, n_bands, tmem_cols;
+    uint32_t n_items;                        // samples * bands
     int pitch, rows_class, planes;           // positions of a row; rows of one (row mod stride) class; planes of positions
     uint32_t plane_pos, k_step;              // positions of a plane; bytes from the first to the second 16 bytes of K
     uint32_t w_bytes, pos_off, patch_off;
@@ -564,24 +566,24 @@ struct StemParams {
 
 // Rows 32 (warp mod 4) .. + 31 of both operands of every tile, half of the channels.
 template <bool kFast, bool kClamp>
-__device__ __forceinline__ bool stem_epilogue(const StemParams &p, uint32_t tmem, uint32_t cst, uint32_t bar_full, uint32_t bar_free, int n_tiles, int band_rows,
-                                              size_t first_px, const volatile int *abort_flag)
+__device__ __forceinline__ bool stem_epilogue(const StemParams &p, uint32_t tmem, uint32_t cst, uint32_t bar_full, uint32_t bar_free, uint32_t first_tile, int n_tiles,
+                                              int band_rows, size_t first_px, const volatile int *abort_flag)
 {
     const GLayer &L = p.L;
     const int N = L.coutp, row = (int)threadIdx.x & (kTileM - 1), half = (N / 16 + 1) / 2 * 16;
     const int c_begin = threadIdx.x >= kTileM ? half : 0, c_end = threadIdx.x >= kTileM ? N : half;
     const uint32_t lanes = tmem + ((uint32_t)(row & ~31) << 16);
     for (int t = 0; t < n_tiles; ++t) {
-        const int slot = p.slots == 2 ? t & 1 : 0, use = p.slots == 2 ? t >> 1 : t;
+        const uint32_t tile = first_tile + (uint32_t)t, slot = p.slots == 2 ? tile & 1u : 0u, use = p.slots == 2 ? tile >> 1 : tile;
         int8_t *dst[2];
 #pragma unroll
         for (int mt = 0; mt < 2; ++mt) {
             const int f = t * 2 * kTileM + mt * kTileM + row, y = f / p.pitch, x = f - y * p.pitch;
             dst[mt] = y < band_rows && x < L.wout ? p.out + (first_px + (size_t)(y * L.wout + x)) * L.coutp : nullptr;
         }
-        if (!wait_bar<kHintEpi>(bar_full + 8u * (uint32_t)slot, (uint32_t)use & 1u, abort_flag)) return false;
+        if (!wait_bar<kHintEpi>(bar_full + 8u * slot, use & 1u, abort_flag)) return false;
         tc_fence_after();
-        const uint32_t acc = lanes + (uint32_t)(slot * 2 * N);
+        const uint32_t acc = lanes + slot * (uint32_t)(2 * N);
 #pragma unroll 1
         for (int c0 = c_begin; c0 < c_end; c0 += 16) {
             int a[2][16];
@@ -605,7 +607,7 @@ __device__ __forceinline__ bool stem_epilogue(const StemParams &p, uint32_t tmem
                 if (dst[mt]) *reinterpret_cast<uint4 *>(dst[mt] + c0) = o[mt];
         }
         tc_fence_before();
-        mbar_arrive(bar_free + 8u * (uint32_t)slot);
+        mbar_arrive(bar_free + 8u * slot);
     }
     return true;
 }
@@ -640,114 +642,124 @@ __global__ void __launch_bounds__(kStemThreads, 2) k_stem(const __grid_constant_
         bulk_g2s(sbase, p.wpack, p.w_bytes, smem_u32(&bar_w));
     }
 
-    // ---- the band's noisy input rows
-    const int b = blockIdx.y;
-    const SampleRun::Sample sample = p.run.at((uint32_t)b);
-    const int64_t j = (int64_t)sample.number;
-    const uint64_t image_id = p.run.image_id0 + sample.image;
-    const uint32_t ctr2 = (uint32_t)image_id;
-    const uint8_t *x = p.x + sample.image * (size_t)(p.in_c * L.hin * L.win);
-    const int oy0 = blockIdx.x * p.band_rows, oy1 = min(L.hout, oy0 + p.band_rows);
-    const int wpad = L.win + 2 * L.pad + 8;                     // 8 more pixels: the windows of the last columns stay inside
-    const int iy0 = oy0 * L.stride - L.pad;
-    const int rows_in = (oy1 - oy0 - 1) * L.stride + kh;
     uint32_t *patch = reinterpret_cast<uint32_t *>(smem + p.patch_off);
     const uint32_t zp_fill = (uint32_t)(L.zp_in & 0xFF) * (0x01010101u >> (8 * (4 - p.in_c)));
-    for (int i = tid; i < rows_in * wpad; i += kStemThreads) patch[i] = zp_fill;
     if (p.tab_off && p.ns.guide) {
         // cumulative table, then the guide table that follows it in memory
         uint32_t *tab = reinterpret_cast<uint32_t *>(smem + p.tab_off);
         for (int i = tid; i < 2 * p.ns.T + 1 + kNoiseGuide + 1; i += kStemThreads) tab[i] = __ldg(p.ns.cum + i);
     }
-    __syncthreads();
-    const int vy0 = max(0, iy0), vy1 = min(L.hin, iy0 + rows_in);
-    if (vy1 > vy0) {
-        uint8_t *pb = reinterpret_cast<uint8_t *>(patch);
-        const uint32_t ctr3 = sample.phase | ((uint32_t)(image_id >> 32) & 0xFFFFu) << 16 | (uint32_t)(((j >> 32) & 0xFF) << 8);
-        const uint32_t ctr1 = (uint32_t)(j & 0xFFFFFFFFll);
-        if ((L.win & 3) == 0 && p.ns.guide) {
-            // every Philox block (four consecutive elements of the CHW order) lies within one image row: a thread
-            // takes whole blocks, all channels of the band's rows as one index space, the four searches interleaved
-            const int qpr = L.win >> 2, qpc = (vy1 - vy0) * qpr;
-            for (int i = tid; i < p.in_c * qpc; i += kStemThreads) {
-                const int c = i / qpc, ic = i - c * qpc;
-                const int hr = ic / qpr, wq = ic - hr * qpr;
-                const int h = vy0 + hr;
-                const uint32_t e = (uint32_t)((c * L.hin + h) * L.win) + 4u * (uint32_t)wq;
-                const uint4 r = philox4x32_10(make_uint4(e >> 2, ctr1, ctr2, ctr3), p.ns.key0, p.ns.key1);
-                const uint32_t clean = __ldg(reinterpret_cast<const uint32_t *>(x + e));
-                int z[4];
-                if (p.tab_off) noise_levels4_shared(r, sbase + p.tab_off, sbase + p.tab_off + 4u * (uint32_t)(2 * p.ns.T + 1), p.ns.T, p.ns.guide_steps, z);
-                else noise_levels4(r, p.ns.cum, p.ns.guide, p.ns.T, p.ns.guide_steps, z);
-                uint8_t *dst = pb + ((h - iy0) * wpad + (4 * wq + L.pad)) * 4 + c;
+    bool ok = true;
+    uint32_t first_tile = 0;                                    // of the item, counted over the CTA's items
+    for (uint32_t item = blockIdx.x; item < p.n_items; item += gridDim.x) {
+        // ---- the band's noisy input rows
+        const uint32_t b = item / (uint32_t)p.n_bands, band = item - b * (uint32_t)p.n_bands;
+        const SampleRun::Sample sample = p.run.at(b);
+        const int64_t j = (int64_t)sample.number;
+        const uint64_t image_id = p.run.image_id0 + sample.image;
+        const uint32_t ctr2 = (uint32_t)image_id;
+        const uint8_t *x = p.x + sample.image * (size_t)(p.in_c * L.hin * L.win);
+        const int oy0 = (int)band * p.band_rows, oy1 = min(L.hout, oy0 + p.band_rows);
+        const int wpad = L.win + 2 * L.pad + 8;                     // 8 more pixels: the windows of the last columns stay inside
+        const int iy0 = oy0 * L.stride - L.pad;
+        const int rows_in = (oy1 - oy0 - 1) * L.stride + kh;
+        for (int i = tid; i < rows_in * wpad; i += kStemThreads) patch[i] = zp_fill;
+        __syncthreads();
+        const int vy0 = max(0, iy0), vy1 = min(L.hin, iy0 + rows_in);
+        if (vy1 > vy0) {
+            uint8_t *pb = reinterpret_cast<uint8_t *>(patch);
+            const uint32_t ctr3 = sample.phase | ((uint32_t)(image_id >> 32) & 0xFFFFu) << 16 | (uint32_t)(((j >> 32) & 0xFF) << 8);
+            const uint32_t ctr1 = (uint32_t)(j & 0xFFFFFFFFll);
+            if ((L.win & 3) == 0 && p.ns.guide) {
+                // every Philox block (four consecutive elements of the CHW order) lies within one image row: a thread
+                // takes whole blocks, all channels of the band's rows as one index space, the four searches interleaved
+                const int qpr = L.win >> 2, qpc = (vy1 - vy0) * qpr;
+                for (int i = tid; i < p.in_c * qpc; i += kStemThreads) {
+                    const int c = i / qpc, ic = i - c * qpc;
+                    const int hr = ic / qpr, wq = ic - hr * qpr;
+                    const int h = vy0 + hr;
+                    const uint32_t e = (uint32_t)((c * L.hin + h) * L.win) + 4u * (uint32_t)wq;
+                    const uint4 r = philox4x32_10(make_uint4(e >> 2, ctr1, ctr2, ctr3), p.ns.key0, p.ns.key1);
+                    const uint32_t clean = __ldg(reinterpret_cast<const uint32_t *>(x + e));
+                    int z[4];
+                    if (p.tab_off) noise_levels4_shared(r, sbase + p.tab_off, sbase + p.tab_off + 4u * (uint32_t)(2 * p.ns.T + 1), p.ns.T, p.ns.guide_steps, z);
+                    else noise_levels4(r, p.ns.cum, p.ns.guide, p.ns.T, p.ns.guide_steps, z);
+                    uint8_t *dst = pb + ((h - iy0) * wpad + (4 * wq + L.pad)) * 4 + c;
 #pragma unroll
-                for (int k = 0; k < 4; ++k) dst[4 * k] = (uint8_t)min(255, max(0, (int)((clean >> (8 * k)) & 0xFFu) + z[k]));
-            }
-        } else {
-            for (int c = 0; c < p.in_c; ++c) {
-                const int64_t e_begin = ((int64_t)c * L.hin + vy0) * L.win, e_end = ((int64_t)c * L.hin + vy1) * L.win;
-                for (int64_t q = (e_begin >> 2) + tid; q < ((e_end + 3) >> 2); q += kStemThreads) {
-                    const uint4 r = philox4x32_10(make_uint4((uint32_t)q, ctr1, ctr2, ctr3), p.ns.key0, p.ns.key1);
-                    const uint32_t u[4] = {r.x, r.y, r.z, r.w};
+                    for (int k = 0; k < 4; ++k) dst[4 * k] = (uint8_t)min(255, max(0, (int)((clean >> (8 * k)) & 0xFFu) + z[k]));
+                }
+            } else {
+                for (int c = 0; c < p.in_c; ++c) {
+                    const int64_t e_begin = ((int64_t)c * L.hin + vy0) * L.win, e_end = ((int64_t)c * L.hin + vy1) * L.win;
+                    for (int64_t q = (e_begin >> 2) + tid; q < ((e_end + 3) >> 2); q += kStemThreads) {
+                        const uint4 r = philox4x32_10(make_uint4((uint32_t)q, ctr1, ctr2, ctr3), p.ns.key0, p.ns.key1);
+                        const uint32_t u[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const int64_t e = q * 4 + k;
-                        if (e < e_begin || e >= e_end) continue;
-                        const int rem = (int)(e - (int64_t)c * L.hin * L.win);
-                        const int h = rem / L.win, w = rem - h * L.win;
-                        int v = (int)__ldg(x + e) + (p.ns.guide ? noise_level_guided(u[k], p.ns.cum, p.ns.guide, p.ns.T) : noise_level(u[k], p.ns.cum, p.ns.T));
-                        v = min(255, max(0, v));
-                        pb[((h - iy0) * wpad + (w + L.pad)) * 4 + c] = (uint8_t)v;
+                        for (int k = 0; k < 4; ++k) {
+                            const int64_t e = q * 4 + k;
+                            if (e < e_begin || e >= e_end) continue;
+                            const int rem = (int)(e - (int64_t)c * L.hin * L.win);
+                            const int h = rem / L.win, w = rem - h * L.win;
+                            int v = (int)__ldg(x + e) + (p.ns.guide ? noise_level_guided(u[k], p.ns.cum, p.ns.guide, p.ns.T) : noise_level(u[k], p.ns.cum, p.ns.T));
+                            v = min(255, max(0, v));
+                            pb[((h - iy0) * wpad + (w + L.pad)) * 4 + c] = (uint8_t)v;
+                        }
                     }
                 }
             }
         }
-    }
-    __syncthreads();
+        __syncthreads();
 
-    // ---- the patch as positions (see above)
-    const uint32_t pos = sbase + p.pos_off;
-    for (int i = tid; i < p.planes * rows_in * p.pitch; i += kStemThreads) {
-        int y = i / p.pitch;
-        const int x = i - y * p.pitch, plane = y >= rows_in ? 1 : 0;
-        y -= plane * rows_in;
-        const uint32_t *src = patch + y * wpad + x * L.stride + 4 * plane;
-        const int at = (y % L.stride * p.rows_class + y / L.stride) * p.pitch + x;
-        st_shared_v4(pos + ((uint32_t)plane * p.plane_pos + (uint32_t)at) * 16u, make_uint4(src[0], src[1], src[2], src[3]));
-    }
-    fence_proxy_async();
-    __syncthreads();
-
-    chain_wait();                                         // the noise needed nothing of the launch before; the output buffer does
-    const int band_rows = oy1 - oy0, n_tiles = (band_rows * p.pitch + 2 * kTileM - 1) / (2 * kTileM);
-    bool ok = true;
-    if (warp < kStemEpi) {
-        const size_t first_px = ((size_t)b * L.hout + oy0) * L.wout;
-        const uint32_t cst = smem_u32(cst_s), full = smem_u32(&bar_full[0]), free_ = smem_u32(&bar_free[0]);
-        if (!p.fast_requant) ok = stem_epilogue<false, true>(p, tmem, cst, full, free_, n_tiles, band_rows, first_px, &abort_s);
-        else if (p.lo > -128) ok = stem_epilogue<true, true>(p, tmem, cst, full, free_, n_tiles, band_rows, first_px, &abort_s);
-        else ok = stem_epilogue<true, false>(p, tmem, cst, full, free_, n_tiles, band_rows, first_px, &abort_s);
-    } else {
-        const uint32_t lane0 = elect_one() ? 1u : 0u;
-        const uint32_t idesc = (2u << 4) | (0u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(kTileM >> 4) << 24);
-        ok = wait_warp(smem_u32(&bar_w), 0u, &abort_s);
-        tc_fence_after();
-        for (int t = 0; t < n_tiles && ok; ++t) {
-            const int slot = p.slots == 2 ? t & 1 : 0, use = p.slots == 2 ? t >> 1 : t;
-            if (use >= 1) {
-                ok = wait_warp(smem_u32(&bar_free[slot]), (uint32_t)(use - 1) & 1u, &abort_s);
-                if (!ok) break;
-                tc_fence_after();
-            }
-            for (int mt = 0; mt < 2; ++mt)
-                for (int r = 0; r < kh; ++r) {
-                    const int at = (r % L.stride * p.rows_class + r / L.stride) * p.pitch + t * 2 * kTileM + mt * kTileM;
-                    const uint64_t ad = make_desc(pos + (uint32_t)at * 16u, p.k_step, 128u);
-                    const uint64_t bd = make_desc(sbase + (uint32_t)r * 2u * (uint32_t)N * 16u, (uint32_t)N * 16u, 128u);
-                    mma_i8_if(lane0, tmem + (uint32_t)((slot * 2 + mt) * N), ad, bd, idesc, r > 0 ? 1u : 0u);
-                }
-            commit_if(lane0, smem_u32(&bar_full[slot]));
+        // ---- the patch as positions (see above)
+        const uint32_t pos = sbase + p.pos_off;
+        for (int i = tid; i < p.planes * rows_in * p.pitch; i += kStemThreads) {
+            int y = i / p.pitch;
+            const int x = i - y * p.pitch, plane = y >= rows_in ? 1 : 0;
+            y -= plane * rows_in;
+            const uint32_t *src = patch + y * wpad + x * L.stride + 4 * plane;
+            const int at = (y % L.stride * p.rows_class + y / L.stride) * p.pitch + x;
+            st_shared_v4(pos + ((uint32_t)plane * p.plane_pos + (uint32_t)at) * 16u, make_uint4(src[0], src[1], src[2], src[3]));
         }
+        fence_proxy_async();
+        __syncthreads();
+
+        if (first_tile == 0) chain_wait();                    // the noise needed nothing of the launch before; the output buffer does
+        const int band_rows = oy1 - oy0, n_tiles = (band_rows * p.pitch + 2 * kTileM - 1) / (2 * kTileM);
+        if (warp < kStemEpi) {
+            const size_t first_px = ((size_t)b * L.hout + oy0) * L.wout;
+            const uint32_t cst = smem_u32(cst_s), full = smem_u32(&bar_full[0]), free_ = smem_u32(&bar_free[0]);
+            if (!p.fast_requant) ok = stem_epilogue<false, true>(p, tmem, cst, full, free_, first_tile, n_tiles, band_rows, first_px, &abort_s);
+            else if (p.lo > -128) ok = stem_epilogue<true, true>(p, tmem, cst, full, free_, first_tile, n_tiles, band_rows, first_px, &abort_s);
+            else ok = stem_epilogue<true, false>(p, tmem, cst, full, free_, first_tile, n_tiles, band_rows, first_px, &abort_s);
+        } else {
+            const uint32_t lane0 = elect_one() ? 1u : 0u;
+            const uint32_t idesc = (2u << 4) | (0u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(kTileM >> 4) << 24);
+            if (first_tile == 0) ok = wait_warp(smem_u32(&bar_w), 0u, &abort_s);
+            tc_fence_after();
+            for (int t = 0; t < n_tiles && ok; ++t) {
+                const uint32_t tile = first_tile + (uint32_t)t, slot = p.slots == 2 ? tile & 1u : 0u, use = p.slots == 2 ? tile >> 1 : tile;
+                if (use >= 1) {
+                    ok = wait_warp(smem_u32(&bar_free[slot]), (use - 1u) & 1u, &abort_s);
+                    if (!ok) break;
+                    tc_fence_after();
+                }
+                for (int mt = 0; mt < 2; ++mt)
+                    for (int r = 0; r < kh; ++r) {
+                        const int at = (r % L.stride * p.rows_class + r / L.stride) * p.pitch + t * 2 * kTileM + mt * kTileM;
+                        const uint64_t ad = make_desc(pos + (uint32_t)at * 16u, p.k_step, 128u);
+                        const uint64_t bd = make_desc(sbase + (uint32_t)r * 2u * (uint32_t)N * 16u, (uint32_t)N * 16u, 128u);
+                        mma_i8_if(lane0, tmem + (slot * 2u + (uint32_t)mt) * (uint32_t)N, ad, bd, idesc, r > 0 ? 1u : 0u);
+                    }
+                commit_if(lane0, smem_u32(&bar_full[slot]));
+            }
+        }
+        first_tile += (uint32_t)n_tiles;
+        if (!ok) abort_s = 1;
+        // the item's MMAs are complete (their accumulators have been read): the next one may overwrite positions and patch
+        tc_fence_before();
+        __syncthreads();
+        tc_fence_after();
+        if (abort_s) break;
     }
     if (!ok) abort_s = 1;
     if (!ok) atomicCAS(p.err, 0, 1 + (int)blockIdx.x);
@@ -1077,29 +1089,49 @@ struct StemConfig {
     size_t smem() const { return (size_t)w_bytes + pos_bytes + patch_bytes; }
 };
 
-// Bands of eight output rows, or of fewer if two CTAs per SM and their noise tables do not fit otherwise.
-bool stem_config(const GLayer &G, int in_c, StemConfig *c)
+// Bands of `rows` output rows, if two CTAs per SM and their noise tables fit then (one row: if one CTA does).
+bool stem_config(const GLayer &G, int in_c, int rows, StemConfig *c)
 {
     if (G.op != ISC_CONV2D || in_c > 4 || G.kw > 8 || G.kh > 8 || G.coutp % 16 != 0 || G.coutp > 256) return false;
     const bool second = G.kw > 4, whole = 4 % G.stride == 0;
     c->planes = second && !whole ? 2 : 1;
     c->pitch = G.wout + (second && whole ? 4 / G.stride : 0);
     c->w_bytes = (uint32_t)stem_pack_bytes(G);
-    for (int rows = 8; rows >= 1; rows >>= 1) {
-        const int rows_in = (rows - 1) * G.stride + G.kh;
-        const size_t patch = ((size_t)rows_in * (G.win + 2 * G.pad + 8) * 4 + 15) & ~(size_t)15;
-        c->band_rows = rows;
-        c->rows_class = (rows_in + G.stride - 1) / G.stride;
-        const size_t plane_pos = (size_t)G.stride * c->rows_class * c->pitch + 2 * kTileM + 8;        // the last tile reads beyond the last row
-        const size_t total = c->w_bytes + plane_pos * c->planes * 16 + patch;
-        if (total > (rows > 1 ? 94 : 214) * (size_t)1024) continue;
-        c->plane_pos = (uint32_t)plane_pos;
-        c->pos_bytes = (uint32_t)(plane_pos * c->planes * 16);
-        c->patch_bytes = (uint32_t)patch;
-        c->k_step = !second ? 16u : whole ? 16u * (uint32_t)(4 / G.stride) : c->plane_pos * 16u;
-        return c->k_step < (1u << 18);
-    }
+    const int rows_in = (rows - 1) * G.stride + G.kh;
+    const size_t patch = ((size_t)rows_in * (G.win + 2 * G.pad + 8) * 4 + 15) & ~(size_t)15;
+    c->band_rows = rows;
+    c->rows_class = (rows_in + G.stride - 1) / G.stride;
+    const size_t plane_pos = (size_t)G.stride * c->rows_class * c->pitch + 2 * kTileM + 8;        // the last tile reads beyond the last row
+    const size_t total = c->w_bytes + plane_pos * c->planes * 16 + patch;
+    if (total > (rows > 1 ? 94 : 214) * (size_t)1024) return false;
+    c->plane_pos = (uint32_t)plane_pos;
+    c->pos_bytes = (uint32_t)(plane_pos * c->planes * 16);
+    c->patch_bytes = (uint32_t)patch;
+    c->k_step = !second ? 16u : whole ? 16u * (uint32_t)(4 / G.stride) : c->plane_pos * 16u;
+    return c->k_step < (1u << 18);
+}
+
+// Bands of eight rows, or of fewer if that does not fit.
+bool stem_config_any(const GLayer &G, int in_c, StemConfig *c)
+{
+    for (int rows = 8; rows >= 1; rows >>= 1)
+        if (stem_config(G, in_c, rows, c)) return true;
     return false;
+}
+
+// Bands for `batch` samples on `ctas` CTAs: between 8 and 32 rows, such that the CTA with the most work has the least.  Long
+// bands draw fewer rows twice and have fewer barriers beside longer phases (some six input rows' worth each; 3 x 3 on
+// 32 x 32, 5,100 samples: 330 us in bands of 8 rows, 220 in one of 32), short ones share out more evenly.
+void stem_bands(const GLayer &G, int in_c, int64_t batch, int64_t ctas, StemConfig *c)
+{
+    int64_t best = INT64_MAX;
+    for (int bands = (G.hout + 31) / 32; bands <= (G.hout + 7) / 8; ++bands) {
+        StemConfig t;
+        const int rows = (G.hout + bands - 1) / bands;
+        if (rows < 8 || !stem_config(G, in_c, rows, &t)) continue;
+        const int64_t cost = (batch * ((G.hout + rows - 1) / rows) + ctas - 1) / ctas * ((rows - 1) * G.stride + G.kh + 6);
+        if (cost < best) { best = cost; *c = t; }
+    }
 }
 
 }  // namespace
@@ -1107,7 +1139,7 @@ bool stem_config(const GLayer &G, int in_c, StemConfig *c)
 bool stem_fits(const GLayer &G, int in_c)
 {
     StemConfig c;
-    return stem_config(G, in_c, &c);
+    return stem_config_any(G, in_c, &c);
 }
 
 // w: [cout][cin][kh][kw] -> [filter row][2 columns of 16 bytes][coutp rows][16]: byte pix * 4 + ch of a row's 32
@@ -1123,14 +1155,15 @@ void stem_pack_weights(const GLayer &G, const int8_t *w, int8_t *out)
                 }
 }
 
-cudaError_t launch_stem_conv(const GLayer &G, const int8_t *wpack, const int32_t *cst, bool fast, const uint8_t *x_chw, int in_c,
+cudaError_t launch_stem_conv(const TcDevice &dev, const GLayer &G, const int8_t *wpack, const int32_t *cst, bool fast, const uint8_t *x_chw, int in_c,
                              const NoiseStream &ns, const SampleRun &run, int batch, int8_t *out, int32_t *err, cudaStream_t st, bool debug_stall, bool chained)
 {
     StemParams p;
     p.L = G;
     p.in_c = in_c;
     StemConfig c;
-    if (!stem_config(G, in_c, &c)) return cudaErrorInvalidValue;
+    if (!stem_config_any(G, in_c, &c)) return cudaErrorInvalidValue;
+    stem_bands(G, in_c, batch, 2ll * dev.n_sms, &c);
     p.band_rows = c.band_rows;
     p.n_bands = (G.hout + p.band_rows - 1) / p.band_rows;
     p.pitch = c.pitch; p.rows_class = c.rows_class; p.planes = c.planes;
@@ -1155,8 +1188,9 @@ cudaError_t launch_stem_conv(const GLayer &G, const int8_t *wpack, const int32_t
         smem += tab_bytes;
     }
     if (batch <= 0) return cudaSuccess;
-    dim3 grid((unsigned)p.n_bands, (unsigned)batch);
-    return launch_chained(chained, k_stem, grid, kStemThreads, smem, st, p);
+    p.n_items = (uint32_t)p.n_bands * (uint32_t)batch;
+    const uint32_t ctas = (uint32_t)dev.n_sms * (smem <= kStemSmemPair ? 2u : 1u);
+    return launch_chained(chained && dev.chained, k_stem, dim3(std::min(p.n_items, ctas)), kStemThreads, smem, st, p);
 }
 
 }  // namespace isc

@@ -138,7 +138,7 @@ cudaError_t launch_halo_conv(const TcDevice &dev, const GLayer &G, const int8_t 
 bool stem_fits(const GLayer &G, int in_c);
 size_t stem_pack_bytes(const GLayer &G);
 void stem_pack_weights(const GLayer &G, const int8_t *w_oihw, int8_t *out);
-cudaError_t launch_stem_conv(const GLayer &G, const int8_t *wpack, const int32_t *cst, bool fast, const uint8_t *x_chw, int in_c,
+cudaError_t launch_stem_conv(const TcDevice &dev, const GLayer &G, const int8_t *wpack, const int32_t *cst, bool fast, const uint8_t *x_chw, int in_c,
                              const NoiseStream &ns, const SampleRun &run, int batch, int8_t *out, int32_t *err, cudaStream_t st, bool debug_stall = false,
                              bool chained = false);
 
