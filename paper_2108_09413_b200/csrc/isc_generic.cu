@@ -216,28 +216,47 @@ k_conv(GLayer L, int batch, const int8_t *__restrict__ in, const int8_t *__restr
 
 // ------------------------------------------------------------------ pools
 
+// A warp takes 32 channels of one sample, four at a time per lane (the layout pads channels to 16), every fourth pixel per group
+// of eight lanes.
 __global__ void k_gavgpool(GLayer L, int batch, const int8_t *in, int8_t *out)
 {
     conv::chain_start();
     conv::chain_wait();
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= batch * L.cinp) return;
-    const int b = idx / L.cinp, c = idx - b * L.cinp;
-    int q = 0;
-    if (c < L.cin) {
-        const int hw = L.hin * L.win;
-        long long sum = 0;
-        const int8_t *p = in + (size_t)b * hw * L.cinp + c;
-        for (int i = 0; i < hw; ++i) sum += (int)p[(size_t)i * L.cinp] - L.zp_in;
-        const int n = 31 + __ldg(L.shift);
-        long long v = (sum * (long long)__ldg(L.mult) + (1ll << (n - 1))) >> n;
+    const int warp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31, words = L.cinp >> 2, groups = (words + 7) >> 3;
+    if (warp >= batch * groups) return;
+    const int b = warp / groups, word = (warp - b * groups) * 8 + (lane & 7), hw = L.hin * L.win;
+    const bool live = word < words;
+    const int *p = reinterpret_cast<const int *>(in + (size_t)b * hw * L.cinp) + (live ? word : 0);
+    long long total[4] = {0, 0, 0, 0};
+    for (int i0 = 0; i0 < hw; i0 += 1 << 20) {                 // 32-bit sums of 2^20 bytes
+        int sum[4] = {0, 0, 0, 0};
+        for (int i = i0 + (lane >> 3); i < min(hw, i0 + (1 << 20)); i += 4) {
+            const int v = p[(size_t)i * words];
+            sum[0] = __dp4a(v, 1, sum[0]);
+            sum[1] = __dp4a(v, 1 << 8, sum[1]);
+            sum[2] = __dp4a(v, 1 << 16, sum[2]);
+            sum[3] = __dp4a(v, 1 << 24, sum[3]);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            sum[k] += __shfl_xor_sync(0xffffffffu, sum[k], 8);
+            sum[k] += __shfl_xor_sync(0xffffffffu, sum[k], 16);
+            total[k] += sum[k];
+        }
+    }
+    if (!live || lane >= 8) return;
+    const int n = 31 + __ldg(L.shift), lo = L.relu ? max(-128, L.zp_out) : -128;
+    uint32_t packed = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (4 * word + k >= L.cin) continue;
+        long long v = ((total[k] - (long long)hw * L.zp_in) * (long long)__ldg(L.mult) + (1ll << (n - 1))) >> n;
         v += L.zp_out;
-        const int lo = L.relu ? max(-128, L.zp_out) : -128;
         v = v < lo ? lo : v;
         v = v > 127 ? 127 : v;
-        q = (int)v;
+        packed |= (uint32_t)((int)v & 0xFF) << (8 * k);
     }
-    out[idx] = (int8_t)q;
+    reinterpret_cast<uint32_t *>(out)[b * words + word] = packed;
 }
 
 // Thread = one output pixel x 16 channels.  A tap outside the image repeats one inside the window, which changes no
@@ -359,8 +378,8 @@ cudaError_t launch_conv(const GLayer &L, int batch, const int8_t *in, const int8
 
 cudaError_t launch_gavgpool(const GLayer &L, int batch, const int8_t *in, int8_t *out, cudaStream_t st, bool chained)
 {
-    const int n = batch * L.cinp;
-    return conv::launch_chained(chained, k_gavgpool, dim3((unsigned)((n + 127) / 128)), 128, 0, st, L, batch, in, out);
+    const int warps = batch * (((L.cinp >> 2) + 7) >> 3);
+    return conv::launch_chained(chained, k_gavgpool, dim3((unsigned)((warps + 3) / 4)), 128, 0, st, L, batch, in, out);
 }
 
 cudaError_t launch_maxpool(const GLayer &L, int batch, const int8_t *in, int8_t *out, cudaStream_t st, bool chained)

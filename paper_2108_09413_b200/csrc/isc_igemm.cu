@@ -689,21 +689,30 @@ __global__ void __launch_bounds__(kStemThreads, 2) k_stem(const __grid_constant_
                     for (int k = 0; k < 4; ++k) dst[4 * k] = (uint8_t)min(255, max(0, (int)((clean >> (8 * k)) & 0xFFu) + z[k]));
                 }
             } else {
-                for (int c = 0; c < p.in_c; ++c) {
-                    const int64_t e_begin = ((int64_t)c * L.hin + vy0) * L.win, e_end = ((int64_t)c * L.hin + vy1) * L.win;
-                    for (int64_t q = (e_begin >> 2) + tid; q < ((e_end + 3) >> 2); q += kStemThreads) {
-                        const uint4 r = philox4x32_10(make_uint4((uint32_t)q, ctr1, ctr2, ctr3), p.ns.key0, p.ns.key1);
+                // any width: a block's elements may lie in two rows, and its first and last in another band or channel
+                const int rows = vy1 - vy0, blocks = (rows * L.win + 3) / 4 + 1;                  // of a channel, at most
+                for (int i = tid; i < p.in_c * blocks; i += kStemThreads) {
+                    const int c = i / blocks;
+                    const int64_t e_begin = ((int64_t)c * L.hin + vy0) * L.win, q = (e_begin >> 2) + (i - c * blocks);
+                    int at = (int)(4 * q - e_begin);                                             // of the block's first element among the band's
+                    if (at >= rows * L.win) continue;
+                    const uint4 r = philox4x32_10(make_uint4((uint32_t)q, ctr1, ctr2, ctr3), p.ns.key0, p.ns.key1);
+                    int z[4];
+                    if (p.ns.guide) {
+                        if (p.tab_off) noise_levels4_shared(r, sbase + p.tab_off, sbase + p.tab_off + 4u * (uint32_t)(2 * p.ns.T + 1), p.ns.T, p.ns.guide_steps, z);
+                        else noise_levels4(r, p.ns.cum, p.ns.guide, p.ns.T, p.ns.guide_steps, z);
+                    } else {
                         const uint32_t u[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            const int64_t e = q * 4 + k;
-                            if (e < e_begin || e >= e_end) continue;
-                            const int rem = (int)(e - (int64_t)c * L.hin * L.win);
-                            const int h = rem / L.win, w = rem - h * L.win;
-                            int v = (int)__ldg(x + e) + (p.ns.guide ? noise_level_guided(u[k], p.ns.cum, p.ns.guide, p.ns.T) : noise_level(u[k], p.ns.cum, p.ns.T));
-                            v = min(255, max(0, v));
-                            pb[((h - iy0) * wpad + (w + L.pad)) * 4 + c] = (uint8_t)v;
-                        }
+                        for (int k = 0; k < 4; ++k) z[k] = noise_level(u[k], p.ns.cum, p.ns.T);
+                    }
+                    int h = at < 0 ? 0 : at / L.win, w = at - h * L.win;                          // (negative before the band's first element)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k, ++at, ++w) {
+                        if (w == L.win) { w = 0; ++h; }
+                        if (at < 0 || at >= rows * L.win) continue;
+                        const int v = min(255, max(0, (int)__ldg(x + e_begin + at) + z[k]));
+                        pb[((vy0 + h - iy0) * wpad + (w + L.pad)) * 4 + c] = (uint8_t)v;
                     }
                 }
             }

@@ -191,22 +191,10 @@ __device__ __forceinline__ int noise_level(uint32_t u, const uint32_t *__restric
     return lo - T;
 }
 
-// Inverse-CDF search min{ z : u < cum[z] } (the last entry always matches) by bisection between the guide table's
-// results for the two uniforms that bracket u's top bits: the same result as the bisection over the whole table,
-// in one or two steps for the bulk of the distribution.
-__device__ __forceinline__ int noise_level_guided(uint32_t u, const uint32_t *__restrict__ cum, const uint32_t *__restrict__ guide, int T)
-{
-    const uint32_t j = u >> (32 - kNoiseGuideBits);
-    uint32_t lo = __ldg(guide + j), hi = __ldg(guide + j + 1);
-    while (lo < hi) {
-        const uint32_t mid = (lo + hi) >> 1;
-        if (u < __ldg(cum + mid)) hi = mid; else lo = mid + 1;
-    }
-    return (int)lo - T;
-}
-
-// The same search for the four uniforms of one Philox block, step by step together, so that the four dependent load chains
-// run interleaved (a step on an interval that has already closed changes nothing, since u < cum[result]).  `steps`
+// Inverse-CDF search min{ z : u < cum[z] } (the last entry always matches) for the four uniforms of one Philox block, by
+// bisection between the guide table's results for the two uniforms that bracket each one's top bits: the same result as the
+// bisection over the whole table, in one or two steps for the bulk of the distribution; step by step together, so that the
+// four dependent load chains run interleaved (a step on an interval that has already closed changes nothing, since u < cum[result]).  `steps`
 // covers the widest guide interval, which lies in the far tail and is ten steps wide; a warp's 128 uniforms seldom
 // need more than four, so the loop ends when all are found.
 __device__ __forceinline__ void noise_levels4(uint4 u4, const uint32_t *__restrict__ cum, const uint32_t *__restrict__ guide, int T,
