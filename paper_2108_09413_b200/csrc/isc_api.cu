@@ -280,7 +280,7 @@ int build_generic_engine(isc_model *m)
                 const int n_cst = halo ? halo_padded_cout(G) : igemm_padded_cout(G);
                 std::vector<int32_t> c4((size_t)n_cst * 4);
                 m->tc_fast[(size_t)i] = igemm_constants(G, bias.data(), mult.data(), shift.data(), c4.data(), n_cst, H.d.res_tensor >= 0, &m->tc_resk[(size_t)i]) ? 1 : 0;
-                if (!halo) igemm_order_constants(G, c4.data(), n_cst);
+                if (halo) halo_order_constants(G, c4.data(), n_cst); else igemm_order_constants(G, c4.data(), n_cst);
                 rc = upload(m, c4, &m->tc_cst[(size_t)i]); if (rc) return rc;
                 m->has_tc = true;
             }

@@ -222,6 +222,24 @@ __device__ __forceinline__ void cp_async_arrive(uint32_t bar)
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
+// activations to and from global memory, past the first-level cache
+__device__ __forceinline__ void st_global_v4(void *p, const uint32_t (&v)[4])
+{
+    asm volatile("st.global.L1::no_allocate.v4.u32 [%0], {%1,%2,%3,%4};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
+}
+__device__ __forceinline__ void ld_global_v4(const void *p, uint32_t (&v)[4])
+{
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "l"(p) : "memory");
+}
+__device__ __forceinline__ void st_global_v2(void *p, uint32_t a, uint32_t b) { asm volatile("st.global.L1::no_allocate.v2.u32 [%0], {%1,%2};" ::"l"(p), "r"(a), "r"(b) : "memory"); }
+__device__ __forceinline__ void st_global_u32(void *p, uint32_t a) { asm volatile("st.global.L1::no_allocate.u32 [%0], %1;" ::"l"(p), "r"(a) : "memory"); }
+__device__ __forceinline__ uint32_t ld_global_u32(const void *p)
+{
+    uint32_t v;
+    asm volatile("ld.global.L1::no_allocate.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
 // A stage ring position: index and how many times the ring has wrapped.
 struct Ring {
     int s = 0, use = 0;

@@ -19,10 +19,13 @@
 // registers took 450 cycles per MMA beside the other roles); one weights warp; sixteen epilogue warps in four teams of
 // four.  An output tile is 256 positions x at most 128 channels; up to 64 channels four of them fit into tensor memory
 // and each team takes every fourth, else two fit and two teams halve the channels of every second.  With eight warps
-// in two teams the epilogue's latency (a few hundred instructions at ten cycles each) was twice the MMAs' time.  A
-// thread requantises one row of both M operands, so that a channel's constants are read once for two outputs: reading
-// them once for each saturates the shared-memory pipe at 6 outputs a clock and SM.  Results leave, and residual rows
-// arrive, as runs of up to 64 bytes through a scratch area.
+// in two teams the epilogue's latency (a few hundred instructions at ten cycles each) was twice the MMAs' time.
+// Accumulators are read as fragments: a thread holds four rows and up to sixteen consecutive channels (the columns of the
+// weights are ordered for that, halo_channel), a constant in registers serves four outputs, and residual rows are read and
+// results written straight from registers.  (With a row per thread, rows' offsets and bytes went through shared memory and
+// a 32-channel layer took 18 instructions per output.)  This and gather_flat, 32 -> 32 channels at 32 x 32, 5,100 samples:
+// 187 -> 166 us, with a residual operand 207 -> 194; what is left is shared memory's bandwidth: the MMAs' operands, the
+// copies and the epilogue's constants keep it busy for 97 % of a 64-channel layer's time.
 // Every wait is bounded; on expiry a role raises the CTA's abort flag and the error word, the others leave their loops,
 // and the CTA frees its tensor memory and returns.
 #include <cuda_runtime.h>
@@ -30,6 +33,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <vector>
 
 #include "isc_conv.cuh"
 #include "isc_epilogue.cuh"
@@ -47,7 +51,7 @@ constexpr int kM = 128, kMT = 2, kTile = kM * kMT;      // rows of one MMA, MMAs
 constexpr int kTeams = 4, kEpi = 4 * kTeams, kGather = 4;
 constexpr int kThreads = 32 * (kEpi + kGather + kMT + 1);
 constexpr int kMaxRing = 8;
-constexpr int kFlat = 12;                               // positions of a tile that a gather lane keeps the addresses of
+constexpr int kFlat = 10;                               // positions of a tile that a gather lane keeps the addresses of
 constexpr int kMaxN = 128;                              // output channels of a tile: two of them, times kMT, fill tensor memory
 constexpr size_t kSmemMax = 226 * 1024;
 
@@ -57,14 +61,13 @@ struct HaloParams {
     int batch, c16s;                         // planes
     int stage_planes, lpp_log;               // planes of an A stage (2 or 4); log2 of the gather lanes that share a position
     int n_stages;                            // A stages of a tile
-    int flat_steps;                          // positions per gather lane if at most kFlat, else 0
+    int flat_steps;                          // positions per gather lane, at most kFlat; 0: copied by rows
     uint32_t positions, tile_pos, plane_bytes, a_bytes;     // of the batch; copied per tile; of a plane; of an A stage
     int ring_a, ring_b, resident;            // stages; B blocks (one tile's after the other when resident)
     int n_tile, tiles_n, n_blocks, tmem_cols;               // B blocks of an output tile: kh for each pair of planes
     int slots_log, col_split;                // log2 of the accumulators in tensor memory (4 or 2); channels per team when two share a tile, else 0
     uint32_t n_items;                        // tiles * tiles_n
-    int lpr_log;                             // log2 of the lanes that share a row in the coalesced accesses
-    uint32_t b_off, cst_off, scratch_off, rowtab_off;
+    uint32_t b_off, cst_off;
     FastDiv by_image, by_wp, by_hp, by_tiles_n;     // positions of an image, of a row; rows of an image; output tiles of a tile
     const int8_t *in, *res;
     int8_t *out;
@@ -91,121 +94,114 @@ template <int kMode, bool kClamp>
 __device__ __forceinline__ bool halo_epilogue(const HaloParams &p, const RoleCtx &c)
 {
     const GLayer &L = p.L;
-    const int lane = c.lane, q = c.warp & 3, team = c.warp >> 2;
-    constexpr bool kHasRes = kMode >= 2;
-    const uint32_t slot = (uint32_t)team & ((1u << p.slots_log) - 1u);
+    const int q = c.warp & 3, team = c.warp >> 2;
+    const bool has_res = kMode >= 2 || (kMode == 0 && p.res);
+    const uint32_t slot = (uint32_t)team & ((1u << p.slots_log) - 1u), word = (uint32_t)c.lane & 3u;
     const int c_first = (team >> p.slots_log) * p.col_split;        // of the output tile: this team's channels
-    const int lpr = 1 << p.lpr_log, rpi = 32 >> p.lpr_log;           // lanes per row, rows per instruction
-    const int crow = lane >> p.lpr_log, cchunk = lane & (lpr - 1);
-    // Scratch: per M operand 32 rows without padding; the 16-byte columns of a row are permuted by the row's number so
-    // that neither the row-wise nor the coalesced access has bank conflicts.  (rpi is a multiple of the period.)
-    const uint32_t row_bytes = 16u << p.lpr_log, mt_step = 32u * row_bytes;
-    const uint32_t scr0 = c.sbase + p.scratch_off + (uint32_t)c.warp * (kMT * mt_step);
-    auto permuted = [&](int row, uint32_t col) { return col ^ (p.lpr_log == 2 ? ((uint32_t)row >> 1) & 3u : ((uint32_t)row >> 2) & 1u); };
-    const uint32_t scr_row = scr0 + (uint32_t)lane * row_bytes;
-    const uint32_t scr_co = scr0 + (uint32_t)crow * row_bytes + permuted(crow, (uint32_t)cchunk) * 16u;
-    const uint32_t rowtab = c.sbase + p.rowtab_off + (uint32_t)c.warp * (uint32_t)(2 * 32 * kMT * 4);
-    const uint32_t i_step = gridDim.x << p.slots_log;
-    // an output tile: item = tile * tiles_n + n.  Its rows' byte offsets in the output go to the warp's table (-1: padding).
-    auto open_item = [&](uint32_t item, uint32_t tab, int &n0, int &n_cols) {
+    const uint32_t acc0 = c.tmem + ((uint32_t)(q * 32) << 16) + slot * (uint32_t)(kMT * p.n_tile) + (uint32_t)c_first;
+    const uint32_t bar_full = c.acc_full + 8u * slot, bar_free = c.acc_free + 8u * slot;
+    uint32_t use = 0;
+    for (uint32_t item = blockIdx.x + slot * gridDim.x; item < p.n_items; item += gridDim.x << p.slots_log, ++use) {
+        // an output tile: item = tile * tiles_n + n
         uint32_t n;
         const uint32_t tile = p.by_tiles_n.divmod(item, n);
-        n0 = (int)n * p.n_tile + c_first;
-        n_cols = min(p.n_tile, L.coutp - (int)n * p.n_tile) - c_first;
+        int n_cols = min(p.n_tile, L.coutp - (int)n * p.n_tile) - c_first;
         if (p.col_split && c_first == 0) n_cols = min(n_cols, p.col_split);
+        const int chunks = n_cols >> 4;                             // of 16 channels; a thread's are 4 * chunks consecutive ones
+        const uint32_t n0 = n * (uint32_t)p.n_tile + (uint32_t)c_first, ch0 = n0 + word * 4u * (uint32_t)chunks;
+        bool ready = false;
+#pragma unroll 1
+        for (int mt = 0; mt < kMT && chunks > 0; ++mt) {
+            // byte offset of the output row whose number is this lane's (-1: padding), and of this thread's four rows
+            int off[4];
+            {
+                const uint32_t f = tile * kTile + (uint32_t)(mt * kM + q * 32 + c.lane);
+                uint32_t r, x;
+                const uint32_t img = p.by_image.divmod(f, r), y = p.by_wp.divmod(r, x);
+                const bool valid = f < p.positions && y < (uint32_t)L.hout && x < (uint32_t)L.wout;
+                const int mine = valid ? (int)(((img * (uint32_t)L.hout + y) * (uint32_t)L.wout + x) * (uint32_t)L.coutp) : -1;
 #pragma unroll
-        for (int mt = 0; mt < kMT; ++mt) {
-            const uint32_t f = tile * kTile + (uint32_t)(mt * kM + q * 32 + lane);
-            uint32_t r, x;
-            const uint32_t img = p.by_image.divmod(f, r), y = p.by_wp.divmod(r, x);
-            const bool valid = f < p.positions && y < (uint32_t)L.hout && x < (uint32_t)L.wout;
-            const int off = valid ? (int)(((img * (uint32_t)L.hout + y) * (uint32_t)L.wout + x) * (uint32_t)L.coutp) : -1;
-            asm volatile("st.shared.u32 [%0], %1;" ::"r"(tab + (uint32_t)(mt * 32 + lane) * 4u), "r"(off) : "memory");
-        }
-        __syncwarp();
-    };
-    auto row_off = [&](uint32_t tab, int mt, int k) { return (int)lds32(tab + (uint32_t)(mt * 32 + k * rpi + crow) * 4u); };
-    auto fetch_residual = [&](uint32_t tab, int n0, int n_cols) {
-        if (cchunk * 16 >= n_cols) return;
-#pragma unroll
-        for (int mt = 0; mt < kMT; ++mt)
-            for (int k = 0; k < lpr; ++k) {
-                const int off = row_off(tab, mt, k);
-                if (off >= 0) cp_async16(scr_co + (uint32_t)mt * mt_step + (uint32_t)(k * rpi) * row_bytes, p.res + off + n0 + cchunk * 16);
+                for (int i = 0; i < 4; ++i) off[i] = __shfl_sync(0xffffffffu, mine, (c.lane >> 2) + 8 * i);
             }
-    };
-    const uint32_t acc0 = c.tmem + ((uint32_t)(q * 32) << 16) + slot * (uint32_t)(kMT * p.n_tile) + (uint32_t)c_first, acc1 = acc0 + (uint32_t)p.n_tile;
-    const uint32_t bar_full = c.acc_full + 8u * slot, bar_free = c.acc_free + 8u * slot;
-    uint32_t item = blockIdx.x + slot * gridDim.x, tab = rowtab;
-    int n0 = 0, n_cols = 0;
-    if (item < p.n_items) {
-        open_item(item, tab, n0, n_cols);
-        if (kHasRes) fetch_residual(tab, n0, n_cols);
-    }
-    for (uint32_t use = 0; item < p.n_items; item += i_step, ++use) {
-        const uint32_t tab_next = 2u * rowtab + (uint32_t)(32 * kMT * 4) - tab;          // the other table
-        int n0_next = 0, cols_next = 0;
-        if (item + i_step < p.n_items) open_item(item + i_step, tab_next, n0_next, cols_next);
-        if (kHasRes) cp_async_wait_all();                               // this tile's residual rows, requested during the previous one
-        __syncwarp();
-        if (!wait_bar<kHintEpi>(bar_full, use & 1u, c.abort_flag)) {
-            cp_async_wait_all();
-            return false;
+            uint32_t io[4][4];                                      // residual bytes, then results
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) io[i][k] = 0;
+                if (has_res && off[i] >= 0) {
+                    const int8_t *src = p.res + (uint32_t)off[i] + ch0;
+                    if (chunks == 4) ld_global_v4(src, io[i]);
+                    else {
+#pragma unroll
+                        for (int k = 0; k < 3; ++k)
+                            if (k < chunks) io[i][k] = ld_global_u32(src + 4 * k);
+                    }
+                }
+            }
+            if (!ready) {
+                ready = __all_sync(0xffffffffu, wait_bar<kHintEpi>(bar_full, use & 1u, c.abort_flag));
+                if (!ready) return false;
+                tc_fence_after();
+            }
+            const uint32_t acc = acc0 + (uint32_t)(mt * p.n_tile), cst = c.sbase + p.cst_off + n0 * 16u + word * 16u;
+            int a[2][8];
+            tmem_ld_frag(acc, a[0]);
+#pragma unroll
+            for (int ch = 0; ch < 4; ++ch) {
+                if (ch >= chunks) break;
+                int4 k4[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(k4[k].x), "=r"(k4[k].y), "=r"(k4[k].z), "=r"(k4[k].w) : "r"(cst + (uint32_t)(ch * 256 + k * 64)));
+#pragma unroll
+                for (int hf = 0; hf < 2; ++hf) {
+                    tmem_ld_frag_wait(a[hf]);
+                    // the next accumulators, before this step's arithmetic
+                    if (hf == 0) tmem_ld_frag(acc + (uint32_t)(ch * 16) + (16u << 16), a[1]);
+                    else if (ch + 1 < chunks) tmem_ld_frag(acc + (uint32_t)(ch * 16 + 16), a[0]);
+                    else if (mt == kMT - 1) {
+                        tc_fence_before();
+                        mbar_arrive(bar_free);                      // the accumulators are in registers: the next tile may overwrite them
+                    }
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        uint32_t &w = io[2 * hf + j][ch];
+                        const uint32_t rw = w ^ 0x80808080u;
+                        int y[4];
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const int v = a[hf][2 * j + (k & 1) + 4 * (k >> 1)];
+                            if (kMode == 0) {
+                                const int o = (int)ch0 + 4 * ch + k;
+                                const long long rt = has_res ? residual_term(byte_of(w, k), L.zp_res, L.res_mult, L.res_shift) : 0ll;
+                                y[k] = o < L.cout ? requant_clamp(v + __ldg(L.bias + o), __ldg(L.mult + o), __ldg(L.shift + o), rt, L.zp_out, p.lo) : 0;
+                            } else {
+                                y[k] = requant1<kMode == 3 ? 2 : kMode == 2 ? 1 : 0, kClamp>(v, k4[k], rw, k, p.res_m2, p.res_r2, p.res_k8, p.lo);
+                            }
+                        }
+                        w = pack4_sat(y[0], y[1], y[2], y[3]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (off[i] < 0) continue;
+                int8_t *dst = p.out + (uint32_t)off[i] + ch0;
+                if (chunks == 4) st_global_v4(dst, io[i]);
+                else if (chunks == 2) st_global_v2(dst, io[i][0], io[i][1]);
+                else {
+#pragma unroll
+                    for (int k = 0; k < 3; ++k)
+                        if (k < chunks) st_global_u32(dst + 4 * k, io[i][k]);
+                }
+            }
         }
-        tc_fence_after();
-        if (n_cols <= 0) {                                              // the second team of a partial tile
+        if (!ready) {                                               // the second team of a partial tile
+            if (!__all_sync(0xffffffffu, wait_bar<kHintEpi>(bar_full, use & 1u, c.abort_flag))) return false;
             tc_fence_before();
             mbar_arrive(bar_free);
         }
-        const uint32_t cst0 = c.sbase + p.cst_off + (uint32_t)n0 * 16u;
-#pragma unroll 1
-        for (int cc = 0; cc < n_cols; cc += 16) {
-            int a[2][16];
-            tmem_ld16_issue(acc0 + (uint32_t)cc, a[0]);
-            tmem_ld16_issue(acc1 + (uint32_t)cc, a[1]);
-            const uint32_t scr = scr_row + permuted(lane, (uint32_t)cc >> 4) * 16u;
-            uint32_t r0[4] = {0, 0, 0, 0}, r1[4] = {0, 0, 0, 0};
-            if (kHasRes) {
-                const uint4 u = ld_shared_v4(scr), v = ld_shared_v4(scr + mt_step);
-                r0[0] = u.x ^ 0x80808080u; r0[1] = u.y ^ 0x80808080u; r0[2] = u.z ^ 0x80808080u; r0[3] = u.w ^ 0x80808080u;
-                r1[0] = v.x ^ 0x80808080u; r1[1] = v.y ^ 0x80808080u; r1[2] = v.z ^ 0x80808080u; r1[3] = v.w ^ 0x80808080u;
-            }
-            tmem_ld32_wait(a);
-            if (cc + 16 >= n_cols) {
-                tc_fence_before();
-                mbar_arrive(bar_free);                                  // the accumulators are in registers: the next tile may overwrite them
-            }
-            uint4 o[2];
-            if (kMode == 0) {
-#pragma unroll
-                for (int mt = 0; mt < 2; ++mt) {
-                    const int off = (int)lds32(tab + (uint32_t)(mt * 32 + lane) * 4u);
-#pragma unroll
-                    for (int k = 0; k < 16; ++k) a[mt][k] += __ldg(L.bias + n0 + cc + k);
-                    o[mt] = epilogue16(a[mt], L, n0 + cc, p.res && off >= 0 ? p.res + off : nullptr);
-                }
-            } else {
-                constexpr int kRes = kMode == 3 ? 2 : kMode == 2 ? 1 : 0;
-                requant16x2<kRes, kClamp>(a, cst0 + (uint32_t)cc * 16u, r0, r1, p.res_m2, p.res_r2, p.res_k8, p.lo, o);
-            }
-            st_shared_v4(scr, o[0]);
-            st_shared_v4(scr + mt_step, o[1]);
-        }
-        __syncwarp();
-        if (cchunk * 16 < n_cols) {
-            int8_t *dst = p.out + n0 + cchunk * 16;
-#pragma unroll
-            for (int mt = 0; mt < kMT; ++mt)
-                for (int k = 0; k < lpr; ++k) {
-                    const int off = row_off(tab, mt, k);
-                    if (off >= 0) *reinterpret_cast<uint4 *>(dst + off) = ld_shared_v4(scr_co + (uint32_t)mt * mt_step + (uint32_t)(k * rpi) * row_bytes);
-                }
-        }
-        __syncwarp();
-        if (kHasRes && cols_next > 0) fetch_residual(tab_next, n0_next, cols_next);
-        tab = tab_next; n0 = n0_next; n_cols = cols_next;
     }
-    cp_async_wait_all();
     return true;
 }
 
@@ -275,9 +271,78 @@ __device__ __forceinline__ bool issue_role(const HaloParams &p, uint32_t sbase, 
     return true;
 }
 
+// A stages, position by position: lanes share a position's planes (16 bytes each).  Where a lane's N positions lie is worked out
+// per tile and kept for the tile's stages: once by division, then by adding the distance from one tile of the CTA to the
+// next, row by row and image by image.  (By division for each tile, and for twelve positions whatever the tile had, four
+// gather warps took as long for a tile as everything else.)
+template <int N>
+__device__ __forceinline__ bool gather_flat(const HaloParams &p, uint32_t sbase, int gw, int lane, uint2 a_bars, const volatile int *abort_flag)
+{
+    const GLayer &L = p.L;
+    const int lpp = 1 << p.lpp_log, per_warp = 32 >> p.lpp_log, chunk = lane & (lpp - 1);
+    const uint32_t first_pos = (uint32_t)(gw * per_warp + (lane >> p.lpp_log)), step_pos = (uint32_t)(kGather * per_warp);
+    const uint32_t win = (uint32_t)L.win, hin = (uint32_t)L.hin, wp = (uint32_t)p.wp, hp = (uint32_t)p.hp, image = wp * hp;
+    Ring ring;
+    uint32_t have = 0;                                              // positions that the tile has
+#pragma unroll
+    for (int i = 0; i < N; ++i) have |= first_pos + (uint32_t)i * step_pos < p.tile_pos ? 1u << i : 0u;
+    // of each position, counted from one image before the first (so that the halo before the first tile is no negative
+    // number): column, row, and byte offset of its pixel in the input, whether it has one or not
+    uint32_t x[N], y[N], at[N], tile = 0;
+    for (uint32_t item = blockIdx.x; item < p.n_items; item += gridDim.x) {
+        const uint32_t next = p.by_tiles_n.div(item);
+        if (item == blockIdx.x) {
+            const uint32_t first = next * kTile + image - (uint32_t)p.halo + first_pos;
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                const uint32_t img = p.by_hp.divmod(p.by_wp.divmod(first + (uint32_t)i * step_pos, x[i]), y[i]);
+                at[i] = ((img - 1u) * hin + y[i]) * win * (uint32_t)L.cinp + x[i] * (uint32_t)L.cinp;
+            }
+        } else {
+            uint32_t dx, dy;
+            const uint32_t di = p.by_hp.divmod(p.by_wp.divmod((next - tile) * kTile, dx), dy);
+            const uint32_t d = ((di * hin + dy) * win + dx) * (uint32_t)L.cinp;
+            const uint32_t wrap_x = (wp - win) * (uint32_t)L.cinp, wrap_y = (hp - hin) * win * (uint32_t)L.cinp;
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                x[i] += dx;
+                y[i] += dy;
+                at[i] += d;
+                if (x[i] >= wp) { x[i] -= wp; y[i] += 1u; at[i] -= wrap_x; }
+                if (y[i] >= hp) { y[i] -= hp; at[i] -= wrap_y; }
+            }
+        }
+        tile = next;
+        // positions of the tile that lie in no image: before the first, from the end of the last on
+        const uint32_t first = tile * kTile + first_pos, begin = (uint32_t)p.halo, end = p.positions + begin;
+        uint32_t inside = 0;
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            const uint32_t f = first + (uint32_t)i * step_pos;
+            inside |= x[i] < win && y[i] < hin && f >= begin && f < end ? 1u << i : 0u;
+        }
+        for (int plane = chunk, st = 0; st < p.n_stages; ++st, plane += p.stage_planes, ring.advance(p.ring_a)) {
+            if (ring.use >= 1 && !wait_bar<kHintLoad>(a_bars.y + 8u * (uint32_t)ring.s, (uint32_t)(ring.use - 1) & 1u, abort_flag)) {
+                cp_async_wait_all();
+                return false;
+            }
+            if (plane < p.c16s) {
+                const uint32_t dst = sbase + (uint32_t)ring.s * p.a_bytes + (uint32_t)chunk * p.plane_bytes + first_pos * 16u;
+                const int8_t *src = p.in + plane * 16;
+#pragma unroll
+                for (int i = 0; i < N; ++i)
+                    if ((have >> i) & 1u) cp_async16_cached(dst + (uint32_t)i * step_pos * 16u, (inside >> i) & 1u ? src + at[i] : p.zp_run);
+            }
+            cp_async_arrive(a_bars.x + 8u * (uint32_t)ring.s);
+        }
+    }
+    cp_async_wait_all();
+    return true;
+}
+
 __global__ void __launch_bounds__(kThreads, 1) k_halo(const __grid_constant__ HaloParams p)
 {
-    extern __shared__ __align__(128) uint8_t smem[];      // A stages | B blocks | constants | epilogue scratch | row tables
+    extern __shared__ __align__(128) uint8_t smem[];      // A stages | B blocks | constants
     __shared__ unsigned long long bar_a_full[kMaxRing], bar_a_free[kMaxRing], bar_b_full[kMaxRing], bar_b_free[kMaxRing], bar_acc_full[4], bar_acc_free[4];
     __shared__ uint32_t tmem_base_s;
     __shared__ volatile int abort_s;
@@ -316,41 +381,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_halo(const __grid_constant__ Ha
         else if (!p.res_short) ok = halo_epilogue<2, true>(p, c);
         else ok = clamp ? halo_epilogue<3, true>(p, c) : halo_epilogue<3, false>(p, c);
     } else if (warp < kEpi + kGather && p.flat_steps > 0) {
-        // ---- A stages, position by position: lanes share a position's planes (16 bytes each).  Where a lane's positions lie
-        // is worked out once per tile, independently of each other, and kept for the tile's stages.  The form below walks
-        // the rows of the images one after the other, a chain of dependent instructions that a short tile does not hide
-        // (4096 samples of a network of 32 to 128 channels on 32 x 32 to 8 x 8 maps: 2.27 -> 2.18 ms); it stays for
-        // tiles with more than kFlat positions per lane (64 channels: maps of more than 56 columns).
-        const int lpp = 1 << p.lpp_log, per_warp = 32 >> p.lpp_log, chunk = lane & (lpp - 1);
-        const uint32_t first_pos = (uint32_t)((warp - kEpi) * per_warp + (lane >> p.lpp_log)), step_pos = (uint32_t)(kGather * per_warp);
-        Ring ring;
-        for (uint32_t item = blockIdx.x; item < p.n_items && ok; item += gridDim.x) {
-            // one image further on, so that the halo before the first tile is no negative number
-            const uint32_t first = p.by_tiles_n.div(item) * kTile + (uint32_t)(p.wp * p.hp) - (uint32_t)p.halo + first_pos;
-            int off[kFlat];                                             // of the pixel's first byte in the input; -1: padding
-#pragma unroll
-            for (int i = 0; i < kFlat; ++i) {
-                uint32_t x, y;
-                const uint32_t img = p.by_hp.divmod(p.by_wp.divmod(first + (uint32_t)i * step_pos, x), y) - 1u;
-                const bool inside = x < (uint32_t)L.win && y < (uint32_t)L.hin && img < (uint32_t)p.batch;
-                off[i] = inside ? (int)(((img * (uint32_t)L.hin + y) * (uint32_t)L.win + x) * (uint32_t)L.cinp) : -1;
-            }
-            for (int plane = chunk, st = 0; st < p.n_stages; ++st, plane += p.stage_planes, ring.advance(p.ring_a)) {
-                if (ring.use >= 1) {
-                    ok = wait_bar<kHintLoad>(a_bars.y + 8u * (uint32_t)ring.s, (uint32_t)(ring.use - 1) & 1u, &abort_s);
-                    if (!ok) break;
-                }
-                if (plane < p.c16s) {
-                    const uint32_t dst = sbase + (uint32_t)ring.s * p.a_bytes + (uint32_t)chunk * p.plane_bytes + first_pos * 16u;
-                    const int8_t *src = p.in + plane * 16;
-#pragma unroll
-                    for (int i = 0; i < kFlat; ++i)
-                        if (first_pos + (uint32_t)i * step_pos < p.tile_pos) cp_async16_cached(dst + (uint32_t)i * step_pos * 16u, off[i] >= 0 ? src + off[i] : p.zp_run);
-                }
-                cp_async_arrive(a_bars.x + 8u * (uint32_t)ring.s);
-            }
-        }
-        cp_async_wait_all();
+        const int gw = warp - kEpi;
+        ok = p.flat_steps <= 6 ? gather_flat<6>(p, sbase, gw, lane, a_bars, &abort_s) : gather_flat<kFlat>(p, sbase, gw, lane, a_bars, &abort_s);
     } else if (warp < kEpi + kGather) {
         // ---- A stages, row by row of the images: rows go round the warps, lanes share a position's planes (16 bytes
         // each), so that a copy costs a handful of instructions
@@ -441,9 +473,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_halo(const __grid_constant__ Ha
 namespace {
 
 struct HaloConfig {
-    int halo, wp, hp, c16s, tiles_n, n_tile, n_blocks, stage_planes, n_stages, ring_a, ring_b, resident, lpr_log, slots_log, col_split;
+    int halo, wp, hp, c16s, tiles_n, n_tile, n_blocks, stage_planes, n_stages, ring_a, ring_b, resident, slots_log, col_split;
     uint32_t positions_tile, plane_positions, plane_bytes, a_bytes;
-    size_t b_off, cst_off, scratch_off, rowtab_off, smem;
+    size_t b_off, cst_off, smem;
 };
 
 bool halo_config(const GLayer &G, HaloConfig *c)
@@ -457,11 +489,9 @@ bool halo_config(const GLayer &G, HaloConfig *c)
     c->n_blocks = (c->c16s + 1) / 2 * G.kh;
     c->slots_log = c->n_tile <= 64 ? 2 : 1;
     c->col_split = c->n_tile <= 64 ? 0 : (c->n_tile / 2 + 15) & ~15;
-    c->lpr_log = c->n_tile <= 32 ? 1 : 2;
     c->positions_tile = (uint32_t)(kTile + 2 * c->halo);
     c->plane_positions = (c->positions_tile + 1u) | 1u;          // an odd number of 16-byte rows: planes start in different banks; one to spare
     c->plane_bytes = c->plane_positions * 16u;
-    const size_t scratch = (size_t)kEpi * 32 * kMT * (16u << c->lpr_log), rowtab = (size_t)kEpi * 2 * 32 * kMT * 4;
     const size_t cst = (size_t)c->tiles_n * c->n_tile * 16;
     const size_t block = (size_t)c->n_tile * G.kh * 32, all = block * (size_t)c->n_blocks * (size_t)c->tiles_n;
     // A stages of two pairs of planes where the channels are multiples of 64, else (or when three do not fit) of one;
@@ -470,7 +500,7 @@ bool halo_config(const GLayer &G, HaloConfig *c)
         c->stage_planes = planes;
         c->n_stages = (c->c16s + planes - 1) / planes;
         c->a_bytes = (c->plane_bytes * (uint32_t)planes + 127u) & ~127u;
-        const size_t fixed = cst + scratch + rowtab;
+        const size_t fixed = cst;
         if (fixed + 3 * (size_t)c->a_bytes + std::min(all, 3 * block) > kSmemMax) continue;
         c->resident = fixed + 3 * (size_t)c->a_bytes + all <= kSmemMax;
         size_t room = kSmemMax - fixed;
@@ -486,12 +516,31 @@ bool halo_config(const GLayer &G, HaloConfig *c)
             c->b_off = (size_t)c->ring_a * c->a_bytes;
             c->cst_off = c->b_off + (size_t)c->ring_b * block;
         }
-        c->scratch_off = c->cst_off + cst;
-        c->rowtab_off = c->scratch_off + scratch;
-        c->smem = c->rowtab_off + rowtab;
+        c->smem = c->cst_off + cst;
         return true;
     }
     return false;
+}
+
+// The team's block of an output tile that column `col` (of the padded output channels) lies in: its first column and width.
+void halo_block(const GLayer &G, const HaloConfig &c, int col, int *first, int *width)
+{
+    const int tile = col / c.n_tile * c.n_tile, valid = std::min(c.n_tile, G.coutp - tile), in_tile = col - tile;
+    const int split = c.col_split && valid > c.col_split ? c.col_split : valid;
+    *first = tile + (in_tile < split ? 0 : split);
+    *width = in_tile < split ? split : valid - split;
+    if (in_tile >= valid) { *first = tile + valid; *width = 0; }          // padding
+}
+
+// The output channel of a column of the accumulators: column 16 t + 8 h + 2 c + e of a block of 16 u is channel
+// 4 u c + 4 t + 2 h + e of it (see halo_epilogue).
+int halo_channel(const GLayer &G, const HaloConfig &c, int col)
+{
+    int first, width;
+    halo_block(G, c, col, &first, &width);
+    if (!width) return col;
+    const int b = col - first;
+    return first + width / 4 * ((b >> 1) & 3) + 4 * (b >> 4) + ((b >> 2) & 2) + (b & 1);
 }
 
 }  // namespace
@@ -541,11 +590,28 @@ void halo_pack(const GLayer &G, const int8_t *w, int8_t *out)
                     const int plane = odd ? 2 * pair : 2 * pair + col, tap_x = odd ? 2 * s + col : s;
                     for (int n = 0; n < c.n_tile; ++n)
                         for (int e = 0; e < 16; ++e, ++at) {
-                            const int oc = t * c.n_tile + n, ci = plane * 16 + e;
+                            const int oc = halo_channel(G, c, t * c.n_tile + n), ci = plane * 16 + e;
                             out[at] = (tap_x < k && oc < G.cout && ci < G.cin) ? w[(((size_t)oc * G.cin + ci) * k + r) * k + tap_x] : (int8_t)0;
                         }
                 }
     for (int e = 0; e < 64; ++e) out[at + e] = (int8_t)G.zp_in;
+}
+
+// The constants of igemm_constants in the order in which the kernel reads them: the four of channels 4 u c + 4 t + k, c = 0 to 3, of
+// a block lie side by side.
+void halo_order_constants(const GLayer &G, int32_t *out4, int n_out)
+{
+    HaloConfig c;
+    if (!halo_config(G, &c)) return;
+    const std::vector<int32_t> in(out4, out4 + 4 * (size_t)n_out);
+    for (int col = 0; col < n_out; ++col) {
+        int first, width;
+        halo_block(G, c, col, &first, &width);
+        if (!width) continue;
+        const int b = col - first;                       // position: t * 16 + k * 4 + c
+        const int channel = first + width / 4 * (b & 3) + 4 * (b >> 4) + ((b >> 2) & 3);
+        memcpy(out4 + 4 * (size_t)col, &in[4 * (size_t)channel], 16);
+    }
 }
 
 cudaError_t halo_prepare() { return cudaFuncSetAttribute(k_halo, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax); }
@@ -566,7 +632,12 @@ cudaError_t launch_halo_conv(const TcDevice &dev, const GLayer &G, const int8_t 
     p.lpp_log = c.c16s == 1 ? 0 : c.stage_planes == 4 ? 2 : 1;
     const uint32_t lane_pos = (uint32_t)kGather * (32u >> p.lpp_log);
     p.flat_steps = (int)((c.positions_tile + lane_pos - 1) / lane_pos);
-    if (p.flat_steps > kFlat) p.flat_steps = 0;
+    // By rows where a row's last step leaves at most an eighth of its lanes idle, or where there are more positions than a
+    // lane keeps.  A layer of 512 samples by rows and by positions: 64 channels at 56 x 56 (rows of 57, steps of 8) 86 and 98
+    // us, 128 at 28 x 28 (29) 51 and 53, 256 at 14 x 14 (15) 57 and 60; rows of one step, 512 at 7 x 7, 67 and 64.  A network of
+    // 32, 64 and 128 channels at 32 x 32 to 8 x 8 (rows of 33 in steps of 16, of 17 and 9 in steps of 8): 2,394 and 2,200.
+    const int step = 32 >> p.lpp_log, full = (c.wp + step - 1) / step * step;
+    if (p.flat_steps > kFlat || (c.wp > step && 8 * (full - c.wp) <= full)) p.flat_steps = 0;
     p.positions = (uint32_t)positions;
     p.tile_pos = c.positions_tile; p.plane_bytes = c.plane_bytes; p.a_bytes = c.a_bytes;
     p.ring_a = c.ring_a; p.ring_b = c.ring_b; p.resident = c.resident;
@@ -579,9 +650,7 @@ cudaError_t launch_halo_conv(const TcDevice &dev, const GLayer &G, const int8_t 
     p.by_wp = FastDiv::make((uint32_t)c.wp);
     p.by_hp = FastDiv::make((uint32_t)c.hp);
     p.by_tiles_n = FastDiv::make((uint32_t)c.tiles_n);
-    p.lpr_log = c.lpr_log;
     p.b_off = (uint32_t)c.b_off; p.cst_off = (uint32_t)c.cst_off;
-    p.scratch_off = (uint32_t)c.scratch_off; p.rowtab_off = (uint32_t)c.rowtab_off;
     p.in = in; p.res = res; p.out = out; p.wpack = wpack;
     p.zp_run = wpack + halo_pack_bytes(G) - 64;
     p.cst = reinterpret_cast<const int4 *>(cst);

@@ -209,15 +209,6 @@ __device__ __forceinline__ bool epilogue_rows(const IgemmParams &p, const EpiCtx
     return true;
 }
 
-__device__ __forceinline__ void st_global_v4(void *p, const uint32_t (&v)[4])
-{
-    asm volatile("st.global.L1::no_allocate.v4.u32 [%0], {%1,%2,%3,%4};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
-}
-__device__ __forceinline__ void ld_global_v4(const void *p, uint32_t (&v)[4])
-{
-    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "l"(p) : "memory");
-}
-
 // The epilogue of whole tiles (every column valid, a multiple of 64 of them).  Accumulators are read as fragments: of 16
 // columns a thread holds four in each of four rows per operand (lane / 4 + 8 i), and the columns of the weights are ordered
 // so that its columns of four such chunks are 16 consecutive channels (igemm_channel).  A thread's four constants of a chunk

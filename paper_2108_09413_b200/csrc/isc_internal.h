@@ -130,6 +130,7 @@ bool halo_offsets_fit(const GLayer &G, int64_t batch);
 int halo_padded_cout(const GLayer &G);
 size_t halo_pack_bytes(const GLayer &G);
 void halo_pack(const GLayer &G, const int8_t *w_oihw, int8_t *out);
+void halo_order_constants(const GLayer &G, int32_t *out4, int n_out);      // igemm_constants' in the order in which k_halo reads them
 cudaError_t halo_prepare();                      // part of tc_prepare
 cudaError_t launch_halo_conv(const TcDevice &dev, const GLayer &G, const int8_t *wpack, const int32_t *cst, bool fast, const ResidualForm &form, int batch,
                              const int8_t *in, const int8_t *res, int8_t *out, int32_t *err, cudaStream_t st, bool debug_stall = false);
