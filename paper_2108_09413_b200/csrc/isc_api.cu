@@ -70,10 +70,11 @@ struct isc_model {
     uint32_t *d_cum = nullptr;    size_t d_cum_n = 0;
     double cum_sigma = -1.0;                    // what d_cum holds
     int cum_kind = -1;
-    // the table on the host: the cumulative one, then the guide
+    // the table on the host: the cumulative one, the guide, the bins if the law has them
     std::vector<uint32_t> h_tab;
     double tab_sigma = -1.0;
-    int tab_T = 0, tab_kind = -1, tab_steps = 0;
+    int tab_T = 0, tab_kind = -1, tab_steps = 0, tab_bin_bits = 0;
+    size_t tab_front = 0;                       // entries before the bins
 
     isc::LinePlan *line = nullptr;
 
@@ -344,13 +345,45 @@ int ensure_workspace(isc_model *m, int batch)
     return ISC_OK;
 }
 
+// The table of bins at `bits` bits; false if more than one uniform in 2^11 lies in an open bin: the 128 of a warp share
+// the way out, which then costs what the bins save (sixteen warps in all meet one).
+bool noise_bins(const uint32_t *cum, size_t n_cum, int bits, std::vector<uint32_t> &out)
+{
+    const uint32_t side = isc::noise_bins_side(bits), one = 1u << bits;
+    out.assign(4 * (size_t)side, 0);
+    uint64_t open = 0;
+    size_t at = 0;                                                                 // neighbouring bins' levels lie close together
+    auto level = [&](uint32_t u) {
+        while (at + 1 < n_cum && u >= cum[at]) ++at;
+        while (at > 0 && u < cum[at - 1]) --at;
+        return at;
+    };
+    for (uint32_t upper = 0; upper < 2; ++upper)
+        for (uint32_t b = 0; b < side; ++b) {
+            const int e = isc::kNoiseBinsFrom + (int)(b >> bits) - bits;
+            const uint64_t v0 = (uint64_t)(one + (b & (one - 1))) << e, v1 = v0 + (1ull << e) - 1, from = 1ull << isc::kNoiseBinsFrom;
+            const uint64_t t0 = v0 - from, t1 = std::min<uint64_t>(v1 - from, 0x7FFFFFFFull);
+            uint32_t *entry = &out[2 * ((size_t)upper * side + b)];
+            entry[1] = (uint32_t)isc::kNoiseOpen;
+            if (t0 > t1) continue;                                                 // no uniform has this bin
+            const size_t i0 = level(upper ? ~(uint32_t)t1 : (uint32_t)t0), i1 = level(upper ? ~(uint32_t)t0 : (uint32_t)t1);
+            if (i1 > i0 + 1 || i0 + 1 == n_cum) {                                  // (the last level has no boundary above it)
+                if ((open += t1 - t0 + 1) > 1ull << 21) return false;
+                continue;
+            }
+            entry[0] = cum[i0];
+            entry[1] = (uint32_t)((int)i0 - (int)(n_cum - 1) / 2);
+        }
+    return true;
+}
+
 // The noise law's table for `sigma` on the host, kept for the next call.
 void host_noise_table(isc_model *m, double sigma)
 {
     if (m->tab_sigma == sigma && m->tab_kind == (int)m->opt_noise) return;
     std::vector<uint32_t> cum;
     if (m->opt_noise) noise_table_rounded(sigma, cum); else noise_table(sigma, cum);
-    // the guide table follows the cumulative one in the same allocation
+    // the guide table and the bins follow the cumulative one in the same allocation
     const size_t n_cum = cum.size();
     uint32_t i = 0;
     for (int j = 0; j <= isc::kNoiseGuide; ++j) {
@@ -364,6 +397,13 @@ void host_noise_table(isc_model *m, double sigma)
     for (int j = 0; j < isc::kNoiseGuide; ++j) span = std::max(span, cum[n_cum + j + 1] - cum[n_cum + j]);
     m->tab_steps = 0;
     while ((1u << m->tab_steps) < span + 1) ++m->tab_steps;
+    m->tab_front = (cum.size() + 3) & ~(size_t)3;
+    cum.resize(m->tab_front, 0);
+    m->tab_bin_bits = 0;
+    std::vector<uint32_t> bins;
+    for (int bits = 6; bits <= 8 && !m->tab_bin_bits; ++bits)
+        if (noise_bins(cum.data(), n_cum, bits, bins)) m->tab_bin_bits = bits;
+    if (m->tab_bin_bits) cum.insert(cum.end(), bins.begin(), bins.end());
     m->h_tab.swap(cum);
     m->tab_sigma = sigma;
     m->tab_kind = (int)m->opt_noise;
@@ -413,6 +453,8 @@ NoiseStream make_stream(const isc_model *m, uint64_t seed, uint64_t image_id, in
     ns.T = m->tab_T;
     ns.guide = m->d_cum ? m->d_cum + (2 * m->tab_T + 1) : nullptr;
     ns.guide_steps = m->tab_steps;
+    ns.bins = m->d_cum && m->tab_bin_bits ? reinterpret_cast<const uint2 *>(m->d_cum + m->tab_front) : nullptr;
+    ns.bin_bits = m->tab_bin_bits;
     return ns;
 }
 
@@ -1156,9 +1198,11 @@ extern "C" int isc_sample_counts_static(isc_model *m, const uint8_t *x_u8, uint6
     if ((rc = static_scratch_base(&base))) return rc;
     cudaStream_t st = (cudaStream_t)cuda_stream;
     // What goes up, as one copy: error word, vote counts (both zero: the array keeps whatever the previous call left),
-    // noise table (the guide too where it fits), image.
+    // noise table (the guide too where it fits, and for the engine that reads them the bins), image.
     host_noise_table(m, sigma);
-    const size_t n_cum = (size_t)(2 * T + 1), n_tab = m->h_tab.size() * sizeof(uint32_t) <= kStaticTableBytes ? m->h_tab.size() : n_cum;
+    const size_t n_cum = (size_t)(2 * T + 1);
+    auto fits = [](size_t n) { return n * sizeof(uint32_t) <= kStaticTableBytes; };
+    const size_t n_tab = engine == 2 && fits(m->h_tab.size()) ? m->h_tab.size() : fits(m->tab_front) ? m->tab_front : n_cum;
     auto up16 = [](size_t v) { return (v + 15) & ~(size_t)15; };
     const size_t counts_off = 16, tab_off = counts_off + up16(C * sizeof(int32_t)), x_off = tab_off + up16(n_tab * sizeof(uint32_t));
     if (x_off + d > fixed + 4096) return ISC_ERR_UNSUPPORTED;
@@ -1173,6 +1217,7 @@ extern "C" int isc_sample_counts_static(isc_model *m, const uint8_t *x_u8, uint6
     ns.T = T;
     ns.guide = n_tab > n_cum ? ns.cum + n_cum : nullptr;
     ns.guide_steps = n_tab > n_cum ? m->tab_steps : 0;
+    ns.bins = n_tab > m->tab_front ? reinterpret_cast<const uint2 *>(ns.cum + m->tab_front) : nullptr;
     // (ResNet-20, 2,000 samples: 4.1 ms with the plain kernels, 0.53 ms on the resident engine.)
     // The resident engine needs no work space but this; the layer-by-layer kernels take their activation buffers from the
     // rest of the array, as many samples at a time as fit.

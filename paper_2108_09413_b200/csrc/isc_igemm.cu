@@ -533,8 +533,9 @@ __global__ void __launch_bounds__(igemm_threads(kWhole, kCopy), 1) k_igemm(const
 // windows into an operand stage moved five times as many bytes and put a CTA barrier before every tile.  A tile is
 // 256 positions (two M operands), so that a thread requantises two rows and reads a channel's constants once for both;
 // the positions behind a row's last pixel are computed and not stored.  A ninth warp issues the MMAs.  7 x 7 stride 2 on
-// 224 x 224, 512 samples: 975 -> 823 us; 3 x 3 on 32 x 32, 4096 samples: 352 -> 311 us.  What is left is the noise: its
-// Philox rounds and table searches take the integer pipes for most of the kernel's time.
+// 224 x 224, 512 samples: 833 -> 640 us with the table of bins (the search by guide and bisection took 260 of them: two loads
+// and two for each step, of 32 lanes from as many places, which is bank conflicts); of what is left the Philox rounds take
+// some 70, the search as much, the epilogue 95 and the copy to positions 47, the rest is the patch and the barriers.
 struct StemParams {
     GLayer L;
     int in_c, band_rows, n_bands, tmem_cols;
@@ -544,6 +545,7 @@ struct StemParams {
     uint32_t w_bytes, pos_off, patch_off;
     int slots;                               // pairs of accumulators in tensor memory
     uint32_t tab_off;                        // the noise tables' copy in shared memory (after the patch), 0: searched in global memory
+    int tab_words, bin_bits;                 // of the copy; bits of the bins if they are what is copied, else 0
     const uint8_t *x;                        // clean images, CHW, one after the other
     NoiseStream ns;                          // the counter's words come from `run`
     const int8_t *wpack;                     // [filter row][2 K columns][coutp rows][16 bytes]
@@ -635,11 +637,21 @@ __global__ void __launch_bounds__(kStemThreads, 2) k_stem(const __grid_constant_
 
     uint32_t *patch = reinterpret_cast<uint32_t *>(smem + p.patch_off);
     const uint32_t zp_fill = (uint32_t)(L.zp_in & 0xFF) * (0x01010101u >> (8 * (4 - p.in_c)));
-    if (p.tab_off && p.ns.guide) {
-        // cumulative table, then the guide table that follows it in memory
+    if (p.tab_off) {
+        // the bins, or the cumulative table and the guide table that follows it in memory
+        const uint32_t *from = p.bin_bits ? reinterpret_cast<const uint32_t *>(p.ns.bins) : p.ns.cum;
         uint32_t *tab = reinterpret_cast<uint32_t *>(smem + p.tab_off);
-        for (int i = tid; i < 2 * p.ns.T + 1 + kNoiseGuide + 1; i += kStemThreads) tab[i] = __ldg(p.ns.cum + i);
+        for (int i = tid; i < p.tab_words; i += kStemThreads) tab[i] = __ldg(from + i);
     }
+    // the levels of a Philox block's four uniforms
+    auto levels4 = [&](uint4 r, int (&z)[4]) {
+        if (p.bin_bits) {
+            if (noise_levels4_bins(r, sbase + p.tab_off, p.bin_bits, z)) return;
+        } else if (p.tab_off) {
+            return noise_levels4_shared(r, sbase + p.tab_off, sbase + p.tab_off + 4u * (uint32_t)(2 * p.ns.T + 1), p.ns.T, p.ns.guide_steps, z);
+        }
+        noise_levels4(r, p.ns.cum, p.ns.guide, p.ns.T, p.ns.guide_steps, z);
+    };
     bool ok = true;
     uint32_t first_tile = 0;                                    // of the item, counted over the CTA's items
     for (uint32_t item = blockIdx.x; item < p.n_items; item += gridDim.x) {
@@ -673,8 +685,7 @@ __global__ void __launch_bounds__(kStemThreads, 2) k_stem(const __grid_constant_
                     const uint4 r = philox4x32_10(make_uint4(e >> 2, ctr1, ctr2, ctr3), p.ns.key0, p.ns.key1);
                     const uint32_t clean = __ldg(reinterpret_cast<const uint32_t *>(x + e));
                     int z[4];
-                    if (p.tab_off) noise_levels4_shared(r, sbase + p.tab_off, sbase + p.tab_off + 4u * (uint32_t)(2 * p.ns.T + 1), p.ns.T, p.ns.guide_steps, z);
-                    else noise_levels4(r, p.ns.cum, p.ns.guide, p.ns.T, p.ns.guide_steps, z);
+                    levels4(r, z);
                     uint8_t *dst = pb + ((h - iy0) * wpad + (4 * wq + L.pad)) * 4 + c;
 #pragma unroll
                     for (int k = 0; k < 4; ++k) dst[4 * k] = (uint8_t)min(255, max(0, (int)((clean >> (8 * k)) & 0xFFu) + z[k]));
@@ -690,8 +701,7 @@ __global__ void __launch_bounds__(kStemThreads, 2) k_stem(const __grid_constant_
                     const uint4 r = philox4x32_10(make_uint4((uint32_t)q, ctr1, ctr2, ctr3), p.ns.key0, p.ns.key1);
                     int z[4];
                     if (p.ns.guide) {
-                        if (p.tab_off) noise_levels4_shared(r, sbase + p.tab_off, sbase + p.tab_off + 4u * (uint32_t)(2 * p.ns.T + 1), p.ns.T, p.ns.guide_steps, z);
-                        else noise_levels4(r, p.ns.cum, p.ns.guide, p.ns.T, p.ns.guide_steps, z);
+                        levels4(r, z);
                     } else {
                         const uint32_t u[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
@@ -1090,7 +1100,7 @@ struct StemConfig {
 };
 
 // Bands of `rows` output rows, if two CTAs per SM and their noise tables fit then (one row: if one CTA does).
-bool stem_config(const GLayer &G, int in_c, int rows, StemConfig *c)
+bool stem_config(const GLayer &G, int in_c, int rows, StemConfig *c, size_t limit = 94 * 1024)
 {
     if (G.op != ISC_CONV2D || in_c > 4 || G.kw > 8 || G.kh > 8 || G.coutp % 16 != 0 || G.coutp > 256) return false;
     const bool second = G.kw > 4, whole = 4 % G.stride == 0;
@@ -1103,7 +1113,7 @@ bool stem_config(const GLayer &G, int in_c, int rows, StemConfig *c)
     c->rows_class = (rows_in + G.stride - 1) / G.stride;
     const size_t plane_pos = (size_t)G.stride * c->rows_class * c->pitch + 2 * kTileM + 8;        // the last tile reads beyond the last row
     const size_t total = c->w_bytes + plane_pos * c->planes * 16 + patch;
-    if (total > (rows > 1 ? 94 : 214) * (size_t)1024) return false;
+    if (total > (rows > 1 ? limit : 214 * (size_t)1024)) return false;
     c->plane_pos = (uint32_t)plane_pos;
     c->pos_bytes = (uint32_t)(plane_pos * c->planes * 16);
     c->patch_bytes = (uint32_t)patch;
@@ -1122,13 +1132,16 @@ bool stem_config_any(const GLayer &G, int in_c, StemConfig *c)
 // Bands for `batch` samples on `ctas` CTAs: between 8 and 32 rows, such that the CTA with the most work has the least.  Long
 // bands draw fewer rows twice and have fewer barriers beside longer phases (some six input rows' worth each; 3 x 3 on
 // 32 x 32, 5,100 samples: 330 us in bands of 8 rows, 220 in one of 32), short ones share out more evenly.
-void stem_bands(const GLayer &G, int in_c, int64_t batch, int64_t ctas, StemConfig *c)
+// A table of bins takes its room from the bands if some of eight rows or more remain.
+void stem_bands(const GLayer &G, int in_c, int64_t batch, int64_t ctas, size_t bins, StemConfig *c)
 {
     int64_t best = INT64_MAX;
+    size_t limit = 94 * 1024;
+    StemConfig t;
+    if (bins && stem_config(G, in_c, 8, &t, kStemSmemPair - bins)) limit = kStemSmemPair - bins;
     for (int bands = (G.hout + 31) / 32; bands <= (G.hout + 7) / 8; ++bands) {
-        StemConfig t;
         const int rows = (G.hout + bands - 1) / bands;
-        if (rows < 8 || !stem_config(G, in_c, rows, &t)) continue;
+        if (rows < 8 || !stem_config(G, in_c, rows, &t, limit)) continue;
         const int64_t cost = (batch * ((G.hout + rows - 1) / rows) + ctas - 1) / ctas * ((rows - 1) * G.stride + G.kh + 6);
         if (cost < best) { best = cost; *c = t; }
     }
@@ -1163,7 +1176,8 @@ cudaError_t launch_stem_conv(const TcDevice &dev, const GLayer &G, const int8_t 
     p.in_c = in_c;
     StemConfig c;
     if (!stem_config_any(G, in_c, &c)) return cudaErrorInvalidValue;
-    stem_bands(G, in_c, batch, 2ll * dev.n_sms, &c);
+    const size_t bins = ns.bins && ns.guide ? (size_t)noise_bins_side(ns.bin_bits) * 16 : 0;
+    stem_bands(G, in_c, batch, 2ll * dev.n_sms, bins, &c);
     p.band_rows = c.band_rows;
     p.n_bands = (G.hout + p.band_rows - 1) / p.band_rows;
     p.pitch = c.pitch; p.rows_class = c.rows_class; p.planes = c.planes;
@@ -1180,12 +1194,15 @@ cudaError_t launch_stem_conv(const TcDevice &dev, const GLayer &G, const int8_t 
     p.out = out; p.err = err;
     p.debug_stall = debug_stall ? 1 : 0;
     size_t smem = c.smem();
-    // the noise tables go to shared memory when two CTAs per SM still fit and the guide table follows the cumulative one
-    const size_t tab_bytes = ((size_t)(2 * ns.T + 1 + kNoiseGuide + 1) * 4 + 15) & ~(size_t)15;
-    p.tab_off = 0;
-    if (ns.guide == ns.cum + (2 * ns.T + 1) && smem + tab_bytes <= (smem <= kStemSmemPair ? kStemSmemPair : kStemSmemLimit)) {
+    // The noise tables go to shared memory when two CTAs per SM still fit and the guide table follows the cumulative one:
+    // the bins if there is room for them.
+    const size_t front_words = (size_t)(2 * ns.T + 1 + kNoiseGuide + 1), room = (smem <= kStemSmemPair ? kStemSmemPair : kStemSmemLimit) - smem;
+    p.tab_off = 0; p.tab_words = 0; p.bin_bits = 0;
+    if (bins && bins <= room) { p.tab_words = (int)(bins / 4); p.bin_bits = ns.bin_bits; }
+    else if (ns.guide == ns.cum + (2 * ns.T + 1) && front_words * 4 <= room) p.tab_words = (int)front_words;
+    if (p.tab_words) {
         p.tab_off = (uint32_t)smem;
-        smem += tab_bytes;
+        smem += ((size_t)p.tab_words * 4 + 15) & ~(size_t)15;
     }
     if (batch <= 0) return cudaSuccess;
     p.n_items = (uint32_t)p.n_bands * (uint32_t)batch;

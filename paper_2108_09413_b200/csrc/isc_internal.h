@@ -17,6 +17,13 @@ struct TShape {
 
 constexpr int kNoiseGuideBits = 10, kNoiseGuide = 1 << kNoiseGuideBits;
 
+// Table of bins, an alternative to guide and bisection.  A uniform's distance t from its nearer end of the range (u or ~u, below
+// 2^31) plus 2^kNoiseBinsFrom, read as a floating-point number of `bits` bits of fraction, is its bin: bins are narrow where
+// levels are, and at few bits nearly all hold at most one boundary between two levels.  Entry {boundary, level below it},
+// level counted from -T, kNoiseOpen where a bin holds more.  First the bins of u, then those of ~u.
+constexpr int kNoiseBinsFrom = 21, kNoiseOpen = 1 << 30;
+constexpr __host__ __device__ uint32_t noise_bins_side(int bits) { return ((uint32_t)(31 - kNoiseBinsFrom) << bits) + 2u; }
+
 // Where the random stream of one launch starts (Philox4x32-10 key and fixed counter words).
 struct NoiseStream {
     uint32_t key0, key1;      // seed halves
@@ -29,6 +36,8 @@ struct NoiseStream {
     // uniform j << (32 - kNoiseGuideBits), a lower bound of the result for every uniform with these top bits.
     const uint32_t *guide;
     int guide_steps;          // bisection steps that close the widest interval [guide[j], guide[j+1]]
+    const uint2 *bins;        // device, or null
+    int bin_bits;
 };
 
 // What the samples of a forward pass of the layer-by-layer kernels are: per image, n_sel samples of the selection phase (numbers
