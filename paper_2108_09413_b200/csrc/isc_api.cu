@@ -1198,11 +1198,11 @@ extern "C" int isc_sample_counts_static(isc_model *m, const uint8_t *x_u8, uint6
     if ((rc = static_scratch_base(&base))) return rc;
     cudaStream_t st = (cudaStream_t)cuda_stream;
     // What goes up, as one copy: error word, vote counts (both zero: the array keeps whatever the previous call left),
-    // noise table (the guide too where it fits, and for the engine that reads them the bins), image.
+    // noise table (the guide too where it fits, and for the engines that read them the bins), image.
     host_noise_table(m, sigma);
     const size_t n_cum = (size_t)(2 * T + 1);
     auto fits = [](size_t n) { return n * sizeof(uint32_t) <= kStaticTableBytes; };
-    const size_t n_tab = engine == 2 && fits(m->h_tab.size()) ? m->h_tab.size() : fits(m->tab_front) ? m->tab_front : n_cum;
+    const size_t n_tab = engine >= 2 && fits(m->h_tab.size()) ? m->h_tab.size() : fits(m->tab_front) ? m->tab_front : n_cum;
     auto up16 = [](size_t v) { return (v + 15) & ~(size_t)15; };
     const size_t counts_off = 16, tab_off = counts_off + up16(C * sizeof(int32_t)), x_off = tab_off + up16(n_tab * sizeof(uint32_t));
     if (x_off + d > fixed + 4096) return ISC_ERR_UNSUPPORTED;

@@ -646,7 +646,7 @@ __global__ void __launch_bounds__(kStemThreads, 2) k_stem(const __grid_constant_
     // the levels of a Philox block's four uniforms
     auto levels4 = [&](uint4 r, int (&z)[4]) {
         if (p.bin_bits) {
-            if (noise_levels4_bins(r, sbase + p.tab_off, p.bin_bits, z)) return;
+            if (noise_levels4_bins(r, sbase + p.tab_off, nullptr, p.bin_bits, z)) return;
         } else if (p.tab_off) {
             return noise_levels4_shared(r, sbase + p.tab_off, sbase + p.tab_off + 4u * (uint32_t)(2 * p.ns.T + 1), p.ns.T, p.ns.guide_steps, z);
         }

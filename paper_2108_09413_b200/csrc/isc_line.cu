@@ -775,8 +775,10 @@ __device__ __forceinline__ GroupJob group_job(const LineParams &p, int grp)
 
 // INPUT: one item = four horizontally adjacent pixels of one sample and input channel, one Philox block (Def. 3.3,
 // Def. 3.4).  Items of all channels share one index space (3072 items of a 32 x 32 x 3 image for 640 threads; with the
-// channels of a pixel in one thread it was 1024, two rounds of which the second is mostly idle), and the four table
-// searches run interleaved, until all four are found, instead of one after the other.
+// channels of a pixel in one thread it was 1024, two rounds of which the second is mostly idle).  The levels come from the
+// table of bins in global memory: one load that depends on the uniforms instead of the guide's and then one for each step of
+// a bisection, which a CTA with nearly no L1 beside its shared memory waits for at L2's latency (a group of the 20-layer
+// network 92.5 -> 89.3 us, the call of the tiny CNN 94 -> 84 us).
 __device__ __forceinline__ void input_phase(const LineParams &p, int grp)
 {
     const int H = p.in_H, W = p.in_W, in_c = p.in_c;
@@ -784,6 +786,7 @@ __device__ __forceinline__ void input_phase(const LineParams &p, int grp)
     const int quads = kG * H * (W >> 2);
     const uint32_t *__restrict__ cum = p.ns.cum;
     const uint32_t *__restrict__ guide = p.ns.guide;
+    const uint2 *__restrict__ bins = p.ns.bins;
     const int T = p.ns.T, steps = p.ns.guide_steps;
     const GroupJob g = group_job(p, grp);
     const unsigned long long image_id = p.image_id0 + (unsigned long long)g.image;
@@ -804,7 +807,8 @@ __device__ __forceinline__ void input_phase(const LineParams &p, int grp)
         const uint4 r = philox4x32_10(make_uint4(e >> 2, (uint32_t)(j & 0xFFFFFFFFll), ctr2, ctr3), key0, key1);
         const uint32_t clean = __ldg(reinterpret_cast<const uint32_t *>(x + e));
         int z[4];
-        if (guide) {
+        if (bins && noise_levels4_bins(r, 0u, bins, p.ns.bin_bits, z)) {
+        } else if (guide) {
             noise_levels4(r, cum, guide, T, steps, z);
         } else {
             const uint32_t u[4] = {r.x, r.y, r.z, r.w};

@@ -247,22 +247,26 @@ __device__ __forceinline__ void noise_levels4_shared(uint4 u4, uint32_t cum_s, u
     for (int k = 0; k < 4; ++k) z[k] = (int)lo[k] - T;
 }
 
-// The same by the table of bins in shared memory (`bins_s`): one load per uniform and no loop.  Which bin a uniform falls into
-// is its sum's exponent and first bits of fraction, truncated.  Returns false if one of the four lies in an open bin.
-__device__ __forceinline__ bool noise_levels4_bins(uint4 u4, uint32_t bins_s, int bits, int (&z)[4])
+// The same by the table of bins, in shared memory at `bins_s` or, if that is 0, in global memory: one load per uniform and no
+// loop.  Which bin a uniform falls into is its sum's exponent and first bits of fraction, truncated.  Returns false if one of
+// the four lies in an open bin.
+__device__ __forceinline__ bool noise_levels4_bins(uint4 u4, uint32_t bins_s, const uint2 *__restrict__ bins, int bits, int (&z)[4])
 {
     const uint32_t u[4] = {u4.x, u4.y, u4.z, u4.w};
     const uint32_t first = bins_s - 8u * ((uint32_t)(127 + kNoiseBinsFrom) << bits), side = 8u * noise_bins_side(bits);
-    int top = 0;
+    uint2 entry[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const uint32_t upper = (uint32_t)((int)u[k] >> 31), t = u[k] ^ upper;
-        const uint32_t b = __float_as_uint(__uint2float_rz(t + (1u << kNoiseBinsFrom))) >> (23 - bits);
-        uint32_t boundary;
-        int level;
-        asm volatile("ld.shared.v2.b32 {%0,%1}, [%2];" : "=r"(boundary), "=r"(level) : "r"(first + 8u * b + (upper & side)));
-        top = max(top, level);
-        z[k] = level + (u[k] >= boundary ? 1 : 0);
+        const uint32_t at = first + 8u * (__float_as_uint(__uint2float_rz(t + (1u << kNoiseBinsFrom))) >> (23 - bits)) + (upper & side);
+        if (bins) entry[k] = __ldg(reinterpret_cast<const uint2 *>(reinterpret_cast<const char *>(bins) + at));
+        else asm volatile("ld.shared.v2.b32 {%0,%1}, [%2];" : "=r"(entry[k].x), "=r"(entry[k].y) : "r"(at));
+    }
+    int top = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        top = max(top, (int)entry[k].y);
+        z[k] = (int)entry[k].y + (u[k] >= entry[k].x ? 1 : 0);
     }
     return top < kNoiseOpen;
 }

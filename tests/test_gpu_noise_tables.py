@@ -1,6 +1,6 @@
-"""The first convolution's noise search: a layer that passes its pixels through shows every drawn level.  Standard deviations
-with tables of bins of every size, too wide for one, and of so few levels that most bins are open; both noise laws;
-widths of whole Philox blocks and not."""
+"""The noise search of the layer-by-layer engine's first convolution, shown by a layer that passes its pixels through, and
+of the resident engine's input phase.  Standard deviations with tables of bins of every size, too wide for one, and of so
+few levels that most bins are open; both noise laws; widths of whole Philox blocks and not."""
 import numpy as np
 import pytest
 
@@ -32,5 +32,21 @@ def test_every_level_that_is_drawn(sigma, noise, h, w):
             want = oracle.noisy_input(x, 9, 1, 1, sample, sigma).astype(np.int32) - 128
             got = np.asarray(gm.debug_tensor(x, 9, 1, 1, sample, sigma, 1, 16 * h * w)).reshape(16, h, w)
             np.testing.assert_array_equal(got[:3], want)
+    finally:
+        oracle.set_noise_kind(0)
+
+
+@pytest.mark.parametrize("sigma", [0.001, 0.01, 0.25, 0.5, 1.0, 1.5])
+@pytest.mark.parametrize("noise", [0, 1])
+def test_every_level_of_the_resident_engine(sigma, noise):
+    gm = isc.Model(wl.spread_model("resnet20"))
+    gm.set_option("engine", 3)
+    gm.set_option("noise", noise)
+    x = np.random.default_rng(8).integers(0, 256, (3, 32, 32)).astype(np.uint8)
+    oracle.set_noise_kind(noise)
+    try:
+        for sample in range(12):
+            want = oracle.noisy_input(x, 9, 1, 1, sample, sigma).ravel()
+            np.testing.assert_array_equal(gm.debug_tensor(x, 9, 1, 1, sample, sigma, 0, x.size), want)
     finally:
         oracle.set_noise_kind(0)
