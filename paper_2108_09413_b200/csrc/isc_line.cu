@@ -19,10 +19,10 @@
 // Stacked convolutions.  For a 3x3, stride-1 convolution the three vertical taps are stacked along N: one MMA
 // chain over input line p (K = three horizontal taps x input channels) accumulates into the accumulator
 // columns of output lines p-1, p, p+1 at once (N = 3 x cout), because the accumulators of consecutive output
-// lines are consecutive column blocks of tensor memory.  The epilogue zeroes a line's columns after reading
-// them.  This triples N for the small channel counts where an MMA is bound by fetching its 128 x 32-byte A
-// operand.  Strided and 1x1 convolutions, and those with cout = 64, run unstacked: one chain per output line
-// over all taps.
+// lines are consecutive column blocks of tensor memory.  The epilogue, once it has read a line's columns, puts there what
+// the next convolution on them starts from: its folded biases.  This triples N where an MMA is bound by fetching its
+// 128 x 32-byte A operand.  With 16 input channels two lines share their odd K units (three MMAs for two lines).  Strided
+// and 1x1 convolutions run unstacked: one chain per output line over all taps.
 //
 // Roles.  Three issuing warps (lane 0 of each) share the MMA chains of a convolution: the host prepares a table of
 // operations (accumulator columns, descriptor offsets, which units of the previous convolution must be stored,
@@ -32,8 +32,11 @@
 // timed wait out of line).  Sixteen epilogue warps requantise: four sets of four warps (one per 32-lane quarter of
 // tensor memory) share the items of a convolution, an item being one unit (two or four output lines: one
 // "accumulators complete" barrier pair, one "stored" counter) and one 16-channel chunk, in the order in which they
-// complete.  The requantisation is integer arithmetic on a pipe that issues multiplies, shifts and packs at half
-// rate: the pass is written for the fewest such instructions (see ChanConst4).  A loader warp copies the next
+// complete.  An epilogue thread reads accumulators as fragments (tcgen05.ld 16x256b: four positions, four consecutive
+// channels of each), so that a channel's constants, held in registers for the pass, serve four outputs and residual and
+// result bytes move as words (with a position per thread every output took its constants from shared memory: a ResNet-110
+// group 460 -> 397 us; the shared K units of 16 input channels then brought it to 375).  The requantisation is integer arithmetic on a pipe that issues multiplies,
+// shifts and packs at half rate: the pass is written for the fewest such instructions (see requant4).  A loader warp copies the next
 // convolution's blob once its place is free.  Consecutive convolutions overlap unit by unit.  Input noise (Def. 3.3,
 // Eq. 2; Def. 3.4), halo fills and the pool / FC / argmax tail are CTA-wide phases between barriers.
 //
