@@ -346,7 +346,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_halo(const __grid_constant__ Ha
     __shared__ unsigned long long bar_a_full[kMaxRing], bar_a_free[kMaxRing], bar_b_full[kMaxRing], bar_b_free[kMaxRing], bar_acc_full[4], bar_acc_free[4];
     __shared__ uint32_t tmem_base_s;
     __shared__ volatile int abort_s;
-    chain_start();
     const GLayer &L = p.L;
     const int tid = threadIdx.x, warp = (int)warp_uniform((uint32_t)tid >> 5), lane = tid & 31;
     const uint32_t sbase = smem_u32(smem);
@@ -366,6 +365,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_halo(const __grid_constant__ Ha
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    chain_start();
     const uint32_t tmem = tmem_base_s;
     chain_wait();
     const uint32_t block_bytes = (uint32_t)(p.n_tile * L.kh) * 32u;

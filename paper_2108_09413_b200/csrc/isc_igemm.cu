@@ -318,7 +318,6 @@ __global__ void __launch_bounds__(igemm_threads(kWhole, kCopy), 1) k_igemm(const
     __shared__ unsigned long long bar_full[kMaxStages], bar_free[kMaxStages], bar_acc_full[4], bar_acc_free[4];
     __shared__ uint32_t tmem_base_s;
     __shared__ volatile int abort_s;
-    chain_start();
     const GLayer &L = p.L;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t sbase = smem_u32(smem);
@@ -338,6 +337,7 @@ __global__ void __launch_bounds__(igemm_threads(kWhole, kCopy), 1) k_igemm(const
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    chain_start();
     const uint32_t tmem = tmem_base_s;
     chain_wait();
 
@@ -612,7 +612,6 @@ __global__ void __launch_bounds__(kStemThreads, 2) k_stem(const __grid_constant_
     __shared__ uint32_t tmem_base_s;
     __shared__ volatile int abort_s;
     __shared__ __align__(16) int4 cst_s[256];
-    chain_start();
     const GLayer &L = p.L;
     const int tid = threadIdx.x, warp = (int)warp_uniform((uint32_t)tid >> 5);
     const uint32_t sbase = smem_u32(smem);
@@ -629,6 +628,7 @@ __global__ void __launch_bounds__(kStemThreads, 2) k_stem(const __grid_constant_
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    chain_start();
     const uint32_t tmem = tmem_base_s;
     if (tid == 0 && !p.debug_stall) {
         mbar_expect_tx(smem_u32(&bar_w), p.w_bytes);
