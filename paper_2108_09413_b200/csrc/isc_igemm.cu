@@ -969,7 +969,7 @@ bool igemm_constants(const GLayer &G, const int32_t *bias_folded, const int32_t 
     for (int o = 0; o < G.cout && short_form; ++o) {
         const int s = shift[o] - 1;
         const long long add = (1ll << (s - 1)) + ((long long)G.zp_out - c_res) * (1ll << s);
-        short_form = add > -(1ll << 31) && add < (1ll << 31);
+        short_form = requant_addend_fits(add);
     }
     if (!short_form) c_res = 0;
     if (form) *form = short_form ? f : ResidualForm();

@@ -118,6 +118,9 @@ struct ResidualForm {
     bool exists() const { return k8 != 0xFFFFFFFFu; }
 };
 ResidualForm residual_form(int res_mult, int res_shift, int zp_res, int32_t *c);
+// The 32-bit epilogues compute (hi32(acc * mult) + addend) >> s.  The loader refuses layers whose accumulators could reach
+// 2^30, so the product's high word lies in [-2^29, 2^29), and this is the room that the addend has to leave it in 32 bits.
+constexpr bool requant_addend_fits(long long addend) { return addend >= -(3ll << 29) && addend <= 3ll << 29; }
 // Per-channel requantisation constants of the kernel's 32-bit epilogue (4 x int32 for `n_out` channels); returns
 // whether the layer qualifies for it (every shift >= 2).
 bool igemm_constants(const GLayer &G, const int32_t *bias_folded, const int32_t *mult, const int32_t *shift, int32_t *out4, int n_out,
