@@ -1484,7 +1484,7 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
             for (int oc = 0; oc < L.cout && !general; ++oc) {
                 const int sft = layers[cp.layer].shift[oc] - 1;
                 const long long add = sft >= 1 ? (1ll << (sft - 1)) + ((long long)L.zp_out - cp.res_c) * (1ll << sft) : (1ll << 40);
-                general = add < -(1ll << 31) || add >= (1ll << 31);
+                general = !requant_addend_fits(add);
             }
             if (general) cp.res_c = 0;
         }

@@ -53,3 +53,12 @@ def test_residual_constants_leave_room_for_the_product(cin, cout, k, res_mult, z
               _wide(rng, 1, cin, cout, k, 1, 0, -128, zp_out, res=2, zp_res=zp_res, shift=shift)]
     layers[2].update(res_mult=res_mult, res_shift=0)
     _check(rng, (3, 12, 8), layers, 2, 700, 96)
+
+
+@pytest.mark.parametrize("res_mult,zp_res,zp_out,shift", [(2032202290, 7, -20, 18), (2032202290, 7, -20, 17), (1798879234, -20, 5, 14)])
+def test_residual_constants_of_the_resident_engine(res_mult, zp_res, zp_out, shift):
+    rng = np.random.default_rng(shift)
+    layers = [_conv(rng, 0, 3, 16, 3, 1, 1, 3, -128), _conv(rng, 1, 16, 32, 3, 2, 0, -128, zp_res), _conv(rng, 2, 32, 32, 3, 1, 1, zp_res, -128),
+              _wide(rng, 3, 32, 32, 3, 1, 0, -128, zp_out, res=2, zp_res=zp_res, shift=shift)]
+    layers[3].update(res_mult=res_mult, res_shift=0)
+    _check(rng, (3, 32, 32), layers, 3, 700, 256)
