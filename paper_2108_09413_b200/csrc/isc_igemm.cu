@@ -76,7 +76,7 @@ struct IgemmParams {
     const int8_t *wpack;                     // [cout tile][block][4 K columns][n_tile rows][16 bytes]
     const int8_t *zp_run;                    // 64 bytes of the input zero-point: the operand row of a pixel outside the image
     const int4 *cst;                         // per output channel: folded bias, multiplier, rounding addend, shift - 1
-    int fast_requant, fast_residual, lo;     // every shift >= 2; residual rescale by 2^-31 or 2^-32; lower clamp
+    int fast_requant, fast_residual, lo;     // the layer has the 32-bit form; residual rescale by 2^-31 or 2^-32; lower clamp
     uint32_t res_m2, res_k8;                 // residual multiplier in the 2^-32 form, or as a single-precision number; that form's offset
     int res_short;                           // the residual term is a single-precision product (see requant16_fast)
     int debug_stall;                         // test hook: the weights are never sent, so every wait of the kernel runs out
@@ -952,34 +952,30 @@ ResidualForm residual_form(int res_mult, int res_shift, int zp_res, int32_t *c_o
     return f;
 }
 
-// Per output channel {folded bias, multiplier, rounding addend, shift - 1}; returns whether every shift is >= 2 (the
-// condition of the 32-bit form).  `bias_folded`, `mult`, `shift` are the layer's host arrays padded to coutp.  For a
+// Per output channel {folded bias, multiplier, rounding addend, shift - 1}; returns whether the layer has the 32-bit form:
+// every shift is >= 2 and every addend leaves room for the product (shifts up to 24 whatever the zero-point).  `bias_folded`, `mult`, `shift` are the layer's host arrays padded to coutp.  For a
 // layer with a residual operand whose term is a single-precision product, that product's constant is folded into the
 // rounding addends.
 bool igemm_constants(const GLayer &G, const int32_t *bias_folded, const int32_t *mult, const int32_t *shift, int32_t *out4, int n_out,
                      bool has_residual, ResidualForm *form)
 {
     // channels beyond the layer's own (padding of the tensor and of the last tile) come out as zero
+    auto addend = [&](int o, int32_t c) { return (1ll << (shift[o] - 2)) + ((long long)G.zp_out - c) * (1ll << (shift[o] - 1)); };
     bool fast = true;
-    for (int o = 0; o < G.cout; ++o) fast = fast && shift[o] - 1 >= 1;
+    for (int o = 0; o < G.cout; ++o) fast = fast && shift[o] >= 2 && requant_addend_fits(addend(o, 0));
     int32_t c_res = 0;
     ResidualForm f;
     if (fast && has_residual) f = residual_form(G.res_mult, G.res_shift, G.zp_res, &c_res);
     bool short_form = f.exists();
-    for (int o = 0; o < G.cout && short_form; ++o) {
-        const int s = shift[o] - 1;
-        const long long add = (1ll << (s - 1)) + ((long long)G.zp_out - c_res) * (1ll << s);
-        short_form = requant_addend_fits(add);
-    }
+    for (int o = 0; o < G.cout && short_form; ++o) short_form = requant_addend_fits(addend(o, c_res));
     if (!short_form) c_res = 0;
     if (form) *form = short_form ? f : ResidualForm();
     memset(out4, 0, sizeof(int32_t) * 4 * (size_t)n_out);
-    for (int o = 0; o < G.cout; ++o) {
-        const int s = shift[o] - 1;
+    for (int o = 0; o < G.cout && fast; ++o) {                  // (the 64-bit form does not read them)
         out4[4 * o + 0] = bias_folded[o];
         out4[4 * o + 1] = mult[o];
-        out4[4 * o + 2] = s >= 1 ? (int32_t)((1ll << (s - 1)) + ((long long)G.zp_out - c_res) * (1ll << s)) : 0;
-        out4[4 * o + 3] = s >= 1 ? s : 0;
+        out4[4 * o + 2] = (int32_t)addend(o, c_res);
+        out4[4 * o + 3] = shift[o] - 1;
     }
     return fast;
 }

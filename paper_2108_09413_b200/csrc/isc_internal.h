@@ -122,7 +122,7 @@ ResidualForm residual_form(int res_mult, int res_shift, int zp_res, int32_t *c);
 // 2^30, so the product's high word lies in [-2^29, 2^29), and this is the room that the addend has to leave it in 32 bits.
 constexpr bool requant_addend_fits(long long addend) { return addend >= -(3ll << 29) && addend <= 3ll << 29; }
 // Per-channel requantisation constants of the kernel's 32-bit epilogue (4 x int32 for `n_out` channels); returns
-// whether the layer qualifies for it (every shift >= 2).
+// whether the layer qualifies for it (every shift >= 2, every addend leaves room for the product).
 bool igemm_constants(const GLayer &G, const int32_t *bias_folded, const int32_t *mult, const int32_t *shift, int32_t *out4, int n_out,
                      bool has_residual, ResidualForm *form);
 void igemm_order_constants(const GLayer &G, int32_t *out4, int n_out);      // ... in the order in which k_igemm reads them

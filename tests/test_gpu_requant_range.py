@@ -55,6 +55,29 @@ def test_residual_constants_leave_room_for_the_product(cin, cout, k, res_mult, z
     _check(rng, (3, 12, 8), layers, 2, 700, 96)
 
 
+# first convolution, resident-tile filter, whole tiles by tensor copy and gathered, paired, the general form, FC; 2^(s - 1) + zp_out 2^s
+# in 32 bits: fits with room for the product up to a shift of 24, without it at 25, not at all from 26 on
+@pytest.mark.parametrize("zp", [-128, 127, 5])
+@pytest.mark.parametrize("shift", [20, 24, 25, 26, 31])
+def test_addends_of_wide_shifts(shift, zp):
+    rng = np.random.default_rng(shift)
+    relu = int(zp == -128)
+    wide = lambda t, cin, cout, k, stride, z, **kw: _wide(rng, t, cin, cout, k, stride, relu, z, zp, shift=shift, **kw)
+    layers = [wide(0, 3, 64, 3, 1, 3), wide(1, 64, 64, 3, 1, zp), wide(2, 64, 256, 1, 1, zp), wide(3, 256, 64, 1, 1, zp),
+              wide(4, 64, 256, 1, 1, zp, res=3, zp_res=zp), wide(5, 256, 128, 1, 2, zp), wide(6, 128, 48, 1, 1, zp)]
+    _check(rng, (3, 16, 12), layers, 2, 400, 48)
+
+
+# a wide shift on one channel among ordinary ones
+def test_one_channel_of_a_wide_shift():
+    rng = np.random.default_rng(3)
+    layers = [_conv(rng, 0, 3, 64, 3, 1, 1, 3, -128), _conv(rng, 1, 64, 64, 3, 1, 1, -128, -128), _conv(rng, 2, 64, 256, 1, 1, 0, -128, -128),
+              _conv(rng, 3, 256, 64, 1, 1, 1, -128, -128)]
+    for layer in layers:
+        layer["shift"][7] = 27
+    _check(rng, (3, 16, 12), layers, 2, 400, 192)
+
+
 @pytest.mark.parametrize("res_mult,zp_res,zp_out,shift", [(2032202290, 7, -20, 18), (2032202290, 7, -20, 17), (1798879234, -20, 5, 14)])
 def test_residual_constants_of_the_resident_engine(res_mult, zp_res, zp_out, shift):
     rng = np.random.default_rng(shift)
