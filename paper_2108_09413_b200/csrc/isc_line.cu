@@ -1507,7 +1507,11 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
         }
         cp.cls = class_of[key];
         cp.use_local = class_uses[(size_t)cp.cls]++;
-        const bool wait_all = pv && (pv->cls != cp.cls || !same_class);
+        // Maps in several bands: the edge rows of a band are copied into the padding lines of its neighbours, and those copies
+        // are ordered line by line through the rows above and below that a stacked filter on the previous convolution's
+        // output waits for.  A 1 x 1 convolution, or one of an older tensor, waits for the rows it adds to only: by then the
+        // copies that it reads may not be written, and others may still be read that its own will overwrite.
+        const bool wait_all = pv && (pv->cls != cp.cls || !same_class || (in.nb > 1 && !(cp.stacked && aligned)));
         // Record i belongs to issuing thread i mod kIssuers; every thread needs a record to carry its arrivals.
         auto null_op = []() { ProtoOp o; o.a_line = 0; o.b_block = 0; o.n_blocks = 0; o.d_line = 0; o.n_chains = 0; o.ready = 0; return o; };
         while (proto.size() < (size_t)kIssuers) proto.push_back(null_op());

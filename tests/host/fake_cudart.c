@@ -12,7 +12,7 @@
 #define MAX_LAUNCHES 65536
 
 typedef struct { const void *host; const char *name; int smem[MAX_DEVICES]; } Func;
-typedef struct { const char *name; int device, stream_device, priority, ok, watched; } Launch;
+typedef struct { const char *name; int device, stream_device, priority, ok, watched; unsigned long long words[5]; } Launch;
 struct CUstream_st { int priority, device; };
 
 static Func funcs[MAX_FUNCS];
@@ -38,6 +38,8 @@ int fake_launch_ok(int i) { return launches[i].ok; }
 /* 1: the word `watch` stands in the launch's first argument */
 void fake_watch(const void *word) { watched = word; }
 int fake_launch_watched(int i) { return launches[i].watched; }
+/* word `k` of the first five of k_line's parameters */
+unsigned long long fake_launch_word(int i, int k) { return launches[i].words[k]; }
 size_t fake_allocated(void) { return allocated; }
 
 static Func *find(const void *host)
@@ -82,7 +84,8 @@ cudaError_t cudaLaunchKernel(const void *func, dim3 grid, dim3 block, void **arg
         /* the first argument of the kernels in question is a structure of more than 256 bytes */
         if (watched && (strstr(f->name, "k_stem") || strstr(f->name, "k_line")))
             for (int i = 0; i < 256 / 8; ++i) seen |= ((const void **)args[0])[i] == watched;
-        launches[n_launches++] = (Launch){f->name, device, st ? st->device : device, st ? st->priority : 0, ok, seen};
+        launches[n_launches++] = (Launch){f->name, device, st ? st->device : device, st ? st->priority : 0, ok, seen, {0}};
+        if (strstr(f->name, "k_line")) memcpy(launches[n_launches - 1].words, args[0], sizeof(launches[0].words));
     }
     pthread_mutex_unlock(&lock);
     if (!ok) last = cudaErrorInvalidValue;

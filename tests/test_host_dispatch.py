@@ -32,6 +32,7 @@ def _fake():
     f.fake_launch_name.restype = C.c_char_p
     f.fake_allocated.restype = C.c_size_t
     f.fake_watch.argtypes = [C.c_void_p]
+    f.fake_launch_word.restype = C.c_ulonglong
     return f
 
 
@@ -225,11 +226,52 @@ def stalled_launches_reach_every_kernel():
         assert _kernels(f) == ([kernel] if tensor_cores else [])
 
 
+def resident_plans_order_rows_of_other_bands():
+    """Maps of 16 x 16 lie in two bands whose edge rows are copied into each other's padding.  Only a stacked filter on the
+    output of the convolution before it waits, through its rows above and below, for those copies' readers and writers
+    one by one; any other convolution has to wait for all of the one before."""
+    import paper_2108_09413_b200 as isc
+    import workloads as wl
+    f = _fake()
+    rng = wl.SplitMix64(6)
+
+    def record(at, count, dtype=np.uint32):
+        return np.frombuffer(C.string_at(int(at), count * np.dtype(dtype).itemsize), dtype)
+
+    def wait_for_all(layers, side):
+        """per convolution: whether each issuing thread's first record waits for all of the convolution before"""
+        n, c = len(layers), layers[-1]["cout"]
+        layers = layers + [wl._gavgpool(n, c, side * side, -128), wl._conv(rng, n + 1, c, 5, 1, 1, 0, False, -128, 0, op=wl.OP_FC)]
+        gm = isc.Model(dict(in_shape=(3, 32, 32), n_classes=5, layers=layers))
+        gm.set_option("engine", 3)
+        f.fake_reset()
+        gm.sample_counts(wl.images(1)[0], 1, 0, 1, 0, 9, 0.25)
+        params = np.array([f.fake_launch_word(0, k) for k in range(5)], np.uint64)       # phase table, blobs' sources, counts, (barriers, phases), (convolutions, ..)
+        out = []
+        for k in range(int(params[4] & 0xFFFFFFFF)):
+            blob = int(record(int(params[1]) + 32 * k, 1, np.uint64)[0])
+            n_ops, _, ops = record(blob + 112, 3)
+            assert n_ops >= 3
+            out.append([bool(record(blob + int(ops) + 32 * r + 30, 1, np.uint16)[0] & 1) for r in range(3)])
+        assert all(len(set(w)) == 1 for w in out)
+        return [w[0] for w in out]
+
+    conv = lambda t, cin, cout, k, stride=1, res=-1: wl._conv(rng, t, cin, cout, k, stride, k // 2, True, 3 if t == 0 else -128, -128)
+    stem = [conv(0, 3, 16, 3), conv(1, 16, 32, 3, 2)]                        # tensor 2: 32 x 16 x 16, in two bands
+    # 1 x 1 in place over tensor 3; a filter on an older tensor than the last, over the last one's input
+    assert wait_for_all(stem + [conv(2, 32, 32, 3), conv(3, 32, 32, 3), conv(4, 32, 32, 1, res=3), conv(5, 32, 32, 3)], 16)[3:] == [False, True, False]
+    assert wait_for_all(stem + [conv(2, 32, 32, 3), conv(3, 32, 32, 3), conv(2, 32, 32, 3, res=4)], 16)[3:] == [False, True]
+    # one band: rows above and below the map are padding
+    assert wait_for_all([conv(0, 3, 16, 3), conv(1, 16, 16, 3), conv(2, 16, 16, 1)], 32)[1:] == [False, False]
+    # basic blocks need no such wait
+    assert not any(wait_for_all(wl.resnet20()["layers"][:-2], 8))
+
+
 # ------------------------------------------------------------------ the tests
 
 SCENARIOS = [layer_too_wide_for_shared_memory, first_calls_in_two_threads, every_device, device_images_of_any_alignment,
              static_entry_point_takes_the_engine_it_is_told, weights_are_on_the_device_once_per_kernel,
-             side_streams_keep_the_callers_priority, stalled_launches_reach_every_kernel]
+             side_streams_keep_the_callers_priority, resident_plans_order_rows_of_other_bands, stalled_launches_reach_every_kernel]
 
 
 @pytest.mark.parametrize("scenario", [s.__name__ for s in SCENARIOS])
