@@ -337,7 +337,10 @@ int isc_debug_residual_form(int32_t res_mult, int32_t res_shift, int32_t zp_res,
  *              changes no result.
  *   "noise"  : 0 = the discrete Gaussian of Def. 3.3 / Eq. 2 (IntRS, the default), 1 = the
  *              rounded continuous Gaussian of the comparison method (isc_noise_table_rounded).
- *   "batch"  : noisy samples per launch (0 = choose automatically).
+ *   "batch"  : noisy samples per launch (0 = choose automatically).  On the layer-by-layer engines a
+ *              handle keeps the activations of one launch's samples on the device: up to 8,192 samples
+ *              by default, and 3 GiB whatever the option says.  Where the device's memory does not hold
+ *              that, launches shrink by halves to what it holds, until the option is set again.
  *   "engine" : 0 = automatic (3 if the model fits it, else 2 if any layer fits it, else 1),
  *              1 = layer-by-layer kernels without tensor cores, 2 = layer-by-layer with
  *              the tcgen05 kernels for every convolution and FC layer, 3 = the line-tiled

@@ -60,6 +60,7 @@ struct isc_model {
     std::vector<size_t> buf_bytes;
     std::vector<DevBuf> bufs;
     int ws_batch = 0;
+    int64_t ws_limit = INT64_MAX;               // samples that the device's memory held when it did not hold more
 
     // per-call device scratch
     // One buffer: error word (16 bytes), vote counts, images.  A call's upload (zeros and images) and its download (error
@@ -329,16 +330,26 @@ int ensure_bytes(void **p, size_t *have, size_t need)
     return ISC_OK;
 }
 
+void free_workspace(isc_model *m)
+{
+    for (DevBuf &b : m->bufs) {
+        if (b.p) cudaFree(b.p);
+        b = DevBuf();
+    }
+    m->ws_batch = 0;
+}
+
 int ensure_workspace(isc_model *m, int batch)
 {
     if (batch <= m->ws_batch) return ISC_OK;
+    free_workspace(m);
     for (size_t b = 0; b < m->bufs.size(); ++b) {
-        if (m->bufs[b].p) cudaFree(m->bufs[b].p);
-        m->bufs[b].p = nullptr;
-    }
-    m->ws_batch = 0;
-    for (size_t b = 0; b < m->bufs.size(); ++b) {
-        CK(cudaMalloc(&m->bufs[b].p, m->buf_bytes[b] * (size_t)batch));
+        const cudaError_t e = cudaMalloc(&m->bufs[b].p, m->buf_bytes[b] * (size_t)batch);
+        if (e != cudaSuccess) {
+            m->bufs[b].p = nullptr;
+            free_workspace(m);
+            CK(e);
+        }
         m->bufs[b].bytes = m->buf_bytes[b] * (size_t)batch;
     }
     m->ws_batch = batch;
@@ -567,14 +578,16 @@ int64_t layerwise_cap(const isc_model *m)
     int64_t cap = m->opt_batch > 0 ? m->opt_batch : 8192;
     const size_t per = std::max<size_t>(generic_bytes_per_sample(m), 1);
     cap = std::min<int64_t>(cap, std::max<int64_t>(1, (int64_t)((3ull << 30) / per)));
-    return std::min<int64_t>(cap, m->last_engine == 2 ? tensor_core_cap(m) : 32768);
+    return std::min<int64_t>(std::min(cap, m->ws_limit), m->last_engine == 2 ? tensor_core_cap(m) : 32768);
 }
 
-// forward_counts in the handle's own buffers.
+// forward_counts in the handle's own buffers.  Where the device's memory does not hold a batch, half of it and so on; the
+// handle then keeps to what fitted, so that later calls do not try in vain.
 int layerwise_counts(isc_model *m, const uint8_t *d_x, uint64_t seed, const SampleRun &run, int64_t total, cudaStream_t st, int32_t *d_counts, int8_t *d_logits, int32_t *d_err)
 {
-    const int64_t cap = layerwise_cap(m);
-    int rc = ensure_workspace(m, (int)std::min<int64_t>(cap, std::max<int64_t>(total, 1)));
+    int64_t cap = std::min<int64_t>(layerwise_cap(m), std::max<int64_t>(total, 1));
+    int rc;
+    while ((rc = ensure_workspace(m, (int)cap)) == ISC_ERR_NOMEM && cap > 1) m->ws_limit = cap = (cap + 1) / 2;
     if (rc) return rc;
     return forward_counts(m, own_buffers(m).data(), cap, m->last_engine == 2, d_x, make_stream(m, seed, 0, 0, 0), run, total, st, d_counts, d_logits, d_err);
 }
@@ -1256,6 +1269,7 @@ int isc_set_option(isc_model *m, const char *name, int64_t value)
     if (!strcmp(name, "batch")) {
         if (value < 0 || value > (1 << 20)) return ISC_ERR_ARG;
         m->opt_batch = value;
+        m->ws_limit = INT64_MAX;
         return ISC_OK;
     }
     if (!strcmp(name, "noise")) {

@@ -18,7 +18,8 @@ struct CUstream_st { int priority, device; };
 static Func funcs[MAX_FUNCS];
 static int n_funcs, n_launches, set_attribute_delay_us;
 static Launch launches[MAX_LAUNCHES];
-static size_t allocated;
+static size_t allocated, largest = (size_t)-1;
+static int refused;
 static const void *watched;
 static pthread_mutex_t lock = PTHREAD_MUTEX_INITIALIZER;
 static __thread int device;
@@ -41,6 +42,9 @@ int fake_launch_watched(int i) { return launches[i].watched; }
 /* word `k` of the first five of k_line's parameters */
 unsigned long long fake_launch_word(int i, int k) { return launches[i].words[k]; }
 size_t fake_allocated(void) { return allocated; }
+/* larger allocations are refused from now on; how many were */
+void fake_set_largest(size_t bytes) { largest = bytes; refused = 0; }
+int fake_refused(void) { return refused; }
 
 static Func *find(const void *host)
 {
@@ -135,8 +139,10 @@ cudaError_t cudaGetSymbolAddress(void **p, const void *symbol)
 cudaError_t cudaMalloc(void **p, size_t bytes)
 {
     pthread_mutex_lock(&lock);
-    allocated += bytes;
+    const int fits = bytes <= largest;
+    if (fits) allocated += bytes; else refused += 1;
     pthread_mutex_unlock(&lock);
+    if (!fits) return last = cudaErrorMemoryAllocation;
     return posix_memalign(p, 256, bytes) ? cudaErrorMemoryAllocation : cudaSuccess;
 }
 cudaError_t cudaFree(void *p) { free(p); return cudaSuccess; }

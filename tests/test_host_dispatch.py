@@ -33,6 +33,7 @@ def _fake():
     f.fake_allocated.restype = C.c_size_t
     f.fake_watch.argtypes = [C.c_void_p]
     f.fake_launch_word.restype = C.c_ulonglong
+    f.fake_set_largest.argtypes = [C.c_size_t]
     return f
 
 
@@ -226,6 +227,42 @@ def stalled_launches_reach_every_kernel():
         assert _kernels(f) == ([kernel] if tensor_cores else [])
 
 
+def batches_shrink_to_the_memory_there_is():
+    """A call whose default batch the device's memory does not hold takes a smaller one, and later calls do not try in vain."""
+    import paper_2108_09413_b200 as isc
+    import workloads as wl
+    f = _fake()
+    model = _filter_net(wl)
+    per_sample = 24 * 36 * 256                                    # the largest activation tensor
+    x = wl.images(1, shape=model["in_shape"])[0]
+    for engine in (1, 2):
+        gm = isc.Model(model)
+        gm.set_option("engine", engine)
+        launches = lambda: sum(k in ("k_stem", "k_first_conv") for k in _kernels(f))
+        cap = 3 * 2 ** 30 // (24 * 36 * (96 + 256))               # 3 GiB of two buffers
+        def call(n):
+            f.fake_reset()
+            gm.sample_counts(x, 1, 0, 1, 0, n, 0.25)
+            return launches()
+        f.fake_set_largest(2 ** 62)
+        assert call(500) == 1
+        f.fake_set_largest(1000 * per_sample)
+        assert call(5000) == -(-5000 // 625) and f.fake_refused() == 3       # 5,000, 2,500 and 1,250 do not fit
+        assert call(5000) == 8 and call(100) == 1 and f.fake_refused() == 3
+        gm.certify_batch(wl.images(3, shape=model["in_shape"]), 3, 1, 0, 100, 900, 0.25, 0.001)
+        assert f.fake_refused() == 3
+        f.fake_set_largest(2 ** 62)
+        gm.set_option("batch", 0)
+        assert call(5000) == -(-5000 // cap) < 8
+        gm.close()
+        gm = isc.Model(model)
+        gm.set_option("engine", engine)
+        f.fake_set_largest(per_sample - 1)
+        with pytest.raises(isc.IscError) as e:
+            gm.sample_counts(x, 1, 0, 1, 0, 5, 0.25)
+        assert e.value.code == -4
+
+
 def resident_plans_order_rows_of_other_bands():
     """Maps of 16 x 16 lie in two bands whose edge rows are copied into each other's padding.  Only a stacked filter on the
     output of the convolution before it waits, through its rows above and below, for those copies' readers and writers
@@ -271,7 +308,8 @@ def resident_plans_order_rows_of_other_bands():
 
 SCENARIOS = [layer_too_wide_for_shared_memory, first_calls_in_two_threads, every_device, device_images_of_any_alignment,
              static_entry_point_takes_the_engine_it_is_told, weights_are_on_the_device_once_per_kernel,
-             side_streams_keep_the_callers_priority, resident_plans_order_rows_of_other_bands, stalled_launches_reach_every_kernel]
+             side_streams_keep_the_callers_priority, resident_plans_order_rows_of_other_bands,
+             batches_shrink_to_the_memory_there_is, stalled_launches_reach_every_kernel]
 
 
 @pytest.mark.parametrize("scenario", [s.__name__ for s in SCENARIOS])
