@@ -356,43 +356,75 @@ int ensure_workspace(isc_model *m, int batch)
     return ISC_OK;
 }
 
-// The table of bins at `bits` bits; false if more than one uniform in 2^11 lies in an open bin: the 128 of a warp share
-// the way out, which then costs what the bins save (sixteen warps in all meet one).
-bool noise_bins(const uint32_t *cum, size_t n_cum, int bits, std::vector<uint32_t> &out)
+// Appends the table of bins at `bits` bits to the tables at `tab`, which begin with the cumulative one; false, and nothing
+// appended, if more than one uniform in 2^11 lies in an open bin: the 128 of a warp share the way out, which then costs what the
+// bins save (sixteen warps in all meet one).  The boundaries are counted per bin, from the middle of the range outwards, so that a
+// vain try ends at once: where bins are too wide for the law, those in the middle are.  (Looking up both ends of every
+// bin, in up to three full tries, took 37 us of a call with a new standard deviation of 1; this takes 14.)
+bool noise_bins(std::vector<uint32_t> &tab, size_t n_cum, int bits)
 {
-    const uint32_t side = isc::noise_bins_side(bits), one = 1u << bits;
-    out.assign(4 * (size_t)side, 0);
-    uint64_t open = 0;
-    size_t at = 0;                                                                 // neighbouring bins' levels lie close together
-    auto level = [&](uint32_t u) {
-        while (at + 1 < n_cum && u >= cum[at]) ++at;
-        while (at > 0 && u < cum[at - 1]) --at;
-        return at;
+    const uint32_t side = isc::noise_bins_side(bits), one = 1u << bits, from = 1u << isc::kNoiseBinsFrom, limit = 1u << 21;
+    const size_t front = tab.size();
+    const uint32_t n_bounds = (uint32_t)n_cum - 1;                       // level i + 1 begins at cum[i]
+    const uint32_t middle = std::min((uint32_t)(std::upper_bound(tab.begin(), tab.begin() + n_cum, 0x7FFFFFFFu) - tab.begin()), n_bounds);
+    // uniforms of bin b: all but the last bins are 2^e of them
+    auto size_of = [&](uint32_t b) {
+        const int e = isc::kNoiseBinsFrom + (int)(b >> bits) - bits;
+        return e + bits < 31 ? 1u << e : b == side - 2 ? from : 0u;      // sums from 2^31 on: one bin up to 2^31 + 2^21, none beyond
     };
-    for (uint32_t upper = 0; upper < 2; ++upper)
-        for (uint32_t b = 0; b < side; ++b) {
-            const int e = isc::kNoiseBinsFrom + (int)(b >> bits) - bits;
-            const uint64_t v0 = (uint64_t)(one + (b & (one - 1))) << e, v1 = v0 + (1ull << e) - 1, from = 1ull << isc::kNoiseBinsFrom;
-            const uint64_t t0 = v0 - from, t1 = std::min<uint64_t>(v1 - from, 0x7FFFFFFFull);
-            uint32_t *entry = &out[2 * ((size_t)upper * side + b)];
-            entry[1] = (uint32_t)isc::kNoiseOpen;
-            if (t0 > t1) continue;                                                 // no uniform has this bin
-            const size_t i0 = level(upper ? ~(uint32_t)t1 : (uint32_t)t0), i1 = level(upper ? ~(uint32_t)t0 : (uint32_t)t1);
-            if (i1 > i0 + 1 || i0 + 1 == n_cum) {                                  // (the last level has no boundary above it)
-                if ((open += t1 - t0 + 1) > 1ull << 21) return false;
-                continue;
+    // per bin: boundaries between two of its uniforms; between its first one (as counted from the end) and the bin before
+    std::vector<uint16_t> counts(4 * (size_t)side, 0);
+    uint64_t open = 0;
+    for (uint32_t upper = 0; upper < 2; ++upper) {
+        uint16_t *inside = counts.data() + 2 * (size_t)upper * side, *before = inside + side;
+        const uint32_t n = upper ? n_bounds - middle : middle;
+        for (uint32_t k = 0; k < n; ++k) {
+            const uint32_t c = tab[upper ? middle + k : middle - 1 - k], first = upper ? 0u - c : c;       // the bound's larger distance from the end
+            if (first > 0x7FFFFFFFu) continue;                           // between the two sides
+            const uint32_t v = first + from;
+            if (v < from + (from >> bits)) {                             // the outermost bin: the rest of the tail lies in it
+                before[0] = upper ? 0 : (uint16_t)(std::upper_bound(tab.begin(), tab.begin() + n_cum, 0u) - tab.begin());
+                inside[0] = (uint16_t)(n - k - before[0]);
+                if (inside[0] > 1) open += size_of(0);
+                break;
             }
-            entry[0] = cum[i0];
-            entry[1] = (uint32_t)((int)i0 - (int)(n_cum - 1) / 2);
+            const int e = 31 - __builtin_clz(v) - bits;
+            const uint32_t b = ((uint32_t)(e + bits - isc::kNoiseBinsFrom) << bits) + (v >> e) - one;
+            if ((v & ((1u << e) - 1)) == 0) before[b] += 1;
+            else if (++inside[b] == 2 && (open += size_of(b)) > limit) return false;
         }
-    return true;
+    }
+    tab.resize(front + 4 * (size_t)side);
+    const uint32_t *cum = tab.data();
+    const uint32_t T = n_bounds / 2;
+    for (uint32_t upper = 0; upper < 2; ++upper) {
+        const uint16_t *inside = counts.data() + 2 * (size_t)upper * side, *before = inside + side;
+        uint32_t *entry = tab.data() + front + 2 * (size_t)upper * side;
+        uint32_t at = upper ? n_bounds : 0;                              // the level from where the bins come from
+        for (uint32_t b = 0; b < side; ++b, entry += 2) {
+            const uint32_t low = upper ? at - before[b] - inside[b] : at + before[b];       // level of its smallest uniform
+            at = upper ? low : low + inside[b];
+            entry[0] = cum[low];
+            entry[1] = low - T;
+            if (inside[b] <= 1 && low != n_bounds) continue;
+            if (inside[b] <= 1) open += size_of(b);                                         // the last level has no boundary above it
+            entry[0] = 0;
+            entry[1] = (uint32_t)isc::kNoiseOpen;
+        }
+        entry[-2] = 0;                                                                      // no uniform has the last bin
+        entry[-1] = (uint32_t)isc::kNoiseOpen;
+    }
+    if (open > limit) tab.resize(front);
+    return open <= limit;
 }
 
 // The noise law's table for `sigma` on the host, kept for the next call.
 void host_noise_table(isc_model *m, double sigma)
 {
     if (m->tab_sigma == sigma && m->tab_kind == (int)m->opt_noise) return;
-    std::vector<uint32_t> cum;
+    std::vector<uint32_t> &cum = m->h_tab;
+    m->tab_sigma = -1.0;
+    cum.reserve((size_t)(2 * noise_halfwidth(sigma) + 1) + (isc::kNoiseGuide + 1) + 3 + 4 * (size_t)isc::noise_bins_side(8));
     if (m->opt_noise) noise_table_rounded(sigma, cum); else noise_table(sigma, cum);
     // the guide table and the bins follow the cumulative one in the same allocation
     const size_t n_cum = cum.size();
@@ -411,11 +443,8 @@ void host_noise_table(isc_model *m, double sigma)
     m->tab_front = (cum.size() + 3) & ~(size_t)3;
     cum.resize(m->tab_front, 0);
     m->tab_bin_bits = 0;
-    std::vector<uint32_t> bins;
     for (int bits = 6; bits <= 8 && !m->tab_bin_bits; ++bits)
-        if (noise_bins(cum.data(), n_cum, bits, bins)) m->tab_bin_bits = bits;
-    if (m->tab_bin_bits) cum.insert(cum.end(), bins.begin(), bins.end());
-    m->h_tab.swap(cum);
+        if (noise_bins(cum, n_cum, bits)) m->tab_bin_bits = bits;
     m->tab_sigma = sigma;
     m->tab_kind = (int)m->opt_noise;
 }

@@ -12,7 +12,7 @@
 #define MAX_LAUNCHES 65536
 
 typedef struct { const void *host; const char *name; int smem[MAX_DEVICES]; } Func;
-typedef struct { const char *name; int device, stream_device, priority, ok, watched; unsigned long long words[5]; } Launch;
+typedef struct { const char *name; int device, stream_device, priority, ok, watched; unsigned long long words[20]; } Launch;
 struct CUstream_st { int priority, device; };
 
 static Func funcs[MAX_FUNCS];
@@ -39,7 +39,7 @@ int fake_launch_ok(int i) { return launches[i].ok; }
 /* 1: the word `watch` stands in the launch's first argument */
 void fake_watch(const void *word) { watched = word; }
 int fake_launch_watched(int i) { return launches[i].watched; }
-/* word `k` of the first five of k_line's parameters */
+/* word `k` of the first twenty of k_line's parameters */
 unsigned long long fake_launch_word(int i, int k) { return launches[i].words[k]; }
 size_t fake_allocated(void) { return allocated; }
 /* larger allocations are refused from now on; how many were */

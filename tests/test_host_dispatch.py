@@ -227,6 +227,46 @@ def stalled_launches_reach_every_kernel():
         assert _kernels(f) == ([kernel] if tensor_cores else [])
 
 
+def bins_hold_the_levels_of_the_search():
+    """The noise law's table of bins against the search in its cumulative table: every boundary between two levels and the
+    uniforms beside it, both ends, the middle, the edges of all bins, and random ones."""
+    import paper_2108_09413_b200 as isc
+    import workloads as wl
+    f = _fake()
+    gm = isc.Model(wl.tiny_cnn())
+    x = wl.images(1)[0]
+    rng = np.random.default_rng(1)
+    sizes = {}
+    for noise in (0, 1):
+        gm.set_option("noise", noise)
+        for sigma in (1e-4, 0.001, 0.003, 0.01, 0.12, 0.25, 0.4, 0.5, 0.65, 0.7, 1.0, 1.31, 1.32, 2.0, 40.0):
+            f.fake_reset()
+            gm.sample_counts(x, 1, 0, 1, 0, 1, sigma)
+            word = [f.fake_launch_word(0, k) for k in range(20)]
+            bits = sizes[noise, sigma] = word[19] & 0xFFFFFFFF if word[18] else 0
+            if not bits:
+                continue
+            cum = isc.noise_table(sigma, rounded=bool(noise)).astype(np.int64)
+            T = cum.size // 2
+            side = (10 << bits) + 2
+            bins = np.frombuffer(C.string_at(word[18], 16 * side), np.uint32).astype(np.int64).reshape(2, side, 2)
+            # distances from the end at which bins begin
+            edges = np.concatenate([((1 << bits) + np.arange(1 << bits)) << (21 + o - bits) for o in range(10)]) - 2 ** 21
+            near = np.concatenate([cum, edges, 2 ** 32 - 1 - edges, [0, 2 ** 31, 2 ** 31 - 2 ** 21, 2 ** 31 + 2 ** 21, 2 ** 32 - 1]])
+            u = np.clip(np.concatenate([near + d for d in (-1, 0, 1)] + [rng.integers(0, 2 ** 32, 200_000)]), 0, 2 ** 32 - 1)
+            want = np.minimum(np.searchsorted(cum, u, side="right"), 2 * T) - T
+            upper = (u >> 31).astype(int)
+            sums = np.where(upper == 1, 2 ** 32 - 1 - u, u) + 2 ** 21
+            e = np.frexp(sums.astype(np.float64))[1] - 1
+            at = ((e - 21) << bits) + (sums >> (e - bits)) - (1 << bits)
+            bound, level = bins[upper, at, 0], bins[upper, at, 1]
+            level = np.where(level >= 2 ** 31, level - 2 ** 32, level)
+            known = level != 1 << 30
+            np.testing.assert_array_equal((level + (u >= bound))[known], want[known])
+            assert known[-200_000:].mean() > 1 - 2 ** -10
+    assert {s: b for (n, s), b in sizes.items() if n == 0} == {1e-4: 6, 0.001: 6, 0.003: 6, 0.01: 6, 0.12: 6, 0.25: 6, 0.4: 7, 0.5: 7, 0.65: 7, 0.7: 8, 1.0: 8, 1.31: 8, 1.32: 0, 2.0: 0, 40.0: 0}
+
+
 def batches_shrink_to_the_memory_there_is():
     """A call whose default batch the device's memory does not hold takes a smaller one, and later calls do not try in vain."""
     import paper_2108_09413_b200 as isc
@@ -309,7 +349,7 @@ def resident_plans_order_rows_of_other_bands():
 SCENARIOS = [layer_too_wide_for_shared_memory, first_calls_in_two_threads, every_device, device_images_of_any_alignment,
              static_entry_point_takes_the_engine_it_is_told, weights_are_on_the_device_once_per_kernel,
              side_streams_keep_the_callers_priority, resident_plans_order_rows_of_other_bands,
-             batches_shrink_to_the_memory_there_is, stalled_launches_reach_every_kernel]
+             batches_shrink_to_the_memory_there_is, bins_hold_the_levels_of_the_search, stalled_launches_reach_every_kernel]
 
 
 @pytest.mark.parametrize("scenario", [s.__name__ for s in SCENARIOS])
