@@ -166,8 +166,14 @@ __device__ __forceinline__ int mad_hi(int a, int b, int c)
     asm("mad.hi.s32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
     return d;
 }
-// round-to-nearest(v * m) for an integer v < 2^23, as an integer: both are read as denormal numbers, whose unit is one
-__device__ __forceinline__ int mul_denormal(uint32_t v, uint32_t m_bits) { return __float_as_int(__fmul_rn(__uint_as_float(v), __uint_as_float(m_bits))); }
+// round-to-nearest(v * m) for an integer v < 2^23, as an integer: both are read as denormal numbers, whose unit is one.  The
+// instruction is named, because a product of __fmul_rn would be zero in a build that flushes denormal numbers.
+__device__ __forceinline__ int mul_denormal(uint32_t v, uint32_t m_bits)
+{
+    float d;
+    asm("mul.rn.f32 %0, %1, %2;" : "=f"(d) : "f"(__uint_as_float(v)), "f"(__uint_as_float(m_bits)));
+    return __float_as_int(d);
+}
 __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1)
 {
 #pragma unroll
