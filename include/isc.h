@@ -318,12 +318,22 @@ int isc_debug_wait_timeout(isc_model *m, int64_t limit_ns, void *cuda_stream, in
 int isc_debug_stalled_launch(isc_model *m, int layer, void *cuda_stream, int32_t *out2);
 
 /*
- * isc_debug_residual_form -- host only.  The residual operand's rescale
- * rs((r - zp_res) * res_mult, 31 - res_shift) (the skip path's term of the residual add) is
- * floor((u * m2 + R2) / 2^32), u = r + 128, and, where an offset k < 4096 exists for which
- * floor((256 k + u) * m2 / 2^32) - c equals that for all 256 values of u, has this shorter form.
- * This call searches it in integers.  The tensor-core engines search the same form for a product in
- * single precision, round((256 k + u) * m) - c, and keep the long form where that does not exist.
+ * isc_debug_residual_product -- host only.  The residual operand's rescale
+ * rs((r - zp_res) * res_mult, 31 - res_shift) (the skip path's term of the residual add) in the form
+ * that the tensor-core engines compute where it exists: round((256 k + u) * m) - c, u = r + 128, for
+ * an offset k < 4096 and a single-precision number m with which this equals the rescale for all 256
+ * values of u (round: to nearest, ties to even).  This call runs the search that the engines run.
+ * They keep the 64-bit form floor((u * m2 + R2) / 2^32) where the product does not exist, and where a
+ * layer's shifts leave its constant c no room in the rounding addends.
+ *   returns : 1 and *k / *m / *c when the form exists, 0 when it does not (including res_shift other
+ *             than 0 or -1, and res_mult below 2^30), ISC_ERR_ARG for a null pointer.
+ */
+int isc_debug_residual_product(int32_t res_mult, int32_t res_shift, int32_t zp_res, int32_t *k, float *m, int32_t *c);
+
+/*
+ * isc_debug_residual_form -- host only.  The same search for the integer form
+ * floor((256 k + u) * m2 / 2^32) - c, m2 = res_mult * 2^(1 + res_shift), which no kernel computes: it
+ * exists for other multipliers than the product does.
  *   returns : 1 and *k / *c when the integer form exists, 0 when it does not
  *             (including res_shift other than 0 or -1), ISC_ERR_ARG for a null pointer.
  */

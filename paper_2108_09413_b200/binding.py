@@ -11,7 +11,7 @@ _LIB_PATH = os.path.join(_HERE, "libisc.so")
 
 EXPORTS = ["isc_load_qmodel", "isc_free_qmodel", "isc_plan_resident", "isc_predict", "isc_certify", "isc_certify_batch",
            "isc_sample_counts", "isc_sample_counts_static", "isc_decide_certify", "isc_decide_predict", "isc_certify_integer", "isc_decide_certify_integer", "isc_noise_table", "isc_noise_table_rounded", "isc_radius_integer", "isc_certified_metrics",
-           "isc_debug_tensor", "isc_debug_wait_timeout", "isc_debug_stalled_launch", "isc_debug_residual_form", "isc_set_option", "isc_get_info", "isc_strerror"]
+           "isc_debug_tensor", "isc_debug_wait_timeout", "isc_debug_stalled_launch", "isc_debug_residual_product", "isc_debug_residual_form", "isc_set_option", "isc_get_info", "isc_strerror"]
 
 
 class IscError(RuntimeError):
@@ -68,6 +68,7 @@ def lib():
                                        C.c_int, vp, vp, C.c_int64]
         L.isc_debug_wait_timeout.argtypes = [vp, C.c_int64, vp, vp]
         L.isc_debug_stalled_launch.argtypes = [vp, C.c_int, vp, vp]
+        L.isc_debug_residual_product.argtypes = [C.c_int32, C.c_int32, C.c_int32, vp, vp, vp]
         L.isc_debug_residual_form.argtypes = [C.c_int32, C.c_int32, C.c_int32, vp, vp]
         L.isc_set_option.argtypes = [vp, C.c_char_p, C.c_int64]
         L.isc_get_info.argtypes = [vp, C.c_char_p, C.POINTER(C.c_int64)]
@@ -293,8 +294,18 @@ def radius_integer(sigma, p_fx):
     return q.value, q2.value
 
 
+def residual_product(res_mult, res_shift, zp_res):
+    """(k, m, c) of isc_debug_residual_product, the form of the residual rescale that the engines compute, or None where it
+    does not exist; host only."""
+    k, m, c = C.c_int32(), C.c_float(), C.c_int32()
+    rc = lib().isc_debug_residual_product(int(res_mult), int(res_shift), int(zp_res), C.byref(k), C.byref(m), C.byref(c))
+    if rc < 0:
+        raise IscError(rc, "isc_debug_residual_product")
+    return (k.value, m.value, c.value) if rc == 1 else None
+
+
 def residual_form(res_mult, res_shift, zp_res):
-    """(k, c) of isc_debug_residual_form when the short form of the residual rescale exists, else None; host only."""
+    """(k, c) of isc_debug_residual_form when the integer short form of the residual rescale exists, else None; host only."""
     k, c = C.c_int32(), C.c_int32()
     rc = lib().isc_debug_residual_form(int(res_mult), int(res_shift), int(zp_res), C.byref(k), C.byref(c))
     if rc < 0:

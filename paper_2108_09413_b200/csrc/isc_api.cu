@@ -1135,15 +1135,41 @@ int isc_debug_tensor(isc_model *m, const uint8_t *x_u8, uint64_t seed, uint64_t 
     return ISC_OK;
 }
 
+int isc_debug_residual_product(int32_t res_mult, int32_t res_shift, int32_t zp_res, int32_t *k, float *m, int32_t *c)
+{
+    if (!k || !m || !c) return ISC_ERR_ARG;
+    int32_t cc = 0;
+    const isc::ResidualForm f = isc::residual_form(res_mult, res_shift, zp_res, &cc);
+    if (!f.exists()) return 0;
+    *k = (int32_t)(f.k8 >> 8);
+    memcpy(m, &f.m_bits, sizeof(*m));
+    *c = cc;
+    return 1;
+}
+
 int isc_debug_residual_form(int32_t res_mult, int32_t res_shift, int32_t zp_res, int32_t *k, int32_t *c)
 {
     if (!k || !c) return ISC_ERR_ARG;
-    uint32_t k8 = 0;
-    int32_t cc = 0;
-    if (!isc::residual_short_form(res_mult, res_shift, zp_res, &k8, &cc)) return 0;
-    *k = (int32_t)(k8 >> 8);
-    *c = cc;
-    return 1;
+    const int n = 31 - res_shift;
+    if ((n != 31 && n != 32) || res_mult <= 0) return 0;
+    const uint64_t m2 = (uint64_t)(uint32_t)res_mult << (32 - n);
+    if (m2 >= (1ull << 32)) return 0;
+    const int64_t r2 = ((1ll << (n - 1)) - (128ll + zp_res) * (int64_t)res_mult) * (1ll << (32 - n));
+    for (uint32_t off = 0; off < 4096; ++off) {
+        int64_t first = 0;
+        bool same = true;
+        for (uint32_t u = 0; u < 256 && same; ++u) {
+            const int64_t want = ((int64_t)(u * m2) + r2) >> 32;                 // arithmetic shift: floor
+            const int64_t got = (int64_t)(((uint64_t)(256u * off + u) * m2) >> 32);
+            if (u == 0) first = got - want;
+            same = got - want == first;
+        }
+        if (!same) continue;
+        *k = (int32_t)off;
+        *c = (int32_t)first;
+        return 1;
+    }
+    return 0;
 }
 
 int isc_debug_wait_timeout(isc_model *m, int64_t limit_ns, void *cuda_stream, int32_t *out4)

@@ -899,28 +899,6 @@ bool conv_offsets_fit(const GLayer &G, int64_t batch)
 
 // The residual term F(u) = floor((u * m2 + R2) / 2^32), u = r + 128 in 0..255 (see requant16_fast), as
 // hi32((256 k + u) * m2) - c: the smallest k < 4096 for which the two agree on all 256 inputs, or false.
-bool residual_short_form(int res_mult, int res_shift, int zp_res, uint32_t *k8, int32_t *c_out)
-{
-    const int n = 31 - res_shift;
-    if (n != 31 && n != 32) return false;
-    if (res_mult <= 0) return false;
-    const uint64_t m2 = (uint64_t)(uint32_t)res_mult << (32 - n);
-    if (m2 >= (1ull << 32)) return false;
-    const int64_t r2 = ((1ll << (n - 1)) - (128ll + zp_res) * (int64_t)res_mult) * (1ll << (32 - n));
-    for (uint32_t k = 0; k < 4096; ++k) {
-        int64_t c = 0;
-        bool same = true;
-        for (uint32_t u = 0; u < 256 && same; ++u) {
-            const int64_t want = ((int64_t)(u * m2) + r2) >> 32;                 // arithmetic shift: floor
-            const int64_t got = (int64_t)(((uint64_t)(256u * k + u) * m2) >> 32);
-            if (u == 0) c = got - want;
-            same = got - want == c;
-        }
-        if (same) { *k8 = k << 8; *c_out = (int32_t)c; return true; }
-    }
-    return false;
-}
-
 ResidualForm residual_form(int res_mult, int res_shift, int zp_res, int32_t *c_out)
 {
     ResidualForm f;

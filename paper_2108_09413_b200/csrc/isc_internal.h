@@ -107,12 +107,10 @@ int igemm_padded_cout(const GLayer &G);          // output channels with the las
 bool conv_offsets_fit(const GLayer &G, int64_t batch);  // the batch's tensors are within the tensor-core kernels' 32-bit offsets
 size_t igemm_pack_bytes(const GLayer &G);
 void igemm_pack_weights(const GLayer &G, const int8_t *w_oihw, int8_t *out);
-// The residual term F(u) = floor((u * m2 + R2) / 2^32), u = r + 128 in 0..255, of the 32-bit epilogues as
-// floor((256 k + u) * m2 / 2^32) - c: the smallest k < 4096 for which the two agree on all 256 inputs (*k8 = 256 k), or false.
-bool residual_short_form(int res_mult, int res_shift, int zp_res, uint32_t *k8, int32_t *c);
-// The same term as a single-precision product, round((256 k + u) * m) - c, with round to nearest even and m one of the
-// three single-precision numbers nearest to the multiplier: what the kernels compute where it exists (for more than 99 %
-// of all multipliers), the 64-bit form otherwise.
+// The residual term floor((u * m2 + R2) / 2^32), u = r + 128 in 0..255, of the 32-bit epilogues as a single-precision product,
+// round((256 k + u) * m) - c, with round to nearest even and m one of the three single-precision numbers nearest to the
+// multiplier: the smallest k < 4096 for which the two agree on all 256 inputs.  What the kernels compute where it exists (for
+// more than 99 % of all multipliers), the 64-bit form otherwise.
 struct ResidualForm {
     uint32_t k8 = 0xFFFFFFFFu, m_bits = 0;       // 256 k; m as stored
     bool exists() const { return k8 != 0xFFFFFFFFu; }

@@ -1,6 +1,7 @@
 """1 x 1 layers in tiles of 256 pixels x 128 channels, against the plain kernels: pixel counts that end in the first or in
-the second half of a tile, one or several tiles of channels, with and without a residual operand (both forms of its
-term), lower clamps at and above -128, and batches on either side of the rule that pairs tiles."""
+the second half of a tile, one or several tiles of channels, with and without a residual operand (its term as a product;
+the 64-bit term is in test_gpu_requant_range.py), lower clamps at and above -128, and batches on either side of the rule that
+pairs tiles."""
 import numpy as np
 import pytest
 

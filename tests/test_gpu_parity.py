@@ -204,13 +204,14 @@ def test_random_bottleneck_nets_on_the_tensor_core_engine(seed):
     _bottleneck_parity(_bottleneck_net(rng), rng, seed, tensor_copy=seed & 1)      # both ways of bringing 1 x 1 operand rows
 
 
-@pytest.mark.parametrize("res", [(1304428746, 0, 77), (1334892440, -1, -63), (1 << 30, 0, 0),         # no offset form
-                                 (1979951843, 0, 0), (1435772024, -1, -128)])                           # offset form
+@pytest.mark.parametrize("res", [(1304428746, 0, 77), (1342155344, 0, 7), (1817091736, -1, 77), (1090259607, -1, -63),         # 64-bit term
+                                 (1334892440, -1, -63), (1 << 30, 0, 0), (1979951843, 0, 0), (1435772024, -1, -128)])           # product
 def test_bottleneck_nets_32_bit_epilogue_both_residual_forms(res):
     """The same networks with every shift >= 2, so that the kernel's 32-bit epilogue runs, and residual rescales
-    with and without the offset form (isc_debug_residual_form): both forms of the residual term against the oracle."""
-    has_form = isc.residual_form(*res) is not None
-    assert has_form == (res[0] in (1979951843, 1435772024))
+    with and without the form of a single-precision product (isc_debug_residual_product): both forms of the residual term
+    against the oracle."""
+    has_form = isc.residual_product(*res) is not None
+    assert has_form == (res[0] in (1334892440, 1 << 30, 1979951843, 1435772024))
     rng = np.random.default_rng(950 + res[0] % 97)
     _bottleneck_parity(_bottleneck_net(rng, fast=res), rng, res[0] % 5, tensor_copy=res[0] % 2)
 

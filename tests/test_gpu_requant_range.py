@@ -1,5 +1,5 @@
 """Requantisation at the ends of its range: rounding addends whose sum with the product's high word needs more than 32 bits,
-with accumulators of both signs.  Every tensor of one sample and the logits of a batch equal the CPU oracle's, or the
+with accumulators of both signs; and the residual term in each of its forms, in every kernel.  Every tensor of one sample and the logits of a batch equal the CPU oracle's, or the
 plain kernels'."""
 import numpy as np
 import pytest
@@ -84,4 +84,33 @@ def test_residual_constants_of_the_resident_engine(res_mult, zp_res, zp_out, shi
     layers = [_conv(rng, 0, 3, 16, 3, 1, 1, 3, -128), _conv(rng, 1, 16, 32, 3, 2, 0, -128, zp_res), _conv(rng, 2, 32, 32, 3, 1, 1, zp_res, -128),
               _wide(rng, 3, 32, 32, 3, 1, 0, -128, zp_out, res=2, zp_res=zp_res, shift=shift)]
     layers[3].update(res_mult=res_mult, res_shift=0)
+    _check(rng, (3, 32, 32), layers, 3, 700, 256)
+
+
+FORMS = [(1304428746, 0, 77), (1342155344, 0, 7), (1817091736, -1, 77), (1090259607, -1, -63),        # no product: the 64-bit term
+         (1334892440, -1, -63), (2032202290, 0, 7), (1 << 30, 0, -128), (1435772024, -1, -128)]      # product
+
+
+# resident-tile filter, whole tiles, paired tiles, the general form; paired tiles need enough of them for every SM
+@pytest.mark.parametrize("cin,cout,k", [(32, 48, 3), (256, 64, 1), (64, 256, 1), (48, 40, 1)])
+@pytest.mark.parametrize("res", FORMS)
+@pytest.mark.parametrize("relu", [0, 1])
+def test_both_forms_of_the_residual_term(cin, cout, k, res, relu):
+    assert (isc.residual_product(*res) is None) == (FORMS.index(res) < 4)
+    rng = np.random.default_rng(res[0] % 1000 + cin)
+    layers = [_conv(rng, 0, 3, cin, 3, 1, 1, 3, -128), _conv(rng, 1, cin, cout, 1, 1, 0, -128, res[2]),
+              _conv(rng, 1, cin, cout, k, 1, relu, -128, res[2], res=2, zp_res=res[2])]
+    layers[2].update(res_mult=res[0], res_shift=res[1])
+    _check(rng, (3, 12, 8), layers, 2, 700, 96)
+
+
+@pytest.mark.parametrize("res", FORMS)
+@pytest.mark.parametrize("relu", [0, 1])
+def test_both_forms_on_the_resident_engine(res, relu):
+    rng = np.random.default_rng(res[0] % 1000)
+    layers = [_conv(rng, 0, 3, 16, 3, 1, 1, 3, res[2]), _conv(rng, 1, 16, 16, 3, 1, 1, res[2], -128),
+              _conv(rng, 2, 16, 16, 3, 1, relu, -128, res[2], res=1, zp_res=res[2]), _conv(rng, 3, 16, 32, 3, 2, 1, res[2], res[2]),
+              _conv(rng, 4, 32, 32, 3, 1, 1, res[2], -128), _conv(rng, 5, 32, 32, 3, 1, relu, -128, res[2], res=4, zp_res=res[2])]
+    for layer in layers:
+        layer.update(res_mult=res[0], res_shift=res[1])
     _check(rng, (3, 32, 32), layers, 3, 700, 256)

@@ -190,8 +190,8 @@ def test_rounded_noise_table_equals_the_oracle():
 
 
 def test_residual_short_form_reproduces_the_rescale_on_every_byte():
-    """The offset form of the residual rescale, floor((256 k + u) m2 / 2^32) - c, is used by the tensor-core engines only
-    when it equals rs((r - zp_res) * res_mult, 31 - res_shift) for all 256 bytes: checked here with exact integers."""
+    """The integer offset form of the residual rescale, floor((256 k + u) m2 / 2^32) - c, is reported only when it equals
+    rs((r - zp_res) * res_mult, 31 - res_shift) for all 256 bytes: checked here with exact integers."""
     rng = np.random.default_rng(0x15174000)
     found = 0
     cases = [(1 << 30, 0, 0), (1 << 30, -1, -128), ((1 << 31) - 1, 0, 127), ((1 << 31) - 1, -1, -128)]
@@ -210,3 +210,35 @@ def test_residual_short_form_reproduces_the_rescale_on_every_byte():
             assert (((256 * k + r + 128) * m2) >> 32) - c == want, (res_mult, res_shift, zp_res, r)
     assert found >= 50                                                        # the form exists for nearly every multiplier
     assert isc.residual_form(1 << 30, -3, 0) is None                         # rescale shifts the engines do not take
+
+
+def test_residual_product_reproduces_the_rescale_on_every_byte():
+    """The form that the tensor-core engines compute, round((256 k + u) m) - c with a single-precision m, to nearest even:
+    equal to rs((r - zp_res) * res_mult, 31 - res_shift) for all 256 bytes, checked here with exact integers."""
+    rng = np.random.default_rng(0x15174001)
+    found, missing = 0, 0
+    cases = [(1 << 30, 0, 0), (1 << 30, -1, -128), ((1 << 31) - 1, 0, 127), ((1 << 31) - 1, -1, -128), (2032202290, 0, 7), (1334892440, -1, -63)]
+    without = [(1304428746, 0, 77), (1342155344, 0, 7), (1817091736, -1, 77), (1090259607, -1, -63)]
+    cases += [(int(rng.integers(1 << 30, 1 << 31)), int(rng.integers(-1, 1)), int(rng.integers(-128, 128))) for _ in range(200)]
+    for res_mult, res_shift, zp_res in cases + without:
+        form = isc.residual_product(res_mult, res_shift, zp_res)
+        if form is None:
+            missing += 1
+            continue
+        found += 1
+        k, m, c = form
+        assert 0 <= k < 4096 and 256 * k + 255 < 2 ** 23                    # the kernels read 256 k + u as a denormal number
+        mant, e = int(m * 2 ** 32), 32                                      # exact: 24 bits, at least 2^-2
+        assert mant == m * 2 ** 32 and np.float32(m) == m
+        n = 31 - res_shift
+        for r in range(-128, 128):
+            want = ((r - zp_res) * res_mult + (1 << (n - 1))) >> n          # rs(): round half up, floor division
+            x = (256 * k + r + 128) * mant
+            q, rest, half = x >> e, x & ((1 << e) - 1), 1 << (e - 1)
+            got = q + (rest > half or (rest == half and q & 1))             # to nearest, ties to even
+            assert got - c == want, (res_mult, res_shift, zp_res, r)
+    assert all(isc.residual_product(*case) is None for case in without)
+    assert found >= 200 and missing <= 10                                   # the form exists for nearly every multiplier
+    assert all(isc.residual_product(m, s, -128) is not None for m in (1 << 30, 1304428746, (1 << 31) - 1) for s in (0, -1))
+    assert isc.residual_product(1 << 30, -3, 0) is None                     # rescale shifts the engines do not take
+    assert isc.lib().isc_debug_residual_product(1 << 30, 0, 0, None, None, None) == -1
