@@ -81,7 +81,7 @@ constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // 2 s per wait
 
 enum { PH_FILL = 0, PH_INPUT = 1, PH_CONV = 2, PH_TAIL = 3 };
 enum { ERR_NONE = 0, ERR_WAIT_DONE = 1, ERR_WAIT_WEIGHTS = 2, ERR_WAIT_READY = 3, ERR_WAIT_FULL = 4, ERR_WAIT_DRAIN = 5 };
-enum { CF_PAIRED = 1, CF_RES = 2, CF_SCATTER = 8, CF_GENERAL = 16 };         // CF_PAIRED: chains over two lines; CF_GENERAL: the pass that decides everything at run time
+enum { CF_PAIRED = 1, CF_RES = 2, CF_RES_LONG = 4, CF_SCATTER = 8, CF_GENERAL = 16 };         // CF_PAIRED: chains over two lines; CF_RES_LONG: the residual term is no product; CF_GENERAL: the pass that decides everything at run time
 // OPF_WAIT_ALL: every unit of the previous convolution; OPF_WAITS / OPF_WAITS4: the record names counters to test (two /
 // four slots in use); bits 4-6: how many of them are distinct; bits 8-9: arrivals; bits 10-12: MMA chains
 enum { OPF_WAIT_ALL = 1, OPF_WAITS = 2, OPF_WAITS4 = 8 };
@@ -535,15 +535,22 @@ struct alignas(16) LPass {
 static_assert(sizeof(LPass) == 32, "one pass is two 16-byte loads");
 
 // Four outputs of one position.
-//   kResidual: y += round((256 k + u) * m) - c_r with u = r + 128 the residual byte as an unsigned number, for an offset k
+//   kRes = 1: y += floor((u * m2 + r2) / 2^32), the residual term of the general form.
+//   kRes = 2: y += round((256 k + u) * m) - c_r with u = r + 128 the residual byte as an unsigned number, for an offset k
 //   and a multiplier m that the planner has checked on all 256 values of u (residual_form): rs((r - zp_res) * res_mult, n).
 //   `k8` holds 256 k, which the byte permute that extracts u merges into it; c_r is folded into the rounding addends.
-template <bool kResidual>
-__device__ __forceinline__ uint32_t requant4(int a0, int a1, int a2, int a3, const ChanConsts &k, uint32_t rword, uint32_t m2, uint32_t k8)
+template <int kRes>
+__device__ __forceinline__ uint32_t requant4(int a0, int a1, int a2, int a3, const ChanConsts &k, uint32_t rword, uint32_t m2, uint32_t k8, long long r2)
 {
     int y0 = mad_hi(a0, k.mult[0], k.c[0]) >> k.s[0], y1 = mad_hi(a1, k.mult[1], k.c[1]) >> k.s[1];
     int y2 = mad_hi(a2, k.mult[2], k.c[2]) >> k.s[2], y3 = mad_hi(a3, k.mult[3], k.c[3]) >> k.s[3];
-    if (kResidual) {
+    if (kRes == 1) {
+        y0 += hi32(mad_wide_u(__byte_perm(rword, 0u, 0x4440u), m2, r2));
+        y1 += hi32(mad_wide_u(__byte_perm(rword, 0u, 0x4441u), m2, r2));
+        y2 += hi32(mad_wide_u(__byte_perm(rword, 0u, 0x4442u), m2, r2));
+        y3 += hi32(mad_wide_u(__byte_perm(rword, 0u, 0x4443u), m2, r2));
+    }
+    if (kRes == 2) {
         y0 += mul_denormal(__byte_perm(rword, k8, 0x7650u), m2);
         y1 += mul_denormal(__byte_perm(rword, k8, 0x7651u), m2);
         y2 += mul_denormal(__byte_perm(rword, k8, 0x7652u), m2);
@@ -583,7 +590,7 @@ __device__ __forceinline__ uint32_t scatter_to(const Scatter &g, uint32_t pos, u
 // The items (unit, chunk) of a convolution that belong to this warp's set: one wait, one or two records of two lines each,
 // one arrival.  kScatter: stride 2, results go to the next geometry (2.1 instead of 4.0 us a convolution of the first
 // transition when that was a pass of run-time decisions, line by line).
-template <bool kResidual, bool kScatter>
+template <int kRes, bool kScatter>
 __device__ __forceinline__ bool epi_conv_fast(Waiter w, uint32_t tmem_lane, uint32_t warp, uint32_t lane, uint32_t desc, uint4 h0, uint4 h1, uint4 h2, uint4 h3, uint32_t use)
 {
     const uint32_t tmem0 = tmem_lane + h0.w, full = CTRL_ADDR(bars) + 8u * (h1.x + (use & 1u) * h2.x), done = CTRL_ADDR(stored) + 4u * h1.y;
@@ -591,6 +598,7 @@ __device__ __forceinline__ bool epi_conv_fast(Waiter w, uint32_t tmem_lane, uint
     const uint32_t out = the_base() + h2.w + (kScatter ? word * 4u : row0 * 16u + word * 4u), res = the_base() + h3.x + row0 * 16u + word * 4u;
     const uint32_t vecs = desc + lds32(desc + offsetof(LConvDesc, vec_rel));
     const uint32_t m2 = h3.y, k8 = h3.z, dup = h3.w;
+    const long long r2 = kRes == 1 ? (long long)(((unsigned long long)lds32(desc + offsetof(LConvDesc, res_r2_hi)) << 32) | k8) : 0ll;
     // The bands of a thread's rows: they differ in bits 3 and 4 of the position, of which a band number has bits 2 and 3 at
     // most.  Bit 0, 1: rows of even number have a band above, below; bit 2, 3: those of odd number.
     const uint32_t nb = lds32(desc + offsetof(LConvDesc, out_nb));
@@ -634,7 +642,7 @@ __device__ __forceinline__ bool epi_conv_fast(Waiter w, uint32_t tmem_lane, uint
                 const uint32_t to = out + (l ? q1.y : q1.x);
                 const uint32_t from = res + (l ? q1.w : q1.z) + (uint32_t)h * 256u;
                 uint32_t r0 = 0, r1 = 0;
-                if (kResidual) { r0 = lds32(from) ^ 0x80808080u; r1 = lds32(from + 128u) ^ 0x80808080u; }
+                if (kRes) { r0 = lds32(from) ^ 0x80808080u; r1 = lds32(from + 128u) ^ 0x80808080u; }
                 tmem_ld_frag_wait(v);
                 if (st < 3) tmem_ld_frag(tmem0 + (st == 0 ? q0.z + (16u << 16) : st == 1 ? q0.w : q0.w + (16u << 16)), acc[(st + 1) & 1]);
                 if (h == 1) tmem_st_columns(tmem0 + (l ? q0.w : q0.z), vecs + (l ? q0.x >> 26 : (q0.x >> 20) & 63u) * kVecBytes);
@@ -645,7 +653,7 @@ __device__ __forceinline__ bool epi_conv_fast(Waiter w, uint32_t tmem_lane, uint
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
                         if ((sc_odd >> j) & 1u) continue;
-                        const uint32_t o = requant4<false>(v[2 * j], v[2 * j + 1], v[2 * j + 4], v[2 * j + 5], k, 0u, 0u, 0u);
+                        const uint32_t o = requant4<0>(v[2 * j], v[2 * j + 1], v[2 * j + 4], v[2 * j + 5], k, 0u, 0u, 0u, 0ll);
                         const uint32_t col = (uint32_t)(16 * h + 8 * j) >> (((sc_log >> 8) & 0xFFu) + 1u) << (sc_log >> 16);
                         const uint32_t at = to + (oline * sc_pitch + sc_at + col + (oband << 2)) * 16u;
                         st_shared_u32(at, o);
@@ -655,9 +663,9 @@ __device__ __forceinline__ bool epi_conv_fast(Waiter w, uint32_t tmem_lane, uint
                         }
                     }
                 } else {
-                    const uint32_t o0 = requant4<kResidual>(v[0], v[1], v[4], v[5], k, r0, m2, k8), at = to + (uint32_t)h * 256u;
+                    const uint32_t o0 = requant4<kRes>(v[0], v[1], v[4], v[5], k, r0, m2, k8, r2), at = to + (uint32_t)h * 256u;
                     st_shared_u32(at, o0);
-                    const uint32_t o1 = requant4<kResidual>(v[2], v[3], v[6], v[7], k, r1, m2, k8);
+                    const uint32_t o1 = requant4<kRes>(v[2], v[3], v[6], v[7], k, r1, m2, k8, r2);
                     st_shared_u32(at + 128u, o1);
                     const uint32_t edges = (q0.x >> (16 + 2 * l)) & 3u;
                     if (dup && edges) {
@@ -955,6 +963,7 @@ struct RoleState {
     int next_copy = 0;
 };
 
+template <bool kLong>
 __device__ __forceinline__ void epilogue_run(const LineParams &p, uint32_t tmem, uint32_t warp, uint32_t lane, int ph, int stop, int it, RoleState &r)
 {
     const Waiter w{p.err};
@@ -967,9 +976,10 @@ __device__ __forceinline__ void epilogue_run(const LineParams &p, uint32_t tmem,
         const uint4 h0 = ld_shared_v4(desc), h1 = ld_shared_v4(desc + 16u), h2 = ld_shared_v4(desc + 32u), h3 = ld_shared_v4(desc + 48u);
         const uint32_t use = (uint32_t)it * h1.w + h1.z;
         if (h0.x & CF_GENERAL) r.ok = epi_conv_general(w, tmem_lane, warp, lane, desc, h0, h1, h2, h3, use);
-        else if (h0.x & CF_SCATTER) r.ok = epi_conv_fast<false, true>(w, tmem_lane, warp, lane, desc, h0, h1, h2, h3, use);
-        else if (h0.x & CF_RES) r.ok = epi_conv_fast<true, false>(w, tmem_lane, warp, lane, desc, h0, h1, h2, h3, use);
-        else r.ok = epi_conv_fast<false, false>(w, tmem_lane, warp, lane, desc, h0, h1, h2, h3, use);
+        else if (h0.x & CF_SCATTER) r.ok = epi_conv_fast<0, true>(w, tmem_lane, warp, lane, desc, h0, h1, h2, h3, use);
+        else if (kLong && (h0.x & CF_RES_LONG)) r.ok = epi_conv_fast<1, false>(w, tmem_lane, warp, lane, desc, h0, h1, h2, h3, use);
+        else if (h0.x & CF_RES) r.ok = epi_conv_fast<2, false>(w, tmem_lane, warp, lane, desc, h0, h1, h2, h3, use);
+        else r.ok = epi_conv_fast<0, false>(w, tmem_lane, warp, lane, desc, h0, h1, h2, h3, use);
     }
 }
 
@@ -985,6 +995,9 @@ __device__ __forceinline__ void loader_run(const LineParams &p, int ph, int stop
         if (r.ok && !Waiter::aborted()) r.ok = loader_copy(p, r.next_copy, r.ws.slot, it);
 }
 
+// kLong: the network has convolutions whose residual term is no product.  A kernel of its own: as a fourth pass beside the other
+// three, which no ResNet's usual multipliers reach, it cost every network 0.7 % (ResNet-110 at 100,100 samples 62.0 -> 62.5 ms).
+template <bool kLong>
 __global__ void __launch_bounds__(kThreads, 1) k_line(const __grid_constant__ LineParams p)
 {
     Ctrl *ctrl = the_ctrl();
@@ -1042,7 +1055,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_line(const __grid_constant__ Li
             }
             const int stop = min(end, ph + (int)e.z);
             if (warp < kEpiWarps) {
-                epilogue_run(p, tmem, warp, lane, ph, stop, it, r);
+                epilogue_run<kLong>(p, tmem, warp, lane, ph, stop, it, r);
             } else if (lane == 0) {
                 if (warp < kLoaderWarp) issuer_run(p, tmem, warp - kEpiWarps, ph, stop, it, r);
                 else loader_run(p, ph, stop, it, r);
@@ -1189,7 +1202,8 @@ struct LinePlan {
     unsigned long long *d_phase_cycles = nullptr;
     uint8_t *d_dump = nullptr;
     int sm_count = 0;
-    int attr_device = -1;                // the device on which k_line's shared-memory limit has been raised
+    bool long_residual = false;          // a convolution needs k_line<true>
+    int attr_device = -1;                // the device on which the kernel's shared-memory limit has been raised
     // launches smaller than the GPU (see line_run)
     cudaStream_t side[kSideStreams] = {};
     int side_priority = 0, side_device = 0;
@@ -1474,19 +1488,18 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
         // counter) covers `upl` lines = one or two records.  Long convolutions take four-line units: every barrier
         // arrival costs an issuing thread a tcgen05.commit and every unit costs an epilogue warp a wait and an arrival.
         const int sup = cp.m >= 2 ? 2 : 1;
-        // the fast pass covers pairs of lines with the saturating pack as the only clamp, and a residual term that is a
-        // single-precision product whose constant fits into every channel's rounding addend
+        // The fast pass covers pairs of lines with the saturating pack as the only clamp.  The residual term is a single-precision
+        // product where that exists and its constant fits into every channel's rounding addend, else the general form's.
         bool general = (cp.m & 1) || (L.relu && L.zp_out > -128);
         for (int oc = 0; oc < L.cout; ++oc) general = general || layers[cp.layer].shift[oc] == 1;
         if (!general && L.res_tensor >= 0) {
             cp.res_form = residual_form(L.res_mult, L.res_shift, L.zp_res, &cp.res_c);
-            general = !cp.res_form.exists();
-            for (int oc = 0; oc < L.cout && !general; ++oc) {
+            bool fits = cp.res_form.exists();
+            for (int oc = 0; oc < L.cout && fits; ++oc) {
                 const int sft = layers[cp.layer].shift[oc] - 1;
-                const long long add = sft >= 1 ? (1ll << (sft - 1)) + ((long long)L.zp_out - cp.res_c) * (1ll << sft) : (1ll << 40);
-                general = !requant_addend_fits(add);
+                fits = sft >= 1 && requant_addend_fits((1ll << (sft - 1)) + ((long long)L.zp_out - cp.res_c) * (1ll << sft));
             }
-            if (general) cp.res_c = 0;
+            if (!fits) { cp.res_form = ResidualForm(); cp.res_c = 0; }
         }
         cp.general = general;
         const int upl = (!general && cp.m >= 16 && cp.m % 4 == 0) ? 4 : sup;
@@ -1763,7 +1776,8 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
         std::vector<uint8_t> blob(w_bytes[(size_t)c], 0);
         LConvDesc D;
         memset(&D, 0, sizeof(D));
-        D.flags = (L.res_tensor >= 0 ? CF_RES : 0u) | (cp.scatter ? CF_SCATTER : 0u) | (cp.general ? CF_GENERAL : 0u) | (cp.paired ? CF_PAIRED : 0u);
+        plan->long_residual |= L.res_tensor >= 0 && !cp.general && !cp.res_form.exists();
+        D.flags = (L.res_tensor >= 0 ? CF_RES : 0u) | (cp.scatter ? CF_SCATTER : 0u) | (cp.general ? CF_GENERAL : 0u) | (L.res_tensor >= 0 && !cp.res_form.exists() ? CF_RES_LONG : 0u) | (cp.paired ? CF_PAIRED : 0u);
         D.n_items = (uint32_t)(cp.n_units * cp.n_chunks); D.recs_per_item = (uint32_t)cp.recs_per_item; D.d_base = (uint32_t)bank_base(c);
         D.bar_full = (uint32_t)class_full[(size_t)cp.cls]; D.bar_done = (uint32_t)class_done[(size_t)cp.cls];
         D.use_local = (uint32_t)cp.use_local; D.uses_per_group = (uint32_t)class_uses[(size_t)cp.cls];
@@ -1790,8 +1804,8 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
             D.gen_res_m2 = (uint32_t)m2;
             D.res_r2_lo = (uint32_t)((unsigned long long)r2 & 0xFFFFFFFFull);
             D.res_r2_hi = (uint32_t)((unsigned long long)r2 >> 32);
-            D.res_m2 = cp.res_form.m_bits;
-            D.res_k8 = cp.res_form.k8;
+            D.res_m2 = cp.res_form.exists() ? cp.res_form.m_bits : (uint32_t)m2;
+            D.res_k8 = cp.res_form.exists() ? cp.res_form.k8 : D.res_r2_lo;
         }
         for (size_t k = 0; k < cp.kunits.size(); ++k) {
             const long long a = (long long)a_base + cp.a_delta[k];
@@ -2075,15 +2089,16 @@ static int line_join(LinePlan *p, cudaStream_t st)
 
 static int line_launch(LinePlan *p, LineParams &q, cudaStream_t st)
 {
+    const auto kernel = p->long_residual ? k_line<true> : k_line<false>;
     int device = -1;
     bool ok = cudaGetDevice(&device) == cudaSuccess;
     if (ok && device != p->attr_device) {
-        ok = cudaFuncSetAttribute(k_line, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) == cudaSuccess;
+        ok = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) == cudaSuccess;
         if (ok) p->attr_device = device;
     }
     if (!ok) { cudaGetLastError(); return ISC_ERR_CUDA; }
     const int grid = std::max(1, std::min(q.n_groups, p->sm_count));
-    k_line<<<grid, kThreads, p->smem_bytes, st>>>(q);
+    kernel<<<grid, kThreads, p->smem_bytes, st>>>(q);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess && getenv("ISC_PLAN_DEBUG")) fprintf(stderr, "line engine: launch failed: %s\n", cudaGetErrorString(e));
     return e == cudaSuccess ? ISC_OK : ISC_ERR_CUDA;

@@ -315,8 +315,7 @@ def resident_plans_order_rows_of_other_bands():
     def record(at, count, dtype=np.uint32):
         return np.frombuffer(C.string_at(int(at), count * np.dtype(dtype).itemsize), dtype)
 
-    def wait_for_all(layers, side):
-        """per convolution: whether each issuing thread's first record waits for all of the convolution before"""
+    def blobs(layers, side):
         n, c = len(layers), layers[-1]["cout"]
         layers = layers + [wl._gavgpool(n, c, side * side, -128), wl._conv(rng, n + 1, c, 5, 1, 1, 0, False, -128, 0, op=wl.OP_FC)]
         gm = isc.Model(dict(in_shape=(3, 32, 32), n_classes=5, layers=layers))
@@ -324,16 +323,20 @@ def resident_plans_order_rows_of_other_bands():
         f.fake_reset()
         gm.sample_counts(wl.images(1)[0], 1, 0, 1, 0, 9, 0.25)
         params = np.array([f.fake_launch_word(0, k) for k in range(5)], np.uint64)       # phase table, blobs' sources, counts, (barriers, phases), (convolutions, ..)
-        out = []
         for k in range(int(params[4] & 0xFFFFFFFF)):
-            blob = int(record(int(params[1]) + 32 * k, 1, np.uint64)[0])
+            yield int(record(int(params[1]) + 32 * k, 1, np.uint64)[0])
+
+    def wait_for_all(layers, side):
+        """per convolution: whether each issuing thread's first record waits for all of the convolution before"""
+        out = []
+        for blob in blobs(layers, side):
             n_ops, _, ops = record(blob + 112, 3)
             assert n_ops >= 3
             out.append([bool(record(blob + int(ops) + 32 * r + 30, 1, np.uint16)[0] & 1) for r in range(3)])
         assert all(len(set(w)) == 1 for w in out)
         return [w[0] for w in out]
 
-    conv = lambda t, cin, cout, k, stride=1, res=-1: wl._conv(rng, t, cin, cout, k, stride, k // 2, True, 3 if t == 0 else -128, -128)
+    conv = lambda t, cin, cout, k, stride=1, res=-1: wl._conv(rng, t, cin, cout, k, stride, k // 2, True, 3 if t == 0 else -128, -128, res, -128)
     stem = [conv(0, 3, 16, 3), conv(1, 16, 32, 3, 2)]                        # tensor 2: 32 x 16 x 16, in two bands
     # 1 x 1 in place over tensor 3; a filter on an older tensor than the last, over the last one's input
     assert wait_for_all(stem + [conv(2, 32, 32, 3), conv(3, 32, 32, 3), conv(4, 32, 32, 1, res=3), conv(5, 32, 32, 3)], 16)[3:] == [False, True, False]
@@ -342,6 +345,14 @@ def resident_plans_order_rows_of_other_bands():
     assert wait_for_all([conv(0, 3, 16, 3), conv(1, 16, 16, 3), conv(2, 16, 16, 1)], 32)[1:] == [False, False]
     # basic blocks need no such wait
     assert not any(wait_for_all(wl.resnet20()["layers"][:-2], 8))
+    # a residual term without the form of a product, or whose constant has no room beside the product, keeps the fast pass
+    for res_mult, zp, shift, flags in ((1304428746, 77, 9, 2 | 4), (1798879234, -20, 14, 2 | 4), (1798879234, -20, 9, 2), (1304428746, -128, 9, 2)):
+        layers = [conv(0, 3, 16, 3), conv(1, 16, 16, 3), conv(2, 16, 16, 3, res=1)]
+        for layer in layers:
+            layer.update(zp_in=3 if layer is layers[0] else zp, zp_out=zp, zp_res=zp, relu=0, shift=np.full(16, shift, np.int8))
+        layers[2].update(res_mult=res_mult, res_shift=0)
+        layers = layers + [dict(conv(3, 16, 32, 3, 2), zp_in=zp)]
+        assert [int(record(blob, 1)[0]) & (2 | 4 | 16) for blob in blobs(layers, 16)][2] == flags
 
 
 # ------------------------------------------------------------------ the tests
