@@ -53,6 +53,7 @@ constexpr int kMaxStages = 16;
 constexpr int kPairN = 128;                  // channels of a paired tile: two operands of 128 rows, two tiles in tensor memory
 constexpr int kStemEpi = 8, kStemThreads = 32 * (kStemEpi + 1);        // k_stem: two threads per tile row and the MMA warp; two CTAs per SM
 constexpr size_t kStemSmemPair = 108 * 1024, kStemSmemLimit = 220 * 1024;       // dynamic shared memory of k_stem: for two CTAs per SM; at most
+constexpr size_t kStemSmemOwn = 5248;        // its static shared memory and what the system takes of a CTA's
 constexpr int kRowTeams = 2, kRowWarps = 4 * kRowTeams;                // epilogue_rows: a team of four warps takes every other tile
 // Warps of k_igemm by role: epilogue, gather, and one each for MMAs and weights.  Whole tiles whose operands come by tensor copy
 // need no gather warps and have sixteen epilogue warps; beside four gather warps sixteen would leave a thread 80 registers,
@@ -1073,8 +1074,8 @@ struct StemConfig {
     size_t smem() const { return (size_t)w_bytes + pos_bytes + patch_bytes; }
 };
 
-// Bands of `rows` output rows, if two CTAs per SM and their noise tables fit then (one row: if one CTA does).
-bool stem_config(const GLayer &G, int in_c, int rows, StemConfig *c, size_t limit = 94 * 1024)
+// Bands of `rows` output rows, if two CTAs per SM and some noise tables fit then (one row: if one CTA does).
+bool stem_config(const GLayer &G, int in_c, int rows, StemConfig *c)
 {
     if (G.op != ISC_CONV2D || in_c > 4 || G.kw > 8 || G.kh > 8 || G.coutp % 16 != 0 || G.coutp > 256) return false;
     const bool second = G.kw > 4, whole = 4 % G.stride == 0;
@@ -1087,7 +1088,7 @@ bool stem_config(const GLayer &G, int in_c, int rows, StemConfig *c, size_t limi
     c->rows_class = (rows_in + G.stride - 1) / G.stride;
     const size_t plane_pos = (size_t)G.stride * c->rows_class * c->pitch + 2 * kTileM + 8;        // the last tile reads beyond the last row
     const size_t total = c->w_bytes + plane_pos * c->planes * 16 + patch;
-    if (total > (rows > 1 ? limit : 214 * (size_t)1024)) return false;
+    if (total > (rows > 1 ? 94 : 214) * (size_t)1024) return false;
     c->plane_pos = (uint32_t)plane_pos;
     c->pos_bytes = (uint32_t)(plane_pos * c->planes * 16);
     c->patch_bytes = (uint32_t)patch;
@@ -1103,21 +1104,31 @@ bool stem_config_any(const GLayer &G, int in_c, StemConfig *c)
     return false;
 }
 
-// Bands for `batch` samples on `ctas` CTAs: between 8 and 32 rows, such that the CTA with the most work has the least.  Long
-// bands draw fewer rows twice and have fewer barriers beside longer phases (some six input rows' worth each; 3 x 3 on
-// 32 x 32, 5,100 samples: 330 us in bands of 8 rows, 220 in one of 32), short ones share out more evenly.
-// A table of bins takes its room from the bands if some of eight rows or more remain.
-void stem_bands(const GLayer &G, int in_c, int64_t batch, int64_t ctas, size_t bins, StemConfig *c)
+// Where a launch finds its noise levels: the bins in shared memory, the guide and cumulative tables there, or those in global memory.
+enum class StemTables { kBins, kFront, kGlobal };
+
+// Bands of at most 32 rows and tables for `batch` samples on `ctas` CTAs, two per SM: such that the CTA with the most work has
+// the least.  An item costs its input rows and some six rows' worth of barriers and phases (3 x 3 on 32 x 32, 5,100 samples:
+// 330 us in bands of 8 rows, 220 in one of 32); short bands share out more evenly.  A row drawn by search costs 1.8 times one
+// drawn by bins with the tables in shared memory, whose copy costs the item too, and twice with them in global memory, or more
+// where the two CTAs' shared memory passes the split of 196 KB and leaves the L1 next to nothing.  So tables take their room from
+// the bands: 7 x 7 stride 2 on 224 x 224, 700 samples with sigma = 1 (41 KB of bins), took 1,404 us in bands of 8 rows with the
+// search in shared memory, 1,540 in bands of 11 without any table there, and takes 1,213 in bands of 6 with the bins; with
+// sigma = 4.6 (70 KB of tables, no bins) 2,330 us in bands of 11 and 1,787 in bands of 10.
+void stem_bands(const GLayer &G, int in_c, int64_t batch, int64_t ctas, size_t bins, size_t front, StemConfig *c, StemTables *tables)
 {
     int64_t best = INT64_MAX;
-    size_t limit = 94 * 1024;
-    StemConfig t;
-    if (bins && stem_config(G, in_c, 8, &t, kStemSmemPair - bins)) limit = kStemSmemPair - bins;
-    for (int bands = (G.hout + 31) / 32; bands <= (G.hout + 7) / 8; ++bands) {
-        const int rows = (G.hout + bands - 1) / bands;
-        if (rows < 8 || !stem_config(G, in_c, rows, &t, limit)) continue;
-        const int64_t cost = (batch * ((G.hout + rows - 1) / rows) + ctas - 1) / ctas * ((rows - 1) * G.stride + G.kh + 6);
-        if (cost < best) { best = cost; *c = t; }
+    for (int want = 32, last = 0; want >= 1; --want) {
+        const int bands = (G.hout + want - 1) / want, rows = (G.hout + bands - 1) / bands;
+        StemConfig t;
+        if (rows == last || !stem_config(G, in_c, rows, &t) || t.smem() > kStemSmemPair) continue;
+        last = rows;
+        StemTables at = StemTables::kGlobal;
+        int row = 2 * (t.smem() + kStemSmemOwn) <= 196 * 1024 ? 20 : 26, item = 60;
+        if (bins && t.smem() + bins <= kStemSmemPair) { at = StemTables::kBins; row = 10; }
+        else if (front && t.smem() + front <= kStemSmemPair) { at = StemTables::kFront; row = 18; item += (int)(front / 1024); }
+        const int64_t cost = (batch * bands + ctas - 1) / ctas * (((rows - 1) * G.stride + G.kh) * row + item);
+        if (cost < best) { best = cost; *c = t; *tables = at; }
     }
 }
 
@@ -1150,8 +1161,13 @@ cudaError_t launch_stem_conv(const TcDevice &dev, const GLayer &G, const int8_t 
     p.in_c = in_c;
     StemConfig c;
     if (!stem_config_any(G, in_c, &c)) return cudaErrorInvalidValue;
+    // the guide table has to follow the cumulative one
     const size_t bins = ns.bins && ns.guide ? (size_t)noise_bins_side(ns.bin_bits) * 16 : 0;
-    stem_bands(G, in_c, batch, 2ll * dev.n_sms, bins, &c);
+    const size_t front = ns.guide && ns.guide == ns.cum + (2 * ns.T + 1) ? ((size_t)(2 * ns.T + 1 + kNoiseGuide + 1) * 4 + 15) & ~(size_t)15 : 0;
+    StemTables tables = StemTables::kGlobal;
+    if (c.smem() <= kStemSmemPair) stem_bands(G, in_c, batch, 2ll * dev.n_sms, bins, front, &c, &tables);
+    else if (bins && c.smem() + bins <= kStemSmemLimit) tables = StemTables::kBins;
+    else if (front && c.smem() + front <= kStemSmemLimit) tables = StemTables::kFront;
     p.band_rows = c.band_rows;
     p.n_bands = (G.hout + p.band_rows - 1) / p.band_rows;
     p.pitch = c.pitch; p.rows_class = c.rows_class; p.planes = c.planes;
@@ -1168,19 +1184,17 @@ cudaError_t launch_stem_conv(const TcDevice &dev, const GLayer &G, const int8_t 
     p.out = out; p.err = err;
     p.debug_stall = debug_stall ? 1 : 0;
     size_t smem = c.smem();
-    // The noise tables go to shared memory when two CTAs per SM still fit and the guide table follows the cumulative one:
-    // the bins if there is room for them.
-    const size_t front_words = (size_t)(2 * ns.T + 1 + kNoiseGuide + 1), room = (smem <= kStemSmemPair ? kStemSmemPair : kStemSmemLimit) - smem;
-    p.tab_off = 0; p.tab_words = 0; p.bin_bits = 0;
-    if (bins && bins <= room) { p.tab_words = (int)(bins / 4); p.bin_bits = ns.bin_bits; }
-    else if (ns.guide == ns.cum + (2 * ns.T + 1) && front_words * 4 <= room) p.tab_words = (int)front_words;
-    if (p.tab_words) {
-        p.tab_off = (uint32_t)smem;
-        smem += ((size_t)p.tab_words * 4 + 15) & ~(size_t)15;
-    }
+    const size_t tab = tables == StemTables::kBins ? bins : tables == StemTables::kFront ? front : 0;
+    p.tab_off = tab ? (uint32_t)smem : 0;
+    p.tab_words = tables == StemTables::kFront ? 2 * ns.T + 1 + kNoiseGuide + 1 : (int)(tab / 4);
+    p.bin_bits = tables == StemTables::kBins ? ns.bin_bits : 0;
+    smem += tab;
     if (batch <= 0) return cudaSuccess;
     p.n_items = (uint32_t)p.n_bands * (uint32_t)batch;
-    const uint32_t ctas = (uint32_t)dev.n_sms * (smem <= kStemSmemPair ? 2u : 1u);
+    // A CTA takes one item after the other; where levels are searched in bands of many pixels, an item (7 x 7 stride 2 on
+    // 300 x 300, 700 samples with sigma = 1: 3,128 and 2,940 us; 32 x 32, 6,000 samples with sigma = 2: 482 and 509; equal with bins).
+    const bool search_long = !p.bin_bits && ((p.band_rows - 1) * G.stride + G.kh) * G.win >= 3000;
+    const uint32_t ctas = search_long ? p.n_items : (uint32_t)dev.n_sms * (smem <= kStemSmemPair ? 2u : 1u);
     return launch_chained(chained && dev.chained, k_stem, dim3(std::min(p.n_items, ctas)), kStemThreads, smem, st, p);
 }
 
