@@ -580,6 +580,8 @@ void halo_pack(const GLayer &G, const int8_t *w, int8_t *out)
     HaloConfig c;
     halo_config(G, &c);
     const int k = G.kh;
+    std::vector<int> channel((size_t)c.tiles_n * c.n_tile);
+    for (size_t col = 0; col < channel.size(); ++col) channel[col] = halo_channel(G, c, (int)col);
     size_t at = 0;
     for (int t = 0; t < c.tiles_n; ++t)
         for (int b = 0; b < c.n_blocks; ++b)
@@ -590,7 +592,7 @@ void halo_pack(const GLayer &G, const int8_t *w, int8_t *out)
                     const int plane = odd ? 2 * pair : 2 * pair + col, tap_x = odd ? 2 * s + col : s;
                     for (int n = 0; n < c.n_tile; ++n)
                         for (int e = 0; e < 16; ++e, ++at) {
-                            const int oc = halo_channel(G, c, t * c.n_tile + n), ci = plane * 16 + e;
+                            const int oc = channel[(size_t)(t * c.n_tile + n)], ci = plane * 16 + e;
                             out[at] = (tap_x < k && oc < G.cout && ci < G.cin) ? w[(((size_t)oc * G.cin + ci) * k + r) * k + tap_x] : (int8_t)0;
                         }
                 }
