@@ -16,10 +16,11 @@
 //     1 x 1 stride-1 layer it also brings the operand rows, one tensor copy (cp.async.bulk.tensor) per block, and
 //     the gather warps idle;
 //   * one thread issues two tcgen05.mma (kind::i8, K = 32) per stage and commits the stage back to the loaders;
-//     accumulators alternate between two column ranges, so a tile's reduction runs under the previous one's
-//     epilogue;
-//   * sixteen warps requantise (fixed-point multiplier, shift, zero-points, residual add, clamp), shared among the
-//     accumulators in flight (epilogue_whole); in the general form eight warps, one tile row per thread (epilogue_rows).
+//     accumulators take two column ranges of tensor memory in turn (four in whole tiles of 64 channels by tensor copy), so a
+//     tile's reduction runs under the previous ones' epilogue;
+//   * the others requantise (fixed-point multiplier, shift, zero-points, residual add, clamp): in whole tiles (channels in
+//     multiples of 64) as fragments (epilogue_whole), sixteen warps where the operands come by tensor copy and eight
+//     where they are gathered; in the general form eight, one tile row per thread (epilogue_rows).
 // 1 x 1 layers that expand the channels, which the epilogue bounds, take tiles of 256 pixels x 128 channels (kPair): a
 // thread then reads a channel's constants once for two operands.
 // Every wait is bounded; on expiry a role raises the CTA's abort flag and the error word, the others leave their
@@ -217,8 +218,9 @@ __device__ __forceinline__ bool epilogue_rows(const IgemmParams &p, const EpiCtx
 // make 64 contiguous bytes of a pixel), nothing passes through shared memory, and sixteen warps have registers enough.  (One row
 // per thread took a 16-byte constant per one or two outputs, a scratch row in shared memory both ways, and eight warps, two
 // per scheduler, which left its latency exposed: 64 -> 256 channels with a residual operand at 56 x 56, 512 samples: 280 us in all, now 253.)
-// n_acc accumulators are in flight.  Of the four warps of a quarter two take every other tile, and in it every other unit; with
-// four accumulators (64 columns) each takes every fourth tile.
+// n_acc accumulators are in flight.  A quarter's four warps (operands by tensor copy) share two: two take every other tile, and
+// in it every other unit; with four accumulators (64 columns) each takes every fourth tile.  Of a quarter's two warps
+// (gathered operands) each takes every other tile, all of it.
 // kMode 0: 64-bit requantisation (any shift), 1: 32-bit form, 2 / 3: 32-bit form with the residual add (3: its
 // single-precision form).  kClamp: the lower clamp is above -128.
 template <int kMode, bool kPair, bool kClamp, int kWarps>

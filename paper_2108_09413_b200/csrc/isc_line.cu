@@ -689,8 +689,8 @@ __device__ __forceinline__ bool epi_conv_fast(Waiter w, uint32_t tmem_lane, uint
     return true;
 }
 
-// The general pass: a lower clamp above -128, a shift of one, a residual term without the single-precision form, a lone
-// line; one line at a time, every property decided at run time.
+// The general pass: a lower clamp above -128, a shift of one, a lone line; one line at a time, every property decided at
+// run time.
 __device__ __forceinline__ bool epi_conv_general(Waiter w, uint32_t tmem_lane, uint32_t warp, uint32_t lane, uint32_t desc, uint4 h0, uint4 h1, uint4 h2, uint4 h3, uint32_t use)
 {
     const bool res = h0.x & CF_RES, scatter = h0.x & CF_SCATTER;

@@ -1,5 +1,5 @@
 """The first convolution on the tensor cores: filter widths on both sides of four pixels, strides that do and do not
-divide four, bands of one to eight rows, rows wider than a tile, 16 to 256 output channels, lower clamps and shifts of
+divide four, bands of one to 32 rows, rows wider than a tile, 16 to 256 output channels, lower clamps and shifts of
 every form.  The layer's output equals the CPU oracle's, a batch's logits the plain kernels'."""
 import numpy as np
 import pytest
