@@ -73,7 +73,15 @@ constexpr int kMaxBars = 128;
 constexpr int kMaxLines = 32;               // output lines of one convolution
 constexpr int kCtrlBytes = 10240;
 constexpr int kMaxConv = 128;
-constexpr int kOpChainTries[] = {2, 1};     // MMA chains of an operation at most; a record of two may name more units than it has room for
+// How a network is planned; the first way that succeeds is taken.  `chains`: MMA chains of an operation at most; a record of
+// several may name more units than it has room for.  The ways from the third on are for networks that keep three tensors of
+// 72 KB and have 6 KB left for blobs: a paired convolution's blob is 1.3 to 1.9 KB larger than an unpaired one's.  Packed:
+// tensors from the top, which leaves the room in one piece, and other places; a blob's header ends with its last K-step;
+// a strided convolution has the units, and may share the barriers, of a general one.
+struct PlanTry { int chains; bool paired, packed; };
+constexpr PlanTry kPlanTries[] = {{2, true, false}, {1, true, false}, {4, false, false}, {1, false, false}, {2, true, true}, {1, true, true}, {4, false, true}, {1, false, true}};
+constexpr int kPlanUsual = 2, kPackAttempts = 200;
+constexpr int kPlanRuleBars = 14, kPlanRuleRoom = 15;          // after another rule's refusal the ways from the third on are no help
 constexpr int kSmemLimit = 227 * 1024;
 constexpr int kTmemCols = 512;
 constexpr int kSideStreams = 8;             // concurrent launches when a launch does not fill the GPU
@@ -372,7 +380,8 @@ __device__ __forceinline__ void op_commit(const IssueCtx &ic, uint4 r1)
     }
 }
 
-template <int KS>
+// kChains: an operation is up to four chains over consecutive lines.
+template <int KS, bool kChains = false>
 __device__ __forceinline__ bool issue_ops(const Waiter &w, const IssueCtx &ic, const PrevConv &prev, uint32_t n_ksteps)
 {
     constexpr int NK = KS > 0 ? KS : 1;
@@ -400,6 +409,13 @@ __device__ __forceinline__ bool issue_ops(const Waiter &w, const IssueCtx &ic, c
         const uint32_t d = ic.d0 + r0.x;
         if (!(r1.w & (7u << 26))) {
             // a record that only carries this thread's arrivals on units it did not add to
+        } else if (kChains) {
+            const uint32_t n_chains = (r1.w >> 26) & 7u;
+            for (uint32_t c = 0; c < n_chains; ++c) {
+#pragma unroll
+                for (int k = 0; k < NK; ++k)
+                    mma_i8(d + c * ic.cols, ((uint64_t)ahi << 32) | (uint64_t)(alo[k] + r0.z + c * ic.pitch16), ((uint64_t)bhi << 32) | (uint64_t)(blo[k] + r0.w), r0.y);
+            }
         } else if (KS > 0) {
 #pragma unroll
             for (int k = 0; k < NK; ++k)
@@ -481,6 +497,7 @@ __device__ __forceinline__ bool loader_copy(const LineParams &p, int target, uin
 }
 
 // One convolution's share of an issuing warp, by its lane 0.  Returns false after a wait has expired.
+template <bool kRare>
 __device__ __forceinline__ bool issuer_conv(const LineParams &p, uint32_t tmem, uint32_t blob_off, WeightSlot ws, uint32_t issuer, int it, PrevConv &prev)
 {
     const Waiter w{p.err};
@@ -502,6 +519,7 @@ __device__ __forceinline__ bool issuer_conv(const LineParams &p, uint32_t tmem, 
     ic.cols = h3.w;
     bool ok;
     if (h0.x & CF_PAIRED) ok = issue_pairs(w, ic, prev);
+    else if (kRare && h2.y == 2u) ok = issue_ops<2, true>(w, ic, prev, 2);
     else switch (h2.y) {
     case 1: ok = issue_ops<1>(w, ic, prev, 1); break;
     case 3: ok = issue_ops<3>(w, ic, prev, 3); break;
@@ -963,7 +981,7 @@ struct RoleState {
     int next_copy = 0;
 };
 
-template <bool kLong>
+template <bool kRare>
 __device__ __forceinline__ void epilogue_run(const LineParams &p, uint32_t tmem, uint32_t warp, uint32_t lane, int ph, int stop, int it, RoleState &r)
 {
     const Waiter w{p.err};
@@ -977,16 +995,17 @@ __device__ __forceinline__ void epilogue_run(const LineParams &p, uint32_t tmem,
         const uint32_t use = (uint32_t)it * h1.w + h1.z;
         if (h0.x & CF_GENERAL) r.ok = epi_conv_general(w, tmem_lane, warp, lane, desc, h0, h1, h2, h3, use);
         else if (h0.x & CF_SCATTER) r.ok = epi_conv_fast<0, true>(w, tmem_lane, warp, lane, desc, h0, h1, h2, h3, use);
-        else if (kLong && (h0.x & CF_RES_LONG)) r.ok = epi_conv_fast<1, false>(w, tmem_lane, warp, lane, desc, h0, h1, h2, h3, use);
+        else if (kRare && (h0.x & CF_RES_LONG)) r.ok = epi_conv_fast<1, false>(w, tmem_lane, warp, lane, desc, h0, h1, h2, h3, use);
         else if (h0.x & CF_RES) r.ok = epi_conv_fast<2, false>(w, tmem_lane, warp, lane, desc, h0, h1, h2, h3, use);
         else r.ok = epi_conv_fast<0, false>(w, tmem_lane, warp, lane, desc, h0, h1, h2, h3, use);
     }
 }
 
+template <bool kRare>
 __device__ __forceinline__ void issuer_run(const LineParams &p, uint32_t tmem, uint32_t issuer, int ph, int stop, int it, RoleState &r)
 {
     for (; ph < stop; ++ph, r.ws.advance())
-        if (r.ok && !Waiter::aborted()) r.ok = issuer_conv(p, tmem, lds32(CTRL_ADDR(ptab) + 16u * (uint32_t)ph + 4u), r.ws, issuer, it, r.prev);
+        if (r.ok && !Waiter::aborted()) r.ok = issuer_conv<kRare>(p, tmem, lds32(CTRL_ADDR(ptab) + 16u * (uint32_t)ph + 4u), r.ws, issuer, it, r.prev);
 }
 
 __device__ __forceinline__ void loader_run(const LineParams &p, int ph, int stop, int it, RoleState &r)
@@ -995,9 +1014,9 @@ __device__ __forceinline__ void loader_run(const LineParams &p, int ph, int stop
         if (r.ok && !Waiter::aborted()) r.ok = loader_copy(p, r.next_copy, r.ws.slot, it);
 }
 
-// kLong: the network has convolutions whose residual term is no product.  A kernel of its own: as a fourth pass beside the other
-// three, which no ResNet's usual multipliers reach, it cost every network 0.7 % (ResNet-110 at 100,100 samples 62.0 -> 62.5 ms).
-template <bool kLong>
+// kRare: the network has convolutions whose residual term is no product, or two K-steps of unpaired lines.  A kernel of its own: the
+// first's pass alone, beside the other three, cost every network 0.7 % (ResNet-110 at 100,100 samples 62.0 -> 62.5 ms).
+template <bool kRare>
 __global__ void __launch_bounds__(kThreads, 1) k_line(const __grid_constant__ LineParams p)
 {
     Ctrl *ctrl = the_ctrl();
@@ -1055,9 +1074,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_line(const __grid_constant__ Li
             }
             const int stop = min(end, ph + (int)e.z);
             if (warp < kEpiWarps) {
-                epilogue_run<kLong>(p, tmem, warp, lane, ph, stop, it, r);
+                epilogue_run<kRare>(p, tmem, warp, lane, ph, stop, it, r);
             } else if (lane == 0) {
-                if (warp < kLoaderWarp) issuer_run(p, tmem, warp - kEpiWarps, ph, stop, it, r);
+                if (warp < kLoaderWarp) issuer_run<kRare>(p, tmem, warp - kEpiWarps, ph, stop, it, r);
                 else loader_run(p, ph, stop, it, r);
             }
             ph = stop;
@@ -1147,19 +1166,29 @@ bool set_geometry(LGeo &t)
 struct PlanBuffer { uint32_t bytes = 0, off = 0; int birth = 0, death = 0, halo = 0; };
 struct AllocReq { uint32_t bytes; int birth, death, slack; uint32_t *off; int conv; };
 
-// First-fit placement of one request among the allocations that are still busy at its birth.
-bool place(std::vector<AllocReq> &done, AllocReq &r, uint32_t capacity)
+// First-fit placement of one request among the allocations that are still busy at its birth, from the bottom or from the top.
+bool place(std::vector<AllocReq> &done, AllocReq &r, uint32_t capacity, bool high)
 {
     std::vector<std::pair<uint32_t, uint32_t>> busy;
     for (const AllocReq &e : done)
         if (e.death >= r.birth - r.slack) busy.push_back({*e.off, *e.off + e.bytes});
     std::sort(busy.begin(), busy.end());
     uint32_t at = kCtrlBytes;
-    for (const auto &b : busy) {
-        if (at + r.bytes <= b.first) break;
-        at = std::max(at, (b.second + 127u) & ~127u);
+    if (high) {
+        uint32_t end = capacity;
+        for (auto b = busy.rbegin(); b != busy.rend() && end >= r.bytes; ++b) {
+            if (((end - r.bytes) & ~127u) >= b->second) break;
+            end = std::min(end, b->first);
+        }
+        at = end >= r.bytes ? (end - r.bytes) & ~127u : 0u;
+        if (at < kCtrlBytes) return false;
+    } else {
+        for (const auto &b : busy) {
+            if (at + r.bytes <= b.first) break;
+            at = std::max(at, (b.second + 127u) & ~127u);
+        }
+        if (at + r.bytes > capacity) return false;
     }
-    if (at + r.bytes > capacity) return false;
     *r.off = at;
     done.push_back(r);
     return true;
@@ -1169,6 +1198,8 @@ bool place(std::vector<AllocReq> &done, AllocReq &r, uint32_t capacity)
 // line_plan_probe, and ISC_PLAN_DEBUG=1 prints it.
 thread_local int g_plan_rule = 0;
 #define PLAN_FAIL(id) do { g_plan_rule = (id); if (getenv("ISC_PLAN_DEBUG")) fprintf(stderr, "line engine: plan rule %d failed\n", id); return false; } while (0)
+
+bool no_other_way(const PlanTry &how) { return &how == kPlanTries + kPlanUsual && g_plan_rule != kPlanRuleRoom && g_plan_rule != kPlanRuleBars; }
 
 bool conv_ok(const isc_layer &L, bool first)
 {
@@ -1202,7 +1233,7 @@ struct LinePlan {
     unsigned long long *d_phase_cycles = nullptr;
     uint8_t *d_dump = nullptr;
     int sm_count = 0;
-    bool long_residual = false;          // a convolution needs k_line<true>
+    bool rare = false;                   // a convolution needs k_line<true>
     int attr_device = -1;                // the device on which the kernel's shared-memory limit has been raised
     // launches smaller than the GPU (see line_run)
     cudaStream_t side[kSideStreams] = {};
@@ -1235,8 +1266,7 @@ struct ConvPlan {
     std::vector<Unit> units;
 };
 
-// op_chains: MMA chains that one operation may hold at most
-bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_w, int n_classes, int op_chains, LinePlan *plan,
+bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_w, int n_classes, const PlanTry &how, LinePlan *plan,
                 std::vector<uint8_t> *blob_out, std::vector<uint32_t> *blob_offsets, std::vector<PhaseEntry> *ptab_out,
                 std::vector<ConvSrc> *csrc_out, std::vector<uint8_t> *bar_counts_out, std::vector<int32_t> *acc_init_out)
 {
@@ -1372,7 +1402,7 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
         // (p: right, p + 1: left), (p + 1: centre, right); the middle one adds to four output lines, with zero weights where a line
         // does not reach.  Three MMAs for two lines instead of four with half of every second one empty: stage 1 of a CIFAR
         // ResNet takes 2,450 instead of 2,990 cycles of operand reads a convolution.
-        cp.paired = cp.stacked && cp.units.size() == 3 && in.n_lines % 2 == 0;
+        cp.paired = how.paired && cp.stacked && cp.units.size() == 3 && in.n_lines % 2 == 0;
         if (cp.paired) {
             const long long u0 = unit_addr(cp.units[0]), u1 = unit_addr(cp.units[1]), u2 = unit_addr(cp.units[2]), pitch = (long long)in.pitch * 16;
             cp.a_delta = {(int)u0, (int)u2, (int)(pitch + u1)};
@@ -1458,14 +1488,15 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
             for (int l : o.need) o.ready = std::max(o.ready, prev_time(l));
         }
         std::stable_sort(proto.begin(), proto.end(), [](const ProtoOp &a, const ProtoOp &b) { return a.ready < b.ready; });
-        // In long paired convolutions two consecutive pairs make one operation: an issuing thread spends as much on a record as on
-        // its MMAs.
-        if (cp.paired && cp.m >= 16) {
+        // In long paired convolutions two consecutive pairs make one operation, where lines are not paired up to four chains: an issuing
+        // thread spends as much on a record as on its MMAs.
+        const int step = cp.paired ? 2 : 1;                          // lines of a chain
+        if (cp.stacked && (cp.paired || cp.kunits.size() == 2) && cp.m >= 16) {
             std::vector<ProtoOp> merged;
             for (const ProtoOp &o : proto) {
                 ProtoOp *l = merged.empty() ? nullptr : &merged.back();
-                if (l && l->n_chains < op_chains && l->a_line + 2 * l->n_chains == o.a_line && l->d_line + 2 * l->n_chains == o.d_line &&
-                    l->b_block == (int)kPairInner && o.b_block == (int)kPairInner) {
+                if (l && l->n_chains < how.chains && l->a_line + step * l->n_chains == o.a_line && l->d_line + step * l->n_chains == o.d_line &&
+                    l->n_blocks == o.n_blocks && l->b_block == o.b_block && (!cp.paired || o.b_block == (int)kPairInner)) {
                     l->n_chains += 1;
                     l->ready = std::max(l->ready, o.ready);
                     for (int n : o.need) if (std::find(l->need.begin(), l->need.end(), n) == l->need.end()) l->need.push_back(n);
@@ -1502,7 +1533,7 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
             if (!fits) { cp.res_form = ResidualForm(); cp.res_c = 0; }
         }
         cp.general = general;
-        const int upl = (!general && cp.m >= 16 && cp.m % 4 == 0) ? 4 : sup;
+        const int upl = (!general && cp.m >= 16 && cp.m % 4 == 0 && !(how.packed && cp.scatter)) ? 4 : sup;
         cp.recs_per_item = upl / sup;
         cp.n_units = (cp.m + upl - 1) / upl;
         cp.unit_of.assign((size_t)cp.m, 0);
@@ -1699,7 +1730,7 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
         class_done[k] = (int)bar_counts_out->size();
         for (int l = 0; l < class_lines[k]; ++l) bar_counts_out->push_back((uint8_t)(4 * class_chunks[k]));
     }
-    if ((int)bar_counts_out->size() > kMaxBars) PLAN_FAIL(14);
+    if ((int)bar_counts_out->size() > kMaxBars) PLAN_FAIL(kPlanRuleBars);
     // ---- blob sizes and shared-memory placement in order of birth
     std::vector<uint32_t> w_bytes((size_t)n_conv), w_off((size_t)n_conv), w_rel((size_t)n_conv), c_rel((size_t)n_conv),
         ops_rel((size_t)n_conv), passes_rel((size_t)n_conv), vec_rel((size_t)n_conv);
@@ -1707,7 +1738,7 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
         const ConvPlan &cp = convs[(size_t)c];
         const isc_layer &L = layers[cp.layer].d;
         const uint32_t rows = (uint32_t)(cp.stacked ? 3 : 1) * (uint32_t)L.cout;
-        uint32_t at = (uint32_t)sizeof(LConvDesc);
+        uint32_t at = how.packed ? (uint32_t)(offsetof(LConvDesc, a_lo) + (cp.kunits.size() + 3) / 4 * 16) : (uint32_t)sizeof(LConvDesc);
         ops_rel[(size_t)c] = at; at += ((uint32_t)cp.ops.size() + (uint32_t)kIssuers) * (uint32_t)sizeof(LOp);    // spare records: reads run one ahead
         passes_rel[(size_t)c] = at; at += (uint32_t)cp.passes.size() * (uint32_t)sizeof(LPass);
         at = (at + 127u) & ~127u;
@@ -1724,28 +1755,47 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
     std::stable_sort(reqs.begin(), reqs.end(), [](const AllocReq &a, const AllocReq &b) { return a.birth < b.birth; });
     uint32_t high = kCtrlBytes;
     std::vector<char> late((size_t)n_conv, 0);
-    for (AllocReq &r : reqs) {
-        bool ok = place(placed, r, kSmemLimit);
-        if (!ok && r.conv > 0) {
-            // A blob is normally copied when the convolution before its own starts, while the one before that may
-            // still be in its epilogue (slack 1).  Where that does not fit, it is copied once that one is complete.
-            r.slack = 0;
-            late[(size_t)r.conv] = 1;
-            ok = place(placed, r, kSmemLimit);
-        }
-        if (!ok) {
-            if (getenv("ISC_PLAN_DEBUG")) {
-                fprintf(stderr, "line engine: no room for %u bytes born at phase %d (dies %d); busy then:\n", r.bytes, r.birth, r.death);
-                for (const AllocReq &e : placed)
-                    if (e.death >= r.birth - r.slack)
-                        fprintf(stderr, "  [%u, %u) phases %d..%d\n", *e.off, *e.off + e.bytes, e.birth, e.death);
+    // Packed plans try other places, tensors from the top and blobs from the bottom first and then either at random.
+    uint32_t dice = 1;
+    auto from_top = [&](const AllocReq &r, int attempt) {
+        if (!how.packed) return false;
+        if (attempt == 0) return r.conv < 0;
+        dice ^= dice << 13; dice ^= dice >> 17; dice ^= dice << 5;
+        return (dice & 4u) != 0;
+    };
+    auto lay_out = [&](int attempt) {
+        placed.clear();
+        std::fill(late.begin(), late.end(), 0);
+        high = kCtrlBytes;
+        for (AllocReq &r : reqs) {
+            r.slack = r.conv > 0 ? 1 : 0;
+            bool ok = place(placed, r, kSmemLimit, from_top(r, attempt));
+            if (!ok && r.conv > 0) {
+                // A blob is normally copied when the convolution before its own starts, while the one before that may
+                // still be in its epilogue (slack 1).  Where that does not fit, it is copied once that one is complete.
+                r.slack = 0;
+                late[(size_t)r.conv] = 1;
+                ok = place(placed, r, kSmemLimit, from_top(r, attempt));
             }
-            PLAN_FAIL(15);
+            if (!ok) {
+                if (getenv("ISC_PLAN_DEBUG") && attempt == 0) {
+                    fprintf(stderr, "line engine: no room for %u bytes born at phase %d (dies %d); busy then:\n", r.bytes, r.birth, r.death);
+                    for (const AllocReq &e : placed)
+                        if (e.death >= r.birth - r.slack)
+                            fprintf(stderr, "  [%u, %u) phases %d..%d\n", *e.off, *e.off + e.bytes, e.birth, e.death);
+                }
+                return false;
+            }
+            high = std::max(high, *r.off + r.bytes);
         }
-        high = std::max(high, *r.off + r.bytes);
-        if (getenv("ISC_PLAN_DEBUG") && atoi(getenv("ISC_PLAN_DEBUG")) > 1)
+        return true;
+    };
+    bool laid_out = false;
+    for (int attempt = 0; attempt < (how.packed ? kPackAttempts : 1) && !laid_out; ++attempt) laid_out = lay_out(attempt);
+    if (!laid_out) PLAN_FAIL(kPlanRuleRoom);
+    if (getenv("ISC_PLAN_DEBUG") && atoi(getenv("ISC_PLAN_DEBUG")) > 1)
+        for (const AllocReq &r : placed)
             fprintf(stderr, "  %s %d: [%u, %u) phases %d..%d\n", r.conv >= 0 ? "blob" : "tensor", r.conv, *r.off, *r.off + r.bytes, r.birth, r.death);
-    }
     plan->tensors = T;
     plan->tensor_off.assign(T.size(), 0);
     for (int t = 0; t <= n_conv_layers; ++t) plan->tensor_off[(size_t)t] = buffers[(size_t)T[(size_t)t].buffer].off;
@@ -1776,7 +1826,7 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
         std::vector<uint8_t> blob(w_bytes[(size_t)c], 0);
         LConvDesc D;
         memset(&D, 0, sizeof(D));
-        plan->long_residual |= L.res_tensor >= 0 && !cp.general && !cp.res_form.exists();
+        plan->rare |= (L.res_tensor >= 0 && !cp.general && !cp.res_form.exists()) || (cp.stacked && cp.kunits.size() == 2);
         D.flags = (L.res_tensor >= 0 ? CF_RES : 0u) | (cp.scatter ? CF_SCATTER : 0u) | (cp.general ? CF_GENERAL : 0u) | (L.res_tensor >= 0 && !cp.res_form.exists() ? CF_RES_LONG : 0u) | (cp.paired ? CF_PAIRED : 0u);
         D.n_items = (uint32_t)(cp.n_units * cp.n_chunks); D.recs_per_item = (uint32_t)cp.recs_per_item; D.d_base = (uint32_t)bank_base(c);
         D.bar_full = (uint32_t)class_full[(size_t)cp.cls]; D.bar_done = (uint32_t)class_done[(size_t)cp.cls];
@@ -1818,10 +1868,10 @@ bool build_plan(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_
         for (size_t k = 0; k < cp.kunits.size(); ++k)
             for (const LOp &op : cp.ops) {
                 const long long lo_b = (long long)in.line0 - (long long)in.pitch * 16 + (long long)op.a_add * 16 + cp.a_delta[k];
-                const long long hi_b = lo_b + cp.a_lbo[k] + 128 * 16 + (long long)std::max(((op.flags >> 10) & 7) - 1, 0) * 2 * in.pitch * 16;
+                const long long hi_b = lo_b + cp.a_lbo[k] + 128 * 16 + (long long)std::max(((op.flags >> 10) & 7) - 1, 0) * (cp.paired ? 2 : 1) * in.pitch * 16;
                 if (lo_b < 0 || hi_b > (long long)in.bytes) PLAN_FAIL(18);
             }
-        memcpy(blob.data(), &D, sizeof(D));
+        memcpy(blob.data(), &D, ops_rel[(size_t)c]);
         memcpy(blob.data() + ops_rel[(size_t)c], cp.ops.data(), cp.ops.size() * sizeof(LOp));
         memcpy(blob.data() + passes_rel[(size_t)c], cp.passes.data(), cp.passes.size() * sizeof(LPass));
         // weights: per K-step, rows = block * cout + column; block b is vertical tap 2 - b when stacked, and 3 - b for the second
@@ -1922,14 +1972,15 @@ int line_plan_probe(const LayerIn *layers, int n_layers, int in_c, int in_h, int
     *smem_bytes = 0;
     bool ok = structure_ok(layers, n_layers, n_classes);
     if (ok) {
-        for (int chains : kOpChainTries) {
+        for (const PlanTry &how : kPlanTries) {
+            if (no_other_way(how)) break;
             LinePlan plan;
             std::vector<uint8_t> blob, bar_counts;
             std::vector<uint32_t> blob_off;
             std::vector<PhaseEntry> ptab;
             std::vector<ConvSrc> csrc;
             std::vector<int32_t> acc_init;
-            ok = build_plan(layers, n_layers, in_c, in_h, in_w, n_classes, chains, &plan, &blob, &blob_off, &ptab, &csrc, &bar_counts, &acc_init);
+            ok = build_plan(layers, n_layers, in_c, in_h, in_w, n_classes, how, &plan, &blob, &blob_off, &ptab, &csrc, &bar_counts, &acc_init);
             if (ok) *smem_bytes = plan.smem_bytes;
             if (ok) break;
         }
@@ -1950,10 +2001,11 @@ int line_build(const LayerIn *layers, int n_layers, int in_c, int in_h, int in_w
     std::vector<PhaseEntry> ptab;
     std::vector<ConvSrc> csrc;
     std::vector<int32_t> acc_init;
-    for (int chains : kOpChainTries) {
+    for (const PlanTry &how : kPlanTries) {
+        if (no_other_way(how)) break;
         plan = new LinePlan();
         blob.clear(); bar_counts.clear(); blob_off.clear(); ptab.clear(); csrc.clear();
-        if (build_plan(layers, n_layers, in_c, in_h, in_w, n_classes, chains, plan, &blob, &blob_off, &ptab, &csrc, &bar_counts, &acc_init)) break;
+        if (build_plan(layers, n_layers, in_c, in_h, in_w, n_classes, how, plan, &blob, &blob_off, &ptab, &csrc, &bar_counts, &acc_init)) break;
         delete plan;
         plan = nullptr;
     }
@@ -2089,7 +2141,7 @@ static int line_join(LinePlan *p, cudaStream_t st)
 
 static int line_launch(LinePlan *p, LineParams &q, cudaStream_t st)
 {
-    const auto kernel = p->long_residual ? k_line<true> : k_line<false>;
+    const auto kernel = p->rare ? k_line<true> : k_line<false>;
     int device = -1;
     bool ok = cudaGetDevice(&device) == cudaSuccess;
     if (ok && device != p->attr_device) {
